@@ -78,6 +78,7 @@ namespace it_stream {
 
 constexpr int THREADS = 256;
 constexpr int UNROLL = IT_GATHER_UNROLL;
+enum { RED_SUM = 0, RED_MAX = 1, RED_MIN = 2 };   // sum also serves mean (the division happens once, at the end)
 
 // One lane's slice of a feature row: SB = 4, 8 or 16 bytes, LPR = row bytes / SB lanes per row (see
 // dispatch_row_bytes for the choice).  A slice stays packed while it is in flight and is widened to fp32
