@@ -159,14 +159,19 @@ it_status launch_gat_lpr(const it_gat_args &a, StreamParams sp, int64_t bound_lo
   auto bytes_of = [=](int b, int64_t rows) {
     return (double)g->h_bucket_edges[b] * (4.0 + 4.0 * heads + row_bytes) + (double)rows * (20.0 + 4.0 * heads + row_bytes);
   };
-  return launch_buckets<T, SB, LPR>(g, sp, pol, bytes_of, IT_K_GAT_CTA, IT_K_GAT_FLAT, IT_K_GAT_EMPTY, bound_lo, bound_hi, a.counters, st);
+  return launch_buckets<T, SB, LPR, false>(g, sp, pol, bytes_of, IT_K_GAT_CTA, IT_K_GAT_FLAT, IT_K_GAT_EMPTY, bound_lo, bound_hi, a.counters, st);
 }
 
 template <typename T>
 it_status launch_gat(const it_gat_args &a, StreamParams sp, cudaStream_t st) {
   // 16-byte slices as long as one never straddles two heads
   const bool wide = (a.head_dim * (int)sizeof(T)) % 16 == 0;
-  return dispatch_row_bytes(a.heads * a.head_dim * (int)sizeof(T), wide, [&]<int SB, int LPR>(int64_t lo, int64_t hi) {
+  const int row_bytes = a.heads * a.head_dim * (int)sizeof(T);
+  if ((row_bytes & (row_bytes - 1)) != 0 || row_bytes < 16 || row_bytes > 512) {
+    it_set_error("feature row of %d bytes is not 16, 32, 64, 128, 256 or 512 bytes", row_bytes);
+    return IT_ERR_UNSUPPORTED;
+  }
+  return dispatch_row_bytes(row_bytes, wide, [&]<int SB, int LPR>(int64_t lo, int64_t hi) {
     if ((a.head_dim * (int)sizeof(T)) % SB != 0) {
       it_set_error("gat: a %d-byte lane slice would straddle two heads (head_dim %d)", SB, a.head_dim);
       return IT_ERR_UNSUPPORTED;
@@ -188,7 +193,7 @@ it_status it_launch_gat(const it_gat_args &a, cudaStream_t st) {
   if (g->n == 0) return IT_OK;
   StreamParams sp;
   sp.meta = g->bucket_meta; sp.owner = g->bucket_owner; sp.indices = a.per_edge_rows ? nullptr : g->indices; sp.weights = nullptr;
-  sp.src = a.z; sp.row_lo = sp.row_hi = 0; sp.dim = a.heads * a.head_dim; sp.batch_rows = 1; sp.counter = nullptr; sp.claim = 1;
+  sp.src = a.z; sp.row_lo = sp.row_hi = 0; sp.dim = a.heads * a.head_dim; sp.batch_rows = 1; sp.counter = nullptr; sp.claim = 1; sp.slices = 0;
   sp.src_pitch = (uint32_t)(sp.dim * it_dtype_size(a.dtype));
   if (a.dtype == IT_F32) IT_TRY(launch_gat<float>(a, sp, st));
   else IT_TRY(launch_gat<__nv_bfloat16>(a, sp, st));

@@ -91,13 +91,13 @@ __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p
 
 }  // namespace
 
-// One column chunk of the rows: `a.dim` is the chunk's width (a power of two between 16 and 512 bytes), the
+// One column chunk of the rows: `a.dim` is the chunk's width (16 to 512 bytes), the
 // pointers already point at its first column, and the *_ld fields / src_ld carry the full row lengths.
 static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
   const it_graph *g = a.g;
   StreamParams sp;
   sp.meta = g->bucket_meta; sp.owner = nullptr; sp.indices = a.per_edge_rows ? nullptr : g->indices; sp.weights = g->edge_weights;
-  sp.src = a.src; sp.row_lo = sp.row_hi = 0; sp.dim = a.dim; sp.batch_rows = 1; sp.counter = nullptr; sp.claim = 1;
+  sp.src = a.src; sp.row_lo = sp.row_hi = 0; sp.dim = a.dim; sp.batch_rows = 1; sp.counter = nullptr; sp.claim = 1; sp.slices = 0;
   sp.src_pitch = (uint32_t)((a.src_ld > 0 ? a.src_ld : a.dim) * it_dtype_size(a.dtype));
   if (a.dtype == IT_F32) IT_TRY(it_launch_gather_rows_f32(a, sp, st));
   else IT_TRY(it_launch_gather_rows_bf16(a, sp, st));
@@ -118,8 +118,8 @@ static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
   return IT_OK;
 }
 
-// Rows of any multiple of 16 bytes: the kernels take rows of 16, 32, ..., 512 bytes, so a wider or odd row is cut
-// into column chunks of those widths (largest first) and each chunk is gathered on its own, reading and writing
+// Rows of any multiple of 16 bytes: the kernels take rows of 16, 32, 64 and 80 to 512 bytes, so a wider row (or one of 48
+// bytes) is cut into column chunks, largest first, and each chunk is gathered on its own, reading and writing
 // its columns in place.  The aggregate is entry by entry, so the chunks are independent; each pass re-reads
 // the edge indices (4 bytes against a chunk of up to 512 per edge).
 it_status it_launch_gather(const it_gather_args &a, cudaStream_t st) {
@@ -134,8 +134,10 @@ it_status it_launch_gather(const it_gather_args &a, cudaStream_t st) {
   const int full = a.dim;
   int c0 = 0;   // first column of the chunk
   while (c0 < full) {
-    int bytes = 512;
-    while (bytes > (full - c0) * es) bytes >>= 1;
+    // what is left as one chunk where a kernel takes it: up to 512 bytes, and from 80 bytes on any multiple of 16 (the
+    // lanes past the row idle); 48 bytes as 32 + 16
+    const int left = (full - c0) * es;
+    const int bytes = left >= 512 ? 512 : (left == 48 ? 32 : left);
     it_gather_args c = a;
     c.dim = bytes / es;
     c.src = (const char *)a.src + (size_t)c0 * es;

@@ -10,8 +10,8 @@
 //   * stream_rows_ring_kernel, stream_cta_ring_kernel (stream_ring.cuh; rows of 128 bytes and more):
 //     a warp walks the edges of a batch of rows (or of its part of one very long row) as one flat
 //     stream and stages the source rows through a per-warp ring in shared memory with cp.async.
-//   * stream_short_rows_kernel (128-byte rows of at most a few dozen edges): one group of 8 lanes
-//     per row, eight row loads back to back, no edge stream.
+//   * stream_short_rows_pipe_kernel, stream_tiny_rows_kernel (the same widths up to 256 bytes, rows of at most a few
+//     dozen edges): one group of 8 or 16 lanes per row, eight row loads back to back, no edge stream.
 //   * stream_rows_kernel (rows narrower than 128 bytes): a *group* of LPR lanes takes a batch of rows
 //     and walks the batch's edges as one flat stream with UNROLL rows in flight per lane in registers.
 //   * stream_cta_kernel (the same rows, very long): one CTA per row, each warp a contiguous chunk,
@@ -55,17 +55,8 @@
 #ifndef IT_RING_CLAIMS_PER_WARP
 #define IT_RING_CLAIMS_PER_WARP 16   // claims a warp of the ring kernel makes on average over a launch
 #endif
-#ifndef IT_SHORT_MIN_BLOCKS
-#define IT_SHORT_MIN_BLOCKS 6   // resident CTAs per SM of the short-row kernel (eight 16-byte slices in flight per lane, staged in shared memory)
-#endif
 #ifndef IT_SHORT_EDGES
 #define IT_SHORT_EDGES 8         // source rows a lane of the short-row kernel has in flight per round
-#endif
-#ifndef IT_SHORT_ASYNC
-#define IT_SHORT_ASYNC 1         // 1: the short-row kernel stages its slices through shared memory with cp.async (0: in registers)
-#endif
-#ifndef IT_SHORT_256
-#define IT_SHORT_256 1           // 1: 256-byte rows of at most IT_SHORT_BELOW edges take the lane-group kernel too (16 lanes per row)
 #endif
 #ifndef IT_SHORT_BELOW
 #define IT_SHORT_BELOW 32       // 128-byte rows: buckets of rows up to this long take the short-row kernel
@@ -221,6 +212,7 @@ struct StreamParams {
   int64_t row_lo, row_hi;                 // range inside the bucket-ordered row list
   int dim;                                // elements of a row that are gathered (one column chunk of the source rows)
   uint32_t src_pitch;                     // bytes from one source row to the next (>= dim elements)
+  int slices;                             // lane slices of a row: <= LPR; lanes beyond them idle (rows that are no power of two)
   int batch_rows;                         // rows a lane group takes at a time (<= LPR)
   int *counter;                           // ring kernel: zeroed device word from which the warps claim their batches after
                                           // their first ones (NULL: every warp walks a fixed stride of the batches)
@@ -367,104 +359,16 @@ __global__ void __launch_bounds__(THREADS, IT_GATHER_MIN_BLOCKS) stream_rows_ker
 // ----------------------------------------------------------------------------- short rows: one lane group each, no edge stream
 // For rows of at most a few dozen edges the bookkeeping of a flat edge stream costs more than the edges.
 // Here a group of LPR lanes (16-byte slices, LPR >= 8) owns one row: lanes 0..7 of the group fetch eight
-// source indices with one load, the group issues the eight row loads back to back and then reduces them;
-// rows longer than eight edges take more rounds.  The slices are staged through shared memory (cp.async, 32 KB per
-// CTA): the kernel is bound by the loads it keeps in flight, and without eight 16-byte slices in registers it fits
-// six CTAs per SM instead of four (measured: 4.6 -> 5.6 TB/s on rows of at most 8 edges).  The groups of a warp run in lockstep (warp-wide loop
-// bounds, predicated edges), so a warp never splits.
-template <typename T, int LPR, class Policy>
-__global__ void __launch_bounds__(THREADS, IT_SHORT_MIN_BLOCKS) stream_short_rows_kernel(StreamParams p, Policy pol) {
-  constexpr int NS = Policy::NS;
-  constexpr int E = IT_SHORT_EDGES;   // edges per round
-  static_assert(LPR >= E, "lanes 0..7 of a group fetch the indices of a round");
-  using Slice = RowSlice<T, 16>;
-  const int lane = threadIdx.x & 31;
-  const int t = lane % LPR, gbase = lane - t;
-  pol.setup(t);
-  const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
-  const uint32_t ROWB = p.src_pitch;
-  const int64_t rows_per_sweep = (int64_t)gridDim.x * (THREADS / LPR);
-#if IT_SHORT_ASYNC
-  __shared__ uint4 sbuf[E][THREADS];
-  const uint32_t my_buf = (uint32_t)__cvta_generic_to_shared(&sbuf[0][threadIdx.x]);
-#endif
-  // warp-uniform loop: every group of the warp takes one row per iteration
-  for (int64_t i0 = p.row_lo + (int64_t)blockIdx.x * (THREADS / LPR) + (threadIdx.x >> 5) * (32 / LPR); i0 < p.row_hi; i0 += rows_per_sweep) {
-    const int64_t i = i0 + lane / LPR;
-    const bool valid = i < p.row_hi;
-    int64_t j0 = 0;
-    int len = 0, dest = 0, owner = 0;
-    if (valid) {
-      const it_row_meta m = load_meta(p.meta + i);
-      j0 = m.j0; len = m.len; dest = m.dest;
-      if (Policy::NEEDS_OWNER) owner = __ldcs(p.owner + i);
-    }
-    const int maxlen = __reduce_max_sync(0xffffffffu, len);
-    float st[NS];
-    pol.init(st);
-    if (valid) pol.begin_row(dest, owner);
-    for (int k0 = 0; k0 < maxlen; k0 += E) {
-      int32_t idx = 0;
-      float w = 1.f;
-      if (t < E && k0 + t < len) {
-        idx = p.indices ? __ldcs(p.indices + j0 + k0 + t) : (int32_t)(j0 + k0 + t);
-        if (Policy::WEIGHTED) w = __ldcs(p.weights + j0 + k0 + t);
-      }
-      float ww[E], xx[E];
-#if IT_SHORT_ASYNC
-      // the slices travel through shared memory (cp.async) instead of registers: each lane later reads back exactly
-      // the bytes it copied, so waiting for its own copy group is all the synchronisation there is, and the
-      // registers saved buy more resident warps
-#pragma unroll
-      for (int k = 0; k < E; ++k) {
-        const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx, gbase + k);
-        ww[k] = Policy::WEIGHTED ? __shfl_sync(0xffffffffu, w, gbase + k) : 1.f;
-        xx[k] = 0.f;
-        if (k0 + k < len) {
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(my_buf + (uint32_t)k * (THREADS * 16)), "l"(my_src + (uint64_t)s * ROWB) : "memory");
-          if (Policy::HAS_EXTRA) xx[k] = pol.extra(s);
-        }
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-#pragma unroll
-      for (int k = 0; k < E; ++k)
-        if (k0 + k < len) {
-          uint4 v;
-          asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(my_buf + (uint32_t)k * (THREADS * 16)) : "memory");
-          pol.edge(st, v, ww[k], xx[k]);
-        }
-#else
-      typename Slice::Raw v[E];
-#pragma unroll
-      for (int k = 0; k < E; ++k) {
-        const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx, gbase + k);
-        ww[k] = Policy::WEIGHTED ? __shfl_sync(0xffffffffu, w, gbase + k) : 1.f;
-        xx[k] = 0.f;
-        if (k0 + k < len) {
-          v[k] = Slice::load(my_src + (uint64_t)s * ROWB);
-          if (Policy::HAS_EXTRA) xx[k] = pol.extra(s);
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < E; ++k)
-        if (k0 + k < len) pol.edge(st, v[k], ww[k], xx[k]);
-#endif
-    }
-    if (valid) pol.end_row(st, dest, owner, len);
-  }
-}
-
-// The same kernel with its three dependent loads (row record -> source indices -> source rows) overlapped across
+// source indices with one load, the group issues the eight row copies back to back through shared memory (cp.async;
+// each lane reads back the bytes it copied) and then reduces them; rows longer than eight edges take more rounds.  The
+// groups of a warp run in lockstep (warp-wide loop bounds, predicated edges), so a warp never splits.
+// The three dependent loads (row record -> source indices -> source rows) are overlapped across
 // rounds: a round is one batch of up to E edges of one row per lane group.  While the source rows of the current
 // round are in flight, the indices of the next round (of the same row if it is longer than E, else of the group's
 // next row) and the record of the row after next are in flight too, so that only one memory round trip per round
 // is exposed instead of three.  Costs a dozen registers per thread (four resident CTAs per SM instead of six).
-// Measured against the plain loop above: 3 % to 6 % less time on the 128-byte rows of at most 32 edges, 2 % on
+// Measured against a loop without the overlap: 3 % to 6 % less time on the 128-byte rows of at most 32 edges, 2 % on
 // the 256-byte fp32 rows, none on the GAT rows (that kernel is bound by its issue slots, not by exposed latency).
-#ifndef IT_SHORT_PIPE
-#define IT_SHORT_PIPE 1          // 1: short rows take the pipelined kernel
-#endif
 #ifndef IT_SHORT_PIPE_BLOCKS
 #define IT_SHORT_PIPE_BLOCKS 4   // resident CTAs per SM the pipelined kernel's register budget is set for (measured: five spill and gain nothing)
 #endif
@@ -474,13 +378,14 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_MIN_BLOCKS) stream_short_row
 #ifndef IT_SHORT_PIPE_WAVES
 #define IT_SHORT_PIPE_WAVES 1    // grid = SMs x resident CTAs x this: every CTA is resident from the start and walks its rows
 #endif
-template <typename T, int LPR, class Policy>
+template <typename T, int LPR, class Policy, bool PAD>
 __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_rows_pipe_kernel(StreamParams p, Policy pol) {
   constexpr int NS = Policy::NS;
   constexpr int E = IT_SHORT_EDGES;   // edges per round
   static_assert(LPR >= E, "lanes 0..7 of a group fetch the indices of a round");
   const int lane = threadIdx.x & 31;
   const int t = lane % LPR, gbase = lane - t;
+  const bool active = !PAD || t < p.slices;   // PAD: the row is narrower than the lane group
   pol.setup(t);
   const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
   const uint32_t ROWB = p.src_pitch;
@@ -518,7 +423,8 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_ro
     const int maxlen = __reduce_max_sync(0xffffffffu, cur.len);
     float st[NS];
     pol.init(st);
-    if (cur.len > 0) pol.begin_row(cur.dest, cur.owner);
+    const int len = active ? cur.len : 0;
+    if (len > 0) pol.begin_row(cur.dest, cur.owner);
     for (int k0 = 0; k0 < maxlen; k0 += E) {
       // the indices of the next round, in flight while this round's rows are
       int32_t idx_n; float w_n;
@@ -530,7 +436,7 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_ro
         const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx_c, gbase + k);
         ww[k] = Policy::WEIGHTED ? __shfl_sync(0xffffffffu, w_c, gbase + k) : 1.f;
         xx[k] = 0.f;
-        if (k0 + k < cur.len) {
+        if (k0 + k < len) {
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(my_buf + (uint32_t)k * (THREADS * 16)), "l"(my_src + (uint64_t)s * ROWB) : "memory");
           if (Policy::HAS_EXTRA) xx[k] = pol.extra(s);
         }
@@ -539,7 +445,7 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_ro
       asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
       for (int k = 0; k < E; ++k) {
-        if (k0 + k < cur.len) {
+        if (k0 + k < len) {
           uint4 v;
           asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(my_buf + (uint32_t)k * (THREADS * 16)) : "memory");
           pol.edge(st, v, ww[k], xx[k]);
@@ -547,7 +453,7 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_ro
       }
       idx_c = idx_n; w_c = w_n;
     }
-    if (cur.len > 0) pol.end_row(st, cur.dest, cur.owner, cur.len);
+    if (len > 0) pol.end_row(st, cur.dest, cur.owner, len);
     cur = nxt; nxt = nn;
   }
 }
@@ -566,7 +472,7 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_ro
 #ifndef IT_SHORT_PIPE2_BLOCKS
 #define IT_SHORT_PIPE2_BLOCKS 3
 #endif
-template <typename T, int LPR, class Policy>
+template <typename T, int LPR, class Policy, bool PAD>
 __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE2_BLOCKS) stream_tiny_rows_kernel(StreamParams p, Policy pol) {
   constexpr int NS = Policy::NS;
   constexpr int E = IT_SHORT_EDGES;
@@ -574,6 +480,7 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE2_BLOCKS) stream_tiny_ro
   extern __shared__ uint4 tiny_buf[];   // [2][E][THREADS]
   const int lane = threadIdx.x & 31;
   const int t = lane % LPR, gbase = lane - t;
+  const bool active = !PAD || t < p.slices;   // PAD: the row is narrower than the lane group
   pol.setup(t);
   const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
   const uint32_t ROWB = p.src_pitch;
@@ -603,7 +510,7 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE2_BLOCKS) stream_tiny_ro
 #pragma unroll
     for (int k = 0; k < E; ++k) {
       const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx, gbase + k);
-      if (k < r.len)
+      if (k < r.len && active)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(buf + (uint32_t)k * SLOT), "l"(my_src + (uint64_t)s * ROWB) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -623,18 +530,19 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE2_BLOCKS) stream_tiny_ro
     issue(r1, idx1, oth);                      // the next row's copies, in flight while this row is reduced
     float st[NS];
     pol.init(st);
-    if (r0.len > 0) pol.begin_row(r0.dest, r0.owner);
+    const int len = active ? r0.len : 0;
+    if (len > 0) pol.begin_row(r0.dest, r0.owner);
     asm volatile("cp.async.wait_group 1;" ::: "memory");   // this row's copies have landed
 #pragma unroll
     for (int k = 0; k < E; ++k) {
       const float ww = Policy::WEIGHTED ? __shfl_sync(0xffffffffu, w0, gbase + k) : 1.f;
-      if (k < r0.len) {
+      if (k < len) {
         uint4 v;
         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(cur + (uint32_t)k * SLOT) : "memory");
         pol.edge(st, v, ww, 0.f);
       }
     }
-    if (r0.len > 0) pol.end_row(st, r0.dest, r0.owner, r0.len);
+    if (len > 0) pol.end_row(st, r0.dest, r0.owner, len);
     r0 = r1; r1 = r2; r2 = r3; r3 = r4;
     idx0 = idx1; w0 = w1; idx1 = idx2; w1 = w2;
     const uint32_t sw = cur; cur = oth; oth = sw;
@@ -734,6 +642,7 @@ template <typename T, int SB, int LPR, class Policy>
 __global__ void __launch_bounds__(THREADS) stream_empty_kernel(StreamParams p, Policy pol) {
   constexpr int NS = Policy::NS;
   const int t = threadIdx.x % LPR;
+  if (t >= p.slices) return;
   pol.setup(t);
   const int64_t groups_total = (int64_t)gridDim.x * (THREADS / LPR);
   for (int64_t i = p.row_lo + (int64_t)blockIdx.x * (THREADS / LPR) + threadIdx.x / LPR; i < p.row_hi; i += groups_total) {
@@ -773,7 +682,7 @@ it_status allow_dynamic_smem(Kernel kernel, int smem, std::atomic<uint64_t> &don
 // rows different slice widths.
 // `counters`: IT_MAX_BUCKETS device words of scratch (or NULL): the ring kernel of bucket b hands out its batches from
 // word b, which is zeroed here, in stream order, before the launches.
-template <typename T, int SB, int LPR, class Policy, class BytesF>
+template <typename T, int SB, int LPR, bool PAD, class Policy, class BytesF>
 it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, BytesF bytes_of, int kid_cta, int kid_rows,
                          int kid_empty, int64_t bound_lo, int64_t bound_hi, int *counters, cudaStream_t st) {
   constexpr bool RING = SB * LPR >= 128;   // rows of 128 bytes and more are staged through shared memory
@@ -782,6 +691,7 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
 #endif
   if (RING && counters) IT_CUDA_TRY(cudaMemsetAsync(counters, 0, IT_MAX_BUCKETS * sizeof(int), st));
   p.counter = nullptr;
+  p.slices = p.dim * (int)sizeof(T) / SB;
   for (int b = g->n_buckets - 1; b >= 0; --b) {
     const int64_t lo = g->h_bucket_offsets[b], hi = g->h_bucket_offsets[b + 1];
     if (hi <= lo || g->bucket_bounds[b] <= bound_lo || g->bucket_bounds[b] > bound_hi) continue;
@@ -798,10 +708,10 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
       if constexpr (RING) {
         constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<SB, Policy::HAS_EXTRA>();
         static std::atomic<uint64_t> configured{0};   // per template instance: one bit per device ordinal
-        IT_TRY(allow_dynamic_smem(stream_cta_ring_kernel<T, SB, LPR, Policy>, smem, configured));
+        IT_TRY(allow_dynamic_smem(stream_cta_ring_kernel<T, SB, LPR, Policy, PAD>, smem, configured));
         // one CTA per row as far as the grid allows: the hardware hands out rows as CTAs retire
         unsigned blocks = (unsigned)(rows < (1 << 20) ? rows : (1 << 20));
-        IT_LAUNCH(kid_cta, bytes, 0, st, stream_cta_ring_kernel<T, SB, LPR, Policy><<<blocks, THREADS, smem, st>>>(p, pol));
+        IT_LAUNCH(kid_cta, bytes, 0, st, stream_cta_ring_kernel<T, SB, LPR, Policy, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
       } else {
         unsigned blocks = (unsigned)(rows < max_blocks ? rows : max_blocks);
         IT_LAUNCH(kid_cta, bytes, 0, st, stream_cta_kernel<T, SB, LPR, Policy><<<blocks, THREADS, 0, st>>>(p, pol));
@@ -810,7 +720,7 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
       // about 256 edges per batch at most: 32 rows of <= 8 edges, 8 rows of <= 32, one longer row (measured: walking
       // several longer rows as one stream, to pay the dependent loads at the start of a row once per batch, is slower)
       int br = bound <= 8 ? 32 : (bound <= 32 ? 8 : 1);
-      if constexpr (SB == 16 && (LPR == 8 || (LPR == 16 && IT_SHORT_256 != 0))) {   // 128-byte rows (and 256-byte rows)
+      if constexpr (SB == 16 && (LPR == 8 || LPR == 16)) {   // 128-byte rows (and 256-byte rows)
         if (bound <= IT_SHORT_BELOW) {   // one lane group per row
           const int64_t want = (rows + (THREADS / LPR) - 1) / (THREADS / LPR);
           if constexpr (IT_SHORT_PIPE2 != 0 && !Policy::HAS_EXTRA) {
@@ -820,22 +730,16 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
             if (bound <= IT_SHORT_EDGES && g->h_bucket_edges[b] <= (int64_t)IT_SHORT_PIPE2_AVG * rows) {
               constexpr int smem = 2 * IT_SHORT_EDGES * THREADS * 16;
               static std::atomic<uint64_t> configured2{0};
-              IT_TRY(allow_dynamic_smem(stream_tiny_rows_kernel<T, LPR, Policy>, smem, configured2));
+              IT_TRY(allow_dynamic_smem(stream_tiny_rows_kernel<T, LPR, Policy, PAD>, smem, configured2));
               const int64_t tiny_max = (int64_t)g->num_sms * IT_SHORT_PIPE2_BLOCKS;
               unsigned blocks = (unsigned)(want < tiny_max ? want : tiny_max);
-              IT_LAUNCH(kid_rows, bytes, 0, st, stream_tiny_rows_kernel<T, LPR, Policy><<<blocks, THREADS, smem, st>>>(p, pol));
+              IT_LAUNCH(kid_rows, bytes, 0, st, stream_tiny_rows_kernel<T, LPR, Policy, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
               continue;
             }
           }
-#if IT_SHORT_PIPE
           const int64_t short_max = (int64_t)g->num_sms * IT_SHORT_PIPE_BLOCKS * IT_SHORT_PIPE_WAVES;
           unsigned blocks = (unsigned)(want < short_max ? want : short_max);
-          IT_LAUNCH(kid_rows, bytes, 0, st, stream_short_rows_pipe_kernel<T, LPR, Policy><<<blocks, THREADS, 0, st>>>(p, pol));
-#else
-          const int64_t short_max = (int64_t)g->num_sms * IT_SHORT_MIN_BLOCKS * 4;
-          unsigned blocks = (unsigned)(want < short_max ? want : short_max);
-          IT_LAUNCH(kid_rows, bytes, 0, st, stream_short_rows_kernel<T, LPR, Policy><<<blocks, THREADS, 0, st>>>(p, pol));
-#endif
+          IT_LAUNCH(kid_rows, bytes, 0, st, stream_short_rows_pipe_kernel<T, LPR, Policy, PAD><<<blocks, THREADS, 0, st>>>(p, pol));
           continue;
         }
       }
@@ -843,8 +747,8 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
         constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<SB, Policy::HAS_EXTRA>();
         static std::atomic<uint64_t> configured{0}, configured1{0};   // per template instance: one bit per device ordinal
         const bool single = IT_RING_SINGLE_ROW && br == 1;
-        if (single) IT_TRY(allow_dynamic_smem(stream_rows_ring_kernel<T, SB, LPR, Policy, true>, smem, configured1));
-        else IT_TRY(allow_dynamic_smem(stream_rows_ring_kernel<T, SB, LPR, Policy, false>, smem, configured));
+        if (single) IT_TRY(allow_dynamic_smem(stream_rows_ring_kernel<T, SB, LPR, Policy, true, PAD>, smem, configured1));
+        else IT_TRY(allow_dynamic_smem(stream_rows_ring_kernel<T, SB, LPR, Policy, false, PAD>, smem, configured));
         p.batch_rows = br;
         const int64_t batches = (rows + br - 1) / br;
         // with a counter every CTA is resident from the start and its warps claim batches as they finish (rows of one
@@ -855,8 +759,8 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
         unsigned blocks = (unsigned)(want < ring_max ? want : ring_max);
         const int64_t per_warp = batches / ((int64_t)blocks * (THREADS / 32));
         p.claim = (int)(per_warp / IT_RING_CLAIMS_PER_WARP < 1 ? 1 : (per_warp / IT_RING_CLAIMS_PER_WARP > 4096 ? 4096 : per_warp / IT_RING_CLAIMS_PER_WARP));
-        if (single) IT_LAUNCH(kid_rows, bytes, 0, st, stream_rows_ring_kernel<T, SB, LPR, Policy, true><<<blocks, THREADS, smem, st>>>(p, pol));
-        else IT_LAUNCH(kid_rows, bytes, 0, st, stream_rows_ring_kernel<T, SB, LPR, Policy, false><<<blocks, THREADS, smem, st>>>(p, pol));
+        if (single) IT_LAUNCH(kid_rows, bytes, 0, st, stream_rows_ring_kernel<T, SB, LPR, Policy, true, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
+        else IT_LAUNCH(kid_rows, bytes, 0, st, stream_rows_ring_kernel<T, SB, LPR, Policy, false, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
         p.counter = nullptr;
       } else {                                // a group of LPR lanes per batch
         if (br > LPR) br = LPR;
@@ -873,33 +777,33 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
 }
 
 // Pick the slice width and group size for a row of `row_bytes` bytes and call
-// f.template operator()<SB, LPR>(bound_lo, bound_hi) for the buckets that take them.  Unless `wide` is false,
-// rows of 128 bytes use 16-byte slices throughout and rows of 256 bytes use them for their long rows, with
-// one slice per lane for the short ones (measured: the cheaper end of row wins there).
-#ifndef IT_WIDE_ABOVE
-#define IT_WIDE_ABOVE 32   // buckets of rows longer than this use 16-byte slices
-#endif
+// f.template operator()<SB, LPR>(bound_lo, bound_hi) for the buckets that take them.  Rows of 80 bytes and more that are
+// no power of two take the lane group of the next power of two with its last lanes idle.  One pass over the edges with
+// whole sectors beats one pass per power-of-two piece even at 25 of 32 lanes: a GCN of widths 100-128-128-48 on 15M
+// edges, whose 400-byte fp32 rows were 256 + 128 + 16, takes 2.98 ms instead of 4.24 (the 16-byte pieces alone moved a
+// 32-byte sector each and an edge index).
+// Unless `wide` is false, rows of 128 bytes use 16-byte slices throughout and rows of 256 bytes use them for every row
+// with edges (short rows: the lane-group kernel); <8, 32> keeps the empty rows.
 template <class F>
 it_status dispatch_row_bytes(int row_bytes, bool wide, F f) {
   constexpr int64_t ALL = INT64_MAX;
+  if (row_bytes > 256 && row_bytes <= 512) return f.template operator()<16, 32>(-1, ALL);
+  if (row_bytes > 128 && row_bytes <= 256) {
+    if (!wide) return f.template operator()<8, 32>(-1, ALL);
+    if (row_bytes < 256) return f.template operator()<16, 16>(-1, ALL);
+    IT_TRY((f.template operator()<16, 16>(0, ALL)));
+    return f.template operator()<8, 32>(-1, 0);
+  }
+  if (row_bytes > 64 && row_bytes <= 128) {
+    if (!wide) return f.template operator()<4, 32>(-1, ALL);
+    return f.template operator()<16, 8>(-1, ALL);
+  }
   switch (row_bytes) {
-    case 512: return f.template operator()<16, 32>(-1, ALL);
-    case 256:
-      if (!wide) return f.template operator()<8, 32>(-1, ALL);
-      if (IT_SHORT_256) {   // every row with edges takes 16-byte slices (short rows: the lane-group kernel); <8, 32> keeps the empty rows
-        IT_TRY((f.template operator()<16, 16>(0, ALL)));
-        return f.template operator()<8, 32>(-1, 0);
-      }
-      IT_TRY((f.template operator()<16, 16>(IT_WIDE_ABOVE, ALL)));
-      return f.template operator()<8, 32>(-1, IT_WIDE_ABOVE);
-    case 128:
-      if (!wide) return f.template operator()<4, 32>(-1, ALL);
-      return f.template operator()<16, 8>(-1, ALL);
     case 64: return f.template operator()<4, 16>(-1, ALL);
     case 32: return f.template operator()<4, 8>(-1, ALL);
     case 16: return f.template operator()<4, 4>(-1, ALL);
   }
-  it_set_error("feature row of %d bytes is not 16, 32, 64, 128, 256 or 512 bytes", row_bytes);
+  it_set_error("feature row of %d bytes has no kernel", row_bytes);
   return IT_ERR_UNSUPPORTED;
 }
 

@@ -65,7 +65,7 @@ template <int SB, bool HAS_EXTRA> constexpr int ring_bytes_per_warp() {
 }
 
 // What a warp needs to drive its ring: addresses, the fill of a stage and the reduction of one group.
-template <typename T, int SB, int LPR, class Policy>
+template <typename T, int SB, int LPR, class Policy, bool PAD>
 struct RingWarp {
   using G = RingGeom<SB, LPR>;
   using Raw = typename SliceRaw<SB>::type;
@@ -73,8 +73,10 @@ struct RingWarp {
   const char *my_src;           // my slice of source row 0
   uint32_t pitch;               // bytes from one source row to the next
   int slot;
+  bool active;                  // my slice lies inside the row (PAD: the row is narrower than the lane group)
 
-  __device__ __forceinline__ void setup(uint32_t ring_base, const void *src, uint32_t src_pitch, int lane) {
+  __device__ __forceinline__ void setup(uint32_t ring_base, const void *src, uint32_t src_pitch, int slices, int lane) {
+    active = !PAD || lane % LPR < slices;
     pitch = src_pitch;
     my_ring = ring_base + lane * SB;
     my_xring = ring_base + G::S * G::R * G::GB + lane * 4;
@@ -89,13 +91,13 @@ struct RingWarp {
 #pragma unroll
       for (int u = 0; u < G::R; ++u) {
         const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idxreg, k0 + u * G::SL + slot);
-        cp_async_slice<SB>(d + u * G::GB, my_src + (uint64_t)s * pitch);
+        if (active) cp_async_slice<SB>(d + u * G::GB, my_src + (uint64_t)s * pitch);
         if (Policy::HAS_EXTRA) cp_async_slice<4>(dx + u * 128, pol.extra_ptr(s));
       }
     } else {
       for (int u = 0; u * G::SL < n; ++u) {
         const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idxreg, k0 + u * G::SL + slot);
-        if (u * G::SL + slot < n) {
+        if (active && u * G::SL + slot < n) {
           cp_async_slice<SB>(d + u * G::GB, my_src + (uint64_t)s * pitch);
           if (Policy::HAS_EXTRA) cp_async_slice<4>(dx + u * 128, pol.extra_ptr(s));
         }
@@ -119,8 +121,8 @@ struct RingWarp {
 //   load_chunk(base, idx, w, ends): lane q gets the source index / weight of edge base + q (0 / 1 past the end)
 //                                   and the warp-uniform mask of the edges of the chunk that end a row;
 //   finish_row():                   warp-uniform; folds the slots, runs the row's epilogue and starts the next row.
-template <typename T, int SB, int LPR, class Policy, class LoadChunk, class FinishRow>
-__device__ __forceinline__ void ring_stream(const RingWarp<T, SB, LPR, Policy> &rw, const Policy &pol, float (&st)[Policy::NS], int total,
+template <typename T, int SB, int LPR, class Policy, bool PAD, class LoadChunk, class FinishRow>
+__device__ __forceinline__ void ring_stream(const RingWarp<T, SB, LPR, Policy, PAD> &rw, const Policy &pol, float (&st)[Policy::NS], int total,
                                             LoadChunk load_chunk, FinishRow finish_row) {
   using G = RingGeom<SB, LPR>;
   using Raw = typename SliceRaw<SB>::type;
@@ -197,14 +199,14 @@ __device__ __forceinline__ void ring_stream(const RingWarp<T, SB, LPR, Policy> &
 // SINGLE: every batch is one row (p.batch_rows == 1): the stream is the row and its end is the end of the stream, so
 // there is no bookkeeping of row ends and no metadata spread over the lanes (fewer instructions per row, fewer
 // registers).
-template <typename T, int SB, int LPR, class Policy, bool SINGLE>
+template <typename T, int SB, int LPR, class Policy, bool SINGLE, bool PAD>
 __global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_rows_ring_kernel(StreamParams p, Policy pol) {
   constexpr int NS = Policy::NS;
   extern __shared__ uint4 ring_raw[];
   const int lane = threadIdx.x & 31;
-  RingWarp<T, SB, LPR, Policy> rw;
+  RingWarp<T, SB, LPR, Policy, PAD> rw;
   rw.setup((uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)(threadIdx.x >> 5) * (uint32_t)ring_bytes_per_warp<SB, Policy::HAS_EXTRA>(),
-           p.src, p.src_pitch, lane);
+           p.src, p.src_pitch, p.slices, lane);
   const int slot = rw.slot;
   pol.setup(lane % LPR);
   const int64_t n_rows = p.row_hi - p.row_lo;
@@ -230,7 +232,7 @@ __global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_rows_ring_
       const int32_t owner = Policy::NEEDS_OWNER ? __ldcs(p.owner + p.row_lo + b) : 0;
       float st[NS];
       pol.init(st);
-      pol.begin_row(m.dest, owner);
+      if (rw.active) pol.begin_row(m.dest, owner);
       const int64_t a = m.j0;
       const int total = m.len;
       auto load_chunk = [&](int base, int32_t &idx, float &w, unsigned &ends) {
@@ -240,9 +242,9 @@ __global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_rows_ring_
           if (Policy::WEIGHTED) w = __ldcs(p.weights + a + base + lane);
         }
       };
-      ring_stream<T, SB, LPR, Policy>(rw, pol, st, total, load_chunk, [] {});
+      ring_stream<T, SB, LPR, Policy, PAD>(rw, pol, st, total, load_chunk, [] {});
       rw.fold(pol, st);
-      if (slot == 0) pol.end_row(st, m.dest, owner, m.len);
+      if (slot == 0 && rw.active) pol.end_row(st, m.dest, owner, m.len);
     } else {
     // ---- batch metadata: lane i owns row i of the batch
     const int64_t i = p.row_lo + b * BR + lane;
@@ -290,35 +292,36 @@ __global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_rows_ring_
     float st[NS];
     pol.init(st);
     int cur = 0;  // row of the batch that st belongs to
-    pol.begin_row(__shfl_sync(0xffffffffu, my_dest, 0), Policy::NEEDS_OWNER ? __shfl_sync(0xffffffffu, my_owner, 0) : 0);
+    const int32_t dest0 = __shfl_sync(0xffffffffu, my_dest, 0), owner0 = Policy::NEEDS_OWNER ? __shfl_sync(0xffffffffu, my_owner, 0) : 0;
+    if (rw.active) pol.begin_row(dest0, owner0);
     auto finish_row = [&]() {   // warp-uniform
       rw.fold(pol, st);
       const int32_t dest = __shfl_sync(0xffffffffu, my_dest, cur);
       const int32_t owner = Policy::NEEDS_OWNER ? __shfl_sync(0xffffffffu, my_owner, cur) : 0;
       const int32_t len = __shfl_sync(0xffffffffu, my_len, cur);
-      if (slot == 0) pol.end_row(st, dest, owner, len);
+      if (slot == 0 && rw.active) pol.end_row(st, dest, owner, len);
       ++cur;
       pol.init(st);
       const int32_t nd = __shfl_sync(0xffffffffu, my_dest, cur & 31);
       const int32_t no = Policy::NEEDS_OWNER ? __shfl_sync(0xffffffffu, my_owner, cur & 31) : 0;
-      if (cur < BR && __shfl_sync(0xffffffffu, my_len, cur & 31) > 0) pol.begin_row(nd, no);
+      if (cur < BR && __shfl_sync(0xffffffffu, my_len, cur & 31) > 0 && rw.active) pol.begin_row(nd, no);
     };
-    ring_stream<T, SB, LPR, Policy>(rw, pol, st, total, load_chunk, finish_row);
+    ring_stream<T, SB, LPR, Policy, PAD>(rw, pol, st, total, load_chunk, finish_row);
     }
   }
 }
 
 // ----------------------------------------------------------------------------- very long rows: one CTA each
 // Each warp streams its part of the row through its ring; there is no end of row inside a part.
-template <typename T, int SB, int LPR, class Policy>
+template <typename T, int SB, int LPR, class Policy, bool PAD>
 __global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_cta_ring_kernel(StreamParams p, Policy pol) {
   constexpr int NS = Policy::NS;
   constexpr int WARPS = THREADS / 32;
   extern __shared__ uint4 ring_raw[];
   __shared__ float red[WARPS][LPR][NS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  RingWarp<T, SB, LPR, Policy> rw;
-  rw.setup((uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)warp * (uint32_t)ring_bytes_per_warp<SB, Policy::HAS_EXTRA>(), p.src, p.src_pitch, lane);
+  RingWarp<T, SB, LPR, Policy, PAD> rw;
+  rw.setup((uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)warp * (uint32_t)ring_bytes_per_warp<SB, Policy::HAS_EXTRA>(), p.src, p.src_pitch, p.slices, lane);
   pol.setup(lane % LPR);
 
   for (int64_t i = p.row_lo + blockIdx.x; i < p.row_hi; i += gridDim.x) {
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_cta_ring_k
     const int64_t a = m.j0 + first;
     float st[NS];
     pol.init(st);
-    pol.begin_row(m.dest, owner);
+    if (rw.active) pol.begin_row(m.dest, owner);
     auto load_chunk = [&](int base, int32_t &idx, float &w, unsigned &ends) {
       idx = 0; w = 1.f; ends = 0u;
       if (base + lane < total) {
@@ -339,7 +342,7 @@ __global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_cta_ring_k
         if (Policy::WEIGHTED) w = __ldcs(p.weights + a + base + lane);
       }
     };
-    if (total > 0) ring_stream<T, SB, LPR, Policy>(rw, pol, st, total, load_chunk, [] {});
+    if (total > 0) ring_stream<T, SB, LPR, Policy, PAD>(rw, pol, st, total, load_chunk, [] {});
     rw.fold(pol, st);
     __syncthreads();  // red[] free again
     if (lane < LPR) {
@@ -354,7 +357,7 @@ __global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_cta_ring_k
         for (int k = 0; k < NS; ++k) other[k] = red[w][lane][k];
         pol.merge(st, other);
       }
-      pol.end_row(st, m.dest, owner, m.len);
+      if (rw.active) pol.end_row(st, m.dest, owner, m.len);
     }
   }
 }
