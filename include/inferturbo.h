@@ -88,8 +88,9 @@ typedef enum { IT_ACT_NONE = 0, IT_ACT_RELU = 1, IT_ACT_ELU = 2 } it_act;
  *
  * GAT with edge features (op = GAT, edge_dim > 0): the edge's features enter its attention logit,
  *       e = LeakyReLU_slope( att_src[k] . z_u^k + att_dst[k] . z_v^k + att_edge[k] . e_{v,u} ),
- *   the messages stay z_u.  One fp32 logit term per edge and head (source score + edge share) and the message
- *   row of every edge are materialised in the workspace ([n_edges, heads] fp32 and [n_edges, out_dim] feat_dtype).
+ *   the messages stay z_u.  One fp32 logit term per edge and head (source score + edge share) is materialised in the
+ *   workspace ([n_edges, heads]); shapes that the batched reduce does not take (heads other than 1, 2, 4 or 8, rows
+ *   narrower than 128 bytes) also a copy of the message row of every edge ([n_edges, out_dim] feat_dtype).
  *
  * Learned messages (msg_dim > 0; pooling layers and GCN): the general apply_edge of the Scatter stage (Section
  *   "InferTurbo Abstraction"; M of Eq. (1)) as one dense layer on the source state and the edge's features,

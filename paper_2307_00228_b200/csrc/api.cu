@@ -95,10 +95,11 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
       w.off_partials = take(it_gat_partial_bytes(g, L->out_dim, L->heads));
       w.off_a = take(n * 2 * (size_t)L->heads * 4);  // scores
       w.off_b = take(n * fo * s);                    // Z
-      // edge features in the logits: per edge its message row and one logit term per head
+      // edge features in the logits: per edge one logit term per head (and its message row where the reduce walks copies)
       // ... or, without them, the source scores of every vertex on their own (read per edge at random: half the bytes
       // of the interleaved score rows, and small enough to stay in the L2)
-      w.off_q = take(fe > 0 ? (size_t)g->e * fo * s + it_align_up((size_t)g->e * (size_t)L->heads * 4)
+      w.off_q = take(fe > 0 ? it_align_up((size_t)g->e * (size_t)L->heads * 4) +
+                                  (it_gat_batched(L->feat_dtype, L->heads, L->out_dim / L->heads) ? 0 : (size_t)g->e * fo * s)
                             : (size_t)g->n_src * (size_t)L->heads * 4);
       break;
     case PLAN_DENSE:
@@ -254,10 +255,14 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
     aa.slope = L->leaky_slope; aa.bias = L->bias; aa.act = L->act; aa.dst = out;
     if (L->edge_dim > 0) {
       IT_REQUIRE(L->att_edge != nullptr, IT_ERR_INVALID_ARG, "GAT layer with edge features needs att_edge");
-      void *Zj = c.ws + c.w.off_q;
-      float *sc = reinterpret_cast<float *>(c.ws + c.w.off_q + it_align_up((size_t)g->e * (size_t)L->out_dim * (size_t)it_dtype_size(dt)));
+      // one logit term per edge and head; the batched reduce reads it next to the source rows, the others walk copies of
+      // the rows in edge order
+      const bool batched = it_gat_batched(dt, L->heads, L->out_dim / L->heads);
+      float *sc = reinterpret_cast<float *>(c.ws + c.w.off_q);
+      void *Zj = batched ? nullptr : c.ws + c.w.off_q + it_align_up((size_t)g->e * (size_t)L->heads * 4);
       IT_TRY(it_launch_gat_edge_rows(g, dt, L->out_dim, L->heads, table, scores, L->att_edge, Zj, sc, c.st));
-      aa.z = Zj; aa.per_edge_rows = 1; aa.src_scores = sc;
+      if (!batched) { aa.z = Zj; aa.per_edge_rows = 1; }
+      aa.per_edge_scores = 1; aa.src_scores = sc;
     } else {
       float *dense = reinterpret_cast<float *>(c.ws + c.w.off_q);
       IT_TRY(it_launch_compact_scores(g->n_src, L->heads, scores, dense, c.st));

@@ -108,17 +108,18 @@ static inline size_t it_align_up(size_t x, size_t a = 256) { return (x + a - 1) 
 // a handful of instructions where expm1f costs a few dozen in the end-of-row code of every short row); close to
 // zero, where that difference cancels, the three-term series x + x^2/2 + x^3/6 takes over (relative error below
 // 2e-6 at the switch point x = -1/32 and falling towards 0), so the result is relatively accurate everywhere.
-#ifndef IT_FAST_ELU
-#define IT_FAST_ELU 1
-#endif
 #ifdef __CUDACC__
+// e^x by the hardware's 2^x; results below 2^-126 are flushed to zero (an attention weight that small against the largest
+// one, which is 1, or an e^x of which 1 is subtracted).  Without the flush the compiler guards every exponential with
+// three more instructions.
+__device__ __forceinline__ float it_exp(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * 1.4426950408889634f));
+  return r;
+}
 __device__ __forceinline__ float it_elu(float x) {
-#if IT_FAST_ELU
   const float series = x * fmaf(x, fmaf(x, 1.f / 6.f, 0.5f), 1.f);
-  return x > 0.f ? x : (x > -0.03125f ? series : __expf(x) - 1.f);
-#else
-  return x > 0.f ? x : expm1f(x);
-#endif
+  return x > 0.f ? x : (x > -0.03125f ? series : it_exp(x) - 1.f);
 }
 #endif
 static inline int it_dtype_size(it_dtype t) { return t == IT_F32 ? 4 : 2; }
@@ -155,6 +156,21 @@ struct it_gather_args {
 };
 it_status it_launch_gather(const it_gather_args &a, cudaStream_t stream);
 
+// Rows [row_lo, row_hi) of the bucket-ordered list all get the same value: what a vertex without in-edges ends up with.
+struct it_const_rows_args {
+  const it_graph *g;
+  int64_t row_lo, row_hi;
+  void *dst;
+  int64_t pitch;           // bytes from one row of dst to the next
+  int dim;                 // entries written
+  it_dtype dtype;          // of dst
+  float value;             // every entry, or
+  const float *bias;       // act(bias[i]) when has_bias (NULL: act(0))
+  int has_bias;
+  it_act act;
+};
+it_status it_launch_const_rows(const it_const_rows_args &a, int kid, double bytes, cudaStream_t stream);
+
 // ----------------------------------------------------------------------------- gat.cu
 struct it_gat_args {
   const it_graph *g;
@@ -163,9 +179,10 @@ struct it_gat_args {
   const void *z;          // [n, heads*head_dim] messages
   const float *scores;    // [n_src, 2*heads]: source scores of the vertex, then its destination scores
   const float *scores_dst;   // the same layout, row v = local destination v (scores + first_vertex * 2*heads for a part; NULL: scores)
-  int per_edge_rows;      // 1: z is [n_edges, dim] and src_scores [n_edges, heads], row j belonging to edge j (edge features in the logits)
+  int per_edge_rows;      // 1: z is [n_edges, dim], row j belonging to edge j
+  int per_edge_scores;    // 1: src_scores is [n_edges, heads], row j belonging to edge j (edge features in the logits)
   const float *src_scores;   // [rows, heads], dense: the source-side logit term that is read per edge (row = source vertex, or the
-                             // edge itself with per_edge_rows); NULL: the first half of the rows of `scores`
+                             // edge itself with per_edge_scores); NULL: the first half of the rows of `scores`
   float *partials;        // it_gat_partial_bytes() of fp32 scratch for the groups of split vertices (may be NULL if none)
   int *counters;          // IT_MAX_BUCKETS device words of scratch from which warps claim their batches (NULL: fixed strides)
   float slope;
@@ -174,6 +191,9 @@ struct it_gat_args {
   void *dst;              // [n, heads*head_dim]
 };
 it_status it_launch_gat(const it_gat_args &a, cudaStream_t stream);
+// Whether the reduce takes this shape with the weights of many edges at a time (then per-edge logit terms need no copies of
+// the source rows in edge order).
+bool it_gat_batched(it_dtype dtype, int heads, int head_dim);
 size_t it_gat_partial_bytes(const it_graph *g, int dim, int heads);
 
 // ----------------------------------------------------------------------------- apply.cu
@@ -234,7 +254,7 @@ it_status it_launch_gemm2_tc(const it_gemm2_args &a, const void *B1, const void 
 // Learned messages, edge by edge: M[j, :] = act(P[indices[j], :] + M[j, :]) in place (M arrives holding the per-edge
 // part Q), rows of `dim` elements of `dtype` (a multiple of 16 bytes).
 it_status it_launch_edge_messages(const it_graph *g, it_dtype dtype, int dim, const void *P, void *M, it_act act, cudaStream_t stream);
-// GAT with edge features: Zj[j, :] = Z[indices[j], :] and sc[j, h] = scores[indices[j], h] + att_edge[h, :] . ef[j, :].
+// GAT with edge features: Zj[j, :] = Z[indices[j], :] (unless Zj is NULL) and sc[j, h] = scores[indices[j], h] + att_edge[h, :] . ef[j, :].
 it_status it_launch_gat_edge_rows(const it_graph *g, it_dtype dtype, int dim, int heads, const void *Z, const float *scores,
                                   const float *att_edge, void *Zj, float *sc, cudaStream_t stream);
 // dense[v, :] = scores[v, 0:heads]: the source scores on their own, 16 bytes per vertex for 4 heads instead of a 32-byte

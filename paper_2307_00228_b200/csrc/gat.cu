@@ -30,7 +30,13 @@ struct GatPolicy {
   // per-thread
   int col, head;
   float s_dst;
+  uint32_t bias_s;   // shared-window address of a copy of the bias (0: none; read it from global memory)
 
+  bool empty_rows(it_const_rows_args &a) const {
+    a.dst = dst; a.dim = dim; a.dtype = sizeof(T) == 4 ? IT_F32 : IT_BF16; a.pitch = (int64_t)dim * (int)sizeof(T);
+    a.value = 0.f; a.has_bias = 1; a.bias = bias; a.act = (it_act)act;
+    return true;
+  }
   __device__ __forceinline__ void setup(int t) { col = t * VEC; head = col / head_dim; s_dst = 0.f; }
   __device__ __forceinline__ void init(float (&st)[NS]) const {
 #pragma unroll
@@ -90,10 +96,30 @@ struct GatPolicy {
     const float inv = st[VEC + 1] > 0.f ? 1.f / st[VEC + 1] : 0.f;
     float o[VEC];
 #pragma unroll
-    for (int i = 0; i < VEC; ++i) o[i] = act_apply(st[i] * inv + (bias ? __ldg(bias + col + i) : 0.f), act);
+    for (int i = 0; i < VEC; ++i) o[i] = 0.f;
+    if (bias_s != 0) {
+#pragma unroll
+      for (int i = 0; i < VEC; i += 4) {   // (only set for 16-byte slices: four columns at a time)
+        const uint4 b = lds_slice<16>(bias_s + (uint32_t)(col + i) * 4);
+        o[i] = __uint_as_float(b.x);
+        if (i + 3 < VEC) { o[i + 1] = __uint_as_float(b.y); o[i + 2] = __uint_as_float(b.z); o[i + 3] = __uint_as_float(b.w); }
+      }
+    } else if (bias) {
+#pragma unroll
+      for (int i = 0; i < VEC; ++i) o[i] = __ldg(bias + col + i);
+    }
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) o[i] = fmaf(st[i], inv, o[i]);
+    act_slice<VEC>(o, act);
     Slice::store(reinterpret_cast<T *>(dst) + (int64_t)dest * dim + col, o);
   }
 };
+
+}  // namespace
+
+#include "gat_rows.cuh"
+
+namespace {
 
 // Merge the partial states of every split vertex in group order; one warp per vertex.
 struct GatCombineParams {
@@ -144,26 +170,57 @@ __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p
   }
 }
 
-template <typename T, int SB, int LPR>
-it_status launch_gat_lpr(const it_gat_args &a, StreamParams sp, int64_t bound_lo, int64_t bound_hi, cudaStream_t st) {
+template <typename T, int SB>
+GatPolicy<T, SB> make_policy(const it_gat_args &a) {
   GatPolicy<T, SB> pol;
   pol.scores = a.src_scores ? a.src_scores : a.scores; pol.src_stride = a.src_scores ? a.heads : 2 * a.heads;
   pol.scores_dst = a.scores_dst ? a.scores_dst : a.scores; pol.bias = a.bias; pol.dst = a.dst; pol.partials = a.partials;
   pol.dim = a.heads * a.head_dim; pol.heads = a.heads; pol.head_dim = a.head_dim; pol.act = a.act; pol.slope = a.slope;
-  pol.col = 0; pol.head = 0; pol.s_dst = 0.f;
+  pol.col = 0; pol.head = 0; pol.s_dst = 0.f; pol.bias_s = 0;
+  return pol;
+}
+
+// algorithmic bytes: per edge the index, one source score per head and one source row; per row its metadata, owner,
+// destination scores and one output row
+auto gat_bytes(const it_gat_args &a) {
   const it_graph *g = a.g;
-  // algorithmic bytes: per edge the index, one source score per head and one source row; per row
-  // its metadata, owner, destination scores and one output row
-  const double row_bytes = (double)pol.dim * sizeof(T);
   const int heads = a.heads;
-  auto bytes_of = [=](int b, int64_t rows) {
+  const double row_bytes = (double)heads * a.head_dim * it_dtype_size(a.dtype);
+  return [=](int b, int64_t rows) {
     return (double)g->h_bucket_edges[b] * (4.0 + 4.0 * heads + row_bytes) + (double)rows * (20.0 + 4.0 * heads + row_bytes);
   };
-  return launch_buckets<T, SB, LPR, false>(g, sp, pol, bytes_of, IT_K_GAT_CTA, IT_K_GAT_FLAT, IT_K_GAT_EMPTY, bound_lo, bound_hi, a.counters, st);
+}
+
+template <typename T, int SB, int LPR>
+it_status launch_gat_lpr(const it_gat_args &a, StreamParams sp, int64_t bound_lo, int64_t bound_hi, cudaStream_t st) {
+  return launch_buckets<T, SB, LPR, false>(a.g, sp, make_policy<T, SB>(a), gat_bytes(a), IT_K_GAT_CTA, IT_K_GAT_FLAT, IT_K_GAT_EMPTY, bound_lo, bound_hi,
+                                           a.counters, st);
+}
+
+// f.template operator()<LPR, H>() for the shapes that the batched kernels take
+template <class F>
+it_status dispatch_batched(int row_bytes, int heads, F f) {
+  auto by_heads = [&]<int LPR>() -> it_status {
+    switch (heads) {
+      case 1: return f.template operator()<LPR, 1>();
+      case 2: return f.template operator()<LPR, 2>();
+      case 4: return f.template operator()<LPR, 4>();
+      default: return f.template operator()<LPR, 8>();
+    }
+  };
+  switch (row_bytes) {
+    case 512: return by_heads.template operator()<32>();
+    case 256: return by_heads.template operator()<16>();
+    default: return by_heads.template operator()<8>();
+  }
 }
 
 template <typename T>
 it_status launch_gat(const it_gat_args &a, StreamParams sp, cudaStream_t st) {
+  if (!a.per_edge_rows && a.counters && a.src_scores && it_gat_batched(a.dtype, a.heads, a.head_dim))
+    return dispatch_batched(a.heads * a.head_dim * (int)sizeof(T), a.heads, [&]<int LPR, int H>() {
+      return launch_gat_rows<T, LPR, H>(a, sp, make_policy<T, 16>(a), gat_bytes(a), st);
+    });
   // 16-byte slices as long as one never straddles two heads
   const bool wide = (a.head_dim * (int)sizeof(T)) % 16 == 0;
   const int row_bytes = a.heads * a.head_dim * (int)sizeof(T);
@@ -181,6 +238,11 @@ it_status launch_gat(const it_gat_args &a, StreamParams sp, cudaStream_t st) {
 }
 
 }  // namespace
+
+bool it_gat_batched(it_dtype dtype, int heads, int head_dim) {
+  const int es = it_dtype_size(dtype), row = heads * head_dim * es;
+  return (heads == 1 || heads == 2 || heads == 4 || heads == 8) && (head_dim * es) % 16 == 0 && (row == 128 || row == 256 || row == 512);
+}
 
 size_t it_gat_partial_bytes(const it_graph *g, int dim, int heads) {
   return (size_t)g->n_partial_rows * gat_partial_stride(dim, heads) * sizeof(float);

@@ -1,0 +1,403 @@
+// The GAT reduce with the attention weights of many edges computed at once, for rows of 128 to 512 bytes in 16-byte
+// slices (bf16 128 or fp32 64 columns: 256 bytes) and 1, 2, 4 or 8 heads.
+//
+// The running-softmax policy of gat.cu works edge by edge: every lane of a row recomputes the logit and the exponential
+// of its head and rescales its accumulators at each edge, about 35 instructions per edge and slice, which kept the
+// kernels at 72-79 % of their issue slots with DRAM half idle.  Here a step covers E edges at once (32 of a warp's row, 8 of a
+// lane group's): the (edge, head) pairs are spread over the lanes, one maximum per head and step is taken by
+// shuffles, each pair's weight exp(e - m) is computed once, accumulators are rescaled once per step, and an edge then
+// costs its slice's multiply-adds.  The state is the same (max, sum, weighted accumulator), so partial states of split
+// vertices merge as before.  Measured on 1.25M vertices, 25M edges, bf16 4 heads of 32 (256-byte rows), before -> after: rows
+// of at most 8 edges 252 -> 194 us, 9..32 edges 188 -> 157, 33..1024 edges 435 -> 418, longer 441 -> 400 (DRAM at 0.8 of its
+// peak, as a copy reaches); with edge features in the logits the source rows are no longer copied in edge order (8M edges,
+// fp32 64 columns: 1.61 -> 0.83 ms for the layer).
+//
+// Included by gat.cu.
+#pragma once
+
+#include "stream.cuh"
+
+namespace {
+
+using namespace it_stream;
+
+struct GatParams {
+  const float *__restrict__ scores;       // source-side logit term: [n_src, H], or [n_edges, H] when per_edge
+  const float *__restrict__ scores_dst;   // [local destinations, 2H]: destination scores in the second half
+  int per_edge;                           // the term belongs to the edge (edge features in the logits), not to its source
+  float slope;
+  int head_dim;
+};
+
+// Accumulators of one slice plus the sum of the weights.  All states of one warp's row share their maximum, so folding
+// slots is a plain sum.
+template <typename T>
+struct GatAcc {
+  using Slice = RowSlice<T, 16>;
+  static constexpr int VEC = Slice::VEC, NS = VEC + 1;
+  static constexpr bool HAS_EXTRA = false, WEIGHTED = false;
+  __device__ __forceinline__ const float *extra_ptr(uint32_t) const { return nullptr; }
+  __device__ __forceinline__ void init(float (&st)[NS]) const {
+#pragma unroll
+    for (int k = 0; k < NS; ++k) st[k] = 0.f;
+  }
+  __device__ __forceinline__ void edge(float (&st)[NS], const uint4 &raw, float w) const {
+    float f[VEC];
+    Slice::unpack(raw, f);
+#pragma unroll
+    for (int k = 0; k < VEC; k += 2) fma_f32x2(st[k], st[k + 1], w, f[k], f[k + 1]);
+    st[VEC] += w;
+  }
+  __device__ __forceinline__ void scale(float (&st)[NS], float s) const {
+#pragma unroll
+    for (int k = 0; k < NS; ++k) st[k] *= s;
+  }
+  __device__ __forceinline__ void merge(float (&st)[NS], const float (&o)[NS]) const {
+#pragma unroll
+    for (int k = 0; k < NS; ++k) st[k] += o[k];
+  }
+};
+
+// The bias in shared memory, for the end of a row (its address need not be 16-byte aligned in global memory).
+template <class Policy>
+__device__ __forceinline__ void stage_bias(Policy &pol, float (&buf)[256]) {
+  for (int i = threadIdx.x; i < pol.dim; i += THREADS) buf[i] = pol.bias ? pol.bias[i] : 0.f;
+  __syncthreads();
+  pol.bias_s = (uint32_t)__cvta_generic_to_shared(&buf[0]);
+}
+
+__device__ __forceinline__ float leaky(float x, float slope) { return x > 0.f ? x : slope * x; }
+
+// ----------------------------------------------------------------------------- one warp per row (or per part of a row)
+// Lane = (edge el = lane / H, head hl = lane % H) for the logits; pair i of a lane is edge el + i * 32 / H of the chunk.
+template <typename T, int LPR, int H>
+struct GatWarp {
+  static constexpr int EP = 32 / H;   // edges covered by one pair per lane
+  const StreamParams &p;
+  const GatParams &q;
+  const int lane, hl, el, hc;         // hc: head of the lane's slice
+  const uint32_t pw;                  // shared-window address of this warp's weights [32][H]
+  float x_c[H], x_n[H];               // logit terms of the current / the next chunk
+  float sd_c, sd_n;                   // destination scores of their rows
+  float m;                            // running maximum of head hl
+  GatAcc<T> acc;
+  float st[GatAcc<T>::NS];
+
+  __device__ __forceinline__ GatWarp(const StreamParams &p_, const GatParams &q_, int lane_, uint32_t pw_)
+      : p(p_), q(q_), lane(lane_), hl(lane_ % H), el(lane_ / H), hc((lane_ % LPR) * GatAcc<T>::VEC / q_.head_dim), pw(pw_) {
+    sd_c = sd_n = 0.f; m = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < H; ++i) x_c[i] = x_n[i] = 0.f;
+    acc.init(st);
+  }
+  // the ids of chunk c have landed: fetch its logit terms (into the "next" registers)
+  __device__ __forceinline__ void ahead(const Chunk &c) {
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const int e = el + i * EP;
+      const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, c.idx, e);
+      if (e < c.cnt) x_n[i] = __ldg(q.scores + (q.per_edge ? (uint64_t)(c.j + e) : (uint64_t)s) * H + hl);
+    }
+    sd_n = __ldg(q.scores_dst + (int64_t)c.owner * (2 * H) + H + hl);
+  }
+  // chunk c becomes the current one: its attention weights
+  __device__ __forceinline__ void begin(const Chunk &c, bool first) {
+    sd_c = sd_n;
+    float mr = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      x_c[i] = el + i * EP < c.cnt ? leaky(x_n[i] + sd_c, q.slope) : -INFINITY;
+      mr = fmaxf(mr, x_c[i]);
+    }
+#pragma unroll
+    for (int o = H; o < 32; o <<= 1) mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
+    if (first) { m = -INFINITY; acc.init(st); }
+    const float m_new = fmaxf(m, mr);
+    const float s = __shfl_sync(0xffffffffu, it_exp(m - m_new), hc);   // exp(-inf) = 0 for the first chunk of a row
+    if (!first) acc.scale(st, s);
+    m = m_new;
+    __syncwarp();   // the previous chunk's weights have been read
+#pragma unroll
+    for (int i = 0; i < H; ++i)
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(pw + (uint32_t)((lane + 32 * i) * 4)), "f"(it_exp(x_c[i] - m)) : "memory");
+    __syncwarp();
+  }
+  __device__ __forceinline__ float weight(int k) const { return lds_f32(pw + (uint32_t)((k * H + hc) * 4)); }
+};
+
+#ifndef IT_GAT_CHUNK_BLOCKS
+#define IT_GAT_CHUNK_BLOCKS 3   // resident CTAs per SM: at four the 64 registers a thread gets spill (measured: 3 to 5 % more time)
+#endif
+template <int H> constexpr int gat_bytes_per_warp() { return ring_bytes_per_warp<16, false>() + 32 * H * 4; }
+
+template <typename T, int LPR, int H>
+__global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol) {
+  extern __shared__ uint4 ring_raw[];
+  const int lane = threadIdx.x & 31;
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)(threadIdx.x >> 5) * (uint32_t)gat_bytes_per_warp<H>();
+  RingWarp<T, 16, LPR, GatAcc<T>, false> rw;
+  rw.setup(base, p.src, p.src_pitch, p.slices, lane);
+  pol.setup(lane % LPR);
+  __shared__ float bias_buf[256];
+  stage_bias(pol, bias_buf);
+  GatWarp<T, LPR, H> gw(p, q, lane, base + ring_bytes_per_warp<16, false>());
+  ChunkCursor<false, true> cur(p, lane);
+  chunk_walk<LPR, true>(rw, gw.acc, cur, [&](Chunk &c) { gw.ahead(c); }, [&](const Chunk &c, bool first) { gw.begin(c, first); },
+      [&](int k, const uint4 &raw, bool valid) {
+        const float w = gw.weight(k);
+        if (valid) gw.acc.edge(gw.st, raw, w);
+      },
+      [&](const Chunk &c) {
+        rw.fold(gw.acc, gw.st);
+        const float mh = __shfl_sync(0xffffffffu, gw.m, gw.hc);
+        float full[GatPolicy<T, 16>::NS];
+#pragma unroll
+        for (int k = 0; k < GatAcc<T>::VEC; ++k) full[k] = gw.st[k];
+        full[GatAcc<T>::VEC] = mh;
+        full[GatAcc<T>::VEC + 1] = gw.st[GatAcc<T>::VEC];
+        if (rw.slot == 0) pol.end_row(full, c.dest, 0, 0);
+      });
+}
+
+// Very long rows: one CTA each, every warp a contiguous part; the warps' states are merged in warp order.
+template <typename T, int LPR, int H>
+__global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) gat_cta_chunk_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol) {
+  constexpr int WARPS = THREADS / 32, NS = GatPolicy<T, 16>::NS;
+  extern __shared__ uint4 ring_raw[];
+  __shared__ float red[WARPS][LPR][NS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)warp * (uint32_t)gat_bytes_per_warp<H>();
+  RingWarp<T, 16, LPR, GatAcc<T>, false> rw;
+  rw.setup(base, p.src, p.src_pitch, p.slices, lane);
+  pol.setup(lane % LPR);
+  __shared__ float bias_buf[256];
+  stage_bias(pol, bias_buf);
+  for (int64_t i = p.row_lo + blockIdx.x; i < p.row_hi; i += gridDim.x) {
+    const it_row_meta mt = load_meta(p.meta + i);
+    const int32_t owner = __ldcs(p.owner + i);
+    const int part = (mt.len + WARPS - 1) / WARPS;
+    const int first = warp * part < mt.len ? warp * part : mt.len;
+    const int total = (mt.len - first) < part ? (mt.len - first) : part;
+    GatWarp<T, LPR, H> gw(p, q, lane, base + ring_bytes_per_warp<16, false>());
+    PartCursor<false> cur(p, lane, mt.j0 + first, total, mt.dest, owner);
+    chunk_walk<LPR, true>(rw, gw.acc, cur, [&](Chunk &c) { gw.ahead(c); }, [&](const Chunk &c, bool f) { gw.begin(c, f); },
+        [&](int k, const uint4 &raw, bool valid) {
+          const float w = gw.weight(k);
+          if (valid) gw.acc.edge(gw.st, raw, w);
+        },
+        [](const Chunk &) {});
+    rw.fold(gw.acc, gw.st);
+    const float mh = __shfl_sync(0xffffffffu, gw.m, gw.hc);
+    float full[NS];
+#pragma unroll
+    for (int k = 0; k < GatAcc<T>::VEC; ++k) full[k] = gw.st[k];
+    full[NS - 2] = mh;
+    full[NS - 1] = gw.st[GatAcc<T>::VEC];
+    __syncthreads();   // red[] free again
+    if (lane < LPR) {
+#pragma unroll
+      for (int k = 0; k < NS; ++k) red[warp][lane][k] = full[k];
+    }
+    __syncthreads();
+    if (warp == 0 && lane < LPR) {
+      for (int w = 1; w < WARPS; ++w) {
+        float other[NS];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) other[k] = red[w][lane][k];
+        pol.merge(full, other);
+      }
+      pol.end_row(full, mt.dest, owner, mt.len);
+    }
+  }
+}
+
+// ----------------------------------------------------------------------------- short rows: one lane group each
+// Rows of at most a few dozen edges, 128- and 256-byte rows: a group of LPR lanes owns a row and walks it in rounds of up
+// to E = 8 edges; the groups of a warp run in lockstep, a round as long as its longest row.  While the rows of one round are
+// reduced, the source rows and logit terms of the next round are in flight (two staging buffers in shared memory), the ids
+// of the round after it, and the records of the rows after that.
+#ifndef IT_GAT_SHORT_BLOCKS
+#define IT_GAT_SHORT_BLOCKS 3   // resident CTAs per SM: 64 KB of staging each
+#endif
+template <typename T, int LPR, int H>
+__global__ void __launch_bounds__(THREADS, IT_GAT_SHORT_BLOCKS) gat_short_rows_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol) {
+  using Acc = GatAcc<T>;
+  constexpr int E = IT_SHORT_EDGES;
+  constexpr int EP = LPR / H;                            // edges covered by one pair per lane
+  constexpr int PP = E > EP ? E / EP : 1;                // (edge, head) pairs per lane
+  static_assert(H <= LPR && E <= LPR, "a group holds its pairs and its ids");
+  extern __shared__ uint4 short_buf[];                   // [2][E][THREADS]
+  const int lane = threadIdx.x & 31, t = lane % LPR, gbase = lane - t;
+  const int hl = t % H, el = t / H;
+  pol.setup(t);
+  __shared__ float bias_buf[256];
+  stage_bias(pol, bias_buf);
+  const int hc = t * Acc::VEC / q.head_dim;              // head of the lane's slice
+  const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
+  const uint32_t ROWB = p.src_pitch;
+  constexpr uint32_t SLOT = THREADS * 16, BUF = E * SLOT;
+  uint32_t buf = (uint32_t)__cvta_generic_to_shared(&short_buf[threadIdx.x]), other = buf + BUF;
+  const int64_t sweep = (int64_t)gridDim.x * (THREADS / LPR);
+
+  struct Row { int64_t j0; int len, most, dest, owner; float sd; };   // most: longest row of the warp's groups (0: no rows left)
+  auto load_row = [&](int64_t i0, Row &r) {
+    r.j0 = 0; r.len = 0; r.dest = 0; r.owner = 0;
+    const int64_t i = i0 + lane / LPR;
+    if (i < p.row_hi) {
+      const it_row_meta m = load_meta(p.meta + i);
+      r.j0 = m.j0; r.len = m.len; r.dest = m.dest;
+      r.owner = __ldcs(p.owner + i);
+    }
+  };
+  auto finish_row = [&](Row &r) {   // the record has landed: what hangs on it
+    r.most = __reduce_max_sync(0xffffffffu, r.len);
+    r.sd = __ldg(q.scores_dst + (int64_t)r.owner * (2 * H) + H + hl);   // owner 0 for a missing row: read, not used
+  };
+  auto load_ids = [&](const Row &r, int k) -> int32_t {
+    if (t < E && k + t < r.len) return p.indices ? __ldcs(p.indices + r.j0 + k + t) : (int32_t)(r.j0 + k + t);
+    return 0;
+  };
+  // the source rows and logit terms of edges [k, k + E) of row r, whose ids are in idx
+  auto issue = [&](const Row &r, int k, int32_t idx, uint32_t d, float (&x)[PP]) {
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+      if (k + u >= r.most) break;   // warp-uniform
+      const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx, gbase + u);
+      if (k + u < r.len) cp_async_slice<16>(d + (uint32_t)u * SLOT, my_src + (uint64_t)s * ROWB);
+    }
+    cp_async_commit();
+#pragma unroll
+    for (int u = 0; u < PP; ++u) {
+      const int e = el + u * EP;
+      const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx, gbase + (e & (E - 1)));
+      x[u] = -INFINITY;
+      if (e < E && k + e < r.len) x[u] = __ldg(q.scores + (q.per_edge ? (uint64_t)(r.j0 + k + e) : (uint64_t)s) * H + hl);
+    }
+  };
+
+  int64_t i0 = p.row_lo + (int64_t)blockIdx.x * (THREADS / LPR) + (threadIdx.x >> 5) * (32 / LPR);   // warp-uniform
+  Row r0, r1, r2;
+  load_row(i0, r0); load_row(i0 + sweep, r1); load_row(i0 + 2 * sweep, r2);
+  finish_row(r0);
+  if (r0.most == 0) return;   // warp-uniform
+  finish_row(r1);
+  float x_a[PP], x_b[PP];
+  int32_t idx_b = load_ids(r0, 0);
+  issue(r0, 0, idx_b, buf, x_a);
+  idx_b = r0.most > E ? load_ids(r0, E) : load_ids(r1, 0);
+  Acc acc;
+  float st[Acc::NS];
+  for (; r0.most > 0; i0 += sweep) {
+    Row r3;
+    load_row(i0 + 3 * sweep, r3);
+    finish_row(r2);
+    float m = -INFINITY;
+    acc.init(st);
+    for (int k0 = 0; k0 < r0.most; k0 += E) {
+      // the next round, and the ids of the one after it
+      if (k0 + E < r0.most) issue(r0, k0 + E, idx_b, other, x_b);
+      else issue(r1, 0, idx_b, other, x_b);
+      if (k0 + 2 * E < r0.most) idx_b = load_ids(r0, k0 + 2 * E);
+      else if (k0 + E < r0.most) idx_b = load_ids(r1, 0);
+      else idx_b = r1.most > E ? load_ids(r1, E) : load_ids(r2, 0);
+      // this round: the weights ...
+      float mr = -INFINITY;
+#pragma unroll
+      for (int u = 0; u < PP; ++u) {
+        x_a[u] = leaky(x_a[u] + r0.sd, q.slope);   // -inf stays -inf for a pair without an edge
+        mr = fmaxf(mr, x_a[u]);
+      }
+#pragma unroll
+      for (int o = H; o < LPR; o <<= 1) mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
+      const float m_new = fmaxf(m, mr);
+      if (k0 > 0) {   // rows whose edges are used up: m_new = m, a factor of 1
+        const float s = __shfl_sync(0xffffffffu, it_exp(m - m_new), gbase + hc);
+        acc.scale(st, s);
+      }
+      m = m_new;
+#pragma unroll
+      for (int u = 0; u < PP; ++u) x_a[u] = it_exp(x_a[u] - m);
+      // ... and the slices
+      cp_async_wait<1>();
+#pragma unroll
+      for (int u = 0; u < E; ++u) {
+        if (k0 + u >= r0.most) break;
+        const float w = __shfl_sync(0xffffffffu, x_a[u / EP], gbase + (u % EP) * H + hc);
+        if (k0 + u < r0.len) acc.edge(st, lds_slice<16>(buf + (uint32_t)u * SLOT), w);
+      }
+#pragma unroll
+      for (int u = 0; u < PP; ++u) x_a[u] = x_b[u];
+      const uint32_t sw = buf; buf = other; other = sw;
+    }
+    const float mh = __shfl_sync(0xffffffffu, m, gbase + hc);
+    if (r0.len > 0) {
+      float full[GatPolicy<T, 16>::NS];
+#pragma unroll
+      for (int k = 0; k < Acc::VEC; ++k) full[k] = st[k];
+      full[Acc::VEC] = mh;
+      full[Acc::VEC + 1] = st[Acc::VEC];
+      pol.end_row(full, r0.dest, 0, 0);
+    }
+    r0 = r1; r1 = r2; r2 = r3;
+  }
+  cp_async_wait<0>();
+}
+
+// ----------------------------------------------------------------------------- launches
+template <typename T, int LPR, int H, class BytesF>
+it_status launch_gat_rows(const it_gat_args &a, StreamParams p, const GatPolicy<T, 16> &pol, BytesF bytes_of, cudaStream_t st) {
+  const it_graph *g = a.g;
+  GatParams q;
+  q.scores = pol.scores; q.scores_dst = pol.scores_dst; q.per_edge = a.per_edge_scores; q.slope = pol.slope; q.head_dim = pol.head_dim;
+  p.slices = LPR;
+  if (a.counters) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, IT_MAX_BUCKETS * sizeof(int), st));
+  bool chunked = false;
+  for (int b = g->n_buckets - 1; b >= 0; --b) {
+    const int64_t lo = g->h_bucket_offsets[b], hi = g->h_bucket_offsets[b + 1], bound = g->bucket_bounds[b];
+    if (hi <= lo) continue;
+    p.row_lo = lo; p.row_hi = hi;
+    const int64_t rows = hi - lo;
+    const double bytes = bytes_of(b, rows);
+    constexpr int smem = (THREADS / 32) * gat_bytes_per_warp<H>();
+    if (bound == 0) {
+      it_const_rows_args cr;
+      pol.empty_rows(cr);
+      cr.g = g; cr.row_lo = lo; cr.row_hi = hi;
+      IT_TRY(it_launch_const_rows(cr, IT_K_GAT_EMPTY, bytes, st));
+    } else if (bound > IT_GATHER_CTA_ABOVE) {
+      static std::atomic<uint64_t> configured{0};
+      IT_TRY(allow_dynamic_smem(gat_cta_chunk_kernel<T, LPR, H>, smem, configured));
+      const unsigned blocks = (unsigned)(rows < (1 << 20) ? rows : (1 << 20));
+      IT_LAUNCH(IT_K_GAT_CTA, bytes, 0, st, gat_cta_chunk_kernel<T, LPR, H><<<blocks, THREADS, smem, st>>>(p, q, pol));
+    } else if (LPR <= 16 && bound <= IT_SHORT_BELOW) {
+      if constexpr (LPR <= 16) {
+        constexpr int sbytes = 2 * IT_SHORT_EDGES * THREADS * 16;
+        static std::atomic<uint64_t> configured{0};
+        IT_TRY(allow_dynamic_smem(gat_short_rows_kernel<T, LPR, H>, sbytes, configured));
+        const int64_t want = (rows + (THREADS / LPR) - 1) / (THREADS / LPR), most = (int64_t)g->num_sms * IT_GAT_SHORT_BLOCKS;
+        const unsigned blocks = (unsigned)(want < most ? want : most);
+        IT_LAUNCH(IT_K_GAT_FLAT, bytes, 0, st, gat_short_rows_kernel<T, LPR, H><<<blocks, THREADS, sbytes, st>>>(p, q, pol));
+      }
+    } else {   // one warp per row: every such bucket in one launch (they are neighbours in the row list), longest rows first
+      if (chunked) continue;
+      chunked = true;
+      double all = bytes;
+      int b0 = b;
+      while (b0 > 0 && g->bucket_bounds[b0 - 1] > (LPR <= 16 ? IT_SHORT_BELOW : 0)) {
+        --b0;
+        all += bytes_of(b0, g->h_bucket_offsets[b0 + 1] - g->h_bucket_offsets[b0]);
+      }
+      p.row_lo = g->h_bucket_offsets[b0];
+      static std::atomic<uint64_t> configured{0};
+      IT_TRY(allow_dynamic_smem(gat_rows_chunk_kernel<T, LPR, H>, smem, configured));
+      p.counter = a.counters + b;
+      const unsigned blocks = chunk_grid(hi - p.row_lo, (int64_t)g->num_sms * IT_GAT_CHUNK_BLOCKS, &p.claim);
+      IT_LAUNCH(IT_K_GAT_FLAT, all, 0, st, gat_rows_chunk_kernel<T, LPR, H><<<blocks, THREADS, smem, st>>>(p, q, pol));
+      p.counter = nullptr;
+    }
+  }
+  IT_CUDA_TRY(cudaGetLastError());
+  return IT_OK;
+}
+
+}  // namespace

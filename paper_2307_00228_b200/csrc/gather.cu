@@ -89,7 +89,68 @@ __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p
   }
 }
 
+// ----------------------------------------------------------------------------- rows without edges
+// The row is built once per block in shared memory; a warp takes 32 rows (their destinations with one coalesced load) and
+// writes them 16 bytes per lane.  Bound by the writes: per-row kernels waited for each record before its row's store
+// (8M vertices, 256-byte rows: 340 -> 255 us; 256-byte GAT rows of 615k vertices 82 -> 22 us).
+struct ConstRowsParams {
+  const it_row_meta *__restrict__ meta;
+  int64_t lo, hi;
+  char *dst;
+  int64_t pitch;
+  int slices, dim, bf16, has_bias, act;   // slices: 16-byte pieces of a row
+  float value;
+  const float *__restrict__ bias;
+};
+
+__global__ void __launch_bounds__(GATHER_THREADS) const_rows_kernel(ConstRowsParams p) {
+  __shared__ uint4 row[128];   // rows of up to 512 entries
+  for (int s = threadIdx.x; s < p.slices; s += GATHER_THREADS) {
+    const int per = p.bf16 ? 8 : 4;
+    float v[8];
+    for (int k = 0; k < 8; ++k) v[k] = p.has_bias ? act_apply(p.bias && k < per ? p.bias[s * per + k] : 0.f, p.act) : p.value;
+    if (p.bf16) {
+      uint32_t w[4];
+      for (int k = 0; k < 4; ++k) {
+        __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+        w[k] = *reinterpret_cast<uint32_t *>(&h);
+      }
+      row[s] = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+      row[s] = make_uint4(__float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
+    }
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int step_r = 32 / p.slices, step_s = 32 % p.slices;
+  for (int64_t b = p.lo + ((int64_t)blockIdx.x * (GATHER_THREADS / 32) + (threadIdx.x >> 5)) * 32; b < p.hi;
+       b += (int64_t)gridDim.x * GATHER_THREADS) {
+    const int n = (int)(p.hi - b < 32 ? p.hi - b : 32);
+    int dest = 0;
+    if (lane < n) dest = __ldcs(&p.meta[b + lane].dest);
+    int r = lane / p.slices, s = lane % p.slices;
+    for (int k = 0; k < p.slices; ++k) {   // 32 rows x slices pieces, 32 at a time
+      const int64_t d = __shfl_sync(0xffffffffu, dest, r & 31);
+      if (r < n) __stcs(reinterpret_cast<uint4 *>(p.dst + d * p.pitch) + s, row[s]);
+      r += step_r; s += step_s;
+      if (s >= p.slices) { s -= p.slices; ++r; }
+    }
+  }
+}
+
 }  // namespace
+
+it_status it_launch_const_rows(const it_const_rows_args &a, int kid, double bytes, cudaStream_t st) {
+  const it_graph *g = a.g;
+  ConstRowsParams p;
+  p.meta = g->bucket_meta; p.lo = a.row_lo; p.hi = a.row_hi; p.dst = (char *)a.dst; p.pitch = a.pitch; p.dim = a.dim;
+  p.slices = a.dim * it_dtype_size(a.dtype) / 16; p.bf16 = a.dtype == IT_BF16; p.has_bias = a.has_bias; p.act = (int)a.act;
+  p.value = a.value; p.bias = a.bias;
+  const int64_t want = (a.row_hi - a.row_lo + GATHER_THREADS - 1) / GATHER_THREADS, cap = (int64_t)g->num_sms * 8;
+  IT_LAUNCH(kid, bytes, 0, st, const_rows_kernel<<<(unsigned)(want < cap ? want : cap), GATHER_THREADS, 0, st>>>(p));
+  IT_CUDA_TRY(cudaGetLastError());
+  return IT_OK;
+}
 
 // One column chunk of the rows: `a.dim` is the chunk's width (16 to 512 bytes), the
 // pointers already point at its first column, and the *_ld fields / src_ld carry the full row lengths.

@@ -26,6 +26,14 @@ struct SagePolicy {
   int col;
   float self[VEC];
 
+  bool empty_rows(it_const_rows_args &a) const {
+    if (epi == IT_EPI_ADD_ACT) return false;   // its self term still has to be read
+    const bool raw = epi == IT_EPI_RAW_F32;
+    a.dst = dst; a.dim = dim; a.dtype = raw || sizeof(T) == 4 ? IT_F32 : IT_BF16; a.pitch = (int64_t)dst_ld * (raw ? 4 : (int)sizeof(T));
+    a.value = raw ? (RED == RED_MAX ? -INFINITY : (RED == RED_MIN ? INFINITY : 0.f)) : 0.f;
+    a.has_bias = epi == IT_EPI_BIAS_ACT; a.bias = bias; a.act = (it_act)act;
+    return true;
+  }
   __device__ __forceinline__ void setup(int t) { col = t * VEC; }
   __device__ __forceinline__ void init(float (&st)[NS]) const {
 #pragma unroll
@@ -89,10 +97,12 @@ struct SagePolicy {
     }
     if (epi == IT_EPI_ADD_ACT) {
 #pragma unroll
-      for (int i = 0; i < VEC; ++i) st[i] = act_apply(st[i] + self[i], act);
+      for (int i = 0; i < VEC; ++i) st[i] += self[i];
+      act_slice<VEC>(st, act);
     } else if (epi == IT_EPI_BIAS_ACT) {
 #pragma unroll
-      for (int i = 0; i < VEC; ++i) st[i] = act_apply(st[i] + (bias ? __ldg(bias + col + i) : 0.f), act);
+      for (int i = 0; i < VEC; ++i) st[i] += bias ? __ldg(bias + col + i) : 0.f;
+      act_slice<VEC>(st, act);
     }
     Slice::store(reinterpret_cast<T *>(dst) + (int64_t)dest * dst_ld + col, st);
   }

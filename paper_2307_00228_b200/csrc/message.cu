@@ -169,7 +169,7 @@ it_status it_launch_gat_edge_rows(const it_graph *g, it_dtype dtype, int dim, in
   const int64_t cap = (int64_t)g->num_sms * 16;
   int64_t want = (total + (int64_t)MSG_THREADS * MSG_UNROLL - 1) / ((int64_t)MSG_THREADS * MSG_UNROLL);
   unsigned blocks = (unsigned)(want < cap ? want : cap);
-  IT_LAUNCH(IT_K_EDGE_MSG, (double)g->e * (4.0 + 2.0 * dim * es), 0, st,
+  if (Zj) IT_LAUNCH(IT_K_EDGE_MSG, (double)g->e * (4.0 + 2.0 * dim * es), 0, st,
             gat_edge_rows_kernel<<<blocks, MSG_THREADS, 0, st>>>(g->indices, reinterpret_cast<const uint4 *>(Z), reinterpret_cast<uint4 *>(Zj), total, slices));
   want = (g->e * heads + MSG_THREADS - 1) / MSG_THREADS;
   blocks = (unsigned)(want < cap ? want : cap);

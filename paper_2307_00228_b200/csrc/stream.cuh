@@ -28,6 +28,7 @@
 //   void merge(float (&st)[NS], const float (&other)[NS]);     // other comes later in edge order
 //   void begin_row(int32_t dest, int32_t owner);               // prefetch what end_row needs
 //   void end_row(float (&st)[NS], int32_t dest, int32_t owner, int64_t len);
+//   bool empty_rows(it_const_rows_args &a);   // host: rows without edges all get the value described in a
 #pragma once
 
 #include <atomic>
@@ -48,9 +49,6 @@
 #endif
 #ifndef IT_RING_STAGES
 #define IT_RING_STAGES 2
-#endif
-#ifndef IT_RING_DYNAMIC
-#define IT_RING_DYNAMIC 1   // 1: the warps of the ring kernel claim their batches from a counter instead of walking a fixed stride
 #endif
 #ifndef IT_RING_CLAIMS_PER_WARP
 #define IT_RING_CLAIMS_PER_WARP 16   // claims a warp of the ring kernel makes on average over a launch
@@ -161,6 +159,16 @@ __device__ __forceinline__ void add_bf16x2_to_f32(float &a0, float &a1, uint32_t
   asm("add.rn.f32.bf16 %0, %1, %0;" : "+f"(a0) : "h"(lo));
   asm("add.rn.f32.bf16 %0, %1, %0;" : "+f"(a1) : "h"(hi));
 }
+// a += w * b (pairwise, scalar w)
+__device__ __forceinline__ void fma_f32x2(float &a0, float &a1, float w, float b0, float b1) {
+#if IT_PACKED_F32
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(pack_f32x2(w, w)), "l"(pack_f32x2(b0, b1)), "l"(pack_f32x2(a0, a1)));
+  unpack_f32x2(d, a0, a1);
+#else
+  a0 = fmaf(w, b0, a0); a1 = fmaf(w, b1, a1);
+#endif
+}
 // a = w * b + a * s (pairwise, scalars w and s): the running-softmax update
 __device__ __forceinline__ void scale_fma_f32x2(float &a0, float &a1, float s, float w, float b0, float b1) {
 #if IT_PACKED_F32
@@ -200,6 +208,18 @@ __device__ __forceinline__ float act_apply(float x, int act) {
   if (act == IT_ACT_RELU) return fmaxf(x, 0.f);
   if (act == IT_ACT_ELU) return it_elu(x);
   return x;
+}
+
+// The activation of a whole slice: one decision instead of one per entry.
+template <int VEC>
+__device__ __forceinline__ void act_slice(float (&v)[VEC], int act) {
+  if (act == IT_ACT_RELU) {
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) v[i] = fmaxf(v[i], 0.f);
+  } else if (act == IT_ACT_ELU) {
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) v[i] = it_elu(v[i]);
+  }
 }
 
 // What every streaming kernel needs besides its policy.
@@ -658,6 +678,7 @@ __global__ void __launch_bounds__(THREADS) stream_empty_kernel(StreamParams p, P
 }  // namespace it_stream
 
 #include "stream_ring.cuh"
+#include "stream_chunk.cuh"
 
 namespace it_stream {
 
@@ -686,11 +707,9 @@ template <typename T, int SB, int LPR, bool PAD, class Policy, class BytesF>
 it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, BytesF bytes_of, int kid_cta, int kid_rows,
                          int kid_empty, int64_t bound_lo, int64_t bound_hi, int *counters, cudaStream_t st) {
   constexpr bool RING = SB * LPR >= 128;   // rows of 128 bytes and more are staged through shared memory
-#if !IT_RING_DYNAMIC
-  counters = nullptr;
-#endif
   if (RING && counters) IT_CUDA_TRY(cudaMemsetAsync(counters, 0, IT_MAX_BUCKETS * sizeof(int), st));
   p.counter = nullptr;
+  bool chunked = false;
   p.slices = p.dim * (int)sizeof(T) / SB;
   for (int b = g->n_buckets - 1; b >= 0; --b) {
     const int64_t lo = g->h_bucket_offsets[b], hi = g->h_bucket_offsets[b + 1];
@@ -701,6 +720,12 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
     const int64_t max_blocks = (int64_t)g->num_sms * IT_GATHER_MIN_BLOCKS * 2;
     const double bytes = bytes_of(b, rows);
     if (bound == 0) {
+      it_const_rows_args cr;
+      if (pol.empty_rows(cr)) {   // the same value for every row: no self term to read
+        cr.g = g; cr.row_lo = lo; cr.row_hi = hi;
+        IT_TRY(it_launch_const_rows(cr, kid_empty, bytes, st));
+        continue;
+      }
       int64_t want = (rows + (THREADS / LPR) - 1) / (THREADS / LPR);
       unsigned blocks = (unsigned)(want < max_blocks ? want : max_blocks);
       IT_LAUNCH(kid_empty, bytes, 0, st, stream_empty_kernel<T, SB, LPR, Policy><<<blocks, THREADS, 0, st>>>(p, pol));
@@ -740,6 +765,29 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
           const int64_t short_max = (int64_t)g->num_sms * IT_SHORT_PIPE_BLOCKS * IT_SHORT_PIPE_WAVES;
           unsigned blocks = (unsigned)(want < short_max ? want : short_max);
           IT_LAUNCH(kid_rows, bytes, 0, st, stream_short_rows_pipe_kernel<T, LPR, Policy, PAD><<<blocks, THREADS, 0, st>>>(p, pol));
+          continue;
+        }
+      }
+      if constexpr (SB == 16 && LPR >= 8 && !Policy::HAS_EXTRA) {
+        // one warp per row: the buckets above IT_SHORT_BELOW edges that have no block per row, in one launch (they are
+        // neighbours in the row list), longest first
+        if (bound > IT_SHORT_BELOW && counters) {
+          if (chunked) continue;
+          chunked = true;
+          double all = bytes;
+          int b0 = b;
+          while (b0 > 0 && g->bucket_bounds[b0 - 1] > IT_SHORT_BELOW) {
+            --b0;
+            all += bytes_of(b0, g->h_bucket_offsets[b0 + 1] - g->h_bucket_offsets[b0]);
+          }
+          p.row_lo = g->h_bucket_offsets[b0];
+          constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<16, false>();
+          static std::atomic<uint64_t> configured{0};   // per template instance: one bit per device ordinal
+          IT_TRY(allow_dynamic_smem(stream_rows_chunk_kernel<T, LPR, Policy, PAD>, smem, configured));
+          p.counter = counters + b;
+          const unsigned blocks = chunk_grid(hi - p.row_lo, (int64_t)g->num_sms * IT_RING_MIN_BLOCKS, &p.claim);
+          IT_LAUNCH(kid_rows, all, 0, st, stream_rows_chunk_kernel<T, LPR, Policy, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
+          p.counter = nullptr;
           continue;
         }
       }
