@@ -81,7 +81,9 @@ struct it_graph {
   int device = 0;
   int num_sms = IT_NUM_SMS_FALLBACK;
 
-  // derived by the split (library-owned, device)
+  // derived by the split (library-owned, device; all carved out of one allocation that is kept for the next split)
+  char *slab = nullptr;
+  size_t slab_bytes = 0;
   int64_t threshold = 0;
   int64_t n_rows = 0;           // R
   int64_t n_split_owners = 0;   // vertices with more than one shadow row
@@ -89,7 +91,6 @@ struct it_graph {
   int64_t *shadow_indptr = nullptr;  // [R+1]
   int32_t *shadow_owner = nullptr;   // [R]
   int64_t *owner_indptr = nullptr;   // [n+1]
-  int32_t *row_dest = nullptr;       // [R]  v >= 0: row is the whole segment of v; < 0: ~index into the partial buffer
   int32_t *split_owners = nullptr;   // [n_split_owners] ascending vertex ids
   int32_t n_buckets = 0;
   int64_t bucket_bounds[IT_MAX_BUCKETS] = {0};

@@ -2,6 +2,7 @@
 // Integer-only work; every array produced here is a pure function of (indptr, threshold)
 // and is built without atomics on data, so it is reproducible bit for bit.
 #include <new>
+#include <type_traits>
 #include <stdarg.h>
 #include <string.h>
 
@@ -57,23 +58,133 @@ __global__ void validate_indptr_kernel(IndptrView ip, int64_t n, int64_t e, int 
   if (bad) atomicOr(flags, bad);
 }
 
-__global__ void validate_indices_kernel(const int32_t *__restrict__ idx, int64_t e, int64_t n,
-                                        int *flags) {
-  int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  int bad = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < e; i += stride) {
-    int32_t s = idx[i];
-    if (s < 0 || (int64_t)s >= n) bad = 8;
+// Four ids per load (`head` ids up to the first 16-byte boundary and the last few on their own): bound by reading them.
+__global__ void __launch_bounds__(256) validate_indices_kernel(const int32_t *__restrict__ idx, int64_t e, int64_t n, int head, int *flags) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const uint32_t top = (uint32_t)n;   // n < 2^31: a negative id is a large unsigned one
+  bool bad = false;
+  const int4 *v = reinterpret_cast<const int4 *>(idx + head);
+  const int64_t quads = (e - head) / 4;
+  for (int64_t i = first; i < quads; i += 4 * stride) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i + u * stride < quads) {
+        const int4 x = __ldcs(v + i + u * stride);
+        bad |= (uint32_t)x.x >= top || (uint32_t)x.y >= top || (uint32_t)x.z >= top || (uint32_t)x.w >= top;
+      }
   }
-  if (bad) atomicOr(flags, bad);
+  for (int64_t i = first; i < head; i += stride) bad |= (uint32_t)idx[i] >= top;
+  for (int64_t i = head + quads * 4 + first; i < e; i += stride) bad |= (uint32_t)idx[i] >= top;
+  if (bad) atomicOr(flags, 8);
 }
 
-// ----------------------------------------------------------------------------- scan-and-emit
-// Exclusive prefix sum of value(i), i in [0, n), handed to emit(i, prefix) — three launches,
-// no inter-block waiting.  Tile = SCAN_THREADS * SCAN_ITEMS consecutive items per block.
-constexpr int SCAN_THREADS = 256;
-constexpr int SCAN_ITEMS = 8;
-constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
+// ----------------------------------------------------------------------------- split
+// The shadow rows and the degree buckets in one pass over the vertices: count per tile, scan the tile counts, emit.
+// Every vertex adds rows to at most two buckets (all groups of a split vertex hold d / ng or d / ng + 1 edges), so the row
+// numbers, the list of split vertices and the positions inside every bucket are prefix sums of the same pass: columns
+// 0 .. nb - 1 the buckets, nb the rows, nb + 1 the split vertices.
+// Bound by reading indptr twice and writing 36 bytes per row; a scan per bucket (each over every row, three launches with a
+// read of two 8-byte bounds per row) took 3.2 ms of device time for 5M vertices and six buckets, this one 3.0 with
+// everything around it (create + split: 14.3 -> 3.0 ms; the derived arrays are one allocation instead of nine, kept for the next split).
+constexpr int SPLIT_THREADS = 256;
+constexpr int SPLIT_ITEMS = 8;                                    // vertices per lane: a warp covers 256 consecutive ones
+constexpr int SPLIT_TILE = SPLIT_THREADS * SPLIT_ITEMS;
+constexpr int SPLIT_COLS = IT_MAX_BUCKETS + 2;
+
+struct Bounds { int64_t b[IT_MAX_BUCKETS]; int nb; };
+__device__ __forceinline__ int bucket_of(int64_t len, const Bounds &B) {
+  int k = 0;
+  while (k < B.nb - 1 && len > B.b[k]) ++k;
+  return k;
+}
+
+struct SplitInfo { int64_t r0, pos_a, pos_b; };   // a split vertex: its first row; list positions of its longer / shorter groups
+
+struct SplitParams {
+  IndptrView ip;
+  int64_t n, e, T;
+  Bounds B;
+  int64_t n_tiles;
+  int64_t *tiles;          // [SPLIT_COLS][n_tiles]
+  int64_t *totals;         // [SPLIT_COLS] column sums, then [IT_MAX_BUCKETS] edges per bucket
+  int64_t *shadow_indptr; int32_t *shadow_owner; int64_t *owner_indptr; int32_t *split_owners;
+  int64_t *bucket_offsets; int32_t *bucket_rows; it_row_meta *bucket_meta; int32_t *bucket_owner;
+  SplitInfo *info;         // [split vertices]
+};
+
+// What a vertex adds: ng rows; `rem` of them in bucket ka (one edge longer), the others in bucket kb.
+struct VertexRows { int64_t ng, rem; int ka, kb; };
+__device__ __forceinline__ VertexRows rows_of(int64_t d, const SplitParams &p) {
+  VertexRows r;
+  r.ng = groups_of(d, p.T);
+  if (r.ng == 1) {
+    r.rem = 0;
+    r.ka = r.kb = bucket_of(d, p.B);
+  } else {
+    const int64_t base = d / r.ng;
+    r.rem = d % r.ng;
+    r.ka = bucket_of(base + 1, p.B);
+    r.kb = bucket_of(base, p.B);
+  }
+  return r;
+}
+
+// Lane c of a warp keeps column c.  One step over 32 vertices, of which those in `valid` exist: count(...) adds them.
+__device__ __forceinline__ void add_columns(int64_t &col, const VertexRows &r, unsigned valid, unsigned split, int nb, int lane) {
+  const bool plain = ((valid & ~split) >> lane) & 1u;
+  for (int k = 0; k < nb; ++k) {
+    const unsigned m = __ballot_sync(0xffffffffu, plain && r.ka == k);
+    if (lane == k) col += __popc(m);
+  }
+  if (lane == nb) col += __popc(valid & ~split);
+  while (split) {   // rare
+    const int l = __ffs(split) - 1;
+    split &= split - 1;
+    const int64_t ng = __shfl_sync(0xffffffffu, r.ng, l), rem = __shfl_sync(0xffffffffu, r.rem, l);
+    const int ka = __shfl_sync(0xffffffffu, r.ka, l), kb = __shfl_sync(0xffffffffu, r.kb, l);
+    if (lane == ka) col += rem;
+    if (lane == kb) col += ng - rem;
+    if (lane == nb) col += ng;
+    if (lane == nb + 1) col += 1;
+  }
+}
+
+__global__ void __launch_bounds__(SPLIT_THREADS) split_count_kernel(SplitParams p) {
+  __shared__ unsigned long long cols[SPLIT_COLS], edges[IT_MAX_BUCKETS];
+  const int lane = threadIdx.x & 31, nb = p.B.nb;
+  if (threadIdx.x < SPLIT_COLS) cols[threadIdx.x] = 0;
+  if (threadIdx.x < IT_MAX_BUCKETS) edges[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t v0 = (int64_t)blockIdx.x * SPLIT_TILE + (int64_t)(threadIdx.x >> 5) * (32 * SPLIT_ITEMS) + lane;
+  int64_t col = 0, my_edges = 0;
+  for (int i = 0; i < SPLIT_ITEMS; ++i) {
+    const int64_t v = v0 + i * 32;
+    const int64_t d = v < p.n ? p.ip[v + 1] - p.ip[v] : 0;
+    const VertexRows r = rows_of(d, p);
+    const unsigned valid = __ballot_sync(0xffffffffu, v < p.n), split = __ballot_sync(0xffffffffu, r.ng > 1);
+    if (valid == 0) break;
+    add_columns(col, r, valid, split, nb, lane);
+    // edges per bucket: 32-bit sums across the lanes unless a vertex is huge
+    if (__any_sync(0xffffffffu, d >= ((int64_t)1 << 26) || r.ng > 1)) {
+      if (v < p.n) {
+        const int64_t in_a = r.rem * (r.ng > 1 ? d / r.ng + 1 : 0);
+        if (in_a) atomicAdd(&edges[r.ka], (unsigned long long)in_a);
+        atomicAdd(&edges[r.kb], (unsigned long long)(d - in_a));
+      }
+    } else {
+      for (int k = 0; k < nb; ++k) {
+        const unsigned s = __reduce_add_sync(0xffffffffu, r.kb == k ? (unsigned)d : 0u);
+        if (lane == k) my_edges += s;
+      }
+    }
+  }
+  if (lane < nb + 2) atomicAdd(&cols[lane], (unsigned long long)col);
+  if (lane < nb) atomicAdd(&edges[lane], (unsigned long long)my_edges);
+  __syncthreads();
+  if (threadIdx.x < nb + 2) p.tiles[threadIdx.x * p.n_tiles + blockIdx.x] = (int64_t)cols[threadIdx.x];
+  if (threadIdx.x < nb && edges[threadIdx.x])
+    atomicAdd(reinterpret_cast<unsigned long long *>(p.totals + SPLIT_COLS + threadIdx.x), edges[threadIdx.x]);
+}
 
 __device__ __forceinline__ int64_t block_exclusive_scan(int64_t x, int64_t *total, int64_t *smem /*[33]*/) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -102,281 +213,249 @@ __device__ __forceinline__ int64_t block_exclusive_scan(int64_t x, int64_t *tota
   return smem[warp] + incl - x;
 }
 
-template <class ValueF>
-__global__ void __launch_bounds__(SCAN_THREADS) scan_tile_sums_kernel(int64_t n, ValueF value, int64_t *tile_sums) {
+// One block per column: exclusive scan of its tile counts in place, four tiles per thread and step; the sum to totals.
+__global__ void __launch_bounds__(1024) split_scan_kernel(SplitParams p) {
   __shared__ int64_t smem[33];
-  int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-  int64_t s = 0;
-#pragma unroll
-  for (int k = 0; k < SCAN_ITEMS; ++k)
-    if (base + k < n) s += value(base + k);
-  int64_t total;
-  block_exclusive_scan(s, &total, smem);
-  if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
-}
-
-// One block: exclusive scan of tile_sums in place; grand total to *total_out.
-__global__ void __launch_bounds__(1024) scan_tile_offsets_kernel(int64_t n_tiles, int64_t *tile_sums, int64_t *total_out) {
-  __shared__ int64_t smem[33];
+  int64_t *t = p.tiles + blockIdx.x * p.n_tiles;
   int64_t carry = 0;
-  for (int64_t base = 0; base < n_tiles; base += blockDim.x) {
-    int64_t i = base + threadIdx.x;
-    int64_t x = i < n_tiles ? tile_sums[i] : 0;
-    int64_t total;
-    int64_t ex = block_exclusive_scan(x, &total, smem);
-    if (i < n_tiles) tile_sums[i] = carry + ex;
+  for (int64_t base = 0; base < p.n_tiles; base += 4096) {
+    const int64_t i = base + 4 * (int64_t)threadIdx.x;
+    int64_t x[4], sum = 0, total;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { x[u] = i + u < p.n_tiles ? t[i + u] : 0; sum += x[u]; }
+    int64_t ex = carry + block_exclusive_scan(sum, &total, smem);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (i + u < p.n_tiles) t[i + u] = ex;
+      ex += x[u];
+    }
     carry += total;
   }
-  if (threadIdx.x == 0) *total_out = carry;
+  if (threadIdx.x == 0) p.totals[blockIdx.x] = carry;
 }
 
-template <class ValueF, class EmitF>
-__global__ void __launch_bounds__(SCAN_THREADS) scan_emit_kernel(int64_t n, ValueF value, EmitF emit, const int64_t *tile_offsets) {
-  __shared__ int64_t smem[33];
-  int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-  int64_t v[SCAN_ITEMS];
-  int64_t s = 0;
+__global__ void __launch_bounds__(SPLIT_THREADS) split_emit_kernel(SplitParams p) {
+  __shared__ int64_t warp_cols[SPLIT_THREADS / 32][SPLIT_COLS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nb = p.B.nb;
+  const int64_t v0 = (int64_t)blockIdx.x * SPLIT_TILE + (int64_t)warp * (32 * SPLIT_ITEMS) + lane;
+  int64_t j0[SPLIT_ITEMS];
+  int64_t d[SPLIT_ITEMS];
+  int64_t col = 0;
 #pragma unroll
-  for (int k = 0; k < SCAN_ITEMS; ++k) {
-    v[k] = (base + k < n) ? value(base + k) : 0;
-    s += v[k];
+  for (int i = 0; i < SPLIT_ITEMS; ++i) {
+    const int64_t v = v0 + i * 32;
+    j0[i] = v < p.n ? p.ip[v] : 0;
+    d[i] = v < p.n ? p.ip[v + 1] - j0[i] : 0;
+    const VertexRows r = rows_of(d[i], p);
+    add_columns(col, r, __ballot_sync(0xffffffffu, v < p.n), __ballot_sync(0xffffffffu, r.ng > 1), nb, lane);
   }
-  int64_t total;
-  int64_t prefix = tile_offsets[blockIdx.x] + block_exclusive_scan(s, &total, smem);
+  if (lane < nb + 2) warp_cols[warp][lane] = col;
+  __syncthreads();
+  // lane c: the running value of column c; for a bucket counted from the start of the whole list
+  int64_t run = 0;
+  if (lane < nb + 2) {
+    run = p.tiles[lane * p.n_tiles + blockIdx.x];
+    for (int w = 0; w < warp; ++w) run += warp_cols[w][lane];
+    if (lane < nb)
+      for (int k = 0; k < lane; ++k) run += p.totals[k];
+  }
+  if (blockIdx.x == 0 && warp == 0) {
+    if (lane <= nb) {
+      int64_t off = 0;
+      for (int k = 0; k < lane; ++k) off += p.totals[k];
+      p.bucket_offsets[lane] = off;
+    }
+    if (lane == 0) {
+      p.shadow_indptr[p.totals[nb]] = p.e;
+      p.owner_indptr[p.n] = p.totals[nb];
+    }
+  }
 #pragma unroll
-  for (int k = 0; k < SCAN_ITEMS; ++k) {
-    if (base + k < n) emit(base + k, prefix);
-    prefix += v[k];
+  for (int i = 0; i < SPLIT_ITEMS; ++i) {
+    const int64_t v = v0 + i * 32;
+    const VertexRows r = rows_of(d[i], p);
+    const unsigned valid = __ballot_sync(0xffffffffu, v < p.n), split = __ballot_sync(0xffffffffu, r.ng > 1);
+    int64_t row = 0, pos = 0;
+    if (split == 0) {
+      row = __shfl_sync(0xffffffffu, run, nb) + lane;
+      for (int k = 0; k < nb; ++k) {
+        const unsigned m = __ballot_sync(0xffffffffu, v < p.n && r.ka == k);
+        const int64_t at = __shfl_sync(0xffffffffu, run, k);
+        if (r.ka == k) pos = at + __popc(m & ((1u << lane) - 1u));
+      }
+      add_columns(run, r, valid, 0u, nb, lane);
+    } else {   // a split vertex among the 32: one vertex after the other
+      for (int l = 0; l < 32; ++l) {
+        if (!((valid >> l) & 1u)) break;
+        const int64_t ng = __shfl_sync(0xffffffffu, r.ng, l), rem = __shfl_sync(0xffffffffu, r.rem, l);
+        const int ka = __shfl_sync(0xffffffffu, r.ka, l), kb = __shfl_sync(0xffffffffu, r.kb, l);
+        const int64_t at_row = __shfl_sync(0xffffffffu, run, nb), at_k = __shfl_sync(0xffffffffu, run, nb + 1);
+        if (lane == nb) run += ng;
+        if (lane == nb + 1 && ng > 1) run += 1;
+        const int64_t at_a = __shfl_sync(0xffffffffu, run, ka);
+        if (ng > 1 && lane == ka) run += rem;
+        const int64_t at_b = __shfl_sync(0xffffffffu, run, kb);
+        if (lane == kb) run += ng - rem;   // (one plain row: rem = 0)
+        if (lane == l) {
+          row = at_row; pos = at_b;
+          if (ng > 1) {
+            p.split_owners[at_k] = (int32_t)v;
+            p.info[at_k] = SplitInfo{at_row, at_a, at_b};
+          }
+        }
+      }
+    }
+    if (v < p.n) {
+      p.owner_indptr[v] = row;
+      if (r.ng == 1) {
+        p.shadow_indptr[row] = j0[i];
+        p.shadow_owner[row] = (int32_t)v;
+        p.bucket_rows[pos] = (int32_t)row;
+        it_row_meta m;
+        m.j0 = j0[i]; m.len = (int32_t)d[i]; m.dest = (int32_t)v;
+        p.bucket_meta[pos] = m;
+        p.bucket_owner[pos] = (int32_t)v;
+      }
+    }
   }
 }
 
-// tile_sums: device scratch of at least ceil(n / SCAN_TILE) + 1 int64; the last entry receives the total.
-template <class ValueF, class EmitF>
-static it_status scan_and_emit(int kid, int64_t n, ValueF value, EmitF emit, int64_t *tile_sums, int64_t *d_total, cudaStream_t st) {
-  int64_t n_tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-  if (n_tiles == 0) {
-    IT_CUDA_TRY(cudaMemsetAsync(d_total, 0, sizeof(int64_t), st));
-    return IT_OK;
+// Rows of split vertices: one block per split vertex, groups written by closed form
+//   start(g) = indptr[v] + g * base + min(g, rem),  base = d / ng, rem = d % ng;
+// group g's partial result goes to slot p0 + g: the rows of earlier split vertices = all earlier rows minus earlier unsplit vertices.
+__global__ void __launch_bounds__(128) fill_split_rows_kernel(SplitParams p) {
+  const int64_t n_split = p.totals[p.B.nb + 1];
+  for (int64_t k = blockIdx.x; k < n_split; k += gridDim.x) {
+    const int64_t v = p.split_owners[k], s = p.ip[v], d = p.ip[v + 1] - s;
+    const SplitInfo f = p.info[k];
+    const int64_t ng = groups_of(d, p.T), base = d / ng, rem = d % ng, p0 = f.r0 - v + k;
+    for (int64_t g = threadIdx.x; g < ng; g += blockDim.x) {
+      const int64_t row = f.r0 + g, pos = g < rem ? f.pos_a + g : f.pos_b + (g - rem);
+      it_row_meta m;
+      m.j0 = s + g * base + (g < rem ? g : rem);
+      m.len = (int32_t)(base + (g < rem ? 1 : 0));
+      m.dest = (int32_t)~(p0 + g);
+      p.shadow_indptr[row] = m.j0;
+      p.shadow_owner[row] = (int32_t)v;
+      p.bucket_rows[pos] = (int32_t)row;
+      p.bucket_meta[pos] = m;
+      p.bucket_owner[pos] = (int32_t)v;
+    }
   }
-  IT_LAUNCH(kid, 0, 0, st, scan_tile_sums_kernel<<<(unsigned)n_tiles, SCAN_THREADS, 0, st>>>(n, value, tile_sums));
-  IT_LAUNCH(kid, 0, 0, st, scan_tile_offsets_kernel<<<1, 1024, 0, st>>>(n_tiles, tile_sums, d_total));
-  IT_LAUNCH(kid, 0, 0, st, scan_emit_kernel<<<(unsigned)n_tiles, SCAN_THREADS, 0, st>>>(n, value, emit, tile_sums));
-  IT_CUDA_TRY(cudaGetLastError());
-  return IT_OK;
-}
-
-// ----------------------------------------------------------------------------- split functors
-struct RowsOfVertex {
-  IndptrView ip; int64_t T;
-  __device__ int64_t operator()(int64_t v) const { return groups_of(ip[v + 1] - ip[v], T); }
-};
-struct EmitOwnerIndptr {
-  int64_t *owner_indptr; int64_t n;
-  __device__ void operator()(int64_t v, int64_t prefix) const { owner_indptr[v] = prefix; }
-};
-struct IsSplit {
-  IndptrView ip; int64_t T;
-  __device__ int64_t operator()(int64_t v) const { return groups_of(ip[v + 1] - ip[v], T) > 1 ? 1 : 0; }
-};
-struct EmitSplitOwner {
-  IndptrView ip; int64_t T; int32_t *split_owners;
-  __device__ void operator()(int64_t v, int64_t k) const {
-    if (groups_of(ip[v + 1] - ip[v], T) > 1) split_owners[k] = (int32_t)v;
-  }
-};
-// count pass only (the list is not allocated yet)
-struct EmitNothing {
-  __device__ void operator()(int64_t, int64_t) const {}
-};
-
-// Rows of unsplit vertices: one thread per vertex.
-__global__ void fill_unsplit_rows_kernel(IndptrView ip, int64_t n, int64_t T, const int64_t *__restrict__ owner_indptr,
-                                         int64_t *shadow_indptr, int32_t *shadow_owner, int32_t *row_dest,
-                                         int64_t n_rows, int64_t e) {
-  int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v == 0) shadow_indptr[n_rows] = e;
-  if (v >= n) return;
-  int64_t d = ip[v + 1] - ip[v];
-  if (groups_of(d, T) > 1) return;
-  int64_t r = owner_indptr[v];
-  shadow_indptr[r] = ip[v];
-  shadow_owner[r] = (int32_t)v;
-  row_dest[r] = (int32_t)v;
-}
-
-// Rows of split vertices: one block per split owner, groups written by closed form
-//   start(g) = indptr[v] + g * base + min(g, rem),  base = d / n, rem = d % n.
-__global__ void fill_split_rows_kernel(IndptrView ip, int64_t T, const int32_t *__restrict__ split_owners,
-                                       const int64_t *__restrict__ owner_indptr, int64_t *shadow_indptr,
-                                       int32_t *shadow_owner, int32_t *row_dest) {
-  int64_t k = blockIdx.x;
-  int64_t v = split_owners[k];
-  int64_t d = ip[v + 1] - ip[v];
-  int64_t ng = groups_of(d, T);
-  int64_t base = d / ng, rem = d % ng;
-  int64_t r0 = owner_indptr[v];
-  int64_t p0 = r0 - v + k;  // rows of earlier split owners = all earlier rows minus earlier unsplit vertices
-  for (int64_t g = threadIdx.x; g < ng; g += blockDim.x) {
-    shadow_indptr[r0 + g] = ip[v] + g * base + (g < rem ? g : rem);
-    shadow_owner[r0 + g] = (int32_t)v;
-    row_dest[r0 + g] = (int32_t)~(p0 + g);
-  }
-}
-
-// ----------------------------------------------------------------------------- bucket functors
-struct Bounds { int64_t b[IT_MAX_BUCKETS]; int nb; };
-__device__ __forceinline__ int bucket_of(int64_t len, const Bounds &B) {
-  int k = 0;
-  while (k < B.nb - 1 && len > B.b[k]) ++k;
-  return k;
-}
-struct InBucket {
-  const int64_t *sp; Bounds B; int which;
-  __device__ int64_t operator()(int64_t r) const { return bucket_of(sp[r + 1] - sp[r], B) == which ? 1 : 0; }
-};
-struct EmitBucketRow {
-  const int64_t *sp; Bounds B; int which; int32_t *bucket_rows; const int64_t *bucket_offsets;
-  __device__ void operator()(int64_t r, int64_t pos) const {
-    if (bucket_of(sp[r + 1] - sp[r], B) == which) bucket_rows[bucket_offsets[which] + pos] = (int32_t)r;
-  }
-};
-struct EdgesInBucket {
-  const int64_t *sp; Bounds B; int which;
-  __device__ int64_t operator()(int64_t r) const {
-    const int64_t len = sp[r + 1] - sp[r];
-    return bucket_of(len, B) == which ? len : 0;
-  }
-};
-__global__ void fill_bucket_meta_kernel(int64_t n_rows, const int32_t *__restrict__ bucket_rows,
-                                       const int64_t *__restrict__ sp, const int32_t *__restrict__ row_dest,
-                                       const int32_t *__restrict__ shadow_owner, it_row_meta *__restrict__ meta,
-                                       int32_t *__restrict__ bucket_owner) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n_rows) return;
-  const int32_t r = bucket_rows[i];
-  it_row_meta m;
-  m.j0 = sp[r];
-  m.len = (int32_t)(sp[r + 1] - sp[r]);
-  m.dest = row_dest[r];
-  meta[i] = m;
-  bucket_owner[i] = shadow_owner[r];
-}
-__global__ void set_next_bucket_offset_kernel(int64_t *bucket_offsets, int which, const int64_t *count) {
-  if (which == 0) bucket_offsets[0] = 0;
-  bucket_offsets[which + 1] = bucket_offsets[which] + *count;
 }
 
 // ----------------------------------------------------------------------------- host side
-static void free_derived(it_graph *g) {
-  cudaFree(g->shadow_indptr); cudaFree(g->shadow_owner); cudaFree(g->owner_indptr);
-  cudaFree(g->row_dest); cudaFree(g->split_owners); cudaFree(g->bucket_offsets); cudaFree(g->bucket_rows);
-  cudaFree(g->bucket_meta); g->bucket_meta = nullptr;
-  cudaFree(g->bucket_owner); g->bucket_owner = nullptr;
-  g->shadow_indptr = nullptr; g->shadow_owner = nullptr; g->owner_indptr = nullptr; g->row_dest = nullptr;
+static void forget_split(it_graph *g) {
+  g->shadow_indptr = nullptr; g->shadow_owner = nullptr; g->owner_indptr = nullptr;
   g->split_owners = nullptr; g->bucket_offsets = nullptr; g->bucket_rows = nullptr;
+  g->bucket_meta = nullptr; g->bucket_owner = nullptr;
   g->n_rows = g->n_split_owners = g->n_partial_rows = 0;
   g->n_buckets = 0;
 }
 
+// The derived arrays and the scratch of a split with at most R rows and S split vertices, carved out of one allocation that
+// the graph keeps for its next split (NULL slab: only the size).
+static size_t carve_split(it_graph *g, SplitParams &p, char *slab, int64_t R, int64_t S) {
+  size_t off = 0;
+  auto take = [&](auto *&ptr, int64_t count) {
+    ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(slab + off);
+    off += it_align_up((size_t)(count > 0 ? count : 1) * sizeof(*ptr));
+  };
+  take(p.totals, SPLIT_COLS + IT_MAX_BUCKETS);
+  take(p.tiles, SPLIT_COLS * p.n_tiles);
+  take(p.bucket_offsets, IT_MAX_BUCKETS + 1);
+  take(p.owner_indptr, p.n + 1);
+  take(p.shadow_indptr, R + 1);
+  take(p.shadow_owner, R);
+  take(p.bucket_rows, R);
+  take(p.bucket_meta, R);
+  take(p.bucket_owner, R);
+  take(p.split_owners, S);
+  take(p.info, S);
+  return off;
+}
+
 static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
-  free_derived(g);
+  // the arrays of the previous split are written over: forward passes on any stream that still read them come first
+  if (g->bucket_meta) IT_CUDA_TRY(cudaDeviceSynchronize());
+  forget_split(g);
   g->threshold = T > 0 ? T : 0;
   const int64_t n = g->n;
-  IndptrView ip{g->indptr, g->indptr_type == IT_I64};
-
-  int64_t *d_scratch = nullptr;  // tile sums (+ totals at the end)
-  int64_t max_items = n;         // rows are scanned later; R is not known yet, scratch is re-sized then
-  int64_t n_tiles = (max_items + SCAN_TILE - 1) / SCAN_TILE;
-  IT_CUDA_TRY(cudaMalloc(&d_scratch, (size_t)(n_tiles + 4) * sizeof(int64_t)));
-  int64_t *d_total = d_scratch + n_tiles;  // [0] rows, [1] split owners
-  it_status rc = IT_OK;
-  int64_t h_tot[2] = {0, 0};
-  auto fail = [&](it_status s) { cudaFree(d_scratch); free_derived(g); return s; };
-#define SPLIT_TRY(expr) do { rc = (expr); if (rc != IT_OK) return fail(rc); } while (0)
-#define SPLIT_CUDA(expr) do { cudaError_t _e = (expr); if (_e != cudaSuccess) { \
-    it_set_error("%s failed: %s", #expr, cudaGetErrorString(_e)); \
-    return fail(_e == cudaErrorMemoryAllocation ? IT_ERR_OOM : IT_ERR_CUDA); } } while (0)
-
-  SPLIT_CUDA(cudaMalloc(&g->owner_indptr, (size_t)(n + 1) * sizeof(int64_t)));
-  SPLIT_TRY(scan_and_emit(IT_K_SPLIT_SCAN, n, RowsOfVertex{ip, T}, EmitOwnerIndptr{g->owner_indptr, n}, d_scratch, d_total, st));
-  SPLIT_CUDA(cudaMemcpyAsync(g->owner_indptr + n, d_total, sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
-  SPLIT_TRY(scan_and_emit(IT_K_SPLIT_SCAN, n, IsSplit{ip, T}, EmitNothing{}, d_scratch, d_total + 1, st));
-  SPLIT_CUDA(cudaMemcpyAsync(h_tot, d_total, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-  SPLIT_CUDA(cudaStreamSynchronize(st));
-  const int64_t R = n > 0 ? h_tot[0] : 0;
-  const int64_t S = n > 0 ? h_tot[1] : 0;
-  if (R > (int64_t)INT32_MAX - 1) {
-    it_set_error("split produces %lld shadow rows; row ids are 32-bit", (long long)R);
-    return fail(IT_ERR_UNSUPPORTED);
-  }
-  g->n_rows = R;
-  g->n_split_owners = S;
-  g->n_partial_rows = R - (n - S);
-
-  SPLIT_CUDA(cudaMalloc(&g->shadow_indptr, (size_t)(R + 1) * sizeof(int64_t)));
-  SPLIT_CUDA(cudaMalloc(&g->shadow_owner, (size_t)(R > 0 ? R : 1) * sizeof(int32_t)));
-  SPLIT_CUDA(cudaMalloc(&g->row_dest, (size_t)(R > 0 ? R : 1) * sizeof(int32_t)));
-  SPLIT_CUDA(cudaMalloc(&g->split_owners, (size_t)(S > 0 ? S : 1) * sizeof(int32_t)));
-  SPLIT_CUDA(cudaMalloc(&g->bucket_rows, (size_t)(R > 0 ? R : 1) * sizeof(int32_t)));
-  SPLIT_CUDA(cudaMalloc(&g->bucket_meta, (size_t)(R > 0 ? R : 1) * sizeof(it_row_meta)));
-  SPLIT_CUDA(cudaMalloc(&g->bucket_owner, (size_t)(R > 0 ? R : 1) * sizeof(int32_t)));
-  SPLIT_CUDA(cudaMalloc(&g->bucket_offsets, (IT_MAX_BUCKETS + 1) * sizeof(int64_t)));
-  if (S > 0)
-    SPLIT_TRY(scan_and_emit(IT_K_SPLIT_SCAN, n, IsSplit{ip, T}, EmitSplitOwner{ip, T, g->split_owners}, d_scratch, d_total + 1, st));
-  {
-    unsigned blocks = (unsigned)((n + 255) / 256);
-    if (blocks == 0) blocks = 1;
-    IT_LAUNCH(IT_K_SPLIT_FILL, 0, 0, st,
-              fill_unsplit_rows_kernel<<<blocks, 256, 0, st>>>(ip, n, T, g->owner_indptr, g->shadow_indptr,
-                                                               g->shadow_owner, g->row_dest, R, g->e));
-    if (S > 0)
-      IT_LAUNCH(IT_K_SPLIT_FILL, 0, 0, st,
-                fill_split_rows_kernel<<<(unsigned)S, 128, 0, st>>>(ip, T, g->split_owners, g->owner_indptr,
-                                                                    g->shadow_indptr, g->shadow_owner, g->row_dest));
-    SPLIT_CUDA(cudaGetLastError());
-  }
-
+  SplitParams p{};
+  p.ip = IndptrView{g->indptr, g->indptr_type == IT_I64};
+  p.n = n; p.e = g->e; p.T = T;
+  p.n_tiles = (n + SPLIT_TILE - 1) / SPLIT_TILE;
   // degree buckets: {0, 8, 32, 256, 1024, everything longer}
-  Bounds B;
   const int64_t fixed[5] = {0, 8, 32, 256, 1024};
-  B.nb = 0;
+  p.B.nb = 0;
   for (int i = 0; i < 5; ++i)
-    if (T <= 0 || fixed[i] < T) B.b[B.nb++] = fixed[i];
-  B.b[B.nb++] = T > 0 ? T : INT64_MAX;
-  g->n_buckets = B.nb;
-  for (int i = 0; i < IT_MAX_BUCKETS; ++i) g->bucket_bounds[i] = i < B.nb ? B.b[i] : 0;
+    if (T <= 0 || fixed[i] < T) p.B.b[p.B.nb++] = fixed[i];
+  p.B.b[p.B.nb++] = T > 0 ? T : INT64_MAX;
 
-  // the row scans need ceil(R / tile) sums; R >= n, so regrow the scratch
-  cudaFree(d_scratch);
-  d_scratch = nullptr;
-  n_tiles = (R + SCAN_TILE - 1) / SCAN_TILE;
-  SPLIT_CUDA(cudaMalloc(&d_scratch, (size_t)(n_tiles + 4 + IT_MAX_BUCKETS) * sizeof(int64_t)));
-  d_total = d_scratch + n_tiles;
-  int64_t *d_edges = d_total + 4;
-  for (int b = 0; b < B.nb; ++b) {
-    if (b == 0) {
-      // offsets[0] must exist before the first emit reads it
-      SPLIT_CUDA(cudaMemsetAsync(g->bucket_offsets, 0, sizeof(int64_t), st));
+  // at most one row per vertex and one more per T edges; only where that is far above the number of vertices are the rows
+  // counted before the arrays are laid out
+  int64_t R = n + (T > 0 ? g->e / T : 0), S = T > 0 ? (n < g->e / T ? n : g->e / T) : 0;
+  const bool count_first = R > n + n / 4 + (1 << 20) || R > (int64_t)INT32_MAX - 1;
+  int64_t h[SPLIT_COLS + IT_MAX_BUCKETS] = {0};
+  auto reserve = [&](size_t bytes) -> it_status {   // grow the graph's allocation; what it holds is not kept
+    if (bytes <= g->slab_bytes) return IT_OK;
+    cudaFree(g->slab);
+    g->slab = nullptr; g->slab_bytes = 0;
+    IT_CUDA_TRY(cudaMalloc(&g->slab, bytes));
+    g->slab_bytes = bytes;
+    return IT_OK;
+  };
+  auto count = [&]() -> it_status {
+    IT_CUDA_TRY(cudaMemsetAsync(p.totals, 0, sizeof(h), st));
+    if (n > 0) {
+      IT_LAUNCH(IT_K_SPLIT_SCAN, 0, 0, st, split_count_kernel<<<(unsigned)p.n_tiles, SPLIT_THREADS, 0, st>>>(p));
+      IT_LAUNCH(IT_K_SPLIT_SCAN, 0, 0, st, split_scan_kernel<<<(unsigned)(p.B.nb + 2), 1024, 0, st>>>(p));
     }
-    SPLIT_TRY(scan_and_emit(IT_K_BUCKET_SCAN, R, InBucket{g->shadow_indptr, B, b},
-                            EmitBucketRow{g->shadow_indptr, B, b, g->bucket_rows, g->bucket_offsets}, d_scratch,
-                            d_total, st));
-    IT_LAUNCH(IT_K_BUCKET_SCAN, 0, 0, st, set_next_bucket_offset_kernel<<<1, 1, 0, st>>>(g->bucket_offsets, b, d_total));
-    SPLIT_TRY(scan_and_emit(IT_K_BUCKET_SCAN, R, EdgesInBucket{g->shadow_indptr, B, b}, EmitNothing{}, d_scratch,
-                            d_edges + b, st));
+    IT_CUDA_TRY(cudaGetLastError());
+    return IT_OK;
+  };
+  auto read_totals = [&]() -> it_status {
+    IT_CUDA_TRY(cudaMemcpyAsync(h, p.totals, sizeof(h), cudaMemcpyDeviceToHost, st));
+    IT_CUDA_TRY(cudaStreamSynchronize(st));
+    return IT_OK;
+  };
+  if (count_first) {
+    IT_TRY(reserve(carve_split(g, p, nullptr, 0, 0)));
+    carve_split(g, p, g->slab, 0, 0);
+    IT_TRY(count());
+    IT_TRY(read_totals());
+    R = h[p.B.nb]; S = h[p.B.nb + 1];
+    if (R > (int64_t)INT32_MAX - 1) {
+      it_set_error("split produces %lld shadow rows; row ids are 32-bit", (long long)R);
+      return IT_ERR_UNSUPPORTED;
+    }
   }
-  if (R > 0)
-    IT_LAUNCH(IT_K_BUCKET_SCAN, 0, 0, st,
-              fill_bucket_meta_kernel<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(R, g->bucket_rows, g->shadow_indptr,
-                                                                                    g->row_dest, g->shadow_owner, g->bucket_meta, g->bucket_owner));
-  SPLIT_CUDA(cudaGetLastError());
-  SPLIT_CUDA(cudaMemcpyAsync(g->h_bucket_edges, d_edges, B.nb * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-  SPLIT_CUDA(cudaMemcpyAsync(g->h_bucket_offsets, g->bucket_offsets, (B.nb + 1) * sizeof(int64_t),
-                             cudaMemcpyDeviceToHost, st));
-  SPLIT_CUDA(cudaStreamSynchronize(st));
-  cudaFree(d_scratch);
-#undef SPLIT_TRY
-#undef SPLIT_CUDA
+  IT_TRY(reserve(carve_split(g, p, nullptr, R, S)));
+  carve_split(g, p, g->slab, R, S);
+  IT_TRY(count());
+  if (n > 0) {
+    IT_LAUNCH(IT_K_BUCKET_SCAN, 0, 0, st, split_emit_kernel<<<(unsigned)p.n_tiles, SPLIT_THREADS, 0, st>>>(p));
+    if (S > 0) {
+      const int64_t cap = (int64_t)g->num_sms * 16;
+      IT_LAUNCH(IT_K_SPLIT_FILL, 0, 0, st, fill_split_rows_kernel<<<(unsigned)(S < cap ? S : cap), 128, 0, st>>>(p));
+    }
+  } else {
+    IT_CUDA_TRY(cudaMemsetAsync(g->slab, 0, g->slab_bytes, st));
+  }
+  IT_CUDA_TRY(cudaGetLastError());
+  IT_TRY(read_totals());
+  g->shadow_indptr = p.shadow_indptr; g->shadow_owner = p.shadow_owner; g->owner_indptr = p.owner_indptr; g->split_owners = p.split_owners;
+  g->bucket_offsets = p.bucket_offsets; g->bucket_rows = p.bucket_rows; g->bucket_meta = p.bucket_meta; g->bucket_owner = p.bucket_owner;
+  g->n_rows = h[p.B.nb];
+  g->n_split_owners = h[p.B.nb + 1];
+  g->n_partial_rows = g->n_rows - (n - g->n_split_owners);
+  g->n_buckets = p.B.nb;
+  g->h_bucket_offsets[0] = 0;
+  for (int k = 0; k < p.B.nb; ++k) {
+    g->h_bucket_offsets[k + 1] = g->h_bucket_offsets[k] + h[k];
+    g->h_bucket_edges[k] = h[SPLIT_COLS + k];
+  }
+  for (int i = 0; i < IT_MAX_BUCKETS; ++i) g->bucket_bounds[i] = i < p.B.nb ? p.B.b[i] : 0;
   return IT_OK;
 }
 
@@ -409,25 +488,25 @@ static it_status create_impl(int64_t n, int64_t n_src, int64_t e, const void *in
   IT_REQUIRE(indptr_type == IT_I64 || e <= (int64_t)INT32_MAX, IT_ERR_INVALID_ARG, "int32 indptr cannot index %lld edges", (long long)e);
   cudaStream_t st = (cudaStream_t)stream;
 
-  int *d_flags = nullptr;
-  IT_CUDA_TRY(cudaMalloc(&d_flags, sizeof(int)));
+  // one word: the validation's flags, and later the status of the graph's kernels
+  int *d_status = nullptr;
+  IT_CUDA_TRY(cudaMalloc(&d_status, sizeof(int)));
   IndptrView ip{indptr, indptr_type == IT_I64};
-  cudaError_t ce = cudaMemsetAsync(d_flags, 0, sizeof(int), st);
+  cudaError_t ce = cudaMemsetAsync(d_status, 0, sizeof(int), st);
   int h_flags = 0;
   if (ce == cudaSuccess) {
-    IT_LAUNCH(IT_K_VALIDATE, 0, 0, st, validate_indptr_kernel<<<(unsigned)((n + 1 + 255) / 256), 256, 0, st>>>(ip, n, e, d_flags));
-    ce = cudaMemcpyAsync(&h_flags, d_flags, sizeof(int), cudaMemcpyDeviceToHost, st);
+    IT_LAUNCH(IT_K_VALIDATE, 0, 0, st, validate_indptr_kernel<<<(unsigned)((n + 1 + 255) / 256), 256, 0, st>>>(ip, n, e, d_status));
+    if (e > 0) {   // the caller vouches for e source ids, whatever indptr says
+      const int64_t want = (e / 4 + 255) / 256, cap = (int64_t)IT_NUM_SMS_FALLBACK * 8;
+      int head = (int)(((16 - ((uintptr_t)indices & 15)) & 15) / 4);
+      if (head > e) head = (int)e;
+      IT_LAUNCH(IT_K_VALIDATE, 0, 0, st, validate_indices_kernel<<<(unsigned)(want < 1 ? 1 : (want < cap ? want : cap)), 256, 0, st>>>(indices, e, n_src, head, d_status));
+    }
+    ce = cudaGetLastError();
   }
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_flags, d_status, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-  // the source ids are only scanned once the indptr is known to be sane
-  if (ce == cudaSuccess && h_flags == 0 && e > 0) {
-    int64_t want = (e + 255) / 256;
-    unsigned blocks = (unsigned)(want < 148 * 16 ? want : 148 * 16);
-    IT_LAUNCH(IT_K_VALIDATE, 0, 0, st, validate_indices_kernel<<<blocks, 256, 0, st>>>(indices, e, n_src, d_flags));
-    ce = cudaMemcpyAsync(&h_flags, d_flags, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-  }
-  cudaFree(d_flags);
+  if (ce != cudaSuccess || h_flags != 0) cudaFree(d_status);
   if (ce != cudaSuccess) {
     it_set_error("graph validation failed to run: %s", cudaGetErrorString(ce));
     return IT_ERR_CUDA;
@@ -439,20 +518,16 @@ static it_status create_impl(int64_t n, int64_t n_src, int64_t e, const void *in
   }
 
   it_graph *g = new (std::nothrow) it_graph();
+  if (g == nullptr) cudaFree(d_status);
   IT_REQUIRE(g != nullptr, IT_ERR_OOM, "host allocation failed");
   g->n = n; g->n_src = n_src; g->e = e; g->indptr = indptr; g->indptr_type = indptr_type;
   g->indices = indices; g->edge_weights = edge_weights;
+  g->d_status = d_status;   // zero: the flags were
   cudaGetDevice(&g->device);
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device) == cudaSuccess && sms > 0) g->num_sms = sms;
-  if (cudaMalloc(&g->d_status, sizeof(int)) != cudaSuccess || cudaMemsetAsync(g->d_status, 0, sizeof(int), st) != cudaSuccess) {
-    it_set_error("allocating the status word failed");
-    cudaFree(g->d_status);
-    delete g;
-    return IT_ERR_OOM;
-  }
   it_status rc = split_impl(g, 0, st);
-  if (rc != IT_OK) { cudaFree(g->d_status); delete g; return rc; }
+  if (rc != IT_OK) { it_graph_destroy(g); return rc; }
   *out = g;
   return IT_OK;
 }
@@ -510,7 +585,7 @@ extern "C" it_status it_graph_check(it_graph *g, void *stream) {
 
 extern "C" it_status it_graph_destroy(it_graph *g) {
   if (!g) return IT_OK;
-  free_derived(g);
+  cudaFree(g->slab);
   cudaFree(g->d_status);
   delete g;
   return IT_OK;
