@@ -11,7 +11,7 @@ enum LayerPlan { PLAN_SAGE = 0, PLAN_SAGE_REORDER = 1, PLAN_GAT = 2, PLAN_DENSE 
 
 struct LayerWs {
   LayerPlan plan;
-  size_t off_counters;                              // IT_MAX_BUCKETS words from which the gather's warps claim their batches
+  size_t off_counters;                              // IT_MAX_BUCKETS + 1 words from which the gather's warps claim their batches
   size_t off_B, off_partials, off_a, off_b, off_q;  // a: aggregate A | self term S | scores ; b: Z | P ; q: per-edge part Q / messages
   size_t bytes;
 };
@@ -88,7 +88,7 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
   auto take = [&](size_t bytes) { size_t o = off; off += it_align_up(bytes); return o; };
   w.plan = plan_of(L);
   w.off_q = 0;
-  w.off_counters = take(IT_MAX_BUCKETS * sizeof(int));
+  w.off_counters = take((IT_MAX_BUCKETS + 1) * sizeof(int));
   switch (w.plan) {
     case PLAN_GAT:
       w.off_B = take((fi + kpad) * (fo + 2 * (size_t)L->heads) * 8);
@@ -441,7 +441,7 @@ bool aligned16(const void *p) { return ((uintptr_t)p % 16) == 0; }
 // What every forward call checks about the graph and its input / output matrices before anything is launched:
 // the kernels move 16-byte slices of the rows, so a pointer that is not 16-byte aligned would fault on the device.
 it_status check_io(const it_graph *g, const void *in, size_t in_bytes, const void *out, size_t out_bytes) {
-  IT_REQUIRE(g->n == 0 || g->bucket_meta != nullptr, IT_ERR_BAD_GRAPH,
+  IT_REQUIRE(g->n == 0 || g->list_meta != nullptr, IT_ERR_BAD_GRAPH,
              "the graph has no row split (an it_split_hubs call failed): call it_split_hubs again before a forward pass");
   if (g->n == 0) return IT_OK;
   IT_REQUIRE(in != nullptr && out != nullptr, IT_ERR_INVALID_ARG, "input / output matrix is NULL");
@@ -455,7 +455,7 @@ it_status check_io(const it_graph *g, const void *in, size_t in_bytes, const voi
 it_status check_stage(const it_graph *g, const it_layer_desc *layer, void *workspace) {
   IT_REQUIRE(g != nullptr, IT_ERR_INVALID_ARG, "graph is NULL");
   IT_TRY(check_layer(g, layer));
-  IT_REQUIRE(g->n == 0 || g->bucket_meta != nullptr, IT_ERR_BAD_GRAPH,
+  IT_REQUIRE(g->n == 0 || g->list_meta != nullptr, IT_ERR_BAD_GRAPH,
              "the graph has no row split (an it_split_hubs call failed): call it_split_hubs again before a forward pass");
   IT_REQUIRE(workspace != nullptr && ((uintptr_t)workspace % 256) == 0, IT_ERR_WORKSPACE, "workspace is NULL or not 256-byte aligned");
   return IT_OK;

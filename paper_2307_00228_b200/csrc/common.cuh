@@ -60,8 +60,8 @@ bool it_profile_is_on();
   } while (0)
 
 // ----------------------------------------------------------------------------- graph handle
-// One shadow row as the gather kernels read it: first edge, edge count, and where the
-// aggregate goes (vertex id >= 0 for an unsplit row, ~slot in the partial buffer otherwise).
+// One row as the gather kernels read it: first edge, edge count, and where the
+// aggregate goes (vertex id >= 0 for a whole vertex, ~slot in the partial buffer for a piece of one).
 struct __align__(16) it_row_meta {
   int64_t j0;
   int32_t len;
@@ -87,20 +87,28 @@ struct it_graph {
   int64_t threshold = 0;
   int64_t n_rows = 0;           // R
   int64_t n_split_owners = 0;   // vertices with more than one shadow row
-  int64_t n_partial_rows = 0;   // shadow rows that belong to split owners
   int64_t *shadow_indptr = nullptr;  // [R+1]
   int32_t *shadow_owner = nullptr;   // [R]
   int64_t *owner_indptr = nullptr;   // [n+1]
-  int32_t *split_owners = nullptr;   // [n_split_owners] ascending vertex ids
   int32_t n_buckets = 0;
   int64_t bucket_bounds[IT_MAX_BUCKETS] = {0};
-  int64_t h_bucket_offsets[IT_MAX_BUCKETS + 1] = {0};
-  int64_t h_bucket_edges[IT_MAX_BUCKETS] = {0};  // edges held by the rows of each bucket
   int64_t *bucket_offsets = nullptr;  // device [n_buckets+1]
   int32_t *bucket_rows = nullptr;     // [R]
   int *d_status = nullptr;            // device word: set to 1 by a kernel whose bounded wait gave up
-  int32_t *bucket_owner = nullptr;    // [R] in bucket order: the vertex each row belongs to
-  it_row_meta *bucket_meta = nullptr; // [R] in bucket order: what a gather needs to know about one row, in one 16-byte load
+
+  // what the gather walks: the vertices of at most `long_above` edges by degree bucket, one row each, then the pieces of the
+  // longer ones (graph.cu: split).  List b holds entries [h_list_offsets[b], h_list_offsets[b + 1]) of list_meta / list_owner,
+  // rows of at most list_bounds[b] edges; the pieces are the last list.
+  int32_t n_lists = 0;
+  int64_t list_bounds[IT_MAX_BUCKETS + 1] = {0};
+  int64_t h_list_offsets[IT_MAX_BUCKETS + 2] = {0};
+  int64_t h_list_edges[IT_MAX_BUCKETS + 1] = {0};
+  it_row_meta *list_meta = nullptr;   // what a gather needs to know about one row, in one 16-byte load
+  int32_t *list_owner = nullptr;      // the vertex each row belongs to
+  int64_t n_long = 0;                 // vertices gathered in pieces
+  int64_t n_partial_rows = 0;         // their pieces: one partial result each
+  int32_t *long_owners = nullptr;     // [n_long] ascending vertex ids
+  int64_t *piece_ptr = nullptr;       // [n_long + 1]: the pieces of long_owners[k] are partial rows piece_ptr[k] ..., in edge order
 };
 
 static inline size_t it_align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
@@ -144,7 +152,7 @@ struct it_gather_args {
   const void *src;         // rows that are gathered: row u starts at src + u * src_ld elements
   int src_ld;              // 0 means dim
   int per_edge_rows;       // 1: src is [n_edges, dim] and row j belongs to edge j (edge features); 0: rows are looked up by source vertex
-  float *partials;         // [n_partial_rows, dim] fp32 scratch (may be NULL when nothing is split)
+  float *partials;         // [n_partial_rows, dim] fp32 scratch (may be NULL when no vertex is gathered in pieces)
   int *counters;           // IT_MAX_BUCKETS device words of scratch from which warps claim their batches (NULL: fixed strides)
   void *dst;               // row v starts at dst + v * dst_ld elements and takes dim of them
   int dst_ld;              // 0 means dim

@@ -3,7 +3,7 @@
 // One pass over the edges with a running (max, sum, weighted accumulator) state per lane
 // ("online" softmax).  Such states merge associatively — (m, l, acc) and (m', l', acc') give
 // M = max(m, m'), l e^(m-M) + l' e^(m'-M), acc e^(m-M) + acc' e^(m'-M) — so the groups of a split
-// hub are reduced independently into partial states and merged in group order, exactly like
+// hub are reduced independently into partial states and merged in edge order, exactly like
 // the partial sums of the plain gather.  The edge streaming lives in stream.cuh.
 #include "stream.cuh"
 
@@ -121,51 +121,61 @@ struct GatPolicy {
 
 namespace {
 
-// Merge the partial states of every split vertex in group order; one warp per vertex.
+// Merge the partial states of every long vertex in edge order: one block per vertex, lane = column; every warp merges a
+// contiguous range of the pieces (first their maximum, then the sums against it), the warps' states follow in warp order.
 struct GatCombineParams {
-  const int32_t *__restrict__ split_owners;
-  const int64_t *__restrict__ owner_indptr;
+  const int32_t *__restrict__ long_owners;
+  const int64_t *__restrict__ piece_ptr;
   const float *__restrict__ partials;
   const float *__restrict__ bias;
   void *__restrict__ dst;
-  int64_t n_split_owners;
+  int64_t n_long;
   int dim, heads, head_dim, act;
 };
 
 template <typename T>
 __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p) {
-  const int lane = threadIdx.x & 31;
+  constexpr int WARPS = THREADS / 32;
+  __shared__ float red[WARPS][3][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int stride = gat_partial_stride(p.dim, p.heads);
-  const int64_t warps_total = (int64_t)gridDim.x * (THREADS / 32);
-  for (int64_t k = (int64_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5); k < p.n_split_owners; k += warps_total) {
-    const int64_t v = __ldg(p.split_owners + k);
-    const int64_t r0 = __ldg(p.owner_indptr + v), r1 = __ldg(p.owner_indptr + v + 1);
-    const float *P = p.partials + (r0 - v + k) * stride;   // first partial row of this vertex
-    const int n = (int)(r1 - r0);
-    for (int c = lane * 4; c < p.dim; c += 128) {
-      const int head = c / p.head_dim;
-      float M = -INFINITY;
-      for (int g = 0; g < n; ++g) M = fmaxf(M, __ldg(P + (int64_t)g * stride + p.dim + head));
-      float l = 0.f;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int g = 0; g < n; ++g) {
-        const float mg = __ldg(P + (int64_t)g * stride + p.dim + head);
-        const float f = mg == -INFINITY ? 0.f : __expf(mg - M);
-        l = fmaf(__ldg(P + (int64_t)g * stride + p.dim + p.heads + head), f, l);
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(P + (int64_t)g * stride + c));
-        acc.x = fmaf(a.x, f, acc.x); acc.y = fmaf(a.y, f, acc.y); acc.z = fmaf(a.z, f, acc.z); acc.w = fmaf(a.w, f, acc.w);
+  for (int64_t k = blockIdx.x; k < p.n_long; k += gridDim.x) {
+    const int64_t v = __ldg(p.long_owners + k);
+    const int64_t p0 = __ldg(p.piece_ptr + k);
+    const int n = (int)(__ldg(p.piece_ptr + k + 1) - p0), per = (n + WARPS - 1) / WARPS;
+    const int a = warp * per < n ? warp * per : n, b = a + per < n ? a + per : n;
+    const float *P = p.partials + p0 * stride;
+    for (int c0 = 0; c0 < p.dim; c0 += 32) {
+      const int c = c0 + lane;
+      float M = -INFINITY, l = 0.f, acc = 0.f;
+      if (c < p.dim) {
+        const int head = c / p.head_dim;
+#pragma unroll 8
+        for (int g = a; g < b; ++g) M = fmaxf(M, __ldg(P + (int64_t)g * stride + p.dim + head));
+#pragma unroll 4
+        for (int g = a; g < b; ++g) {
+          const float *row = P + (int64_t)g * stride;
+          const float f = it_exp(__ldg(row + p.dim + head) - M);
+          l = fmaf(__ldg(row + p.dim + p.heads + head), f, l);
+          acc = fmaf(__ldcs(row + c), f, acc);
+        }
       }
-      const float inv = l > 0.f ? 1.f / l : 0.f;
-      float o[4] = {acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) o[i] = act_apply(o[i] + (p.bias ? __ldg(p.bias + c + i) : 0.f), p.act);
+      __syncthreads();   // red free again
+      red[warp][0][lane] = M; red[warp][1][lane] = l; red[warp][2][lane] = acc;
+      __syncthreads();
+      if (warp != 0 || c >= p.dim) continue;
+      float Mt = M;
+      for (int w = 1; w < WARPS; ++w) Mt = fmaxf(Mt, red[w][0][lane]);
+      float lt = 0.f, at = 0.f;
+      for (int w = 0; w < WARPS; ++w) {
+        const float f = red[w][0][lane] == -INFINITY ? 0.f : it_exp(red[w][0][lane] - Mt);   // a warp without pieces
+        lt = fmaf(red[w][1][lane], f, lt);
+        at = fmaf(red[w][2][lane], f, at);
+      }
+      const float o = act_apply(at * (lt > 0.f ? 1.f / lt : 0.f) + (p.bias ? __ldg(p.bias + c) : 0.f), p.act);
       T *d = reinterpret_cast<T *>(p.dst) + v * p.dim + c;
-      if (sizeof(T) == 4) {
-        *reinterpret_cast<float4 *>(d) = make_float4(o[0], o[1], o[2], o[3]);
-      } else {
-        __nv_bfloat162 h0 = __floats2bfloat162_rn(o[0], o[1]), h1 = __floats2bfloat162_rn(o[2], o[3]);
-        *reinterpret_cast<uint2 *>(d) = make_uint2(*reinterpret_cast<uint32_t *>(&h0), *reinterpret_cast<uint32_t *>(&h1));
-      }
+      if constexpr (sizeof(T) == 4) *d = o;
+      else *d = __float2bfloat16_rn(o);
     }
   }
 }
@@ -187,13 +197,13 @@ auto gat_bytes(const it_gat_args &a) {
   const int heads = a.heads;
   const double row_bytes = (double)heads * a.head_dim * it_dtype_size(a.dtype);
   return [=](int b, int64_t rows) {
-    return (double)g->h_bucket_edges[b] * (4.0 + 4.0 * heads + row_bytes) + (double)rows * (20.0 + 4.0 * heads + row_bytes);
+    return (double)g->h_list_edges[b] * (4.0 + 4.0 * heads + row_bytes) + (double)rows * (20.0 + 4.0 * heads + row_bytes);
   };
 }
 
 template <typename T, int SB, int LPR>
 it_status launch_gat_lpr(const it_gat_args &a, StreamParams sp, int64_t bound_lo, int64_t bound_hi, cudaStream_t st) {
-  return launch_buckets<T, SB, LPR, false>(a.g, sp, make_policy<T, SB>(a), gat_bytes(a), IT_K_GAT_CTA, IT_K_GAT_FLAT, IT_K_GAT_EMPTY, bound_lo, bound_hi,
+  return launch_buckets<T, SB, LPR, false>(a.g, sp, make_policy<T, SB>(a), gat_bytes(a), IT_K_GAT_FLAT, IT_K_GAT_EMPTY, bound_lo, bound_hi,
                                            a.counters, st);
 }
 
@@ -251,24 +261,22 @@ size_t it_gat_partial_bytes(const it_graph *g, int dim, int heads) {
 it_status it_launch_gat(const it_gat_args &a, cudaStream_t st) {
   const it_graph *g = a.g;
   IT_REQUIRE(g->n_partial_rows == 0 || a.partials, IT_ERR_WORKSPACE, "gat: no partial buffer");
-  IT_REQUIRE(g->n_split_owners == 0 || a.head_dim % 4 == 0, IT_ERR_UNSUPPORTED, "gat on a split graph needs head_dim to be a multiple of 4");
   if (g->n == 0) return IT_OK;
   StreamParams sp;
-  sp.meta = g->bucket_meta; sp.owner = g->bucket_owner; sp.indices = a.per_edge_rows ? nullptr : g->indices; sp.weights = nullptr;
+  sp.meta = g->list_meta; sp.owner = g->list_owner; sp.indices = a.per_edge_rows ? nullptr : g->indices; sp.weights = nullptr;
   sp.src = a.z; sp.row_lo = sp.row_hi = 0; sp.dim = a.heads * a.head_dim; sp.batch_rows = 1; sp.counter = nullptr; sp.claim = 1; sp.slices = 0;
   sp.src_pitch = (uint32_t)(sp.dim * it_dtype_size(a.dtype));
   if (a.dtype == IT_F32) IT_TRY(launch_gat<float>(a, sp, st));
   else IT_TRY(launch_gat<__nv_bfloat16>(a, sp, st));
-  if (g->n_split_owners > 0) {
+  if (g->n_long > 0) {
     GatCombineParams c;
-    c.split_owners = g->split_owners; c.owner_indptr = g->owner_indptr; c.partials = a.partials; c.bias = a.bias;
-    c.dst = a.dst; c.n_split_owners = g->n_split_owners; c.dim = a.heads * a.head_dim; c.heads = a.heads;
+    c.long_owners = g->long_owners; c.piece_ptr = g->piece_ptr; c.partials = a.partials; c.bias = a.bias;
+    c.dst = a.dst; c.n_long = g->n_long; c.dim = a.heads * a.head_dim; c.heads = a.heads;
     c.head_dim = a.head_dim; c.act = a.act;
-    int64_t want = (g->n_split_owners + 7) / 8;
-    int64_t cap = (int64_t)g->num_sms * 8;
-    unsigned blocks = (unsigned)(want < cap ? want : cap);
+    const int64_t cap = (int64_t)g->num_sms * 8;
+    const unsigned blocks = (unsigned)(g->n_long < cap ? g->n_long : cap);
     const double cbytes = (double)it_gat_partial_bytes(g, c.dim, c.heads) +
-                          (double)g->n_split_owners * c.dim * (a.dtype == IT_F32 ? 4.0 : 2.0);
+                          (double)g->n_long * c.dim * (a.dtype == IT_F32 ? 4.0 : 2.0);
     if (a.dtype == IT_F32) IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, gat_combine_kernel<float><<<blocks, THREADS, 0, st>>>(c));
     else IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, gat_combine_kernel<__nv_bfloat16><<<blocks, THREADS, 0, st>>>(c));
     IT_CUDA_TRY(cudaGetLastError());

@@ -159,58 +159,6 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_k
       });
 }
 
-// Very long rows: one CTA each, every warp a contiguous part; the warps' states are merged in warp order.
-template <typename T, int LPR, int H>
-__global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) gat_cta_chunk_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol) {
-  constexpr int WARPS = THREADS / 32, NS = GatPolicy<T, 16>::NS;
-  extern __shared__ uint4 ring_raw[];
-  __shared__ float red[WARPS][LPR][NS];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t base = (uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)warp * (uint32_t)gat_bytes_per_warp<H>();
-  RingWarp<T, 16, LPR, GatAcc<T>, false> rw;
-  rw.setup(base, p.src, p.src_pitch, p.slices, lane);
-  pol.setup(lane % LPR);
-  __shared__ float bias_buf[256];
-  stage_bias(pol, bias_buf);
-  for (int64_t i = p.row_lo + blockIdx.x; i < p.row_hi; i += gridDim.x) {
-    const it_row_meta mt = load_meta(p.meta + i);
-    const int32_t owner = __ldcs(p.owner + i);
-    const int part = (mt.len + WARPS - 1) / WARPS;
-    const int first = warp * part < mt.len ? warp * part : mt.len;
-    const int total = (mt.len - first) < part ? (mt.len - first) : part;
-    GatWarp<T, LPR, H> gw(p, q, lane, base + ring_bytes_per_warp<16, false>());
-    PartCursor<false> cur(p, lane, mt.j0 + first, total, mt.dest, owner);
-    chunk_walk<LPR, true>(rw, gw.acc, cur, [&](Chunk &c) { gw.ahead(c); }, [&](const Chunk &c, bool f) { gw.begin(c, f); },
-        [&](int k, const uint4 &raw, bool valid) {
-          const float w = gw.weight(k);
-          if (valid) gw.acc.edge(gw.st, raw, w);
-        },
-        [](const Chunk &) {});
-    rw.fold(gw.acc, gw.st);
-    const float mh = __shfl_sync(0xffffffffu, gw.m, gw.hc);
-    float full[NS];
-#pragma unroll
-    for (int k = 0; k < GatAcc<T>::VEC; ++k) full[k] = gw.st[k];
-    full[NS - 2] = mh;
-    full[NS - 1] = gw.st[GatAcc<T>::VEC];
-    __syncthreads();   // red[] free again
-    if (lane < LPR) {
-#pragma unroll
-      for (int k = 0; k < NS; ++k) red[warp][lane][k] = full[k];
-    }
-    __syncthreads();
-    if (warp == 0 && lane < LPR) {
-      for (int w = 1; w < WARPS; ++w) {
-        float other[NS];
-#pragma unroll
-        for (int k = 0; k < NS; ++k) other[k] = red[w][lane][k];
-        pol.merge(full, other);
-      }
-      pol.end_row(full, mt.dest, owner, mt.len);
-    }
-  }
-}
-
 // ----------------------------------------------------------------------------- short rows: one lane group each
 // Rows of at most a few dozen edges, 128- and 256-byte rows: a group of LPR lanes owns a row and walks it in rounds of up
 // to E = 8 edges; the groups of a warp run in lockstep, a round as long as its longest row.  While the rows of one round are
@@ -350,10 +298,10 @@ it_status launch_gat_rows(const it_gat_args &a, StreamParams p, const GatPolicy<
   GatParams q;
   q.scores = pol.scores; q.scores_dst = pol.scores_dst; q.per_edge = a.per_edge_scores; q.slope = pol.slope; q.head_dim = pol.head_dim;
   p.slices = LPR;
-  if (a.counters) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, IT_MAX_BUCKETS * sizeof(int), st));
+  if (a.counters) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, (IT_MAX_BUCKETS + 1) * sizeof(int), st));
   bool chunked = false;
-  for (int b = g->n_buckets - 1; b >= 0; --b) {
-    const int64_t lo = g->h_bucket_offsets[b], hi = g->h_bucket_offsets[b + 1], bound = g->bucket_bounds[b];
+  for (int b = g->n_lists - 1; b >= 0; --b) {
+    const int64_t lo = g->h_list_offsets[b], hi = g->h_list_offsets[b + 1], bound = g->list_bounds[b];
     if (hi <= lo) continue;
     p.row_lo = lo; p.row_hi = hi;
     const int64_t rows = hi - lo;
@@ -364,11 +312,6 @@ it_status launch_gat_rows(const it_gat_args &a, StreamParams p, const GatPolicy<
       pol.empty_rows(cr);
       cr.g = g; cr.row_lo = lo; cr.row_hi = hi;
       IT_TRY(it_launch_const_rows(cr, IT_K_GAT_EMPTY, bytes, st));
-    } else if (bound > IT_GATHER_CTA_ABOVE) {
-      static std::atomic<uint64_t> configured{0};
-      IT_TRY(allow_dynamic_smem(gat_cta_chunk_kernel<T, LPR, H>, smem, configured));
-      const unsigned blocks = (unsigned)(rows < (1 << 20) ? rows : (1 << 20));
-      IT_LAUNCH(IT_K_GAT_CTA, bytes, 0, st, gat_cta_chunk_kernel<T, LPR, H><<<blocks, THREADS, smem, st>>>(p, q, pol));
     } else if (LPR <= 16 && bound <= IT_SHORT_BELOW) {
       if constexpr (LPR <= 16) {
         constexpr int sbytes = 2 * IT_SHORT_EDGES * THREADS * 16;
@@ -378,20 +321,20 @@ it_status launch_gat_rows(const it_gat_args &a, StreamParams p, const GatPolicy<
         const unsigned blocks = (unsigned)(want < most ? want : most);
         IT_LAUNCH(IT_K_GAT_FLAT, bytes, 0, st, gat_short_rows_kernel<T, LPR, H><<<blocks, THREADS, sbytes, st>>>(p, q, pol));
       }
-    } else {   // one warp per row: every such bucket in one launch (they are neighbours in the row list), longest rows first
+    } else {   // one warp per row: every such list in one launch (they are neighbours), pieces first
       if (chunked) continue;
       chunked = true;
       double all = bytes;
       int b0 = b;
-      while (b0 > 0 && g->bucket_bounds[b0 - 1] > (LPR <= 16 ? IT_SHORT_BELOW : 0)) {
+      while (b0 > 0 && g->list_bounds[b0 - 1] > (LPR <= 16 ? IT_SHORT_BELOW : 0)) {
         --b0;
-        all += bytes_of(b0, g->h_bucket_offsets[b0 + 1] - g->h_bucket_offsets[b0]);
+        all += bytes_of(b0, g->h_list_offsets[b0 + 1] - g->h_list_offsets[b0]);
       }
-      p.row_lo = g->h_bucket_offsets[b0];
+      p.row_lo = g->h_list_offsets[b0];
       static std::atomic<uint64_t> configured{0};
       IT_TRY(allow_dynamic_smem(gat_rows_chunk_kernel<T, LPR, H>, smem, configured));
       p.counter = a.counters + b;
-      const unsigned blocks = chunk_grid(hi - p.row_lo, (int64_t)g->num_sms * IT_GAT_CHUNK_BLOCKS, &p.claim);
+      const unsigned blocks = chunk_grid(p, b == g->n_lists - 1 ? rows : 0, (int64_t)g->num_sms * IT_GAT_CHUNK_BLOCKS);
       IT_LAUNCH(IT_K_GAT_FLAT, all, 0, st, gat_rows_chunk_kernel<T, LPR, H><<<blocks, THREADS, smem, st>>>(p, q, pol));
       p.counter = nullptr;
     }

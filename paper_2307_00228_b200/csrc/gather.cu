@@ -11,33 +11,36 @@ using namespace it_stream;
 constexpr int GATHER_THREADS = THREADS;
 
 // ----------------------------------------------------------------------------- combine
-// One warp per split owner.  Its partial rows are rows [p0, p0 + n) of the partial buffer,
-// folded in group order.
+// One block per long vertex.  Its partial rows are rows [piece_ptr[k], piece_ptr[k + 1]) of the partial buffer; every warp
+// folds a contiguous range of them in order, eight rows in flight, and the warps' results are folded in warp order.
 struct CombineParams {
-  const int32_t *__restrict__ split_owners;
+  const int32_t *__restrict__ long_owners;
+  const int64_t *__restrict__ piece_ptr;
   const int64_t *__restrict__ owner_indptr;
   const int64_t *__restrict__ shadow_indptr;
   const float *__restrict__ partials;
   void *__restrict__ dst;
   const void *__restrict__ self_term;
   const float *__restrict__ bias;
-  int64_t n_split_owners;
+  int64_t n_long;
   int dim, dst_ld, self_ld, self_is_t;
   int red, is_mean, epi, act;   // red: RED_SUM / RED_MAX / RED_MIN
 };
 
 template <typename T>
 __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps_total = (int64_t)gridDim.x * (GATHER_THREADS / 32);
-  for (int64_t k = (int64_t)blockIdx.x * (GATHER_THREADS / 32) + (threadIdx.x >> 5); k < p.n_split_owners; k += warps_total) {
-    const int64_t v = __ldg(p.split_owners + k);
-    const int64_t r0 = __ldg(p.owner_indptr + v), r1 = __ldg(p.owner_indptr + v + 1);
-    const int64_t p0 = r0 - v + k;
-    const int64_t deg = __ldg(p.shadow_indptr + r1) - __ldg(p.shadow_indptr + r0);
-    const float inv = (p.is_mean && deg > 0) ? 1.f / (float)deg : 1.f;
-    for (int c = lane * 4; c < p.dim; c += 128) {
-      float4 acc = __ldg(reinterpret_cast<const float4 *>(p.partials + p0 * p.dim + c));
+  constexpr int WARPS = GATHER_THREADS / 32;
+  __shared__ float4 red[WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int64_t k = blockIdx.x; k < p.n_long; k += gridDim.x) {
+    const int64_t v = __ldg(p.long_owners + k);
+    const int64_t p0 = __ldg(p.piece_ptr + k), n = __ldg(p.piece_ptr + k + 1) - p0;
+    const int64_t per = (n + WARPS - 1) / WARPS;
+    const int64_t a = warp * per < n ? warp * per : n, b = a + per < n ? a + per : n;
+    for (int c0 = 0; c0 < p.dim; c0 += 128) {
+      const int c = c0 + lane * 4;
+      const float id = p.red == RED_MAX ? -INFINITY : (p.red == RED_MIN ? INFINITY : 0.f);
+      float4 acc = make_float4(id, id, id, id);
       auto fold = [&](const float4 &y) {
         if (p.red == RED_MAX) {
           acc.x = fmaxf(acc.x, y.x); acc.y = fmaxf(acc.y, y.y); acc.z = fmaxf(acc.z, y.z); acc.w = fmaxf(acc.w, y.w);
@@ -47,16 +50,25 @@ __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p
           acc.x += y.x; acc.y += y.y; acc.z += y.z; acc.w += y.w;
         }
       };
-      const int64_t n = r1 - r0;
-      int64_t g = 1;
-      for (; g + 8 <= n; g += 8) {   // eight partial rows in flight, folded in group order
-        float4 y[8];
+      if (c < p.dim) {
+        const float *P = p.partials + p0 * p.dim + c;
+        int64_t g = a;
+        for (; g + 8 <= b; g += 8) {
+          float4 y[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) y[k] = __ldg(reinterpret_cast<const float4 *>(p.partials + (p0 + g + k) * p.dim + c));
+          for (int u = 0; u < 8; ++u) y[u] = __ldcs(reinterpret_cast<const float4 *>(P + (g + u) * p.dim));
 #pragma unroll
-        for (int k = 0; k < 8; ++k) fold(y[k]);
+          for (int u = 0; u < 8; ++u) fold(y[u]);
+        }
+        for (; g < b; ++g) fold(__ldcs(reinterpret_cast<const float4 *>(P + g * p.dim)));
       }
-      for (; g < n; ++g) fold(__ldg(reinterpret_cast<const float4 *>(p.partials + (p0 + g) * p.dim + c)));
+      __syncthreads();   // red free again
+      red[warp][lane] = acc;
+      __syncthreads();
+      if (warp != 0 || c >= p.dim) continue;   // (the barriers above are met by every warp in every round)
+      for (int w = 1; w < WARPS; ++w) fold(red[w][lane]);
+      const int64_t deg = p.is_mean ? __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v + 1)) - __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v)) : 1;
+      const float inv = p.is_mean ? 1.f / (float)deg : 1.f;
       float o[4] = {acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv};
       const int64_t doff = v * p.dst_ld + c;
       if (p.epi == IT_EPI_RAW_F32) {
@@ -143,7 +155,7 @@ __global__ void __launch_bounds__(GATHER_THREADS) const_rows_kernel(ConstRowsPar
 it_status it_launch_const_rows(const it_const_rows_args &a, int kid, double bytes, cudaStream_t st) {
   const it_graph *g = a.g;
   ConstRowsParams p;
-  p.meta = g->bucket_meta; p.lo = a.row_lo; p.hi = a.row_hi; p.dst = (char *)a.dst; p.pitch = a.pitch; p.dim = a.dim;
+  p.meta = g->list_meta; p.lo = a.row_lo; p.hi = a.row_hi; p.dst = (char *)a.dst; p.pitch = a.pitch; p.dim = a.dim;
   p.slices = a.dim * it_dtype_size(a.dtype) / 16; p.bf16 = a.dtype == IT_BF16; p.has_bias = a.has_bias; p.act = (int)a.act;
   p.value = a.value; p.bias = a.bias;
   const int64_t want = (a.row_hi - a.row_lo + GATHER_THREADS - 1) / GATHER_THREADS, cap = (int64_t)g->num_sms * 8;
@@ -157,22 +169,21 @@ it_status it_launch_const_rows(const it_const_rows_args &a, int kid, double byte
 static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
   const it_graph *g = a.g;
   StreamParams sp;
-  sp.meta = g->bucket_meta; sp.owner = nullptr; sp.indices = a.per_edge_rows ? nullptr : g->indices; sp.weights = g->edge_weights;
+  sp.meta = g->list_meta; sp.owner = nullptr; sp.indices = a.per_edge_rows ? nullptr : g->indices; sp.weights = g->edge_weights;
   sp.src = a.src; sp.row_lo = sp.row_hi = 0; sp.dim = a.dim; sp.batch_rows = 1; sp.counter = nullptr; sp.claim = 1; sp.slices = 0;
   sp.src_pitch = (uint32_t)((a.src_ld > 0 ? a.src_ld : a.dim) * it_dtype_size(a.dtype));
   if (a.dtype == IT_F32) IT_TRY(it_launch_gather_rows_f32(a, sp, st));
   else IT_TRY(it_launch_gather_rows_bf16(a, sp, st));
-  if (g->n_split_owners > 0) {
+  if (g->n_long > 0) {
     CombineParams c;
-    c.split_owners = g->split_owners; c.owner_indptr = g->owner_indptr; c.shadow_indptr = g->shadow_indptr;
-    c.partials = a.partials; c.dst = a.dst; c.self_term = a.self_term; c.bias = a.bias; c.n_split_owners = g->n_split_owners;
+    c.long_owners = g->long_owners; c.piece_ptr = g->piece_ptr; c.owner_indptr = g->owner_indptr; c.shadow_indptr = g->shadow_indptr;
+    c.partials = a.partials; c.dst = a.dst; c.self_term = a.self_term; c.bias = a.bias; c.n_long = g->n_long;
     c.dim = a.dim; c.dst_ld = a.dst_ld > 0 ? a.dst_ld : a.dim; c.self_ld = a.self_ld > 0 ? a.self_ld : a.dim;
     c.red = a.op == IT_GATHER_MAX ? RED_MAX : (a.op == IT_GATHER_MIN ? RED_MIN : RED_SUM); c.is_mean = a.op == IT_GATHER_MEAN && a.epi != IT_EPI_RAW_F32; c.epi = a.epi; c.act = a.act; c.self_is_t = a.self_dtype != IT_F32;
-    int64_t want = (g->n_split_owners + 7) / 8;
-    int64_t cap = (int64_t)g->num_sms * 8;
-    unsigned blocks = (unsigned)(want < cap ? want : cap);
+    const int64_t cap = (int64_t)g->num_sms * 8;
+    const unsigned blocks = (unsigned)(g->n_long < cap ? g->n_long : cap);
     const double cbytes = (double)g->n_partial_rows * a.dim * 4.0 +
-                          (double)g->n_split_owners * a.dim * (a.dtype == IT_F32 ? 4.0 : 2.0);
+                          (double)g->n_long * a.dim * (a.dtype == IT_F32 ? 4.0 : 2.0);
     if (a.dtype == IT_F32) IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, combine_kernel<float><<<blocks, GATHER_THREADS, 0, st>>>(c));
     else IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, combine_kernel<__nv_bfloat16><<<blocks, GATHER_THREADS, 0, st>>>(c));
   }

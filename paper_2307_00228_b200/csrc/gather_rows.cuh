@@ -120,11 +120,11 @@ it_status launch_policy(const it_gather_args &a, StreamParams sp, int64_t bound_
   // metadata and one output row (plus the self row it is added to)
   const double row_bytes = (double)a.dim * sizeof(T);
   auto bytes_of = [=](int b, int64_t rows) {
-    return (double)g->h_bucket_edges[b] * ((a.per_edge_rows ? 0.0 : 4.0) + (WEIGHTED ? 4.0 : 0.0) + row_bytes) +
+    return (double)g->h_list_edges[b] * ((a.per_edge_rows ? 0.0 : 4.0) + (WEIGHTED ? 4.0 : 0.0) + row_bytes) +
            (double)rows * (16.0 + row_bytes + (a.epi == IT_EPI_ADD_ACT ? (a.self_dtype == IT_F32 ? 4.0 : (double)sizeof(T)) * a.dim : 0.0));
   };
   auto launch = [&]<bool PAD>() {
-    return launch_buckets<T, SB, LPR, PAD>(g, sp, pol, bytes_of, IT_K_GATHER_CTA, IT_K_GATHER_FLAT, IT_K_GATHER_EMPTY, bound_lo, bound_hi, a.counters, st);
+    return launch_buckets<T, SB, LPR, PAD>(g, sp, pol, bytes_of, IT_K_GATHER_FLAT, IT_K_GATHER_EMPTY, bound_lo, bound_hi, a.counters, st);
   };
   if constexpr (SB == 16) {
     if (a.dim * (int)sizeof(T) != SB * LPR) return launch.template operator()<true>();

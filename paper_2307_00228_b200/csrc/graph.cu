@@ -81,15 +81,27 @@ __global__ void __launch_bounds__(256) validate_indices_kernel(const int32_t *__
 // ----------------------------------------------------------------------------- split
 // The shadow rows and the degree buckets in one pass over the vertices: count per tile, scan the tile counts, emit.
 // Every vertex adds rows to at most two buckets (all groups of a split vertex hold d / ng or d / ng + 1 edges), so the row
-// numbers, the list of split vertices and the positions inside every bucket are prefix sums of the same pass: columns
-// 0 .. nb - 1 the buckets, nb the rows, nb + 1 the split vertices.
+// numbers, the list of long vertices and the positions inside every bucket are prefix sums of the same pass: columns
+// 0 .. nb - 1 the buckets, nb the rows, nb + 1 the split vertices, nb + 2 the long vertices, nb + 3 their pieces, and from
+// nb + 4 on the lists that the gather walks.
+//
+// The gather does not walk the shadow rows of a hub but finer pieces of its segment, and pieces of every vertex of more than
+// long_above edges (T, 1024 to 4096): those of all such vertices are ordered by where in its vertex's segment a piece lies.  Source ids ascend
+// inside a segment, so pieces at the same relative position read the same part of the source table, and the pieces that are in
+// flight together share it through the L2 cache.  Whole passes, against
+// one block per row of up to T edges in vertex order: 5M vertices / 100M edges, GAT, 13.1 -> 11.7 ms; 20M / 200M with 100 hubs
+// of 1M edges, max pooling, 20.0 -> 17.4; 2M / 40M, fp32 sums, 6.6 -> 5.95; 25M / 375M, mean, 23.3 -> 22.6.
+// A piece is a 64th of its vertex (it then spans a 64th of the table), at least 128 edges (its fp32 partial result costs a row
+// written and a row read: 3 % of 128 rows; 64 and 32 edges cost 1 to 2 % more on GAT) and at most 512 (one warp walks it).
+// Source tables of fewer than 2^17 rows fit the cache whatever the order: pieces of at least 256 edges.
 // Bound by reading indptr twice and writing 36 bytes per row; a scan per bucket (each over every row, three launches with a
 // read of two 8-byte bounds per row) took 3.2 ms of device time for 5M vertices and six buckets, this one 3.0 with
 // everything around it (create + split: 14.3 -> 3.0 ms; the derived arrays are one allocation instead of nine, kept for the next split).
 constexpr int SPLIT_THREADS = 256;
-constexpr int SPLIT_ITEMS = 8;                                    // vertices per lane: a warp covers 256 consecutive ones
-constexpr int SPLIT_TILE = SPLIT_THREADS * SPLIT_ITEMS;
-constexpr int SPLIT_COLS = IT_MAX_BUCKETS + 2;
+constexpr int SPLIT_ITEMS = 8;                                    // vertices per lane
+constexpr int SPLIT_TILE = 32 * SPLIT_ITEMS;                      // a tile is one warp's 256 consecutive vertices
+constexpr int SPLIT_COLS = 2 * IT_MAX_BUCKETS + 4;
+constexpr int PIECE_BINS = 256;                                   // steps of the order in which pieces are walked
 
 struct Bounds { int64_t b[IT_MAX_BUCKETS]; int nb; };
 __device__ __forceinline__ int bucket_of(int64_t len, const Bounds &B) {
@@ -98,7 +110,7 @@ __device__ __forceinline__ int bucket_of(int64_t len, const Bounds &B) {
   return k;
 }
 
-struct SplitInfo { int64_t r0, pos_a, pos_b; };   // a split vertex: its first row; list positions of its longer / shorter groups
+struct LongInfo { int64_t r0, pos_a, pos_b; };   // a long vertex: its first row; bucket positions of its longer / shorter groups
 
 struct SplitParams {
   IndptrView ip;
@@ -106,11 +118,20 @@ struct SplitParams {
   Bounds B;
   int64_t n_tiles;
   int64_t *tiles;          // [SPLIT_COLS][n_tiles]
-  int64_t *totals;         // [SPLIT_COLS] column sums, then [IT_MAX_BUCKETS] edges per bucket
-  int64_t *shadow_indptr; int32_t *shadow_owner; int64_t *owner_indptr; int32_t *split_owners;
-  int64_t *bucket_offsets; int32_t *bucket_rows; it_row_meta *bucket_meta; int32_t *bucket_owner;
-  SplitInfo *info;         // [split vertices]
+  int64_t *totals;         // [SPLIT_COLS] column sums, then [IT_MAX_BUCKETS] edges per list (the last one: of the pieces)
+  int64_t long_above;      // vertices of more edges are gathered in pieces
+  int piece_min;
+  int64_t *shadow_indptr; int32_t *shadow_owner; int64_t *owner_indptr;
+  int64_t *bucket_offsets; int32_t *bucket_rows;
+  it_row_meta *list_meta; int32_t *list_owner;
+  int32_t *long_owners; int64_t *piece_ptr; LongInfo *info;   // [long vertices]
+  int *bins;               // [2][PIECE_BINS]: pieces per bin, then the next free place
 };
+
+__device__ __forceinline__ int64_t pieces_of(int64_t d, const SplitParams &p) {
+  const int64_t by_share = d / 64, least = by_share < p.piece_min ? p.piece_min : by_share, len = least > 512 ? 512 : least;
+  return (d + len - 1) / len;
+}
 
 // What a vertex adds: ng rows; `rem` of them in bucket ka (one edge longer), the others in bucket kb.
 struct VertexRows { int64_t ng, rem; int ka, kb; };
@@ -129,60 +150,73 @@ __device__ __forceinline__ VertexRows rows_of(int64_t d, const SplitParams &p) {
   return r;
 }
 
-// Lane c of a warp keeps column c.  One step over 32 vertices, of which those in `valid` exist: count(...) adds them.
-__device__ __forceinline__ void add_columns(int64_t &col, const VertexRows &r, unsigned valid, unsigned split, int nb, int lane) {
-  const bool plain = ((valid & ~split) >> lane) & 1u;
+// Lane c of a warp keeps column c.  One step over 32 vertices; `mine`: lane of bucket or list k: the vertices in bucket k.
+__device__ __forceinline__ unsigned bucket_mask(int kb, int nb, int lane) {
+  unsigned mine = 0;
   for (int k = 0; k < nb; ++k) {
-    const unsigned m = __ballot_sync(0xffffffffu, plain && r.ka == k);
-    if (lane == k) col += __popc(m);
+    const unsigned m = __ballot_sync(0xffffffffu, kb == k);
+    if (lane == k || lane == nb + 4 + k) mine = m;
   }
-  if (lane == nb) col += __popc(valid & ~split);
-  while (split) {   // rare
-    const int l = __ffs(split) - 1;
-    split &= split - 1;
-    const int64_t ng = __shfl_sync(0xffffffffu, r.ng, l), rem = __shfl_sync(0xffffffffu, r.rem, l);
-    const int ka = __shfl_sync(0xffffffffu, r.ka, l), kb = __shfl_sync(0xffffffffu, r.kb, l);
-    if (lane == ka) col += rem;
-    if (lane == kb) col += ng - rem;
-    if (lane == nb) col += ng;
-    if (lane == nb + 1) col += 1;
-  }
+  return mine;
+}
+// vertices `plain`, gathered whole
+__device__ __forceinline__ void add_plain(int64_t &col, unsigned mine, unsigned plain, int nb, int lane) {
+  if (lane == nb) col += __popc(plain);
+  else col += __popc(mine & plain);   // (0 for the columns of long vertices)
+}
+// vertex l, gathered in pieces
+struct LongCols { int64_t ng, rem, np; int ka, kb; };
+__device__ __forceinline__ LongCols long_cols(int64_t d, const VertexRows &r, int l, const SplitParams &p) {
+  LongCols c;
+  c.ng = __shfl_sync(0xffffffffu, r.ng, l); c.rem = __shfl_sync(0xffffffffu, r.rem, l);
+  c.ka = __shfl_sync(0xffffffffu, r.ka, l); c.kb = __shfl_sync(0xffffffffu, r.kb, l);
+  c.np = pieces_of(__shfl_sync(0xffffffffu, d, l), p);
+  return c;
+}
+__device__ __forceinline__ void add_long(int64_t &col, const LongCols &c, int nb, int lane) {
+  if (lane == c.ka) col += c.rem;
+  if (lane == c.kb) col += c.ng - c.rem;
+  if (lane == nb) col += c.ng;
+  if (lane == nb + 1 && c.ng > 1) col += 1;
+  if (lane == nb + 2) col += 1;
+  if (lane == nb + 3) col += c.np;
 }
 
 __global__ void __launch_bounds__(SPLIT_THREADS) split_count_kernel(SplitParams p) {
-  __shared__ unsigned long long cols[SPLIT_COLS], edges[IT_MAX_BUCKETS];
+  __shared__ unsigned long long edges[IT_MAX_BUCKETS];
   const int lane = threadIdx.x & 31, nb = p.B.nb;
-  if (threadIdx.x < SPLIT_COLS) cols[threadIdx.x] = 0;
   if (threadIdx.x < IT_MAX_BUCKETS) edges[threadIdx.x] = 0;
   __syncthreads();
-  const int64_t v0 = (int64_t)blockIdx.x * SPLIT_TILE + (int64_t)(threadIdx.x >> 5) * (32 * SPLIT_ITEMS) + lane;
+  const int64_t tile = (int64_t)blockIdx.x * (SPLIT_THREADS / 32) + (threadIdx.x >> 5);
+  const int64_t v0 = tile * SPLIT_TILE + lane;
   int64_t col = 0, my_edges = 0;
+  int64_t d[SPLIT_ITEMS];
+#pragma unroll
   for (int i = 0; i < SPLIT_ITEMS; ++i) {
     const int64_t v = v0 + i * 32;
-    const int64_t d = v < p.n ? p.ip[v + 1] - p.ip[v] : 0;
-    const VertexRows r = rows_of(d, p);
-    const unsigned valid = __ballot_sync(0xffffffffu, v < p.n), split = __ballot_sync(0xffffffffu, r.ng > 1);
-    if (valid == 0) break;
-    add_columns(col, r, valid, split, nb, lane);
-    // edges per bucket: 32-bit sums across the lanes unless a vertex is huge
-    if (__any_sync(0xffffffffu, d >= ((int64_t)1 << 26) || r.ng > 1)) {
-      if (v < p.n) {
-        const int64_t in_a = r.rem * (r.ng > 1 ? d / r.ng + 1 : 0);
-        if (in_a) atomicAdd(&edges[r.ka], (unsigned long long)in_a);
-        atomicAdd(&edges[r.kb], (unsigned long long)(d - in_a));
-      }
-    } else {
-      for (int k = 0; k < nb; ++k) {
-        const unsigned s = __reduce_add_sync(0xffffffffu, r.kb == k ? (unsigned)d : 0u);
-        if (lane == k) my_edges += s;
-      }
-    }
+    d[i] = v < p.n ? p.ip[v + 1] - p.ip[v] : 0;
   }
-  if (lane < nb + 2) atomicAdd(&cols[lane], (unsigned long long)col);
-  if (lane < nb) atomicAdd(&edges[lane], (unsigned long long)my_edges);
+#pragma unroll
+  for (int i = 0; i < SPLIT_ITEMS; ++i) {
+    const VertexRows r = rows_of(d[i], p);
+    const unsigned valid = __ballot_sync(0xffffffffu, v0 + i * 32 < p.n), mine = bucket_mask(r.kb, nb, lane);
+    unsigned lng = __ballot_sync(0xffffffffu, d[i] > p.long_above);
+    add_plain(col, mine, valid & ~lng, nb, lane);
+    while (lng) {   // rare
+      const int l = __ffs(lng) - 1;
+      lng &= lng - 1;
+      add_long(col, long_cols(d[i], r, l, p), nb, lane);
+    }
+    for (int k = 1; k < nb; ++k) {   // whole vertices have at most 4096 edges: 32-bit sums
+      const unsigned sum = __reduce_add_sync(0xffffffffu, r.kb == k && d[i] <= p.long_above ? (unsigned)d[i] : 0u);
+      if (lane == k) my_edges += sum;
+    }
+    if (d[i] > p.long_above) atomicAdd(&edges[IT_MAX_BUCKETS - 1], (unsigned long long)d[i]);
+  }
+  if (lane < 2 * nb + 4 && tile < p.n_tiles) p.tiles[lane * p.n_tiles + tile] = col;
+  if (lane < nb && my_edges) atomicAdd(&edges[lane], (unsigned long long)my_edges);
   __syncthreads();
-  if (threadIdx.x < nb + 2) p.tiles[threadIdx.x * p.n_tiles + blockIdx.x] = (int64_t)cols[threadIdx.x];
-  if (threadIdx.x < nb && edges[threadIdx.x])
+  if (threadIdx.x < IT_MAX_BUCKETS && edges[threadIdx.x])
     atomicAdd(reinterpret_cast<unsigned long long *>(p.totals + SPLIT_COLS + threadIdx.x), edges[threadIdx.x]);
 }
 
@@ -235,31 +269,27 @@ __global__ void __launch_bounds__(1024) split_scan_kernel(SplitParams p) {
 }
 
 __global__ void __launch_bounds__(SPLIT_THREADS) split_emit_kernel(SplitParams p) {
-  __shared__ int64_t warp_cols[SPLIT_THREADS / 32][SPLIT_COLS];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nb = p.B.nb;
-  const int64_t v0 = (int64_t)blockIdx.x * SPLIT_TILE + (int64_t)warp * (32 * SPLIT_ITEMS) + lane;
+  const int lane = threadIdx.x & 31, nb = p.B.nb;
+  const unsigned below = (1u << lane) - 1u;
+  const int64_t tile = (int64_t)blockIdx.x * (SPLIT_THREADS / 32) + (threadIdx.x >> 5);
+  if (tile >= p.n_tiles) return;   // whole warps
+  const int64_t v0 = tile * SPLIT_TILE + lane;
   int64_t j0[SPLIT_ITEMS];
   int64_t d[SPLIT_ITEMS];
-  int64_t col = 0;
 #pragma unroll
   for (int i = 0; i < SPLIT_ITEMS; ++i) {
     const int64_t v = v0 + i * 32;
     j0[i] = v < p.n ? p.ip[v] : 0;
     d[i] = v < p.n ? p.ip[v + 1] - j0[i] : 0;
-    const VertexRows r = rows_of(d[i], p);
-    add_columns(col, r, __ballot_sync(0xffffffffu, v < p.n), __ballot_sync(0xffffffffu, r.ng > 1), nb, lane);
   }
-  if (lane < nb + 2) warp_cols[warp][lane] = col;
-  __syncthreads();
-  // lane c: the running value of column c; for a bucket counted from the start of the whole list
+  // lane c: the running value of column c; for a bucket or list counted from the start of all of them
   int64_t run = 0;
-  if (lane < nb + 2) {
-    run = p.tiles[lane * p.n_tiles + blockIdx.x];
-    for (int w = 0; w < warp; ++w) run += warp_cols[w][lane];
-    if (lane < nb)
-      for (int k = 0; k < lane; ++k) run += p.totals[k];
+  if (lane < 2 * nb + 4) {
+    run = p.tiles[lane * p.n_tiles + tile];
+    const int first = lane < nb ? 0 : (lane >= nb + 4 ? nb + 4 : lane);
+    for (int k = first; k < lane; ++k) run += p.totals[k];
   }
-  if (blockIdx.x == 0 && warp == 0) {
+  if (tile == 0) {
     if (lane <= nb) {
       int64_t off = 0;
       for (int k = 0; k < lane; ++k) off += p.totals[k];
@@ -268,42 +298,43 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_emit_kernel(SplitParams p
     if (lane == 0) {
       p.shadow_indptr[p.totals[nb]] = p.e;
       p.owner_indptr[p.n] = p.totals[nb];
+      p.piece_ptr[p.totals[nb + 2]] = p.totals[nb + 3];
     }
   }
 #pragma unroll
   for (int i = 0; i < SPLIT_ITEMS; ++i) {
     const int64_t v = v0 + i * 32;
     const VertexRows r = rows_of(d[i], p);
-    const unsigned valid = __ballot_sync(0xffffffffu, v < p.n), split = __ballot_sync(0xffffffffu, r.ng > 1);
-    int64_t row = 0, pos = 0;
-    if (split == 0) {
-      row = __shfl_sync(0xffffffffu, run, nb) + lane;
-      for (int k = 0; k < nb; ++k) {
-        const unsigned m = __ballot_sync(0xffffffffu, v < p.n && r.ka == k);
-        const int64_t at = __shfl_sync(0xffffffffu, run, k);
-        if (r.ka == k) pos = at + __popc(m & ((1u << lane) - 1u));
+    const bool is_long = d[i] > p.long_above;
+    const unsigned lng = __ballot_sync(0xffffffffu, is_long), mine = bucket_mask(r.kb, nb, lane);
+    const unsigned same = __match_any_sync(0xffffffffu, r.kb);
+    unsigned todo = __ballot_sync(0xffffffffu, v < p.n);
+    int64_t row = 0, pos = 0, at = 0;   // first row; position in the buckets / in the lists
+    for (;;) {   // the whole vertices up to the next long one, then that one
+      const unsigned longs = lng & todo;
+      const int l = longs ? __ffs(longs) - 1 : 32;
+      const unsigned plain = l == 32 ? todo : todo & ((1u << l) - 1u);
+      const int64_t at_row = __shfl_sync(0xffffffffu, run, nb), at_bucket = __shfl_sync(0xffffffffu, run, r.kb);
+      const int64_t at_list = __shfl_sync(0xffffffffu, run, nb + 4 + r.kb);
+      if ((plain >> lane) & 1u) {
+        row = at_row + __popc(plain & below);
+        pos = at_bucket + __popc(plain & same & below);
+        at = at_list + __popc(plain & same & below);
       }
-      add_columns(run, r, valid, 0u, nb, lane);
-    } else {   // a split vertex among the 32: one vertex after the other
-      for (int l = 0; l < 32; ++l) {
-        if (!((valid >> l) & 1u)) break;
-        const int64_t ng = __shfl_sync(0xffffffffu, r.ng, l), rem = __shfl_sync(0xffffffffu, r.rem, l);
-        const int ka = __shfl_sync(0xffffffffu, r.ka, l), kb = __shfl_sync(0xffffffffu, r.kb, l);
-        const int64_t at_row = __shfl_sync(0xffffffffu, run, nb), at_k = __shfl_sync(0xffffffffu, run, nb + 1);
-        if (lane == nb) run += ng;
-        if (lane == nb + 1 && ng > 1) run += 1;
-        const int64_t at_a = __shfl_sync(0xffffffffu, run, ka);
-        if (ng > 1 && lane == ka) run += rem;
-        const int64_t at_b = __shfl_sync(0xffffffffu, run, kb);
-        if (lane == kb) run += ng - rem;   // (one plain row: rem = 0)
-        if (lane == l) {
-          row = at_row; pos = at_b;
-          if (ng > 1) {
-            p.split_owners[at_k] = (int32_t)v;
-            p.info[at_k] = SplitInfo{at_row, at_a, at_b};
-          }
-        }
+      add_plain(run, mine, plain, nb, lane);
+      if (l == 32) break;
+      const LongCols c = long_cols(d[i], r, l, p);
+      const int64_t l_row = __shfl_sync(0xffffffffu, run, nb), l_k = __shfl_sync(0xffffffffu, run, nb + 2);
+      const int64_t l_piece = __shfl_sync(0xffffffffu, run, nb + 3), l_a = __shfl_sync(0xffffffffu, run, c.ka);
+      const int64_t l_b = __shfl_sync(0xffffffffu, run, c.kb) + (c.ka == c.kb ? c.rem : 0);
+      if (lane == l) {
+        row = l_row; pos = l_b;
+        p.long_owners[l_k] = (int32_t)v;
+        p.piece_ptr[l_k] = l_piece;
+        p.info[l_k] = LongInfo{l_row, l_a, l_b};
       }
+      add_long(run, c, nb, lane);
+      todo &= ~((2u << l) - 1u);   // (l = 31: 2u << 31 = 0, nothing left)
     }
     if (v < p.n) {
       p.owner_indptr[v] = row;
@@ -311,35 +342,67 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_emit_kernel(SplitParams p
         p.shadow_indptr[row] = j0[i];
         p.shadow_owner[row] = (int32_t)v;
         p.bucket_rows[pos] = (int32_t)row;
+      }
+      if (!is_long) {
         it_row_meta m;
         m.j0 = j0[i]; m.len = (int32_t)d[i]; m.dest = (int32_t)v;
-        p.bucket_meta[pos] = m;
-        p.bucket_owner[pos] = (int32_t)v;
+        p.list_meta[at] = m;
+        p.list_owner[at] = (int32_t)v;
       }
     }
   }
 }
 
-// Rows of split vertices: one block per split vertex, groups written by closed form
+// pieces [first, last) of a vertex with np of them lie in bin b of the order
+__device__ __forceinline__ int64_t bin_first(int64_t b, int64_t np) { return (b * np + PIECE_BINS - 1) / PIECE_BINS; }
+
+// Long vertices, one block each (grid-stride).  Shadow rows by closed form
 //   start(g) = indptr[v] + g * base + min(g, rem),  base = d / ng, rem = d % ng;
-// group g's partial result goes to slot p0 + g: the rows of earlier split vertices = all earlier rows minus earlier unsplit vertices.
-__global__ void __launch_bounds__(128) fill_split_rows_kernel(SplitParams p) {
-  const int64_t n_split = p.totals[p.B.nb + 1];
-  for (int64_t k = blockIdx.x; k < n_split; k += gridDim.x) {
-    const int64_t v = p.split_owners[k], s = p.ip[v], d = p.ip[v + 1] - s;
-    const SplitInfo f = p.info[k];
-    const int64_t ng = groups_of(d, p.T), base = d / ng, rem = d % ng, p0 = f.r0 - v + k;
-    for (int64_t g = threadIdx.x; g < ng; g += blockDim.x) {
-      const int64_t row = f.r0 + g, pos = g < rem ? f.pos_a + g : f.pos_b + (g - rem);
+// and how many of its pieces lie in every bin.
+__global__ void __launch_bounds__(PIECE_BINS) long_rows_kernel(SplitParams p) {
+  const int64_t n_long = p.totals[p.B.nb + 2];
+  int in_bin = 0;   // thread = bin
+  for (int64_t k = blockIdx.x; k < n_long; k += gridDim.x) {
+    const int64_t v = p.long_owners[k], s = p.ip[v], d = p.ip[v + 1] - s;
+    const LongInfo f = p.info[k];
+    const int64_t ng = groups_of(d, p.T), base = d / ng, rem = d % ng;
+    if (ng > 1)
+      for (int64_t g = threadIdx.x; g < ng; g += blockDim.x) {
+        const int64_t row = f.r0 + g;
+        p.shadow_indptr[row] = s + g * base + (g < rem ? g : rem);
+        p.shadow_owner[row] = (int32_t)v;
+        p.bucket_rows[g < rem ? f.pos_a + g : f.pos_b + (g - rem)] = (int32_t)row;
+      }
+    const int64_t np = p.piece_ptr[k + 1] - p.piece_ptr[k];
+    in_bin += (int)(bin_first(threadIdx.x + 1, np) - bin_first(threadIdx.x, np));
+  }
+  if (in_bin > 0) atomicAdd(p.bins + threadIdx.x, in_bin);
+}
+
+// The pieces, bin after bin behind the lists of whole vertices.  (Inside a bin the order of the blocks is that of
+// their atomics: it decides when a piece is walked, not what it holds or where its result goes.)
+__global__ void __launch_bounds__(PIECE_BINS) long_pieces_kernel(SplitParams p) {
+  __shared__ int64_t smem[33];
+  const int64_t n_long = p.totals[p.B.nb + 2], first_piece = p.n - n_long;
+  int64_t total;
+  int64_t pos = first_piece + block_exclusive_scan(p.bins[threadIdx.x], &total, smem);
+  int in_bin = 0;
+  for (int64_t k = blockIdx.x; k < n_long; k += gridDim.x) {
+    const int64_t np = p.piece_ptr[k + 1] - p.piece_ptr[k];
+    in_bin += (int)(bin_first(threadIdx.x + 1, np) - bin_first(threadIdx.x, np));
+  }
+  if (in_bin > 0) pos += atomicAdd(p.bins + PIECE_BINS + threadIdx.x, in_bin);   // this block's share of the bin
+  for (int64_t k = blockIdx.x; k < n_long; k += gridDim.x) {
+    const int64_t v = p.long_owners[k], s = p.ip[v], d = p.ip[v + 1] - s;
+    const int64_t p0 = p.piece_ptr[k], np = p.piece_ptr[k + 1] - p0, base = d / np, rem = d % np;
+    const int64_t g0 = bin_first(threadIdx.x, np), g1 = bin_first(threadIdx.x + 1, np);
+    for (int64_t g = g0; g < g1; ++g, ++pos) {
       it_row_meta m;
       m.j0 = s + g * base + (g < rem ? g : rem);
       m.len = (int32_t)(base + (g < rem ? 1 : 0));
       m.dest = (int32_t)~(p0 + g);
-      p.shadow_indptr[row] = m.j0;
-      p.shadow_owner[row] = (int32_t)v;
-      p.bucket_rows[pos] = (int32_t)row;
-      p.bucket_meta[pos] = m;
-      p.bucket_owner[pos] = (int32_t)v;
+      p.list_meta[pos] = m;
+      p.list_owner[pos] = (int32_t)v;
     }
   }
 }
@@ -347,37 +410,39 @@ __global__ void __launch_bounds__(128) fill_split_rows_kernel(SplitParams p) {
 // ----------------------------------------------------------------------------- host side
 static void forget_split(it_graph *g) {
   g->shadow_indptr = nullptr; g->shadow_owner = nullptr; g->owner_indptr = nullptr;
-  g->split_owners = nullptr; g->bucket_offsets = nullptr; g->bucket_rows = nullptr;
-  g->bucket_meta = nullptr; g->bucket_owner = nullptr;
-  g->n_rows = g->n_split_owners = g->n_partial_rows = 0;
-  g->n_buckets = 0;
+  g->long_owners = nullptr; g->piece_ptr = nullptr; g->bucket_offsets = nullptr; g->bucket_rows = nullptr;
+  g->list_meta = nullptr; g->list_owner = nullptr;
+  g->n_rows = g->n_split_owners = g->n_partial_rows = g->n_long = 0;
+  g->n_buckets = g->n_lists = 0;
 }
 
-// The derived arrays and the scratch of a split with at most R rows and S split vertices, carved out of one allocation that
-// the graph keeps for its next split (NULL slab: only the size).
-static size_t carve_split(it_graph *g, SplitParams &p, char *slab, int64_t R, int64_t S) {
+// The derived arrays and the scratch of a split with at most R rows, L long vertices and P pieces, carved out of one
+// allocation that the graph keeps for its next split (NULL slab: only the size).
+static size_t carve_split(SplitParams &p, char *slab, int64_t R, int64_t L, int64_t P) {
   size_t off = 0;
   auto take = [&](auto *&ptr, int64_t count) {
     ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(slab + off);
     off += it_align_up((size_t)(count > 0 ? count : 1) * sizeof(*ptr));
   };
   take(p.totals, SPLIT_COLS + IT_MAX_BUCKETS);
+  take(p.bins, 2 * PIECE_BINS);   // next to the totals: cleared with them
   take(p.tiles, SPLIT_COLS * p.n_tiles);
   take(p.bucket_offsets, IT_MAX_BUCKETS + 1);
   take(p.owner_indptr, p.n + 1);
   take(p.shadow_indptr, R + 1);
   take(p.shadow_owner, R);
   take(p.bucket_rows, R);
-  take(p.bucket_meta, R);
-  take(p.bucket_owner, R);
-  take(p.split_owners, S);
-  take(p.info, S);
+  take(p.list_meta, p.n + P);
+  take(p.list_owner, p.n + P);
+  take(p.long_owners, L);
+  take(p.piece_ptr, L + 1);
+  take(p.info, L);
   return off;
 }
 
 static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   // the arrays of the previous split are written over: forward passes on any stream that still read them come first
-  if (g->bucket_meta) IT_CUDA_TRY(cudaDeviceSynchronize());
+  if (g->list_meta) IT_CUDA_TRY(cudaDeviceSynchronize());
   forget_split(g);
   g->threshold = T > 0 ? T : 0;
   const int64_t n = g->n;
@@ -385,6 +450,7 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   p.ip = IndptrView{g->indptr, g->indptr_type == IT_I64};
   p.n = n; p.e = g->e; p.T = T;
   p.n_tiles = (n + SPLIT_TILE - 1) / SPLIT_TILE;
+  const unsigned split_blocks = (unsigned)((p.n_tiles + SPLIT_THREADS / 32 - 1) / (SPLIT_THREADS / 32));
   // degree buckets: {0, 8, 32, 256, 1024, everything longer}
   const int64_t fixed[5] = {0, 8, 32, 256, 1024};
   p.B.nb = 0;
@@ -392,10 +458,18 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
     if (T <= 0 || fixed[i] < T) p.B.b[p.B.nb++] = fixed[i];
   p.B.b[p.B.nb++] = T > 0 ? T : INT64_MAX;
 
-  // at most one row per vertex and one more per T edges; only where that is far above the number of vertices are the rows
-  // counted before the arrays are laid out
-  int64_t R = n + (T > 0 ? g->e / T : 0), S = T > 0 ? (n < g->e / T ? n : g->e / T) : 0;
-  const bool count_first = R > n + n / 4 + (1 << 20) || R > (int64_t)INT32_MAX - 1;
+  // A piece spans 128 / d of the source table, which has to stay small against the cache: the larger the table, the longer
+  // the vertices that are worth it (25M sources: pieces above 1024 edges 26.3 ms, above 4096 22.9, above 2048 22.6; 5M: above 1024
+  // 11.7, above 2441 12.1).
+  p.long_above = g->n_src / 12288 < 1024 ? 1024 : (g->n_src / 12288 > 4096 ? 4096 : g->n_src / 12288);
+  if (T > 0 && T < p.long_above) p.long_above = T;
+  p.piece_min = g->n_src < ((int64_t)1 << 17) ? 256 : 128;
+
+  // at most one row per vertex and one more per T edges, a long vertex per long_above edges, a piece per piece_min of them
+  // and one more each; only where that is far above the number of vertices are they counted before the arrays are laid out
+  const int64_t e = g->e;
+  int64_t R = n + (T > 0 ? e / T : 0), L = n < e / p.long_above ? n : e / p.long_above, P = e / p.piece_min + L;
+  const bool count_first = R + P > n + n / 2 + (1 << 22) || R > (int64_t)INT32_MAX - 1;
   int64_t h[SPLIT_COLS + IT_MAX_BUCKETS] = {0};
   auto reserve = [&](size_t bytes) -> it_status {   // grow the graph's allocation; what it holds is not kept
     if (bytes <= g->slab_bytes) return IT_OK;
@@ -406,10 +480,10 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
     return IT_OK;
   };
   auto count = [&]() -> it_status {
-    IT_CUDA_TRY(cudaMemsetAsync(p.totals, 0, sizeof(h), st));
+    IT_CUDA_TRY(cudaMemsetAsync(p.totals, 0, (size_t)((char *)p.tiles - (char *)p.totals), st));
     if (n > 0) {
-      IT_LAUNCH(IT_K_SPLIT_SCAN, 0, 0, st, split_count_kernel<<<(unsigned)p.n_tiles, SPLIT_THREADS, 0, st>>>(p));
-      IT_LAUNCH(IT_K_SPLIT_SCAN, 0, 0, st, split_scan_kernel<<<(unsigned)(p.B.nb + 2), 1024, 0, st>>>(p));
+      IT_LAUNCH(IT_K_SPLIT_SCAN, 0, 0, st, split_count_kernel<<<split_blocks, SPLIT_THREADS, 0, st>>>(p));
+      IT_LAUNCH(IT_K_SPLIT_SCAN, 0, 0, st, split_scan_kernel<<<(unsigned)(2 * p.B.nb + 4), 1024, 0, st>>>(p));
     }
     IT_CUDA_TRY(cudaGetLastError());
     return IT_OK;
@@ -420,41 +494,55 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
     return IT_OK;
   };
   if (count_first) {
-    IT_TRY(reserve(carve_split(g, p, nullptr, 0, 0)));
-    carve_split(g, p, g->slab, 0, 0);
+    IT_TRY(reserve(carve_split(p, nullptr, 0, 0, 0)));
+    carve_split(p, g->slab, 0, 0, 0);
     IT_TRY(count());
     IT_TRY(read_totals());
-    R = h[p.B.nb]; S = h[p.B.nb + 1];
+    R = h[p.B.nb]; L = h[p.B.nb + 2]; P = h[p.B.nb + 3];
     if (R > (int64_t)INT32_MAX - 1) {
       it_set_error("split produces %lld shadow rows; row ids are 32-bit", (long long)R);
       return IT_ERR_UNSUPPORTED;
     }
   }
-  IT_TRY(reserve(carve_split(g, p, nullptr, R, S)));
-  carve_split(g, p, g->slab, R, S);
+  IT_TRY(reserve(carve_split(p, nullptr, R, L, P)));
+  carve_split(p, g->slab, R, L, P);
   IT_TRY(count());
   if (n > 0) {
-    IT_LAUNCH(IT_K_BUCKET_SCAN, 0, 0, st, split_emit_kernel<<<(unsigned)p.n_tiles, SPLIT_THREADS, 0, st>>>(p));
-    if (S > 0) {
-      const int64_t cap = (int64_t)g->num_sms * 16;
-      IT_LAUNCH(IT_K_SPLIT_FILL, 0, 0, st, fill_split_rows_kernel<<<(unsigned)(S < cap ? S : cap), 128, 0, st>>>(p));
+    IT_LAUNCH(IT_K_BUCKET_SCAN, 0, 0, st, split_emit_kernel<<<split_blocks, SPLIT_THREADS, 0, st>>>(p));
+    if (L > 0) {
+      const int64_t cap = (int64_t)g->num_sms * 8;
+      const unsigned blocks = (unsigned)(L < cap ? L : cap);
+      IT_LAUNCH(IT_K_SPLIT_FILL, 0, 0, st, long_rows_kernel<<<blocks, PIECE_BINS, 0, st>>>(p));
+      IT_LAUNCH(IT_K_SPLIT_FILL, 0, 0, st, long_pieces_kernel<<<blocks, PIECE_BINS, 0, st>>>(p));
     }
   } else {
     IT_CUDA_TRY(cudaMemsetAsync(g->slab, 0, g->slab_bytes, st));
   }
   IT_CUDA_TRY(cudaGetLastError());
   IT_TRY(read_totals());
-  g->shadow_indptr = p.shadow_indptr; g->shadow_owner = p.shadow_owner; g->owner_indptr = p.owner_indptr; g->split_owners = p.split_owners;
-  g->bucket_offsets = p.bucket_offsets; g->bucket_rows = p.bucket_rows; g->bucket_meta = p.bucket_meta; g->bucket_owner = p.bucket_owner;
-  g->n_rows = h[p.B.nb];
-  g->n_split_owners = h[p.B.nb + 1];
-  g->n_partial_rows = g->n_rows - (n - g->n_split_owners);
-  g->n_buckets = p.B.nb;
-  g->h_bucket_offsets[0] = 0;
-  for (int k = 0; k < p.B.nb; ++k) {
-    g->h_bucket_offsets[k + 1] = g->h_bucket_offsets[k] + h[k];
-    g->h_bucket_edges[k] = h[SPLIT_COLS + k];
+  const int nb = p.B.nb;
+  if (h[nb + 3] > (int64_t)INT32_MAX - 1) {
+    it_set_error("%lld pieces of long vertices; they are numbered with 31 bits", (long long)h[nb + 3]);
+    return IT_ERR_UNSUPPORTED;
   }
+  g->shadow_indptr = p.shadow_indptr; g->shadow_owner = p.shadow_owner; g->owner_indptr = p.owner_indptr;
+  g->bucket_offsets = p.bucket_offsets; g->bucket_rows = p.bucket_rows; g->list_meta = p.list_meta; g->list_owner = p.list_owner;
+  g->long_owners = p.long_owners; g->piece_ptr = p.piece_ptr;
+  g->n_rows = h[nb];
+  g->n_split_owners = h[nb + 1];
+  g->n_long = h[nb + 2];
+  g->n_partial_rows = h[nb + 3];
+  g->n_buckets = nb;
+  g->n_lists = nb + 1;
+  g->h_list_offsets[0] = 0;
+  for (int k = 0; k < nb; ++k) {
+    g->h_list_offsets[k + 1] = g->h_list_offsets[k] + h[nb + 4 + k];
+    g->h_list_edges[k] = h[SPLIT_COLS + k];
+    g->list_bounds[k] = p.B.b[k] < p.long_above ? p.B.b[k] : p.long_above;   // whole vertices have no more edges
+  }
+  g->h_list_offsets[nb + 1] = n + (g->n_partial_rows - g->n_long);
+  g->h_list_edges[nb] = h[SPLIT_COLS + IT_MAX_BUCKETS - 1];
+  g->list_bounds[nb] = 512;
   for (int i = 0; i < IT_MAX_BUCKETS; ++i) g->bucket_bounds[i] = i < p.B.nb ? p.B.b[i] : 0;
   return IT_OK;
 }

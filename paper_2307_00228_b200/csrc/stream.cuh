@@ -7,15 +7,14 @@
 //
 // Work decomposition.  A feature row is cut into lane slices of SB bytes and is LPR = row bytes / SB
 // lanes wide; rows are bucketed by length and each bucket gets the kernel that suits it.
-//   * stream_rows_ring_kernel, stream_cta_ring_kernel (stream_ring.cuh; rows of 128 bytes and more):
-//     a warp walks the edges of a batch of rows (or of its part of one very long row) as one flat
+//   * stream_rows_chunk_kernel (stream_chunk.cuh; rows of 80 bytes and more, more than a few dozen edges): one warp per
+//     row, chunk after chunk without a break between rows.
+//   * stream_rows_ring_kernel (stream_ring.cuh): a warp walks the edges of a batch of rows as one flat
 //     stream and stages the source rows through a per-warp ring in shared memory with cp.async.
 //   * stream_short_rows_pipe_kernel, stream_tiny_rows_kernel (the same widths up to 256 bytes, rows of at most a few
 //     dozen edges): one group of 8 or 16 lanes per row, eight row loads back to back, no edge stream.
 //   * stream_rows_kernel (rows narrower than 128 bytes): a *group* of LPR lanes takes a batch of rows
 //     and walks the batch's edges as one flat stream with UNROLL rows in flight per lane in registers.
-//   * stream_cta_kernel (the same rows, very long): one CTA per row, each warp a contiguous chunk,
-//     SLOTS = 32 / LPR edges at once per warp; slot and warp states are merged in a fixed order.
 //   * stream_empty_kernel: rows without edges.
 //
 // Policy interface (all __device__):
@@ -59,10 +58,6 @@
 #ifndef IT_SHORT_BELOW
 #define IT_SHORT_BELOW 32       // 128-byte rows: buckets of rows up to this long take the short-row kernel
 #endif
-#ifndef IT_GATHER_CTA_ABOVE
-#define IT_GATHER_CTA_ABOVE 1024   // rows longer than this get a whole CTA; shorter ones a lane group or a warp
-#endif
-
 namespace it_stream {
 
 constexpr int THREADS = 256;
@@ -237,6 +232,7 @@ struct StreamParams {
   int *counter;                           // ring kernel: zeroed device word from which the warps claim their batches after
                                           // their first ones (NULL: every warp walks a fixed stride of the batches)
   int claim;                              // batches per claim
+  int n_pieces, piece_claim, piece_claims;   // chunk kernel: entries at the end of the range that are claimed first, how many at a time
 };
 
 __device__ __forceinline__ it_row_meta load_meta(const it_row_meta *p) {
@@ -570,93 +566,6 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE2_BLOCKS) stream_tiny_ro
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// ----------------------------------------------------------------------------- very long rows: one CTA each
-template <typename T, int SB, int LPR, class Policy>
-__global__ void __launch_bounds__(THREADS, IT_GATHER_MIN_BLOCKS) stream_cta_kernel(StreamParams p, Policy pol) {
-  constexpr int NS = Policy::NS;
-  constexpr int WARPS = THREADS / 32;
-  constexpr int SLOTS = 32 / LPR;
-  constexpr int U = UNROLL * (16 / SB);   // the same bytes in flight per lane whatever the slice width
-  __shared__ float red[WARPS][LPR][NS];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int slot = lane / LPR, t = lane % LPR;
-  pol.setup(t);
-  const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * SB;
-  using Slice = RowSlice<T, SB>;
-  const uint32_t row_bytes = p.src_pitch;
-  for (int64_t i = p.row_lo + blockIdx.x; i < p.row_hi; i += gridDim.x) {
-    const it_row_meta m = load_meta(p.meta + i);
-    const int32_t owner = Policy::NEEDS_OWNER ? __ldcs(p.owner + i) : 0;
-    const int64_t j0 = m.j0, j1 = m.j0 + m.len;
-    const int64_t chunk = ((int64_t)m.len + WARPS - 1) / WARPS;
-    int64_t a = j0 + warp * chunk, b = a + chunk;
-    if (a > j1) a = j1;
-    if (b > j1) b = j1;
-    float st[NS];
-    pol.init(st);
-    pol.begin_row(m.dest, owner);
-    // edges [a, b) with the whole warp: SLOTS edges at once, index chunk of 32 prefetched one step ahead
-    auto load_chunk = [&](int64_t base, int32_t &idx, float &w) {
-      idx = 0; w = 1.f;
-      if (base + lane < b) {
-        idx = p.indices ? __ldcs(p.indices + base + lane) : (int32_t)(base + lane);
-        if (Policy::WEIGHTED) w = __ldcs(p.weights + base + lane);
-      }
-    };
-    int32_t idx_c, idx_n;
-    float w_c, w_n;
-    load_chunk(a, idx_c, w_c);
-    for (int64_t base = a; base < b; base += 32) {
-      load_chunk(base + 32, idx_n, w_n);
-      const int cnt = (int)((b - base) < 32 ? (b - base) : 32);
-      for (int k0 = 0; k0 < cnt; k0 += SLOTS * U) {
-        typename Slice::Raw v[U];
-        float w[U], x[U];
-        bool ok[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int e = k0 + u * SLOTS + slot;
-          const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx_c, e & 31);
-          w[u] = Policy::WEIGHTED ? __shfl_sync(0xffffffffu, w_c, e & 31) : 1.f;
-          ok[u] = e < cnt;
-          x[u] = 0.f;
-          if (ok[u]) {
-            v[u] = Slice::load(my_src + (uint64_t)s * row_bytes);
-            if (Policy::HAS_EXTRA) x[u] = pol.extra(s);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (ok[u]) pol.edge(st, v[u], w[u], x[u]);
-      }
-      idx_c = idx_n; w_c = w_n;
-    }
-    // fold the SLOTS edge slots into slot 0, lower slot first
-#pragma unroll
-    for (int o = 16; o >= LPR; o >>= 1) {
-      float other[NS];
-#pragma unroll
-      for (int k = 0; k < NS; ++k) other[k] = __shfl_xor_sync(0xffffffffu, st[k], o);
-      pol.merge(st, other);   // only slot 0 is read at the end, and it is always the first operand
-    }
-    __syncthreads();  // red[] free again
-    if (lane < LPR) {
-#pragma unroll
-      for (int k = 0; k < NS; ++k) red[warp][lane][k] = st[k];
-    }
-    __syncthreads();
-    if (warp == 0 && lane < LPR) {
-      for (int w = 1; w < WARPS; ++w) {
-        float other[NS];
-#pragma unroll
-        for (int k = 0; k < NS; ++k) other[k] = red[w][lane][k];
-        pol.merge(st, other);
-      }
-      pol.end_row(st, m.dest, owner, m.len);
-    }
-  }
-}
-
 // ----------------------------------------------------------------------------- empty rows
 template <typename T, int SB, int LPR, class Policy>
 __global__ void __launch_bounds__(THREADS) stream_empty_kernel(StreamParams p, Policy pol) {
@@ -704,18 +613,18 @@ it_status allow_dynamic_smem(Kernel kernel, int smem, std::atomic<uint64_t> &don
 // `counters`: IT_MAX_BUCKETS device words of scratch (or NULL): the ring kernel of bucket b hands out its batches from
 // word b, which is zeroed here, in stream order, before the launches.
 template <typename T, int SB, int LPR, bool PAD, class Policy, class BytesF>
-it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, BytesF bytes_of, int kid_cta, int kid_rows,
-                         int kid_empty, int64_t bound_lo, int64_t bound_hi, int *counters, cudaStream_t st) {
+it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, BytesF bytes_of, int kid_rows, int kid_empty,
+                          int64_t bound_lo, int64_t bound_hi, int *counters, cudaStream_t st) {
   constexpr bool RING = SB * LPR >= 128;   // rows of 128 bytes and more are staged through shared memory
-  if (RING && counters) IT_CUDA_TRY(cudaMemsetAsync(counters, 0, IT_MAX_BUCKETS * sizeof(int), st));
+  if (RING && counters) IT_CUDA_TRY(cudaMemsetAsync(counters, 0, (IT_MAX_BUCKETS + 1) * sizeof(int), st));
   p.counter = nullptr;
   bool chunked = false;
   p.slices = p.dim * (int)sizeof(T) / SB;
-  for (int b = g->n_buckets - 1; b >= 0; --b) {
-    const int64_t lo = g->h_bucket_offsets[b], hi = g->h_bucket_offsets[b + 1];
-    if (hi <= lo || g->bucket_bounds[b] <= bound_lo || g->bucket_bounds[b] > bound_hi) continue;
+  for (int b = g->n_lists - 1; b >= 0; --b) {
+    const int64_t lo = g->h_list_offsets[b], hi = g->h_list_offsets[b + 1];
+    if (hi <= lo || g->list_bounds[b] <= bound_lo || g->list_bounds[b] > bound_hi) continue;
     p.row_lo = lo; p.row_hi = hi;
-    const int64_t bound = g->bucket_bounds[b];
+    const int64_t bound = g->list_bounds[b];
     const int64_t rows = hi - lo;
     const int64_t max_blocks = (int64_t)g->num_sms * IT_GATHER_MIN_BLOCKS * 2;
     const double bytes = bytes_of(b, rows);
@@ -729,18 +638,6 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
       int64_t want = (rows + (THREADS / LPR) - 1) / (THREADS / LPR);
       unsigned blocks = (unsigned)(want < max_blocks ? want : max_blocks);
       IT_LAUNCH(kid_empty, bytes, 0, st, stream_empty_kernel<T, SB, LPR, Policy><<<blocks, THREADS, 0, st>>>(p, pol));
-    } else if (bound > IT_GATHER_CTA_ABOVE) {
-      if constexpr (RING) {
-        constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<SB, Policy::HAS_EXTRA>();
-        static std::atomic<uint64_t> configured{0};   // per template instance: one bit per device ordinal
-        IT_TRY(allow_dynamic_smem(stream_cta_ring_kernel<T, SB, LPR, Policy, PAD>, smem, configured));
-        // one CTA per row as far as the grid allows: the hardware hands out rows as CTAs retire
-        unsigned blocks = (unsigned)(rows < (1 << 20) ? rows : (1 << 20));
-        IT_LAUNCH(kid_cta, bytes, 0, st, stream_cta_ring_kernel<T, SB, LPR, Policy, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
-      } else {
-        unsigned blocks = (unsigned)(rows < max_blocks ? rows : max_blocks);
-        IT_LAUNCH(kid_cta, bytes, 0, st, stream_cta_kernel<T, SB, LPR, Policy><<<blocks, THREADS, 0, st>>>(p, pol));
-      }
     } else {
       // about 256 edges per batch at most: 32 rows of <= 8 edges, 8 rows of <= 32, one longer row (measured: walking
       // several longer rows as one stream, to pay the dependent loads at the start of a row once per batch, is slower)
@@ -752,7 +649,7 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
             // one round per row, and rows so short (at most IT_SHORT_PIPE2_AVG edges on average) that one row per lane
             // group leaves the memory system short of bytes in flight: two rows per lane group in flight (measured:
             // 2.7 % less time on power-law rows of 2.9 edges on average, 7 % more on rows of 4.9)
-            if (bound <= IT_SHORT_EDGES && g->h_bucket_edges[b] <= (int64_t)IT_SHORT_PIPE2_AVG * rows) {
+            if (bound <= IT_SHORT_EDGES && g->h_list_edges[b] <= (int64_t)IT_SHORT_PIPE2_AVG * rows) {
               constexpr int smem = 2 * IT_SHORT_EDGES * THREADS * 16;
               static std::atomic<uint64_t> configured2{0};
               IT_TRY(allow_dynamic_smem(stream_tiny_rows_kernel<T, LPR, Policy, PAD>, smem, configured2));
@@ -769,23 +666,23 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
         }
       }
       if constexpr (SB == 16 && LPR >= 8 && !Policy::HAS_EXTRA) {
-        // one warp per row: the buckets above IT_SHORT_BELOW edges that have no block per row, in one launch (they are
-        // neighbours in the row list), longest first
+        // one warp per row: the pieces and the whole vertices of more than IT_SHORT_BELOW edges, in one launch (they are
+        // neighbours in the list), pieces first
         if (bound > IT_SHORT_BELOW && counters) {
           if (chunked) continue;
           chunked = true;
           double all = bytes;
           int b0 = b;
-          while (b0 > 0 && g->bucket_bounds[b0 - 1] > IT_SHORT_BELOW) {
+          while (b0 > 0 && g->list_bounds[b0 - 1] > IT_SHORT_BELOW) {
             --b0;
-            all += bytes_of(b0, g->h_bucket_offsets[b0 + 1] - g->h_bucket_offsets[b0]);
+            all += bytes_of(b0, g->h_list_offsets[b0 + 1] - g->h_list_offsets[b0]);
           }
-          p.row_lo = g->h_bucket_offsets[b0];
+          p.row_lo = g->h_list_offsets[b0];
           constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<16, false>();
           static std::atomic<uint64_t> configured{0};   // per template instance: one bit per device ordinal
           IT_TRY(allow_dynamic_smem(stream_rows_chunk_kernel<T, LPR, Policy, PAD>, smem, configured));
           p.counter = counters + b;
-          const unsigned blocks = chunk_grid(hi - p.row_lo, (int64_t)g->num_sms * IT_RING_MIN_BLOCKS, &p.claim);
+          const unsigned blocks = chunk_grid(p, b == g->n_lists - 1 ? rows : 0, (int64_t)g->num_sms * IT_RING_MIN_BLOCKS);
           IT_LAUNCH(kid_rows, all, 0, st, stream_rows_chunk_kernel<T, LPR, Policy, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
           p.counter = nullptr;
           continue;

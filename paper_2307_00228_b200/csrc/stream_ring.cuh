@@ -311,55 +311,4 @@ __global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_rows_ring_
   }
 }
 
-// ----------------------------------------------------------------------------- very long rows: one CTA each
-// Each warp streams its part of the row through its ring; there is no end of row inside a part.
-template <typename T, int SB, int LPR, class Policy, bool PAD>
-__global__ void __launch_bounds__(THREADS, IT_RING_MIN_BLOCKS) stream_cta_ring_kernel(StreamParams p, Policy pol) {
-  constexpr int NS = Policy::NS;
-  constexpr int WARPS = THREADS / 32;
-  extern __shared__ uint4 ring_raw[];
-  __shared__ float red[WARPS][LPR][NS];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  RingWarp<T, SB, LPR, Policy, PAD> rw;
-  rw.setup((uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)warp * (uint32_t)ring_bytes_per_warp<SB, Policy::HAS_EXTRA>(), p.src, p.src_pitch, p.slices, lane);
-  pol.setup(lane % LPR);
-
-  for (int64_t i = p.row_lo + blockIdx.x; i < p.row_hi; i += gridDim.x) {
-    const it_row_meta m = load_meta(p.meta + i);
-    const int32_t owner = Policy::NEEDS_OWNER ? __ldcs(p.owner + i) : 0;
-    // this warp's part of the row: edges [a, a + total)
-    const int part = (m.len + WARPS - 1) / WARPS;
-    const int first = warp * part < m.len ? warp * part : m.len;
-    const int total = (m.len - first) < part ? (m.len - first) : part;
-    const int64_t a = m.j0 + first;
-    float st[NS];
-    pol.init(st);
-    if (rw.active) pol.begin_row(m.dest, owner);
-    auto load_chunk = [&](int base, int32_t &idx, float &w, unsigned &ends) {
-      idx = 0; w = 1.f; ends = 0u;
-      if (base + lane < total) {
-        idx = p.indices ? __ldcs(p.indices + a + base + lane) : (int32_t)(a + base + lane);
-        if (Policy::WEIGHTED) w = __ldcs(p.weights + a + base + lane);
-      }
-    };
-    if (total > 0) ring_stream<T, SB, LPR, Policy, PAD>(rw, pol, st, total, load_chunk, [] {});
-    rw.fold(pol, st);
-    __syncthreads();  // red[] free again
-    if (lane < LPR) {
-#pragma unroll
-      for (int k = 0; k < NS; ++k) red[warp][lane][k] = st[k];
-    }
-    __syncthreads();
-    if (warp == 0 && lane < LPR) {
-      for (int w = 1; w < WARPS; ++w) {
-        float other[NS];
-#pragma unroll
-        for (int k = 0; k < NS; ++k) other[k] = red[w][lane][k];
-        pol.merge(st, other);
-      }
-      if (rw.active) pol.end_row(st, m.dest, owner, m.len);
-    }
-  }
-}
-
 }  // namespace it_stream
