@@ -279,7 +279,7 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
       return it_launch_gather(gg, c.st);
     case PLAN_SAGE_REORDER:
       gg.dim = L->out_dim; gg.src = table; gg.dst = out; gg.epi = IT_EPI_ADD_ACT;
-      gg.self_term = self_term ? self_term : c.ws + c.w.off_a; gg.self_dtype = dt; gg.act = L->act;
+      gg.self_term = self_term ? self_term : c.ws + c.w.off_a; gg.act = L->act;
       return it_launch_gather(gg, c.st);
     case PLAN_MSG:
       gg.dim = L->msg_dim; gg.dst = out; gg.dst_ld = L->msg_dim; gg.epi = IT_EPI_STORE; gg.act = IT_ACT_NONE;

@@ -137,7 +137,7 @@ static inline int it_dtype_size(it_dtype t) { return t == IT_F32 ? 4 : 2; }
 // What a gather / combine kernel does with the finished aggregate of vertex v.
 enum it_epilogue_kind {
   IT_EPI_STORE = 0,      // dst[v, :] = agg                      (feat dtype)
-  IT_EPI_ADD_ACT = 1,    // dst[v, :] = act(self[v, :] + agg)    (self fp32 or feat dtype, dst feat dtype)
+  IT_EPI_ADD_ACT = 1,    // dst[v, :] = act(self[v, :] + agg)    (both feat dtype)
   IT_EPI_BIAS_ACT = 2,   // dst[v, :] = act(bias + agg)          (bias fp32 [dim] or NULL)
   IT_EPI_RAW_F32 = 3     // dst[v, :] = the raw reduce in fp32: plain sum (mean undivided), max or min, and the identity of
                          // the reduce (0, -inf, +inf) for a row without edges: one part's share of a partial-gather
@@ -157,28 +157,30 @@ struct it_gather_args {
   void *dst;               // row v starts at dst + v * dst_ld elements and takes dim of them
   int dst_ld;              // 0 means dim
   it_epilogue_kind epi;
-  const void *self_term;   // IT_EPI_ADD_ACT only: row v starts at self_term + v * self_ld elements of self_dtype
-  it_dtype self_dtype;     // IT_F32, or the dtype of the rows (the self term of a transform-first layer is stored like the rows)
+  const void *self_term;   // IT_EPI_ADD_ACT only: row v starts at self_term + v * self_ld elements (stored like the rows)
   int self_ld;             // 0 means dim
   const float *bias;       // [dim] fp32 or NULL, IT_EPI_BIAS_ACT only
   it_act act;              // IT_EPI_ADD_ACT and IT_EPI_BIAS_ACT
 };
 it_status it_launch_gather(const it_gather_args &a, cudaStream_t stream);
 
-// Rows [row_lo, row_hi) of the bucket-ordered list all get the same value: what a vertex without in-edges ends up with.
-struct it_const_rows_args {
+// What the vertices without in-edges (entries [row_lo, row_hi) of the list) end up with.
+enum it_empty_kind { IT_EMPTY_VALUE = 0 /* every entry `value` */, IT_EMPTY_BIAS = 1 /* act(bias[i]), NULL: act(0) */, IT_EMPTY_SELF = 2 /* act(self[v, i]) */ };
+struct it_empty_rows_args {
   const it_graph *g;
   int64_t row_lo, row_hi;
+  it_empty_kind kind;
   void *dst;
   int64_t pitch;           // bytes from one row of dst to the next
+  const void *self;        // rows of dtype
+  int64_t self_pitch;
   int dim;                 // entries written
   it_dtype dtype;          // of dst
-  float value;             // every entry, or
-  const float *bias;       // act(bias[i]) when has_bias (NULL: act(0))
-  int has_bias;
+  float value;
+  const float *bias;
   it_act act;
 };
-it_status it_launch_const_rows(const it_const_rows_args &a, int kid, double bytes, cudaStream_t stream);
+it_status it_launch_empty_rows(const it_empty_rows_args &a, int kid, double bytes, cudaStream_t stream);
 
 // ----------------------------------------------------------------------------- gat.cu
 struct it_gat_args {

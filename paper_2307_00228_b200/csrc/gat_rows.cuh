@@ -308,10 +308,10 @@ it_status launch_gat_rows(const it_gat_args &a, StreamParams p, const GatPolicy<
     const double bytes = bytes_of(b, rows);
     constexpr int smem = (THREADS / 32) * gat_bytes_per_warp<H>();
     if (bound == 0) {
-      it_const_rows_args cr;
-      pol.empty_rows(cr);
-      cr.g = g; cr.row_lo = lo; cr.row_hi = hi;
-      IT_TRY(it_launch_const_rows(cr, IT_K_GAT_EMPTY, bytes, st));
+      it_empty_rows_args er;
+      pol.empty_rows(er);
+      er.g = g; er.row_lo = lo; er.row_hi = hi;
+      IT_TRY(it_launch_empty_rows(er, IT_K_GAT_EMPTY, bytes, st));
     } else if (LPR <= 16 && bound <= IT_SHORT_BELOW) {
       if constexpr (LPR <= 16) {
         constexpr int sbytes = 2 * IT_SHORT_EDGES * THREADS * 16;

@@ -23,7 +23,7 @@ struct CombineParams {
   const void *__restrict__ self_term;
   const float *__restrict__ bias;
   int64_t n_long;
-  int dim, dst_ld, self_ld, self_is_t;
+  int dim, dst_ld, self_ld;
   int red, is_mean, epi, act;   // red: RED_SUM / RED_MAX / RED_MIN
 };
 
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p
       }
       if (p.epi == IT_EPI_ADD_ACT) {
         float4 s;
-        if (sizeof(T) == 2 && p.self_is_t) {
+        if constexpr (sizeof(T) == 2) {
           const uint2 raw = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const T *>(p.self_term) + v * p.self_ld + c));
           s = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u), __uint_as_float(raw.y << 16),
                           __uint_as_float(raw.y & 0xffff0000u));
@@ -102,37 +102,43 @@ __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p
 }
 
 // ----------------------------------------------------------------------------- rows without edges
-// The row is built once per block in shared memory; a warp takes 32 rows (their destinations with one coalesced load) and
-// writes them 16 bytes per lane.  Bound by the writes: per-row kernels waited for each record before its row's store
-// (8M vertices, 256-byte rows: 340 -> 255 us; 256-byte GAT rows of 615k vertices 82 -> 22 us).
-struct ConstRowsParams {
+// A warp takes 32 rows (their destinations with one coalesced load) and writes them 16 bytes per lane, four pieces in
+// flight; a value that is the same for every row is built once per block in shared memory.  Bound by the writes (and the
+// self terms): per-row kernels waited for each row's record, then its self term, before the row's store (5.3M raw 256-byte
+// rows: 340 -> 255 us; 615k GAT rows of 256 bytes: 82 -> 22; two layers of 8M rows of 128 bytes, one with self terms: 851 -> 638).
+struct EmptyRowsParams {
   const it_row_meta *__restrict__ meta;
   int64_t lo, hi;
   char *dst;
-  int64_t pitch;
-  int slices, dim, bf16, has_bias, act;   // slices: 16-byte pieces of a row
+  const char *self;
+  int64_t pitch, self_pitch;
+  int kind, slices, dim, bf16, act;   // slices: 16-byte pieces of a row
   float value;
   const float *__restrict__ bias;
 };
 
-__global__ void __launch_bounds__(GATHER_THREADS) const_rows_kernel(ConstRowsParams p) {
-  __shared__ uint4 row[128];   // rows of up to 512 entries
-  for (int s = threadIdx.x; s < p.slices; s += GATHER_THREADS) {
-    const int per = p.bf16 ? 8 : 4;
-    float v[8];
-    for (int k = 0; k < 8; ++k) v[k] = p.has_bias ? act_apply(p.bias && k < per ? p.bias[s * per + k] : 0.f, p.act) : p.value;
-    if (p.bf16) {
-      uint32_t w[4];
-      for (int k = 0; k < 4; ++k) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
-        w[k] = *reinterpret_cast<uint32_t *>(&h);
-      }
-      row[s] = make_uint4(w[0], w[1], w[2], w[3]);
-    } else {
-      row[s] = make_uint4(__float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
-    }
+__device__ __forceinline__ uint4 pack_piece(const float (&v)[8], int bf16) {
+  if (!bf16) return make_uint4(__float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
+  uint32_t w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+    w[k] = *reinterpret_cast<uint32_t *>(&h);
   }
-  __syncthreads();
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+__global__ void __launch_bounds__(GATHER_THREADS) empty_rows_kernel(EmptyRowsParams p) {
+  __shared__ uint4 row[128];   // rows of up to 512 entries
+  if (p.kind != IT_EMPTY_SELF) {
+    for (int s = threadIdx.x; s < p.slices; s += GATHER_THREADS) {
+      const int per = p.bf16 ? 8 : 4;
+      float v[8];
+      for (int k = 0; k < 8; ++k) v[k] = p.kind == IT_EMPTY_BIAS ? act_apply(p.bias && k < per ? p.bias[s * per + k] : 0.f, p.act) : p.value;
+      row[s] = pack_piece(v, p.bf16);
+    }
+    __syncthreads();
+  }
   const int lane = threadIdx.x & 31;
   const int step_r = 32 / p.slices, step_s = 32 % p.slices;
   for (int64_t b = p.lo + ((int64_t)blockIdx.x * (GATHER_THREADS / 32) + (threadIdx.x >> 5)) * 32; b < p.hi;
@@ -141,25 +147,54 @@ __global__ void __launch_bounds__(GATHER_THREADS) const_rows_kernel(ConstRowsPar
     int dest = 0;
     if (lane < n) dest = __ldcs(&p.meta[b + lane].dest);
     int r = lane / p.slices, s = lane % p.slices;
-    for (int k = 0; k < p.slices; ++k) {   // 32 rows x slices pieces, 32 at a time
-      const int64_t d = __shfl_sync(0xffffffffu, dest, r & 31);
-      if (r < n) __stcs(reinterpret_cast<uint4 *>(p.dst + d * p.pitch) + s, row[s]);
-      r += step_r; s += step_s;
-      if (s >= p.slices) { s -= p.slices; ++r; }
+    for (int k = 0; k < p.slices; k += 4) {   // 32 rows x slices pieces, 32 at a time, four of those in flight
+      uint4 x[4];
+      int64_t at[4];
+      int sl[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int d = __shfl_sync(0xffffffffu, dest, r & 31);
+        sl[u] = s;
+        at[u] = r < n && k + u < p.slices ? (int64_t)d : -1;
+        if (at[u] >= 0) x[u] = p.kind == IT_EMPTY_SELF ? __ldcs(reinterpret_cast<const uint4 *>(p.self + at[u] * p.self_pitch) + s) : row[s];
+        r += step_r; s += step_s;
+        if (s >= p.slices) { s -= p.slices; ++r; }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (at[u] < 0) continue;
+        if (p.kind == IT_EMPTY_SELF && p.act != IT_ACT_NONE) {
+          float v[8];
+          const uint32_t w[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (p.bf16) {
+              v[2 * q] = act_apply(__uint_as_float(w[q] << 16), p.act);
+              v[2 * q + 1] = act_apply(__uint_as_float(w[q] & 0xffff0000u), p.act);
+            } else {
+              v[q] = act_apply(__uint_as_float(w[q]), p.act);
+              v[4 + q] = 0.f;
+            }
+          }
+          x[u] = pack_piece(v, p.bf16);
+        }
+        __stcs(reinterpret_cast<uint4 *>(p.dst + at[u] * p.pitch) + sl[u], x[u]);
+      }
     }
   }
 }
 
 }  // namespace
 
-it_status it_launch_const_rows(const it_const_rows_args &a, int kid, double bytes, cudaStream_t st) {
+it_status it_launch_empty_rows(const it_empty_rows_args &a, int kid, double bytes, cudaStream_t st) {
   const it_graph *g = a.g;
-  ConstRowsParams p;
+  EmptyRowsParams p;
   p.meta = g->list_meta; p.lo = a.row_lo; p.hi = a.row_hi; p.dst = (char *)a.dst; p.pitch = a.pitch; p.dim = a.dim;
-  p.slices = a.dim * it_dtype_size(a.dtype) / 16; p.bf16 = a.dtype == IT_BF16; p.has_bias = a.has_bias; p.act = (int)a.act;
+  p.self = (const char *)a.self; p.self_pitch = a.self_pitch; p.kind = (int)a.kind;
+  p.slices = a.dim * it_dtype_size(a.dtype) / 16; p.bf16 = a.dtype == IT_BF16; p.act = (int)a.act;
   p.value = a.value; p.bias = a.bias;
   const int64_t want = (a.row_hi - a.row_lo + GATHER_THREADS - 1) / GATHER_THREADS, cap = (int64_t)g->num_sms * 8;
-  IT_LAUNCH(kid, bytes, 0, st, const_rows_kernel<<<(unsigned)(want < cap ? want : cap), GATHER_THREADS, 0, st>>>(p));
+  IT_LAUNCH(kid, bytes, 0, st, empty_rows_kernel<<<(unsigned)(want < cap ? want : cap), GATHER_THREADS, 0, st>>>(p));
   IT_CUDA_TRY(cudaGetLastError());
   return IT_OK;
 }
@@ -179,7 +214,7 @@ static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
     c.long_owners = g->long_owners; c.piece_ptr = g->piece_ptr; c.owner_indptr = g->owner_indptr; c.shadow_indptr = g->shadow_indptr;
     c.partials = a.partials; c.dst = a.dst; c.self_term = a.self_term; c.bias = a.bias; c.n_long = g->n_long;
     c.dim = a.dim; c.dst_ld = a.dst_ld > 0 ? a.dst_ld : a.dim; c.self_ld = a.self_ld > 0 ? a.self_ld : a.dim;
-    c.red = a.op == IT_GATHER_MAX ? RED_MAX : (a.op == IT_GATHER_MIN ? RED_MIN : RED_SUM); c.is_mean = a.op == IT_GATHER_MEAN && a.epi != IT_EPI_RAW_F32; c.epi = a.epi; c.act = a.act; c.self_is_t = a.self_dtype != IT_F32;
+    c.red = a.op == IT_GATHER_MAX ? RED_MAX : (a.op == IT_GATHER_MIN ? RED_MIN : RED_SUM); c.is_mean = a.op == IT_GATHER_MEAN && a.epi != IT_EPI_RAW_F32; c.epi = a.epi; c.act = a.act;
     const int64_t cap = (int64_t)g->num_sms * 8;
     const unsigned blocks = (unsigned)(g->n_long < cap ? g->n_long : cap);
     const double cbytes = (double)g->n_partial_rows * a.dim * 4.0 +
@@ -216,7 +251,7 @@ it_status it_launch_gather(const it_gather_args &a, cudaStream_t st) {
     c.src_ld = a.src_ld > 0 ? a.src_ld : full;
     c.dst = (char *)a.dst + (size_t)c0 * (a.epi == IT_EPI_RAW_F32 ? 4 : es);
     c.dst_ld = a.dst_ld > 0 ? a.dst_ld : full;
-    c.self_term = a.self_term ? (const char *)a.self_term + (size_t)c0 * (a.self_dtype == IT_F32 ? 4 : es) : nullptr;
+    c.self_term = a.self_term ? (const char *)a.self_term + (size_t)c0 * es : nullptr;
     c.self_ld = a.self_ld > 0 ? a.self_ld : full;
     c.bias = a.bias ? a.bias + c0 : nullptr;
     IT_TRY(launch_gather_chunk(c, st));

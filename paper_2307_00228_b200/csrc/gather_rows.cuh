@@ -21,18 +21,17 @@ struct SagePolicy {
   const void *__restrict__ self_term;
   const float *__restrict__ bias;
   int dim, dst_ld, self_ld, is_mean, epi, act;   // dim: width of this column chunk; *_ld: row lengths of dst / the self term
-  int self_is_t;                                 // the self term is stored in T (else fp32)
   // per-thread
   int col;
   float self[VEC];
 
-  bool empty_rows(it_const_rows_args &a) const {
-    if (epi == IT_EPI_ADD_ACT) return false;   // its self term still has to be read
+  void empty_rows(it_empty_rows_args &a) const {
     const bool raw = epi == IT_EPI_RAW_F32;
+    a.kind = epi == IT_EPI_ADD_ACT ? IT_EMPTY_SELF : (epi == IT_EPI_BIAS_ACT ? IT_EMPTY_BIAS : IT_EMPTY_VALUE);
     a.dst = dst; a.dim = dim; a.dtype = raw || sizeof(T) == 4 ? IT_F32 : IT_BF16; a.pitch = (int64_t)dst_ld * (raw ? 4 : (int)sizeof(T));
+    a.self = self_term; a.self_pitch = (int64_t)self_ld * (int)sizeof(T);
     a.value = raw ? (RED == RED_MAX ? -INFINITY : (RED == RED_MIN ? INFINITY : 0.f)) : 0.f;
-    a.has_bias = epi == IT_EPI_BIAS_ACT; a.bias = bias; a.act = (it_act)act;
-    return true;
+    a.bias = bias; a.act = (it_act)act;
   }
   __device__ __forceinline__ void setup(int t) { col = t * VEC; }
   __device__ __forceinline__ void init(float (&st)[NS]) const {
@@ -70,12 +69,8 @@ struct SagePolicy {
   }
   // the matching slice of the self term is fetched when the row starts, so that end_row does not wait for it
   __device__ __forceinline__ void begin_row(int32_t dest, int32_t) {
-    if (epi == IT_EPI_ADD_ACT && dest >= 0) {
-      if (sizeof(T) == 2 && self_is_t)
-        Slice::unpack(Slice::load(reinterpret_cast<const char *>(self_term) + ((int64_t)dest * self_ld + col) * (int64_t)sizeof(T)), self);
-      else
-        load_floats_stream<VEC>(reinterpret_cast<const float *>(self_term) + (int64_t)dest * self_ld + col, self);
-    }
+    if (epi == IT_EPI_ADD_ACT && dest >= 0)
+      Slice::unpack(Slice::load_stream(reinterpret_cast<const char *>(self_term) + ((int64_t)dest * self_ld + col) * (int64_t)sizeof(T)), self);
   }
   __device__ __forceinline__ void end_row(float (&st)[NS], int32_t dest, int32_t, int64_t len) const {
     if (RED != RED_SUM && len == 0 && epi != IT_EPI_RAW_F32) {
@@ -114,14 +109,13 @@ it_status launch_policy(const it_gather_args &a, StreamParams sp, int64_t bound_
   SagePolicy<T, SB, RED, WEIGHTED> pol;
   pol.partials = a.partials; pol.dst = a.dst; pol.self_term = a.self_term; pol.bias = a.bias; pol.dim = a.dim; pol.dst_ld = a.dst_ld > 0 ? a.dst_ld : a.dim; pol.self_ld = a.self_ld > 0 ? a.self_ld : a.dim;
   pol.is_mean = a.op == IT_GATHER_MEAN && a.epi != IT_EPI_RAW_F32; pol.epi = a.epi; pol.act = a.act; pol.col = 0;
-  pol.self_is_t = a.self_dtype != IT_F32;
   const it_graph *g = a.g;
   // algorithmic bytes: per edge the index, the optional weight and one source row; per row its
   // metadata and one output row (plus the self row it is added to)
   const double row_bytes = (double)a.dim * sizeof(T);
   auto bytes_of = [=](int b, int64_t rows) {
     return (double)g->h_list_edges[b] * ((a.per_edge_rows ? 0.0 : 4.0) + (WEIGHTED ? 4.0 : 0.0) + row_bytes) +
-           (double)rows * (16.0 + row_bytes + (a.epi == IT_EPI_ADD_ACT ? (a.self_dtype == IT_F32 ? 4.0 : (double)sizeof(T)) * a.dim : 0.0));
+           (double)rows * (16.0 + row_bytes + (a.epi == IT_EPI_ADD_ACT ? row_bytes : 0.0));
   };
   auto launch = [&]<bool PAD>() {
     return launch_buckets<T, SB, LPR, PAD>(g, sp, pol, bytes_of, IT_K_GATHER_FLAT, IT_K_GATHER_EMPTY, bound_lo, bound_hi, a.counters, st);

@@ -15,7 +15,7 @@
 //     dozen edges): one group of 8 or 16 lanes per row, eight row loads back to back, no edge stream.
 //   * stream_rows_kernel (rows narrower than 128 bytes): a *group* of LPR lanes takes a batch of rows
 //     and walks the batch's edges as one flat stream with UNROLL rows in flight per lane in registers.
-//   * stream_empty_kernel: rows without edges.
+//   * rows without edges: gather.cu.
 //
 // Policy interface (all __device__):
 //   static constexpr int NS;                 // floats of per-lane state
@@ -27,7 +27,7 @@
 //   void merge(float (&st)[NS], const float (&other)[NS]);     // other comes later in edge order
 //   void begin_row(int32_t dest, int32_t owner);               // prefetch what end_row needs
 //   void end_row(float (&st)[NS], int32_t dest, int32_t owner, int64_t len);
-//   bool empty_rows(it_const_rows_args &a);   // host: rows without edges all get the value described in a
+//   void empty_rows(it_empty_rows_args &a);   // host: what rows without edges get
 #pragma once
 
 #include <atomic>
@@ -89,6 +89,7 @@ template <typename T, int SB> struct RowSlice {
   static constexpr int VEC = SB / (int)sizeof(T);
   using Raw = typename SliceRaw<SB>::type;
   __device__ static __forceinline__ Raw load(const char *p) { return __ldg(reinterpret_cast<const Raw *>(p)); }
+  __device__ static __forceinline__ Raw load_stream(const char *p) { return __ldcs(reinterpret_cast<const Raw *>(p)); }
   __device__ static __forceinline__ void unpack(const Raw &x, float (&v)[VEC]) {
     uint32_t w[SB / 4];
     raw_words<SB>(x, w);
@@ -186,19 +187,6 @@ __device__ __forceinline__ void store_floats(float *p, const float (&v)[VEC]) {
     for (int i = 0; i < VEC; i += 4) *reinterpret_cast<float4 *>(p + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
   }
 }
-template <int VEC>
-__device__ __forceinline__ void load_floats_stream(const float *p, float (&v)[VEC]) {
-  if constexpr (VEC == 1) { v[0] = __ldcs(p); }
-  else if constexpr (VEC == 2) { const float2 x = __ldcs(reinterpret_cast<const float2 *>(p)); v[0] = x.x; v[1] = x.y; }
-  else {
-#pragma unroll
-    for (int i = 0; i < VEC; i += 4) {
-      const float4 x = __ldcs(reinterpret_cast<const float4 *>(p + i));
-      v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
-    }
-  }
-}
-
 __device__ __forceinline__ float act_apply(float x, int act) {
   if (act == IT_ACT_RELU) return fmaxf(x, 0.f);
   if (act == IT_ACT_ELU) return it_elu(x);
@@ -566,24 +554,6 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE2_BLOCKS) stream_tiny_ro
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// ----------------------------------------------------------------------------- empty rows
-template <typename T, int SB, int LPR, class Policy>
-__global__ void __launch_bounds__(THREADS) stream_empty_kernel(StreamParams p, Policy pol) {
-  constexpr int NS = Policy::NS;
-  const int t = threadIdx.x % LPR;
-  if (t >= p.slices) return;
-  pol.setup(t);
-  const int64_t groups_total = (int64_t)gridDim.x * (THREADS / LPR);
-  for (int64_t i = p.row_lo + (int64_t)blockIdx.x * (THREADS / LPR) + threadIdx.x / LPR; i < p.row_hi; i += groups_total) {
-    const it_row_meta m = load_meta(p.meta + i);
-    const int32_t owner = Policy::NEEDS_OWNER ? __ldcs(p.owner + i) : 0;
-    float st[NS];
-    pol.init(st);
-    pol.begin_row(m.dest, owner);
-    pol.end_row(st, m.dest, owner, 0);
-  }
-}
-
 }  // namespace it_stream
 
 #include "stream_ring.cuh"
@@ -629,15 +599,10 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
     const int64_t max_blocks = (int64_t)g->num_sms * IT_GATHER_MIN_BLOCKS * 2;
     const double bytes = bytes_of(b, rows);
     if (bound == 0) {
-      it_const_rows_args cr;
-      if (pol.empty_rows(cr)) {   // the same value for every row: no self term to read
-        cr.g = g; cr.row_lo = lo; cr.row_hi = hi;
-        IT_TRY(it_launch_const_rows(cr, kid_empty, bytes, st));
-        continue;
-      }
-      int64_t want = (rows + (THREADS / LPR) - 1) / (THREADS / LPR);
-      unsigned blocks = (unsigned)(want < max_blocks ? want : max_blocks);
-      IT_LAUNCH(kid_empty, bytes, 0, st, stream_empty_kernel<T, SB, LPR, Policy><<<blocks, THREADS, 0, st>>>(p, pol));
+      it_empty_rows_args er;
+      pol.empty_rows(er);
+      er.g = g; er.row_lo = lo; er.row_hi = hi;
+      IT_TRY(it_launch_empty_rows(er, kid_empty, bytes, st));
     } else {
       // about 256 edges per batch at most: 32 rows of <= 8 edges, 8 rows of <= 32, one longer row (measured: walking
       // several longer rows as one stream, to pay the dependent loads at the start of a row once per batch, is slower)
@@ -727,17 +692,14 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
 // whole sectors beats one pass per power-of-two piece even at 25 of 32 lanes: a GCN of widths 100-128-128-48 on 15M
 // edges, whose 400-byte fp32 rows were 256 + 128 + 16, takes 2.98 ms instead of 4.24 (the 16-byte pieces alone moved a
 // 32-byte sector each and an edge index).
-// Unless `wide` is false, rows of 128 bytes use 16-byte slices throughout and rows of 256 bytes use them for every row
-// with edges (short rows: the lane-group kernel); <8, 32> keeps the empty rows.
+// Rows of 128 and 256 bytes use 16-byte slices unless `wide` is false (a slice would straddle two attention heads).
 template <class F>
 it_status dispatch_row_bytes(int row_bytes, bool wide, F f) {
   constexpr int64_t ALL = INT64_MAX;
   if (row_bytes > 256 && row_bytes <= 512) return f.template operator()<16, 32>(-1, ALL);
   if (row_bytes > 128 && row_bytes <= 256) {
     if (!wide) return f.template operator()<8, 32>(-1, ALL);
-    if (row_bytes < 256) return f.template operator()<16, 16>(-1, ALL);
-    IT_TRY((f.template operator()<16, 16>(0, ALL)));
-    return f.template operator()<8, 32>(-1, 0);
+    return f.template operator()<16, 16>(-1, ALL);
   }
   if (row_bytes > 64 && row_bytes <= 128) {
     if (!wide) return f.template operator()<4, 32>(-1, ALL);
