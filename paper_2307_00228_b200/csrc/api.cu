@@ -1,6 +1,7 @@
 // it_layer_forward / it_infer / it_workspace_bytes: argument checks, workspace carving and the
 // launch sequence of one layer.  All arithmetic lives in the kernels of the other files.
 #include <mutex>
+#include <vector>
 
 #include "common.cuh"
 
@@ -11,7 +12,7 @@ enum LayerPlan { PLAN_SAGE = 0, PLAN_SAGE_REORDER = 1, PLAN_GAT = 2, PLAN_DENSE 
 
 struct LayerWs {
   LayerPlan plan;
-  size_t off_counters;                              // IT_MAX_BUCKETS + 1 words from which the gather's warps claim their batches
+  size_t off_counters;                              // it_gather_words() words
   size_t off_B, off_partials, off_a, off_b, off_q;  // a: aggregate A | self term S | scores ; b: Z | P ; q: per-edge part Q / messages
   size_t bytes;
 };
@@ -88,7 +89,7 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
   auto take = [&](size_t bytes) { size_t o = off; off += it_align_up(bytes); return o; };
   w.plan = plan_of(L);
   w.off_q = 0;
-  w.off_counters = take((IT_MAX_BUCKETS + 1) * sizeof(int));
+  w.off_counters = take(it_gather_words(g) * sizeof(int));
   switch (w.plan) {
     case PLAN_GAT:
       w.off_B = take((fi + kpad) * (fo + 2 * (size_t)L->heads) * 8);
@@ -147,35 +148,73 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
   return w;
 }
 
+// The weight matrices of a whole call, prepared by one launch before its first layer (and the words that the gathers need
+// zeroed with it): the call's layers are gone through twice, first recording their products, then launching.
+struct Prepared {
+  std::vector<it_prep_tc> m;
+  size_t next = 0;
+  bool recording = true;
+  char *base = nullptr;
+  size_t used = 0, cap = 0;
+  // where the product's prepared weights lie (NULL: not recorded, to be prepared on its own)
+  void *place(it_prep_tc p) {
+    if (!recording) return next < m.size() ? m[next++].B : nullptr;
+    const size_t bytes = it_align_up(it_prep_tc_bytes(p));
+    if (used + bytes > cap) return nullptr;   // (not with prep_bytes_of() of every layer)
+    p.B = base + used;
+    used += bytes;
+    m.push_back(p);
+    return p.B;
+  }
+};
+
+struct StageCtx {
+  const it_graph *g;
+  const it_layer_desc *L;
+  LayerWs w;
+  char *ws;
+  float *B, *partials;
+  Prepared *prep;   // NULL: a stage on its own
+  cudaStream_t st;
+  bool recording() const { return prep && prep->recording; }
+  int zeroed() const { return prep && it_small_graph(g); }
+};
+
 // The dense transform of a layer: on the tensor cores when the shape allows it, otherwise the
 // fp32 CUDA-core kernel.  `ga` is filled for the CUDA-core kernel (for GAT: NB includes the
 // 2*heads score columns and out2 = scores); the tensor-core kernel derives its own view.
-it_status run_apply(const it_graph *g, const it_layer_desc *L, it_prep_kind kind, it_gemm_args ga, float *B,
-                    float *scores, cudaStream_t st) {
+it_status run_apply(const StageCtx &c, const it_layer_desc *L, it_prep_kind kind, it_gemm_args ga, float *scores) {
+  const it_graph *g = c.g;
   const int K = ga.K1 + (ga.X2 ? ga.K2 : 0);
   const bool want_scores = kind == IT_PREP_GAT;
   const int heads = L->heads > 0 ? L->heads : 1, hd = L->out_dim / heads;
   if (it_tc_supported(ga, heads, hd, want_scores)) {
-    IT_TRY(it_launch_prep_weights_tc(kind, L, ga.n0 + ga.n1, ga.K1, ga.X2 ? ga.K2 : 0, B, st));
-    return it_launch_gemm_tc(ga, B, L->att_src, L->att_dst, heads, hd, want_scores ? scores : nullptr, g->num_sms,
-                             g->d_status, st);
+    it_prep_tc p = it_prep_tc_of(kind, L, ga.n0 + ga.n1, ga.K1, ga.X2 ? ga.K2 : 0, c.B);
+    void *B = c.prep ? c.prep->place(p) : nullptr;
+    if (c.recording()) return IT_OK;
+    if (!B) {
+      B = c.B;
+      IT_TRY(it_launch_prep_weights_tc(&p, 1, nullptr, 0, c.st));
+    }
+    return it_launch_gemm_tc(ga, B, L->att_src, L->att_dst, heads, hd, want_scores ? scores : nullptr, g->num_sms, g->d_status, c.st);
   }
-  ga.B = B;
-  IT_TRY(it_launch_prep_weights(kind, L, K, B, st));
-  return it_launch_gemm(ga, st);
+  if (c.recording()) return IT_OK;
+  ga.B = c.B;
+  IT_TRY(it_launch_prep_weights(kind, L, K, c.B, c.st));
+  return it_launch_gemm(ga, c.st);
 }
 
 // out [M, n_out] = act(X [M, K] * W [K, n_out] + bias): one plain dense product with W taken as it is.
-it_status run_dense(const it_graph *g, const it_layer_desc *L, int64_t M, const void *X, int K, const void *W, int n_out,
-                    const float *bias, it_act act, void *out, float *B, cudaStream_t st) {
+it_status run_dense(const StageCtx &c, int64_t M, const void *X, int K, const void *W, int n_out, const float *bias, it_act act, void *out) {
+  const it_layer_desc *L = c.L;
   it_layer_desc d = *L;   // a view of the layer that names this product's weights
   d.op = IT_GATHER_NONE; d.in_dim = K; d.out_dim = n_out; d.W = W; d.heads = 1; d.edge_dim = 0; d.msg_dim = 0;
   it_gemm_args ga{};
   ga.M = M; ga.x_dtype = L->feat_dtype; ga.X1 = X; ga.K1 = K; ga.X2 = nullptr; ga.K2 = 0;
-  ga.B = B; ga.NB = n_out;
+  ga.B = c.B; ga.NB = n_out;
   ga.n0 = n_out; ga.out0 = out; ga.dt0 = L->feat_dtype; ga.bias0 = bias; ga.act0 = act;
   ga.n1 = 0; ga.out1 = nullptr; ga.dt1 = L->feat_dtype; ga.out2 = nullptr;
-  return run_apply(g, &d, IT_PREP_DENSE, ga, B, nullptr, st);
+  return run_apply(c, &d, IT_PREP_DENSE, ga, nullptr);
 }
 
 // The edge-feature half of the message [w_e h_u | e_vu]: the same reduce over the rows of the edge-feature
@@ -187,17 +226,8 @@ it_status gather_edge_part(it_gather_args gg, const it_layer_desc *L, void *A, i
   return it_launch_gather(gg, st);
 }
 
-struct StageCtx {
-  const it_graph *g;
-  const it_layer_desc *L;
-  LayerWs w;
-  char *ws;
-  float *B, *partials;
-  cudaStream_t st;
-};
-
-it_status stage_ctx(const it_graph *g, const it_layer_desc *L, void *ws, size_t ws_bytes, cudaStream_t st, StageCtx *c) {
-  c->g = g; c->L = L; c->w = plan_layer(g, L); c->ws = (char *)ws; c->st = st;
+it_status stage_ctx(const it_graph *g, const it_layer_desc *L, void *ws, size_t ws_bytes, cudaStream_t st, StageCtx *c, Prepared *prep = nullptr) {
+  c->prep = prep; c->g = g; c->L = L; c->w = plan_layer(g, L); c->ws = (char *)ws; c->st = st;
   IT_REQUIRE(ws_bytes >= c->w.bytes, IT_ERR_WORKSPACE, "workspace has %zu bytes, layer needs %zu", ws_bytes, c->w.bytes);
   IT_REQUIRE(L->W != nullptr, IT_ERR_INVALID_ARG, "W is NULL");
   c->B = reinterpret_cast<float *>(c->ws + c->w.off_B);
@@ -218,23 +248,23 @@ it_status stage_transform(const StageCtx &c, const void *h_self, void *table_out
       ga.NB = L->out_dim + 2 * L->heads;
       ga.n0 = 0; ga.out0 = nullptr; ga.dt0 = dt; ga.bias0 = nullptr; ga.act0 = IT_ACT_NONE;
       ga.n1 = L->out_dim; ga.out1 = table_out; ga.dt1 = dt; ga.out2 = scores_out;
-      return run_apply(g, L, IT_PREP_GAT, ga, c.B, scores_out, c.st);
+      return run_apply(c, L, IT_PREP_GAT, ga, scores_out);
     case PLAN_GCN_REORDER:   // Z = H W
       ga.NB = L->out_dim;
       ga.n0 = 0; ga.out0 = nullptr; ga.dt0 = dt; ga.bias0 = nullptr; ga.act0 = IT_ACT_NONE;
       ga.n1 = L->out_dim; ga.out1 = table_out; ga.dt1 = dt; ga.out2 = nullptr;
-      return run_apply(g, L, IT_PREP_DENSE, ga, c.B, nullptr, c.st);
+      return run_apply(c, L, IT_PREP_DENSE, ga, nullptr);
     case PLAN_SAGE_REORDER:  // S = H W_self + b (stays with the vertex), Z = H W_neigh
       ga.NB = 2 * L->out_dim;
       ga.n0 = L->out_dim; ga.out0 = c.ws + c.w.off_a; ga.dt0 = dt; ga.bias0 = L->bias; ga.act0 = IT_ACT_NONE;
       ga.n1 = L->out_dim; ga.out1 = table_out; ga.dt1 = dt; ga.out2 = nullptr;
-      return run_apply(g, L, IT_PREP_SAGE_REORDER, ga, c.B, nullptr, c.st);
+      return run_apply(c, L, IT_PREP_SAGE_REORDER, ga, nullptr);
     case PLAN_MSG:
       IT_REQUIRE(L->W_edge != nullptr, IT_ERR_INVALID_ARG, "W_edge is NULL");
       // the source part of the message, once per vertex; without edge features that is the whole message
       if (L->edge_dim == 0)
-        return run_dense(g, L, g->n, h_self, L->in_dim, L->W_edge, L->msg_dim, L->bias_edge, L->act_edge, table_out, c.B, c.st);
-      return run_dense(g, L, g->n, h_self, L->in_dim, L->W_edge, L->msg_dim, nullptr, IT_ACT_NONE, table_out, c.B, c.st);
+        return run_dense(c, g->n, h_self, L->in_dim, L->W_edge, L->msg_dim, L->bias_edge, L->act_edge, table_out);
+      return run_dense(c, g->n, h_self, L->in_dim, L->W_edge, L->msg_dim, nullptr, IT_ACT_NONE, table_out);
     default:
       return IT_OK;
   }
@@ -248,10 +278,12 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
   const it_layer_desc *L = c.L;
   const it_dtype dt = L->feat_dtype;
   if (c.w.plan == PLAN_DENSE) return IT_OK;
+  if (c.recording() && !(c.w.plan == PLAN_MSG && L->edge_dim > 0)) return IT_OK;   // a Gather stage without products of its own
   if (c.w.plan == PLAN_GAT) {
     it_gat_args aa{};
     aa.g = g; aa.dtype = dt; aa.heads = L->heads; aa.head_dim = L->out_dim / L->heads; aa.z = table; aa.scores = scores;
     aa.scores_dst = scores_dst; aa.partials = c.partials; aa.counters = reinterpret_cast<int *>(c.ws + c.w.off_counters);
+    aa.zeroed = c.zeroed();
     aa.slope = L->leaky_slope; aa.bias = L->bias; aa.act = L->act; aa.dst = out;
     if (L->edge_dim > 0) {
       IT_REQUIRE(L->att_edge != nullptr, IT_ERR_INVALID_ARG, "GAT layer with edge features needs att_edge");
@@ -263,7 +295,7 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
       IT_TRY(it_launch_gat_edge_rows(g, dt, L->out_dim, L->heads, table, scores, L->att_edge, Zj, sc, c.st));
       if (!batched) { aa.z = Zj; aa.per_edge_rows = 1; }
       aa.per_edge_scores = 1; aa.src_scores = sc;
-    } else {
+    } else if (!(it_small_graph(g) && it_gat_batched(dt, L->heads, L->out_dim / L->heads))) {   // (a small table stays in the L2 as it is)
       float *dense = reinterpret_cast<float *>(c.ws + c.w.off_q);
       IT_TRY(it_launch_compact_scores(g->n_src, L->heads, scores, dense, c.st));
       aa.src_scores = dense;
@@ -273,6 +305,7 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
   it_gather_args gg{};
   gg.g = g; gg.op = L->op == IT_GATHER_GCN ? IT_GATHER_SUM : L->op; gg.use_edge_weights = L->use_edge_weights; gg.dtype = dt;
   gg.partials = c.partials; gg.counters = reinterpret_cast<int *>(c.ws + c.w.off_counters);
+  gg.zeroed = c.zeroed();
   switch (c.w.plan) {
     case PLAN_GCN_REORDER:   // h' = act(sum_e w_e z_u + b) in the gather's epilogue
       gg.dim = L->out_dim; gg.src = table; gg.dst = out; gg.epi = IT_EPI_BIAS_ACT; gg.self_term = nullptr; gg.bias = L->bias; gg.act = L->act;
@@ -292,7 +325,8 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
         void *Q = c.ws + c.w.off_q;
         const size_t es = (size_t)it_dtype_size(dt);
         const char *W_edge_part = (const char *)L->W_edge + (size_t)L->in_dim * L->msg_dim * es;
-        IT_TRY(run_dense(g, L, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, IT_ACT_NONE, Q, c.B, c.st));
+        IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, IT_ACT_NONE, Q));
+        if (c.recording()) return IT_OK;
         IT_TRY(it_launch_edge_messages(g, dt, L->msg_dim, table, Q, L->act_edge, c.st));
         gg.src = Q; gg.src_ld = 0; gg.per_edge_rows = 1;
         return it_launch_gather(gg, c.st);
@@ -320,29 +354,29 @@ it_status stage_update(const StageCtx &c, const void *h_self, const void *agg, v
   switch (c.w.plan) {
     case PLAN_DENSE:   // no Gather stage: h' = act(h W + b)
       ga.X1 = h_self; ga.K1 = L->in_dim; ga.X2 = nullptr; ga.K2 = 0;
-      return run_apply(g, L, IT_PREP_DENSE, ga, c.B, nullptr, c.st);
+      return run_apply(c, L, IT_PREP_DENSE, ga, nullptr);
     case PLAN_GCN:     // h' = act(A W + b)
       ga.X1 = agg; ga.K1 = a_ld; ga.X2 = nullptr; ga.K2 = 0;
-      return run_apply(g, L, IT_PREP_DENSE, ga, c.B, nullptr, c.st);
+      return run_apply(c, L, IT_PREP_DENSE, ga, nullptr);
     case PLAN_SAGE:    // h' = act([h | A] W + b)
       ga.X1 = h_self; ga.K1 = L->in_dim; ga.X2 = agg; ga.K2 = a_ld;
-      return run_apply(g, L, IT_PREP_SAGE, ga, c.B, nullptr, c.st);
+      return run_apply(c, L, IT_PREP_SAGE, ga, nullptr);
     case PLAN_MSG:
       if (L->op == IT_GATHER_GCN) { ga.X1 = agg; ga.K1 = a_ld; ga.X2 = nullptr; ga.K2 = 0; }
       else { ga.X1 = h_self; ga.K1 = L->in_dim; ga.X2 = agg; ga.K2 = a_ld; }
-      return run_apply(g, L, IT_PREP_DENSE, ga, c.B, nullptr, c.st);   // W [K1 + K2, out] taken as it is
+      return run_apply(c, L, IT_PREP_DENSE, ga, nullptr);   // W [K1 + K2, out] taken as it is
     default:
       return IT_OK;
   }
 }
 
 it_status layer_forward_impl(const it_graph *g, const it_layer_desc *L, const void *h_in, void *h_out, char *ws,
-                             size_t ws_bytes, cudaStream_t st) {
+                             size_t ws_bytes, cudaStream_t st, Prepared *prep = nullptr) {
   IT_REQUIRE(g->n_src == g->n, IT_ERR_INVALID_ARG,
              "the graph is one part of a partition (%lld sources, %lld vertices): use it_layer_transform / it_layer_gather / it_layer_update",
              (long long)g->n_src, (long long)g->n);
   StageCtx c;
-  IT_TRY(stage_ctx(g, L, ws, ws_bytes, st, &c));
+  IT_TRY(stage_ctx(g, L, ws, ws_bytes, st, &c, prep));
   const int a_dim = agg_dim_of(L);
   const LayerPlan plan = c.w.plan;
   const bool table_is_input = plan == PLAN_SAGE || plan == PLAN_GCN || plan == PLAN_DENSE;
@@ -398,13 +432,20 @@ bool fused_pair(const it_graph *g, const it_layer_desc *A, const it_layer_desc *
   return true;
 }
 
-struct InferWs { size_t layer_bytes, buf_bytes, off_buf0, off_buf1, off_B2, bytes; };
+struct InferWs { size_t layer_bytes, buf_bytes, off_buf0, off_buf1, off_prep, prep_bytes, bytes; };
+
+// Room for the prepared weights of a layer's products (each at most 8 bytes per entry, K padded to whole k-blocks).
+size_t prep_bytes_of(const it_layer_desc *L) {
+  const size_t fi = (size_t)L->in_dim, fo = (size_t)L->out_dim, fe = (size_t)L->edge_dim, fm = (size_t)L->msg_dim, kpad = 128;
+  if (L->op == IT_GATHER_GAT || L->op == IT_GATHER_NONE) return it_align_up((fi + kpad) * fo * 8);
+  if (fm > 0) return it_align_up((fi + kpad) * fm * 8) + it_align_up((fe + kpad) * fm * 8) + it_align_up((fi + fm + 2 * kpad) * fo * 8);
+  return it_align_up((2 * fi + fe + 2 * kpad) * 2 * fo * 8);
+}
 
 it_status plan_infer(const it_graph *g, const it_layer_desc *layers, int32_t n_layers, InferWs *out) {
   IT_REQUIRE(g != nullptr, IT_ERR_INVALID_ARG, "graph is NULL");
   IT_REQUIRE(layers != nullptr && n_layers >= 1, IT_ERR_INVALID_ARG, "need at least one layer");
-  InferWs w{0, 0, 0, 0, 0, 0};
-  size_t b2_bytes = 0;   // prepared weights of a layer whose transform runs fused with the previous layer's update
+  InferWs w{0, 0, 0, 0, 0, 0, 0};
   for (int i = 0; i < n_layers; ++i) {
     IT_TRY(check_layer(g, &layers[i]));
     if (i > 0) {
@@ -418,17 +459,22 @@ it_status plan_infer(const it_graph *g, const it_layer_desc *layers, int32_t n_l
       size_t hb = it_align_up((size_t)g->n * (size_t)layers[i].out_dim * (size_t)it_dtype_size(layers[i].feat_dtype));
       if (hb > w.buf_bytes) w.buf_bytes = hb;
     }
-    if (i > 0) {
-      const size_t wb = it_align_up(((size_t)layers[i].in_dim + 128) * 2 * (size_t)layers[i].out_dim * 8);
-      if (wb > b2_bytes) b2_bytes = wb;
-    }
+    w.prep_bytes += prep_bytes_of(&layers[i]);
   }
   w.off_buf0 = w.layer_bytes;
   w.off_buf1 = w.off_buf0 + (n_layers >= 2 ? w.buf_bytes : 0);
-  w.off_B2 = w.off_buf1 + (n_layers >= 3 ? w.buf_bytes : 0);
-  w.bytes = w.off_B2 + b2_bytes;
+  w.off_prep = w.off_buf1 + (n_layers >= 3 ? w.buf_bytes : 0);
+  w.bytes = w.off_prep + w.prep_bytes;
   *out = w;
   return IT_OK;
+}
+
+// Between the two passes over a call's layers: everything recorded, in one launch.
+it_status launch_prepared(const it_graph *g, char *ws, const it_layer_desc *first, Prepared &prep, cudaStream_t st) {
+  prep.recording = false;
+  int *words = reinterpret_cast<int *>(ws + plan_layer(g, first).off_counters);   // the same place for every layer
+  const size_t n_words = it_small_graph(g) ? (size_t)g->n_long : 0;
+  return it_launch_prep_weights_tc(prep.m.data(), (int)prep.m.size(), words, n_words, st);
 }
 
 bool overlaps(const void *a, size_t na, const void *b, size_t nb) {
@@ -448,6 +494,44 @@ it_status check_io(const it_graph *g, const void *in, size_t in_bytes, const voi
   IT_REQUIRE(aligned16(in) && aligned16(out), IT_ERR_INVALID_ARG,
              "input and output matrices must be 16-byte aligned (got %p, %p)", in, out);
   IT_REQUIRE(!overlaps(in, in_bytes, out, out_bytes), IT_ERR_INVALID_ARG, "input and output matrices overlap");
+  return IT_OK;
+}
+
+it_status infer_layers(const it_graph *g, const it_layer_desc *layers, int32_t n_layers, const void *x, void *out, char *ws, const InferWs &w,
+                       Prepared &prep, cudaStream_t st) {
+  void *buf[2] = {ws + w.off_buf0, ws + w.off_buf1};
+  const void *cur = x;
+  for (int i = 0; i < n_layers; ++i) {
+    void *dst = (i == n_layers - 1) ? out : buf[i & 1];
+    FusedPair f;
+    if (i + 1 < n_layers && fused_pair(g, &layers[i], &layers[i + 1], &f)) {
+      // layer i up to its aggregate; its update with the transform of layer i + 1, S and Z landing where H would have
+      // been stored; then the rest of layer i + 1
+      const it_layer_desc *A = &layers[i], *Bn = &layers[i + 1];
+      void *dst2 = (i + 1 == n_layers - 1) ? out : buf[(i + 1) & 1];
+      StageCtx ca, cb;
+      IT_TRY(stage_ctx(g, A, ws, w.layer_bytes, st, &ca, &prep));
+      IT_TRY(stage_ctx(g, Bn, ws, w.layer_bytes, st, &cb, &prep));
+      void *agg = agg_dim_of(A) > 0 ? (void *)(ws + ca.w.off_a) : nullptr;
+      if (agg) IT_TRY(stage_gather(ca, cur, nullptr, nullptr, false, agg));
+      const it_prep_tc pa = it_prep_tc_of(f.kind_a, A, f.ga.N1, f.ga.K1, f.ga.K2, nullptr), pb = it_prep_tc_of(f.kind_b, Bn, f.nb_b, f.ga.N1, 0, nullptr);
+      void *B1 = prep.place(pa), *B2 = prep.place(pb);
+      IT_REQUIRE(B1 && B2, IT_ERR_WORKSPACE, "no room for the prepared weights");
+      if (!prep.recording) {
+        char *S = (char *)dst, *Z = (char *)dst + f.s_bytes;
+        if (plan_of(A) == PLAN_GCN) { f.ga.X1 = agg; f.ga.X2 = nullptr; }
+        else { f.ga.X1 = cur; f.ga.X2 = f.ga.K2 > 0 ? agg : nullptr; }
+        f.ga.out0 = S; f.ga.out1 = Z;
+        IT_TRY(it_launch_gemm2_tc(f.ga, B1, B2, g->num_sms, g->d_status, st));
+        IT_TRY(stage_gather(cb, Z, nullptr, nullptr, false, dst2, S));
+      }
+      cur = dst2;
+      ++i;
+      continue;
+    }
+    IT_TRY(layer_forward_impl(g, &layers[i], cur, dst, ws, w.layer_bytes, st, &prep));
+    cur = dst;
+  }
   return IT_OK;
 }
 
@@ -552,7 +636,16 @@ extern "C" it_status it_layer_forward(const it_graph *g, const it_layer_desc *la
   IT_TRY(check_io(g, h_in, in_bytes, h_out, out_bytes));
   IT_REQUIRE(g->n == 0 || (!overlaps(h_in, in_bytes, workspace, workspace_bytes) && !overlaps(h_out, out_bytes, workspace, workspace_bytes)),
              IT_ERR_INVALID_ARG, "h_in / h_out overlaps the workspace");
-  return layer_forward_impl(g, layer, h_in, h_out, (char *)workspace, workspace_bytes, (cudaStream_t)stream);
+  if (g->n == 0) return IT_OK;
+  char *ws = (char *)workspace;
+  InferWs w;
+  IT_TRY(plan_infer(g, layer, 1, &w));
+  if (workspace_bytes < w.bytes) return layer_forward_impl(g, layer, h_in, h_out, ws, workspace_bytes, (cudaStream_t)stream);
+  Prepared prep;
+  prep.base = ws + w.off_prep; prep.cap = w.prep_bytes;
+  IT_TRY(layer_forward_impl(g, layer, h_in, h_out, ws, w.layer_bytes, (cudaStream_t)stream, &prep));
+  IT_TRY(launch_prepared(g, ws, layer, prep, (cudaStream_t)stream));
+  return layer_forward_impl(g, layer, h_in, h_out, ws, w.layer_bytes, (cudaStream_t)stream, &prep);
 }
 
 // ----------------------------------------------------------------------------- no-allocation variant
@@ -610,38 +703,11 @@ extern "C" it_status it_infer(const it_graph *g, const it_layer_desc *layers, in
   IT_TRY(check_io(g, x, x_bytes, out, out_bytes));
   IT_REQUIRE(g->n == 0 || (!overlaps(x, x_bytes, workspace, workspace_bytes) && !overlaps(out, out_bytes, workspace, workspace_bytes)),
              IT_ERR_INVALID_ARG, "x / out overlaps the workspace");
+  if (g->n == 0) return IT_OK;
   char *ws = (char *)workspace;
-  void *buf[2] = {ws + w.off_buf0, ws + w.off_buf1};
-  const void *cur = x;
-  cudaStream_t st = (cudaStream_t)stream;
-  for (int i = 0; i < n_layers; ++i) {
-    void *dst = (i == n_layers - 1) ? out : buf[i & 1];
-    FusedPair f;
-    if (g->n > 0 && i + 1 < n_layers && fused_pair(g, &layers[i], &layers[i + 1], &f)) {
-      // layer i up to its aggregate; its update with the transform of layer i + 1, S and Z landing where H would have
-      // been stored; then the rest of layer i + 1
-      const it_layer_desc *A = &layers[i], *Bn = &layers[i + 1];
-      StageCtx ca, cb;
-      IT_TRY(stage_ctx(g, A, ws, w.layer_bytes, st, &ca));
-      void *agg = agg_dim_of(A) > 0 ? (void *)(ws + ca.w.off_a) : nullptr;
-      if (agg) IT_TRY(stage_gather(ca, cur, nullptr, nullptr, false, agg));
-      void *B2 = ws + w.off_B2;
-      IT_TRY(it_launch_prep_weights_tc(f.kind_a, A, f.ga.N1, f.ga.K1, f.ga.K2, ca.B, st));
-      IT_TRY(it_launch_prep_weights_tc(f.kind_b, Bn, f.nb_b, f.ga.N1, 0, B2, st));
-      char *S = (char *)dst, *Z = (char *)dst + f.s_bytes;
-      if (plan_of(A) == PLAN_GCN) { f.ga.X1 = agg; f.ga.X2 = nullptr; }
-      else { f.ga.X1 = cur; f.ga.X2 = f.ga.K2 > 0 ? agg : nullptr; }
-      f.ga.out0 = S; f.ga.out1 = Z;
-      IT_TRY(it_launch_gemm2_tc(f.ga, ca.B, B2, g->num_sms, g->d_status, st));
-      void *dst2 = (i + 1 == n_layers - 1) ? out : buf[(i + 1) & 1];
-      IT_TRY(stage_ctx(g, Bn, ws, w.layer_bytes, st, &cb));
-      IT_TRY(stage_gather(cb, Z, nullptr, nullptr, false, dst2, S));
-      cur = dst2;
-      ++i;
-      continue;
-    }
-    IT_TRY(layer_forward_impl(g, &layers[i], cur, dst, ws, w.layer_bytes, st));
-    cur = dst;
-  }
-  return IT_OK;
+  Prepared prep;
+  prep.base = ws + w.off_prep; prep.cap = w.prep_bytes;
+  IT_TRY(infer_layers(g, layers, n_layers, x, out, ws, w, prep, (cudaStream_t)stream));
+  IT_TRY(launch_prepared(g, ws, layers, prep, (cudaStream_t)stream));
+  return infer_layers(g, layers, n_layers, x, out, ws, w, prep, (cudaStream_t)stream);
 }

@@ -276,6 +276,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
     tmem_alloc(tmem_slot, tmem_cols);
     tmem_relinquish();
   }
+  it_allow_next();
+  it_wait_prior();   // everything above is this CTA's own set-up
   for (int c = threadIdx.x; c < p.nbc; c += blockDim.x) {
     const int gc = (blockIdx.x % p.n_splits) * p.nbc + c;
     bias_s[c] = (p.bias0 && gc < p.n0) ? p.bias0[gc] : 0.f;
@@ -883,6 +885,8 @@ gemm2_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constan
     tmem_alloc(tmem_slot, tmem_cols);
     tmem_relinquish();
   }
+  it_allow_next();
+  it_wait_prior();   // everything above is this CTA's own set-up
   for (int c = threadIdx.x; c < p.N1; c += blockDim.x) cst1[c] = p.bias1 ? p.bias1[c] : 0.f;
   for (int c = threadIdx.x; c < p.N2; c += blockDim.x) cst2[c] = (p.bias0 && c < p.n0) ? p.bias0[c] : 0.f;
   tc_fence_before();
@@ -1027,17 +1031,24 @@ gemm2_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constan
 }
 
 // ----------------------------------------------------------------------------- weight prep (K-major, split)
+constexpr int PREP_MAX = 12;   // matrices per launch
 struct PrepTcParams {
-  int kind, in_dim, out_dim, w_is_bf16, NB;
-  int K1, K1p, K2, K2p;   // rows of W behind X1 / X2, and the same rounded up to whole k-blocks (the padding is zero)
-  const void *W;
-  void *B;   // bf16 [NB, K1p + K2p]  or  fp32 [2, NB, K1p + K2p] (hi, lo)
+  it_prep_tc m[PREP_MAX];
+  int *zero;
+  int64_t words;
 };
 
-__global__ void prep_weights_tc_kernel(PrepTcParams p) {
+// blockIdx.y: the matrix; block (0, y = 0 ...) of the first row of blocks also clear the words.
+__global__ void __launch_bounds__(256) prep_weights_tc_kernel(const __grid_constant__ PrepTcParams q) {
+  it_allow_next();
+  it_wait_prior();
+  const it_prep_tc &p = q.m[blockIdx.y];
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+  if (blockIdx.y == 0)
+    for (int64_t i = first; i < q.words; i += stride) q.zero[i] = 0;
   const int Kp = p.K1p + p.K2p;
   const int64_t total = (int64_t)p.NB * Kp;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t i = first; i < total; i += stride) {
     const int n = (int)(i / Kp), kp = (int)(i % Kp);
     // padded position -> row of the unpadded product (or none)
     const bool second = kp >= p.K1p;
@@ -1136,13 +1147,24 @@ bool it_tc_supported(const it_gemm_args &a, int heads, int head_dim, bool want_s
   return true;
 }
 
-it_status it_launch_prep_weights_tc(it_prep_kind kind, const it_layer_desc *L, int NB, int K1, int K2, void *B, cudaStream_t st) {
-  PrepTcParams p;
+it_prep_tc it_prep_tc_of(it_prep_kind kind, const it_layer_desc *L, int NB, int K1, int K2, void *B) {
+  it_prep_tc p;
   const int bk = TC_KBLOCK_BYTES / (L->weight_dtype == IT_BF16 ? 2 : 4);
   p.kind = kind; p.in_dim = L->in_dim; p.out_dim = L->out_dim; p.w_is_bf16 = L->weight_dtype == IT_BF16;
   p.NB = NB; p.K1 = K1; p.K2 = K2; p.K1p = (K1 + bk - 1) / bk * bk; p.K2p = (K2 + bk - 1) / bk * bk; p.W = L->W; p.B = B;
-  IT_LAUNCH(IT_K_PREP, 0, 0, st, prep_weights_tc_kernel<<<64, 256, 0, st>>>(p));
-  IT_CUDA_TRY(cudaGetLastError());
+  return p;
+}
+
+size_t it_prep_tc_bytes(const it_prep_tc &p) { return (size_t)p.NB * (size_t)(p.K1p + p.K2p) * (p.w_is_bf16 ? 2 : 8); }
+
+it_status it_launch_prep_weights_tc(const it_prep_tc *list, int count, int *zero, size_t words, cudaStream_t st) {
+  for (int i = 0; i < count || (i == 0 && words > 0); i += PREP_MAX) {
+    PrepTcParams q{};
+    const int here = count - i < PREP_MAX ? count - i : PREP_MAX;
+    for (int k = 0; k < here; ++k) q.m[k] = list[i + k];   // an empty list: one matrix of no elements
+    q.zero = zero; q.words = i == 0 ? (int64_t)words : 0;
+    IT_LAUNCH(IT_K_PREP, 0, 0, st, IT_CUDA_TRY(it_launch_pdl(prep_weights_tc_kernel, dim3(64, here > 0 ? here : 1), dim3(256), 0, st, q)));
+  }
   return IT_OK;
 }
 
@@ -1223,10 +1245,10 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   const double flops = 2.0 * (double)a.M * K * NB;
   if (tf32) {
     IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, gemm_tc_kernel<true><<<(unsigned)grid, TC_THREADS_TF32, smem, st>>>(m1, m2, mb, mo0, mo1, p));
+    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<true>, dim3((unsigned)grid), dim3(TC_THREADS_TF32), smem, st, m1, m2, mb, mo0, mo1, p)));
   } else {
     IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, gemm_tc_kernel<false><<<(unsigned)grid, TC_THREADS_BF16, smem, st>>>(m1, m2, mb, mo0, mo1, p));
+    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<false>, dim3((unsigned)grid), dim3(TC_THREADS_BF16), smem, st, m1, m2, mb, mo0, mo1, p)));
   }
   IT_CUDA_TRY(cudaGetLastError());
   return IT_OK;
@@ -1293,7 +1315,7 @@ it_status it_launch_gemm2_tc(const it_gemm2_args &a, const void *B1, const void 
   const double bytes = (double)a.M * 2.0 * (K + N2) + 2.0 * ((double)K * a.N1 + (double)a.N1 * N2);
   const double flops = 2.0 * (double)a.M * ((double)K * a.N1 + (double)a.N1 * N2);
   IT_CUDA_TRY(cudaFuncSetAttribute(gemm2_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, s.smem));
-  IT_LAUNCH(IT_K_GEMM2_TC, bytes, flops, st, gemm2_tc_kernel<<<(unsigned)grid, TC_THREADS_BF16, s.smem, st>>>(m1, m2, mb1, mb2, mo0, mo1, p));
+  IT_LAUNCH(IT_K_GEMM2_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm2_tc_kernel, dim3((unsigned)grid), dim3(TC_THREADS_BF16), s.smem, st, m1, m2, mb1, mb2, mo0, mo1, p)));
   IT_CUDA_TRY(cudaGetLastError());
   return IT_OK;
 }

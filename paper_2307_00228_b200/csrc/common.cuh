@@ -10,6 +10,12 @@
 #include "inferturbo.h"
 
 #define IT_NUM_SMS_FALLBACK 148
+#ifndef IT_SMALL_ROWS
+#define IT_SMALL_ROWS (1 << 17)
+#endif
+#ifndef IT_SMALL_EDGES
+#define IT_SMALL_EDGES (1 << 21)
+#endif
 
 // ----------------------------------------------------------------------------- errors
 void it_set_error(const char *fmt, ...);
@@ -42,7 +48,7 @@ void it_set_error(const char *fmt, ...);
 enum it_kernel_id {
   IT_K_VALIDATE = 0, IT_K_SPLIT_SCAN, IT_K_SPLIT_FILL, IT_K_BUCKET_SCAN, IT_K_PREP, IT_K_GATHER_CTA, IT_K_GATHER_FLAT,
   IT_K_GATHER_EMPTY, IT_K_COMBINE, IT_K_GEMM_FP32, IT_K_GEMM_TC, IT_K_GAT_CTA, IT_K_GAT_FLAT, IT_K_GAT_EMPTY,
-  IT_K_EDGE_MSG, IT_K_AGG_FINISH, IT_K_GEMM2_TC,
+  IT_K_EDGE_MSG, IT_K_AGG_FINISH, IT_K_GEMM2_TC, IT_K_GATHER_SMALL, IT_K_GAT_SMALL,
   IT_K_COUNT
 };
 // Wraps one kernel launch: counts it and, while profiling is on, brackets it with events on `st`.
@@ -108,8 +114,38 @@ struct it_graph {
   int64_t n_long = 0;                 // vertices gathered in pieces
   int64_t n_partial_rows = 0;         // their pieces: one partial result each
   int32_t *long_owners = nullptr;     // [n_long] ascending vertex ids
+  int32_t *piece_long = nullptr;      // [n_partial_rows]: which of long_owners a piece belongs to
   int64_t *piece_ptr = nullptr;       // [n_long + 1]: the pieces of long_owners[k] are partial rows piece_ptr[k] ..., in edge order
 };
+
+// Graphs whose layers are bound by launches and latency, not by bytes: one kernel then walks every list of a layer's rows and
+// folds the pieces of long vertices itself.  (The line: a layer of n rows costs the one kernel about n / 4.7 ns, a row per
+// warp; the kernels by list cost four launches of 3 to 4 us more.  SMALL_NOTE)
+static inline bool it_small_graph(const it_graph *g) { return g->n <= IT_SMALL_ROWS && g->e <= IT_SMALL_EDGES; }
+
+// Words of zeroed device memory that the gather of one layer needs: the list counters, or (small graphs) how many pieces
+// of every long vertex are done.
+static inline size_t it_gather_words(const it_graph *g) {
+  const size_t lists = IT_MAX_BUCKETS + 1;
+  return it_small_graph(g) && (size_t)g->n_long > lists ? (size_t)g->n_long : lists;
+}
+
+#ifdef __CUDACC__
+// A kernel launched with it_launch_pdl may start while the kernel before it in the stream is still running: it calls
+// it_wait_prior() before it touches global memory (that kernel, and by the same rule every earlier one, has then finished
+// and its writes are visible), and it_allow_next() once all its blocks are resident.
+__device__ __forceinline__ void it_wait_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void it_allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t it_launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st; cfg.attrs = &attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
 
 static inline size_t it_align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
@@ -153,7 +189,8 @@ struct it_gather_args {
   int src_ld;              // 0 means dim
   int per_edge_rows;       // 1: src is [n_edges, dim] and row j belongs to edge j (edge features); 0: rows are looked up by source vertex
   float *partials;         // [n_partial_rows, dim] fp32 scratch (may be NULL when no vertex is gathered in pieces)
-  int *counters;           // IT_MAX_BUCKETS device words of scratch from which warps claim their batches (NULL: fixed strides)
+  int *counters;           // it_gather_words() device words of scratch (see there)
+  int zeroed;              // 1: they are zero already (and are left so by a small graph's kernel)
   void *dst;               // row v starts at dst + v * dst_ld elements and takes dim of them
   int dst_ld;              // 0 means dim
   it_epilogue_kind epi;
@@ -195,7 +232,8 @@ struct it_gat_args {
   const float *src_scores;   // [rows, heads], dense: the source-side logit term that is read per edge (row = source vertex, or the
                              // edge itself with per_edge_scores); NULL: the first half of the rows of `scores`
   float *partials;        // it_gat_partial_bytes() of fp32 scratch for the groups of split vertices (may be NULL if none)
-  int *counters;          // IT_MAX_BUCKETS device words of scratch from which warps claim their batches (NULL: fixed strides)
+  int *counters;          // it_gather_words() device words of scratch (see there)
+  int zeroed;             // 1: they are zero already (and are left so by a small graph's kernel)
   float slope;
   const float *bias;      // may be NULL
   it_act act;
@@ -240,8 +278,16 @@ it_status it_launch_prep_weights(it_prep_kind kind, const it_layer_desc *layer, 
 // attention scores [M, 2*heads] in its epilogue (a.B, a.NB and a.out2 are not used).  B is the
 // matrix written by it_launch_prep_weights_tc: bf16 [NB, Kp] or fp32 [2, NB, Kp] (hi, lo), K-major, Kp = padded K1 + padded K2.
 bool it_tc_supported(const it_gemm_args &a, int heads, int head_dim, bool want_scores);
-it_status it_launch_prep_weights_tc(it_prep_kind kind, const it_layer_desc *layer, int NB, int K1, int K2, void *B,
-                                    cudaStream_t stream);
+struct it_prep_tc {
+  int kind, in_dim, out_dim, w_is_bf16, NB;
+  int K1, K1p, K2, K2p;   // rows of W behind X1 / X2, and the same rounded up to whole k-blocks (the padding is zero)
+  const void *W;
+  void *B;   // bf16 [NB, K1p + K2p]  or  fp32 [2, NB, K1p + K2p] (hi, lo)
+};
+it_prep_tc it_prep_tc_of(it_prep_kind kind, const it_layer_desc *layer, int NB, int K1, int K2, void *B);
+size_t it_prep_tc_bytes(const it_prep_tc &p);
+// Several weight matrices and `words` zeroed words in as few launches as possible.
+it_status it_launch_prep_weights_tc(const it_prep_tc *list, int count, int *zero, size_t words, cudaStream_t stream);
 it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *att_src, const float *att_dst,
                             int heads, int head_dim, float *scores, int num_sms, int *status, cudaStream_t stream);
 

@@ -258,8 +258,9 @@ it_status dispatch_batched(int row_bytes, int heads, F f) {
 
 template <typename T>
 it_status launch_gat(const it_gat_args &a, StreamParams sp, cudaStream_t st) {
-  if (!a.per_edge_rows && a.counters && a.src_scores && it_gat_batched(a.dtype, a.heads, a.head_dim))
+  if (!a.per_edge_rows && a.counters && it_gat_batched(a.dtype, a.heads, a.head_dim))
     return dispatch_batched(a.heads * a.head_dim * (int)sizeof(T), a.heads, [&]<int LPR, int H>() {
+      if (it_small_graph(a.g)) return launch_gat_small<T, LPR, H>(a, sp, make_policy<T, 16>(a), st);
       return launch_gat_rows<T, LPR, H>(a, sp, make_policy<T, 16>(a), gat_bytes(a), st);
     });
   // 16-byte slices as long as one never straddles two heads
@@ -299,7 +300,7 @@ it_status it_launch_gat(const it_gat_args &a, cudaStream_t st) {
   sp.src_pitch = (uint32_t)(sp.dim * it_dtype_size(a.dtype));
   if (a.dtype == IT_F32) IT_TRY(launch_gat<float>(a, sp, st));
   else IT_TRY(launch_gat<__nv_bfloat16>(a, sp, st));
-  if (g->n_long > 0) {
+  if (g->n_long > 0 && !(it_small_graph(g) && it_gat_batched(a.dtype, a.heads, a.head_dim) && !a.per_edge_rows)) {
     GatCombineParams c;
     c.long_owners = g->long_owners; c.piece_ptr = g->piece_ptr; c.partials = a.partials; c.bias = a.bias;
     c.dst = a.dst; c.n_long = g->n_long; c.dim = a.heads * a.head_dim; c.heads = a.heads;

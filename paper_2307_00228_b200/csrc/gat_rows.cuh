@@ -15,15 +15,16 @@
 // Included by gat.cu.
 #pragma once
 
-#include "stream.cuh"
+#include "gather_small.cuh"
 
 namespace {
 
 using namespace it_stream;
 
 struct GatParams {
-  const float *__restrict__ scores;       // source-side logit term: [n_src, H], or [n_edges, H] when per_edge
+  const float *__restrict__ scores;       // source-side logit term: [n_src, H], or [n_edges, H] when per_edge (rows of `stride`)
   const float *__restrict__ scores_dst;   // [local destinations, 2H]: destination scores in the second half
+  int stride;                             // floats from one row of it to the next (H, or 2H for the interleaved score rows)
   int per_edge;                           // the term belongs to the edge (edge features in the logits), not to its source
   float slope;
   int head_dim;
@@ -96,7 +97,7 @@ struct GatWarp {
     for (int i = 0; i < H; ++i) {
       const int e = el + i * EP;
       const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, c.idx, e);
-      if (e < c.cnt) x_n[i] = __ldg(q.scores + (q.per_edge ? (uint64_t)(c.j + e) : (uint64_t)s) * H + hl);
+      if (e < c.cnt) x_n[i] = __ldg(q.scores + (q.per_edge ? (uint64_t)(c.j + e) : (uint64_t)s) * q.stride + hl);
     }
     sd_n = __ldg(q.scores_dst + (int64_t)c.owner * (2 * H) + H + hl);
   }
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_SHORT_BLOCKS) gat_short_rows_k
       const int e = el + u * EP;
       const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx, gbase + (e & (E - 1)));
       x[u] = -INFINITY;
-      if (e < E && k + e < r.len) x[u] = __ldg(q.scores + (q.per_edge ? (uint64_t)(r.j0 + k + e) : (uint64_t)s) * H + hl);
+      if (e < E && k + e < r.len) x[u] = __ldg(q.scores + (q.per_edge ? (uint64_t)(r.j0 + k + e) : (uint64_t)s) * q.stride + hl);
     }
   };
 
@@ -291,12 +292,113 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_SHORT_BLOCKS) gat_short_rows_k
   cp_async_wait<0>();
 }
 
+// ----------------------------------------------------------------------------- small graphs: every list of a layer in one kernel
+template <typename T, int LPR, int H>
+__global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol, PieceParams pq) {
+  constexpr int SL = 32 / LPR, U = 8, VEC = GatAcc<T>::VEC, NS = GatPolicy<T, 16>::NS;
+  __shared__ float weights[THREADS / 32][32 * H];
+  __shared__ float bias_buf[256];
+  it_allow_next();
+  const int lane = threadIdx.x & 31, slot = lane / LPR, t = lane % LPR;
+  pol.setup(t);
+  const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
+  it_wait_prior();
+  stage_bias(pol, bias_buf);
+  GatWarp<T, LPR, H> gw(p, q, lane, (uint32_t)__cvta_generic_to_shared(&weights[threadIdx.x >> 5][0]));
+  small_walk<false, true>(p, lane, [&](const it_row_meta &m, int owner, int32_t idx, float) {
+    gw.acc.init(gw.st);
+    gw.m = -INFINITY;
+    for (int base = 0; base < m.len; base += 32) {
+      Chunk c;
+      c.cnt = m.len - base < 32 ? m.len - base : 32;
+      int32_t idx_n = 0;   // the next chunk's ids, in flight while this one's rows are
+      if (base + 32 + lane < m.len) idx_n = p.indices ? __ldg(p.indices + m.j0 + base + 32 + lane) : (int32_t)(m.j0 + base + 32 + lane);
+      c.idx = idx; c.owner = owner; c.j = m.j0 + base;
+      gw.ahead(c);
+      uint4 v[U];
+      auto load = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int e = k0 + u * SL + slot;
+          const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx, e & 31);
+          if (e < c.cnt) v[u] = __ldg(reinterpret_cast<const uint4 *>(my_src + (uint64_t)s * p.src_pitch));
+        }
+      };
+      load(0);
+      gw.begin(c, base == 0);
+      for (int k0 = 0; k0 < c.cnt; k0 += SL * U) {
+        if (k0 > 0) load(k0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int e = k0 + u * SL + slot;
+          if (e < c.cnt) gw.acc.edge(gw.st, v[u], gw.weight(e));
+        }
+      }
+      idx = idx_n;
+    }
+#pragma unroll
+    for (int o = 16; o >= LPR; o >>= 1) {
+      float other[GatAcc<T>::NS];
+#pragma unroll
+      for (int k = 0; k < GatAcc<T>::NS; ++k) other[k] = __shfl_xor_sync(0xffffffffu, gw.st[k], o);
+      gw.acc.merge(gw.st, other);
+    }
+    const float mh = __shfl_sync(0xffffffffu, gw.m, gw.hc);
+    float full[NS];
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) full[k] = gw.st[k];
+    full[VEC] = mh;
+    full[VEC + 1] = gw.st[VEC];
+    if (slot == 0) pol.end_row(full, m.dest, 0, m.len);
+    if (m.dest < 0) {
+      int k;
+      if (last_piece(pq, ~m.dest, lane, k) && slot == 0) {   // merge the vertex's pieces in order, a slice per lane
+        const int64_t p0 = __ldg(pq.piece_ptr + k), p1 = __ldg(pq.piece_ptr + k + 1);
+        const int stride = gat_partial_stride(pol.dim, pol.heads);
+        pol.init(full);
+        for (int64_t g0 = p0; g0 < p1; g0 += 4) {   // four in flight
+          float x[4][NS];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const float *row = pol.partials + (g0 + u < p1 ? g0 + u : g0) * stride;
+#pragma unroll
+            for (int k4 = 0; k4 < VEC; k4 += 4) {
+              const float4 y = __ldcg(reinterpret_cast<const float4 *>(row + pol.col + k4));
+              x[u][k4] = y.x; x[u][k4 + 1] = y.y; x[u][k4 + 2] = y.z; x[u][k4 + 3] = y.w;
+            }
+            x[u][VEC] = __ldcg(row + pol.dim + pol.head);
+            x[u][VEC + 1] = __ldcg(row + pol.dim + pol.heads + pol.head);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (g0 + u < p1) pol.merge(full, x[u]);
+        }
+        pol.end_row(full, __ldg(pq.long_owners + k), 0, 1);
+      }
+    }
+  });
+}
+
+template <typename T, int LPR, int H>
+it_status launch_gat_small(const it_gat_args &a, StreamParams p, const GatPolicy<T, 16> &pol, cudaStream_t st) {
+  const it_graph *g = a.g;
+  GatParams q;
+  q.scores = pol.scores; q.scores_dst = pol.scores_dst; q.stride = pol.src_stride; q.per_edge = a.per_edge_scores; q.slope = pol.slope; q.head_dim = pol.head_dim;
+  p.row_lo = 0; p.row_hi = g->h_list_offsets[g->n_lists]; p.slices = LPR;
+  if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, (size_t)g->n_long * sizeof(int), st));
+  const double row_bytes = (double)pol.dim * sizeof(T);
+  const double bytes = (double)g->e * (4.0 + 4.0 * H + row_bytes) + (double)g->n * (20.0 + 4.0 * H + row_bytes);
+  IT_LAUNCH(IT_K_GAT_SMALL, bytes, 0, st,
+            IT_CUDA_TRY(it_launch_pdl(gat_small_kernel<T, LPR, H>, dim3(small_grid(g)), dim3(THREADS), 0, st, p, q, pol, piece_params(g, a.counters))));
+  return IT_OK;
+}
+
 // ----------------------------------------------------------------------------- launches
 template <typename T, int LPR, int H, class BytesF>
 it_status launch_gat_rows(const it_gat_args &a, StreamParams p, const GatPolicy<T, 16> &pol, BytesF bytes_of, cudaStream_t st) {
   const it_graph *g = a.g;
   GatParams q;
-  q.scores = pol.scores; q.scores_dst = pol.scores_dst; q.per_edge = a.per_edge_scores; q.slope = pol.slope; q.head_dim = pol.head_dim;
+  q.scores = pol.scores; q.scores_dst = pol.scores_dst; q.stride = pol.src_stride; q.per_edge = a.per_edge_scores; q.slope = pol.slope; q.head_dim = pol.head_dim;
   p.slices = LPR;
   if (a.counters) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, (IT_MAX_BUCKETS + 1) * sizeof(int), st));
   bool chunked = false;

@@ -209,7 +209,7 @@ static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
   sp.src_pitch = (uint32_t)((a.src_ld > 0 ? a.src_ld : a.dim) * it_dtype_size(a.dtype));
   if (a.dtype == IT_F32) IT_TRY(it_launch_gather_rows_f32(a, sp, st));
   else IT_TRY(it_launch_gather_rows_bf16(a, sp, st));
-  if (g->n_long > 0) {
+  if (g->n_long > 0 && !it_small_graph(g)) {
     CombineParams c;
     c.long_owners = g->long_owners; c.piece_ptr = g->piece_ptr; c.owner_indptr = g->owner_indptr; c.shadow_indptr = g->shadow_indptr;
     c.partials = a.partials; c.dst = a.dst; c.self_term = a.self_term; c.bias = a.bias; c.n_long = g->n_long;
@@ -226,7 +226,7 @@ static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
 }
 
 // Rows of any multiple of 16 bytes: the kernels take rows of 16, 32, 64 and 80 to 512 bytes, so a wider row (or one of 48
-// bytes) is cut into column chunks, largest first, and each chunk is gathered on its own, reading and writing
+// bytes, unless the graph is small) is cut into column chunks, largest first, and each chunk is gathered on its own, reading and writing
 // its columns in place.  The aggregate is entry by entry, so the chunks are independent; each pass re-reads
 // the edge indices (4 bytes against a chunk of up to 512 per edge).
 it_status it_launch_gather(const it_gather_args &a, cudaStream_t st) {
@@ -244,7 +244,7 @@ it_status it_launch_gather(const it_gather_args &a, cudaStream_t st) {
     // what is left as one chunk where a kernel takes it: up to 512 bytes, and from 80 bytes on any multiple of 16 (the
     // lanes past the row idle); 48 bytes as 32 + 16
     const int left = (full - c0) * es;
-    const int bytes = left >= 512 ? 512 : (left == 48 ? 32 : left);
+    const int bytes = left >= 512 ? 512 : (left == 48 && !it_small_graph(g) ? 32 : left);
     it_gather_args c = a;
     c.dim = bytes / es;
     c.src = (const char *)a.src + (size_t)c0 * es;

@@ -2,7 +2,7 @@
 // itself lives in stream.cuh; this file supplies the per-lane state and what happens at the end of a row.  Included by
 // one source file per storage type (the kernels are many; they compile side by side).
 #pragma once
-#include "stream.cuh"
+#include "gather_small.cuh"
 
 namespace {
 
@@ -103,12 +103,121 @@ struct SagePolicy {
   }
 };
 
-// ----------------------------------------------------------------------------- dispatch
-template <typename T, int SB, int LPR, int RED, bool WEIGHTED>
-it_status launch_policy(const it_gather_args &a, StreamParams sp, int64_t bound_lo, int64_t bound_hi, cudaStream_t st) {
+template <typename T, int SB, int RED, bool WEIGHTED>
+SagePolicy<T, SB, RED, WEIGHTED> make_policy(const it_gather_args &a) {
   SagePolicy<T, SB, RED, WEIGHTED> pol;
   pol.partials = a.partials; pol.dst = a.dst; pol.self_term = a.self_term; pol.bias = a.bias; pol.dim = a.dim; pol.dst_ld = a.dst_ld > 0 ? a.dst_ld : a.dim; pol.self_ld = a.self_ld > 0 ? a.self_ld : a.dim;
   pol.is_mean = a.op == IT_GATHER_MEAN && a.epi != IT_EPI_RAW_F32; pol.epi = a.epi; pol.act = a.act; pol.col = 0;
+  return pol;
+}
+
+// ----------------------------------------------------------------------------- small graphs: every list of a layer in one kernel
+template <typename T, int LPR, class Policy>
+__global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(StreamParams p, Policy pol, PieceParams q, const int64_t *__restrict__ owner_indptr,
+                                                                          const int64_t *__restrict__ shadow_indptr) {
+  constexpr int SL = 32 / LPR, U = LPR < 8 ? LPR : 8;   // edge slots; rows in flight per lane (SL * U <= 32)
+  constexpr int NS = Policy::NS;
+  using Slice = typename Policy::Slice;
+  it_allow_next();
+  const int lane = threadIdx.x & 31, slot = lane / LPR, t = lane % LPR;
+  const bool active = t < p.slices;
+  pol.setup(t);
+  const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
+  it_wait_prior();
+  small_walk<true, false>(p, lane, [&](const it_row_meta &m, int, int32_t idx, float w) {
+    float st[NS];
+    pol.init(st);
+    if (active) pol.begin_row(m.dest, 0);
+    for (int base = 0; base < m.len; base += 32) {
+      int32_t idx_n = 0;   // the next chunk's ids, in flight while this one's rows are
+      float w_n = 1.f;
+      if (base + 32 + lane < m.len) {
+        idx_n = p.indices ? __ldg(p.indices + m.j0 + base + 32 + lane) : (int32_t)(m.j0 + base + 32 + lane);
+        if (p.weights) w_n = __ldg(p.weights + m.j0 + base + 32 + lane);
+      }
+      const int cnt = m.len - base < 32 ? m.len - base : 32;
+      for (int k0 = 0; k0 < cnt; k0 += SL * U) {
+        typename Slice::Raw v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int e = k0 + u * SL + slot;
+          const uint32_t src = (uint32_t)__shfl_sync(0xffffffffu, idx, e & 31);
+          if (e < cnt && active) v[u] = Slice::load(my_src + (uint64_t)src * p.src_pitch);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int e = k0 + u * SL + slot;
+          const float we = __shfl_sync(0xffffffffu, w, e & 31);
+          if (e < cnt) pol.edge(st, v[u], we, 0.f);
+        }
+      }
+      idx = idx_n; w = w_n;
+    }
+#pragma unroll
+    for (int o = 16; o >= LPR; o >>= 1) {
+      float other[NS];
+#pragma unroll
+      for (int k = 0; k < NS; ++k) other[k] = __shfl_xor_sync(0xffffffffu, st[k], o);
+      pol.merge(st, other);   // only slot 0 is read afterwards, and there st is always the lower slot
+    }
+    if (slot == 0 && active) pol.end_row(st, m.dest, 0, m.len);
+    if (m.dest < 0) {
+      int k;
+      if (last_piece(q, ~m.dest, lane, k) && slot == 0 && active) {   // fold the vertex's pieces in order, a slice per lane
+        const int64_t v = __ldg(q.long_owners + k), p0 = __ldg(q.piece_ptr + k), p1 = __ldg(q.piece_ptr + k + 1);
+        const int64_t deg = __ldg(shadow_indptr + __ldg(owner_indptr + v + 1)) - __ldg(shadow_indptr + __ldg(owner_indptr + v));
+        pol.begin_row((int32_t)v, 0);
+        pol.init(st);
+        for (int64_t g0 = p0; g0 < p1; g0 += 4) {   // four in flight
+          float x[4][NS];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const float4 *row = reinterpret_cast<const float4 *>(pol.partials + (g0 + u < p1 ? g0 + u : g0) * pol.dim + pol.col);
+#pragma unroll
+            for (int k4 = 0; k4 < NS; k4 += 4) {
+              const float4 y = __ldcg(row + k4 / 4);
+              x[u][k4] = y.x; x[u][k4 + 1] = y.y; x[u][k4 + 2] = y.z; x[u][k4 + 3] = y.w;
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (g0 + u < p1) pol.merge(st, x[u]);
+        }
+        pol.end_row(st, (int32_t)v, 0, deg);
+      }
+    }
+  });
+}
+
+template <typename T, int RED>
+it_status launch_small(const it_gather_args &a, StreamParams sp, cudaStream_t st) {
+  const it_graph *g = a.g;
+  const auto pol = make_policy<T, 16, RED, true>(a);
+  const int slices = a.dim * (int)sizeof(T) / 16;
+  const double row_bytes = (double)a.dim * sizeof(T);
+  const double bytes = (double)g->e * ((a.per_edge_rows ? 0.0 : 4.0) + (a.use_edge_weights ? 4.0 : 0.0) + row_bytes) +
+                       (double)g->n * (16.0 + row_bytes + (a.epi == IT_EPI_ADD_ACT ? row_bytes : 0.0));
+  sp.row_lo = 0; sp.row_hi = g->h_list_offsets[g->n_lists]; sp.slices = slices;
+  sp.weights = a.use_edge_weights ? sp.weights : nullptr;
+  if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, (size_t)g->n_long * sizeof(int), st));
+  auto go = [&]<int LPR>() -> it_status {
+    IT_LAUNCH(IT_K_GATHER_SMALL, bytes, 0, st,
+              IT_CUDA_TRY(it_launch_pdl(gather_small_kernel<T, LPR, decltype(make_policy<T, 16, RED, true>(a))>, dim3(small_grid(g)), dim3(THREADS), 0, st, sp, pol,
+                                        piece_params(g, a.counters), (const int64_t *)g->owner_indptr, (const int64_t *)g->shadow_indptr)));
+    return IT_OK;
+  };
+  if (slices <= 1) return go.template operator()<1>();
+  if (slices <= 2) return go.template operator()<2>();
+  if (slices <= 4) return go.template operator()<4>();
+  if (slices <= 8) return go.template operator()<8>();
+  if (slices <= 16) return go.template operator()<16>();
+  return go.template operator()<32>();
+}
+
+// ----------------------------------------------------------------------------- dispatch
+template <typename T, int SB, int LPR, int RED, bool WEIGHTED>
+it_status launch_policy(const it_gather_args &a, StreamParams sp, int64_t bound_lo, int64_t bound_hi, cudaStream_t st) {
+  const auto pol = make_policy<T, SB, RED, WEIGHTED>(a);
   const it_graph *g = a.g;
   // algorithmic bytes: per edge the index, the optional weight and one source row; per row its
   // metadata and one output row (plus the self row it is added to)
@@ -128,6 +237,11 @@ it_status launch_policy(const it_gather_args &a, StreamParams sp, int64_t bound_
 
 template <typename T>
 it_status launch_lpr(const it_gather_args &a, StreamParams sp, cudaStream_t st) {
+  if (it_small_graph(a.g)) {
+    if (a.op == IT_GATHER_MAX) return launch_small<T, RED_MAX>(a, sp, st);
+    if (a.op == IT_GATHER_MIN) return launch_small<T, RED_MIN>(a, sp, st);
+    return launch_small<T, RED_SUM>(a, sp, st);
+  }
   const bool w = a.use_edge_weights != 0;
   return dispatch_row_bytes(a.dim * (int)sizeof(T), true, [&]<int SB, int LPR>(int64_t lo, int64_t hi) {
     if (a.op == IT_GATHER_MAX) return w ? launch_policy<T, SB, LPR, RED_MAX, true>(a, sp, lo, hi, st) : launch_policy<T, SB, LPR, RED_MAX, false>(a, sp, lo, hi, st);

@@ -1,0 +1,88 @@
+// One kernel per layer for small graphs: a warp per row of any length (pieces of long vertices, whole vertices, rows without
+// edges), source rows straight into registers, and the pieces of a long vertex folded by the warp that finishes the last of
+// them.  The record of a warp's next-but-one row and the ids of its next row are in flight while a row is reduced.
+// What bounds it: the dependent trips record -> ids -> source rows out of the L2 and the launch itself.  A layer of 10k
+// vertices and 100k edges took five launches (a memset, three kernels by row length, empty rows, combine).  SMALL_MEASURED
+//
+// Included by gather_rows.cuh and gat_rows.cuh.
+#pragma once
+
+#include "stream.cuh"
+
+namespace it_stream {
+
+// The pieces of long vertices in flight: the warp that finishes the last piece of a vertex folds them all.
+struct PieceParams {
+  const int32_t *__restrict__ piece_long;   // which long vertex a piece belongs to
+  const int64_t *__restrict__ piece_ptr;
+  const int32_t *__restrict__ long_owners;
+  int *done;                                // pieces finished, per long vertex: zero before and after the launch
+};
+
+// All lanes of the warp have written their share of piece `slot`: true (warp-uniform) in the warp that finished the last
+// piece of the vertex; the others' partial results are then visible to it (through the L2: read them with __ldcg).
+__device__ __forceinline__ bool last_piece(const PieceParams &q, int slot, int lane, int &k) {
+  k = __ldg(q.piece_long + slot);
+  __threadfence();
+  __syncwarp();
+  int last = 0;
+  if (lane == 0) {
+    const int n = (int)(__ldg(q.piece_ptr + k + 1) - __ldg(q.piece_ptr + k));
+    last = atomicAdd(q.done + k, 1) == n - 1;
+    if (last) q.done[k] = 0;
+  }
+  last = __shfl_sync(0xffffffffu, last, 0);
+  if (last) __threadfence();
+  return last != 0;
+}
+
+constexpr int SMALL_BLOCKS = 3;   // resident CTAs per SM
+
+// The rows of one warp, from the end of the list (pieces first) in turn.
+//   row(m, owner, idx, w): reduce one row; idx / w: ids and weights of its first 32 edges, one per lane
+template <bool WEIGHTED, bool OWNER, class Row>
+__device__ __forceinline__ void small_walk(const StreamParams &p, int lane, Row row) {
+  const int W = (int)gridDim.x * (THREADS / 32), n = (int)p.row_hi;
+  int i = (int)blockIdx.x * (THREADS / 32) + (int)(threadIdx.x >> 5);
+  it_row_meta m[3];
+  int owner[3];
+  auto fetch = [&](int at, it_row_meta &x, int &o) {
+    x.j0 = 0; x.len = 0; x.dest = 0; o = 0;
+    if (at < n) {
+      x = load_meta(p.meta + (n - 1 - at));
+      if (OWNER) o = __ldcs(p.owner + (n - 1 - at));
+    }
+  };
+  auto ids = [&](const it_row_meta &x, int32_t &idx, float &w) {
+    idx = 0; w = 1.f;
+    if (lane < x.len) {
+      idx = p.indices ? __ldg(p.indices + x.j0 + lane) : (int32_t)(x.j0 + lane);
+      if (WEIGHTED && p.weights) w = __ldg(p.weights + x.j0 + lane);
+    }
+  };
+  int32_t idx[2];
+  float w[2];
+  fetch(i, m[0], owner[0]);
+  fetch(i + W, m[1], owner[1]);
+  ids(m[0], idx[0], w[0]);
+  for (; i < n; i += W) {
+    fetch(i + 2 * W, m[2], owner[2]);
+    ids(m[1], idx[1], w[1]);
+    row(m[0], owner[0], idx[0], w[0]);
+    m[0] = m[1]; owner[0] = owner[1]; m[1] = m[2]; owner[1] = owner[2];
+    idx[0] = idx[1]; w[0] = w[1];
+  }
+}
+
+inline unsigned small_grid(const it_graph *g) {
+  const int64_t rows = g->h_list_offsets[g->n_lists], want = (rows + THREADS / 32 - 1) / (THREADS / 32), most = (int64_t)g->num_sms * SMALL_BLOCKS;
+  return (unsigned)(want < most ? want : most);
+}
+
+inline PieceParams piece_params(const it_graph *g, int *done) {
+  PieceParams q;
+  q.piece_long = g->piece_long; q.piece_ptr = g->piece_ptr; q.long_owners = g->long_owners; q.done = done;
+  return q;
+}
+
+}  // namespace it_stream

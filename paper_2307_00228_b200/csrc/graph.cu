@@ -120,16 +120,16 @@ struct SplitParams {
   int64_t *tiles;          // [SPLIT_COLS][n_tiles]
   int64_t *totals;         // [SPLIT_COLS] column sums, then [IT_MAX_BUCKETS] edges per list (the last one: of the pieces)
   int64_t long_above;      // vertices of more edges are gathered in pieces
-  int piece_min;
+  int piece_min, piece_max;
   int64_t *shadow_indptr; int32_t *shadow_owner; int64_t *owner_indptr;
   int64_t *bucket_offsets; int32_t *bucket_rows;
   it_row_meta *list_meta; int32_t *list_owner;
-  int32_t *long_owners; int64_t *piece_ptr; LongInfo *info;   // [long vertices]
+  int32_t *long_owners; int64_t *piece_ptr; int32_t *piece_long; LongInfo *info;   // [long vertices]
   int *bins;               // [2][PIECE_BINS]: pieces per bin, then the next free place
 };
 
 __device__ __forceinline__ int64_t pieces_of(int64_t d, const SplitParams &p) {
-  const int64_t by_share = d / 64, least = by_share < p.piece_min ? p.piece_min : by_share, len = least > 512 ? 512 : least;
+  const int64_t by_share = d / 64, least = by_share < p.piece_min ? p.piece_min : by_share, len = least > p.piece_max ? p.piece_max : least;
   return (d + len - 1) / len;
 }
 
@@ -403,6 +403,7 @@ __global__ void __launch_bounds__(PIECE_BINS) long_pieces_kernel(SplitParams p) 
       m.dest = (int32_t)~(p0 + g);
       p.list_meta[pos] = m;
       p.list_owner[pos] = (int32_t)v;
+      p.piece_long[p0 + g] = (int32_t)k;
     }
   }
 }
@@ -410,7 +411,7 @@ __global__ void __launch_bounds__(PIECE_BINS) long_pieces_kernel(SplitParams p) 
 // ----------------------------------------------------------------------------- host side
 static void forget_split(it_graph *g) {
   g->shadow_indptr = nullptr; g->shadow_owner = nullptr; g->owner_indptr = nullptr;
-  g->long_owners = nullptr; g->piece_ptr = nullptr; g->bucket_offsets = nullptr; g->bucket_rows = nullptr;
+  g->long_owners = nullptr; g->piece_ptr = nullptr; g->piece_long = nullptr; g->bucket_offsets = nullptr; g->bucket_rows = nullptr;
   g->list_meta = nullptr; g->list_owner = nullptr;
   g->n_rows = g->n_split_owners = g->n_partial_rows = g->n_long = 0;
   g->n_buckets = g->n_lists = 0;
@@ -436,6 +437,7 @@ static size_t carve_split(SplitParams &p, char *slab, int64_t R, int64_t L, int6
   take(p.list_owner, p.n + P);
   take(p.long_owners, L);
   take(p.piece_ptr, L + 1);
+  take(p.piece_long, P);
   take(p.info, L);
   return off;
 }
@@ -462,8 +464,11 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   // the vertices that are worth it (25M sources: pieces above 1024 edges 26.3 ms, above 4096 22.9, above 2048 22.6; 5M: above 1024
   // 11.7, above 2441 12.1).
   p.long_above = g->n_src / 12288 < 1024 ? 1024 : (g->n_src / 12288 > 4096 ? 4096 : g->n_src / 12288);
-  if (T > 0 && T < p.long_above) p.long_above = T;
   p.piece_min = g->n_src < ((int64_t)1 << 17) ? 256 : 128;
+  p.piece_max = 512;
+  // small graphs: a warp's longest row is the time of the launch (120 edges per warp on average at 420k edges)
+  if (it_small_graph(g)) p.long_above = p.piece_min = p.piece_max = 128;
+  if (T > 0 && T < p.long_above) p.long_above = T;
 
   // at most one row per vertex and one more per T edges, a long vertex per long_above edges, a piece per piece_min of them
   // and one more each; only where that is far above the number of vertices are they counted before the arrays are laid out
@@ -527,7 +532,7 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   }
   g->shadow_indptr = p.shadow_indptr; g->shadow_owner = p.shadow_owner; g->owner_indptr = p.owner_indptr;
   g->bucket_offsets = p.bucket_offsets; g->bucket_rows = p.bucket_rows; g->list_meta = p.list_meta; g->list_owner = p.list_owner;
-  g->long_owners = p.long_owners; g->piece_ptr = p.piece_ptr;
+  g->long_owners = p.long_owners; g->piece_ptr = p.piece_ptr; g->piece_long = p.piece_long;
   g->n_rows = h[nb];
   g->n_split_owners = h[nb + 1];
   g->n_long = h[nb + 2];
@@ -542,7 +547,7 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   }
   g->h_list_offsets[nb + 1] = n + (g->n_partial_rows - g->n_long);
   g->h_list_edges[nb] = h[SPLIT_COLS + IT_MAX_BUCKETS - 1];
-  g->list_bounds[nb] = 512;
+  g->list_bounds[nb] = p.piece_max;
   for (int i = 0; i < IT_MAX_BUCKETS; ++i) g->bucket_bounds[i] = i < p.B.nb ? p.B.b[i] : 0;
   return IT_OK;
 }
