@@ -18,7 +18,7 @@ struct GatPolicy {
   using Slice = RowSlice<T, SB>;
   static constexpr int VEC = Slice::VEC;
   static constexpr int NS = VEC + 2;   // accumulators, running max, running sum
-  static constexpr bool WEIGHTED = false, HAS_EXTRA = true, NEEDS_OWNER = true;
+  static constexpr bool WEIGHTED = false, HAS_EXTRA = true, NEEDS_OWNER = true, NULLABLE = false;
   const float *__restrict__ scores;    // [n_src, 2*heads]: source scores of the vertex, then its destination scores
   const float *__restrict__ scores_dst;   // the same rows, counted from the first local destination
   const float *__restrict__ bias;

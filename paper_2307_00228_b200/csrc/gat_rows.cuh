@@ -168,25 +168,22 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_k
 #ifndef IT_GAT_SHORT_BLOCKS
 #define IT_GAT_SHORT_BLOCKS 3   // resident CTAs per SM: 64 KB of staging each
 #endif
+// block / blocks: which share of the rows p.row_lo .. p.row_hi this block walks; short_buf: [2][E][THREADS] in shared memory.
 template <typename T, int LPR, int H>
-__global__ void __launch_bounds__(THREADS, IT_GAT_SHORT_BLOCKS) gat_short_rows_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol) {
+__device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatParams &q, const GatPolicy<T, 16> &pol, int block, int blocks, uint4 *short_buf) {
   using Acc = GatAcc<T>;
   constexpr int E = IT_SHORT_EDGES;
   constexpr int EP = LPR / H;                            // edges covered by one pair per lane
   constexpr int PP = E > EP ? E / EP : 1;                // (edge, head) pairs per lane
   static_assert(H <= LPR && E <= LPR, "a group holds its pairs and its ids");
-  extern __shared__ uint4 short_buf[];                   // [2][E][THREADS]
   const int lane = threadIdx.x & 31, t = lane % LPR, gbase = lane - t;
   const int hl = t % H, el = t / H;
-  pol.setup(t);
-  __shared__ float bias_buf[256];
-  stage_bias(pol, bias_buf);
   const int hc = t * Acc::VEC / q.head_dim;              // head of the lane's slice
   const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
   const uint32_t ROWB = p.src_pitch;
   constexpr uint32_t SLOT = THREADS * 16, BUF = E * SLOT;
-  uint32_t buf = (uint32_t)__cvta_generic_to_shared(&short_buf[threadIdx.x]), other = buf + BUF;
-  const int64_t sweep = (int64_t)gridDim.x * (THREADS / LPR);
+  uint32_t buf = (uint32_t)__cvta_generic_to_shared(short_buf + threadIdx.x), other = buf + BUF;
+  const int64_t sweep = (int64_t)blocks * (THREADS / LPR);
 
   struct Row { int64_t j0; int len, most, dest, owner; float sd; };   // most: longest row of the warp's groups (0: no rows left)
   auto load_row = [&](int64_t i0, Row &r) {
@@ -224,7 +221,7 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_SHORT_BLOCKS) gat_short_rows_k
     }
   };
 
-  int64_t i0 = p.row_lo + (int64_t)blockIdx.x * (THREADS / LPR) + (threadIdx.x >> 5) * (32 / LPR);   // warp-uniform
+  int64_t i0 = p.row_lo + (int64_t)block * (THREADS / LPR) + (threadIdx.x >> 5) * (32 / LPR);   // warp-uniform
   Row r0, r1, r2;
   load_row(i0, r0); load_row(i0 + sweep, r1); load_row(i0 + 2 * sweep, r2);
   finish_row(r0);
@@ -291,11 +288,20 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_SHORT_BLOCKS) gat_short_rows_k
   }
   cp_async_wait<0>();
 }
+template <typename T, int LPR, int H>
+__global__ void __launch_bounds__(THREADS, IT_GAT_SHORT_BLOCKS) gat_short_rows_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol) {
+  extern __shared__ uint4 short_buf[];
+  __shared__ float bias_buf[256];
+  pol.setup(threadIdx.x % LPR);
+  stage_bias(pol, bias_buf);
+  gat_short_rows<T, LPR, H>(p, q, pol, blockIdx.x, gridDim.x, short_buf);
+}
 
 // ----------------------------------------------------------------------------- small graphs: every list of a layer in one kernel
 template <typename T, int LPR, int H>
-__global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol, PieceParams pq) {
-  constexpr int SL = 32 / LPR, U = 8, VEC = GatAcc<T>::VEC, NS = GatPolicy<T, 16>::NS;
+__global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol, PieceParams pq, SmallShare sh) {
+  constexpr int SL = 32 / LPR, U = LPR == 8 ? 4 : 8, VEC = GatAcc<T>::VEC, NS = GatPolicy<T, 16>::NS;   // U rows in flight per lane
+  extern __shared__ uint4 short_buf[];
   __shared__ float weights[THREADS / 32][32 * H];
   __shared__ float bias_buf[256];
   it_allow_next();
@@ -304,8 +310,15 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(Stream
   const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
   it_wait_prior();
   stage_bias(pol, bias_buf);
+  if constexpr (LPR <= 16) {
+    if ((int)blockIdx.x < sh.short_blocks) {
+      p.row_lo = sh.short_lo; p.row_hi = sh.short_hi;
+      gat_short_rows<T, LPR, H>(p, q, pol, blockIdx.x, sh.short_blocks, short_buf);
+      return;
+    }
+  }
   GatWarp<T, LPR, H> gw(p, q, lane, (uint32_t)__cvta_generic_to_shared(&weights[threadIdx.x >> 5][0]));
-  small_walk<false, true>(p, lane, [&](const it_row_meta &m, int owner, int32_t idx, float) {
+  small_walk<false, true>(p, sh, lane, [&](const it_row_meta &m, int owner, int32_t idx, float) {
     gw.acc.init(gw.st);
     gw.m = -INFINITY;
     for (int base = 0; base < m.len; base += 32) {
@@ -384,12 +397,16 @@ it_status launch_gat_small(const it_gat_args &a, StreamParams p, const GatPolicy
   const it_graph *g = a.g;
   GatParams q;
   q.scores = pol.scores; q.scores_dst = pol.scores_dst; q.stride = pol.src_stride; q.per_edge = a.per_edge_scores; q.slope = pol.slope; q.head_dim = pol.head_dim;
-  p.row_lo = 0; p.row_hi = g->h_list_offsets[g->n_lists]; p.slices = LPR;
+  p.slices = LPR;
   if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, (size_t)g->n_long * sizeof(int), st));
   const double row_bytes = (double)pol.dim * sizeof(T);
   const double bytes = (double)g->e * (4.0 + 4.0 * H + row_bytes) + (double)g->n * (20.0 + 4.0 * H + row_bytes);
+  const SmallShare sh = small_share(g, LPR <= 16, LPR);
+  const int smem = sh.short_blocks ? 2 * IT_SHORT_EDGES * THREADS * 16 : 0;
+  static std::atomic<uint64_t> configured{0};
+  IT_TRY(allow_dynamic_smem(gat_small_kernel<T, LPR, H>, 2 * IT_SHORT_EDGES * THREADS * 16, configured));
   IT_LAUNCH(IT_K_GAT_SMALL, bytes, 0, st,
-            IT_CUDA_TRY(it_launch_pdl(gat_small_kernel<T, LPR, H>, dim3(small_grid(g)), dim3(THREADS), 0, st, p, q, pol, piece_params(g, a.counters))));
+            IT_CUDA_TRY(it_launch_pdl(gat_small_kernel<T, LPR, H>, dim3(sh.blocks), dim3(THREADS), smem, st, p, q, pol, piece_params(g, a.counters), sh)));
   return IT_OK;
 }
 

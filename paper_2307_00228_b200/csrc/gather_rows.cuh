@@ -15,7 +15,7 @@ struct SagePolicy {
   using Slice = RowSlice<T, SB>;
   static constexpr int VEC = Slice::VEC;
   static constexpr int NS = VEC;
-  static constexpr bool WEIGHTED = WEIGHTED_, HAS_EXTRA = false, NEEDS_OWNER = false;
+  static constexpr bool WEIGHTED = WEIGHTED_, HAS_EXTRA = false, NEEDS_OWNER = false, NULLABLE = false;
   float *__restrict__ partials;
   void *__restrict__ dst;
   const void *__restrict__ self_term;
@@ -112,19 +112,33 @@ SagePolicy<T, SB, RED, WEIGHTED> make_policy(const it_gather_args &a) {
 }
 
 // ----------------------------------------------------------------------------- small graphs: every list of a layer in one kernel
+// The weighted policy for graphs with and without weights (a weight of 1 changes no result).
+template <typename T, int RED>
+struct SmallPolicy : SagePolicy<T, 16, RED, true> {
+  static constexpr bool NULLABLE = true;
+};
+
 template <typename T, int LPR, class Policy>
-__global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(StreamParams p, Policy pol, PieceParams q, const int64_t *__restrict__ owner_indptr,
+__global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(StreamParams p, Policy pol, PieceParams q, SmallShare sh, const int64_t *__restrict__ owner_indptr,
                                                                           const int64_t *__restrict__ shadow_indptr) {
   constexpr int SL = 32 / LPR, U = LPR < 8 ? LPR : 8;   // edge slots; rows in flight per lane (SL * U <= 32)
   constexpr int NS = Policy::NS;
   using Slice = typename Policy::Slice;
+  extern __shared__ uint4 small_stage[];
   it_allow_next();
   const int lane = threadIdx.x & 31, slot = lane / LPR, t = lane % LPR;
   const bool active = t < p.slices;
   pol.setup(t);
   const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
   it_wait_prior();
-  small_walk<true, false>(p, lane, [&](const it_row_meta &m, int, int32_t idx, float w) {
+  if constexpr (LPR == 8 || LPR == 16) {
+    if ((int)blockIdx.x < sh.short_blocks) {
+      p.row_lo = sh.short_lo; p.row_hi = sh.short_hi;
+      short_rows_pipe<T, LPR, Policy, true>(p, pol, blockIdx.x, sh.short_blocks, small_stage);
+      return;
+    }
+  }
+  small_walk<true, false>(p, sh, lane, [&](const it_row_meta &m, int, int32_t idx, float w) {
     float st[NS];
     pol.init(st);
     if (active) pol.begin_row(m.dest, 0);
@@ -192,18 +206,21 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(Str
 template <typename T, int RED>
 it_status launch_small(const it_gather_args &a, StreamParams sp, cudaStream_t st) {
   const it_graph *g = a.g;
-  const auto pol = make_policy<T, 16, RED, true>(a);
+  using Policy = SmallPolicy<T, RED>;
+  Policy pol;
+  static_cast<SagePolicy<T, 16, RED, true> &>(pol) = make_policy<T, 16, RED, true>(a);
   const int slices = a.dim * (int)sizeof(T) / 16;
   const double row_bytes = (double)a.dim * sizeof(T);
   const double bytes = (double)g->e * ((a.per_edge_rows ? 0.0 : 4.0) + (a.use_edge_weights ? 4.0 : 0.0) + row_bytes) +
                        (double)g->n * (16.0 + row_bytes + (a.epi == IT_EPI_ADD_ACT ? row_bytes : 0.0));
-  sp.row_lo = 0; sp.row_hi = g->h_list_offsets[g->n_lists]; sp.slices = slices;
+  sp.slices = slices;
   sp.weights = a.use_edge_weights ? sp.weights : nullptr;
   if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, (size_t)g->n_long * sizeof(int), st));
   auto go = [&]<int LPR>() -> it_status {
+    const SmallShare sh = small_share(g, LPR == 8 || LPR == 16, LPR);
     IT_LAUNCH(IT_K_GATHER_SMALL, bytes, 0, st,
-              IT_CUDA_TRY(it_launch_pdl(gather_small_kernel<T, LPR, decltype(make_policy<T, 16, RED, true>(a))>, dim3(small_grid(g)), dim3(THREADS), 0, st, sp, pol,
-                                        piece_params(g, a.counters), (const int64_t *)g->owner_indptr, (const int64_t *)g->shadow_indptr)));
+              IT_CUDA_TRY(it_launch_pdl(gather_small_kernel<T, LPR, Policy>, dim3(sh.blocks), dim3(THREADS), sh.short_blocks ? SHORT_STAGE_BYTES : 0, st, sp, pol,
+                                        piece_params(g, a.counters), sh, (const int64_t *)g->owner_indptr, (const int64_t *)g->shadow_indptr)));
     return IT_OK;
   };
   if (slices <= 1) return go.template operator()<1>();

@@ -1,6 +1,8 @@
-// One kernel per layer for small graphs: a warp per row of any length (pieces of long vertices, whole vertices, rows without
-// edges), source rows straight into registers, and the pieces of a long vertex folded by the warp that finishes the last of
-// them.  The record of a warp's next-but-one row and the ids of its next row are in flight while a row is reduced.
+// One kernel per layer for small graphs.  Some blocks walk the rows of at most 32 edges, a lane group per row, as the kernel
+// for short rows does (where the row width has one); the others take the remaining rows, a warp per row (pieces of long
+// vertices, whole vertices, rows without edges), source rows straight into registers, and fold the pieces of a long vertex
+// in the warp that finishes the last of them.  The record of a warp's next-but-one row and the ids of its next row are in
+// flight while a row is reduced.
 // What bounds it: the dependent trips record -> ids -> source rows out of the L2 and the launch itself.  A layer of 10k
 // vertices and 100k edges took five launches (a memset, three kernels by row length, empty rows, combine).  SMALL_MEASURED
 //
@@ -38,19 +40,51 @@ __device__ __forceinline__ bool last_piece(const PieceParams &q, int slot, int l
 
 constexpr int SMALL_BLOCKS = 3;   // resident CTAs per SM
 
-// The rows of one warp, from the end of the list (pieces first) in turn.
+// How a launch is shared out: blocks [0, short_blocks) take entries [short_lo, short_hi) of the list, the others the rest.
+struct SmallShare {
+  unsigned blocks;
+  int short_blocks, short_lo, short_hi, total;
+};
+inline SmallShare small_share(const it_graph *g, bool groups, int lpr) {
+  SmallShare s;
+  s.total = (int)g->h_list_offsets[g->n_lists];
+  int64_t short_cost = 0, cost = 0;
+  s.short_lo = s.short_hi = 0;
+  for (int b = 0; b < g->n_lists; ++b) {
+    const int64_t rows = g->h_list_offsets[b + 1] - g->h_list_offsets[b];
+    if (groups && g->list_bounds[b] > 0 && g->list_bounds[b] <= IT_SHORT_BELOW && b != g->n_lists - 1) {
+      if (s.short_hi == s.short_lo) s.short_lo = (int)g->h_list_offsets[b];
+      s.short_hi = (int)g->h_list_offsets[b + 1];
+      short_cost += (rows * 8 + g->h_list_edges[b]) * lpr / 32;   // edge slots, and about eight of them for a row
+    } else {
+      cost += rows * 8 + g->h_list_edges[b];
+    }
+  }
+  const int rows = s.total - (s.short_hi - s.short_lo), most = g->num_sms * SMALL_BLOCKS;
+  const int want_short = (int)((s.short_hi - s.short_lo + THREADS / lpr - 1) / (THREADS / lpr)), want = (rows + THREADS / 32 - 1) / (THREADS / 32);
+  int share = short_cost > 0 ? (int)(most * short_cost / (short_cost + cost)) : 0;
+  if (share < 1 && want_short > 0) share = 1;
+  if (share > most - 1) share = most - 1;
+  s.short_blocks = share < want_short ? share : want_short;
+  const int left = most - s.short_blocks;
+  s.blocks = (unsigned)(s.short_blocks + (want < 1 ? 1 : (want < left ? want : left)));
+  return s;
+}
+
+// The rows of one warp, from the end of the list (pieces first) in turn, without the short rows.
 //   row(m, owner, idx, w): reduce one row; idx / w: ids and weights of its first 32 edges, one per lane
 template <bool WEIGHTED, bool OWNER, class Row>
-__device__ __forceinline__ void small_walk(const StreamParams &p, int lane, Row row) {
-  const int W = (int)gridDim.x * (THREADS / 32), n = (int)p.row_hi;
-  int i = (int)blockIdx.x * (THREADS / 32) + (int)(threadIdx.x >> 5);
+__device__ __forceinline__ void small_walk(const StreamParams &p, const SmallShare &sh, int lane, Row row) {
+  const int W = ((int)gridDim.x - sh.short_blocks) * (THREADS / 32), above = sh.total - sh.short_hi, n = above + sh.short_lo;
+  int i = ((int)blockIdx.x - sh.short_blocks) * (THREADS / 32) + (int)(threadIdx.x >> 5);
   it_row_meta m[3];
   int owner[3];
   auto fetch = [&](int at, it_row_meta &x, int &o) {
     x.j0 = 0; x.len = 0; x.dest = 0; o = 0;
     if (at < n) {
-      x = load_meta(p.meta + (n - 1 - at));
-      if (OWNER) o = __ldcs(p.owner + (n - 1 - at));
+      const int entry = at < above ? sh.total - 1 - at : n - 1 - at;
+      x = load_meta(p.meta + entry);
+      if (OWNER) o = __ldcs(p.owner + entry);
     }
   };
   auto ids = [&](const it_row_meta &x, int32_t &idx, float &w) {
@@ -72,11 +106,6 @@ __device__ __forceinline__ void small_walk(const StreamParams &p, int lane, Row 
     m[0] = m[1]; owner[0] = owner[1]; m[1] = m[2]; owner[1] = owner[2];
     idx[0] = idx[1]; w[0] = w[1];
   }
-}
-
-inline unsigned small_grid(const it_graph *g) {
-  const int64_t rows = g->h_list_offsets[g->n_lists], want = (rows + THREADS / 32 - 1) / (THREADS / 32), most = (int64_t)g->num_sms * SMALL_BLOCKS;
-  return (unsigned)(want < most ? want : most);
 }
 
 inline PieceParams piece_params(const it_graph *g, int *done) {

@@ -382,8 +382,10 @@ __global__ void __launch_bounds__(THREADS, IT_GATHER_MIN_BLOCKS) stream_rows_ker
 #ifndef IT_SHORT_PIPE_WAVES
 #define IT_SHORT_PIPE_WAVES 1    // grid = SMs x resident CTAs x this: every CTA is resident from the start and walks its rows
 #endif
+// block / blocks: which share of the rows p.row_lo .. p.row_hi this block walks; sbuf: SHORT_STAGE_BYTES of shared memory.
+constexpr int SHORT_STAGE_BYTES = IT_SHORT_EDGES * THREADS * 16;
 template <typename T, int LPR, class Policy, bool PAD>
-__global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_rows_pipe_kernel(StreamParams p, Policy pol) {
+__device__ __forceinline__ void short_rows_pipe(const StreamParams &p, Policy &pol, int block, int blocks, uint4 *sbuf) {
   constexpr int NS = Policy::NS;
   constexpr int E = IT_SHORT_EDGES;   // edges per round
   static_assert(LPR >= E, "lanes 0..7 of a group fetch the indices of a round");
@@ -393,9 +395,8 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_ro
   pol.setup(t);
   const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
   const uint32_t ROWB = p.src_pitch;
-  const int64_t sweep = (int64_t)gridDim.x * (THREADS / LPR);
-  __shared__ uint4 sbuf[E][THREADS];
-  const uint32_t my_buf = (uint32_t)__cvta_generic_to_shared(&sbuf[0][threadIdx.x]);
+  const int64_t sweep = (int64_t)blocks * (THREADS / LPR);
+  const uint32_t my_buf = (uint32_t)__cvta_generic_to_shared(sbuf + threadIdx.x);
 
   struct Row { int64_t j0; int len, dest, owner; };
   // the row this lane group takes in the sweep that starts at i0 (len 0: none; rows of these buckets have edges)
@@ -414,11 +415,11 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_ro
     idx = 0; w = 1.f;
     if (t < E && k + t < r.len) {
       idx = p.indices ? __ldcs(p.indices + r.j0 + k + t) : (int32_t)(r.j0 + k + t);
-      if (Policy::WEIGHTED) w = __ldcs(p.weights + r.j0 + k + t);
+      if (Policy::WEIGHTED && (!Policy::NULLABLE || p.weights)) w = __ldcs(p.weights + r.j0 + k + t);
     }
   };
 
-  int64_t i0 = p.row_lo + (int64_t)blockIdx.x * (THREADS / LPR) + (threadIdx.x >> 5) * (32 / LPR);   // warp-uniform
+  int64_t i0 = p.row_lo + (int64_t)block * (THREADS / LPR) + (threadIdx.x >> 5) * (32 / LPR);   // warp-uniform
   Row cur = load_row(i0), nxt = load_row(i0 + sweep);
   int32_t idx_c; float w_c;
   load_idx(cur, 0, idx_c, w_c);
@@ -460,6 +461,11 @@ __global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_ro
     if (len > 0) pol.end_row(st, cur.dest, cur.owner, len);
     cur = nxt; nxt = nn;
   }
+}
+template <typename T, int LPR, class Policy, bool PAD>
+__global__ void __launch_bounds__(THREADS, IT_SHORT_PIPE_BLOCKS) stream_short_rows_pipe_kernel(StreamParams p, Policy pol) {
+  __shared__ uint4 sbuf[SHORT_STAGE_BYTES / 16];
+  short_rows_pipe<T, LPR, Policy, PAD>(p, pol, blockIdx.x, gridDim.x, sbuf);
 }
 
 // Rows of at most E edges (one round each), two rows per lane group in flight: the copies of the group's next row are
