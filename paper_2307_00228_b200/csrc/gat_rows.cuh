@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_SHORT_BLOCKS) gat_short_rows_k
 // ----------------------------------------------------------------------------- small graphs: every list of a layer in one kernel
 template <typename T, int LPR, int H>
 __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol, PieceParams pq, SmallShare sh) {
-  constexpr int SL = 32 / LPR, U = LPR == 8 ? 4 : 8, VEC = GatAcc<T>::VEC, NS = GatPolicy<T, 16>::NS;   // U rows in flight per lane
+  constexpr int SL = 32 / LPR, U = 4, VEC = GatAcc<T>::VEC, NS = GatPolicy<T, 16>::NS;   // U rows in flight per lane
   extern __shared__ uint4 short_buf[];
   __shared__ float weights[THREADS / 32][32 * H];
   __shared__ float bias_buf[256];
@@ -308,7 +308,6 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(Stream
   const int lane = threadIdx.x & 31, slot = lane / LPR, t = lane % LPR;
   pol.setup(t);
   const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
-  it_wait_prior();
   stage_bias(pol, bias_buf);
   if constexpr (LPR <= 16) {
     if ((int)blockIdx.x < sh.short_blocks) {
@@ -318,15 +317,15 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(Stream
     }
   }
   GatWarp<T, LPR, H> gw(p, q, lane, (uint32_t)__cvta_generic_to_shared(&weights[threadIdx.x >> 5][0]));
-  small_walk<false, true>(p, sh, lane, [&](const it_row_meta &m, int owner, int32_t idx, float) {
+  small_walk<false, true>(p, sh, lane, [&](const SmallRow &m, int32_t idx, float) {
     gw.acc.init(gw.st);
     gw.m = -INFINITY;
     for (int base = 0; base < m.len; base += 32) {
       Chunk c;
       c.cnt = m.len - base < 32 ? m.len - base : 32;
       int32_t idx_n = 0;   // the next chunk's ids, in flight while this one's rows are
-      if (base + 32 + lane < m.len) idx_n = p.indices ? __ldg(p.indices + m.j0 + base + 32 + lane) : (int32_t)(m.j0 + base + 32 + lane);
-      c.idx = idx; c.owner = owner; c.j = m.j0 + base;
+      if (base + 32 + lane < m.len) idx_n = p.indices ? __ldg(p.indices + m.j0 + base + 32 + lane) : m.j0 + base + 32 + lane;
+      c.idx = idx; c.owner = m.owner; c.j = m.j0 + base;
       gw.ahead(c);
       uint4 v[U];
       auto load = [&](int k0) {
@@ -365,28 +364,30 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(Stream
     if (slot == 0) pol.end_row(full, m.dest, 0, m.len);
     if (m.dest < 0) {
       int k;
-      if (last_piece(pq, ~m.dest, lane, k) && slot == 0) {   // merge the vertex's pieces in order, a slice per lane
-        const int64_t p0 = __ldg(pq.piece_ptr + k), p1 = __ldg(pq.piece_ptr + k + 1);
+      if (last_piece(pq, ~m.dest, lane, k)) {   // merge the vertex's pieces: every slot a share of them, a slice per lane, then the slots
+        const int p0 = (int)__ldg(pq.piece_ptr + k), p1 = (int)__ldg(pq.piece_ptr + k + 1);
         const int stride = gat_partial_stride(pol.dim, pol.heads);
         pol.init(full);
-        for (int64_t g0 = p0; g0 < p1; g0 += 4) {   // four in flight
-          float x[4][NS];
+        for (int g = p0 + slot; g < p1; g += SL) {
+          const float *row = pol.partials + (int64_t)g * stride;
+          float x[NS];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float *row = pol.partials + (g0 + u < p1 ? g0 + u : g0) * stride;
-#pragma unroll
-            for (int k4 = 0; k4 < VEC; k4 += 4) {
-              const float4 y = __ldcg(reinterpret_cast<const float4 *>(row + pol.col + k4));
-              x[u][k4] = y.x; x[u][k4 + 1] = y.y; x[u][k4 + 2] = y.z; x[u][k4 + 3] = y.w;
-            }
-            x[u][VEC] = __ldcg(row + pol.dim + pol.head);
-            x[u][VEC + 1] = __ldcg(row + pol.dim + pol.heads + pol.head);
+          for (int k4 = 0; k4 < VEC; k4 += 4) {
+            const float4 y = __ldcg(reinterpret_cast<const float4 *>(row + pol.col + k4));
+            x[k4] = y.x; x[k4 + 1] = y.y; x[k4 + 2] = y.z; x[k4 + 3] = y.w;
           }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (g0 + u < p1) pol.merge(full, x[u]);
+          x[VEC] = __ldcg(row + pol.dim + pol.head);
+          x[VEC + 1] = __ldcg(row + pol.dim + pol.heads + pol.head);
+          pol.merge(full, x);
         }
-        pol.end_row(full, __ldg(pq.long_owners + k), 0, 1);
+#pragma unroll
+        for (int o = 16; o >= LPR; o >>= 1) {
+          float x[NS];
+#pragma unroll
+          for (int k4 = 0; k4 < NS; ++k4) x[k4] = __shfl_xor_sync(0xffffffffu, full[k4], o);
+          pol.merge(full, x);
+        }
+        if (slot == 0) pol.end_row(full, __ldg(pq.long_owners + k), 0, 1);
       }
     }
   });
@@ -405,8 +406,10 @@ it_status launch_gat_small(const it_gat_args &a, StreamParams p, const GatPolicy
   const int smem = sh.short_blocks ? 2 * IT_SHORT_EDGES * THREADS * 16 : 0;
   static std::atomic<uint64_t> configured{0};
   IT_TRY(allow_dynamic_smem(gat_small_kernel<T, LPR, H>, 2 * IT_SHORT_EDGES * THREADS * 16, configured));
+  // (Not started early: on SMs split for the dense product's shared memory it finds little L1, which its score and row loads
+  // live on: 30k vertices, two layers 84 us, started early 98.)
   IT_LAUNCH(IT_K_GAT_SMALL, bytes, 0, st,
-            IT_CUDA_TRY(it_launch_pdl(gat_small_kernel<T, LPR, H>, dim3(sh.blocks), dim3(THREADS), smem, st, p, q, pol, piece_params(g, a.counters), sh)));
+            gat_small_kernel<T, LPR, H><<<sh.blocks, THREADS, smem, st>>>(p, q, pol, piece_params(g, a.counters), sh));
   return IT_OK;
 }
 

@@ -121,7 +121,7 @@ struct SmallPolicy : SagePolicy<T, 16, RED, true> {
 template <typename T, int LPR, class Policy>
 __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(StreamParams p, Policy pol, PieceParams q, SmallShare sh, const int64_t *__restrict__ owner_indptr,
                                                                           const int64_t *__restrict__ shadow_indptr) {
-  constexpr int SL = 32 / LPR, U = LPR < 8 ? LPR : 8;   // edge slots; rows in flight per lane (SL * U <= 32)
+  constexpr int SL = 32 / LPR, U = LPR < 4 ? LPR : 4;   // edge slots; rows in flight per lane (SL * U <= 32)
   constexpr int NS = Policy::NS;
   using Slice = typename Policy::Slice;
   extern __shared__ uint4 small_stage[];
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(Str
       return;
     }
   }
-  small_walk<true, false>(p, sh, lane, [&](const it_row_meta &m, int, int32_t idx, float w) {
+  small_walk<true, false>(p, sh, lane, [&](const SmallRow &m, int32_t idx, float w) {
     float st[NS];
     pol.init(st);
     if (active) pol.begin_row(m.dest, 0);
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(Str
       int32_t idx_n = 0;   // the next chunk's ids, in flight while this one's rows are
       float w_n = 1.f;
       if (base + 32 + lane < m.len) {
-        idx_n = p.indices ? __ldg(p.indices + m.j0 + base + 32 + lane) : (int32_t)(m.j0 + base + 32 + lane);
+        idx_n = p.indices ? __ldg(p.indices + m.j0 + base + 32 + lane) : m.j0 + base + 32 + lane;
         if (p.weights) w_n = __ldg(p.weights + m.j0 + base + 32 + lane);
       }
       const int cnt = m.len - base < 32 ? m.len - base : 32;
@@ -167,37 +167,40 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(Str
       }
       idx = idx_n; w = w_n;
     }
+    auto fold = [&]() {
 #pragma unroll
-    for (int o = 16; o >= LPR; o >>= 1) {
-      float other[NS];
+      for (int o = 16; o >= LPR; o >>= 1) {
+        float other[NS];
 #pragma unroll
-      for (int k = 0; k < NS; ++k) other[k] = __shfl_xor_sync(0xffffffffu, st[k], o);
-      pol.merge(st, other);   // only slot 0 is read afterwards, and there st is always the lower slot
-    }
+        for (int k = 0; k < NS; ++k) other[k] = __shfl_xor_sync(0xffffffffu, st[k], o);
+        pol.merge(st, other);   // only slot 0 is read afterwards, and there st is always the lower slot
+      }
+    };
+    fold();
     if (slot == 0 && active) pol.end_row(st, m.dest, 0, m.len);
     if (m.dest < 0) {
       int k;
-      if (last_piece(q, ~m.dest, lane, k) && slot == 0 && active) {   // fold the vertex's pieces in order, a slice per lane
-        const int64_t v = __ldg(q.long_owners + k), p0 = __ldg(q.piece_ptr + k), p1 = __ldg(q.piece_ptr + k + 1);
-        const int64_t deg = __ldg(shadow_indptr + __ldg(owner_indptr + v + 1)) - __ldg(shadow_indptr + __ldg(owner_indptr + v));
-        pol.begin_row((int32_t)v, 0);
+      if (last_piece(q, ~m.dest, lane, k)) {   // fold the vertex's pieces: every slot a share of them, a slice per lane, then the slots
+        const int p0 = (int)__ldg(q.piece_ptr + k), p1 = (int)__ldg(q.piece_ptr + k + 1);
         pol.init(st);
-        for (int64_t g0 = p0; g0 < p1; g0 += 4) {   // four in flight
-          float x[4][NS];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float4 *row = reinterpret_cast<const float4 *>(pol.partials + (g0 + u < p1 ? g0 + u : g0) * pol.dim + pol.col);
+        if (active)
+          for (int g = p0 + slot; g < p1; g += SL) {
+            float x[NS];
+            const float4 *row = reinterpret_cast<const float4 *>(pol.partials + (int64_t)g * pol.dim + pol.col);
 #pragma unroll
             for (int k4 = 0; k4 < NS; k4 += 4) {
               const float4 y = __ldcg(row + k4 / 4);
-              x[u][k4] = y.x; x[u][k4 + 1] = y.y; x[u][k4 + 2] = y.z; x[u][k4 + 3] = y.w;
+              x[k4] = y.x; x[k4 + 1] = y.y; x[k4 + 2] = y.z; x[k4 + 3] = y.w;
             }
+            pol.merge(st, x);
           }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (g0 + u < p1) pol.merge(st, x[u]);
+        fold();
+        if (slot == 0 && active) {
+          const int64_t v = __ldg(q.long_owners + k);
+          const int64_t deg = __ldg(shadow_indptr + __ldg(owner_indptr + v + 1)) - __ldg(shadow_indptr + __ldg(owner_indptr + v));
+          pol.begin_row((int32_t)v, 0);
+          pol.end_row(st, (int32_t)v, 0, deg);
         }
-        pol.end_row(st, (int32_t)v, 0, deg);
       }
     }
   });

@@ -72,38 +72,39 @@ inline SmallShare small_share(const it_graph *g, bool groups, int lpr) {
 }
 
 // The rows of one warp, from the end of the list (pieces first) in turn, without the short rows.
-//   row(m, owner, idx, w): reduce one row; idx / w: ids and weights of its first 32 edges, one per lane
+//   row(m, idx, w): reduce one row; idx / w: ids and weights of its first 32 edges, one per lane
+struct SmallRow { int j0, len, dest, owner; };   // (edges of a small graph are counted with 31 bits)
 template <bool WEIGHTED, bool OWNER, class Row>
 __device__ __forceinline__ void small_walk(const StreamParams &p, const SmallShare &sh, int lane, Row row) {
   const int W = ((int)gridDim.x - sh.short_blocks) * (THREADS / 32), above = sh.total - sh.short_hi, n = above + sh.short_lo;
   int i = ((int)blockIdx.x - sh.short_blocks) * (THREADS / 32) + (int)(threadIdx.x >> 5);
-  it_row_meta m[3];
-  int owner[3];
-  auto fetch = [&](int at, it_row_meta &x, int &o) {
-    x.j0 = 0; x.len = 0; x.dest = 0; o = 0;
+  SmallRow m[3];
+  auto fetch = [&](int at, SmallRow &x) {
+    x = SmallRow{0, 0, 0, 0};
     if (at < n) {
       const int entry = at < above ? sh.total - 1 - at : n - 1 - at;
-      x = load_meta(p.meta + entry);
-      if (OWNER) o = __ldcs(p.owner + entry);
+      const it_row_meta r = load_meta(p.meta + entry);
+      x.j0 = (int)r.j0; x.len = r.len; x.dest = r.dest;
+      if (OWNER) x.owner = __ldcs(p.owner + entry);
     }
   };
-  auto ids = [&](const it_row_meta &x, int32_t &idx, float &w) {
+  auto ids = [&](const SmallRow &x, int32_t &idx, float &w) {
     idx = 0; w = 1.f;
     if (lane < x.len) {
-      idx = p.indices ? __ldg(p.indices + x.j0 + lane) : (int32_t)(x.j0 + lane);
+      idx = p.indices ? __ldg(p.indices + x.j0 + lane) : x.j0 + lane;
       if (WEIGHTED && p.weights) w = __ldg(p.weights + x.j0 + lane);
     }
   };
   int32_t idx[2];
   float w[2];
-  fetch(i, m[0], owner[0]);
-  fetch(i + W, m[1], owner[1]);
+  fetch(i, m[0]);
+  fetch(i + W, m[1]);
   ids(m[0], idx[0], w[0]);
   for (; i < n; i += W) {
-    fetch(i + 2 * W, m[2], owner[2]);
+    fetch(i + 2 * W, m[2]);
     ids(m[1], idx[1], w[1]);
-    row(m[0], owner[0], idx[0], w[0]);
-    m[0] = m[1]; owner[0] = owner[1]; m[1] = m[2]; owner[1] = owner[2];
+    row(m[0], idx[0], w[0]);
+    m[0] = m[1]; m[1] = m[2];
     idx[0] = idx[1]; w[0] = w[1];
   }
 }
