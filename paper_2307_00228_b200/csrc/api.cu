@@ -472,7 +472,7 @@ it_status plan_infer(const it_graph *g, const it_layer_desc *layers, int32_t n_l
 // Between the two passes over a call's layers: everything recorded, in one launch.
 it_status launch_prepared(const it_graph *g, char *ws, const it_layer_desc *first, Prepared &prep, cudaStream_t st) {
   prep.recording = false;
-  int *words = reinterpret_cast<int *>(ws + plan_layer(g, first).off_counters);   // the same place for every layer
+  int *words = it_done_words(reinterpret_cast<int *>(ws + plan_layer(g, first).off_counters));   // the same place for every layer
   const size_t n_words = it_small_graph(g) ? (size_t)g->n_long : 0;
   return it_launch_prep_weights_tc(prep.m.data(), (int)prep.m.size(), words, n_words, st);
 }

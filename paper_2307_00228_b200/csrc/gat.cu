@@ -233,9 +233,8 @@ auto gat_bytes(const it_gat_args &a) {
 }
 
 template <typename T, int SB, int LPR>
-it_status launch_gat_lpr(const it_gat_args &a, StreamParams sp, int64_t bound_lo, int64_t bound_hi, cudaStream_t st) {
-  return launch_buckets<T, SB, LPR, false>(a.g, sp, make_policy<T, SB>(a), gat_bytes(a), IT_K_GAT_FLAT, IT_K_GAT_EMPTY, bound_lo, bound_hi,
-                                           a.counters, st);
+it_status launch_gat_lpr(const it_gat_args &a, StreamParams sp, cudaStream_t st) {
+  return launch_buckets<T, SB, LPR, false>(a.g, sp, make_policy<T, SB>(a), gat_bytes(a), IT_K_GAT_FLAT, IT_K_GAT_EMPTY, a.counters, st);
 }
 
 // f.template operator()<LPR, H>() for the shapes that the batched kernels take
@@ -246,13 +245,16 @@ it_status dispatch_batched(int row_bytes, int heads, F f) {
       case 1: return f.template operator()<LPR, 1>();
       case 2: return f.template operator()<LPR, 2>();
       case 4: return f.template operator()<LPR, 4>();
-      default: return f.template operator()<LPR, 8>();
     }
+    if constexpr (LPR >= 8) return f.template operator()<LPR, 8>();
+    it_set_error("gat: %d heads in a row of %d bytes", heads, row_bytes);   // (not with it_gat_batched())
+    return IT_ERR_UNSUPPORTED;
   };
   switch (row_bytes) {
     case 512: return by_heads.template operator()<32>();
     case 256: return by_heads.template operator()<16>();
-    default: return by_heads.template operator()<8>();
+    case 128: return by_heads.template operator()<8>();
+    default: return by_heads.template operator()<4>();
   }
 }
 
@@ -270,12 +272,12 @@ it_status launch_gat(const it_gat_args &a, StreamParams sp, cudaStream_t st) {
     it_set_error("feature row of %d bytes is not 16, 32, 64, 128, 256 or 512 bytes", row_bytes);
     return IT_ERR_UNSUPPORTED;
   }
-  return dispatch_row_bytes(row_bytes, wide, [&]<int SB, int LPR>(int64_t lo, int64_t hi) {
+  return dispatch_row_bytes(row_bytes, wide && row_bytes >= 128, [&]<int SB, int LPR>() {
     if ((a.head_dim * (int)sizeof(T)) % SB != 0) {
       it_set_error("gat: a %d-byte lane slice would straddle two heads (head_dim %d)", SB, a.head_dim);
       return IT_ERR_UNSUPPORTED;
     }
-    return launch_gat_lpr<T, SB, LPR>(a, sp, lo, hi, st);
+    return launch_gat_lpr<T, SB, LPR>(a, sp, st);
   });
 }
 
@@ -283,7 +285,7 @@ it_status launch_gat(const it_gat_args &a, StreamParams sp, cudaStream_t st) {
 
 bool it_gat_batched(it_dtype dtype, int heads, int head_dim) {
   const int es = it_dtype_size(dtype), row = heads * head_dim * es;
-  return (heads == 1 || heads == 2 || heads == 4 || heads == 8) && (head_dim * es) % 16 == 0 && (row == 128 || row == 256 || row == 512);
+  return (heads == 1 || heads == 2 || heads == 4 || heads == 8) && (head_dim * es) % 16 == 0 && (row == 128 || row == 256 || row == 512 || (row == 64 && heads <= 4));
 }
 
 size_t it_gat_partial_bytes(const it_graph *g, int dim, int heads) {

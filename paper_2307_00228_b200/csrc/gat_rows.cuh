@@ -1,4 +1,4 @@
-// The GAT reduce with the attention weights of many edges computed at once, for rows of 128 to 512 bytes in 16-byte
+// The GAT reduce with the attention weights of many edges computed at once, for rows of 64 to 512 bytes in 16-byte
 // slices (bf16 128 or fp32 64 columns: 256 bytes) and 1, 2, 4 or 8 heads.
 //
 // The running-softmax policy of gat.cu works edge by edge: every lane of a row recomputes the logit and the exponential
@@ -161,8 +161,8 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_k
 }
 
 // ----------------------------------------------------------------------------- short rows: one lane group each
-// Rows of at most a few dozen edges, 128- and 256-byte rows: a group of LPR lanes owns a row and walks it in rounds of up
-// to E = 8 edges; the groups of a warp run in lockstep, a round as long as its longest row.  While the rows of one round are
+// Rows of at most a few dozen edges, up to 256 bytes each: a group of LPR lanes owns a row and walks it in rounds of up
+// to E = 8 edges (4 for 64-byte rows); the groups of a warp run in lockstep, a round as long as its longest row.  While the rows of one round are
 // reduced, the source rows and logit terms of the next round are in flight (two staging buffers in shared memory), the ids
 // of the round after it, and the records of the rows after that.
 #ifndef IT_GAT_SHORT_BLOCKS
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_k
 template <typename T, int LPR, int H>
 __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatParams &q, const GatPolicy<T, 16> &pol, int block, int blocks, uint4 *short_buf) {
   using Acc = GatAcc<T>;
-  constexpr int E = IT_SHORT_EDGES;
+  constexpr int E = LPR < IT_SHORT_EDGES ? LPR : IT_SHORT_EDGES;
   constexpr int EP = LPR / H;                            // edges covered by one pair per lane
   constexpr int PP = E > EP ? E / EP : 1;                // (edge, head) pairs per lane
   static_assert(H <= LPR && E <= LPR, "a group holds its pairs and its ids");
@@ -399,7 +399,7 @@ it_status launch_gat_small(const it_gat_args &a, StreamParams p, const GatPolicy
   GatParams q;
   q.scores = pol.scores; q.scores_dst = pol.scores_dst; q.stride = pol.src_stride; q.per_edge = a.per_edge_scores; q.slope = pol.slope; q.head_dim = pol.head_dim;
   p.slices = LPR;
-  if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, (size_t)g->n_long * sizeof(int), st));
+  if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(it_done_words(a.counters), 0, (size_t)g->n_long * sizeof(int), st));
   const double row_bytes = (double)pol.dim * sizeof(T);
   const double bytes = (double)g->e * (4.0 + 4.0 * H + row_bytes) + (double)g->n * (20.0 + 4.0 * H + row_bytes);
   const SmallShare sh = small_share(g, LPR <= 16, LPR);
@@ -409,7 +409,7 @@ it_status launch_gat_small(const it_gat_args &a, StreamParams p, const GatPolicy
   // (Not started early: on SMs split for the dense product's shared memory it finds little L1, which its score and row loads
   // live on: 30k vertices, two layers 84 us, started early 98.)
   IT_LAUNCH(IT_K_GAT_SMALL, bytes, 0, st,
-            gat_small_kernel<T, LPR, H><<<sh.blocks, THREADS, smem, st>>>(p, q, pol, piece_params(g, a.counters), sh));
+            gat_small_kernel<T, LPR, H><<<sh.blocks, THREADS, smem, st>>>(p, q, pol, piece_params(g, it_done_words(a.counters)), sh));
   return IT_OK;
 }
 

@@ -2,8 +2,8 @@
 // vertex are folded here.
 #include "stream.cuh"
 
-it_status it_launch_gather_rows_f32(const it_gather_args &a, const it_stream::StreamParams &sp, cudaStream_t st);
-it_status it_launch_gather_rows_bf16(const it_gather_args &a, const it_stream::StreamParams &sp, cudaStream_t st);
+it_status it_launch_gather_rows_f32(const it_gather_args &a, const it_stream::StreamParams &sp, bool *folded, cudaStream_t st);
+it_status it_launch_gather_rows_bf16(const it_gather_args &a, const it_stream::StreamParams &sp, bool *folded, cudaStream_t st);
 
 namespace {
 
@@ -203,13 +203,14 @@ it_status it_launch_empty_rows(const it_empty_rows_args &a, int kid, double byte
 // pointers already point at its first column, and the *_ld fields / src_ld carry the full row lengths.
 static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
   const it_graph *g = a.g;
+  bool folded = false;   // the pieces of long vertices, by the kernel that walked them
   StreamParams sp;
   sp.meta = g->list_meta; sp.owner = nullptr; sp.indices = a.per_edge_rows ? nullptr : g->indices; sp.weights = g->edge_weights;
   sp.src = a.src; sp.row_lo = sp.row_hi = 0; sp.dim = a.dim; sp.batch_rows = 1; sp.counter = nullptr; sp.claim = 1; sp.slices = 0;
   sp.src_pitch = (uint32_t)((a.src_ld > 0 ? a.src_ld : a.dim) * it_dtype_size(a.dtype));
-  if (a.dtype == IT_F32) IT_TRY(it_launch_gather_rows_f32(a, sp, st));
-  else IT_TRY(it_launch_gather_rows_bf16(a, sp, st));
-  if (g->n_long > 0 && !it_small_graph(g)) {
+  if (a.dtype == IT_F32) IT_TRY(it_launch_gather_rows_f32(a, sp, &folded, st));
+  else IT_TRY(it_launch_gather_rows_bf16(a, sp, &folded, st));
+  if (g->n_long > 0 && !folded) {
     CombineParams c;
     c.long_owners = g->long_owners; c.piece_ptr = g->piece_ptr; c.owner_indptr = g->owner_indptr; c.shadow_indptr = g->shadow_indptr;
     c.partials = a.partials; c.dst = a.dst; c.self_term = a.self_term; c.bias = a.bias; c.n_long = g->n_long;
@@ -225,8 +226,8 @@ static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
   return IT_OK;
 }
 
-// Rows of any multiple of 16 bytes: the kernels take rows of 16, 32, 64 and 80 to 512 bytes, so a wider row (or one of 48
-// bytes, unless the graph is small) is cut into column chunks, largest first, and each chunk is gathered on its own, reading and writing
+// Rows of any multiple of 16 bytes: the kernels take rows of up to 512 bytes, so a wider row is cut into column chunks and
+// each chunk is gathered on its own, reading and writing
 // its columns in place.  The aggregate is entry by entry, so the chunks are independent; each pass re-reads
 // the edge indices (4 bytes against a chunk of up to 512 per edge).
 it_status it_launch_gather(const it_gather_args &a, cudaStream_t st) {
@@ -241,10 +242,8 @@ it_status it_launch_gather(const it_gather_args &a, cudaStream_t st) {
   const int full = a.dim;
   int c0 = 0;   // first column of the chunk
   while (c0 < full) {
-    // what is left as one chunk where a kernel takes it: up to 512 bytes, and from 80 bytes on any multiple of 16 (the
-    // lanes past the row idle); 48 bytes as 32 + 16
     const int left = (full - c0) * es;
-    const int bytes = left >= 512 ? 512 : (left == 48 && !it_small_graph(g) ? 32 : left);
+    const int bytes = left >= 512 ? 512 : left;
     it_gather_args c = a;
     c.dim = bytes / es;
     c.src = (const char *)a.src + (size_t)c0 * es;

@@ -218,12 +218,12 @@ it_status launch_small(const it_gather_args &a, StreamParams sp, cudaStream_t st
                        (double)g->n * (16.0 + row_bytes + (a.epi == IT_EPI_ADD_ACT ? row_bytes : 0.0));
   sp.slices = slices;
   sp.weights = a.use_edge_weights ? sp.weights : nullptr;
-  if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, (size_t)g->n_long * sizeof(int), st));
+  if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(it_done_words(a.counters), 0, (size_t)g->n_long * sizeof(int), st));
   auto go = [&]<int LPR>() -> it_status {
     const SmallShare sh = small_share(g, LPR == 8 || LPR == 16, LPR);
     IT_LAUNCH(IT_K_GATHER_SMALL, bytes, 0, st,
               IT_CUDA_TRY(it_launch_pdl(gather_small_kernel<T, LPR, Policy>, dim3(sh.blocks), dim3(THREADS), sh.short_blocks ? SHORT_STAGE_BYTES : 0, st, sp, pol,
-                                        piece_params(g, a.counters), sh, (const int64_t *)g->owner_indptr, (const int64_t *)g->shadow_indptr)));
+                                        piece_params(g, it_done_words(a.counters)), sh, (const int64_t *)g->owner_indptr, (const int64_t *)g->shadow_indptr)));
     return IT_OK;
   };
   if (slices <= 1) return go.template operator()<1>();
@@ -236,7 +236,7 @@ it_status launch_small(const it_gather_args &a, StreamParams sp, cudaStream_t st
 
 // ----------------------------------------------------------------------------- dispatch
 template <typename T, int SB, int LPR, int RED, bool WEIGHTED>
-it_status launch_policy(const it_gather_args &a, StreamParams sp, int64_t bound_lo, int64_t bound_hi, cudaStream_t st) {
+it_status launch_policy(const it_gather_args &a, StreamParams sp, cudaStream_t st) {
   const auto pol = make_policy<T, SB, RED, WEIGHTED>(a);
   const it_graph *g = a.g;
   // algorithmic bytes: per edge the index, the optional weight and one source row; per row its
@@ -247,7 +247,7 @@ it_status launch_policy(const it_gather_args &a, StreamParams sp, int64_t bound_
            (double)rows * (16.0 + row_bytes + (a.epi == IT_EPI_ADD_ACT ? row_bytes : 0.0));
   };
   auto launch = [&]<bool PAD>() {
-    return launch_buckets<T, SB, LPR, PAD>(g, sp, pol, bytes_of, IT_K_GATHER_FLAT, IT_K_GATHER_EMPTY, bound_lo, bound_hi, a.counters, st);
+    return launch_buckets<T, SB, LPR, PAD>(g, sp, pol, bytes_of, IT_K_GATHER_FLAT, IT_K_GATHER_EMPTY, a.counters, st);
   };
   if constexpr (SB == 16) {
     if (a.dim * (int)sizeof(T) != SB * LPR) return launch.template operator()<true>();
@@ -256,17 +256,21 @@ it_status launch_policy(const it_gather_args &a, StreamParams sp, int64_t bound_
 }
 
 template <typename T>
-it_status launch_lpr(const it_gather_args &a, StreamParams sp, cudaStream_t st) {
-  if (it_small_graph(a.g)) {
+it_status launch_lpr(const it_gather_args &a, StreamParams sp, bool *folded, cudaStream_t st) {
+  // (rows of 80 to 128 bytes cost the one kernel more than the kernels by list from about a million edges on: 60k vertices, 1M
+  // edges, two layers 130 against 137 us, 130k vertices, 1.3M edges 191 against 165)
+  const int row_bytes = a.dim * (int)sizeof(T);
+  if (it_small_graph(a.g) && (row_bytes <= 64 || row_bytes > 128 || a.g->e + 6 * a.g->n <= 1400000)) {
+    *folded = true;
     if (a.op == IT_GATHER_MAX) return launch_small<T, RED_MAX>(a, sp, st);
     if (a.op == IT_GATHER_MIN) return launch_small<T, RED_MIN>(a, sp, st);
     return launch_small<T, RED_SUM>(a, sp, st);
   }
   const bool w = a.use_edge_weights != 0;
-  return dispatch_row_bytes(a.dim * (int)sizeof(T), true, [&]<int SB, int LPR>(int64_t lo, int64_t hi) {
-    if (a.op == IT_GATHER_MAX) return w ? launch_policy<T, SB, LPR, RED_MAX, true>(a, sp, lo, hi, st) : launch_policy<T, SB, LPR, RED_MAX, false>(a, sp, lo, hi, st);
-    if (a.op == IT_GATHER_MIN) return w ? launch_policy<T, SB, LPR, RED_MIN, true>(a, sp, lo, hi, st) : launch_policy<T, SB, LPR, RED_MIN, false>(a, sp, lo, hi, st);
-    return w ? launch_policy<T, SB, LPR, RED_SUM, true>(a, sp, lo, hi, st) : launch_policy<T, SB, LPR, RED_SUM, false>(a, sp, lo, hi, st);
+  return dispatch_row_bytes(row_bytes, true, [&]<int SB, int LPR>() {
+    if (a.op == IT_GATHER_MAX) return w ? launch_policy<T, SB, LPR, RED_MAX, true>(a, sp, st) : launch_policy<T, SB, LPR, RED_MAX, false>(a, sp, st);
+    if (a.op == IT_GATHER_MIN) return w ? launch_policy<T, SB, LPR, RED_MIN, true>(a, sp, st) : launch_policy<T, SB, LPR, RED_MIN, false>(a, sp, st);
+    return w ? launch_policy<T, SB, LPR, RED_SUM, true>(a, sp, st) : launch_policy<T, SB, LPR, RED_SUM, false>(a, sp, st);
   });
 }
 

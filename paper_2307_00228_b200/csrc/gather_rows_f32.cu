@@ -1,3 +1,3 @@
 #include "gather_rows.cuh"
 
-it_status it_launch_gather_rows_f32(const it_gather_args &a, const it_stream::StreamParams &sp, cudaStream_t st) { return launch_lpr<float>(a, sp, st); }
+it_status it_launch_gather_rows_f32(const it_gather_args &a, const it_stream::StreamParams &sp, bool *folded, cudaStream_t st) { return launch_lpr<float>(a, sp, folded, st); }

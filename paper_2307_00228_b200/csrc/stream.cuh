@@ -584,13 +584,11 @@ it_status allow_dynamic_smem(Kernel kernel, int smem, std::atomic<uint64_t> &don
 // ----------------------------------------------------------------------------- bucket dispatch
 // Longest rows first so that the tail of the launch sequence is made of short rows.
 // bytes_of(bucket, rows) gives the algorithmic bytes of a launch; kid_* the instrumentation ids.
-// Only the buckets whose bound lies in (bound_lo, bound_hi] are launched: callers may give long and short
-// rows different slice widths.
 // `counters`: IT_MAX_BUCKETS device words of scratch (or NULL): the ring kernel of bucket b hands out its batches from
 // word b, which is zeroed here, in stream order, before the launches.
 template <typename T, int SB, int LPR, bool PAD, class Policy, class BytesF>
 it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, BytesF bytes_of, int kid_rows, int kid_empty,
-                          int64_t bound_lo, int64_t bound_hi, int *counters, cudaStream_t st) {
+                          int *counters, cudaStream_t st) {
   constexpr bool RING = SB * LPR >= 128;   // rows of 128 bytes and more are staged through shared memory
   if (RING && counters) IT_CUDA_TRY(cudaMemsetAsync(counters, 0, (IT_MAX_BUCKETS + 1) * sizeof(int), st));
   p.counter = nullptr;
@@ -598,7 +596,7 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
   p.slices = p.dim * (int)sizeof(T) / SB;
   for (int b = g->n_lists - 1; b >= 0; --b) {
     const int64_t lo = g->h_list_offsets[b], hi = g->h_list_offsets[b + 1];
-    if (hi <= lo || g->list_bounds[b] <= bound_lo || g->list_bounds[b] > bound_hi) continue;
+    if (hi <= lo) continue;
     p.row_lo = lo; p.row_hi = hi;
     const int64_t bound = g->list_bounds[b];
     const int64_t rows = hi - lo;
@@ -692,29 +690,24 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
   return IT_OK;
 }
 
-// Pick the slice width and group size for a row of `row_bytes` bytes and call
-// f.template operator()<SB, LPR>(bound_lo, bound_hi) for the buckets that take them.  Rows of 80 bytes and more that are
-// no power of two take the lane group of the next power of two with its last lanes idle.  One pass over the edges with
-// whole sectors beats one pass per power-of-two piece even at 25 of 32 lanes: a GCN of widths 100-128-128-48 on 15M
-// edges, whose 400-byte fp32 rows were 256 + 128 + 16, takes 2.98 ms instead of 4.24 (the 16-byte pieces alone moved a
-// 32-byte sector each and an edge index).
-// Rows of 128 and 256 bytes use 16-byte slices unless `wide` is false (a slice would straddle two attention heads).
+// Pick the slice width and group size for a row of `row_bytes` bytes (16 to 512) and call f.template operator()<SB, LPR>().
+// Rows that are no power of two, and those of less than 128 bytes, take the lane group of the next width with its last lanes
+// idle.  One pass over the edges with whole sectors beats one pass per power-of-two piece even at 25 of 32 lanes: a GCN of
+// widths 100-128-128-48 on 15M edges, whose 400-byte fp32 rows were 256 + 128 + 16, takes 2.98 ms instead of 4.24 (the
+// 16-byte pieces alone moved a 32-byte sector each and an edge index).  Rows of 16 to 64 bytes in lane groups of their own
+// width, staged in registers, kept too little in flight: 5M vertices, 60M edges, 64-byte
+// rows 2.90 -> 0.98 ms, 32-byte rows 2.45 -> 1.01; 64-byte GAT rows 4.86 -> 1.73.
+// `wide`: 16-byte slices do not straddle two attention heads; else slices of a 32nd of the row.
 template <class F>
 it_status dispatch_row_bytes(int row_bytes, bool wide, F f) {
-  constexpr int64_t ALL = INT64_MAX;
-  if (row_bytes > 256 && row_bytes <= 512) return f.template operator()<16, 32>(-1, ALL);
-  if (row_bytes > 128 && row_bytes <= 256) {
-    if (!wide) return f.template operator()<8, 32>(-1, ALL);
-    return f.template operator()<16, 16>(-1, ALL);
-  }
-  if (row_bytes > 64 && row_bytes <= 128) {
-    if (!wide) return f.template operator()<4, 32>(-1, ALL);
-    return f.template operator()<16, 8>(-1, ALL);
-  }
+  if (row_bytes > 256) return f.template operator()<16, 32>();
+  if (row_bytes > 128) return wide ? f.template operator()<16, 16>() : f.template operator()<8, 32>();
+  if (wide) return f.template operator()<16, 8>();
   switch (row_bytes) {
-    case 64: return f.template operator()<4, 16>(-1, ALL);
-    case 32: return f.template operator()<4, 8>(-1, ALL);
-    case 16: return f.template operator()<4, 4>(-1, ALL);
+    case 128: return f.template operator()<4, 32>();
+    case 64: return f.template operator()<4, 16>();
+    case 32: return f.template operator()<4, 8>();
+    case 16: return f.template operator()<4, 4>();
   }
   it_set_error("feature row of %d bytes has no kernel", row_bytes);
   return IT_ERR_UNSUPPORTED;

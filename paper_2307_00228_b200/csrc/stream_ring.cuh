@@ -58,7 +58,7 @@ struct RingGeom {
   static constexpr int GE = R * SL;                          // edges per stage
   static constexpr int S = IT_RING_STAGES;
   static constexpr int AHEAD = (S - 1) * GE;                 // the stage being filled is this many edges ahead of the one reduced
-  static_assert(GE <= 16 && 32 % GE == 0 && AHEAD <= 32, "an index chunk of 32 edges is a whole number of stages and the fill reaches at most into the next chunk");
+  static_assert(GE <= 32 && 32 % GE == 0 && AHEAD <= 32, "an index chunk of 32 edges is a whole number of stages and the fill reaches at most into the next chunk");
 };
 template <int SB, bool HAS_EXTRA> constexpr int ring_bytes_per_warp() {
   return IT_RING_STAGES * IT_RING_STAGE_ROWS * (512 + (HAS_EXTRA ? (16 / SB) * 128 : 0));
@@ -127,6 +127,7 @@ __device__ __forceinline__ void ring_stream(const RingWarp<T, SB, LPR, Policy, P
   using G = RingGeom<SB, LPR>;
   using Raw = typename SliceRaw<SB>::type;
   constexpr int SL = G::SL, GE = G::GE, R = G::R, S = G::S, AHEAD = G::AHEAD, GB = G::GB;
+  static_assert(GE <= 16, "the ends of rows inside a stage are bits of a mask");
   const int slot = rw.slot;
 
   // reduce the edges [k0, k0 + n) of the current chunk out of the stage at (sr, sx)

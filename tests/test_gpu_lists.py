@@ -1,0 +1,57 @@
+"""Graphs beyond the line of the one-kernel path: the kernels by row length (very short, short, one warp per row, pieces of long
+vertices, rows without edges) on more than 2^17 vertices, against the oracle; and both sides of that line against each other."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import check_against_oracle, make_gat_layer, make_plain_layer, make_sage_layer, run_device, small_workload
+from paper_2307_00228_b200 import binding as B
+from paper_2307_00228_b200 import host
+
+pytestmark = pytest.mark.gpu
+
+N = (1 << 17) + 77
+HUBS = (20000, 4097, 2100, 1025, 1024, 700, 257, 256, 65, 64, 63, 33, 32, 31, 9, 8)
+
+
+@pytest.mark.parametrize("dtype,fi", [("f32", 4), ("f32", 16), ("f32", 32), ("f32", 60), ("f32", 64), ("f32", 100), ("f32", 132), ("bf16", 8), ("bf16", 32),
+                                      ("bf16", 64), ("bf16", 120), ("bf16", 128), ("bf16", 264)])
+@pytest.mark.parametrize("op,max_deg", [("mean", 5), ("max", 14)])   # rows of at most four edges on average, and longer ones
+def test_pooling(dtype, fi, op, max_deg):
+    layer = make_sage_layer(21, op, "relu", fi, 16, dtype, weights=op == "max", allow_reorder=False)
+    w = small_workload(22, N, max_deg, dtype, [layer], hubs=HUBS, weights=op == "max", threshold=4096)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(dtype, fi, op), exact=False)
+
+
+@pytest.mark.parametrize("dtype,heads,hd", [("f32", 4, 4), ("f32", 4, 16), ("f32", 2, 64), ("bf16", 2, 16), ("bf16", 8, 8), ("bf16", 4, 32), ("f32", 1, 8)])
+def test_gat(dtype, heads, hd):
+    layer = make_gat_layer(23, "elu", 32, heads, hd, dtype)
+    w = small_workload(24, N, 9, dtype, [layer], hubs=HUBS, threshold=4096, p_zero=0.4)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(dtype, heads, hd), exact=False)
+
+
+def test_self_term_and_bias_of_rows_without_edges():
+    for layer in (make_sage_layer(25, "mean", "elu", 64, 32, "bf16"), make_plain_layer(26, "gcn", "elu", 64, 32, "bf16")):
+        w = small_workload(27, N, 4, "bf16", [layer], hubs=HUBS[:6], p_zero=0.9)
+        got, _ = run_device(w)
+        check_against_oracle(w, got, label=layer.op, exact=False)
+
+
+@pytest.mark.parametrize("dtype,dims,kind", [("f32", (64, 64), "mean"), ("bf16", (128, 128), "gat"), ("f32", (16, 48), "max")])
+def test_both_sides_of_the_small_graph_line(dtype, dims, kind):
+    """The same rows in a graph of 2^17 vertices (one kernel per layer) and in one of more (kernels by list): sums may differ by
+    the order of at most a few hundred additions, 2^-24 each, or one rounding of a stored bf16 result (2^-8)."""
+    layer = make_gat_layer(28, "none", dims[0], 4, dims[1] // 4, dtype) if kind == "gat" else make_sage_layer(28, kind, "none", *dims, dtype)
+    w = small_workload(29, 1 << 17, 6, dtype, [layer], hubs=HUBS[1:])
+    d = host.upload(w)
+    small = d.infer().float()
+    extra = np.concatenate([w.indptr, np.full(500, w.indptr[-1])])   # 500 more vertices without edges
+    g = B.it_graph_create(torch.from_numpy(extra).cuda(), torch.from_numpy(w.indices).cuda())
+    x = torch.cat([d.x, torch.zeros((500, dims[0]), dtype=d.x.dtype, device="cuda")])
+    out = torch.empty((x.shape[0], dims[1]), dtype=x.dtype, device="cuda")
+    ws = torch.empty(B.it_workspace_bytes(g, d.layers), dtype=torch.uint8, device="cuda")
+    big = B.it_infer(g, d.layers, x, out, ws)[: w.n].float()
+    scale = small.abs().mean()
+    assert float((big - small).abs().max()) <= (2.0 ** -24 * 4096 if dtype == "f32" else 2.0 ** -6) * float(torch.maximum(small.abs().max(), scale))
