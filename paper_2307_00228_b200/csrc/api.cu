@@ -84,6 +84,7 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
   LayerWs w;
   const size_t n = (size_t)g->n, s = (size_t)it_dtype_size(L->feat_dtype);
   const size_t fi = (size_t)L->in_dim, fo = (size_t)L->out_dim, fe = (size_t)L->edge_dim, fm = (size_t)L->msg_dim;
+  const size_t fop = fo + 256;   // ... and its columns: each output to a multiple of 16, all to whole splits (at most 16 of at most 16 more)
   const size_t kpad = 128;   // the tensor-core path pads the K of each operand to whole k-blocks (at most 63 + 63 rows)
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += it_align_up(bytes); return o; };
@@ -92,7 +93,7 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
   w.off_counters = take(it_gather_words(g) * sizeof(int));
   switch (w.plan) {
     case PLAN_GAT:
-      w.off_B = take((fi + kpad) * (fo + 2 * (size_t)L->heads) * 8);
+      w.off_B = take((fi + kpad) * (fop + 2 * (size_t)L->heads) * 8);
       w.off_partials = take(it_gat_partial_bytes(g, L->out_dim, L->heads));
       w.off_a = take(n * 2 * (size_t)L->heads * 4);  // scores
       w.off_b = take(n * fo * s);                    // Z
@@ -104,38 +105,38 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
                             : (size_t)g->n_src * (size_t)L->heads * 4);
       break;
     case PLAN_DENSE:
-      w.off_B = take((fi + kpad) * fo * 8);
+      w.off_B = take((fi + kpad) * fop * 8);
       w.off_partials = w.off_a = w.off_b = off;
       break;
     case PLAN_GCN_REORDER:
-      w.off_B = take((fi + fe + kpad) * fo * 8);
+      w.off_B = take((fi + fe + kpad) * fop * 8);
       w.off_partials = take((size_t)g->n_partial_rows * fo * 4);
       w.off_a = off;
       w.off_b = take(n * fo * s);  // Z
       break;
     case PLAN_GCN:
-      w.off_B = take((fi + fe + kpad) * fo * 8);
+      w.off_B = take((fi + fe + kpad) * fop * 8);
       w.off_partials = take((size_t)g->n_partial_rows * (fi > fe ? fi : fe) * 4);
       w.off_a = take(n * (fi + fe) * s);  // A = [sum_e w_e h_u | sum_e e_vu]
       w.off_b = off;
       break;
     case PLAN_SAGE_REORDER:
-      w.off_B = take((fi + kpad) * 2 * fo * 8);
+      w.off_B = take((fi + kpad) * 2 * fop * 8);
       w.off_partials = take((size_t)g->n_partial_rows * fo * 4);
       w.off_a = take(n * fo * s);  // S (the self term, stored like the rows)
       w.off_b = take(n * fo * s);  // Z
       break;
     case PLAN_SAGE:
-      w.off_B = take((2 * fi + fe + kpad) * fo * 8);
+      w.off_B = take((2 * fi + fe + kpad) * fop * 8);
       w.off_partials = take((size_t)g->n_partial_rows * (fi > fe ? fi : fe) * 4);
       w.off_a = take(n * (fi + fe) * s);  // A = [aggregate of w_e h_u | aggregate of e_vu]
       w.off_b = off;
       break;
     case PLAN_MSG: {
       // the largest of the three weight matrices prepared in turn: W_edge[:in] (in x msg), W_edge[in:] (edge x msg), W ((in + msg) x out)
-      size_t wb = (fi + kpad) * fm;
-      if ((fe + kpad) * fm > wb) wb = (fe + kpad) * fm;
-      if ((fi + fm + 2 * kpad) * fo > wb) wb = (fi + fm + 2 * kpad) * fo;
+      size_t wb = (fi + kpad) * (fm + 256);
+      if ((fe + kpad) * (fm + 256) > wb) wb = (fe + kpad) * (fm + 256);
+      if ((fi + fm + 2 * kpad) * fop > wb) wb = (fi + fm + 2 * kpad) * fop;
       w.off_B = take(wb * 8);
       w.off_partials = take((size_t)g->n_partial_rows * fm * 4);
       w.off_a = take(n * fm * s);                            // A: aggregate of the messages
@@ -189,7 +190,9 @@ it_status run_apply(const StageCtx &c, const it_layer_desc *L, it_prep_kind kind
   const bool want_scores = kind == IT_PREP_GAT;
   const int heads = L->heads > 0 ? L->heads : 1, hd = L->out_dim / heads;
   if (it_tc_supported(ga, heads, hd, want_scores)) {
-    it_prep_tc p = it_prep_tc_of(kind, L, ga.n0 + ga.n1, ga.K1, ga.X2 ? ga.K2 : 0, c.B);
+    it_tc_cols cols;
+    it_tc_columns(ga, hd, want_scores, &cols);
+    it_prep_tc p = it_prep_tc_of(kind, L, cols.NB, cols.n0p, ga.K1, ga.X2 ? ga.K2 : 0, c.B);
     void *B = c.prep ? c.prep->place(p) : nullptr;
     if (c.recording()) return IT_OK;
     if (!B) {
@@ -436,9 +439,9 @@ struct InferWs { size_t layer_bytes, buf_bytes, off_buf0, off_buf1, off_prep, pr
 
 // Room for the prepared weights of a layer's products (each at most 8 bytes per entry, K padded to whole k-blocks).
 size_t prep_bytes_of(const it_layer_desc *L) {
-  const size_t fi = (size_t)L->in_dim, fo = (size_t)L->out_dim, fe = (size_t)L->edge_dim, fm = (size_t)L->msg_dim, kpad = 128;
+  const size_t fi = (size_t)L->in_dim, fo = (size_t)L->out_dim + 256, fe = (size_t)L->edge_dim, fm = (size_t)L->msg_dim, kpad = 128;
   if (L->op == IT_GATHER_GAT || L->op == IT_GATHER_NONE) return it_align_up((fi + kpad) * fo * 8);
-  if (fm > 0) return it_align_up((fi + kpad) * fm * 8) + it_align_up((fe + kpad) * fm * 8) + it_align_up((fi + fm + 2 * kpad) * fo * 8);
+  if (fm > 0) return it_align_up((fi + kpad) * (fm + 256) * 8) + it_align_up((fe + kpad) * (fm + 256) * 8) + it_align_up((fi + fm + 2 * kpad) * fo * 8);
   return it_align_up((2 * fi + fe + 2 * kpad) * 2 * fo * 8);
 }
 
@@ -514,7 +517,7 @@ it_status infer_layers(const it_graph *g, const it_layer_desc *layers, int32_t n
       IT_TRY(stage_ctx(g, Bn, ws, w.layer_bytes, st, &cb, &prep));
       void *agg = agg_dim_of(A) > 0 ? (void *)(ws + ca.w.off_a) : nullptr;
       if (agg) IT_TRY(stage_gather(ca, cur, nullptr, nullptr, false, agg));
-      const it_prep_tc pa = it_prep_tc_of(f.kind_a, A, f.ga.N1, f.ga.K1, f.ga.K2, nullptr), pb = it_prep_tc_of(f.kind_b, Bn, f.nb_b, f.ga.N1, 0, nullptr);
+      const it_prep_tc pa = it_prep_tc_of(f.kind_a, A, f.ga.N1, 0, f.ga.K1, f.ga.K2, nullptr), pb = it_prep_tc_of(f.kind_b, Bn, f.nb_b, f.ga.n0, f.ga.N1, 0, nullptr);
       void *B1 = prep.place(pa), *B2 = prep.place(pb);
       IT_REQUIRE(B1 && B2, IT_ERR_WORKSPACE, "no room for the prepared weights");
       if (!prep.recording) {

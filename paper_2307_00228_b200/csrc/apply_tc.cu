@@ -206,8 +206,8 @@ struct TcParams {
   int stages;
   int tstages;                    // fp32 mode: split A k-blocks in flight in TMEM
   // epilogue routing (columns are global column ids)
-  int n0; void *out0; int out0_bf16; const float *bias0; int act0;
-  int n1; void *out1; int out1_bf16;
+  int n0, n0_real; void *out0; int out0_bf16; const float *bias0; int act0;   // n0, n1: with their padding; *_real: what is stored
+  int n1, n1_real; void *out1; int out1_bf16;
   float *scores; const float *att_src; const float *att_dst; int heads, head_dim;  // GAT: scores [M, 2*heads]
   int *status;                    // set to 1 if a bounded wait gave up
   int tma_store;                  // 1: the epilogue stages each output tile in shared memory and writes it with TMA stores
@@ -280,7 +280,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
   it_wait_prior();   // everything above is this CTA's own set-up
   for (int c = threadIdx.x; c < p.nbc; c += blockDim.x) {
     const int gc = (blockIdx.x % p.n_splits) * p.nbc + c;
-    bias_s[c] = (p.bias0 && gc < p.n0) ? p.bias0[gc] : 0.f;
+    bias_s[c] = (p.bias0 && gc < p.n0_real) ? p.bias0[gc] : 0.f;
     if (p.scores) {
       att_s[c] = p.att_src[gc];
       att_s[p.nbc + c] = p.att_dst[gc];
@@ -394,14 +394,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       // ---- staged epilogue: every warp converts its 16-column groups and drops them, 128-byte-swizzled, into the
       // panels of the staging tile; one thread then writes each panel with a TMA store (whole 128-byte lines, and
       // per lane only: TMEM load, bias, activation, pack, shared-memory store).  The output columns of this CTA
-      // are a run of out0 columns [lo0, hi0) and a run of out1 columns; each run is a whole number of panels.
+      // are a run of out0 columns [lo0, hi0) and a run of out1 columns; each run is a whole number of panels or ends its output.
       const int s0 = p.out0_bf16 ? 2 : 4, s1 = p.out1_bf16 ? 2 : 4;
       const int lo0 = col_base < p.n0 ? col_base : p.n0;
       const int hi0 = (col_base + p.nbc) < p.n0 ? (col_base + p.nbc) : p.n0;
       const int lo1 = col_base > p.n0 ? col_base : p.n0;
       const int hi1 = (col_base + p.nbc) < n01 ? (col_base + p.nbc) : n01;
-      const int pan0 = hi0 > lo0 ? ((hi0 - lo0) * s0) / 128 : 0;
-      const int pan1 = hi1 > lo1 ? ((hi1 - lo1) * s1) / 128 : 0;
+      const int pan0 = hi0 > lo0 ? ((hi0 - lo0) * s0 + 127) / 128 : 0;   // a last panel past the output's width is clipped by the copy
+      const int pan1 = hi1 > lo1 ? ((hi1 - lo1) * s1 + 127) / 128 : 0;
       // With two groups, group g takes the tiles that land in accumulator g, so that the epilogues of two tiles run
       // side by side (one tile's epilogue is a chain of latencies: barrier, TMEM loads, shared-memory stores, fence).
       const int G = p.epi_groups, wpg = TC_EPI_WARPS / G;   // groups, warps per group
@@ -588,7 +588,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
               }
             }
             if (gc >= n01) continue;
-            void *dst; int bf16; int ld; int lc;
+            void *dst; int bf16; int ld; int lc;   // (ld - lc < 16: the last columns of the group are padding)
             if (gc < p.n0) {
               const float4 *bs = reinterpret_cast<const float4 *>(bias_s + c);
 #pragma unroll
@@ -603,9 +603,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
 #pragma unroll
                 for (int i = 0; i < 16; ++i) v[i] = it_elu(v[i]);
               }
-              dst = p.out0; bf16 = p.out0_bf16; ld = p.n0; lc = gc;
+              dst = p.out0; bf16 = p.out0_bf16; ld = p.n0_real; lc = gc;
             } else {
-              dst = p.out1; bf16 = p.out1_bf16; ld = p.n1; lc = gc - p.n0;
+              dst = p.out1; bf16 = p.out1_bf16; ld = p.n1_real; lc = gc - p.n0;
             }
             // A lane pair (rows m_even, m_odd) swaps halves so that every store instruction writes whole
             // 32-byte sectors: the even lane takes the low 16 bytes of each 32-byte piece, the odd lane the high.
@@ -624,8 +624,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
               __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(dst) + lc + (odd ? 8 : 0);
               const uint4 first = odd ? make_uint4(got[0], got[1], got[2], got[3]) : make_uint4(w[0], w[1], w[2], w[3]);
               const uint4 second = odd ? make_uint4(w[4], w[5], w[6], w[7]) : make_uint4(got[0], got[1], got[2], got[3]);
-              if (m_even < p.M) *reinterpret_cast<uint4 *>(o + m_even * ld) = first;
-              if (m_odd < p.M) *reinterpret_cast<uint4 *>(o + m_odd * ld) = second;
+              const bool in = lc + (odd ? 8 : 0) < ld;
+              if (m_even < p.M && in) *reinterpret_cast<uint4 *>(o + m_even * ld) = first;
+              if (m_odd < p.M && in) *reinterpret_cast<uint4 *>(o + m_odd * ld) = second;
             } else {
               float got[8];
 #pragma unroll
@@ -1053,11 +1054,12 @@ __global__ void __launch_bounds__(256) prep_weights_tc_kernel(const __grid_const
     // padded position -> row of the unpadded product (or none)
     const bool second = kp >= p.K1p;
     const int kin = second ? kp - p.K1p : kp;
-    const bool real = kin < (second ? p.K2 : p.K1);
+    const bool reorder = p.kind == IT_PREP_SAGE_REORDER, half = reorder && n >= p.seg;
+    const int c = half ? n - p.seg : n;
+    const bool real = kin < (second ? p.K2 : p.K1) && c < p.out_dim;
     const int k = second ? p.K1 + kin : kin;
     int64_t src;   // element of W that is B[k, n]
-    if (p.kind == IT_PREP_SAGE_REORDER) src = n < p.out_dim ? (int64_t)k * p.out_dim + n : (int64_t)(p.in_dim + k) * p.out_dim + (n - p.out_dim);
-    else src = (int64_t)k * p.out_dim + n;
+    src = (int64_t)(half ? p.in_dim + k : k) * p.out_dim + c;
     if (p.w_is_bf16) {
       reinterpret_cast<__nv_bfloat16 *>(p.B)[i] = real ? reinterpret_cast<const __nv_bfloat16 *>(p.W)[src] : __float2bfloat16_rn(0.f);
     } else {
@@ -1109,22 +1111,24 @@ constexpr int kSmemAux = 1024 /*alignment slack*/ + 288 /*barriers, TMEM slot, a
 
 }  // namespace
 
-size_t it_tc_weights_bytes(const it_layer_desc *L, int NB, int K) {
-  return (size_t)NB * (K + 128) * (L->feat_dtype == IT_BF16 ? 2 : 8);   // room for the padding of both operands' K
-}
-
-// Column split of the tensor-core path: the largest columns-per-CTA count (a multiple of 16 that divides NB, at
-// most 256) whose resident weights leave room for three operand stages (which already give the time of eight)
-// and one 32 KB staging tile of the epilogue.
+// Column split of the tensor-core path: the fewest splits whose columns (a multiple of 16, at most 256; of a head's width where
+// scores are computed) have resident weights that leave room for three operand stages (which already give the time of eight)
+// and one 32 KB staging tile of the epilogue.  Columns past the last output are padding.
 constexpr size_t kWeightBudget = kSmemBudget - kSmemAux - 1024 /*per-column constants*/ - 3 * TC_BM * TC_KBLOCK_BYTES - 32 * 1024;
-static bool tc_split(bool tf32, int NB, int KB, int *n_splits, int *nbc) {
+bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_cols *out) {
+  const bool tf32 = a.x_dtype == IT_F32;
+  const int bk = TC_KBLOCK_BYTES / (tf32 ? 4 : 2), KB = (a.K1 + bk - 1) / bk + ((a.X2 ? a.K2 : 0) + bk - 1) / bk;
+  out->n0p = (a.n0 + 15) / 16 * 16;
+  out->n1p = (a.n1 + 15) / 16 * 16;
+  const int n = out->n0p + out->n1p, step = want_scores ? head_dim : 16;
+  if (n <= 0 || step % 16 != 0) return false;
   for (int s = 1; s <= 16; ++s) {
-    if (NB % s != 0) continue;
-    const int c = NB / s;
+    const int c = ((n + s - 1) / s + step - 1) / step * step;
     // fp32 mode issues MMAs of 2 c columns and keeps 4 c TMEM columns of accumulators next to the split A stages
-    if (c % 16 != 0 || c > (tf32 ? 64 : 256)) continue;
+    if (c > (tf32 ? 64 : 256)) continue;
     if ((size_t)(tf32 ? 2 : 1) * KB * c * TC_KBLOCK_BYTES > kWeightBudget) continue;
-    *n_splits = s; *nbc = c;
+    if (want_scores && c * s != n) continue;
+    out->n_splits = s; out->nbc = c; out->NB = c * s;
     return true;
   }
   return false;
@@ -1133,25 +1137,22 @@ static bool tc_split(bool tf32, int NB, int KB, int *n_splits, int *nbc) {
 bool it_tc_supported(const it_gemm_args &a, int heads, int head_dim, bool want_scores) {
   const bool tf32 = a.x_dtype == IT_F32;
   const int elem = tf32 ? 4 : 2;
-  const int bk = TC_KBLOCK_BYTES / elem;
   if (a.M <= 0 || a.M > (int64_t)INT32_MAX) return false;
   const int K2 = a.X2 ? a.K2 : 0;
   // operand rows must be TMA-addressable (a multiple of 16 bytes); a K that is not a whole number of k-blocks is
   // padded: the TMA copy fills what lies beyond a row with zeros and the prepared weights carry zero rows there
   if (a.K1 <= 0 || (a.K1 * elem) % 16 != 0 || (K2 * elem) % 16 != 0) return false;
-  const int NB = a.n0 + a.n1;   // score columns are not materialised on this path
-  if (NB <= 0 || NB % 16 != 0 || a.n0 % 16 != 0) return false;
-  int n_splits, nbc;
-  if (!tc_split(tf32, NB, (a.K1 + bk - 1) / bk + (K2 + bk - 1) / bk, &n_splits, &nbc)) return false;
-  if (want_scores && (heads > 8 || head_dim % 16 != 0 || nbc % head_dim != 0)) return false;
-  return true;
+  if (tf32 && (a.n0 % 16 != 0 || a.n1 % 16 != 0)) return false;
+  if (want_scores && heads > 8) return false;
+  it_tc_cols cols;   // score columns are not materialised on this path
+  return it_tc_columns(a, head_dim, want_scores, &cols);
 }
 
-it_prep_tc it_prep_tc_of(it_prep_kind kind, const it_layer_desc *L, int NB, int K1, int K2, void *B) {
+it_prep_tc it_prep_tc_of(it_prep_kind kind, const it_layer_desc *L, int NB, int seg, int K1, int K2, void *B) {
   it_prep_tc p;
   const int bk = TC_KBLOCK_BYTES / (L->weight_dtype == IT_BF16 ? 2 : 4);
   p.kind = kind; p.in_dim = L->in_dim; p.out_dim = L->out_dim; p.w_is_bf16 = L->weight_dtype == IT_BF16;
-  p.NB = NB; p.K1 = K1; p.K2 = K2; p.K1p = (K1 + bk - 1) / bk * bk; p.K2p = (K2 + bk - 1) / bk * bk; p.W = L->W; p.B = B;
+  p.NB = NB; p.seg = seg; p.K1 = K1; p.K2 = K2; p.K1p = (K1 + bk - 1) / bk * bk; p.K2p = (K2 + bk - 1) / bk * bk; p.W = L->W; p.B = B;
   return p;
 }
 
@@ -1176,29 +1177,30 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   const bool tf32 = a.x_dtype == IT_F32;
   const int elem = tf32 ? 4 : 2;
   const int bk = TC_KBLOCK_BYTES / elem;
-  const int NB = a.n0 + a.n1;
   const int K2 = a.X2 ? a.K2 : 0;
   const int K = a.K1 + K2;
   const int kb1 = (a.K1 + bk - 1) / bk, kb2 = (K2 + bk - 1) / bk;
   const int KB = kb1 + kb2;
-  int n_splits = 1, nbc = NB;
-  IT_REQUIRE(tc_split(tf32, NB, KB, &n_splits, &nbc), IT_ERR_UNSUPPORTED, "tensor-core apply: cannot tile %d columns with K = %d", NB, K);
+  it_tc_cols cols;
+  IT_REQUIRE(it_tc_columns(a, head_dim, scores != nullptr, &cols), IT_ERR_UNSUPPORTED, "tensor-core apply: cannot tile %d columns with K = %d", a.n0 + a.n1, K);
+  const int NB = cols.NB, n_splits = cols.n_splits, nbc = cols.nbc, n0p = cols.n0p, n1p = cols.n1p;
   const int b_bytes = (tf32 ? 2 : 1) * KB * nbc * TC_KBLOCK_BYTES;
   const int stage_bytes = TC_BM * TC_KBLOCK_BYTES;             // one operand tile (fp32 mode: the raw tile)
   const int const_bytes = nbc * 4 * (scores ? 3 : 1);          // bias (+ attention vectors) of this CTA's columns
   // Staged epilogue (TMA stores): possible when, for every column split, the out0 columns and the out1 columns of
-  // the CTA are whole 128-byte panels that start on a panel boundary, and three operand stages still fit beside
-  // the staging tile (three stages already give the time of eight).
+  // the CTA are whole 128-byte panels or reach the end of their output (the copy clips what lies past it), and three operand
+  // stages still fit beside the staging tile (three stages already give the time of eight).
   const int s0 = a.dt0 == IT_BF16 ? 2 : 4, s1 = a.dt1 == IT_BF16 ? 2 : 4;
   int out_panels = 0;
   bool staged = IT_TC_TMA_STORE != 0;
   for (int sp = 0; sp < n_splits && staged; ++sp) {
-    const int cb = sp * nbc, ce = cb + nbc;
-    const int lo0 = cb < a.n0 ? cb : a.n0, hi0 = ce < a.n0 ? ce : a.n0;
-    const int lo1 = cb > a.n0 ? cb : a.n0, hi1 = ce < NB ? ce : NB;
+    const int cb = sp * nbc, ce = cb + nbc, n01 = n0p + n1p;
+    const int lo0 = cb < n0p ? cb : n0p, hi0 = ce < n0p ? ce : n0p;
+    const int lo1 = cb > n0p ? cb : n0p, hi1 = ce < n01 ? ce : n01;
     const int b0 = hi0 > lo0 ? (hi0 - lo0) * s0 : 0, b1 = hi1 > lo1 ? (hi1 - lo1) * s1 : 0;
-    if (b0 % 128 != 0 || b1 % 128 != 0 || (b0 > 0 && (lo0 * s0) % 128 != 0) || (b1 > 0 && ((lo1 - a.n0) * s1) % 128 != 0)) staged = false;
-    if (b0 / 128 + b1 / 128 > out_panels) out_panels = b0 / 128 + b1 / 128;
+    if ((b0 % 128 != 0 && hi0 != n0p) || (b1 % 128 != 0 && hi1 != n01)) staged = false;
+    const int panels = (b0 + 127) / 128 + (b1 + 127) / 128;
+    if (panels > out_panels) out_panels = panels;
   }
   // two groups of epilogue warps (alternate tiles, a staging tile each) when the second staging tile still fits
   int epi_groups = IT_TC_EPI_GROUPS;
@@ -1229,8 +1231,8 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   TcParams p;
   p.M = a.M; p.n_tiles_m = (int)((a.M + TC_BM - 1) / TC_BM); p.n_splits = n_splits; p.nbc = nbc;
   p.kb1 = kb1; p.kb2 = kb2; p.NB = NB; p.stages = stages; p.tstages = tstages;
-  p.n0 = a.n0; p.out0 = a.out0; p.out0_bf16 = a.dt0 == IT_BF16; p.bias0 = a.bias0; p.act0 = a.act0;
-  p.n1 = a.n1; p.out1 = a.out1; p.out1_bf16 = a.dt1 == IT_BF16;
+  p.n0 = n0p; p.n0_real = a.n0; p.out0 = a.out0; p.out0_bf16 = a.dt0 == IT_BF16; p.bias0 = a.bias0; p.act0 = a.act0;
+  p.n1 = n1p; p.n1_real = a.n1; p.out1 = a.out1; p.out1_bf16 = a.dt1 == IT_BF16;
   p.scores = scores; p.att_src = att_src; p.att_dst = att_dst; p.heads = heads; p.head_dim = head_dim > 0 ? head_dim : 1;
   p.status = status;
   p.tma_store = staged ? 1 : 0; p.out_panels = out_panels; p.epi_groups = epi_groups;
@@ -1241,8 +1243,8 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   if (grid > n_tiles) grid = n_tiles;   // n_tiles is a multiple of n_splits
   const double xs = elem;
   const double bytes = (double)a.M * (K * xs + a.n0 * (a.dt0 == IT_F32 ? 4.0 : 2.0) + a.n1 * (a.dt1 == IT_F32 ? 4.0 : 2.0) +
-                                     (scores ? 8.0 * heads : 0.0)) + (double)K * NB * xs;
-  const double flops = 2.0 * (double)a.M * K * NB;
+                                     (scores ? 8.0 * heads : 0.0)) + (double)K * (a.n0 + a.n1) * xs;
+  const double flops = 2.0 * (double)a.M * K * (a.n0 + a.n1);
   if (tf32) {
     IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<true>, dim3((unsigned)grid), dim3(TC_THREADS_TF32), smem, st, m1, m2, mb, mo0, mo1, p)));

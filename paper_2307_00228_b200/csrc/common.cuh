@@ -273,17 +273,22 @@ it_status it_launch_prep_weights(it_prep_kind kind, const it_layer_desc *layer, 
 
 // ----------------------------------------------------------------------------- apply_tc.cu
 // The same product on the tensor cores (tcgen05 + TMEM + TMA).  Needs operand rows that are multiples of 16
-// bytes (K1, K2 are padded to whole 128-byte k-blocks with zeros) and n0, n0 + n1 multiples of 16; computes the n0 + n1 columns and, for GAT, the
+// bytes (K1, K2 are padded to whole 128-byte k-blocks with zeros) and, for fp32, n0 and n1 multiples of 16 (bf16 outputs of any
+// width are padded: the products are exact either way, where fp32 splits its operands); computes the n0 + n1 columns and, for GAT, the
 // attention scores [M, 2*heads] in its epilogue (a.B, a.NB and a.out2 are not used).  B is the
 // matrix written by it_launch_prep_weights_tc: bf16 [NB, Kp] or fp32 [2, NB, Kp] (hi, lo), K-major, Kp = padded K1 + padded K2.
 bool it_tc_supported(const it_gemm_args &a, int heads, int head_dim, bool want_scores);
 struct it_prep_tc {
-  int kind, in_dim, out_dim, w_is_bf16, NB;
+  int kind, in_dim, out_dim, w_is_bf16, NB;   // NB: columns with their padding; columns of no weight are zero
+  int seg;                // IT_PREP_SAGE_REORDER: first column of the neighbour half
   int K1, K1p, K2, K2p;   // rows of W behind X1 / X2, and the same rounded up to whole k-blocks (the padding is zero)
   const void *W;
   void *B;   // bf16 [NB, K1p + K2p]  or  fp32 [2, NB, K1p + K2p] (hi, lo)
 };
-it_prep_tc it_prep_tc_of(it_prep_kind kind, const it_layer_desc *layer, int NB, int K1, int K2, void *B);
+it_prep_tc it_prep_tc_of(it_prep_kind kind, const it_layer_desc *layer, int NB, int seg, int K1, int K2, void *B);
+// How the product's columns are laid out: each output padded to a multiple of 16 columns, all of them to whole splits.
+struct it_tc_cols { int n0p, n1p, n_splits, nbc, NB; };
+bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_cols *out);
 size_t it_prep_tc_bytes(const it_prep_tc &p);
 // Several weight matrices and `words` zeroed words in as few launches as possible.
 it_status it_launch_prep_weights_tc(const it_prep_tc *list, int count, int *zero, size_t words, cudaStream_t stream);

@@ -16,3 +16,17 @@ def test_padded_rows_in_every_bucket(dtype, fi, max_deg):
         w = small_workload(8, 900, max_deg, dtype, [layer], hubs=(2100, 700, 300, 90), weights=weights)
         got, _ = run_device(w)
         check_against_oracle(w, got, label=(dtype, fi, op, max_deg))
+
+
+@pytest.mark.parametrize("dtype,dims", [("bf16", (64, 8)), ("bf16", (64, 24)), ("bf16", (96, 40)), ("bf16", (64, 104)), ("bf16", (40, 200)), ("bf16", (600, 40)),
+                                        ("bf16", (128, 264)), ("bf16", (64, 48)), ("bf16", (64, 96)), ("f32", (64, 48)), ("f32", (128, 112)), ("f32", (128, 80)),
+                                        ("f32", (64, 100)), ("f32", (20, 12)), ("f32", (32, 176))])
+def test_output_widths_of_the_dense_products(dtype, dims):
+    """Outputs that are no whole 128-byte panel, no multiple of 16 columns, or split over several column ranges; one output, and
+    two side by side (transform-first layers), with rows that end inside a 128-row tile."""
+    fi, fo = dims
+    for op, reorder, n in (("mean", False, 300), ("sum", True, 1285)):
+        layer = make_sage_layer(9, op, "relu", fi, fo, dtype, allow_reorder=reorder)
+        w = small_workload(10, n, 9, dtype, [layer], hubs=(200,))
+        got, _ = run_device(w)
+        check_against_oracle(w, got, label=(dtype, dims, op))
