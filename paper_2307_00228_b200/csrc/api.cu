@@ -208,7 +208,8 @@ it_status run_apply(const StageCtx &c, const it_layer_desc *L, it_prep_kind kind
 }
 
 // out [M, n_out] = act(X [M, K] * W [K, n_out] + bias): one plain dense product with W taken as it is.
-it_status run_dense(const StageCtx &c, int64_t M, const void *X, int K, const void *W, int n_out, const float *bias, it_act act, void *out) {
+it_status run_dense(const StageCtx &c, int64_t M, const void *X, int K, const void *W, int n_out, const float *bias, it_act act, void *out,
+                    const void *add_rows = nullptr, const int32_t *add_idx = nullptr) {
   const it_layer_desc *L = c.L;
   it_layer_desc d = *L;   // a view of the layer that names this product's weights
   d.op = IT_GATHER_NONE; d.in_dim = K; d.out_dim = n_out; d.W = W; d.heads = 1; d.edge_dim = 0; d.msg_dim = 0;
@@ -217,7 +218,15 @@ it_status run_dense(const StageCtx &c, int64_t M, const void *X, int K, const vo
   ga.B = c.B; ga.NB = n_out;
   ga.n0 = n_out; ga.out0 = out; ga.dt0 = L->feat_dtype; ga.bias0 = bias; ga.act0 = act;
   ga.n1 = 0; ga.out1 = nullptr; ga.dt1 = L->feat_dtype; ga.out2 = nullptr;
+  ga.add_rows = add_rows; ga.add_idx = add_idx;
   return run_apply(c, &d, IT_PREP_DENSE, ga, nullptr);
+}
+
+// Whether the per-edge product of learned messages can add the source part and finish the message itself.
+bool message_in_product(const it_graph *g, const it_layer_desc *L) {
+  it_gemm_args ga{};
+  ga.M = g->e; ga.x_dtype = L->feat_dtype; ga.X1 = g; ga.K1 = L->edge_dim; ga.n0 = L->msg_dim; ga.dt0 = ga.dt1 = L->feat_dtype;
+  return it_tc_adds_rows(ga);
 }
 
 // The edge-feature half of the message [w_e h_u | e_vu]: the same reduce over the rows of the edge-feature
@@ -323,14 +332,16 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
         gg.src = table;
         return it_launch_gather(gg, c.st);
       } else {
-        // the edge part Q = e W_edge[in:] + b_edge, once per edge; then m_j = act_edge(P[u_j] + Q[j]) in place; then the
-        // reduce over the message rows, which lie in edge order
+        // the edge part Q = e W_edge[in:] + b_edge, once per edge; m_j = act_edge(P[u_j] + Q[j]) in the product's epilogue, or
+        // (shapes that it does not take) in place; then the reduce over the message rows, which lie in edge order
         void *Q = c.ws + c.w.off_q;
         const size_t es = (size_t)it_dtype_size(dt);
         const char *W_edge_part = (const char *)L->W_edge + (size_t)L->in_dim * L->msg_dim * es;
-        IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, IT_ACT_NONE, Q));
+        const bool whole = message_in_product(g, L);
+        IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, whole ? L->act_edge : IT_ACT_NONE, Q,
+                         whole ? table : nullptr, whole ? g->indices : nullptr));
         if (c.recording()) return IT_OK;
-        IT_TRY(it_launch_edge_messages(g, dt, L->msg_dim, table, Q, L->act_edge, c.st));
+        if (!whole) IT_TRY(it_launch_edge_messages(g, dt, L->msg_dim, table, Q, L->act_edge, c.st));
         gg.src = Q; gg.src_ld = 0; gg.per_edge_rows = 1;
         return it_launch_gather(gg, c.st);
       }

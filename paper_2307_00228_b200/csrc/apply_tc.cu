@@ -208,6 +208,7 @@ struct TcParams {
   // epilogue routing (columns are global column ids)
   int n0, n0_real; void *out0; int out0_bf16; const float *bias0; int act0;   // n0, n1: with their padding; *_real: what is stored
   int n1, n1_real; void *out1; int out1_bf16;
+  const char *add_rows; const int32_t *add_idx; int add_pitch;   // staged epilogue: rows added to out0 (NULL: none); bytes from one to the next
   float *scores; const float *att_src; const float *att_dst; int heads, head_dim;  // GAT: scores [M, 2*heads]
   int *status;                    // set to 1 if a bounded wait gave up
   int tma_store;                  // 1: the epilogue stages each output tile in shared memory and writes it with TMA stores
@@ -414,6 +415,35 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       int last_u = -1;   // the last unit this warp owns (ownership: (unit0 + u) % n_sub == gsub)
       for (int u = n_units - 1; u >= 0; --u)
         if ((unit0 + u) % n_sub == gsub) { last_u = u; break; }
+      // Rows added to out0: the first pieces of this lane's row of the NEXT tile are fetched as soon as this tile's are used up,
+      // so that they are in flight across the barrier, the stores and the wait for the accumulator (fetched at the start of
+      // their own tile they made a product over 16M edges take 1.7 ms: ADD_NOTE).
+      constexpr int GP = TF32 ? 4 : 2;          // 16-byte pieces of a 16-column group
+      constexpr int PRE = 4, NPRE = PRE / GP;   // pieces fetched ahead: two groups of bf16, one of fp32
+      constexpr int ES = TF32 ? 4 : 2;
+      uint4 pre[PRE];
+      auto add_source = [&](int tile) -> int32_t {
+        const int64_t m = (int64_t)(tile / p.n_splits) * TC_BM + row_in_tile;
+        return p.add_rows && tile < n_tiles && m < p.M ? __ldcs(p.add_idx + m) : 0;
+      };
+      auto fetch_ahead = [&](int32_t src) {
+        const char *row = p.add_rows + (int64_t)src * p.add_pitch;
+#pragma unroll
+        for (int u = 0; u < NPRE; ++u) {
+          const int unit = u * n_sub + (gsub + n_sub - unit0 % n_sub) % n_sub;   // the (u + 1)-th unit that this warp owns
+          const int at = (col_base + unit * 16) * ES;
+#pragma unroll
+          for (int q = 0; q < GP; ++q) {
+            pre[u * GP + q] = make_uint4(0u, 0u, 0u, 0u);
+            if (unit < n_units && at + q * 16 < p.add_pitch) pre[u * GP + q] = __ldg(reinterpret_cast<const uint4 *>(row + at) + q);
+          }
+        }
+      };
+      int32_t src_c = 0;
+      if (p.add_rows) {
+        src_c = add_source((int)blockIdx.x + group * (int)gridDim.x);
+        fetch_ahead(src_c);
+      }
       int it = 0;   // tiles of this CTA so far: tile `it` uses accumulator it % 2, for the (it / 2)-th time
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
         if (G == 2 && (it & 1) != group) continue;
@@ -421,6 +451,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
         acc_phase = ((uint32_t)it >> 1) & 1u;
         const int m0 = (tile / p.n_splits) * TC_BM;
         const int64_t m = (int64_t)m0 + row_in_tile;
+        const int next = tile + G * (int)gridDim.x;   // this group's next tile
+        const int32_t src_n = add_source(next);       // its row's source, in flight during this tile
+        const char *add_row = p.add_rows + (int64_t)src_c * p.add_pitch;   // (used with rows to add only)
+        int nth = 0;   // units of this warp so far
         ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, p.spin_limit, IT_TC_EPI_BACKOFF);
         if (issuer) tma_store_wait_read();   // the stores of this group's previous tile have read the staging tile
         // one decision for all warps of the group (they meet at named barriers below, so none may leave alone)
@@ -476,6 +510,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
                 const float4 b4 = bs[i];
                 v[4 * i] += b4.x; v[4 * i + 1] += b4.y; v[4 * i + 2] += b4.z; v[4 * i + 3] += b4.w;
               }
+              if (p.add_rows) {
+#pragma unroll
+                for (int q = 0; q < GP; ++q) {
+                  uint4 x = make_uint4(0u, 0u, 0u, 0u);
+                  if (nth == 0) x = pre[q];
+                  else if (NPRE > 1 && nth == 1) x = pre[NPRE > 1 ? GP + q : q];
+                  else if (gc * ES + q * 16 < p.add_pitch) x = __ldg(reinterpret_cast<const uint4 *>(add_row + gc * ES) + q);
+                  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                  for (int i = 0; i < 4; ++i) {
+                    if (TF32) {
+                      v[4 * q + i] += __uint_as_float(w[i]);
+                    } else {
+                      const __nv_bfloat162 h = __floats2bfloat162_rn(v[8 * q + 2 * i], v[8 * q + 2 * i + 1]);
+                      v[8 * q + 2 * i] = __low2float(h) + __uint_as_float(w[i] << 16);
+                      v[8 * q + 2 * i + 1] = __high2float(h) + __uint_as_float(w[i] & 0xffff0000u);
+                    }
+                  }
+                }
+                ++nth;
+              }
               if (p.act0 == IT_ACT_RELU) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) v[i] = fmaxf(v[i], 0.f);
@@ -516,6 +571,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&acc_empty[acc]);
+        }
+        if (p.add_rows) {
+          src_c = src_n;
+          if (next < n_tiles) fetch_ahead(src_c);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the TMA store's reads
         epi_bar_sync(G, group);
@@ -1169,24 +1228,16 @@ it_status it_launch_prep_weights_tc(const it_prep_tc *list, int count, int *zero
   return IT_OK;
 }
 
-// B: weights prepared by it_launch_prep_weights_tc.  a.B / a.NB / a.out2 of the generic args are ignored:
-// the tensor-core path computes n0 + n1 columns and, for GAT, the scores in its epilogue.
-it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *att_src, const float *att_dst, int heads,
-                            int head_dim, float *scores, int num_sms, int *status, cudaStream_t st) {
-  if (a.M == 0) return IT_OK;
+namespace {
+struct TcShape { int b_bytes, const_bytes, out_panels, epi_groups, stages; bool staged; };
+
+// How a product's shared memory is used.
+bool tc_shape(const it_gemm_args &a, const it_tc_cols &cols, int KB, bool want_scores, TcShape *out) {
   const bool tf32 = a.x_dtype == IT_F32;
-  const int elem = tf32 ? 4 : 2;
-  const int bk = TC_KBLOCK_BYTES / elem;
-  const int K2 = a.X2 ? a.K2 : 0;
-  const int K = a.K1 + K2;
-  const int kb1 = (a.K1 + bk - 1) / bk, kb2 = (K2 + bk - 1) / bk;
-  const int KB = kb1 + kb2;
-  it_tc_cols cols;
-  IT_REQUIRE(it_tc_columns(a, head_dim, scores != nullptr, &cols), IT_ERR_UNSUPPORTED, "tensor-core apply: cannot tile %d columns with K = %d", a.n0 + a.n1, K);
-  const int NB = cols.NB, n_splits = cols.n_splits, nbc = cols.nbc, n0p = cols.n0p, n1p = cols.n1p;
+  const int n_splits = cols.n_splits, nbc = cols.nbc, n0p = cols.n0p, n1p = cols.n1p;
   const int b_bytes = (tf32 ? 2 : 1) * KB * nbc * TC_KBLOCK_BYTES;
   const int stage_bytes = TC_BM * TC_KBLOCK_BYTES;             // one operand tile (fp32 mode: the raw tile)
-  const int const_bytes = nbc * 4 * (scores ? 3 : 1);          // bias (+ attention vectors) of this CTA's columns
+  const int const_bytes = nbc * 4 * (want_scores ? 3 : 1);          // bias (+ attention vectors) of this CTA's columns
   // Staged epilogue (TMA stores): possible when, for every column split, the out0 columns and the out1 columns of
   // the CTA are whole 128-byte panels or reach the end of their output (the copy clips what lies past it), and three operand
   // stages still fit beside the staging tile (three stages already give the time of eight).
@@ -1212,7 +1263,41 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   if (!staged) { out_panels = 0; epi_groups = 1; }
   int stages = (kSmemBudget - kSmemAux - const_bytes - b_bytes - epi_groups * out_panels * stage_bytes) / stage_bytes;
   if (stages > IT_TC_MAX_STAGES) stages = IT_TC_MAX_STAGES;
-  IT_REQUIRE(stages >= 2, IT_ERR_UNSUPPORTED, "tensor-core apply: no room for two operand stages");
+  if (stages < 2) return false;
+  out->b_bytes = b_bytes; out->const_bytes = const_bytes; out->out_panels = out_panels; out->epi_groups = epi_groups;
+  out->stages = stages; out->staged = staged;
+  return true;
+}
+}  // namespace
+
+bool it_tc_adds_rows(const it_gemm_args &a) {
+  it_tc_cols cols;
+  TcShape sh;
+  const int bk = TC_KBLOCK_BYTES / (a.x_dtype == IT_F32 ? 4 : 2), KB = (a.K1 + bk - 1) / bk + ((a.X2 ? a.K2 : 0) + bk - 1) / bk;
+  return it_tc_supported(a, 1, a.n0, false) && it_tc_columns(a, a.n0, false, &cols) && tc_shape(a, cols, KB, false, &sh) && sh.staged && a.n1 == 0;
+}
+
+// B: weights prepared by it_launch_prep_weights_tc.  a.B / a.NB / a.out2 of the generic args are ignored:
+// the tensor-core path computes n0 + n1 columns and, for GAT, the scores in its epilogue.
+it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *att_src, const float *att_dst, int heads,
+                            int head_dim, float *scores, int num_sms, int *status, cudaStream_t st) {
+  if (a.M == 0) return IT_OK;
+  const bool tf32 = a.x_dtype == IT_F32;
+  const int elem = tf32 ? 4 : 2;
+  const int bk = TC_KBLOCK_BYTES / elem;
+  const int K2 = a.X2 ? a.K2 : 0;
+  const int K = a.K1 + K2;
+  const int kb1 = (a.K1 + bk - 1) / bk, kb2 = (K2 + bk - 1) / bk;
+  const int KB = kb1 + kb2;
+  it_tc_cols cols;
+  IT_REQUIRE(it_tc_columns(a, head_dim, scores != nullptr, &cols), IT_ERR_UNSUPPORTED, "tensor-core apply: cannot tile %d columns with K = %d", a.n0 + a.n1, K);
+  const int NB = cols.NB, n_splits = cols.n_splits, nbc = cols.nbc, n0p = cols.n0p, n1p = cols.n1p;
+  TcShape sh;
+  IT_REQUIRE(tc_shape(a, cols, KB, scores != nullptr, &sh), IT_ERR_UNSUPPORTED, "tensor-core apply: no room for two operand stages");
+  IT_REQUIRE(!a.add_rows || sh.staged, IT_ERR_UNSUPPORTED, "tensor-core apply: rows are added by the staged epilogue only");
+  const int b_bytes = sh.b_bytes, stage_bytes = TC_BM * TC_KBLOCK_BYTES, const_bytes = sh.const_bytes, out_panels = sh.out_panels;
+  const int epi_groups = sh.epi_groups, stages = sh.stages, s0 = a.dt0 == IT_BF16 ? 2 : 4, s1 = a.dt1 == IT_BF16 ? 2 : 4;
+  const bool staged = sh.staged;
   const int smem = b_bytes + (stages + epi_groups * out_panels) * stage_bytes + kSmemAux + const_bytes;
   // fp32 mode: TMEM holds two accumulators of 2 nbc columns; what is left of its 512 columns stages the split A
   int tstages = tf32 ? (512 - 4 * nbc) / TC_TSTAGE_COLS : 0;
@@ -1233,6 +1318,7 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   p.kb1 = kb1; p.kb2 = kb2; p.NB = NB; p.stages = stages; p.tstages = tstages;
   p.n0 = n0p; p.n0_real = a.n0; p.out0 = a.out0; p.out0_bf16 = a.dt0 == IT_BF16; p.bias0 = a.bias0; p.act0 = a.act0;
   p.n1 = n1p; p.n1_real = a.n1; p.out1 = a.out1; p.out1_bf16 = a.dt1 == IT_BF16;
+  p.add_rows = (const char *)a.add_rows; p.add_idx = a.add_idx; p.add_pitch = a.n0 * s0;
   p.scores = scores; p.att_src = att_src; p.att_dst = att_dst; p.heads = heads; p.head_dim = head_dim > 0 ? head_dim : 1;
   p.status = status;
   p.tma_store = staged ? 1 : 0; p.out_panels = out_panels; p.epi_groups = epi_groups;

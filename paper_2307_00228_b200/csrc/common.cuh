@@ -260,6 +260,9 @@ struct it_gemm_args {
   int n0; void *out0; it_dtype dt0; const float *bias0; it_act act0;
   int n1; void *out1; it_dtype dt1;
   void *out2;
+  // tensor-core path, staged stores only (it_tc_adds_rows): out0[m, :] = act0(round(C + bias0) + add_rows[add_idx[m], :]), rows of
+  // n0 elements of dt0; `round` to dt0, as if the product had been stored and read back
+  const void *add_rows; const int32_t *add_idx;
   uint32_t spin_limit;   // tensor-core path: polls after which a barrier wait gives up (0 = the default)
   int no_loads;          // tensor-core path, test hook: issue no operand copies
 };
@@ -292,6 +295,7 @@ bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_
 size_t it_prep_tc_bytes(const it_prep_tc &p);
 // Several weight matrices and `words` zeroed words in as few launches as possible.
 it_status it_launch_prep_weights_tc(const it_prep_tc *list, int count, int *zero, size_t words, cudaStream_t stream);
+bool it_tc_adds_rows(const it_gemm_args &a);
 it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *att_src, const float *att_dst,
                             int heads, int head_dim, float *scores, int num_sms, int *status, cudaStream_t stream);
 
