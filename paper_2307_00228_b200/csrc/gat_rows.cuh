@@ -129,19 +129,24 @@ struct GatWarp {
 #ifndef IT_GAT_CHUNK_BLOCKS
 #define IT_GAT_CHUNK_BLOCKS 3   // resident CTAs per SM: at four the 64 registers a thread gets spill (measured: 3 to 5 % more time)
 #endif
-template <int H> constexpr int gat_bytes_per_warp() { return ring_bytes_per_warp<16, false>() + 32 * H * 4; }
+#ifndef IT_GAT_STAGE_ROWS
+#define IT_GAT_STAGE_ROWS 8   // 512-byte groups of rows per stage of the chunk kernel's ring (4: 2.5 % more time on 5M vertices / 100M edges)
+#endif
+// (64-byte rows: 32 edges are four groups)
+template <int LPR> constexpr int gat_stage_rows() { return LPR == 4 ? 4 : IT_GAT_STAGE_ROWS; }
+template <int LPR, int H> constexpr int gat_bytes_per_warp() { return ring_bytes_per_warp<16, false, gat_stage_rows<LPR>()>() + 32 * H * 4; }
 
 template <typename T, int LPR, int H>
 __global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol) {
   extern __shared__ uint4 ring_raw[];
   const int lane = threadIdx.x & 31;
-  const uint32_t base = (uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)(threadIdx.x >> 5) * (uint32_t)gat_bytes_per_warp<H>();
-  RingWarp<T, 16, LPR, GatAcc<T>, false> rw;
+  const uint32_t base = (uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)(threadIdx.x >> 5) * (uint32_t)gat_bytes_per_warp<LPR, H>();
+  RingWarp<T, 16, LPR, GatAcc<T>, false, gat_stage_rows<LPR>()> rw;
   rw.setup(base, p.src, p.src_pitch, p.slices, lane);
   pol.setup(lane % LPR);
   __shared__ float bias_buf[256];
   stage_bias(pol, bias_buf);
-  GatWarp<T, LPR, H> gw(p, q, lane, base + ring_bytes_per_warp<16, false>());
+  GatWarp<T, LPR, H> gw(p, q, lane, base + ring_bytes_per_warp<16, false, gat_stage_rows<LPR>()>());
   ChunkCursor<false, true> cur(p, lane);
   chunk_walk<LPR, true>(rw, gw.acc, cur, [&](Chunk &c) { gw.ahead(c); }, [&](const Chunk &c, bool first) { gw.begin(c, first); },
       [&](int k, const uint4 &raw, bool valid) {
@@ -428,7 +433,7 @@ it_status launch_gat_rows(const it_gat_args &a, StreamParams p, const GatPolicy<
     p.row_lo = lo; p.row_hi = hi;
     const int64_t rows = hi - lo;
     const double bytes = bytes_of(b, rows);
-    constexpr int smem = (THREADS / 32) * gat_bytes_per_warp<H>();
+    constexpr int smem = (THREADS / 32) * gat_bytes_per_warp<LPR, H>();
     if (bound == 0) {
       it_empty_rows_args er;
       pol.empty_rows(er);

@@ -14,7 +14,10 @@ template <typename T, int SB, int RED, bool WEIGHTED_>
 struct SagePolicy {
   using Slice = RowSlice<T, SB>;
   static constexpr int VEC = Slice::VEC;
-  static constexpr int NS = VEC;
+  // Plain max / min of bf16 rows stays packed, two entries per word: a quarter of the instructions (the largest of bf16 values
+  // is one of them, so nothing is rounded): extreme hubs, 20M vertices / 200M edges, three layers, 17.4 -> 15.2 ms.
+  static constexpr bool PACKED = RED != RED_SUM && !WEIGHTED_ && sizeof(T) == 2 && SB == 16;
+  static constexpr int NS = PACKED ? VEC / 2 : VEC;
   static constexpr bool WEIGHTED = WEIGHTED_, HAS_EXTRA = false, NEEDS_OWNER = false, NULLABLE = false;
   float *__restrict__ partials;
   void *__restrict__ dst;
@@ -34,7 +37,18 @@ struct SagePolicy {
     a.bias = bias; a.act = (it_act)act;
   }
   __device__ __forceinline__ void setup(int t) { col = t * VEC; }
+  static __device__ __forceinline__ float pick2(float a, float b) {   // two bf16 entries per word
+    uint32_t r;
+    if (RED == RED_MAX) asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(__float_as_uint(a)), "r"(__float_as_uint(b)));
+    else asm("min.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(__float_as_uint(a)), "r"(__float_as_uint(b)));
+    return __uint_as_float(r);
+  }
   __device__ __forceinline__ void init(float (&st)[NS]) const {
+    if constexpr (PACKED) {
+#pragma unroll
+      for (int k = 0; k < NS; ++k) st[k] = __uint_as_float(RED == RED_MAX ? 0xff80ff80u : 0x7f807f80u);   // -inf / +inf
+      return;
+    }
 #pragma unroll
     for (int k = 0; k < NS; ++k) st[k] = RED == RED_MAX ? -INFINITY : (RED == RED_MIN ? INFINITY : 0.f);
   }
@@ -49,9 +63,17 @@ struct SagePolicy {
       for (int i = 0; i < SB / 4; ++i) add_bf16x2_to_f32(st[2 * i], st[2 * i + 1], w[i]);
       return;
     }
+    if constexpr (PACKED) {
+      uint32_t q[SB / 4];
+      raw_words<SB>(raw, q);
+#pragma unroll
+      for (int k = 0; k < NS; ++k) st[k] = pick2(st[k], __uint_as_float(q[k]));
+      return;
+    }
     float f[VEC];
     Slice::unpack(raw, f);
-    if constexpr (RED == RED_SUM && !WEIGHTED && VEC % 2 == 0) {   // two accumulators per instruction (measured: 1 % on the
+    if constexpr (PACKED) {
+    } else if constexpr (RED == RED_SUM && !WEIGHTED && VEC % 2 == 0) {   // two accumulators per instruction (measured: 1 % on the
 #pragma unroll                                                      // 128-byte rows; with a weight the pair set-up eats the gain)
       for (int k = 0; k < VEC; k += 2) add_f32x2(st[k], st[k + 1], f[k], f[k + 1]);
     } else {
@@ -64,6 +86,11 @@ struct SagePolicy {
     }
   }
   __device__ __forceinline__ void merge(float (&st)[NS], const float (&o)[NS]) const {
+    if constexpr (PACKED) {
+#pragma unroll
+      for (int k = 0; k < NS; ++k) st[k] = pick2(st[k], o[k]);
+      return;
+    }
 #pragma unroll
     for (int k = 0; k < NS; ++k) st[k] = RED == RED_MAX ? fmaxf(st[k], o[k]) : (RED == RED_MIN ? fminf(st[k], o[k]) : st[k] + o[k]);
   }
@@ -72,7 +99,13 @@ struct SagePolicy {
     if (epi == IT_EPI_ADD_ACT && dest >= 0)
       Slice::unpack(Slice::load_stream(reinterpret_cast<const char *>(self_term) + ((int64_t)dest * self_ld + col) * (int64_t)sizeof(T)), self);
   }
-  __device__ __forceinline__ void end_row(float (&st)[NS], int32_t dest, int32_t, int64_t len) const {
+  __device__ __forceinline__ void end_row(float (&packed)[NS], int32_t dest, int32_t, int64_t len) const {
+    float st[VEC];
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) {
+      if constexpr (PACKED) st[i] = __uint_as_float((i & 1) ? (__float_as_uint(packed[i / 2]) & 0xffff0000u) : (__float_as_uint(packed[i / 2]) << 16));
+      else st[i] = packed[i];
+    }
     if (RED != RED_SUM && len == 0 && epi != IT_EPI_RAW_F32) {
 #pragma unroll
       for (int i = 0; i < VEC; ++i) st[i] = 0.f;

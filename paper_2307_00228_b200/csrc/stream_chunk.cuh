@@ -88,7 +88,7 @@ struct ChunkCursor {
 // DEEP: chunks are asked for two ahead of the current one (ahead() then finds their ids landed), else one.
 template <int LPR, bool DEEP, class Warp, class Policy, class Cursor, class Ahead, class Begin, class Edge, class End>
 __device__ __forceinline__ void chunk_walk(const Warp &rw, const Policy &pol, Cursor &cur, Ahead ahead, Begin begin, Edge edge, End end) {
-  using G = RingGeom<16, LPR>;
+  using G = typename Warp::G;
   constexpr int SL = G::SL, GE = G::GE, R = G::R, GB = G::GB;
   static_assert(G::S == 2, "one stage in flight, one being reduced");
   Chunk c, n, nn;

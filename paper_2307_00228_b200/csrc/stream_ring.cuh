@@ -48,26 +48,26 @@ __device__ __forceinline__ float lds_f32(uint32_t a) {
   return v;
 }
 
-// Geometry of the ring for rows of LPR slices of SB bytes.  A stage always holds IT_RING_STAGE_ROWS * 512 bytes of rows.
-template <int SB, int LPR>
+// Geometry of the ring for rows of LPR slices of SB bytes.  A stage always holds ROWS * 512 bytes of rows.
+template <int SB, int LPR, int ROWS = IT_RING_STAGE_ROWS>
 struct RingGeom {
   static constexpr int SL = 32 / LPR;                        // edge slots: rows a warp moves per instruction
   static constexpr int ROWB = LPR * SB;                      // bytes of a row that are gathered (the source rows may be wider)
   static constexpr int GB = 32 * SB;                         // bytes of a group: what one instruction moves
-  static constexpr int R = IT_RING_STAGE_ROWS * (16 / SB);   // groups per stage
+  static constexpr int R = ROWS * (16 / SB);   // groups per stage
   static constexpr int GE = R * SL;                          // edges per stage
   static constexpr int S = IT_RING_STAGES;
   static constexpr int AHEAD = (S - 1) * GE;                 // the stage being filled is this many edges ahead of the one reduced
   static_assert(GE <= 32 && 32 % GE == 0 && AHEAD <= 32, "an index chunk of 32 edges is a whole number of stages and the fill reaches at most into the next chunk");
 };
-template <int SB, bool HAS_EXTRA> constexpr int ring_bytes_per_warp() {
-  return IT_RING_STAGES * IT_RING_STAGE_ROWS * (512 + (HAS_EXTRA ? (16 / SB) * 128 : 0));
+template <int SB, bool HAS_EXTRA, int ROWS = IT_RING_STAGE_ROWS> constexpr int ring_bytes_per_warp() {
+  return IT_RING_STAGES * ROWS * (512 + (HAS_EXTRA ? (16 / SB) * 128 : 0));
 }
 
 // What a warp needs to drive its ring: addresses, the fill of a stage and the reduction of one group.
-template <typename T, int SB, int LPR, class Policy, bool PAD>
+template <typename T, int SB, int LPR, class Policy, bool PAD, int ROWS = IT_RING_STAGE_ROWS>
 struct RingWarp {
-  using G = RingGeom<SB, LPR>;
+  using G = RingGeom<SB, LPR, ROWS>;
   using Raw = typename SliceRaw<SB>::type;
   uint32_t my_ring, my_xring;   // shared-window addresses of my slice / my per-edge scalar in group 0 of stage 0
   const char *my_src;           // my slice of source row 0
