@@ -647,11 +647,11 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
             all += bytes_of(b0, g->h_list_offsets[b0 + 1] - g->h_list_offsets[b0]);
           }
           p.row_lo = g->h_list_offsets[b0];
-          constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<16, false>();
+          constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<16, false, IT_CHUNK_STAGE_ROWS>();
           static std::atomic<uint64_t> configured{0};   // per template instance: one bit per device ordinal
           IT_TRY(allow_dynamic_smem(stream_rows_chunk_kernel<T, LPR, Policy, PAD>, smem, configured));
           p.counter = counters + b;
-          const unsigned blocks = chunk_grid(p, b == g->n_lists - 1 ? rows : 0, (int64_t)g->num_sms * IT_RING_MIN_BLOCKS);
+          const unsigned blocks = chunk_grid(p, b == g->n_lists - 1 ? rows : 0, (int64_t)g->num_sms * IT_CHUNK_BLOCKS);
           IT_LAUNCH(kid_rows, all, 0, st, stream_rows_chunk_kernel<T, LPR, Policy, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
           p.counter = nullptr;
           continue;
