@@ -90,6 +90,7 @@ struct it_graph {
   // derived by the split (library-owned, device; all carved out of one allocation that is kept for the next split)
   char *slab = nullptr;
   size_t slab_bytes = 0;
+  bool slab_pooled = false;   // from the library's memory pool
   int64_t threshold = 0;
   int64_t n_rows = 0;           // R
   int64_t n_split_owners = 0;   // vertices with more than one shadow row
