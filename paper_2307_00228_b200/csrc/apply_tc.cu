@@ -208,7 +208,7 @@ struct TcParams {
   // epilogue routing (columns are global column ids)
   int n0, n0_real; void *out0; int out0_bf16; const float *bias0; int act0;   // n0, n1: with their padding; *_real: what is stored
   int n1, n1_real; void *out1; int out1_bf16;
-  const char *add_rows; const int32_t *add_idx; int add_pitch;   // staged epilogue: rows added to out0 (NULL: none); bytes from one to the next
+  const char *add_rows; const int32_t *add_idx; int add_pitch, add_stage_bytes;   // ADD: the rows, bytes from one to the next, bytes of a ring stage
   float *scores; const float *att_src; const float *att_dst; int heads, head_dim;  // GAT: scores [M, 2*heads]
   int *status;                    // set to 1 if a bounded wait gave up
   int tma_store;                  // 1: the epilogue stages each output tile in shared memory and writes it with TMA stores
@@ -218,8 +218,13 @@ struct TcParams {
   int no_loads;                   // test hook: the producer issues no copies, so every wait runs out
 };
 
-template <bool TF32>
-__global__ void __launch_bounds__(TF32 ? TC_THREADS_TF32 : TC_THREADS_BF16, 1)
+// ADD (bf16): four more warps gather a row per row of the tile into a ring in shared memory, copied asynchronously and ahead of
+// the product, and the epilogue adds it (learned messages: the source part of every edge's message).  The copies of up to four
+// tiles are in flight; with the epilogue's own loads in their place the kernel waited for them: 16M edges, 64 columns, whole layer 2.16 -> 1.95 ms.
+constexpr int TC_ADD_STAGES = 4;
+constexpr int TC_THREADS_ADD = TC_THREADS_BF16 + 128;
+template <bool TF32, bool ADD>
+__global__ void __launch_bounds__(TF32 ? TC_THREADS_TF32 : (ADD ? TC_THREADS_ADD : TC_THREADS_BF16), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_x2,
                const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_o0,
                const __grid_constant__ CUtensorMap map_o1, const TcParams p) {
@@ -236,7 +241,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
   unsigned char *smem_b = base;
   unsigned char *smem_a = base + b_bytes;   // b_bytes is a multiple of 1024 (nbc is a multiple of 16)
   unsigned char *smem_out = smem_a + (size_t)p.stages * a_tile_bytes;   // output staging panels (TMA-store epilogue), 1024-byte aligned
-  uint64_t *bars = reinterpret_cast<uint64_t *>(smem_out + (size_t)p.out_panels * p.epi_groups * a_tile_bytes);
+  unsigned char *smem_add = smem_out + (size_t)p.out_panels * p.epi_groups * a_tile_bytes;   // ADD: ring of gathered rows, panels like the output's
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem_add + (ADD ? (size_t)TC_ADD_STAGES * p.add_stage_bytes : 0));
   uint64_t *full = bars;                    // [stages]  TMA landed
   uint64_t *empty = bars + p.stages;        // [stages]  the stage's readers are done (bf16: its MMAs; fp32: the split warps)
   uint64_t *ready = bars + 2 * p.stages;    // [TC_TSTAGES_MAX]  (fp32 mode) hi / lo parts written to TMEM
@@ -244,7 +250,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
   uint64_t *b_full = a_free + TC_TSTAGES_MAX;  // [1]
   uint64_t *acc_full = b_full + 1;          // [2]
   uint64_t *acc_empty = acc_full + 2;       // [2]
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
+  uint64_t *add_full = acc_empty + 2;       // [TC_ADD_STAGES]  (ADD) the tile's rows have landed
+  uint64_t *add_empty = add_full + (ADD ? TC_ADD_STAGES : 0);   // [TC_ADD_STAGES]  (ADD) the epilogue has read them
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(add_empty + (ADD ? TC_ADD_STAGES : 0));
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   // per-column constants of this CTA's columns, 16-byte aligned: bias (0 where none applies), GAT attention vectors
   float *bias_s = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(tmem_slot + 2) + 15) & ~(uintptr_t)15);   // [nbc]
@@ -266,6 +274,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       mbar_init(&a_free[s], 1);
     }
     mbar_init(b_full, 1);
+    if (ADD)
+      for (int a = 0; a < TC_ADD_STAGES; ++a) {
+        mbar_init(&add_full[a], 128);
+        mbar_init(&add_empty[a], TC_EPI_WARPS / p.epi_groups);
+      }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
       mbar_init(&acc_empty[a], p.tma_store ? TC_EPI_WARPS / p.epi_groups : TC_EPI_WARPS);
@@ -415,35 +428,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       int last_u = -1;   // the last unit this warp owns (ownership: (unit0 + u) % n_sub == gsub)
       for (int u = n_units - 1; u >= 0; --u)
         if ((unit0 + u) % n_sub == gsub) { last_u = u; break; }
-      // Rows added to out0: the first pieces of this lane's row of the NEXT tile are fetched as soon as this tile's are used up,
-      // so that they are in flight across the barrier, the stores and the wait for the accumulator (fetched at the start of
-      // their own tile they made a product over 16M edges take 1.7 ms: ADD_NOTE).
-      constexpr int GP = TF32 ? 4 : 2;          // 16-byte pieces of a 16-column group
-      constexpr int PRE = 4, NPRE = PRE / GP;   // pieces fetched ahead: two groups of bf16, one of fp32
-      constexpr int ES = TF32 ? 4 : 2;
-      uint4 pre[PRE];
-      auto add_source = [&](int tile) -> int32_t {
-        const int64_t m = (int64_t)(tile / p.n_splits) * TC_BM + row_in_tile;
-        return p.add_rows && tile < n_tiles && m < p.M ? __ldcs(p.add_idx + m) : 0;
-      };
-      auto fetch_ahead = [&](int32_t src) {
-        const char *row = p.add_rows + (int64_t)src * p.add_pitch;
-#pragma unroll
-        for (int u = 0; u < NPRE; ++u) {
-          const int unit = u * n_sub + (gsub + n_sub - unit0 % n_sub) % n_sub;   // the (u + 1)-th unit that this warp owns
-          const int at = (col_base + unit * 16) * ES;
-#pragma unroll
-          for (int q = 0; q < GP; ++q) {
-            pre[u * GP + q] = make_uint4(0u, 0u, 0u, 0u);
-            if (unit < n_units && at + q * 16 < p.add_pitch) pre[u * GP + q] = __ldg(reinterpret_cast<const uint4 *>(row + at) + q);
-          }
-        }
-      };
-      int32_t src_c = 0;
-      if (p.add_rows) {
-        src_c = add_source((int)blockIdx.x + group * (int)gridDim.x);
-        fetch_ahead(src_c);
-      }
       int it = 0;   // tiles of this CTA so far: tile `it` uses accumulator it % 2, for the (it / 2)-th time
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
         if (G == 2 && (it & 1) != group) continue;
@@ -451,11 +435,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
         acc_phase = ((uint32_t)it >> 1) & 1u;
         const int m0 = (tile / p.n_splits) * TC_BM;
         const int64_t m = (int64_t)m0 + row_in_tile;
-        const int next = tile + G * (int)gridDim.x;   // this group's next tile
-        const int32_t src_n = add_source(next);       // its row's source, in flight during this tile
-        const char *add_row = p.add_rows + (int64_t)src_c * p.add_pitch;   // (used with rows to add only)
-        int nth = 0;   // units of this warp so far
         ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, p.spin_limit, IT_TC_EPI_BACKOFF);
+        if (ADD && ok) ok = mbar_wait(&add_full[it % TC_ADD_STAGES], (uint32_t)(it / TC_ADD_STAGES) & 1u, abort_flag, p.spin_limit);
         if (issuer) tma_store_wait_read();   // the stores of this group's previous tile have read the staging tile
         // one decision for all warps of the group (they meet at named barriers below, so none may leave alone)
         __syncwarp();
@@ -510,26 +491,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
                 const float4 b4 = bs[i];
                 v[4 * i] += b4.x; v[4 * i + 1] += b4.y; v[4 * i + 2] += b4.z; v[4 * i + 3] += b4.w;
               }
-              if (p.add_rows) {
+              if constexpr (ADD) {   // round the product as if it had been stored, add the gathered row's 16 columns
+                const uint32_t row = smem_u32(smem_add) + (uint32_t)(it % TC_ADD_STAGES) * (uint32_t)p.add_stage_bytes + (uint32_t)row_in_tile * 128u;
 #pragma unroll
-                for (int q = 0; q < GP; ++q) {
-                  uint4 x = make_uint4(0u, 0u, 0u, 0u);
-                  if (nth == 0) x = pre[q];
-                  else if (NPRE > 1 && nth == 1) x = pre[NPRE > 1 ? GP + q : q];
-                  else if (gc * ES + q * 16 < p.add_pitch) x = __ldg(reinterpret_cast<const uint4 *>(add_row + gc * ES) + q);
-                  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+                for (int q = 0; q < 2; ++q) {
+                  const uint32_t ch = (uint32_t)(c >> 3) + q;   // 16-byte piece of the row
+                  uint32_t w[4];
+                  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                               : "r"(row + (ch >> 3) * (uint32_t)a_tile_bytes + (((ch & 7u) ^ swz) << 4)) : "memory");
 #pragma unroll
                   for (int i = 0; i < 4; ++i) {
-                    if (TF32) {
-                      v[4 * q + i] += __uint_as_float(w[i]);
-                    } else {
-                      const __nv_bfloat162 h = __floats2bfloat162_rn(v[8 * q + 2 * i], v[8 * q + 2 * i + 1]);
-                      v[8 * q + 2 * i] = __low2float(h) + __uint_as_float(w[i] << 16);
-                      v[8 * q + 2 * i + 1] = __high2float(h) + __uint_as_float(w[i] & 0xffff0000u);
-                    }
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(v[8 * q + 2 * i], v[8 * q + 2 * i + 1]);
+                    v[8 * q + 2 * i] = __low2float(h) + __uint_as_float(w[i] << 16);
+                    v[8 * q + 2 * i + 1] = __high2float(h) + __uint_as_float(w[i] & 0xffff0000u);
                   }
                 }
-                ++nth;
               }
               if (p.act0 == IT_ACT_RELU) {
 #pragma unroll
@@ -572,9 +548,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           __syncwarp();
           if (lane == 0) mbar_arrive(&acc_empty[acc]);
         }
-        if (p.add_rows) {
-          src_c = src_n;
-          if (next < n_tiles) fetch_ahead(src_c);
+        if (ADD) {   // the gathered rows have been read
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&add_empty[it % TC_ADD_STAGES]);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the TMA store's reads
         epi_bar_sync(G, group);
@@ -724,6 +700,45 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       if (!released) release();   // a warp that owns no columns of this CTA still has to sign off
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
+  } else if (ADD) {
+    // ------------------------------------------------------------------ gather the rows that the epilogue adds
+    // A warp copies 32 rows of the tile, 16 bytes per lane: pieces / row lanes per row, whole rows side by side; piece ch of row
+    // r lands where the epilogue's lane of row r looks for it: panel ch / 8, position (ch % 8) ^ (r % 8).
+    const int gw = warp - (TC_THREADS_BF16 >> 5);
+    const int pieces = p.add_pitch >> 4;   // of a row; 1 .. 16
+    const bool even = 32 % pieces == 0;
+    const int r_first = lane / pieces, r_step = 32 / pieces, ch_mine = lane % pieces;
+    int32_t src = 0;
+    auto source = [&](int tile) -> int32_t {
+      const int64_t m = (int64_t)(tile / p.n_splits) * TC_BM + gw * 32 + lane;
+      return tile < n_tiles && m < p.M ? __ldcs(p.add_idx + m) : 0;   // (rows past the end: row 0, not stored)
+    };
+    src = source(blockIdx.x);
+    bool ok = true;
+    int it = 0;
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
+      const int s = it % TC_ADD_STAGES;
+      const int32_t next = source(tile + gridDim.x);
+      ok = mbar_wait(&add_empty[s], ((uint32_t)(it / TC_ADD_STAGES) & 1u) ^ 1u, abort_flag, p.spin_limit, IT_TC_TMA_BACKOFF);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const uint32_t stage = smem_u32(smem_add) + (uint32_t)s * (uint32_t)p.add_stage_bytes;
+      auto copy = [&](int r, int ch) {
+        const int row = gw * 32 + r;
+        const uint32_t from = (uint32_t)__shfl_sync(0xffffffffu, src, r);
+        const uint32_t to = stage + (uint32_t)(ch >> 3) * (uint32_t)a_tile_bytes + (uint32_t)row * 128u + (uint32_t)(((ch & 7) ^ (row & 7)) << 4);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to), "l"(p.add_rows + (uint64_t)from * (uint32_t)p.add_pitch + ch * 16) : "memory");
+      };
+      if (even) {   // the same piece of a row every time
+#pragma unroll 8
+        for (int r = r_first; r < 32; r += r_step) copy(r, ch_mine);
+      } else {
+        for (int q = lane; q < 32 * pieces; q += 32) copy(q / pieces, q % pieces);
+      }
+      asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&add_full[s])) : "memory");
+      src = next;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");   // no copy of this CTA may be in flight when it exits
   } else {
     // ------------------------------------------------------------------ fp32 mode: split A into hi + lo, into TMEM
     // Thread = one row of the tile (TMEM lane quarter = warp index % 4).  The row's 128 bytes of the k-block are
@@ -1232,12 +1247,13 @@ namespace {
 struct TcShape { int b_bytes, const_bytes, out_panels, epi_groups, stages; bool staged; };
 
 // How a product's shared memory is used.
-bool tc_shape(const it_gemm_args &a, const it_tc_cols &cols, int KB, bool want_scores, TcShape *out) {
+bool tc_shape(const it_gemm_args &a, const it_tc_cols &cols, int KB, bool want_scores, bool add, TcShape *out) {
   const bool tf32 = a.x_dtype == IT_F32;
   const int n_splits = cols.n_splits, nbc = cols.nbc, n0p = cols.n0p, n1p = cols.n1p;
   const int b_bytes = (tf32 ? 2 : 1) * KB * nbc * TC_KBLOCK_BYTES;
   const int stage_bytes = TC_BM * TC_KBLOCK_BYTES;             // one operand tile (fp32 mode: the raw tile)
-  const int const_bytes = nbc * 4 * (want_scores ? 3 : 1);          // bias (+ attention vectors) of this CTA's columns
+  const int add_bytes = add ? TC_ADD_STAGES * ((a.n0 * 2 + 127) / 128) * stage_bytes + 2 * TC_ADD_STAGES * 8 : 0;   // ring of rows to add, its barriers
+  const int const_bytes = nbc * 4 * (want_scores ? 3 : 1) + add_bytes;          // bias (+ attention vectors) of this CTA's columns
   // Staged epilogue (TMA stores): possible when, for every column split, the out0 columns and the out1 columns of
   // the CTA are whole 128-byte panels or reach the end of their output (the copy clips what lies past it), and three operand
   // stages still fit beside the staging tile (three stages already give the time of eight).
@@ -1274,7 +1290,8 @@ bool it_tc_adds_rows(const it_gemm_args &a) {
   it_tc_cols cols;
   TcShape sh;
   const int bk = TC_KBLOCK_BYTES / (a.x_dtype == IT_F32 ? 4 : 2), KB = (a.K1 + bk - 1) / bk + ((a.X2 ? a.K2 : 0) + bk - 1) / bk;
-  return it_tc_supported(a, 1, a.n0, false) && it_tc_columns(a, a.n0, false, &cols) && tc_shape(a, cols, KB, false, &sh) && sh.staged && a.n1 == 0;
+  return a.x_dtype == IT_BF16 && a.n1 == 0 && a.n0 <= 128 && it_tc_supported(a, 1, a.n0, false) && it_tc_columns(a, a.n0, false, &cols) &&
+         cols.n_splits == 1 && tc_shape(a, cols, KB, false, true, &sh) && sh.staged;
 }
 
 // B: weights prepared by it_launch_prep_weights_tc.  a.B / a.NB / a.out2 of the generic args are ignored:
@@ -1293,7 +1310,7 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   IT_REQUIRE(it_tc_columns(a, head_dim, scores != nullptr, &cols), IT_ERR_UNSUPPORTED, "tensor-core apply: cannot tile %d columns with K = %d", a.n0 + a.n1, K);
   const int NB = cols.NB, n_splits = cols.n_splits, nbc = cols.nbc, n0p = cols.n0p, n1p = cols.n1p;
   TcShape sh;
-  IT_REQUIRE(tc_shape(a, cols, KB, scores != nullptr, &sh), IT_ERR_UNSUPPORTED, "tensor-core apply: no room for two operand stages");
+  IT_REQUIRE(tc_shape(a, cols, KB, scores != nullptr, a.add_rows != nullptr, &sh), IT_ERR_UNSUPPORTED, "tensor-core apply: no room for two operand stages");
   IT_REQUIRE(!a.add_rows || sh.staged, IT_ERR_UNSUPPORTED, "tensor-core apply: rows are added by the staged epilogue only");
   const int b_bytes = sh.b_bytes, stage_bytes = TC_BM * TC_KBLOCK_BYTES, const_bytes = sh.const_bytes, out_panels = sh.out_panels;
   const int epi_groups = sh.epi_groups, stages = sh.stages, s0 = a.dt0 == IT_BF16 ? 2 : 4, s1 = a.dt1 == IT_BF16 ? 2 : 4;
@@ -1318,7 +1335,7 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   p.kb1 = kb1; p.kb2 = kb2; p.NB = NB; p.stages = stages; p.tstages = tstages;
   p.n0 = n0p; p.n0_real = a.n0; p.out0 = a.out0; p.out0_bf16 = a.dt0 == IT_BF16; p.bias0 = a.bias0; p.act0 = a.act0;
   p.n1 = n1p; p.n1_real = a.n1; p.out1 = a.out1; p.out1_bf16 = a.dt1 == IT_BF16;
-  p.add_rows = (const char *)a.add_rows; p.add_idx = a.add_idx; p.add_pitch = a.n0 * s0;
+  p.add_rows = (const char *)a.add_rows; p.add_idx = a.add_idx; p.add_pitch = a.n0 * s0; p.add_stage_bytes = (p.add_pitch + 127) / 128 * stage_bytes;
   p.scores = scores; p.att_src = att_src; p.att_dst = att_dst; p.heads = heads; p.head_dim = head_dim > 0 ? head_dim : 1;
   p.status = status;
   p.tma_store = staged ? 1 : 0; p.out_panels = out_panels; p.epi_groups = epi_groups;
@@ -1332,11 +1349,15 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
                                      (scores ? 8.0 * heads : 0.0)) + (double)K * (a.n0 + a.n1) * xs;
   const double flops = 2.0 * (double)a.M * K * (a.n0 + a.n1);
   if (tf32) {
-    IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<true>, dim3((unsigned)grid), dim3(TC_THREADS_TF32), smem, st, m1, m2, mb, mo0, mo1, p)));
+    IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<true, false>, dim3((unsigned)grid), dim3(TC_THREADS_TF32), smem, st, m1, m2, mb, mo0, mo1, p)));
+  } else if (a.add_rows) {
+    IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    IT_LAUNCH(IT_K_GEMM_TC, bytes + (double)a.M * (4.0 + a.n0 * 2.0), flops, st,
+              IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<false, true>, dim3((unsigned)grid), dim3(TC_THREADS_ADD), smem, st, m1, m2, mb, mo0, mo1, p)));
   } else {
-    IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<false>, dim3((unsigned)grid), dim3(TC_THREADS_BF16), smem, st, m1, m2, mb, mo0, mo1, p)));
+    IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<false, false>, dim3((unsigned)grid), dim3(TC_THREADS_BF16), smem, st, m1, m2, mb, mo0, mo1, p)));
   }
   IT_CUDA_TRY(cudaGetLastError());
   return IT_OK;

@@ -261,7 +261,7 @@ struct it_gemm_args {
   int n0; void *out0; it_dtype dt0; const float *bias0; it_act act0;
   int n1; void *out1; it_dtype dt1;
   void *out2;
-  // tensor-core path, staged stores only (it_tc_adds_rows): out0[m, :] = act0(round(C + bias0) + add_rows[add_idx[m], :]), rows of
+  // tensor-core path, the shapes of it_tc_adds_rows: out0[m, :] = act0(round(C + bias0) + add_rows[add_idx[m], :]), rows of
   // n0 elements of dt0; `round` to dt0, as if the product had been stored and read back
   const void *add_rows; const int32_t *add_idx;
   uint32_t spin_limit;   // tensor-core path: polls after which a barrier wait gives up (0 = the default)
