@@ -4,7 +4,8 @@
 // in the warp that finishes the last of them.  The record of a warp's next-but-one row and the ids of its next row are in
 // flight while a row is reduced.
 // What bounds it: the dependent trips record -> ids -> source rows out of the L2 and the launch itself.  A layer of 10k
-// vertices and 100k edges took five launches (a memset, three kernels by row length, empty rows, combine).  SMALL_MEASURED
+// vertices and 100k edges took five launches (a memset, three kernels by row length, empty rows, combine).  Measured: two fp32
+// layers of that graph 150 -> 40 us; the layers of a GAT on 30k vertices and 420k edges 184 -> 84 us.
 //
 // Included by gather_rows.cuh and gat_rows.cuh.
 #pragma once
