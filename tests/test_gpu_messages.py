@@ -38,6 +38,17 @@ def test_message_shapes(dtype, dims):
     check_against_oracle(w, got, label=(dtype, dims))
 
 
+@pytest.mark.parametrize("act", ["none", "relu", "elu"])
+@pytest.mark.parametrize("fm", [8, 24, 72, 120, 128])
+def test_messages_finished_in_the_product(fm, act):
+    """bf16 messages leave the per-edge product finished: widths that are no multiple of 16 columns or of a 128-byte panel, every
+    activation, a last tile with few rows (oracle and metric of the other layers: one more rounding to bf16 is in both)."""
+    layer = make_msg_layer(9, "sum", "none", 32, fm, 32, "bf16", act_edge=act, edge_dim=16)
+    w = small_workload(10, 701, 13, "bf16", [layer], hubs=(300, 41), threshold=128, edge_dim=16)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(fm, act))
+
+
 def test_message_layers_stack_with_plain_layers():
     layers = [make_msg_layer(5, "mean", "relu", 32, 64, 32, "f32", act_edge="relu", edge_dim=8),
               make_sage_layer(6, "sum", "relu", 32, 32, "f32", edge_dim=8),
