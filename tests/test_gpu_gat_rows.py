@@ -23,6 +23,19 @@ def test_heads_widths_and_row_lengths(dtype, heads, hd, threshold):
     check_against_oracle(w, got, label=(dtype, heads, hd, threshold))
 
 
+@pytest.mark.parametrize("n", [700, (1 << 17) + 77])   # one kernel per layer, and kernels by row length
+@pytest.mark.parametrize("slope", [-0.3, 0.0])
+@pytest.mark.parametrize("dtype,heads,hd", [("f32", 4, 4), ("f32", 2, 16), ("bf16", 4, 32), ("bf16", 8, 8)])
+def test_any_leaky_slope(dtype, heads, hd, slope, n):
+    """A slope that is zero or negative: places of a round without an edge must stay out of the softmax (rows of 1 to 33 edges
+    leave every number of such places)."""
+    layer = make_gat_layer(17, "none", 32, heads, hd, dtype)
+    layer.leaky_slope = slope
+    w = small_workload(18, n, 9, dtype, [layer], hubs=tuple(range(1, 34)) + (300, 65), p_zero=0.3)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(dtype, heads, hd, slope, n), exact=False)
+
+
 def test_bias_need_not_be_aligned():
     layer = make_gat_layer(13, "none", 32, 4, 16, "f32")
     w = small_workload(14, 300, 12, "f32", [layer], hubs=(300, 40))
