@@ -60,7 +60,9 @@ __global__ void validate_indptr_kernel(IndptrView ip, int64_t n, int64_t e, int 
 }
 
 // Four ids per load (`head` ids up to the first 16-byte boundary and the last few on their own): bound by reading them.
+// Runs after validate_indptr_kernel and reads no id of an indptr that failed: `e` is then no count of ids that the caller holds.
 __global__ void __launch_bounds__(256) validate_indices_kernel(const int32_t *__restrict__ idx, int64_t e, int64_t n, int head, int *flags) {
+  if (*reinterpret_cast<volatile int *>(flags) != 0) return;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const uint32_t top = (uint32_t)n;   // n < 2^31: a negative id is a large unsigned one
   bool bad = false;
@@ -653,7 +655,7 @@ static it_status create_impl(int64_t n, int64_t n_src, int64_t e, const void *in
   int h_flags = 0;
   if (ce == cudaSuccess) {
     IT_LAUNCH(IT_K_VALIDATE, 0, 0, st, validate_indptr_kernel<<<(unsigned)((n + 1 + 255) / 256), 256, 0, st>>>(ip, n, e, d_status));
-    if (e > 0) {   // the caller vouches for e source ids, whatever indptr says
+    if (e > 0) {
       const int64_t want = (e / 4 + 255) / 256, cap = (int64_t)IT_NUM_SMS_FALLBACK * 8;
       int head = (int)(((16 - ((uintptr_t)indices & 15)) & 15) / 4);
       if (head > e) head = (int)e;

@@ -116,6 +116,16 @@ def test_bad_csr_is_rejected_with_a_status(kind):
     assert torch.ones(4, device="cuda").sum().item() == 4
 
 
+@pytest.mark.parametrize("extra", [1, 1 << 30])
+def test_no_id_is_read_where_indptr_does_not_hold_the_edges(extra):
+    """n_edges above what indptr says: refused before any of the ids that are not there is read."""
+    ip, ix = random_csr(1, 200, 5)
+    with pytest.raises(B.ItError) as ei:
+        B.it_graph_create(torch.from_numpy(ip).cuda(), torch.from_numpy(ix).cuda(), n_edges=ix.shape[0] + extra)
+    assert ei.value.status_name == "IT_ERR_BAD_GRAPH" and "source id" not in str(ei.value)
+    assert torch.ones(4, device="cuda").sum().item() == 4
+
+
 def test_invalid_arguments():
     ip, ix = random_csr(1, 20, 3)
     with pytest.raises(B.ItError) as ei:
