@@ -503,6 +503,7 @@ bool aligned16(const void *p) { return ((uintptr_t)p % 16) == 0; }
 it_status check_io(const it_graph *g, const void *in, size_t in_bytes, const void *out, size_t out_bytes) {
   IT_REQUIRE(g->n == 0 || g->list_meta != nullptr, IT_ERR_BAD_GRAPH,
              "the graph has no row split (an it_split_hubs call failed): call it_split_hubs again before a forward pass");
+  g->used = true;
   if (g->n == 0) return IT_OK;
   IT_REQUIRE(in != nullptr && out != nullptr, IT_ERR_INVALID_ARG, "input / output matrix is NULL");
   IT_REQUIRE(aligned16(in) && aligned16(out), IT_ERR_INVALID_ARG,
@@ -556,6 +557,7 @@ it_status check_stage(const it_graph *g, const it_layer_desc *layer, void *works
   IT_REQUIRE(g->n == 0 || g->list_meta != nullptr, IT_ERR_BAD_GRAPH,
              "the graph has no row split (an it_split_hubs call failed): call it_split_hubs again before a forward pass");
   IT_REQUIRE(workspace != nullptr && ((uintptr_t)workspace % 256) == 0, IT_ERR_WORKSPACE, "workspace is NULL or not 256-byte aligned");
+  g->used = true;
   return IT_OK;
 }
 

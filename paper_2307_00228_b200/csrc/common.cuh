@@ -2,6 +2,7 @@
 // the launch entry points of each kernel file).  sm_100a only.
 #pragma once
 
+#include <atomic>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -90,7 +91,7 @@ struct it_graph {
   // derived by the split (library-owned, device; all carved out of one allocation that is kept for the next split)
   char *slab = nullptr;
   size_t slab_bytes = 0;
-  bool slab_pooled = false;   // from the library's memory pool
+  mutable std::atomic<bool> used{false};   // the arrays of the present split have been handed out: to a forward pass or to the caller
   int64_t threshold = 0;
   int64_t n_rows = 0;           // R
   int64_t n_split_owners = 0;   // vertices with more than one shadow row

@@ -1,7 +1,6 @@
 // Graph ingest, validation, hub split into shadow rows, degree buckets.
 // Integer-only work; every array produced here is a pure function of (indptr, threshold)
 // and is built without atomics on data, so it is reproducible bit for bit.
-#include <mutex>
 #include <new>
 #include <type_traits>
 #include <stdarg.h>
@@ -412,65 +411,10 @@ __global__ void __launch_bounds__(PIECE_BINS) long_pieces_kernel(SplitParams p) 
 }
 
 // ----------------------------------------------------------------------------- host side
-// The derived arrays of graphs come from one memory pool per device.  cudaMalloc and cudaFree of a few hundred megabytes take
-// 0.4 ms each on an idle machine and have been seen to take tens of milliseconds on a busy one, against 0.5 ms of kernels for
-// a graph of 5M vertices (create + split: 2.5 -> 1.4 ms).  The pool keeps at most POOL_KEEP bytes between graphs: what is
-// freed beyond that goes back to the device at the next synchronisation, all of it when an allocation of the library fails.
-// Allocation and release are ordered by the driver and safe from any thread and stream.
-constexpr uint64_t POOL_KEEP = 512ull << 20;
-constexpr int POOL_DEVICES = 64;
-static std::mutex g_pool_mu;
-static cudaMemPool_t g_pools[POOL_DEVICES];
-
-static cudaMemPool_t device_pool(int device) {   // NULL: none (then plain allocations)
-  if (device < 0 || device >= POOL_DEVICES) return nullptr;
-  std::lock_guard<std::mutex> lk(g_pool_mu);
-  if (!g_pools[device]) {
-    int supported = 0;
-    if (cudaDeviceGetAttribute(&supported, cudaDevAttrMemoryPoolsSupported, device) != cudaSuccess || !supported) return nullptr;
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = device;
-    cudaMemPool_t pool;
-    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    uint64_t keep = POOL_KEEP;
-    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    g_pools[device] = pool;
-  }
-  return g_pools[device];
-}
-
-// `st` is synchronised by the caller before the memory is used from another stream.
-static cudaError_t slab_alloc(it_graph *g, size_t bytes, cudaStream_t st) {
-  cudaMemPool_t pool = device_pool(g->device);
-  g->slab_pooled = pool != nullptr;
-  if (!pool) return cudaMalloc(&g->slab, bytes);
-  cudaError_t e = cudaMallocFromPoolAsync((void **)&g->slab, bytes, pool, st);
-  if (e == cudaErrorMemoryAllocation) {
-    cudaGetLastError();
-    cudaDeviceSynchronize();
-    cudaMemPoolTrimTo(pool, 0);
-    e = cudaMallocFromPoolAsync((void **)&g->slab, bytes, pool, st);
-  }
-  return e;
-}
-
-// Nothing on the device may still use the graph's arrays: waits for it, as cudaFree does.
+// Nothing on the device may still use the graph's arrays: cudaFree waits for it.  (It may also be called while another thread
+// captures a stream, which a synchronisation of the device may not.)
 static void slab_free(it_graph *g) {
-  if (!g->slab) return;
-  if (g->slab_pooled) {
-    int current = -1;
-    cudaGetDevice(&current);
-    if (current != g->device) cudaSetDevice(g->device);
-    cudaDeviceSynchronize();
-    // released for good before the next allocation asks, on whichever stream: else the pool would grow by another copy
-    cudaFreeAsync(g->slab, cudaStreamPerThread);
-    cudaStreamSynchronize(cudaStreamPerThread);
-    if (current != g->device && current >= 0) cudaSetDevice(current);
-  } else {
-    cudaFree(g->slab);
-  }
+  cudaFree(g->slab);
   g->slab = nullptr;
   g->slab_bytes = 0;
 }
@@ -509,8 +453,9 @@ static size_t carve_split(SplitParams &p, char *slab, int64_t R, int64_t L, int6
 }
 
 static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
-  // the arrays of the previous split are written over: forward passes on any stream that still read them come first
-  if (g->list_meta) IT_CUDA_TRY(cudaDeviceSynchronize());
+  // The arrays of the previous split are written over.  Where nothing but that split itself, which waited for its stream, has
+  // used them this needs no wait; else what still reads them, on any stream, comes first.
+  if (g->used.exchange(false)) slab_free(g);
   forget_split(g);
   g->threshold = T > 0 ? T : 0;
   const int64_t n = g->n;
@@ -546,7 +491,7 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
     if (bytes <= g->slab_bytes) return IT_OK;
     slab_free(g);
     bytes += bytes / 8;   // room for the few more rows of another threshold
-    IT_CUDA_TRY(slab_alloc(g, bytes, st));
+    IT_CUDA_TRY(cudaMalloc(&g->slab, bytes));
     g->slab_bytes = bytes;
     return IT_OK;
   };
@@ -717,6 +662,7 @@ extern "C" it_status it_graph_get_split(const it_graph *g, int64_t *n_rows, cons
                                         const int64_t **bucket_offsets, const int32_t **bucket_rows,
                                         int32_t *n_buckets, int64_t *bucket_bounds) {
   IT_REQUIRE(g != nullptr, IT_ERR_INVALID_ARG, "graph is NULL");
+  g->used = true;
   if (n_rows) *n_rows = g->n_rows;
   if (shadow_indptr) *shadow_indptr = g->shadow_indptr;
   if (shadow_owner) *shadow_owner = g->shadow_owner;

@@ -126,6 +126,59 @@ def test_no_id_is_read_where_indptr_does_not_hold_the_edges(extra):
     assert torch.ones(4, device="cuda").sum().item() == 4
 
 
+def test_set_up_while_another_thread_captures():
+    """Set-up, a forward pass, another split and the end of a graph on one thread, while another thread captures a stream: neither may
+    disturb the other (a wait for the whole device would break the capture, and fail itself)."""
+    import threading
+    from gpu_util import make_sage_layer
+    from paper_2307_00228_b200 import host
+    ip, ix = random_csr(3, 400, 30)
+    ip, ix = torch.from_numpy(ip).cuda(), torch.from_numpy(ix).cuda()
+    layer = host.layer_to_device(make_sage_layer(4, "max", "none", 16, 16, "f32"), "f32")
+    x, out, ws = torch.randn(400, 16, device="cuda"), torch.empty(400, 16, device="cuda"), torch.empty(4 << 20, dtype=torch.uint8, device="cuda")
+    side, capturing = torch.cuda.Stream(), torch.cuda.Stream()
+
+    def all_of_it():
+        g = B.it_graph_create(ip, ix, stream=side)
+        B.it_split_hubs(g, 8, stream=side)
+        B.it_layer_forward(g, layer, x, out, ws, stream=side)
+        rows, _ = B.it_split_hubs(g, 16, stream=side)
+        B.it_layer_forward(g, layer, x, out, ws, stream=side)
+        B.it_graph_destroy(g)
+        return rows
+
+    want_rows = all_of_it()
+    want = out.clone()
+    y = torch.ones(64, device="cuda")
+    torch.cuda.synchronize()
+    graph, begun, go_on, failed = torch.cuda.CUDAGraph(), threading.Event(), threading.Event(), []
+
+    def capture():
+        try:
+            with torch.cuda.graph(graph, stream=capturing, capture_error_mode="thread_local"):
+                y.mul_(2)
+                begun.set()
+                go_on.wait(60)
+                y.add_(1)
+        except Exception as e:   # noqa: BLE001
+            failed.append(e)
+            begun.set()
+
+    t = threading.Thread(target=capture)
+    t.start()
+    begun.wait(60)
+    try:
+        rows = all_of_it()
+    finally:
+        go_on.set()
+        t.join()
+    assert not failed, failed
+    graph.replay()
+    torch.cuda.synchronize()
+    assert rows == want_rows and torch.equal(out, want)
+    assert bool((y == 3).all())
+
+
 def test_invalid_arguments():
     ip, ix = random_csr(1, 20, 3)
     with pytest.raises(B.ItError) as ei:
