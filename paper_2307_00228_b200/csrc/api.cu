@@ -1,7 +1,7 @@
 // it_layer_forward / it_infer / it_workspace_bytes: argument checks, workspace carving and the
 // launch sequence of one layer.  All arithmetic lives in the kernels of the other files.
 #include <mutex>
-#include <vector>
+#include <new>
 
 #include "common.cuh"
 
@@ -152,19 +152,34 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
 // The weight matrices of a whole call, prepared by one launch before its first layer (and the words that the gathers need
 // zeroed with it): the call's layers are gone through twice, first recording their products, then launching.
 struct Prepared {
-  std::vector<it_prep_tc> m;
-  size_t next = 0;
+  static constexpr int PER_LAYER = 3, INLINE = 8 * PER_LAYER;   // products of a layer; longer models take memory from the heap
+  it_prep_tc few[INLINE];
+  it_prep_tc *m = few;
+  size_t count = 0, next = 0;
   bool recording = true;
   char *base = nullptr;
   size_t used = 0, cap = 0;
+  Prepared() = default;
+  Prepared(const Prepared &) = delete;
+  Prepared &operator=(const Prepared &) = delete;
+  ~Prepared() { if (m != few) delete[] m; }
+  it_status reserve(int32_t n_layers) {
+    const size_t want = (size_t)n_layers * PER_LAYER;
+    if (want <= INLINE) return IT_OK;
+    m = new (std::nothrow) it_prep_tc[want];
+    if (m) return IT_OK;
+    m = few;
+    it_set_error("host allocation failed");
+    return IT_ERR_OOM;
+  }
   // where the product's prepared weights lie (NULL: not recorded, to be prepared on its own)
   void *place(it_prep_tc p) {
-    if (!recording) return next < m.size() ? m[next++].B : nullptr;
+    if (!recording) return next < count ? m[next++].B : nullptr;
     const size_t bytes = it_align_up(it_prep_tc_bytes(p));
     if (used + bytes > cap) return nullptr;   // (not with prep_bytes_of() of every layer)
     p.B = base + used;
     used += bytes;
-    m.push_back(p);
+    m[count++] = p;
     return p.B;
   }
 };
@@ -488,7 +503,7 @@ it_status launch_prepared(const it_graph *g, char *ws, const it_layer_desc *firs
   prep.recording = false;
   int *words = it_done_words(reinterpret_cast<int *>(ws + plan_layer(g, first).off_counters));   // the same place for every layer
   const size_t n_words = it_small_graph(g) ? (size_t)g->n_long : 0;
-  return it_launch_prep_weights_tc(prep.m.data(), (int)prep.m.size(), words, n_words, st);
+  return it_launch_prep_weights_tc(prep.m, (int)prep.count, words, n_words, st);
 }
 
 bool overlaps(const void *a, size_t na, const void *b, size_t nb) {
@@ -723,6 +738,7 @@ extern "C" it_status it_infer(const it_graph *g, const it_layer_desc *layers, in
   char *ws = (char *)workspace;
   Prepared prep;
   prep.base = ws + w.off_prep; prep.cap = w.prep_bytes;
+  IT_TRY(prep.reserve(n_layers));
   IT_TRY(infer_layers(g, layers, n_layers, x, out, ws, w, prep, (cudaStream_t)stream));
   IT_TRY(launch_prepared(g, ws, layers, prep, (cudaStream_t)stream));
   return infer_layers(g, layers, n_layers, x, out, ws, w, prep, (cudaStream_t)stream);

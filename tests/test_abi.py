@@ -38,6 +38,16 @@ def test_binding_has_the_same_names_and_fails_loudly_without_the_library(monkeyp
         binding.lib()
 
 
+def test_forward_calls_allocate_without_throwing():
+    """Errors are return codes: the file of the layer calls may not reach an operator new that throws across the C boundary."""
+    import subprocess
+    from paper_2307_00228_b200 import build
+    build.build()
+    names = subprocess.check_output(["nm", "--undefined-only", os.path.join(build.OBJ_DIR, "api.o")], text=True)
+    assert "_ZnamRKSt9nothrow_t" in names
+    assert not re.search(r"\b(_Znwm|_Znam|_ZSt20__throw_length_errorPKc|_ZSt17__throw_bad_allocv)\b", names), names
+
+
 def test_status_strings():
     from paper_2307_00228_b200 import binding
     assert [binding.it_status_string(i) for i in range(8)] == binding.STATUS_NAMES

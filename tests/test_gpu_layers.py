@@ -165,6 +165,20 @@ def test_multi_layer_infer_matches_layer_by_layer_and_oracle(dtype):
     assert torch.equal(h, d.out)
 
 
+def test_a_model_of_many_layers():
+    """More products than a call keeps room for without the heap: as layer by layer."""
+    layers = [make_sage_layer(60 + i, "mean", "relu", 16, 16, "f32") for i in range(30)]
+    w = small_workload(61, 300, 6, "f32", layers, hubs=(200,), threshold=64)
+    _, d = run_device(w)
+    h = d.x
+    for lay in d.layers:
+        o = torch.empty_like(d.out)
+        B.it_layer_forward(d.graph, lay, h, o, d.workspace)
+        h = o
+    torch.cuda.synchronize()
+    assert torch.equal(h, d.out)
+
+
 def test_run_to_run_results_are_bit_identical():
     """The paper's consistency requirement: the same prediction at every run."""
     layers = [make_sage_layer(15, "sum", "relu", 64, 64, "f32", weights=True), make_sage_layer(16, "mean", "none", 64, 16, "f32")]
