@@ -27,6 +27,7 @@ void it_set_error(const char *fmt, ...);
     if (_e != cudaSuccess) {                                                         \
       it_set_error("%s failed: %s (%s:%d)", #expr, cudaGetErrorString(_e), __FILE__, \
                    __LINE__);                                                        \
+      cudaGetLastError(); /* reported here, not by a later call */                   \
       return (_e == cudaErrorMemoryAllocation) ? IT_ERR_OOM : IT_ERR_CUDA;           \
     }                                                                                \
   } while (0)

@@ -416,6 +416,7 @@ it_status launch_gat_small(const it_gat_args &a, StreamParams p, const GatPolicy
   // live on: 30k vertices, two layers 84 us, started early 98.)
   IT_LAUNCH(IT_K_GAT_SMALL, bytes, 0, st,
             gat_small_kernel<T, LPR, H><<<sh.blocks, THREADS, smem, st>>>(p, q, pol, piece_params(g, it_done_words(a.counters)), sh));
+  IT_CUDA_TRY(cudaGetLastError());
   return IT_OK;
 }
 

@@ -222,6 +222,7 @@ static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
                           (double)g->n_long * a.dim * (a.dtype == IT_F32 ? 4.0 : 2.0);
     if (a.dtype == IT_F32) IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, combine_kernel<float><<<blocks, GATHER_THREADS, 0, st>>>(c));
     else IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, combine_kernel<__nv_bfloat16><<<blocks, GATHER_THREADS, 0, st>>>(c));
+    IT_CUDA_TRY(cudaGetLastError());
   }
   return IT_OK;
 }
