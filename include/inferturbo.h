@@ -305,8 +305,11 @@ it_status it_aggregate_finish(int64_t n, int32_t dim, it_dtype dtype, const floa
  * this call is ever made, which is why the limit is modest.
  *
  * Same arguments, results and errors as it_layer_forward, minus the workspace.  A layer whose
- * scratch need (it_workspace_bytes of that one layer) exceeds IT_STATIC_WORKSPACE_BYTES is
- * rejected with IT_ERR_WORKSPACE and nothing is launched.  The call itself performs no
+ * tables and largest prepared weight matrix exceed IT_STATIC_WORKSPACE_BYTES is rejected with
+ * IT_ERR_WORKSPACE and nothing is launched; the error text gives the need, which is below
+ * it_workspace_bytes of that one layer (that call has room for all weights at once).  Where only the
+ * partial rows of long vertices do not fit, those vertices are reduced whole, one block each: slower,
+ * and sums are taken in another order.  The call itself performs no
  * cudaMalloc / cudaFree and calls no allocating routine; for that reason it refuses to run
  * (IT_ERR_UNSUPPORTED) while it_profile_begin instrumentation is active, since that creates
  * CUDA events on demand.  (it_graph_create / it_split_hubs do allocate: build the graph

@@ -80,21 +80,57 @@ int agg_dim_of(const it_layer_desc *L) {
   }
 }
 
-LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
+// What the weights of a layer's dense products take when prepared: the largest, and all of them.
+struct WeightBytes { size_t largest, sum; };
+WeightBytes weight_bytes(const it_graph *g, const it_layer_desc *L) {
+  WeightBytes w{0, 0};
+  const it_dtype dt = L->feat_dtype;
+  const size_t bk = (size_t)(128 / it_dtype_size(dt));   // a k-block of an operand row: 128 bytes
+  auto product = [&](int64_t M, int K1, int K2, int n0, int n1, int heads) {
+    it_gemm_args a{};
+    a.M = M; a.x_dtype = dt; a.X1 = g; a.K1 = K1; a.X2 = K2 > 0 ? g : nullptr; a.K2 = K2; a.n0 = n0; a.n1 = n1; a.dt0 = a.dt1 = dt;
+    it_tc_cols cols;
+    const int hd = heads > 0 ? L->out_dim / heads : L->out_dim;
+    const size_t NB = it_tc_columns(a, hd, heads > 0, &cols) ? (size_t)cols.NB : (size_t)(n0 + n1);
+    const size_t core = (size_t)(K1 + K2) * (size_t)(n0 + n1 + 2 * heads) * 4;
+    const size_t Kp = ((size_t)K1 + bk - 1) / bk * bk + ((size_t)K2 + bk - 1) / bk * bk, tc = NB * Kp * (dt == IT_BF16 ? 2 : 8);
+    const size_t most = core > tc ? core : tc;
+    if (most > w.largest) w.largest = most;
+    w.sum += it_align_up(tc);
+  };
+  const int fi = L->in_dim, fo = L->out_dim, fe = L->edge_dim, fm = L->msg_dim;
+  switch (plan_of(L)) {
+    case PLAN_GAT: product(g->n, fi, 0, 0, fo, L->heads); break;
+    case PLAN_DENSE: product(g->n, fi, 0, fo, 0, 0); break;
+    case PLAN_GCN_REORDER: product(g->n, fi, 0, 0, fo, 0); break;
+    case PLAN_SAGE_REORDER: product(g->n, fi, 0, fo, fo, 0); break;
+    case PLAN_GCN: product(g->n, fi + fe, 0, fo, 0, 0); break;
+    case PLAN_SAGE: product(g->n, fi, fi + fe, fo, 0, 0); break;
+    case PLAN_MSG:
+      product(g->n, fi, 0, fm, 0, 0);
+      if (fe > 0) product(g->e, fe, 0, fm, 0, 0);
+      if (L->op == IT_GATHER_GCN) product(g->n, fm, 0, fo, 0, 0);
+      else product(g->n, fi, fm, fo, 0, 0);
+      break;
+  }
+  return w;
+}
+
+// The scratch of a layer.  lean: without partial rows (long vertices are then reduced whole, one block each).
+LayerWs plan_layer(const it_graph *g, const it_layer_desc *L, bool lean = false) {
   LayerWs w;
   const size_t n = (size_t)g->n, s = (size_t)it_dtype_size(L->feat_dtype);
   const size_t fi = (size_t)L->in_dim, fo = (size_t)L->out_dim, fe = (size_t)L->edge_dim, fm = (size_t)L->msg_dim;
-  const size_t fop = fo + 256;   // ... and its columns: each output to a multiple of 16, all to whole splits (at most 16 of at most 16 more)
-  const size_t kpad = 128;   // the tensor-core path pads the K of each operand to whole k-blocks (at most 63 + 63 rows)
+  const size_t pieces = lean ? 0 : (size_t)g->n_partial_rows;
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += it_align_up(bytes); return o; };
   w.plan = plan_of(L);
   w.off_q = 0;
-  w.off_counters = take(it_gather_words(g) * sizeof(int));
+  w.off_counters = take((lean ? IT_MAX_BUCKETS + 1 : it_gather_words(g)) * sizeof(int));
+  w.off_B = take(weight_bytes(g, L).largest);
   switch (w.plan) {
     case PLAN_GAT:
-      w.off_B = take((fi + kpad) * (fop + 2 * (size_t)L->heads) * 8);
-      w.off_partials = take(it_gat_partial_bytes(g, L->out_dim, L->heads));
+      w.off_partials = take(lean ? 0 : it_gat_partial_bytes(g, L->out_dim, L->heads));
       w.off_a = take(n * 2 * (size_t)L->heads * 4);  // scores
       w.off_b = take(n * fo * s);                    // Z
       // edge features in the logits: per edge one logit term per head (and its message row where the reduce walks copies)
@@ -105,45 +141,34 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L) {
                             : (size_t)g->n_src * (size_t)L->heads * 4);
       break;
     case PLAN_DENSE:
-      w.off_B = take((fi + kpad) * fop * 8);
       w.off_partials = w.off_a = w.off_b = off;
       break;
     case PLAN_GCN_REORDER:
-      w.off_B = take((fi + fe + kpad) * fop * 8);
-      w.off_partials = take((size_t)g->n_partial_rows * fo * 4);
+      w.off_partials = take(pieces * fo * 4);
       w.off_a = off;
       w.off_b = take(n * fo * s);  // Z
       break;
     case PLAN_GCN:
-      w.off_B = take((fi + fe + kpad) * fop * 8);
-      w.off_partials = take((size_t)g->n_partial_rows * (fi > fe ? fi : fe) * 4);
+      w.off_partials = take(pieces * (fi > fe ? fi : fe) * 4);
       w.off_a = take(n * (fi + fe) * s);  // A = [sum_e w_e h_u | sum_e e_vu]
       w.off_b = off;
       break;
     case PLAN_SAGE_REORDER:
-      w.off_B = take((fi + kpad) * 2 * fop * 8);
-      w.off_partials = take((size_t)g->n_partial_rows * fo * 4);
+      w.off_partials = take(pieces * fo * 4);
       w.off_a = take(n * fo * s);  // S (the self term, stored like the rows)
       w.off_b = take(n * fo * s);  // Z
       break;
     case PLAN_SAGE:
-      w.off_B = take((2 * fi + fe + kpad) * fop * 8);
-      w.off_partials = take((size_t)g->n_partial_rows * (fi > fe ? fi : fe) * 4);
+      w.off_partials = take(pieces * (fi > fe ? fi : fe) * 4);
       w.off_a = take(n * (fi + fe) * s);  // A = [aggregate of w_e h_u | aggregate of e_vu]
       w.off_b = off;
       break;
-    case PLAN_MSG: {
-      // the largest of the three weight matrices prepared in turn: W_edge[:in] (in x msg), W_edge[in:] (edge x msg), W ((in + msg) x out)
-      size_t wb = (fi + kpad) * (fm + 256);
-      if ((fe + kpad) * (fm + 256) > wb) wb = (fe + kpad) * (fm + 256);
-      if ((fi + fm + 2 * kpad) * fop > wb) wb = (fi + fm + 2 * kpad) * fop;
-      w.off_B = take(wb * 8);
-      w.off_partials = take((size_t)g->n_partial_rows * fm * 4);
+    case PLAN_MSG:
+      w.off_partials = take(pieces * fm * 4);
       w.off_a = take(n * fm * s);                            // A: aggregate of the messages
       w.off_b = take(n * fm * s);                            // P: source part of the message, one row per vertex
       w.off_q = take(fe > 0 ? (size_t)g->e * fm * s : 0);    // Q, then the messages in place: one row per edge
       break;
-    }
   }
   w.bytes = off;
   return w;
@@ -176,7 +201,7 @@ struct Prepared {
   void *place(it_prep_tc p) {
     if (!recording) return next < count ? m[next++].B : nullptr;
     const size_t bytes = it_align_up(it_prep_tc_bytes(p));
-    if (used + bytes > cap) return nullptr;   // (not with prep_bytes_of() of every layer)
+    if (used + bytes > cap) return nullptr;   // (not with weight_bytes() of every layer)
     p.B = base + used;
     used += bytes;
     m[count++] = p;
@@ -253,12 +278,13 @@ it_status gather_edge_part(it_gather_args gg, const it_layer_desc *L, void *A, i
   return it_launch_gather(gg, st);
 }
 
-it_status stage_ctx(const it_graph *g, const it_layer_desc *L, void *ws, size_t ws_bytes, cudaStream_t st, StageCtx *c, Prepared *prep = nullptr) {
-  c->prep = prep; c->g = g; c->L = L; c->w = plan_layer(g, L); c->ws = (char *)ws; c->st = st;
+it_status stage_ctx(const it_graph *g, const it_layer_desc *L, void *ws, size_t ws_bytes, cudaStream_t st, StageCtx *c, Prepared *prep = nullptr,
+                    bool lean = false) {
+  c->prep = prep; c->g = g; c->L = L; c->w = plan_layer(g, L, lean); c->ws = (char *)ws; c->st = st;
   IT_REQUIRE(ws_bytes >= c->w.bytes, IT_ERR_WORKSPACE, "workspace has %zu bytes, layer needs %zu", ws_bytes, c->w.bytes);
   IT_REQUIRE(L->W != nullptr, IT_ERR_INVALID_ARG, "W is NULL");
   c->B = reinterpret_cast<float *>(c->ws + c->w.off_B);
-  c->partials = g->n_partial_rows > 0 ? reinterpret_cast<float *>(c->ws + c->w.off_partials) : nullptr;
+  c->partials = g->n_partial_rows > 0 && !lean ? reinterpret_cast<float *>(c->ws + c->w.off_partials) : nullptr;
   return IT_OK;
 }
 
@@ -400,12 +426,12 @@ it_status stage_update(const StageCtx &c, const void *h_self, const void *agg, v
 }
 
 it_status layer_forward_impl(const it_graph *g, const it_layer_desc *L, const void *h_in, void *h_out, char *ws,
-                             size_t ws_bytes, cudaStream_t st, Prepared *prep = nullptr) {
+                             size_t ws_bytes, cudaStream_t st, Prepared *prep = nullptr, bool lean = false) {
   IT_REQUIRE(g->n_src == g->n, IT_ERR_INVALID_ARG,
              "the graph is one part of a partition (%lld sources, %lld vertices): use it_layer_transform / it_layer_gather / it_layer_update",
              (long long)g->n_src, (long long)g->n);
   StageCtx c;
-  IT_TRY(stage_ctx(g, L, ws, ws_bytes, st, &c, prep));
+  IT_TRY(stage_ctx(g, L, ws, ws_bytes, st, &c, prep, lean));
   const int a_dim = agg_dim_of(L);
   const LayerPlan plan = c.w.plan;
   const bool table_is_input = plan == PLAN_SAGE || plan == PLAN_GCN || plan == PLAN_DENSE;
@@ -463,14 +489,6 @@ bool fused_pair(const it_graph *g, const it_layer_desc *A, const it_layer_desc *
 
 struct InferWs { size_t layer_bytes, buf_bytes, off_buf0, off_buf1, off_prep, prep_bytes, bytes; };
 
-// Room for the prepared weights of a layer's products (each at most 8 bytes per entry, K padded to whole k-blocks).
-size_t prep_bytes_of(const it_layer_desc *L) {
-  const size_t fi = (size_t)L->in_dim, fo = (size_t)L->out_dim + 256, fe = (size_t)L->edge_dim, fm = (size_t)L->msg_dim, kpad = 128;
-  if (L->op == IT_GATHER_GAT || L->op == IT_GATHER_NONE) return it_align_up((fi + kpad) * fo * 8);
-  if (fm > 0) return it_align_up((fi + kpad) * (fm + 256) * 8) + it_align_up((fe + kpad) * (fm + 256) * 8) + it_align_up((fi + fm + 2 * kpad) * fo * 8);
-  return it_align_up((2 * fi + fe + 2 * kpad) * 2 * fo * 8);
-}
-
 it_status plan_infer(const it_graph *g, const it_layer_desc *layers, int32_t n_layers, InferWs *out) {
   IT_REQUIRE(g != nullptr, IT_ERR_INVALID_ARG, "graph is NULL");
   IT_REQUIRE(layers != nullptr && n_layers >= 1, IT_ERR_INVALID_ARG, "need at least one layer");
@@ -488,7 +506,7 @@ it_status plan_infer(const it_graph *g, const it_layer_desc *layers, int32_t n_l
       size_t hb = it_align_up((size_t)g->n * (size_t)layers[i].out_dim * (size_t)it_dtype_size(layers[i].feat_dtype));
       if (hb > w.buf_bytes) w.buf_bytes = hb;
     }
-    w.prep_bytes += prep_bytes_of(&layers[i]);
+    w.prep_bytes += weight_bytes(g, &layers[i]).sum;
   }
   w.off_buf0 = w.layer_bytes;
   w.off_buf1 = w.off_buf0 + (n_layers >= 2 ? w.buf_bytes : 0);
@@ -714,13 +732,15 @@ extern "C" it_status it_layer_forward_static(const it_graph *g, const it_layer_d
   IT_TRY(check_io(g, h_in, (size_t)g->n * layer->in_dim * s, h_out, (size_t)g->n * layer->out_dim * s));
   IT_REQUIRE(!it_profile_is_on(), IT_ERR_UNSUPPORTED,
              "it_layer_forward_static does not run while instrumentation is on (it would create CUDA events)");
-  const size_t need = plan_layer(g, layer).bytes;
+  size_t need = plan_layer(g, layer).bytes;
+  const bool lean = need > (size_t)IT_STATIC_WORKSPACE_BYTES;   // partial rows are left out where the layer does not fit with them
+  if (lean) need = plan_layer(g, layer, true).bytes;
   IT_REQUIRE(need <= (size_t)IT_STATIC_WORKSPACE_BYTES, IT_ERR_WORKSPACE,
              "layer needs %zu bytes of scratch, the built-in array holds %zu; use it_layer_forward with a caller workspace",
              need, (size_t)IT_STATIC_WORKSPACE_BYTES);
   void *ws = nullptr;
   IT_TRY(static_workspace_ptr(&ws));
-  return layer_forward_impl(g, layer, h_in, h_out, (char *)ws, (size_t)IT_STATIC_WORKSPACE_BYTES, (cudaStream_t)stream);
+  return layer_forward_impl(g, layer, h_in, h_out, (char *)ws, (size_t)IT_STATIC_WORKSPACE_BYTES, (cudaStream_t)stream, nullptr, lean);
 }
 
 extern "C" it_status it_infer(const it_graph *g, const it_layer_desc *layers, int32_t n_layers, const void *x, void *out,

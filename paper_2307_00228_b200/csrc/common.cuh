@@ -190,7 +190,7 @@ struct it_gather_args {
   const void *src;         // rows that are gathered: row u starts at src + u * src_ld elements
   int src_ld;              // 0 means dim
   int per_edge_rows;       // 1: src is [n_edges, dim] and row j belongs to edge j (edge features); 0: rows are looked up by source vertex
-  float *partials;         // [n_partial_rows, dim] fp32 scratch (may be NULL when no vertex is gathered in pieces)
+  float *partials;         // [n_partial_rows, dim] fp32 scratch; NULL: long vertices are reduced whole, one block each
   int *counters;           // it_gather_words() device words of scratch (see there)
   int zeroed;              // 1: the second part of them is zero already (and is left so)
   void *dst;               // row v starts at dst + v * dst_ld elements and takes dim of them
@@ -233,7 +233,7 @@ struct it_gat_args {
   int per_edge_scores;    // 1: src_scores is [n_edges, heads], row j belonging to edge j (edge features in the logits)
   const float *src_scores;   // [rows, heads], dense: the source-side logit term that is read per edge (row = source vertex, or the
                              // edge itself with per_edge_scores); NULL: the first half of the rows of `scores`
-  float *partials;        // it_gat_partial_bytes() of fp32 scratch for the groups of split vertices (may be NULL if none)
+  float *partials;        // it_gat_partial_bytes() of fp32 scratch; NULL: long vertices are reduced whole, one block each
   int *counters;          // it_gather_words() device words of scratch (see there)
   int zeroed;             // 1: the second part of them is zero already (and is left so)
   float slope;

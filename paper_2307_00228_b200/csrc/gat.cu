@@ -125,6 +125,8 @@ namespace {
 // (four where a head's width allows it: one pass over the partial rows of up to 128 columns); every warp merges a contiguous
 // range of the pieces, four in flight, the warps' states follow in warp order.  (One column per lane and two passes over each
 // took 465 us for the two layers of 5M vertices / 100M edges: now 176.)
+// EDGES: where there is no partial buffer (a layer that just fits the built-in scratch) the same over the vertex's edges, each a state
+// of its own: its logit, a weight of 1, its source row.
 struct GatCombineParams {
   const int32_t *__restrict__ long_owners;
   const int64_t *__restrict__ piece_ptr;
@@ -133,6 +135,14 @@ struct GatCombineParams {
   void *__restrict__ dst;
   int64_t n_long;
   int dim, heads, head_dim, act;
+  const int64_t *__restrict__ owner_indptr;    // EDGES: the vertex's edges, ...
+  const int64_t *__restrict__ shadow_indptr;
+  const int32_t *__restrict__ indices;         // ... their sources (NULL: z has a row per edge), ...
+  const void *__restrict__ z;                  // ... source rows, ...
+  const float *__restrict__ scores;            // ... and logit terms, rows of `stride` by source or by edge; destination scores
+  const float *__restrict__ scores_dst;
+  int stride, per_edge_scores;
+  float slope;
 };
 
 // a state of C columns: maximum, sum of weights, weighted sums
@@ -153,7 +163,7 @@ struct MergeState {
   }
 };
 
-template <typename T, int C>
+template <typename T, int C, bool EDGES>
 __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p) {
   constexpr int WARPS = THREADS / 32;
   __shared__ MergeState<C> red[WARPS][32];
@@ -161,9 +171,9 @@ __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p
   const int stride = gat_partial_stride(p.dim, p.heads);
   for (int64_t k = blockIdx.x; k < p.n_long; k += gridDim.x) {
     const int64_t v = __ldg(p.long_owners + k);
-    const int64_t p0 = __ldg(p.piece_ptr + k);
-    const int n = (int)(__ldg(p.piece_ptr + k + 1) - p0), per = (n + WARPS - 1) / WARPS;
-    const int a = warp * per < n ? warp * per : n, b = a + per < n ? a + per : n;
+    const int64_t p0 = EDGES ? __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v)) : __ldg(p.piece_ptr + k);
+    const int64_t n = (EDGES ? __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v + 1)) : __ldg(p.piece_ptr + k + 1)) - p0;
+    const int64_t per = (n + WARPS - 1) / WARPS, a = warp * per < n ? warp * per : n, b = a + per < n ? a + per : n;
     for (int c0 = 0; c0 < p.dim; c0 += 32 * C) {
       const int c = c0 + lane * C;
       MergeState<C> s;
@@ -171,8 +181,18 @@ __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p
       if (c < p.dim) {
         const int head = c / p.head_dim;
         const float *P = p.partials + p0 * stride;
-        auto load = [&](int g, MergeState<C> &x) {
-          const float *row = P + (int64_t)g * stride;
+        const float sd = EDGES ? __ldg(p.scores_dst + v * (2 * p.heads) + p.heads + head) : 0.f;
+        auto load = [&](int64_t g, MergeState<C> &x) {
+          if constexpr (EDGES) {
+            using Slice = RowSlice<T, C * (int)sizeof(T)>;
+            const int64_t j = p0 + g, u = p.indices ? (int64_t)__ldg(p.indices + j) : j;
+            const float e = __ldg(p.scores + (p.per_edge_scores ? j : u) * p.stride + head) + sd;
+            x.m = e > 0.f ? e : p.slope * e;
+            x.l = 1.f;
+            Slice::unpack(Slice::load(reinterpret_cast<const char *>(p.z) + (u * p.dim + c) * (int64_t)sizeof(T)), x.acc);
+            return;
+          }
+          const float *row = P + g * stride;
           x.m = __ldg(row + p.dim + head);
           x.l = __ldg(row + p.dim + p.heads + head);
           if constexpr (C == 4) {
@@ -183,18 +203,30 @@ __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p
             for (int i = 0; i < C; ++i) x.acc[i] = __ldcs(row + c + i);
           }
         };
-        int g = a;
-        for (; g + 4 <= b; g += 4) {
-          MergeState<C> x[4];
+        int64_t g = a;
+        auto merge_to = [&](MergeState<C> &t, int64_t end) {
+          for (; g + 4 <= end; g += 4) {
+            MergeState<C> x[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) load(g + u, x[u]);
+            for (int u = 0; u < 4; ++u) load(g + u, x[u]);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) s.merge(x[u]);
-        }
-        for (; g < b; ++g) {
-          MergeState<C> x;
-          load(g, x);
-          s.merge(x);
+            for (int u = 0; u < 4; ++u) t.merge(x[u]);
+          }
+          for (; g < end; ++g) {
+            MergeState<C> x;
+            load(g, x);
+            t.merge(x);
+          }
+        };
+        if constexpr (EDGES) {
+          while (g < b) {   // in runs as long as a piece, so that sums are rounded no more often than with partial rows
+            MergeState<C> run;
+            run.clear();
+            merge_to(run, b - g < 512 ? b : g + 512);
+            s.merge(run);
+          }
+        } else {
+          merge_to(s, b);
         }
       }
       __syncthreads();   // red free again
@@ -260,9 +292,10 @@ it_status dispatch_batched(int row_bytes, int heads, F f) {
 
 template <typename T>
 it_status launch_gat(const it_gat_args &a, StreamParams sp, cudaStream_t st) {
+  const bool whole = !a.partials && a.g->n_long > 0;   // long vertices are left to the combine
   if (!a.per_edge_rows && a.counters && it_gat_batched(a.dtype, a.heads, a.head_dim))
     return dispatch_batched(a.heads * a.head_dim * (int)sizeof(T), a.heads, [&]<int LPR, int H>() {
-      if (it_small_graph(a.g)) return launch_gat_small<T, LPR, H>(a, sp, make_policy<T, 16>(a), st);
+      if (it_small_graph(a.g) && !whole) return launch_gat_small<T, LPR, H>(a, sp, make_policy<T, 16>(a), st);
       return launch_gat_rows<T, LPR, H>(a, sp, make_policy<T, 16>(a), gat_bytes(a), st);
     });
   // 16-byte slices as long as one never straddles two heads
@@ -294,7 +327,6 @@ size_t it_gat_partial_bytes(const it_graph *g, int dim, int heads) {
 
 it_status it_launch_gat(const it_gat_args &a, cudaStream_t st) {
   const it_graph *g = a.g;
-  IT_REQUIRE(g->n_partial_rows == 0 || a.partials, IT_ERR_WORKSPACE, "gat: no partial buffer");
   if (g->n == 0) return IT_OK;
   StreamParams sp;
   sp.meta = g->list_meta; sp.owner = g->list_owner; sp.indices = a.per_edge_rows ? nullptr : g->indices; sp.weights = nullptr;
@@ -302,23 +334,26 @@ it_status it_launch_gat(const it_gat_args &a, cudaStream_t st) {
   sp.src_pitch = (uint32_t)(sp.dim * it_dtype_size(a.dtype));
   if (a.dtype == IT_F32) IT_TRY(launch_gat<float>(a, sp, st));
   else IT_TRY(launch_gat<__nv_bfloat16>(a, sp, st));
-  if (g->n_long > 0 && !(it_small_graph(g) && it_gat_batched(a.dtype, a.heads, a.head_dim) && !a.per_edge_rows)) {
+  if (g->n_long > 0 && !(it_small_graph(g) && a.partials && it_gat_batched(a.dtype, a.heads, a.head_dim) && !a.per_edge_rows)) {
     GatCombineParams c;
     c.long_owners = g->long_owners; c.piece_ptr = g->piece_ptr; c.partials = a.partials; c.bias = a.bias;
     c.dst = a.dst; c.n_long = g->n_long; c.dim = a.heads * a.head_dim; c.heads = a.heads;
     c.head_dim = a.head_dim; c.act = a.act;
     const int64_t cap = (int64_t)g->num_sms * 8;
     const unsigned blocks = (unsigned)(g->n_long < cap ? g->n_long : cap);
-    const double cbytes = (double)it_gat_partial_bytes(g, c.dim, c.heads) +
-                          (double)g->n_long * c.dim * (a.dtype == IT_F32 ? 4.0 : 2.0);
+    c.owner_indptr = g->owner_indptr; c.shadow_indptr = g->shadow_indptr; c.indices = sp.indices; c.z = a.z;
+    c.scores = a.src_scores ? a.src_scores : a.scores; c.stride = a.src_scores ? a.heads : 2 * a.heads; c.per_edge_scores = a.per_edge_scores;
+    c.scores_dst = a.scores_dst ? a.scores_dst : a.scores; c.slope = a.slope;
+    const double es = it_dtype_size(a.dtype);
+    const double cbytes = (a.partials ? (double)it_gat_partial_bytes(g, c.dim, c.heads)
+                                      : (double)g->h_list_edges[g->n_lists - 1] * (4.0 + 4.0 * c.heads + c.dim * es)) + (double)g->n_long * c.dim * es;
+    auto go = [&]<typename T, int C>() {
+      if (a.partials) IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, gat_combine_kernel<T, C, false><<<blocks, THREADS, 0, st>>>(c));
+      else IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, gat_combine_kernel<T, C, true><<<blocks, THREADS, 0, st>>>(c));
+    };
     const bool four = a.head_dim % 4 == 0;
-    if (a.dtype == IT_F32) {
-      if (four) IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, gat_combine_kernel<float, 4><<<blocks, THREADS, 0, st>>>(c));
-      else IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, gat_combine_kernel<float, 1><<<blocks, THREADS, 0, st>>>(c));
-    } else {
-      if (four) IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, gat_combine_kernel<__nv_bfloat16, 4><<<blocks, THREADS, 0, st>>>(c));
-      else IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, gat_combine_kernel<__nv_bfloat16, 2><<<blocks, THREADS, 0, st>>>(c));
-    }
+    if (a.dtype == IT_F32) { if (four) go.template operator()<float, 4>(); else go.template operator()<float, 1>(); }
+    else { if (four) go.template operator()<__nv_bfloat16, 4>(); else go.template operator()<__nv_bfloat16, 2>(); }
     IT_CUDA_TRY(cudaGetLastError());
   }
   return IT_OK;

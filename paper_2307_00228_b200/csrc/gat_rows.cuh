@@ -429,7 +429,7 @@ it_status launch_gat_rows(const it_gat_args &a, StreamParams p, const GatPolicy<
   p.slices = LPR;
   if (a.counters) IT_CUDA_TRY(cudaMemsetAsync(a.counters, 0, (IT_MAX_BUCKETS + 1) * sizeof(int), st));
   bool chunked = false;
-  for (int b = g->n_lists - 1; b >= 0; --b) {
+  for (int b = g->n_lists - (pol.partials ? 1 : 2); b >= 0; --b) {   // (without room for partial rows no pieces are walked)
     const int64_t lo = g->h_list_offsets[b], hi = g->h_list_offsets[b + 1], bound = g->list_bounds[b];
     if (hi <= lo) continue;
     p.row_lo = lo; p.row_hi = hi;

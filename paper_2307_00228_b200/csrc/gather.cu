@@ -9,32 +9,39 @@ namespace {
 
 using namespace it_stream;
 constexpr int GATHER_THREADS = THREADS;
+constexpr int64_t EDGE_RUN = 512;
 
 // ----------------------------------------------------------------------------- combine
 // One block per long vertex.  Its partial rows are rows [piece_ptr[k], piece_ptr[k + 1]) of the partial buffer; every warp
 // folds a contiguous range of them in order, eight rows in flight, and the warps' results are folded in warp order.
+// EDGES: where there is no partial buffer (a layer that just fits the built-in scratch) the same is done over the source rows of
+// the vertex's edges.
 struct CombineParams {
   const int32_t *__restrict__ long_owners;
   const int64_t *__restrict__ piece_ptr;
   const int64_t *__restrict__ owner_indptr;
   const int64_t *__restrict__ shadow_indptr;
   const float *__restrict__ partials;
+  const char *__restrict__ src;          // EDGES: rows of T, src_pitch bytes from one to the next, ...
+  const int32_t *__restrict__ indices;   // ... by source vertex (NULL: by edge), ...
+  const float *__restrict__ weights;     // ... and their weights (NULL: 1)
   void *__restrict__ dst;
   const void *__restrict__ self_term;
   const float *__restrict__ bias;
-  int64_t n_long;
+  int64_t n_long, src_pitch;
   int dim, dst_ld, self_ld;
   int red, is_mean, epi, act;   // red: RED_SUM / RED_MAX / RED_MIN
 };
 
-template <typename T>
+template <typename T, bool EDGES>
 __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p) {
   constexpr int WARPS = GATHER_THREADS / 32;
   __shared__ float4 red[WARPS][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int64_t k = blockIdx.x; k < p.n_long; k += gridDim.x) {
     const int64_t v = __ldg(p.long_owners + k);
-    const int64_t p0 = __ldg(p.piece_ptr + k), n = __ldg(p.piece_ptr + k + 1) - p0;
+    const int64_t j0 = __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v)), deg = __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v + 1)) - j0;
+    const int64_t p0 = EDGES ? j0 : __ldg(p.piece_ptr + k), n = EDGES ? deg : __ldg(p.piece_ptr + k + 1) - p0;
     const int64_t per = (n + WARPS - 1) / WARPS;
     const int64_t a = warp * per < n ? warp * per : n, b = a + per < n ? a + per : n;
     for (int c0 = 0; c0 < p.dim; c0 += 128) {
@@ -50,7 +57,35 @@ __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p
           acc.x += y.x; acc.y += y.y; acc.z += y.z; acc.w += y.w;
         }
       };
-      if (c < p.dim) {
+      if constexpr (EDGES) {
+        using Slice = RowSlice<T, 4 * (int)sizeof(T)>;
+        if (c < p.dim) {
+          auto edge = [&](const typename Slice::Raw &raw, float w) {
+            float y[4];
+            Slice::unpack(raw, y);
+            if (p.red == RED_SUM) { acc.x = fmaf(w, y[0], acc.x); acc.y = fmaf(w, y[1], acc.y); acc.z = fmaf(w, y[2], acc.z); acc.w = fmaf(w, y[3], acc.w); }
+            else fold(make_float4(w * y[0], w * y[1], w * y[2], w * y[3]));
+          };
+          auto load = [&](int64_t j) { return Slice::load(p.src + (p.indices ? (int64_t)__ldg(p.indices + j) : j) * p.src_pitch + (size_t)c * sizeof(T)); };
+          float4 total = acc;
+          for (int64_t g = a; g < b;) {   // in runs as long as a piece, so that sums are rounded no more often than with partial rows
+            const int64_t end = b - g < EDGE_RUN ? b : g + EDGE_RUN;
+            acc = make_float4(id, id, id, id);
+            for (; g + 8 <= end; g += 8) {
+              typename Slice::Raw y[8];
+#pragma unroll
+              for (int u = 0; u < 8; ++u) y[u] = load(p0 + g + u);
+#pragma unroll
+              for (int u = 0; u < 8; ++u) edge(y[u], p.weights ? __ldg(p.weights + p0 + g + u) : 1.f);
+            }
+            for (; g < end; ++g) edge(load(p0 + g), p.weights ? __ldg(p.weights + p0 + g) : 1.f);
+            const float4 run = acc;
+            acc = total;
+            fold(run);
+            total = acc;
+          }
+        }
+      } else if (c < p.dim) {
         const float *P = p.partials + p0 * p.dim + c;
         int64_t g = a;
         for (; g + 8 <= b; g += 8) {
@@ -67,7 +102,6 @@ __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p
       __syncthreads();
       if (warp != 0 || c >= p.dim) continue;   // (the barriers above are met by every warp in every round)
       for (int w = 1; w < WARPS; ++w) fold(red[w][lane]);
-      const int64_t deg = p.is_mean ? __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v + 1)) - __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v)) : 1;
       const float inv = p.is_mean ? 1.f / (float)deg : 1.f;
       float o[4] = {acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv};
       const int64_t doff = v * p.dst_ld + c;
@@ -213,15 +247,20 @@ static it_status launch_gather_chunk(const it_gather_args &a, cudaStream_t st) {
   if (g->n_long > 0 && !folded) {
     CombineParams c;
     c.long_owners = g->long_owners; c.piece_ptr = g->piece_ptr; c.owner_indptr = g->owner_indptr; c.shadow_indptr = g->shadow_indptr;
-    c.partials = a.partials; c.dst = a.dst; c.self_term = a.self_term; c.bias = a.bias; c.n_long = g->n_long;
+    c.partials = a.partials; c.src = (const char *)a.src; c.src_pitch = sp.src_pitch; c.indices = sp.indices; c.weights = a.use_edge_weights ? g->edge_weights : nullptr;
+    c.dst = a.dst; c.self_term = a.self_term; c.bias = a.bias; c.n_long = g->n_long;
     c.dim = a.dim; c.dst_ld = a.dst_ld > 0 ? a.dst_ld : a.dim; c.self_ld = a.self_ld > 0 ? a.self_ld : a.dim;
     c.red = a.op == IT_GATHER_MAX ? RED_MAX : (a.op == IT_GATHER_MIN ? RED_MIN : RED_SUM); c.is_mean = a.op == IT_GATHER_MEAN && a.epi != IT_EPI_RAW_F32; c.epi = a.epi; c.act = a.act;
     const int64_t cap = (int64_t)g->num_sms * 8;
     const unsigned blocks = (unsigned)(g->n_long < cap ? g->n_long : cap);
-    const double cbytes = (double)g->n_partial_rows * a.dim * 4.0 +
-                          (double)g->n_long * a.dim * (a.dtype == IT_F32 ? 4.0 : 2.0);
-    if (a.dtype == IT_F32) IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, combine_kernel<float><<<blocks, GATHER_THREADS, 0, st>>>(c));
-    else IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, combine_kernel<__nv_bfloat16><<<blocks, GATHER_THREADS, 0, st>>>(c));
+    const double es = it_dtype_size(a.dtype);
+    const double cbytes = (a.partials ? (double)g->n_partial_rows * a.dim * 4.0 : (double)g->h_list_edges[g->n_lists - 1] * (4.0 + a.dim * es)) + (double)g->n_long * a.dim * es;
+    auto go = [&]<typename T>() {
+      if (a.partials) IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, combine_kernel<T, false><<<blocks, GATHER_THREADS, 0, st>>>(c));
+      else IT_LAUNCH(IT_K_COMBINE, cbytes, 0, st, combine_kernel<T, true><<<blocks, GATHER_THREADS, 0, st>>>(c));
+    };
+    if (a.dtype == IT_F32) go.template operator()<float>();
+    else go.template operator()<__nv_bfloat16>();
     IT_CUDA_TRY(cudaGetLastError());
   }
   return IT_OK;
@@ -236,7 +275,6 @@ it_status it_launch_gather(const it_gather_args &a, cudaStream_t st) {
   IT_REQUIRE(a.op == IT_GATHER_SUM || a.op == IT_GATHER_MEAN || a.op == IT_GATHER_MAX || a.op == IT_GATHER_MIN, IT_ERR_INVALID_ARG,
              "gather: bad op");
   IT_REQUIRE(!a.use_edge_weights || g->edge_weights, IT_ERR_INVALID_ARG, "layer uses edge weights but the graph has none");
-  IT_REQUIRE(g->n_partial_rows == 0 || a.partials, IT_ERR_WORKSPACE, "gather: no partial buffer");
   const int es = it_dtype_size(a.dtype);
   IT_REQUIRE(a.dim > 0 && (a.dim * es) % 16 == 0, IT_ERR_INVALID_ARG, "gather: a row of %d bytes is not a multiple of 16", a.dim * es);
   if (g->n == 0) return IT_OK;

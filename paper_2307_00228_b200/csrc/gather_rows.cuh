@@ -293,7 +293,7 @@ it_status launch_lpr(const it_gather_args &a, StreamParams sp, bool *folded, cud
   // (rows of 80 to 128 bytes cost the one kernel more than the kernels by list from about a million edges on: 60k vertices, 1M
   // edges, two layers 130 against 137 us, 130k vertices, 1.3M edges 191 against 165)
   const int row_bytes = a.dim * (int)sizeof(T);
-  if (it_small_graph(a.g) && (row_bytes <= 64 || row_bytes > 128 || a.g->e + 6 * a.g->n <= 1400000)) {
+  if (it_small_graph(a.g) && (a.partials || a.g->n_long == 0) && (row_bytes <= 64 || row_bytes > 128 || a.g->e + 6 * a.g->n <= 1400000)) {
     *folded = true;
     if (a.op == IT_GATHER_MAX) return launch_small<T, RED_MAX>(a, sp, st);
     if (a.op == IT_GATHER_MIN) return launch_small<T, RED_MIN>(a, sp, st);

@@ -594,7 +594,7 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
   p.counter = nullptr;
   bool chunked = false;
   p.slices = p.dim * (int)sizeof(T) / SB;
-  for (int b = g->n_lists - 1; b >= 0; --b) {
+  for (int b = g->n_lists - (pol.partials ? 1 : 2); b >= 0; --b) {   // (without room for partial rows no pieces are walked)
     const int64_t lo = g->h_list_offsets[b], hi = g->h_list_offsets[b + 1];
     if (hi <= lo) continue;
     p.row_lo = lo; p.row_hi = hi;

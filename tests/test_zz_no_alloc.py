@@ -115,6 +115,53 @@ def test_layer_larger_than_the_built_in_scratch_is_rejected():
     assert bool(torch.isfinite(out).all())
 
 
+def dense_graph(n, e, dtype, fi, weighted=False, edge_dim=0):
+    """n vertices of about e / n edges each, small whole numbers as features (their sums are exact in any order)."""
+    g = torch.Generator(device="cuda").manual_seed(7)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    indptr = (torch.arange(n + 1, device="cuda", dtype=torch.int64) * e) // n
+    indices = torch.randint(0, n, (e,), generator=g, device="cuda", dtype=torch.int32)
+    weights = torch.randint(1, 3, (e,), generator=g, device="cuda").float() if weighted else None
+    graph = B.it_graph_create(indptr, indices, weights)
+    if edge_dim:
+        B.it_graph_set_edge_features(graph, torch.randint(-1, 2, (e, edge_dim), generator=g, device="cuda").to(dt))
+    return graph, torch.randint(-1, 2, (n, fi), generator=g, device="cuda").to(dt)
+
+
+@pytest.mark.parametrize("case", ["sum", "weighted_min", "reorder", "small_max", "edge_features", "gat_f32", "gat_bf16", "gat_16_heads"])
+def test_layers_that_fit_without_partial_rows(case):
+    """Few vertices of very many edges: the tables are small, the partial rows of the vertices' pieces are not.  Sums of whole numbers,
+    maxima and minima are equal bit for bit; other sums may be taken in another order (2^-24 times the square root of the terms or
+    less in fp32, then one rounding of the stored bf16 result)."""
+    n, e = (3000, 2_000_000) if case == "small_max" else (100, 40_000_000 if case in ("gat_f32", "gat_16_heads") else 18_000_000)
+    dtype = "bf16" if case in ("reorder", "gat_bf16") else "f32"
+    if "gat" in case:
+        heads, hd, slope = {"gat_f32": (4, 32, 0.2), "gat_bf16": (8, 32, -0.1), "gat_16_heads": (16, 8, 0.2)}[case]
+        layer = make_gat_layer(60, "elu", 32, heads, hd, dtype)
+        layer.leaky_slope = slope
+    elif case == "reorder":
+        layer = make_sage_layer(61, "mean", "relu", 512, 256, dtype)
+    else:
+        op = {"sum": "sum", "weighted_min": "min", "small_max": "max", "edge_features": "mean"}[case]
+        layer = make_sage_layer(62, op, "relu", 512 if case == "small_max" else 256, 16, dtype, weights=case == "weighted_min", allow_reorder=False,
+                                edge_dim=4 if case == "edge_features" else 0)
+    graph, x = dense_graph(n, e, dtype, layer.in_dim, case == "weighted_min", layer.edge_dim)
+    lay = host.layer_to_device(layer, dtype)
+    ws = torch.empty(B.it_workspace_bytes(graph, [lay]), dtype=torch.uint8, device="cuda")
+    assert ws.numel() > B.STATIC_WORKSPACE_BYTES
+    want = torch.empty((n, layer.out_dim), dtype=x.dtype, device="cuda")
+    B.it_layer_forward(graph, lay, x, want, ws)
+    for _ in range(2):
+        got = torch.full_like(want, float("nan"))
+        B.it_layer_forward_static(graph, lay, x, got)
+        torch.cuda.synchronize()
+        if "gat" in case or case == "reorder":
+            err = float((got.float() - want.float()).norm() / want.float().norm())
+            assert err <= (2.0 ** -24 * (e / n) ** 0.5 if dtype == "f32" else 2.0 ** -8), err
+        else:
+            assert torch.equal(got, want)
+
+
 def test_static_variant_refuses_to_run_under_instrumentation():
     layer = make_sage_layer(52, "sum", "relu", 16, 16, "f32")
     w = small_workload(53, 200, 4, "f32", [layer])
