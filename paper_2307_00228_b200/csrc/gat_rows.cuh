@@ -221,7 +221,7 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
     for (int u = 0; u < PP; ++u) {
       const int e = el + u * EP;
       const uint32_t s = (uint32_t)__shfl_sync(0xffffffffu, idx, gbase + (e & (E - 1)));
-      x[u] = 0.f;
+      x[u] = __int_as_float(0x7fffffff);   // NaN stays NaN whatever the slope; the weight of a pair without an edge is not used
       if (e < E && k + e < r.len) x[u] = __ldg(q.scores + (q.per_edge ? (uint64_t)(r.j0 + k + e) : (uint64_t)s) * q.stride + hl);
     }
   };
@@ -254,10 +254,9 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
       // this round: the weights ...
       float mr = -INFINITY;
 #pragma unroll
-      for (int u = 0; u < PP; ++u) {   // a pair without an edge is masked after the activation, whose slope may have any sign
-        const int e = el + u * EP;
-        x_a[u] = e < E && k0 + e < r0.len ? leaky(x_a[u] + r0.sd, q.slope) : -INFINITY;
-        mr = fmaxf(mr, x_a[u]);
+      for (int u = 0; u < PP; ++u) {
+        x_a[u] = leaky(x_a[u] + r0.sd, q.slope);
+        mr = fmaxf(mr, x_a[u]);   // (of a NaN and a number the number: pairs without an edge do not count)
       }
 #pragma unroll
       for (int o = H; o < LPR; o <<= 1) mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
