@@ -52,6 +52,9 @@
 #ifndef IT_RING_CLAIMS_PER_WARP
 #define IT_RING_CLAIMS_PER_WARP 16   // claims a warp of the ring kernel makes on average over a launch
 #endif
+#ifndef IT_RING_FEW
+#define IT_RING_FEW 3            // rows of more than 128 bytes: fewer rows than this per warp are walked one at a time
+#endif
 #ifndef IT_SHORT_EDGES
 #define IT_SHORT_EDGES 8         // source rows a lane of the short-row kernel has in flight per round
 #endif
@@ -594,6 +597,15 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
   p.counter = nullptr;
   bool chunked = false;
   p.slices = p.dim * (int)sizeof(T) / SB;
+  // Graphs whose vertices all lie below the pieces' length.  128-byte rows: more warps with shorter stages win (bf16 64 columns, two
+  // layers: 200k vertices of 300 edges 614 -> 550 us, 1M of 100 1531 -> 1445, 6M of 40 6159 -> 5964).  And with few rows for every
+  // warp the chunk kernel's claims, made ahead, leave warps idle at the end: then a row at a time (20k vertices of 500 edges, 128-byte
+  // rows 115 -> 102; wider rows lose by it at 6 rows per warp, 273 -> 291, so only below IT_RING_FEW).
+  const bool no_pieces = !pol.partials || g->h_list_offsets[g->n_lists] == g->h_list_offsets[g->n_lists - 1];
+  int64_t warp_rows = 0;
+  for (int b = 0; b < g->n_lists - 1; ++b)
+    if (g->list_bounds[b] > IT_SHORT_BELOW) warp_rows += g->h_list_offsets[b + 1] - g->h_list_offsets[b];
+  const bool ring_rows = no_pieces && warp_rows < (LPR == 8 ? 8 : IT_RING_FEW) * (int64_t)g->num_sms * IT_RING_MIN_BLOCKS * (THREADS / 32);
   for (int b = g->n_lists - (pol.partials ? 1 : 2); b >= 0; --b) {   // (without room for partial rows no pieces are walked)
     const int64_t lo = g->h_list_offsets[b], hi = g->h_list_offsets[b + 1];
     if (hi <= lo) continue;
@@ -637,7 +649,7 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
       if constexpr (SB == 16 && LPR >= 8 && !Policy::HAS_EXTRA) {
         // one warp per row: the pieces and the whole vertices of more than IT_SHORT_BELOW edges, in one launch (they are
         // neighbours in the list), pieces first
-        if (bound > IT_SHORT_BELOW && counters) {
+        if (bound > IT_SHORT_BELOW && counters && !ring_rows) {
           if (chunked) continue;
           chunked = true;
           double all = bytes;
@@ -647,12 +659,21 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
             all += bytes_of(b0, g->h_list_offsets[b0 + 1] - g->h_list_offsets[b0]);
           }
           p.row_lo = g->h_list_offsets[b0];
-          constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<16, false, IT_CHUNK_STAGE_ROWS>();
-          static std::atomic<uint64_t> configured{0};   // per template instance: one bit per device ordinal
-          IT_TRY(allow_dynamic_smem(stream_rows_chunk_kernel<T, LPR, Policy, PAD>, smem, configured));
           p.counter = counters + b;
-          const unsigned blocks = chunk_grid(p, b == g->n_lists - 1 ? rows : 0, (int64_t)g->num_sms * IT_CHUNK_BLOCKS);
-          IT_LAUNCH(kid_rows, all, 0, st, stream_rows_chunk_kernel<T, LPR, Policy, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
+          auto launch = [&]<int BLOCKS, int ROWS>() -> it_status {
+            constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<16, false, ROWS>();
+            static std::atomic<uint64_t> configured{0};   // per template instance: one bit per device ordinal
+            IT_TRY(allow_dynamic_smem(stream_rows_chunk_kernel<T, LPR, Policy, PAD, BLOCKS, ROWS>, smem, configured));
+            const unsigned blocks = chunk_grid(p, b == g->n_lists - 1 ? rows : 0, (int64_t)g->num_sms * BLOCKS);
+            IT_LAUNCH(kid_rows, all, 0, st, stream_rows_chunk_kernel<T, LPR, Policy, PAD, BLOCKS, ROWS><<<blocks, THREADS, smem, st>>>(p, pol));
+            return IT_OK;
+          };
+          bool plain = false;
+          if constexpr (LPR == 8) {
+            plain = no_pieces;
+            if (plain) IT_TRY((launch.template operator()<IT_CHUNK_BLOCKS_PLAIN, IT_CHUNK_STAGE_ROWS_PLAIN>()));
+          }
+          if (!plain) IT_TRY((launch.template operator()<IT_CHUNK_BLOCKS, IT_CHUNK_STAGE_ROWS>()));
           p.counter = nullptr;
           continue;
         }

@@ -139,12 +139,18 @@ __device__ __forceinline__ void chunk_walk(const Warp &rw, const Policy &pol, Cu
 #ifndef IT_CHUNK_STAGE_ROWS
 #define IT_CHUNK_STAGE_ROWS 8   // ... 512-byte groups of rows per stage (four CTAs with stages of 4: GCN on 15M edges 2.76 against 2.67 ms,
 #endif                          // fp32 sums on 40M 6.11 against 5.88, mean on 375M 22.4 against 22.2, 16M wide rows 3.26 against 3.20)
-template <typename T, int LPR, class Policy, bool PAD>
-__global__ void __launch_bounds__(THREADS, IT_CHUNK_BLOCKS) stream_rows_chunk_kernel(StreamParams p, Policy pol) {
+#ifndef IT_CHUNK_BLOCKS_PLAIN
+#define IT_CHUNK_BLOCKS_PLAIN 4       // the same for 128-byte rows of graphs without pieces (launch_buckets)
+#endif
+#ifndef IT_CHUNK_STAGE_ROWS_PLAIN
+#define IT_CHUNK_STAGE_ROWS_PLAIN 4
+#endif
+template <typename T, int LPR, class Policy, bool PAD, int BLOCKS, int ROWS>
+__global__ void __launch_bounds__(THREADS, BLOCKS) stream_rows_chunk_kernel(StreamParams p, Policy pol) {
   extern __shared__ uint4 ring_raw[];
   const int lane = threadIdx.x & 31;
-  RingWarp<T, 16, LPR, Policy, PAD, IT_CHUNK_STAGE_ROWS> rw;
-  rw.setup((uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)(threadIdx.x >> 5) * (uint32_t)ring_bytes_per_warp<16, false, IT_CHUNK_STAGE_ROWS>(), p.src, p.src_pitch,
+  RingWarp<T, 16, LPR, Policy, PAD, ROWS> rw;
+  rw.setup((uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)(threadIdx.x >> 5) * (uint32_t)ring_bytes_per_warp<16, false, ROWS>(), p.src, p.src_pitch,
            p.slices, lane);
   pol.setup(lane % LPR);
   ChunkCursor<Policy::WEIGHTED, false> cur(p, lane);

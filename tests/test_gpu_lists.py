@@ -24,6 +24,16 @@ def test_pooling(dtype, fi, op, max_deg):
     check_against_oracle(w, got, label=(dtype, fi, op), exact=False)
 
 
+@pytest.mark.parametrize("dtype,fi", [("bf16", 64), ("f32", 20), ("f32", 32), ("bf16", 128), ("f32", 100)])
+@pytest.mark.parametrize("op,weights,max_deg", [("max", False, 9), ("sum", True, 9), ("mean", False, 60), ("min", True, 60)])
+def test_no_vertex_in_pieces(dtype, fi, op, weights, max_deg):
+    """Rows of at most 1024 edges only: few long ones (walked one at a time), and tens of thousands (chunks of one row after the other)."""
+    layer = make_sage_layer(30, op, "relu", fi, 16, dtype, weights=weights, allow_reorder=False)
+    w = small_workload(31, N, max_deg, dtype, [layer], hubs=HUBS[4:], weights=weights)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(dtype, fi, op, max_deg), exact=False)
+
+
 @pytest.mark.parametrize("dtype,heads,hd", [("f32", 4, 4), ("f32", 4, 16), ("f32", 2, 64), ("bf16", 2, 16), ("bf16", 8, 8), ("bf16", 4, 32), ("f32", 1, 8)])
 def test_gat(dtype, heads, hd):
     layer = make_gat_layer(23, "elu", 32, heads, hd, dtype)
