@@ -292,8 +292,16 @@ it_status dispatch_batched(int row_bytes, int heads, F f) {
 
 template <typename T>
 it_status launch_gat(const it_gat_args &a, StreamParams sp, cudaStream_t st) {
-  const bool whole = !a.partials && a.g->n_long > 0;   // long vertices are left to the combine
-  if (!a.per_edge_rows && a.counters && it_gat_batched(a.dtype, a.heads, a.head_dim))
+  const it_graph *g = a.g;
+  const bool whole = !a.partials && g->n_long > 0;   // long vertices are left to the combine
+  // A lane of a 128-byte row holds half a head of four or one of eight: a step then computes as many exponentials per lane as the
+  // per-edge softmax, and that one has no step to set up.  It wins but for rows of a few edges and, for four heads in bf16, where
+  // vertices are gathered in pieces (batched against per edge: bf16 4 heads, 1M vertices of 31 / 40 / 100 edges 1019 / 1343 / 2604
+  // against 925 / 1209 / 2410 us, 6M of 2 / 12 / 40 edges 1259 / 3787 / 11039 against 1350 / 3726 / 10030, 1M / 15M power law 549
+  // against 566; the same graph, 8 heads, 1266 against 1204, fp32 4 heads 811 against 795, 8 heads 909 against 827).
+  const bool per_edge = a.heads * a.head_dim * (int)sizeof(T) == 128 && !a.per_edge_scores && !it_small_graph(g) && g->e > 8 * g->n &&
+                        (a.heads == 8 || (a.heads == 4 && (g->n_long == 0 || sizeof(T) == 4)));
+  if (!a.per_edge_rows && a.counters && !per_edge && it_gat_batched(a.dtype, a.heads, a.head_dim))
     return dispatch_batched(a.heads * a.head_dim * (int)sizeof(T), a.heads, [&]<int LPR, int H>() {
       if (it_small_graph(a.g) && !whole) return launch_gat_small<T, LPR, H>(a, sp, make_policy<T, 16>(a), st);
       return launch_gat_rows<T, LPR, H>(a, sp, make_policy<T, 16>(a), gat_bytes(a), st);

@@ -42,6 +42,17 @@ def test_gat(dtype, heads, hd):
     check_against_oracle(w, got, label=(dtype, heads, hd), exact=False)
 
 
+@pytest.mark.parametrize("dtype,heads,hd", [("f32", 4, 8), ("bf16", 4, 16), ("f32", 8, 4), ("bf16", 8, 8)])
+@pytest.mark.parametrize("hubs", [HUBS, HUBS[4:]])   # with and without pieces
+def test_gat_of_128_byte_rows_with_many_heads(dtype, heads, hd, hubs):
+    """More than eight edges per vertex on average: the per-edge softmax, or the batched one where it wins."""
+    layer = make_gat_layer(32, "elu", 32, heads, hd, dtype)
+    w = small_workload(33, N, 24, dtype, [layer], hubs=hubs, p_zero=0.1)
+    assert w.e > 8 * w.n
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(dtype, heads, hd), exact=False)
+
+
 def test_self_term_and_bias_of_rows_without_edges():
     for layer in (make_sage_layer(25, "mean", "elu", 64, 32, "bf16"), make_plain_layer(26, "gcn", "elu", 64, 32, "bf16")):
         w = small_workload(27, N, 4, "bf16", [layer], hubs=HUBS[:6], p_zero=0.9)
