@@ -17,6 +17,15 @@
 #ifndef IT_SMALL_EDGES
 #define IT_SMALL_EDGES (1 << 21)
 #endif
+#ifndef IT_SMALL_DENSE
+#define IT_SMALL_DENSE 256
+#endif
+#ifndef IT_SMALL_DENSE_ROWS
+#define IT_SMALL_DENSE_ROWS 2048
+#endif
+#ifndef IT_SMALL_DENSE_EDGES
+#define IT_SMALL_DENSE_EDGES (7 << 17)
+#endif
 
 // ----------------------------------------------------------------------------- errors
 void it_set_error(const char *fmt, ...);
@@ -125,7 +134,15 @@ struct it_graph {
 // folds the pieces of long vertices itself.  Measured on both sides of the line (two layers, one kernel against kernels by list):
 // fp32 64-64-16, 10k vertices / 100k edges 41 against 238 us, 130k / 2M 192 against 402; fp32 128-128 60k / 2M 167 against 219,
 // 130k / 2M 244 against 259; GAT 130k / 2M 141 against 195.
-static inline bool it_small_graph(const it_graph *g) { return g->n <= IT_SMALL_ROWS && g->e <= IT_SMALL_EDGES; }
+// Graphs of IT_SMALL_DENSE_ROWS vertices and more with more than IT_SMALL_DENSE edges each and more than IT_SMALL_DENSE_EDGES in all keep
+// the kernels by list: there are whole rows for the warps, and pieces of 128 edges only add partial rows (fp32 mean 64 / bf16 max 64 /
+// fp32 max 512 / fp32 sum 128, one kernel against kernels by list: 3000 vertices, 1M edges 74 / 70 / 266 / 66 against 58 / 47 / 183 / 58
+// us; 6000, 2M 124 / 107 / 466 / 117 against 80 / 63 / 316 / 89; on the other sides 8000, 2M 144 / 132 / 508 against 140 / 119 / 642;
+// 1000, 1.2M 73 / 70 / 270 / 70 against 83 / 71 / 244 / 73, GAT 60 against 76; 3000, 500k 60 / 66 / 191 against 67 / 66 / 216).
+static inline bool it_small_graph(const it_graph *g) {
+  const bool dense = g->n >= IT_SMALL_DENSE_ROWS && g->e > IT_SMALL_DENSE * g->n && g->e > IT_SMALL_DENSE_EDGES;
+  return g->n <= IT_SMALL_ROWS && g->e <= IT_SMALL_EDGES && !dense;
+}
 
 // Words of device memory that the gather of one layer needs: the list counters (zeroed by the launch that uses them), then,
 // for small graphs, how many pieces of every long vertex are done.

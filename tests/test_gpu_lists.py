@@ -53,6 +53,16 @@ def test_gat_of_128_byte_rows_with_many_heads(dtype, heads, hd, hubs):
     check_against_oracle(w, got, label=(dtype, heads, hd), exact=False)
 
 
+@pytest.mark.parametrize("n,deg", [(1000, 1100), (3700, 245), (3700, 270), (3000, 400)])
+@pytest.mark.parametrize("kind", ["sum", "max", "gat"])
+def test_few_vertices_of_many_edges(n, deg, kind):
+    """Both sides of the line between one kernel and kernels by list: about 245 and 270 edges per vertex, fewer vertices, and far beyond it."""
+    layer = make_gat_layer(34, "elu", 32, 4, 16, "f32") if kind == "gat" else make_sage_layer(34, kind, "relu", 132, 16, "f32", allow_reorder=False)
+    w = small_workload(35, n, 2 * deg, "f32", [layer], hubs=(5000, 129, 128, 127), p_zero=0.0)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(n, deg, kind), exact=False)
+
+
 def test_self_term_and_bias_of_rows_without_edges():
     for layer in (make_sage_layer(25, "mean", "elu", 64, 32, "bf16"), make_plain_layer(26, "gcn", "elu", 64, 32, "bf16")):
         w = small_workload(27, N, 4, "bf16", [layer], hubs=HUBS[:6], p_zero=0.9)

@@ -133,7 +133,7 @@ def test_layers_that_fit_without_partial_rows(case):
     """Few vertices of very many edges: the tables are small, the partial rows of the vertices' pieces are not.  Sums of whole numbers,
     maxima and minima are equal bit for bit; other sums may be taken in another order (2^-24 times the square root of the terms or
     less in fp32, then one rounding of the stored bf16 result)."""
-    n, e = (3000, 2_000_000) if case == "small_max" else (100, 40_000_000 if case in ("gat_f32", "gat_16_heads") else 18_000_000)
+    n, e = (1500, 2_000_000) if case == "small_max" else (100, 40_000_000 if case in ("gat_f32", "gat_16_heads") else 18_000_000)
     dtype = "bf16" if case in ("reorder", "gat_bf16") else "f32"
     if "gat" in case:
         heads, hd, slope = {"gat_f32": (4, 32, 0.2), "gat_bf16": (8, 32, -0.1), "gat_16_heads": (16, 8, 0.2)}[case]
