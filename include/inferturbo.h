@@ -157,9 +157,11 @@ it_status it_graph_set_edge_features(it_graph *g, const void *edge_feat, int32_t
  * own and the partial results combined (Partial-Gather, same section).
  *   n = 1 if d <= T (or T <= 0), else ceil(d / T) groups; group g takes the next
  *   d / n + (g < d % n) consecutive edges.  Row id = owner_indptr[v] + g.
- * (These rows are what it_graph_get_split reports.  The Gather stage cuts every vertex of more than min(T, about 1024 to
- * 4096) edges into finer pieces of its own and orders them for the cache, whatever T is; results do not depend on when a
- * piece is gathered.)
+ * (These rows are what it_graph_get_split reports.  The Gather stage does not walk them: it cuts every vertex of more than
+ * about 1024 to 4096 edges (128 on small graphs) into pieces of its own, whatever T is, and orders them by their place in the
+ * vertex's edges.  Results do not depend on that order.  Where the source ids of every vertex ascend, pieces that are gathered
+ * side by side read the same part of the source table, which then stays in the cache: sorting them pays on graphs whose table
+ * does not fit it.)
  * Also builds the degree buckets: shadow rows partitioned stably by length class
  * (bounds from it_graph_get_split).  Rebuilds everything derived; edge arrays are not
  * permuted.  out_n_rows / out_n_split_owners may be NULL.  Synchronises `stream`.

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256) validate_indices_kernel(const int32_t *__
 // nb + 4 on the lists that the gather walks.
 //
 // The gather does not walk the shadow rows of a hub but finer pieces of its segment, and pieces of every vertex of more than
-// long_above edges (T, 1024 to 4096): those of all such vertices are ordered by where in its vertex's segment a piece lies.  Source ids ascend
+// long_above edges (1024 to 4096, whatever T is): those of all such vertices are ordered by where in its vertex's segment a piece lies.  Source ids ascend
 // inside a segment, so pieces at the same relative position read the same part of the source table, and the pieces that are in
 // flight together share it through the L2 cache.  Whole passes, against
 // one block per row of up to T edges in vertex order: 5M vertices / 100M edges, GAT, 13.1 -> 11.7 ms; 20M / 200M with 100 hubs
@@ -103,6 +103,8 @@ constexpr int SPLIT_THREADS = 256;
 constexpr int SPLIT_ITEMS = 8;                                    // vertices per lane
 constexpr int SPLIT_TILE = 32 * SPLIT_ITEMS;                      // a tile is one warp's 256 consecutive vertices
 constexpr int SPLIT_COLS = 2 * IT_MAX_BUCKETS + 4;
+constexpr int N_FIXED = 5;                                        // bounds of the buckets below T, of the lists below long_above
+constexpr int N_LISTS = N_FIXED + 1;                              // lists of whole vertices
 constexpr int PIECE_BINS = 256;                                   // steps of the order in which pieces are walked
 
 struct Bounds { int64_t b[IT_MAX_BUCKETS]; int nb; };
@@ -111,6 +113,10 @@ __device__ __forceinline__ int bucket_of(int64_t len, const Bounds &B) {
   while (k < B.nb - 1 && len > B.b[k]) ++k;
   return k;
 }
+
+// The list of a vertex that is gathered whole: bounds 0, 8, 32, 256, 1024, long_above.  For a vertex of at most T edges it has the
+// number of its bucket (whose bounds are those of these below T, then T).
+__device__ __forceinline__ int list_of(int64_t len) { return (len > 0) + (len > 8) + (len > 32) + (len > 256) + (len > 1024); }
 
 struct LongInfo { int64_t r0, pos_a, pos_b; };   // a long vertex: its first row; bucket positions of its longer / shorter groups
 
@@ -166,13 +172,15 @@ __device__ __forceinline__ void add_plain(int64_t &col, unsigned mine, unsigned 
   if (lane == nb) col += __popc(plain);
   else col += __popc(mine & plain);   // (0 for the columns of long vertices)
 }
-// vertex l, gathered in pieces
-struct LongCols { int64_t ng, rem, np; int ka, kb; };
+// vertex l, of several groups or gathered in pieces (np > 0; else whole, from list kl)
+struct LongCols { int64_t ng, rem, np; int ka, kb, kl; };
 __device__ __forceinline__ LongCols long_cols(int64_t d, const VertexRows &r, int l, const SplitParams &p) {
   LongCols c;
   c.ng = __shfl_sync(0xffffffffu, r.ng, l); c.rem = __shfl_sync(0xffffffffu, r.rem, l);
   c.ka = __shfl_sync(0xffffffffu, r.ka, l); c.kb = __shfl_sync(0xffffffffu, r.kb, l);
-  c.np = pieces_of(__shfl_sync(0xffffffffu, d, l), p);
+  const int64_t dl = __shfl_sync(0xffffffffu, d, l);
+  c.np = dl > p.long_above ? pieces_of(dl, p) : 0;
+  c.kl = list_of(dl);
   return c;
 }
 __device__ __forceinline__ void add_long(int64_t &col, const LongCols &c, int nb, int lane) {
@@ -180,9 +188,12 @@ __device__ __forceinline__ void add_long(int64_t &col, const LongCols &c, int nb
   if (lane == c.kb) col += c.ng - c.rem;
   if (lane == nb) col += c.ng;
   if (lane == nb + 1 && c.ng > 1) col += 1;
-  if (lane == nb + 2) col += 1;
+  if (lane == nb + 2 && c.np > 0) col += 1;
   if (lane == nb + 3) col += c.np;
+  if (lane == nb + 4 + c.kl && c.np == 0) col += 1;
 }
+// vertices that take their turn one by one: of several groups, or gathered in pieces
+__device__ __forceinline__ bool one_by_one(int64_t d, const VertexRows &r, const SplitParams &p) { return r.ng > 1 || d > p.long_above; }
 
 __global__ void __launch_bounds__(SPLIT_THREADS) split_count_kernel(SplitParams p) {
   __shared__ unsigned long long edges[IT_MAX_BUCKETS];
@@ -202,21 +213,23 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_count_kernel(SplitParams 
   for (int i = 0; i < SPLIT_ITEMS; ++i) {
     const VertexRows r = rows_of(d[i], p);
     const unsigned valid = __ballot_sync(0xffffffffu, v0 + i * 32 < p.n), mine = bucket_mask(r.kb, nb, lane);
-    unsigned lng = __ballot_sync(0xffffffffu, d[i] > p.long_above);
+    unsigned lng = __ballot_sync(0xffffffffu, one_by_one(d[i], r, p));
     add_plain(col, mine, valid & ~lng, nb, lane);
     while (lng) {   // rare
       const int l = __ffs(lng) - 1;
       lng &= lng - 1;
       add_long(col, long_cols(d[i], r, l, p), nb, lane);
     }
-    for (int k = 1; k < nb; ++k) {   // whole vertices have at most 4096 edges: 32-bit sums
-      const unsigned sum = __reduce_add_sync(0xffffffffu, r.kb == k && d[i] <= p.long_above ? (unsigned)d[i] : 0u);
+    const int kl = list_of(d[i]);
+#pragma unroll
+    for (int k = 1; k < N_LISTS; ++k) {   // whole vertices have at most 4096 edges: 32-bit sums
+      const unsigned sum = __reduce_add_sync(0xffffffffu, kl == k && d[i] <= p.long_above ? (unsigned)d[i] : 0u);
       if (lane == k) my_edges += sum;
     }
     if (d[i] > p.long_above) atomicAdd(&edges[IT_MAX_BUCKETS - 1], (unsigned long long)d[i]);
   }
-  if (lane < 2 * nb + 4 && tile < p.n_tiles) p.tiles[lane * p.n_tiles + tile] = col;
-  if (lane < nb && my_edges) atomicAdd(&edges[lane], (unsigned long long)my_edges);
+  if (lane < nb + 4 + N_LISTS && tile < p.n_tiles) p.tiles[lane * p.n_tiles + tile] = col;
+  if (lane < N_LISTS && my_edges) atomicAdd(&edges[lane], (unsigned long long)my_edges);
   __syncthreads();
   if (threadIdx.x < IT_MAX_BUCKETS && edges[threadIdx.x])
     atomicAdd(reinterpret_cast<unsigned long long *>(p.totals + SPLIT_COLS + threadIdx.x), edges[threadIdx.x]);
@@ -286,7 +299,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_emit_kernel(SplitParams p
   }
   // lane c: the running value of column c; for a bucket or list counted from the start of all of them
   int64_t run = 0;
-  if (lane < 2 * nb + 4) {
+  if (lane < nb + 4 + N_LISTS) {
     run = p.tiles[lane * p.n_tiles + tile];
     const int first = lane < nb ? 0 : (lane >= nb + 4 ? nb + 4 : lane);
     for (int k = first; k < lane; ++k) run += p.totals[k];
@@ -308,7 +321,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_emit_kernel(SplitParams p
     const int64_t v = v0 + i * 32;
     const VertexRows r = rows_of(d[i], p);
     const bool is_long = d[i] > p.long_above;
-    const unsigned lng = __ballot_sync(0xffffffffu, is_long), mine = bucket_mask(r.kb, nb, lane);
+    const unsigned lng = __ballot_sync(0xffffffffu, one_by_one(d[i], r, p)), mine = bucket_mask(r.kb, nb, lane);
     const unsigned same = __match_any_sync(0xffffffffu, r.kb);
     unsigned todo = __ballot_sync(0xffffffffu, v < p.n);
     int64_t row = 0, pos = 0, at = 0;   // first row; position in the buckets / in the lists
@@ -329,11 +342,23 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_emit_kernel(SplitParams p
       const int64_t l_row = __shfl_sync(0xffffffffu, run, nb), l_k = __shfl_sync(0xffffffffu, run, nb + 2);
       const int64_t l_piece = __shfl_sync(0xffffffffu, run, nb + 3), l_a = __shfl_sync(0xffffffffu, run, c.ka);
       const int64_t l_b = __shfl_sync(0xffffffffu, run, c.kb) + (c.ka == c.kb ? c.rem : 0);
+      const int64_t l_at = __shfl_sync(0xffffffffu, run, nb + 4 + c.kl);
       if (lane == l) {
-        row = l_row; pos = l_b;
-        p.long_owners[l_k] = (int32_t)v;
-        p.piece_ptr[l_k] = l_piece;
-        p.info[l_k] = LongInfo{l_row, l_a, l_b};
+        row = l_row; pos = l_b; at = l_at;
+        if (is_long) {
+          p.long_owners[l_k] = (int32_t)v;
+          p.piece_ptr[l_k] = l_piece;
+          p.info[l_k] = LongInfo{l_row, l_a, l_b};
+        }
+      }
+      if (c.np == 0) {   // its groups (those of long vertices: long_rows_kernel)
+        const int64_t s0 = __shfl_sync(0xffffffffu, j0[i], l), base = __shfl_sync(0xffffffffu, d[i], l) / c.ng;
+        const int32_t owner = (int32_t)(v - lane + l);
+        for (int64_t g = lane; g < c.ng; g += 32) {
+          p.shadow_indptr[l_row + g] = s0 + g * base + (g < c.rem ? g : c.rem);
+          p.shadow_owner[l_row + g] = owner;
+          p.bucket_rows[g < c.rem ? l_a + g : l_b + (g - c.rem)] = (int32_t)(l_row + g);
+        }
       }
       add_long(run, c, nb, lane);
       todo &= ~((2u << l) - 1u);   // (l = 31: 2u << 31 = 0, nothing left)
@@ -465,9 +490,9 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   p.n_tiles = (n + SPLIT_TILE - 1) / SPLIT_TILE;
   const unsigned split_blocks = (unsigned)((p.n_tiles + SPLIT_THREADS / 32 - 1) / (SPLIT_THREADS / 32));
   // degree buckets: {0, 8, 32, 256, 1024, everything longer}
-  const int64_t fixed[5] = {0, 8, 32, 256, 1024};
+  const int64_t fixed[N_FIXED] = {0, 8, 32, 256, 1024};   // (list_of)
   p.B.nb = 0;
-  for (int i = 0; i < 5; ++i)
+  for (int i = 0; i < N_FIXED; ++i)
     if (T <= 0 || fixed[i] < T) p.B.b[p.B.nb++] = fixed[i];
   p.B.b[p.B.nb++] = T > 0 ? T : INT64_MAX;
 
@@ -479,7 +504,6 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   p.piece_max = 512;
   // small graphs: a warp's longest row is the time of the launch (120 edges per warp on average at 420k edges)
   if (it_small_graph(g)) p.long_above = p.piece_min = p.piece_max = 128;
-  if (T > 0 && T < p.long_above) p.long_above = T;
 
   // at most one row per vertex and one more per T edges, a long vertex per long_above edges, a piece per piece_min of them
   // and one more each; only where that is far above the number of vertices are they counted before the arrays are laid out
@@ -499,7 +523,7 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
     IT_CUDA_TRY(cudaMemsetAsync(p.totals, 0, (size_t)((char *)p.tiles - (char *)p.totals), st));
     if (n > 0) {
       IT_LAUNCH(IT_K_SPLIT_SCAN, 0, 0, st, split_count_kernel<<<split_blocks, SPLIT_THREADS, 0, st>>>(p));
-      IT_LAUNCH(IT_K_SPLIT_SCAN, 0, 0, st, split_scan_kernel<<<(unsigned)(2 * p.B.nb + 4), 1024, 0, st>>>(p));
+      IT_LAUNCH(IT_K_SPLIT_SCAN, 0, 0, st, split_scan_kernel<<<(unsigned)(p.B.nb + 4 + N_LISTS), 1024, 0, st>>>(p));
     }
     IT_CUDA_TRY(cudaGetLastError());
     return IT_OK;
@@ -549,16 +573,16 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   g->n_long = h[nb + 2];
   g->n_partial_rows = h[nb + 3];
   g->n_buckets = nb;
-  g->n_lists = nb + 1;
+  g->n_lists = N_LISTS + 1;
   g->h_list_offsets[0] = 0;
-  for (int k = 0; k < nb; ++k) {
+  for (int k = 0; k < N_LISTS; ++k) {
     g->h_list_offsets[k + 1] = g->h_list_offsets[k] + h[nb + 4 + k];
     g->h_list_edges[k] = h[SPLIT_COLS + k];
-    g->list_bounds[k] = p.B.b[k] < p.long_above ? p.B.b[k] : p.long_above;   // whole vertices have no more edges
+    g->list_bounds[k] = k < N_FIXED && fixed[k] < p.long_above ? fixed[k] : p.long_above;   // whole vertices have no more edges
   }
-  g->h_list_offsets[nb + 1] = n + (g->n_partial_rows - g->n_long);
-  g->h_list_edges[nb] = h[SPLIT_COLS + IT_MAX_BUCKETS - 1];
-  g->list_bounds[nb] = p.piece_max;
+  g->h_list_offsets[N_LISTS + 1] = n + (g->n_partial_rows - g->n_long);
+  g->h_list_edges[N_LISTS] = h[SPLIT_COLS + IT_MAX_BUCKETS - 1];
+  g->list_bounds[N_LISTS] = p.piece_max;
   for (int i = 0; i < IT_MAX_BUCKETS; ++i) g->bucket_bounds[i] = i < p.B.nb ? p.B.b[i] : 0;
   return IT_OK;
 }

@@ -63,6 +63,21 @@ def test_few_vertices_of_many_edges(n, deg, kind):
     check_against_oracle(w, got, label=(n, deg, kind), exact=False)
 
 
+@pytest.mark.parametrize("n", [900, N])
+@pytest.mark.parametrize("kind", ["sum", "gat"])
+def test_the_threshold_changes_no_bit(n, kind):
+    """What is gathered in pieces does not depend on the shadow rows: thresholds far below, between and above the bounds of the lists."""
+    layer = make_gat_layer(36, "elu", 32, 4, 8, "f32") if kind == "gat" else make_sage_layer(36, "sum", "relu", 32, 16, "f32", weights=True, allow_reorder=False)
+    w = small_workload(37, n, 40, "f32", [layer], hubs=HUBS, weights=True)
+    base, d = run_device(w, threshold=0)
+    check_against_oracle(w, base, label=(n, kind), exact=False)
+    deg = np.diff(w.indptr)
+    for T in (1, 7, 8, 9, 32, 33, 300, 1024, 1025, 4096, 20000):
+        rows, split = B.it_split_hubs(d.graph, T)
+        assert rows == int(np.maximum(1, -(-deg // T)).sum()) and split == int((deg > T).sum())
+        assert np.array_equal(d.infer().double().cpu().numpy(), base), T
+
+
 def test_self_term_and_bias_of_rows_without_edges():
     for layer in (make_sage_layer(25, "mean", "elu", 64, 32, "bf16"), make_plain_layer(26, "gcn", "elu", 64, 32, "bf16")):
         w = small_workload(27, N, 4, "bf16", [layer], hubs=HUBS[:6], p_zero=0.9)
