@@ -94,7 +94,8 @@ __global__ void __launch_bounds__(256) validate_indices_kernel(const int32_t *__
 // one block per row of up to T edges in vertex order: 5M vertices / 100M edges, GAT, 13.1 -> 11.7 ms; 20M / 200M with 100 hubs
 // of 1M edges, max pooling, 20.0 -> 17.4; 2M / 40M, fp32 sums, 6.6 -> 5.95; 25M / 375M, mean, 23.3 -> 22.6.
 // A piece is a 64th of its vertex (it then spans a 64th of the table), at least 128 edges (its fp32 partial result costs a row
-// written and a row read: 3 % of 128 rows; 64 and 32 edges cost 1 to 2 % more on GAT) and at most 512 (one warp walks it).
+// written and a row read: 3 % of 128 rows; 64 and 32 edges cost 1 to 2 % more on GAT) and at most 512 (one warp walks it), more only
+// where a vertex would have more than PIECES_MOST of them.
 // Source tables of fewer than 2^17 rows fit the cache whatever the order: pieces of at least 256 edges.
 // Bound by reading indptr twice and writing 36 bytes per row; a scan per bucket (each over every row, three launches with a
 // read of two 8-byte bounds per row) took 3.2 ms of device time for 5M vertices and six buckets, this one 3.0 with
@@ -105,6 +106,7 @@ constexpr int SPLIT_TILE = 32 * SPLIT_ITEMS;                      // a tile is o
 constexpr int SPLIT_COLS = 2 * IT_MAX_BUCKETS + 4;
 constexpr int N_FIXED = 5;                                        // bounds of the buckets below T, of the lists below long_above
 constexpr int N_LISTS = N_FIXED + 1;                              // lists of whole vertices
+constexpr int64_t PIECES_MOST = 8192;                             // of one vertex (or one more): one block or warp folds them
 constexpr int PIECE_BINS = 256;                                   // steps of the order in which pieces are walked
 
 struct Bounds { int64_t b[IT_MAX_BUCKETS]; int nb; };
@@ -137,7 +139,8 @@ struct SplitParams {
 };
 
 __device__ __forceinline__ int64_t pieces_of(int64_t d, const SplitParams &p) {
-  const int64_t by_share = d / 64, least = by_share < p.piece_min ? p.piece_min : by_share, len = least > p.piece_max ? p.piece_max : least;
+  const int64_t by_share = d / 64, least = by_share < p.piece_min ? p.piece_min : by_share, most = least > p.piece_max ? p.piece_max : least;
+  const int64_t len = d / PIECES_MOST > most ? d / PIECES_MOST : most;
   return (d + len - 1) / len;
 }
 

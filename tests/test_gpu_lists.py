@@ -78,6 +78,15 @@ def test_the_threshold_changes_no_bit(n, kind):
         assert np.array_equal(d.infer().double().cpu().numpy(), base), T
 
 
+@pytest.mark.parametrize("kind", ["mean", "gat"])
+def test_a_vertex_of_more_pieces_than_one_block_should_fold(kind):
+    """5M edges on one vertex: pieces longer than 512 edges, and a remainder."""
+    layer = make_gat_layer(38, "none", 8, 1, 16, "f32") if kind == "gat" else make_sage_layer(38, kind, "none", 8, 16, "f32", allow_reorder=False)
+    w = small_workload(39, N, 4, "f32", [layer], hubs=(5_000_011, 8192 * 512, 8192 * 512 + 1, 5000))
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=kind, exact=False)
+
+
 def test_self_term_and_bias_of_rows_without_edges():
     for layer in (make_sage_layer(25, "mean", "elu", 64, 32, "bf16"), make_plain_layer(26, "gcn", "elu", 64, 32, "bf16")):
         w = small_workload(27, N, 4, "bf16", [layer], hubs=HUBS[:6], p_zero=0.9)
