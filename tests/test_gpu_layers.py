@@ -301,18 +301,20 @@ def test_buckets_of_very_short_rows(dtype, fi, max_deg):
     for op, weights, fo in (("mean", False, fi), ("sum", True, fi), ("max", False, fi), ("min", True, fi),
                             ("mean", False, fi // 2), ("sum", True, fi // 2)):
         layer = make_sage_layer(7, op, "relu", fi, fo, dtype, weights=weights)
-        w = small_workload(8, 4000, max_deg, dtype, [layer], hubs=(300,), weights=weights, threshold=128, p_zero=0.1)
-        got, d = run_device(w)
-        B.it_graph_check(d.graph)
-        check_against_oracle(w, got, label=(dtype, fi, max_deg, op, weights, fo))
+        for n in (4000, 140_000):   # one kernel for all rows, and kernels by row length
+            w = small_workload(8, n, max_deg, dtype, [layer], hubs=(300,), weights=weights, threshold=128, p_zero=0.1)
+            got, d = run_device(w)
+            B.it_graph_check(d.graph)
+            check_against_oracle(w, got, label=(dtype, fi, max_deg, op, weights, fo, n))
 
 
-def test_very_short_rows_beyond_one_sweep_of_the_grid():
+@pytest.mark.parametrize("n", [60_000, 160_000])   # one kernel for all rows, and kernels by row length
+def test_very_short_rows_beyond_one_sweep_of_the_grid(n):
     """More rows of at most 3 edges than the resident lane groups of the whole GPU take in one sweep (148 SMs x 3
     CTAs x 32 lane groups), so that every lane group walks several rows and the row records loaded ahead run past
     the end of the bucket."""
     layer = make_sage_layer(9, "mean", "none", 64, 64, "bf16")
-    w = small_workload(10, 60_000, 3, "bf16", [layer], p_zero=0.05)
+    w = small_workload(10, n, 3, "bf16", [layer], p_zero=0.05)
     got, d = run_device(w)
     B.it_graph_check(d.graph)
     check_against_oracle(w, got)

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from gpu_util import check_against_oracle, make_gat_layer, make_plain_layer, make_sage_layer, run_device, small_workload
+from gpu_util import check_against_oracle, make_gat_layer, make_msg_layer, make_plain_layer, make_sage_layer, run_device, small_workload
 from paper_2307_00228_b200 import binding as B
 from paper_2307_00228_b200 import host
 
@@ -79,6 +79,58 @@ def test_the_threshold_changes_no_bit(n, kind):
 
 
 @pytest.mark.parametrize("kind", ["mean", "gat"])
+@pytest.mark.parametrize("dtype,fi", [("bf16", 64), ("bf16", 40), ("bf16", 264), ("f32", 32), ("f32", 132)])
+@pytest.mark.parametrize("op,weights", [("max", False), ("min", False), ("min", True), ("sum", True)])
+def test_every_reduce(dtype, fi, op, weights):
+    """Plain maxima and minima (packed pairs in bf16), weighted ones and weighted sums, rows that fill their lane group and rows that do
+    not, rows of more than one column chunk; very short, short and long rows, and pieces."""
+    layer = make_sage_layer(40, op, "none", fi, 16, dtype, weights=weights, allow_reorder=False)
+    w = small_workload(41, N, 7, dtype, [layer], hubs=HUBS, weights=weights, threshold=300)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(dtype, fi, op, weights), exact=False)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("kind", ["edge_features", "messages", "gat_edge_logits", "wide"])
+def test_rows_in_edge_order_and_column_chunks(dtype, kind):
+    """Edge features next to the source rows, learned messages, attention logits with an edge term, rows of more than 512 bytes."""
+    if kind == "edge_features":
+        layer = make_sage_layer(42, "mean", "relu", 32, 16, dtype, edge_dim=16)
+    elif kind == "messages":
+        layer = make_msg_layer(43, "max", "relu", 32, 32, 16, dtype, edge_dim=8)
+    elif kind == "gat_edge_logits":
+        layer = make_gat_layer(44, "elu", 32, 4, 16, dtype, edge_dim=8)
+    else:
+        layer = make_sage_layer(45, "mean", "relu", 320, 16, dtype, allow_reorder=False)
+    w = small_workload(46, N, 6, dtype, [layer], hubs=HUBS, threshold=64, edge_dim=layer.edge_dim)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(dtype, kind), exact=False)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("op", ["sum", "mean", "max", "min"])
+def test_raw_partial_results(dtype, op):
+    """What a part hands to the others, by value: whole numbers, so that fp32 sums are exact in any order."""
+    layer = make_sage_layer(47, op, "none", 32, 16, dtype, allow_reorder=False)
+    w = small_workload(48, N, 6, "f32", [layer], hubs=HUBS, p_zero=0.5)
+    w.x, w.dtype = np.round(w.x * 2).astype(np.float32), "f32"
+    d = host.upload(w)
+    x = d.x.to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    lay = host.layer_to_device(layer, dtype)
+    out = torch.full((w.n, 32), float("nan"), device="cuda")
+    ws = torch.empty(B.it_workspace_bytes(d.graph, [lay]), dtype=torch.uint8, device="cuda")
+    B.it_layer_gather(d.graph, lay, x, None, 0, True, out, ws)
+    rows = torch.from_numpy(np.repeat(np.arange(w.n), np.diff(w.indptr))).cuda()
+    src = d.x[torch.from_numpy(w.indices.astype(np.int64)).cuda()]
+    start = {"max": float("-inf"), "min": float("inf")}.get(op, 0.0)
+    want = torch.full((w.n, 32), start, device="cuda")
+    if op in ("max", "min"):
+        want.scatter_reduce_(0, rows[:, None].expand(-1, 32), src, "amax" if op == "max" else "amin")
+    else:
+        want = want.double().index_add_(0, rows, src.double()).float()
+    assert torch.equal(out, want)
+
+
 def test_a_vertex_of_more_pieces_than_one_block_should_fold(kind):
     """5M edges on one vertex: pieces longer than 512 edges, and a remainder."""
     layer = make_gat_layer(38, "none", 8, 1, 16, "f32") if kind == "gat" else make_sage_layer(38, kind, "none", 8, 16, "f32", allow_reorder=False)

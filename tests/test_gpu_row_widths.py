@@ -1,5 +1,6 @@
 """Rows of 80 bytes and more that are no power of two fill a lane group up to its last lanes: the narrowest and widest
-row of every group, in buckets of every length class (very short, short, one warp, one block), against the oracle."""
+row of every group, with rows of every length in one kernel (graphs of 900 vertices; the kernels by row length:
+test_gpu_lists.py), against the oracle."""
 import pytest
 
 from gpu_util import check_against_oracle, make_sage_layer, run_device, small_workload
