@@ -463,8 +463,8 @@ def measure(name: str, args, steps: int, world: int, rank: int, dev, full: bool)
     check("per-layer loops")
     rec["edges_per_sec_per_layer"] = layer_stats
 
-    # ---- the same pass with no vertex split (threshold 0: hubs keep their whole in-edge segment as one row), so that
-    # what the shadow rows buy on this workload is a measured figure; the graph is split again at its threshold after
+    # ---- the same pass with the graph split at threshold 0.  The gather cuts long vertices into pieces of its own at every
+    # threshold, so this is the same work: the figure shows that the shadow rows cost the pass nothing.  The graph is split again after
     if full and w.threshold > 0 and d.n_split_owners > 0:
         B.it_split_hubs(d.graph, 0)
         if B.it_workspace_bytes(d.graph, d.layers) <= d.workspace.numel():

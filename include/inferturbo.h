@@ -12,9 +12,10 @@
  *     enqueued on it; a call synchronises that stream only where it must read a status
  *     or a count back (it_graph_create, it_split_hubs).
  *   - Matrices are row-major and dense.  Feature rows (layer inputs and outputs, edge features) must be a
- *     multiple of 16 bytes; the pooling layers and GCN take any such width (rows other than 16, 32, ..., 512
- *     bytes are gathered in column chunks of those widths), GAT rows must be one of those widths.  The dense
- *     transform runs on the tensor cores when out_dim is a multiple of 16 and on the CUDA cores otherwise.
+ *     multiple of 16 bytes; the pooling layers and GCN take any such width (rows of more than 512 bytes are gathered
+ *     in column chunks of 512), GAT rows must be 16, 32, 64, 128, 256 or 512 bytes.  The dense
+ *     transform runs on the tensor cores for every bf16 width, and for fp32 widths that are a multiple of 16, as far as the
+ *     weights fit the SMs' shared memory, and on the CUDA cores otherwise.
  *   - Errors are return codes only: nothing throws, aborts or traps the device.  On
  *     error no output is defined.  it_status_string() names a code;
  *     it_last_error_message() gives the detail of the calling thread's last failure.
@@ -89,8 +90,9 @@ typedef enum { IT_ACT_NONE = 0, IT_ACT_RELU = 1, IT_ACT_ELU = 2 } it_act;
  * GAT with edge features (op = GAT, edge_dim > 0): the edge's features enter its attention logit,
  *       e = LeakyReLU_slope( att_src[k] . z_u^k + att_dst[k] . z_v^k + att_edge[k] . e_{v,u} ),
  *   the messages stay z_u.  One fp32 logit term per edge and head (source score + edge share) is materialised in the
- *   workspace ([n_edges, heads]); shapes that the batched reduce does not take (heads other than 1, 2, 4 or 8, rows
- *   narrower than 128 bytes) also a copy of the message row of every edge ([n_edges, out_dim] feat_dtype).
+ *   workspace ([n_edges, heads]); shapes that the batched reduce does not take (heads other than 1, 2, 4 or 8, or a head
+ *   of no multiple of 16 bytes; rows narrower than 128 bytes but those of 64 bytes and up to 4 heads) also a copy of the
+ *   message row of every edge ([n_edges, out_dim] feat_dtype).
  *
  * Learned messages (msg_dim > 0; pooling layers and GCN): the general apply_edge of the Scatter stage (Section
  *   "InferTurbo Abstraction"; M of Eq. (1)) as one dense layer on the source state and the edge's features,
@@ -164,7 +166,8 @@ it_status it_graph_set_edge_features(it_graph *g, const void *edge_feat, int32_t
  * does not fit it.)
  * Also builds the degree buckets: shadow rows partitioned stably by length class
  * (bounds from it_graph_get_split).  Rebuilds everything derived; edge arrays are not
- * permuted.  out_n_rows / out_n_split_owners may be NULL.  Synchronises `stream`.
+ * permuted.  out_n_rows / out_n_split_owners may be NULL.  Synchronises `stream`; waits for the device where the arrays
+ * of the present split have been used (by a forward pass, or handed out by it_graph_get_split), as cudaFree does.
  */
 it_status it_split_hubs(it_graph *g, int64_t threshold, void *stream, int64_t *out_n_rows,
                         int64_t *out_n_split_owners);
