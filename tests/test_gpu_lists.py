@@ -78,7 +78,6 @@ def test_the_threshold_changes_no_bit(n, kind):
         assert np.array_equal(d.infer().double().cpu().numpy(), base), T
 
 
-@pytest.mark.parametrize("kind", ["mean", "gat"])
 @pytest.mark.parametrize("dtype,fi", [("bf16", 64), ("bf16", 40), ("bf16", 264), ("f32", 32), ("f32", 132)])
 @pytest.mark.parametrize("op,weights", [("max", False), ("min", False), ("min", True), ("sum", True)])
 def test_every_reduce(dtype, fi, op, weights):
@@ -131,6 +130,7 @@ def test_raw_partial_results(dtype, op):
     assert torch.equal(out, want)
 
 
+@pytest.mark.parametrize("kind", ["mean", "gat"])
 def test_a_vertex_of_more_pieces_than_one_block_should_fold(kind):
     """5M edges on one vertex: pieces longer than 512 edges, and a remainder."""
     layer = make_gat_layer(38, "none", 8, 1, 16, "f32") if kind == "gat" else make_sage_layer(38, kind, "none", 8, 16, "f32", allow_reorder=False)
