@@ -5,6 +5,8 @@
 // M = max(m, m'), l e^(m-M) + l' e^(m'-M), acc e^(m-M) + acc' e^(m'-M) — so the groups of a split
 // hub are reduced independently into partial states and merged in edge order, exactly like
 // the partial sums of the plain gather.  The edge streaming lives in stream.cuh.
+#include <type_traits>
+
 #include "stream.cuh"
 
 namespace {
@@ -165,6 +167,7 @@ struct MergeState {
 
 template <typename T, int C, bool EDGES>
 __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p) {
+  using Index = std::conditional_t<EDGES, int64_t, int>;   // (pieces are counted with 31 bits)
   constexpr int WARPS = THREADS / 32;
   __shared__ MergeState<C> red[WARPS][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -172,8 +175,8 @@ __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p
   for (int64_t k = blockIdx.x; k < p.n_long; k += gridDim.x) {
     const int64_t v = __ldg(p.long_owners + k);
     const int64_t p0 = EDGES ? __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v)) : __ldg(p.piece_ptr + k);
-    const int64_t n = (EDGES ? __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v + 1)) : __ldg(p.piece_ptr + k + 1)) - p0;
-    const int64_t per = (n + WARPS - 1) / WARPS, a = warp * per < n ? warp * per : n, b = a + per < n ? a + per : n;
+    const Index n = (Index)((EDGES ? __ldg(p.shadow_indptr + __ldg(p.owner_indptr + v + 1)) : __ldg(p.piece_ptr + k + 1)) - p0);
+    const Index per = (n + WARPS - 1) / WARPS, a = warp * per < n ? warp * per : n, b = a + per < n ? a + per : n;
     for (int c0 = 0; c0 < p.dim; c0 += 32 * C) {
       const int c = c0 + lane * C;
       MergeState<C> s;
@@ -182,17 +185,17 @@ __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p
         const int head = c / p.head_dim;
         const float *P = p.partials + p0 * stride;
         const float sd = EDGES ? __ldg(p.scores_dst + v * (2 * p.heads) + p.heads + head) : 0.f;
-        auto load = [&](int64_t g, MergeState<C> &x) {
+        auto load = [&](Index g, MergeState<C> &x) {
           if constexpr (EDGES) {
             using Slice = RowSlice<T, C * (int)sizeof(T)>;
-            const int64_t j = p0 + g, u = p.indices ? (int64_t)__ldg(p.indices + j) : j;
+            const int64_t j = p0 + (int64_t)g, u = p.indices ? (int64_t)__ldg(p.indices + j) : j;
             const float e = __ldg(p.scores + (p.per_edge_scores ? j : u) * p.stride + head) + sd;
             x.m = e > 0.f ? e : p.slope * e;
             x.l = 1.f;
             Slice::unpack(Slice::load(reinterpret_cast<const char *>(p.z) + (u * p.dim + c) * (int64_t)sizeof(T)), x.acc);
             return;
           }
-          const float *row = P + g * stride;
+          const float *row = P + (int64_t)g * stride;
           x.m = __ldg(row + p.dim + head);
           x.l = __ldg(row + p.dim + p.heads + head);
           if constexpr (C == 4) {
@@ -203,8 +206,8 @@ __global__ void __launch_bounds__(THREADS) gat_combine_kernel(GatCombineParams p
             for (int i = 0; i < C; ++i) x.acc[i] = __ldcs(row + c + i);
           }
         };
-        int64_t g = a;
-        auto merge_to = [&](MergeState<C> &t, int64_t end) {
+        Index g = a;
+        auto merge_to = [&](MergeState<C> &t, Index end) {
           for (; g + 4 <= end; g += 4) {
             MergeState<C> x[4];
 #pragma unroll
