@@ -519,9 +519,14 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   auto reserve = [&](size_t bytes) -> it_status {   // grow the graph's allocation; what it holds is not kept
     if (bytes <= g->slab_bytes) return IT_OK;
     slab_free(g);
-    bytes += bytes / 8;   // room for the few more rows of another threshold
-    IT_CUDA_TRY(cudaMalloc(&g->slab, bytes));
-    g->slab_bytes = bytes;
+    size_t room = bytes + bytes / 8;   // for the few more rows of another threshold, where the device has it
+    if (cudaMalloc(&g->slab, room) != cudaSuccess) {
+      cudaGetLastError();
+      g->slab = nullptr;
+      room = bytes;
+      IT_CUDA_TRY(cudaMalloc(&g->slab, room));
+    }
+    g->slab_bytes = room;
     return IT_OK;
   };
   auto count = [&]() -> it_status {
