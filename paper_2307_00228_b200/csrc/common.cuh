@@ -57,8 +57,8 @@ void it_set_error(const char *fmt, ...);
 
 // ----------------------------------------------------------------------------- instrumentation
 enum it_kernel_id {
-  IT_K_VALIDATE = 0, IT_K_SPLIT_SCAN, IT_K_SPLIT_FILL, IT_K_BUCKET_SCAN, IT_K_PREP, IT_K_GATHER_CTA, IT_K_GATHER_FLAT,
-  IT_K_GATHER_EMPTY, IT_K_COMBINE, IT_K_GEMM_FP32, IT_K_GEMM_TC, IT_K_GAT_CTA, IT_K_GAT_FLAT, IT_K_GAT_EMPTY,
+  IT_K_VALIDATE = 0, IT_K_SPLIT_SCAN, IT_K_SPLIT_FILL, IT_K_BUCKET_SCAN, IT_K_PREP, IT_K_GATHER_FLAT,
+  IT_K_GATHER_EMPTY, IT_K_COMBINE, IT_K_GEMM_FP32, IT_K_GEMM_TC, IT_K_GAT_FLAT, IT_K_GAT_EMPTY,
   IT_K_EDGE_MSG, IT_K_AGG_FINISH, IT_K_GEMM2_TC, IT_K_GATHER_SMALL, IT_K_GAT_SMALL,
   IT_K_COUNT
 };

@@ -72,8 +72,7 @@ struct SagePolicy {
     }
     float f[VEC];
     Slice::unpack(raw, f);
-    if constexpr (PACKED) {
-    } else if constexpr (RED == RED_SUM && !WEIGHTED && VEC % 2 == 0) {   // two accumulators per instruction (measured: 1 % on the
+    if constexpr (RED == RED_SUM && !WEIGHTED && VEC % 2 == 0) {   // two accumulators per instruction (measured: 1 % on the
 #pragma unroll                                                      // 128-byte rows; with a weight the pair set-up eats the gain)
       for (int k = 0; k < VEC; k += 2) add_f32x2(st[k], st[k + 1], f[k], f[k + 1]);
     } else {
@@ -282,9 +281,7 @@ it_status launch_policy(const it_gather_args &a, StreamParams sp, cudaStream_t s
   auto launch = [&]<bool PAD>() {
     return launch_buckets<T, SB, LPR, PAD>(g, sp, pol, bytes_of, IT_K_GATHER_FLAT, IT_K_GATHER_EMPTY, a.counters, st);
   };
-  if constexpr (SB == 16) {
-    if (a.dim * (int)sizeof(T) != SB * LPR) return launch.template operator()<true>();
-  }
+  if (a.dim * (int)sizeof(T) != SB * LPR) return launch.template operator()<true>();
   return launch.template operator()<false>();
 }
 
@@ -300,7 +297,7 @@ it_status launch_lpr(const it_gather_args &a, StreamParams sp, bool *folded, cud
     return launch_small<T, RED_SUM>(a, sp, st);
   }
   const bool w = a.use_edge_weights != 0;
-  return dispatch_row_bytes(row_bytes, true, [&]<int SB, int LPR>() {
+  return dispatch_wide_rows(row_bytes, [&]<int SB, int LPR>() {
     if (a.op == IT_GATHER_MAX) return w ? launch_policy<T, SB, LPR, RED_MAX, true>(a, sp, st) : launch_policy<T, SB, LPR, RED_MAX, false>(a, sp, st);
     if (a.op == IT_GATHER_MIN) return w ? launch_policy<T, SB, LPR, RED_MIN, true>(a, sp, st) : launch_policy<T, SB, LPR, RED_MIN, false>(a, sp, st);
     return w ? launch_policy<T, SB, LPR, RED_SUM, true>(a, sp, st) : launch_policy<T, SB, LPR, RED_SUM, false>(a, sp, st);

@@ -7,14 +7,15 @@
 //
 // Work decomposition.  A feature row is cut into lane slices of SB bytes and is LPR = row bytes / SB
 // lanes wide; rows are bucketed by length and each bucket gets the kernel that suits it.
-//   * stream_rows_chunk_kernel (stream_chunk.cuh; rows of 80 bytes and more, more than a few dozen edges): one warp per
-//     row, chunk after chunk without a break between rows.
-//   * stream_rows_ring_kernel (stream_ring.cuh): a warp walks the edges of a batch of rows as one flat
-//     stream and stages the source rows through a per-warp ring in shared memory with cp.async.
-//   * stream_short_rows_pipe_kernel, stream_tiny_rows_kernel (the same widths up to 256 bytes, rows of at most a few
-//     dozen edges): one group of 8 or 16 lanes per row, eight row loads back to back, no edge stream.
-//   * stream_rows_kernel (rows narrower than 128 bytes): a *group* of LPR lanes takes a batch of rows
-//     and walks the batch's edges as one flat stream with UNROLL rows in flight per lane in registers.
+//   * stream_rows_chunk_kernel (stream_chunk.cuh; pooling, more than a few dozen edges): one warp per row, chunk after
+//     chunk without a break between rows.
+//   * stream_rows_ring_kernel (stream_ring.cuh; the per-edge softmax, short rows of more than 256 bytes, and pooling rows
+//     that are few): a warp walks the edges of a row, or of a batch of short ones, as one flat stream and stages the source
+//     rows through a per-warp ring in shared memory with cp.async.
+//   * stream_short_rows_pipe_kernel, stream_tiny_rows_kernel (rows of up to 256 bytes, at most a few dozen edges): one
+//     group of 8 or 16 lanes per row, eight row loads back to back, no edge stream.
+//   * stream_rows_kernel (attention rows narrower than 128 bytes whose shape the batched reduce does not take): a *group* of
+//     LPR lanes takes a batch of rows and walks its edges as one flat stream with UNROLL rows in flight per lane in registers.
 //   * rows without edges: gather.cu.
 //
 // Policy interface (all __device__):
@@ -681,9 +682,12 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
       if constexpr (RING) {   // a whole warp per batch
         constexpr int smem = (THREADS / 32) * ring_bytes_per_warp<SB, Policy::HAS_EXTRA>();
         static std::atomic<uint64_t> configured{0}, configured1{0};   // per template instance: one bit per device ordinal
-        const bool single = IT_RING_SINGLE_ROW && br == 1;
+        constexpr bool ALL_SINGLE = IT_RING_SINGLE_ROW && SB == 16 && LPR <= 16;   // batches of short rows have kernels of their own
+        const bool single = ALL_SINGLE || (IT_RING_SINGLE_ROW && br == 1);
         if (single) IT_TRY(allow_dynamic_smem(stream_rows_ring_kernel<T, SB, LPR, Policy, true, PAD>, smem, configured1));
-        else IT_TRY(allow_dynamic_smem(stream_rows_ring_kernel<T, SB, LPR, Policy, false, PAD>, smem, configured));
+        if constexpr (!ALL_SINGLE) {
+          if (!single) IT_TRY(allow_dynamic_smem(stream_rows_ring_kernel<T, SB, LPR, Policy, false, PAD>, smem, configured));
+        }
         p.batch_rows = br;
         const int64_t batches = (rows + br - 1) / br;
         // with a counter every CTA is resident from the start and its warps claim batches as they finish (rows of one
@@ -695,7 +699,9 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
         const int64_t per_warp = batches / ((int64_t)blocks * (THREADS / 32));
         p.claim = (int)(per_warp / IT_RING_CLAIMS_PER_WARP < 1 ? 1 : (per_warp / IT_RING_CLAIMS_PER_WARP > 4096 ? 4096 : per_warp / IT_RING_CLAIMS_PER_WARP));
         if (single) IT_LAUNCH(kid_rows, bytes, 0, st, stream_rows_ring_kernel<T, SB, LPR, Policy, true, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
-        else IT_LAUNCH(kid_rows, bytes, 0, st, stream_rows_ring_kernel<T, SB, LPR, Policy, false, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
+        if constexpr (!ALL_SINGLE) {
+          if (!single) IT_LAUNCH(kid_rows, bytes, 0, st, stream_rows_ring_kernel<T, SB, LPR, Policy, false, PAD><<<blocks, THREADS, smem, st>>>(p, pol));
+        }
         p.counter = nullptr;
       } else {                                // a group of LPR lanes per batch
         if (br > LPR) br = LPR;
@@ -718,12 +724,17 @@ it_status launch_buckets(const it_graph *g, StreamParams p, const Policy &pol, B
 // 16-byte pieces alone moved a 32-byte sector each and an edge index).  Rows of 16 to 64 bytes in lane groups of their own
 // width, staged in registers, kept too little in flight: 5M vertices, 60M edges, 64-byte
 // rows 2.90 -> 0.98 ms, 32-byte rows 2.45 -> 1.01; 64-byte GAT rows 4.86 -> 1.73.
-// `wide`: 16-byte slices do not straddle two attention heads; else slices of a 32nd of the row.
+template <class F>
+it_status dispatch_wide_rows(int row_bytes, F f) {
+  if (row_bytes > 256) return f.template operator()<16, 32>();
+  if (row_bytes > 128) return f.template operator()<16, 16>();
+  return f.template operator()<16, 8>();
+}
+// The same for attention heads, whose 16-byte slices (`wide`) may not straddle two of them; else slices of a 32nd of the row.
 template <class F>
 it_status dispatch_row_bytes(int row_bytes, bool wide, F f) {
-  if (row_bytes > 256) return f.template operator()<16, 32>();
-  if (row_bytes > 128) return wide ? f.template operator()<16, 16>() : f.template operator()<8, 32>();
-  if (wide) return f.template operator()<16, 8>();
+  if (wide || row_bytes > 256) return dispatch_wide_rows(row_bytes, f);
+  if (row_bytes > 128) return f.template operator()<8, 32>();
   switch (row_bytes) {
     case 128: return f.template operator()<4, 32>();
     case 64: return f.template operator()<4, 16>();
