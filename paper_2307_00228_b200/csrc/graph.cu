@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256) validate_indices_kernel(const int32_t *__
 // of 1M edges, max pooling, 20.0 -> 17.4; 2M / 40M, fp32 sums, 6.6 -> 5.95; 25M / 375M, mean, 23.3 -> 22.6.
 // A piece is a 64th of its vertex (it then spans a 64th of the table), at least 128 edges (its fp32 partial result costs a row
 // written and a row read: 3 % of 128 rows; 64 and 32 edges cost 1 to 2 % more on GAT) and at most 512 (one warp walks it), more only
-// where a vertex would have more than PIECES_MOST of them.
+// where a vertex would have more than PIECES_MOST of them (one block folds them: a single vertex of 20M edges 556 -> 325 us).
 // Source tables of fewer than 2^17 rows fit the cache whatever the order: pieces of at least 256 edges.
 // Bound by reading indptr twice and writing 36 bytes per row; a scan per bucket (each over every row, three launches with a
 // read of two 8-byte bounds per row) took 3.2 ms of device time for 5M vertices and six buckets, this one 3.0 with
