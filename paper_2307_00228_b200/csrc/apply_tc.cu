@@ -223,7 +223,9 @@ struct TcParams {
 // tiles are in flight; with the epilogue's own loads in their place the kernel waited for them: 16M edges, 64 columns, whole layer 2.16 -> 1.95 ms.
 constexpr int TC_ADD_STAGES = 4;
 constexpr int TC_THREADS_ADD = TC_THREADS_BF16 + 128;
-template <bool TF32, bool ADD>
+// STREAM: the weights do not stay in shared memory; the k-block of them that belongs to an operand tile comes with it, in the same
+// stage.  (For weights so large that a CTA could keep few columns of them only: it_tc_columns.)
+template <bool TF32, bool ADD, bool STREAM>
 __global__ void __launch_bounds__(TF32 ? TC_THREADS_TF32 : (ADD ? TC_THREADS_ADD : TC_THREADS_BF16), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_x2,
                const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_o0,
@@ -232,15 +234,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int KB = p.kb1 + p.kb2;
   const int b_tile_bytes = p.nbc * TC_KBLOCK_BYTES;              // one k-block of B (one part)
-  const int b_bytes = (TF32 ? 2 : 1) * KB * b_tile_bytes;
+  constexpr int parts = TF32 ? 2 : 1;                            // fp32 mode: hi and lo of the weights
+  const int b_bytes = STREAM ? 0 : parts * KB * b_tile_bytes;    // resident weights
   constexpr int a_tile_bytes = TC_BM * TC_KBLOCK_BYTES;          // 16 KB
+  const int stage_bytes = a_tile_bytes + (STREAM ? parts * b_tile_bytes : 0);
 
   // shared memory: resident weights | operand stages (bf16 tiles the MMAs read, or raw fp32 tiles the split warps read) |
   // output staging panels | barriers
   unsigned char *base = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char *smem_b = base;
   unsigned char *smem_a = base + b_bytes;   // b_bytes is a multiple of 1024 (nbc is a multiple of 16)
-  unsigned char *smem_out = smem_a + (size_t)p.stages * a_tile_bytes;   // output staging panels (TMA-store epilogue), 1024-byte aligned
+  unsigned char *smem_out = smem_a + (size_t)p.stages * stage_bytes;   // output staging panels (TMA-store epilogue), 1024-byte aligned
   unsigned char *smem_add = smem_out + (size_t)p.out_panels * p.epi_groups * a_tile_bytes;   // ADD: ring of gathered rows, panels like the output's
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem_add + (ADD ? (size_t)TC_ADD_STAGES * p.add_stage_bytes : 0));
   uint64_t *full = bars;                    // [stages]  TMA landed
@@ -267,7 +271,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], TF32 ? 4 : 1);
+      mbar_init(&empty[s], TF32 ? (STREAM ? 5 : 4) : 1);
     }
     for (int s = 0; s < TC_TSTAGES_MAX; ++s) {
       mbar_init(&ready[s], 4);
@@ -312,15 +316,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0 && !p.no_loads) {
-      // the weights of this CTA's columns, once
-      mbar_arrive_expect_tx(b_full, (uint32_t)b_bytes);
       const int bk_elems = TF32 ? 32 : 64;
       // fp32 mode: the hi and the lo tile of a k-block sit next to each other, so that one descriptor covers
       // both as a single operand of 2 nbc columns
-      constexpr int parts = TF32 ? 2 : 1;
-      for (int part = 0; part < parts; ++part)
-        for (int kb = 0; kb < KB; ++kb)
-          tma_load_2d(smem_b + (size_t)(kb * parts + part) * b_tile_bytes, &map_b, kb * bk_elems, part * p.NB + col_base, b_full);
+      if (!STREAM) {   // the weights of this CTA's columns, once
+        mbar_arrive_expect_tx(b_full, (uint32_t)b_bytes);
+        for (int part = 0; part < parts; ++part)
+          for (int kb = 0; kb < KB; ++kb)
+            tma_load_2d(smem_b + (size_t)(kb * parts + part) * b_tile_bytes, &map_b, kb * bk_elems, part * p.NB + col_base, b_full);
+      }
       uint32_t stage = 0, phase = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
@@ -328,9 +332,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
         for (int kb = 0; kb < KB; ++kb) {
           ok = mbar_wait(&empty[stage], phase ^ 1u, abort_flag, p.spin_limit, IT_TC_TMA_BACKOFF);
           if (!ok) break;
-          mbar_arrive_expect_tx(&full[stage], (uint32_t)a_tile_bytes);
-          if (kb < p.kb1) tma_load_2d(smem_a + (size_t)stage * a_tile_bytes, &map_x1, kb * bk_elems, m0, &full[stage]);
-          else tma_load_2d(smem_a + (size_t)stage * a_tile_bytes, &map_x2, (kb - p.kb1) * bk_elems, m0, &full[stage]);
+          unsigned char *to = smem_a + (size_t)stage * stage_bytes;
+          mbar_arrive_expect_tx(&full[stage], (uint32_t)stage_bytes);
+          if (kb < p.kb1) tma_load_2d(to, &map_x1, kb * bk_elems, m0, &full[stage]);
+          else tma_load_2d(to, &map_x2, (kb - p.kb1) * bk_elems, m0, &full[stage]);
+          if (STREAM)
+            for (int part = 0; part < parts; ++part)
+              tma_load_2d(to + a_tile_bytes + part * b_tile_bytes, &map_b, kb * bk_elems, part * p.NB + col_base, &full[stage]);
           if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -348,7 +356,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       const uint32_t fmt = TF32 ? 2u : 1u;
       const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(p.nbc >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
       const uint32_t idesc_wide = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)((2 * p.nbc) >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
-      bool ok = mbar_wait(b_full, 0, abort_flag, p.spin_limit);
+      bool ok = STREAM || mbar_wait(b_full, 0, abort_flag, p.spin_limit);
       uint32_t stage = 0, phase = 0;
       uint32_t acc = 0, acc_phase = 0;
       uint32_t ts = 0, tphase = 0;   // fp32 mode: TMEM stage of the split A k-block
@@ -358,9 +366,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * acc_cols;
         for (int kb = 0; kb < KB; ++kb) {
-          const uint32_t b_hi = smem_u32(smem_b + (size_t)kb * (TF32 ? 2 : 1) * b_tile_bytes);
+          const uint32_t b_hi = smem_u32(STREAM ? smem_a + (size_t)stage * stage_bytes + a_tile_bytes : smem_b + (size_t)kb * parts * b_tile_bytes);
           if (TF32) {
-            ok = mbar_wait(&ready[ts], tphase, abort_flag, p.spin_limit);
+            ok = (!STREAM || mbar_wait(&full[stage], phase, abort_flag, p.spin_limit)) && mbar_wait(&ready[ts], tphase, abort_flag, p.spin_limit);
             if (!ok) break;
             tc_fence_after();
             const uint32_t a_hi = tmem_base + a_col0 + ts * TC_TSTAGE_COLS, a_lo = a_hi + 32;
@@ -372,11 +380,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
             }
             tc_commit(&a_free[ts]);   // TMEM stage reusable once these MMAs have read it
             if (++ts == (uint32_t)p.tstages) { ts = 0; tphase ^= 1u; }
+            if (STREAM) {   // the stage's weights too (its raw tile: the split warps)
+              tc_commit(&empty[stage]);
+              if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
+            }
           } else {
             ok = mbar_wait(&full[stage], phase, abort_flag, p.spin_limit);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t a_s = smem_u32(smem_a + (size_t)stage * a_tile_bytes);
+            const uint32_t a_s = smem_u32(smem_a + (size_t)stage * stage_bytes);
 #pragma unroll
             for (int k = 0; k < 4; ++k)   // four 32-byte K steps inside the 128-byte swizzle row
               tc_mma<TF32>(d_tmem, make_desc(a_s + k * 32), make_desc(b_hi + k * 32), idesc, (kb | k) != 0);
@@ -785,7 +797,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           ok = mbar_wait(&full[stage], phase, abort_flag, p.spin_limit);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
-          const unsigned char *row_base = smem_a + (size_t)stage * a_tile_bytes + (size_t)row * TC_KBLOCK_BYTES;
+          const unsigned char *row_base = smem_a + (size_t)stage * stage_bytes + (size_t)row * TC_KBLOCK_BYTES;
           float4 x[8];
 #pragma unroll
           for (int c = 0; c < 8; ++c) x[c] = *reinterpret_cast<const float4 *>(row_base + ((c ^ (row & 7)) << 4));
@@ -1213,20 +1225,40 @@ constexpr int kSmemAux = 1024 /*alignment slack*/ + 288 /*barriers, TMEM slot, a
 // scores are computed) have resident weights that leave room for three operand stages (which already give the time of eight)
 // and one 32 KB staging tile of the epilogue.  Columns past the last output are padding.
 constexpr size_t kWeightBudget = kSmemBudget - kSmemAux - 1024 /*per-column constants*/ - 3 * TC_BM * TC_KBLOCK_BYTES - 32 * 1024;
+//
+// Weights that leave a CTA fewer columns than the tensor core takes (256, in fp32 mode 64) would have every further split read the
+// input again: they are streamed through the stages instead, and every row tile reads them again out of the L2 (a CTA then loads
+// 48 KB for 128 x 256 x 64 multiply-adds, as before for 128 x 96 x 64, but in four stages of 48 KB instead of five of 16: resident
+// weights kept 80 KB in flight).  Resident against streamed, 1M rows: bf16 K = 768, 512 columns 1404 against 724 us; 512, 256 360 / 286;
+// 384, 256 309 / 244; 448, 192 322 / 254; 1024, 128 675 / 400; fp32 (500k rows) 600, 256 3970 / 1323; 512, 256 1686 / 1125; 1M rows
+// 320, 64 544 / 381; 384, 128 1000 / 879.  20k rows bf16 768, 512 73 / 51; 512, 256 16.0 / 15.0; but 10k rows fp32 384, 128 18.5 / 22.1:
+// there the splits fill the SMs, so fp32 products of few tiles are streamed only from twice as many splits on.
 bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_cols *out) {
   const bool tf32 = a.x_dtype == IT_F32;
   const int bk = TC_KBLOCK_BYTES / (tf32 ? 4 : 2), KB = (a.K1 + bk - 1) / bk + ((a.X2 ? a.K2 : 0) + bk - 1) / bk;
   out->n0p = (a.n0 + 15) / 16 * 16;
   out->n1p = (a.n1 + 15) / 16 * 16;
+  out->stream = 0;
   const int n = out->n0p + out->n1p, step = want_scores ? head_dim : 16;
   if (n <= 0 || step % 16 != 0) return false;
+  // fp32 mode issues MMAs of 2 c columns and keeps 4 c TMEM columns of accumulators next to the split A stages
+  const int most = tf32 ? 64 : 256;
   for (int s = 1; s <= 16; ++s) {
     const int c = ((n + s - 1) / s + step - 1) / step * step;
-    // fp32 mode issues MMAs of 2 c columns and keeps 4 c TMEM columns of accumulators next to the split A stages
-    if (c > (tf32 ? 64 : 256)) continue;
+    if (c > most) continue;
     if ((size_t)(tf32 ? 2 : 1) * KB * c * TC_KBLOCK_BYTES > kWeightBudget) continue;
     if (want_scores && c * s != n) continue;
     out->n_splits = s; out->nbc = c; out->NB = c * s;
+    int few = (n + most - 1) / most, wide = 0;
+    for (; few < s; ++few) {   // (no more prepared columns than the resident form has: scratch does not grow)
+      wide = ((n + few - 1) / few + 15) / 16 * 16;
+      if (wide * few <= c * s) break;
+    }
+    const bool few_tiles = tf32 && (a.M + TC_BM - 1) / TC_BM * few < 512;
+    if (few < s && !want_scores && (!few_tiles || s >= 2 * few)) {
+      out->stream = 1;
+      out->n_splits = few; out->nbc = wide; out->NB = wide * few;
+    }
     return true;
   }
   return false;
@@ -1268,22 +1300,25 @@ it_status it_launch_prep_weights_tc(const it_prep_tc *list, int count, int *zero
 }
 
 namespace {
-struct TcShape { int b_bytes, const_bytes, out_panels, epi_groups, stages; bool staged; };
+struct TcShape { int b_bytes, const_bytes, out_panels, epi_groups, stages, stage_bytes; bool staged; };
 
 // How a product's shared memory is used.
 bool tc_shape(const it_gemm_args &a, const it_tc_cols &cols, int KB, bool want_scores, bool add, TcShape *out) {
   const bool tf32 = a.x_dtype == IT_F32;
   const int n_splits = cols.n_splits, nbc = cols.nbc, n0p = cols.n0p, n1p = cols.n1p;
-  const int b_bytes = (tf32 ? 2 : 1) * KB * nbc * TC_KBLOCK_BYTES;
-  const int stage_bytes = TC_BM * TC_KBLOCK_BYTES;             // one operand tile (fp32 mode: the raw tile)
-  const int add_bytes = add ? TC_ADD_STAGES * ((a.n0 * 2 + 127) / 128) * stage_bytes + 2 * TC_ADD_STAGES * 8 : 0;   // ring of rows to add, its barriers
+  const int b_bytes = cols.stream ? 0 : (tf32 ? 2 : 1) * KB * nbc * TC_KBLOCK_BYTES;
+  const int panel_bytes = TC_BM * TC_KBLOCK_BYTES;
+  // one operand tile (fp32 mode: the raw tile), and the weights that are streamed with it
+  const int stage_bytes = panel_bytes + (cols.stream ? (tf32 ? 2 : 1) * nbc * TC_KBLOCK_BYTES : 0);
+  const int add_bytes = add ? TC_ADD_STAGES * ((a.n0 * 2 + 127) / 128) * panel_bytes + 2 * TC_ADD_STAGES * 8 : 0;   // ring of rows to add, its barriers
   const int const_bytes = nbc * 4 * (want_scores ? 3 : 1) + add_bytes;          // bias (+ attention vectors) of this CTA's columns
   // Staged epilogue (TMA stores): possible when, for every column split, the out0 columns and the out1 columns of
   // the CTA are whole 128-byte panels or reach the end of their output (the copy clips what lies past it), and three operand
   // stages still fit beside the staging tile (three stages already give the time of eight).
   const int s0 = a.dt0 == IT_BF16 ? 2 : 4, s1 = a.dt1 == IT_BF16 ? 2 : 4;
   int out_panels = 0;
-  bool staged = IT_TC_TMA_STORE != 0;
+  // (streamed bf16 weights: a fourth stage is worth more than the staging tile: 1M rows, K = 768, 512 columns 815 against 728 us)
+  bool staged = IT_TC_TMA_STORE != 0 && (!cols.stream || tf32);
   for (int sp = 0; sp < n_splits && staged; ++sp) {
     const int cb = sp * nbc, ce = cb + nbc, n01 = n0p + n1p;
     const int lo0 = cb < n0p ? cb : n0p, hi0 = ce < n0p ? ce : n0p;
@@ -1295,17 +1330,17 @@ bool tc_shape(const it_gemm_args &a, const it_tc_cols &cols, int KB, bool want_s
   }
   // two groups of epilogue warps (alternate tiles, a staging tile each) when the second staging tile still fits
   int epi_groups = IT_TC_EPI_GROUPS;
-  if (staged && epi_groups == 2 && (kSmemBudget - kSmemAux - const_bytes - b_bytes - 2 * out_panels * stage_bytes) / stage_bytes < 3) {
+  if (staged && epi_groups == 2 && (kSmemBudget - kSmemAux - const_bytes - b_bytes - 2 * out_panels * panel_bytes) / stage_bytes < 3) {
     epi_groups = 1;
     if (!tf32) staged = false;   // measured: one group beats the direct stores in fp32 mode only (its tiles take long enough)
   }
-  if (staged && (kSmemBudget - kSmemAux - const_bytes - b_bytes - epi_groups * out_panels * stage_bytes) / stage_bytes < 3) staged = false;
+  if (staged && (kSmemBudget - kSmemAux - const_bytes - b_bytes - epi_groups * out_panels * panel_bytes) / stage_bytes < 3) staged = false;
   if (!staged) { out_panels = 0; epi_groups = 1; }
-  int stages = (kSmemBudget - kSmemAux - const_bytes - b_bytes - epi_groups * out_panels * stage_bytes) / stage_bytes;
+  int stages = (kSmemBudget - kSmemAux - const_bytes - b_bytes - epi_groups * out_panels * panel_bytes) / stage_bytes;
   if (stages > IT_TC_MAX_STAGES) stages = IT_TC_MAX_STAGES;
   if (stages < 2) return false;
   out->b_bytes = b_bytes; out->const_bytes = const_bytes; out->out_panels = out_panels; out->epi_groups = epi_groups;
-  out->stages = stages; out->staged = staged;
+  out->stages = stages; out->staged = staged; out->stage_bytes = stage_bytes;
   return true;
 }
 }  // namespace
@@ -1315,7 +1350,7 @@ bool it_tc_adds_rows(const it_gemm_args &a) {
   TcShape sh;
   const int bk = TC_KBLOCK_BYTES / (a.x_dtype == IT_F32 ? 4 : 2), KB = (a.K1 + bk - 1) / bk + ((a.X2 ? a.K2 : 0) + bk - 1) / bk;
   return a.x_dtype == IT_BF16 && a.n1 == 0 && a.n0 <= 128 && it_tc_supported(a, 1, a.n0, false) && it_tc_columns(a, a.n0, false, &cols) &&
-         cols.n_splits == 1 && tc_shape(a, cols, KB, false, true, &sh) && sh.staged;
+         cols.n_splits == 1 && !cols.stream && tc_shape(a, cols, KB, false, true, &sh) && sh.staged;
 }
 
 // B: weights prepared by it_launch_prep_weights_tc.  a.B / a.NB / a.out2 of the generic args are ignored:
@@ -1336,10 +1371,10 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   TcShape sh;
   IT_REQUIRE(tc_shape(a, cols, KB, scores != nullptr, a.add_rows != nullptr, &sh), IT_ERR_UNSUPPORTED, "tensor-core apply: no room for two operand stages");
   IT_REQUIRE(!a.add_rows || sh.staged, IT_ERR_UNSUPPORTED, "tensor-core apply: rows are added by the staged epilogue only");
-  const int b_bytes = sh.b_bytes, stage_bytes = TC_BM * TC_KBLOCK_BYTES, const_bytes = sh.const_bytes, out_panels = sh.out_panels;
+  const int b_bytes = sh.b_bytes, panel_bytes = TC_BM * TC_KBLOCK_BYTES, const_bytes = sh.const_bytes, out_panels = sh.out_panels;
   const int epi_groups = sh.epi_groups, stages = sh.stages, s0 = a.dt0 == IT_BF16 ? 2 : 4, s1 = a.dt1 == IT_BF16 ? 2 : 4;
   const bool staged = sh.staged;
-  const int smem = b_bytes + (stages + epi_groups * out_panels) * stage_bytes + kSmemAux + const_bytes;
+  const int smem = b_bytes + stages * sh.stage_bytes + epi_groups * out_panels * panel_bytes + kSmemAux + const_bytes;
   // fp32 mode: TMEM holds two accumulators of 2 nbc columns; what is left of its 512 columns stages the split A
   int tstages = tf32 ? (512 - 4 * nbc) / TC_TSTAGE_COLS : 0;
   if (tstages > TC_TSTAGES_MAX) tstages = TC_TSTAGES_MAX;
@@ -1359,7 +1394,7 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   p.kb1 = kb1; p.kb2 = kb2; p.NB = NB; p.stages = stages; p.tstages = tstages;
   p.n0 = n0p; p.n0_real = a.n0; p.out0 = a.out0; p.out0_bf16 = a.dt0 == IT_BF16; p.bias0 = a.bias0; p.act0 = a.act0;
   p.n1 = n1p; p.n1_real = a.n1; p.out1 = a.out1; p.out1_bf16 = a.dt1 == IT_BF16;
-  p.add_rows = (const char *)a.add_rows; p.add_idx = a.add_idx; p.add_pitch = a.n0 * s0; p.add_stage_bytes = (p.add_pitch + 127) / 128 * stage_bytes;
+  p.add_rows = (const char *)a.add_rows; p.add_idx = a.add_idx; p.add_pitch = a.n0 * s0; p.add_stage_bytes = (p.add_pitch + 127) / 128 * panel_bytes;
   p.scores = scores; p.att_src = att_src; p.att_dst = att_dst; p.heads = heads; p.head_dim = head_dim > 0 ? head_dim : 1;
   p.status = status;
   p.tma_store = staged ? 1 : 0; p.out_panels = out_panels; p.epi_groups = epi_groups;
@@ -1372,17 +1407,14 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   const double bytes = (double)a.M * (K * xs + a.n0 * (a.dt0 == IT_F32 ? 4.0 : 2.0) + a.n1 * (a.dt1 == IT_F32 ? 4.0 : 2.0) +
                                      (scores ? 8.0 * heads : 0.0)) + (double)K * (a.n0 + a.n1) * xs;
   const double flops = 2.0 * (double)a.M * K * (a.n0 + a.n1);
-  if (tf32) {
-    IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<true, false>, dim3((unsigned)grid), dim3(TC_THREADS_TF32), smem, st, m1, m2, mb, mo0, mo1, p)));
-  } else if (a.add_rows) {
-    IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    IT_LAUNCH(IT_K_GEMM_TC, bytes + (double)a.M * (4.0 + a.n0 * 2.0), flops, st,
-              IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<false, true>, dim3((unsigned)grid), dim3(TC_THREADS_ADD), smem, st, m1, m2, mb, mo0, mo1, p)));
-  } else {
-    IT_CUDA_TRY(cudaFuncSetAttribute(gemm_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    IT_LAUNCH(IT_K_GEMM_TC, bytes, flops, st, IT_CUDA_TRY(it_launch_pdl(gemm_tc_kernel<false, false>, dim3((unsigned)grid), dim3(TC_THREADS_BF16), smem, st, m1, m2, mb, mo0, mo1, p)));
-  }
+  auto go = [&](auto kernel, int threads, double more) -> it_status {
+    IT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    IT_LAUNCH(IT_K_GEMM_TC, bytes + more, flops, st, IT_CUDA_TRY(it_launch_pdl(kernel, dim3((unsigned)grid), dim3(threads), smem, st, m1, m2, mb, mo0, mo1, p)));
+    return IT_OK;
+  };
+  if (tf32) IT_TRY(cols.stream ? go(gemm_tc_kernel<true, false, true>, TC_THREADS_TF32, 0.0) : go(gemm_tc_kernel<true, false, false>, TC_THREADS_TF32, 0.0));
+  else if (a.add_rows) IT_TRY(go(gemm_tc_kernel<false, true, false>, TC_THREADS_ADD, (double)a.M * (4.0 + a.n0 * 2.0)));
+  else IT_TRY(cols.stream ? go(gemm_tc_kernel<false, false, true>, TC_THREADS_BF16, 0.0) : go(gemm_tc_kernel<false, false, false>, TC_THREADS_BF16, 0.0));
   IT_CUDA_TRY(cudaGetLastError());
   return IT_OK;
 }

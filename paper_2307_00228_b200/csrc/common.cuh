@@ -310,7 +310,8 @@ struct it_prep_tc {
 };
 it_prep_tc it_prep_tc_of(it_prep_kind kind, const it_layer_desc *layer, int NB, int seg, int K1, int K2, void *B);
 // How the product's columns are laid out: each output padded to a multiple of 16 columns, all of them to whole splits.
-struct it_tc_cols { int n0p, n1p, n_splits, nbc, NB; };
+// stream: the weights are read again with every row tile instead of staying in shared memory.
+struct it_tc_cols { int n0p, n1p, n_splits, nbc, NB, stream; };
 bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_cols *out);
 size_t it_prep_tc_bytes(const it_prep_tc &p);
 // Several weight matrices and `words` zeroed words in as few launches as possible.
