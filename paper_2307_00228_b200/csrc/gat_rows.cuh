@@ -72,7 +72,7 @@ __device__ __forceinline__ float leaky(float x, float slope) { return x > 0.f ? 
 // ----------------------------------------------------------------------------- one warp per row (or per part of a row)
 // Lane = (edge el = lane / H, head hl = lane % H) for the logits; pair i of a lane is edge el + i * 32 / H of the chunk.
 template <typename T, int LPR, int H>
-struct GatWarp {
+struct GatPairs {
   static constexpr int EP = 32 / H;   // edges covered by one pair per lane
   const StreamParams &p;
   const GatParams &q;
@@ -84,7 +84,7 @@ struct GatWarp {
   GatAcc<T> acc;
   float st[GatAcc<T>::NS];
 
-  __device__ __forceinline__ GatWarp(const StreamParams &p_, const GatParams &q_, int lane_, uint32_t pw_)
+  __device__ __forceinline__ GatPairs(const StreamParams &p_, const GatParams &q_, int lane_, uint32_t pw_)
       : p(p_), q(q_), lane(lane_), hl(lane_ % H), el(lane_ / H), hc((lane_ % LPR) * GatAcc<T>::VEC / q_.head_dim), pw(pw_) {
     sd_c = sd_n = 0.f; m = -INFINITY;
 #pragma unroll
@@ -123,8 +123,99 @@ struct GatWarp {
       asm volatile("st.shared.f32 [%0], %1;" ::"r"(pw + (uint32_t)((lane + 32 * i) * 4)), "f"(it_exp(x_c[i] - m)) : "memory");
     __syncwarp();
   }
+  __device__ __forceinline__ void clear() { m = -INFINITY; acc.init(st); }
+  __device__ __forceinline__ float maximum() const { return __shfl_sync(0xffffffffu, m, hc); }   // of the slice's head
   __device__ __forceinline__ float weight(int k) const { return lds_f32(pw + (uint32_t)((k * H + hc) * 4)); }
 };
+
+// The largest x of the warp (of numbers: a NaN is no candidate).
+__device__ __forceinline__ float warp_max(float x) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+// H consecutive floats, aligned to H of them (at most 16 bytes)
+template <int H>
+__device__ __forceinline__ void load_heads(const float *p, float (&x)[H]) {
+  if constexpr (H == 1) x[0] = __ldg(p);
+  else if constexpr (H == 2) { const float2 v = __ldg(reinterpret_cast<const float2 *>(p)); x[0] = v.x; x[1] = v.y; }
+  else {
+#pragma unroll
+    for (int i = 0; i < H; i += 4) {
+      const float4 v = __ldg(reinterpret_cast<const float4 *>(p + i));
+      x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
+    }
+  }
+}
+template <int H>
+__device__ __forceinline__ float pick(const float (&x)[H], int h) {   // x[h], h not known at compile time
+  float r = x[0];
+#pragma unroll
+  for (int i = 1; i < H; ++i) r = h == i ? x[i] : r;
+  return r;
+}
+
+// Lane = edge of the chunk, with all its heads: one load of its logit terms and one warp reduction per head, where a lane per pair of
+// edge and head takes a load, an id shuffle and a store per head.
+template <typename T, int LPR, int H>
+struct GatEdges {
+  const StreamParams &p;
+  const GatParams &q;
+  const int lane, hc;                 // hc: head of the lane's slice
+  const uint32_t pw;                  // shared-window address of this warp's weights [32][H]
+  float x_n[H], sd_n[H];              // of the next chunk: logit terms, destination scores of its row
+  float m[H];                         // running maxima
+  GatAcc<T> acc;
+  float st[GatAcc<T>::NS];
+
+  __device__ __forceinline__ GatEdges(const StreamParams &p_, const GatParams &q_, int lane_, uint32_t pw_)
+      : p(p_), q(q_), lane(lane_), hc((lane_ % LPR) * GatAcc<T>::VEC / q_.head_dim), pw(pw_) {
+#pragma unroll
+    for (int i = 0; i < H; ++i) { x_n[i] = sd_n[i] = 0.f; m[i] = -INFINITY; }
+    acc.init(st);
+  }
+  // the ids of chunk c have landed: fetch its logit terms (into the "next" registers)
+  __device__ __forceinline__ void ahead(const Chunk &c) {
+    if (lane < c.cnt) load_heads<H>(q.scores + (q.per_edge ? (uint64_t)(c.j + lane) : (uint64_t)(uint32_t)c.idx) * q.stride, x_n);
+    load_heads<H>(q.scores_dst + (int64_t)c.owner * (2 * H) + H, sd_n);
+  }
+  // chunk c becomes the current one: its attention weights
+  __device__ __forceinline__ void begin(const Chunk &c, bool first) {
+    float x[H], s[H];
+    if (first) acc.init(st);
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      x[i] = lane < c.cnt ? leaky(x_n[i] + sd_n[i], q.slope) : -INFINITY;
+      const float was = first ? -INFINITY : m[i];
+      m[i] = fmaxf(was, warp_max(x[i]));
+      s[i] = it_exp(was - m[i]);   // exp(-inf) = 0 for the first chunk of a row
+      x[i] = it_exp(x[i] - m[i]);
+    }
+    if (!first) acc.scale(st, pick<H>(s, hc));
+    __syncwarp();   // the previous chunk's weights have been read
+    const uint32_t at = pw + (uint32_t)(lane * H * 4);
+    if constexpr (H == 1) asm volatile("st.shared.f32 [%0], %1;" ::"r"(at), "f"(x[0]) : "memory");
+    else if constexpr (H == 2) asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(at), "f"(x[0]), "f"(x[1]) : "memory");
+    else {
+#pragma unroll
+      for (int i = 0; i < H; i += 4)
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + i * 4), "f"(x[i]), "f"(x[i + 1]), "f"(x[i + 2]), "f"(x[i + 3]) : "memory");
+    }
+    __syncwarp();
+  }
+  __device__ __forceinline__ float weight(int k) const { return lds_f32(pw + (uint32_t)((k * H + hc) * 4)); }
+  __device__ __forceinline__ float maximum() const { return pick<H>(m, hc); }   // of the slice's head
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < H; ++i) m[i] = -INFINITY;
+    acc.init(st);
+  }
+};
+// Which of the two: the registers of eight heads spill, and so do those of bf16 rows in the chunk kernel, whose accumulators are twice
+// as many (5M vertices / 100M edges, 4 heads: pairs 10.8 ms, edges 11.3; fp32 4 heads of 16, 500k / 8M with edge features: pairs 572 us,
+// edges 533).  In the kernel for small graphs 30k / 420k, bf16 4 heads: pairs 65 us, edges 63.
+template <typename T, int LPR, int H> using GatWarp = std::conditional_t<sizeof(T) == 4 && H <= 4, GatEdges<T, LPR, H>, GatPairs<T, LPR, H>>;
+template <typename T, int LPR, int H> using GatSmallWarp = std::conditional_t<H <= 4, GatEdges<T, LPR, H>, GatPairs<T, LPR, H>>;
 
 #ifndef IT_GAT_CHUNK_BLOCKS
 #define IT_GAT_CHUNK_BLOCKS 3   // resident CTAs per SM: at four the 64 registers a thread gets spill (measured: 3 to 5 % more time)
@@ -155,7 +246,7 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_k
       },
       [&](const Chunk &c) {
         rw.fold(gw.acc, gw.st);
-        const float mh = __shfl_sync(0xffffffffu, gw.m, gw.hc);
+        const float mh = gw.maximum();
         float full[GatPolicy<T, 16>::NS];
 #pragma unroll
         for (int k = 0; k < GatAcc<T>::VEC; ++k) full[k] = gw.st[k];
@@ -174,7 +265,8 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_k
 #define IT_GAT_SHORT_BLOCKS 3   // resident CTAs per SM: 64 KB of staging each
 #endif
 // block / blocks: which share of the rows p.row_lo .. p.row_hi this block walks; short_buf: [2][E][THREADS] in shared memory.
-template <typename T, int LPR, int H>
+// EMPTY: rows without edges are among them.
+template <typename T, int LPR, int H, bool EMPTY = false>
 __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatParams &q, const GatPolicy<T, 16> &pol, int block, int blocks, uint4 *short_buf) {
   using Acc = GatAcc<T>;
   constexpr int E = LPR < IT_SHORT_EDGES ? LPR : IT_SHORT_EDGES;
@@ -189,10 +281,11 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
   constexpr uint32_t SLOT = THREADS * 16, BUF = E * SLOT;
   uint32_t buf = (uint32_t)__cvta_generic_to_shared(short_buf + threadIdx.x), other = buf + BUF;
   const int64_t sweep = (int64_t)blocks * (THREADS / LPR);
+  constexpr int NONE = EMPTY ? -1 : 0;   // length of a missing row
 
-  struct Row { int64_t j0; int len, most, dest, owner; float sd; };   // most: longest row of the warp's groups (0: no rows left)
+  struct Row { int64_t j0; int len, most, dest, owner; float sd; };   // most: longest row of the warp's groups (NONE: no rows left)
   auto load_row = [&](int64_t i0, Row &r) {
-    r.j0 = 0; r.len = 0; r.dest = 0; r.owner = 0;
+    r.j0 = 0; r.len = NONE; r.dest = 0; r.owner = 0;
     const int64_t i = i0 + lane / LPR;
     if (i < p.row_hi) {
       const it_row_meta m = load_meta(p.meta + i);
@@ -202,6 +295,7 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
   };
   auto finish_row = [&](Row &r) {   // the record has landed: what hangs on it
     r.most = __reduce_max_sync(0xffffffffu, r.len);
+    if (EMPTY && r.most == 0) r.most = 1;   // only rows without edges: a round in any case, which fetches what follows
     r.sd = __ldg(q.scores_dst + (int64_t)r.owner * (2 * H) + H + hl);   // owner 0 for a missing row: read, not used
   };
   auto load_ids = [&](const Row &r, int k) -> int32_t {
@@ -230,7 +324,7 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
   Row r0, r1, r2;
   load_row(i0, r0); load_row(i0 + sweep, r1); load_row(i0 + 2 * sweep, r2);
   finish_row(r0);
-  if (r0.most == 0) return;   // warp-uniform
+  if (r0.most == NONE) return;   // warp-uniform
   finish_row(r1);
   float x_a[PP], x_b[PP];
   int32_t idx_b = load_ids(r0, 0);
@@ -238,7 +332,7 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
   idx_b = r0.most > E ? load_ids(r0, E) : load_ids(r1, 0);
   Acc acc;
   float st[Acc::NS];
-  for (; r0.most > 0; i0 += sweep) {
+  for (; r0.most > NONE; i0 += sweep) {
     Row r3;
     load_row(i0 + 3 * sweep, r3);
     finish_row(r2);
@@ -262,8 +356,9 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
       for (int o = H; o < LPR; o <<= 1) mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
       const float m_new = fmaxf(m, mr);
       if (k0 > 0) {   // rows whose edges are used up: m_new = m, a factor of 1
-        const float s = __shfl_sync(0xffffffffu, it_exp(m - m_new), gbase + hc);
-        acc.scale(st, s);
+        float s = it_exp(m - m_new);
+        if (EMPTY && m_new == -INFINITY) s = 1.f;   // (a row without edges: nothing to rescale)
+        acc.scale(st, __shfl_sync(0xffffffffu, s, gbase + hc));
       }
       m = m_new;
 #pragma unroll
@@ -281,7 +376,7 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
       const uint32_t sw = buf; buf = other; other = sw;
     }
     const float mh = __shfl_sync(0xffffffffu, m, gbase + hc);
-    if (r0.len > 0) {
+    if (r0.len > NONE) {
       float full[GatPolicy<T, 16>::NS];
 #pragma unroll
       for (int k = 0; k < Acc::VEC; ++k) full[k] = st[k];
@@ -314,17 +409,14 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(Stream
   pol.setup(t);
   const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
   stage_bias(pol, bias_buf);
-  if constexpr (LPR <= 16) {
-    if ((int)blockIdx.x < sh.short_blocks) {
-      p.row_lo = sh.short_lo; p.row_hi = sh.short_hi;
-      gat_short_rows<T, LPR, H>(p, q, pol, blockIdx.x, sh.short_blocks, short_buf);
-      return;
-    }
+  if ((int)blockIdx.x < sh.short_blocks) {
+    p.row_lo = sh.short_lo; p.row_hi = sh.short_hi;
+    gat_short_rows<T, LPR, H, true>(p, q, pol, blockIdx.x, sh.short_blocks, short_buf);
+    return;
   }
-  GatWarp<T, LPR, H> gw(p, q, lane, (uint32_t)__cvta_generic_to_shared(&weights[threadIdx.x >> 5][0]));
+  GatSmallWarp<T, LPR, H> gw(p, q, lane, (uint32_t)__cvta_generic_to_shared(&weights[threadIdx.x >> 5][0]));
   small_walk<false, true>(p, sh, lane, [&](const SmallRow &m, int32_t idx, float) {
-    gw.acc.init(gw.st);
-    gw.m = -INFINITY;
+    gw.clear();
     for (int base = 0; base < m.len; base += 32) {
       Chunk c;
       c.cnt = m.len - base < 32 ? m.len - base : 32;
@@ -360,7 +452,7 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(Stream
       for (int k = 0; k < GatAcc<T>::NS; ++k) other[k] = __shfl_xor_sync(0xffffffffu, gw.st[k], o);
       gw.acc.merge(gw.st, other);
     }
-    const float mh = __shfl_sync(0xffffffffu, gw.m, gw.hc);
+    const float mh = gw.maximum();
     float full[NS];
 #pragma unroll
     for (int k = 0; k < VEC; ++k) full[k] = gw.st[k];
@@ -407,7 +499,7 @@ it_status launch_gat_small(const it_gat_args &a, StreamParams p, const GatPolicy
   if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(it_done_words(a.counters), 0, (size_t)g->n_long * sizeof(int), st));
   const double row_bytes = (double)pol.dim * sizeof(T);
   const double bytes = (double)g->e * (4.0 + 4.0 * H + row_bytes) + (double)g->n * (20.0 + 4.0 * H + row_bytes);
-  const SmallShare sh = small_share(g, LPR <= 16, LPR);
+  const SmallShare sh = small_share(g, LPR);
   const int smem = sh.short_blocks ? 2 * IT_SHORT_EDGES * THREADS * 16 : 0;
   static std::atomic<uint64_t> configured{0};
   IT_TRY(allow_dynamic_smem(gat_small_kernel<T, LPR, H>, 2 * IT_SHORT_EDGES * THREADS * 16, configured));

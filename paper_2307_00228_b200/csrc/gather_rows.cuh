@@ -153,7 +153,8 @@ struct SmallPolicy : SagePolicy<T, 16, RED, true> {
 template <typename T, int LPR, class Policy>
 __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(StreamParams p, Policy pol, PieceParams q, SmallShare sh, const int64_t *__restrict__ owner_indptr,
                                                                           const int64_t *__restrict__ shadow_indptr) {
-  constexpr int SL = 32 / LPR, U = LPR < 4 ? LPR : 4;   // edge slots; rows in flight per lane (SL * U <= 32)
+  constexpr int SL = 32 / LPR, U = LPR < 4 ? LPR : 4;   // edge slots; rows in flight per lane (SL * U <= 32; eight spill)
+  constexpr int LPRS = LPR < 8 ? 8 : LPR;               // lane group of a short row
   constexpr int NS = Policy::NS;
   using Slice = typename Policy::Slice;
   extern __shared__ uint4 small_stage[];
@@ -163,12 +164,10 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(Str
   pol.setup(t);
   const char *my_src = reinterpret_cast<const char *>(p.src) + (size_t)t * 16;
   it_wait_prior();
-  if constexpr (LPR == 8 || LPR == 16) {
-    if ((int)blockIdx.x < sh.short_blocks) {
-      p.row_lo = sh.short_lo; p.row_hi = sh.short_hi;
-      short_rows_pipe<T, LPR, Policy, true>(p, pol, blockIdx.x, sh.short_blocks, small_stage);
-      return;
-    }
+  if ((int)blockIdx.x < sh.short_blocks) {
+    p.row_lo = sh.short_lo; p.row_hi = sh.short_hi;
+    short_rows_pipe<T, LPRS, Policy, true, true>(p, pol, blockIdx.x, sh.short_blocks, small_stage);
+    return;
   }
   small_walk<true, false>(p, sh, lane, [&](const SmallRow &m, int32_t idx, float w) {
     float st[NS];
@@ -252,7 +251,7 @@ it_status launch_small(const it_gather_args &a, StreamParams sp, cudaStream_t st
   sp.weights = a.use_edge_weights ? sp.weights : nullptr;
   if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(it_done_words(a.counters), 0, (size_t)g->n_long * sizeof(int), st));
   auto go = [&]<int LPR>() -> it_status {
-    const SmallShare sh = small_share(g, LPR == 8 || LPR == 16, LPR);
+    const SmallShare sh = small_share(g, LPR < 8 ? 8 : LPR);
     IT_LAUNCH(IT_K_GATHER_SMALL, bytes, 0, st,
               IT_CUDA_TRY(it_launch_pdl(gather_small_kernel<T, LPR, Policy>, dim3(sh.blocks), dim3(THREADS), sh.short_blocks ? SHORT_STAGE_BYTES : 0, st, sp, pol,
                                         piece_params(g, it_done_words(a.counters)), sh, (const int64_t *)g->owner_indptr, (const int64_t *)g->shadow_indptr)));

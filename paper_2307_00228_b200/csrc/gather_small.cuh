@@ -1,11 +1,11 @@
-// One kernel per layer for small graphs.  Some blocks walk the rows of at most 32 edges, a lane group per row, as the kernel
-// for short rows does (where the row width has one); the others take the remaining rows, a warp per row (pieces of long
-// vertices, whole vertices, rows without edges), source rows straight into registers, and fold the pieces of a long vertex
+// One kernel per layer for small graphs.  Some blocks walk the rows of at most 32 edges and those of none, a lane group per row, as
+// the kernel for short rows does; the others take the remaining rows, a warp per row (pieces of long
+// vertices, whole vertices), source rows straight into registers, and fold the pieces of a long vertex
 // in the warp that finishes the last of them.  The record of a warp's next-but-one row and the ids of its next row are in
 // flight while a row is reduced.
 // What bounds it: the dependent trips record -> ids -> source rows out of the L2 and the launch itself.  A layer of 10k
 // vertices and 100k edges took five launches (a memset, three kernels by row length, empty rows, combine).  Measured: two fp32
-// layers of that graph 150 -> 40 us; the layers of a GAT on 30k vertices and 420k edges 184 -> 84 us.
+// layers of that graph 150 -> 35 us; the layers of a GAT on 30k vertices and 420k edges 184 -> 63 us.
 //
 // Included by gather_rows.cuh and gat_rows.cuh.
 #pragma once
@@ -41,24 +41,28 @@ __device__ __forceinline__ bool last_piece(const PieceParams &q, int slot, int l
 
 constexpr int SMALL_BLOCKS = 3;   // resident CTAs per SM
 
-// How a launch is shared out: blocks [0, short_blocks) take entries [short_lo, short_hi) of the list, the others the rest.
+// How a launch is shared out: blocks [0, short_blocks) take entries [short_lo, short_hi) of the list, the others the rest, in
+// proportion to what they cost, since a launch is as long as its longer share.  A lane group's row costs about eight edges besides its
+// own, and a warp has 32 / lpr of them at a time; a warp's row about as much as sixteen, and the more steps the more lanes an edge
+// takes.  Rows without edges, which had a warp each, cost a lane group half a row.  Measured against twice / half of the lane groups'
+// share: attention, 30k vertices / 420k edges, 128-byte rows 63 us against 65 / 79; 30k / 400k, 512-byte rows 62 against 76 / 63; 100k /
+// 1.8M, 256-byte rows 127 against 143 / 147; GCN, 8k / 190k, 128- and 64-byte rows 33 against 34 / 38.
 struct SmallShare {
   unsigned blocks;
   int short_blocks, short_lo, short_hi, total;
 };
-inline SmallShare small_share(const it_graph *g, bool groups, int lpr) {
+inline SmallShare small_share(const it_graph *g, int lpr) {
   SmallShare s;
   s.total = (int)g->h_list_offsets[g->n_lists];
   int64_t short_cost = 0, cost = 0;
   s.short_lo = s.short_hi = 0;
   for (int b = 0; b < g->n_lists; ++b) {
-    const int64_t rows = g->h_list_offsets[b + 1] - g->h_list_offsets[b];
-    if (groups && g->list_bounds[b] > 0 && g->list_bounds[b] <= IT_SHORT_BELOW && b != g->n_lists - 1) {
-      if (s.short_hi == s.short_lo) s.short_lo = (int)g->h_list_offsets[b];
+    const int64_t rows = g->h_list_offsets[b + 1] - g->h_list_offsets[b], edges = g->h_list_edges[b];
+    if (g->list_bounds[b] <= IT_SHORT_BELOW && b != g->n_lists - 1) {
       s.short_hi = (int)g->h_list_offsets[b + 1];
-      short_cost += (rows * 8 + g->h_list_edges[b]) * lpr / 32;   // edge slots, and about eight of them for a row
+      short_cost += (b == 0 ? rows * 4 : rows * 8 + edges) * lpr / 16;
     } else {
-      cost += rows * 8 + g->h_list_edges[b];
+      cost += rows * 16 + edges * 2 * lpr / 16;
     }
   }
   const int rows = s.total - (s.short_hi - s.short_lo), most = g->num_sms * SMALL_BLOCKS;

@@ -507,8 +507,10 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   p.long_above = g->n_src / 12288 < 1024 ? 1024 : (g->n_src / 12288 > 4096 ? 4096 : g->n_src / 12288);
   p.piece_min = g->n_src < ((int64_t)1 << 17) ? 256 : 128;
   p.piece_max = 512;
-  // small graphs: a warp's longest row is the time of the launch (120 edges per warp on average at 420k edges)
-  if (it_small_graph(g)) p.long_above = p.piece_min = p.piece_max = 128;
+  // Small graphs: a warp's longest row is the time of the launch, so pieces are shorter where 24 warps per SM have at most 64 edges each
+  // (64 against 128 edges: 10k vertices / 100k edges 35.1 against 39.4 us, GAT 10k / 150k 24.7 / 26.8, 1000 / 150k of 2 KB rows 197 / 215;
+  // beyond, 10k / 300k 47.5 / 44.4, GAT 30k / 420k 82.5 / 78.7).
+  if (it_small_graph(g)) p.long_above = p.piece_min = p.piece_max = g->e <= 64 * 24 * (int64_t)g->num_sms ? 64 : 128;
 
   // at most one row per vertex and one more per T edges, a long vertex per long_above edges, a piece per piece_min of them
   // and one more each; only where that is far above the number of vertices are they counted before the arrays are laid out

@@ -387,8 +387,9 @@ __global__ void __launch_bounds__(THREADS, IT_GATHER_MIN_BLOCKS) stream_rows_ker
 #define IT_SHORT_PIPE_WAVES 1    // grid = SMs x resident CTAs x this: every CTA is resident from the start and walks its rows
 #endif
 // block / blocks: which share of the rows p.row_lo .. p.row_hi this block walks; sbuf: SHORT_STAGE_BYTES of shared memory.
+// EMPTY: rows without edges are among them.
 constexpr int SHORT_STAGE_BYTES = IT_SHORT_EDGES * THREADS * 16;
-template <typename T, int LPR, class Policy, bool PAD>
+template <typename T, int LPR, class Policy, bool PAD, bool EMPTY = false>
 __device__ __forceinline__ void short_rows_pipe(const StreamParams &p, Policy &pol, int block, int blocks, uint4 *sbuf) {
   constexpr int NS = Policy::NS;
   constexpr int E = IT_SHORT_EDGES;   // edges per round
@@ -403,9 +404,10 @@ __device__ __forceinline__ void short_rows_pipe(const StreamParams &p, Policy &p
   const uint32_t my_buf = (uint32_t)__cvta_generic_to_shared(sbuf + threadIdx.x);
 
   struct Row { int64_t j0; int len, dest, owner; };
-  // the row this lane group takes in the sweep that starts at i0 (len 0: none; rows of these buckets have edges)
+  constexpr int NONE = EMPTY ? -1 : 0;   // length of a missing row
+  // the row this lane group takes in the sweep that starts at i0
   auto load_row = [&](int64_t i0) {
-    Row r{0, 0, 0, 0};
+    Row r{0, NONE, 0, 0};
     const int64_t i = i0 + lane / LPR;
     if (i < p.row_hi) {
       const it_row_meta m = load_meta(p.meta + i);
@@ -429,11 +431,12 @@ __device__ __forceinline__ void short_rows_pipe(const StreamParams &p, Policy &p
   load_idx(cur, 0, idx_c, w_c);
   for (; i0 < p.row_hi; i0 += sweep) {
     const Row nn = load_row(i0 + 2 * sweep);   // in flight for two rows
-    const int maxlen = __reduce_max_sync(0xffffffffu, cur.len);
+    int maxlen = __reduce_max_sync(0xffffffffu, cur.len);
+    if (EMPTY && maxlen < 1) maxlen = 1;   // (a round in any case: it fetches the ids of the next rows)
     float st[NS];
     pol.init(st);
-    const int len = active ? cur.len : 0;
-    if (len > 0) pol.begin_row(cur.dest, cur.owner);
+    const int len = active ? cur.len : NONE;
+    if (len > NONE) pol.begin_row(cur.dest, cur.owner);
     for (int k0 = 0; k0 < maxlen; k0 += E) {
       // the indices of the next round, in flight while this round's rows are
       int32_t idx_n; float w_n;
@@ -462,7 +465,7 @@ __device__ __forceinline__ void short_rows_pipe(const StreamParams &p, Policy &p
       }
       idx_c = idx_n; w_c = w_n;
     }
-    if (len > 0) pol.end_row(st, cur.dest, cur.owner, len);
+    if (len > NONE) pol.end_row(st, cur.dest, cur.owner, len);
     cur = nxt; nxt = nn;
   }
 }

@@ -53,6 +53,23 @@ def test_gat_of_128_byte_rows_with_many_heads(dtype, heads, hd, hubs):
     check_against_oracle(w, got, label=(dtype, heads, hd), exact=False)
 
 
+@pytest.mark.parametrize("kind,dtype,fi", [("mean", "f32", 4), ("max", "f32", 8), ("min", "bf16", 32), ("sum", "f32", 64), ("mean", "bf16", 128), ("max", "f32", 128),
+                                           ("gat", "f32", (4, 4)), ("gat", "bf16", (4, 16)), ("gat", "bf16", (8, 8)), ("gat", "f32", (2, 32)), ("gat", "f32", (8, 16)),
+                                           ("gat", "bf16", (1, 256))])
+@pytest.mark.parametrize("p_zero", [0.0, 0.97])
+def test_small_graph_rows_without_edges_among_the_short_ones(kind, dtype, fi, p_zero):
+    """One kernel per layer: lane groups of every width whose rows all have edges, and whose warps mostly have none; rows and pieces of
+    64 and 65 edges (graphs of few edges) next to them."""
+    hubs = (500, 193, 129, 128, 66, 65, 64, 63, 33, 32, 31, 17, 16, 9, 8, 7)
+    if kind == "gat":
+        layer = make_gat_layer(35, "elu", 32, *fi, dtype)
+    else:
+        layer = make_sage_layer(35, kind, "relu", fi, 16, dtype, weights=kind == "sum", allow_reorder=False)
+    w = small_workload(36, 5001, 24, dtype, [layer], hubs=hubs, weights=kind == "sum", p_zero=p_zero)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(kind, dtype, fi, p_zero))
+
+
 @pytest.mark.parametrize("n,deg", [(1000, 1100), (3700, 245), (3700, 270), (3000, 400)])
 @pytest.mark.parametrize("kind", ["sum", "max", "gat"])
 def test_few_vertices_of_many_edges(n, deg, kind):
