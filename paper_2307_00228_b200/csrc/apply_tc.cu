@@ -205,6 +205,7 @@ struct TcParams {
   int NB;                         // total columns
   int stages;
   int tstages;                    // fp32 mode: split A k-blocks in flight in TMEM
+  int n_acc;                      // fp32 mode: accumulators, 2 or (columns beyond 64) 1
   // epilogue routing (columns are global column ids)
   int n0, n0_real; void *out0; int out0_bf16; const float *bias0; int act0;   // n0, n1: with their padding; *_real: what is stored
   int n1, n1_real; void *out1; int out1_bf16;
@@ -252,9 +253,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
   uint64_t *ready = bars + 2 * p.stages;    // [TC_TSTAGES_MAX]  (fp32 mode) hi / lo parts written to TMEM
   uint64_t *a_free = ready + TC_TSTAGES_MAX;   // [TC_TSTAGES_MAX]  (fp32 mode) MMAs that read a TMEM stage are done
   uint64_t *b_full = a_free + TC_TSTAGES_MAX;  // [1]
-  uint64_t *acc_full = b_full + 1;          // [2]
-  uint64_t *acc_empty = acc_full + 2;       // [2]
-  uint64_t *add_full = acc_empty + 2;       // [TC_ADD_STAGES]  (ADD) the tile's rows have landed
+  const int NACC = TF32 ? p.n_acc : 2;      // accumulators: tiles in flight
+  uint64_t *acc_full = b_full + 1;          // [NACC]
+  uint64_t *acc_empty = acc_full + NACC;    // [NACC]
+  uint64_t *add_full = acc_empty + NACC;       // [TC_ADD_STAGES]  (ADD) the tile's rows have landed
   uint64_t *add_empty = add_full + (ADD ? TC_ADD_STAGES : 0);   // [TC_ADD_STAGES]  (ADD) the epilogue has read them
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(add_empty + (ADD ? TC_ADD_STAGES : 0));
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
@@ -264,9 +266,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
 
   // fp32 mode: columns [nbc, 2 nbc) of an accumulator hold A_hi * B_lo, added to the first half by the epilogue
   const uint32_t acc_cols = (uint32_t)p.nbc * (TF32 ? 2u : 1u);
-  const uint32_t a_col0 = 2 * acc_cols;   // fp32 mode: the split A stages follow the two accumulators
+  const uint32_t a_col0 = NACC * acc_cols;   // fp32 mode: the split A stages follow the two accumulators
   uint32_t tmem_cols = 32;
-  while (tmem_cols < 2 * acc_cols + (TF32 ? (uint32_t)p.tstages * TC_TSTAGE_COLS : 0u)) tmem_cols <<= 1;
+  while (tmem_cols < NACC * acc_cols + (TF32 ? (uint32_t)p.tstages * TC_TSTAGE_COLS : 0u)) tmem_cols <<= 1;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -283,7 +285,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
         mbar_init(&add_full[a], 128);
         mbar_init(&add_empty[a], TC_EPI_WARPS / p.epi_groups);
       }
-    for (int a = 0; a < 2; ++a) {
+    for (int a = 0; a < NACC; ++a) {
       mbar_init(&acc_full[a], 1);
       mbar_init(&acc_empty[a], p.tma_store ? TC_EPI_WARPS / p.epi_groups : TC_EPI_WARPS);
     }
@@ -398,7 +400,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
         }
         if (!ok) break;
         tc_commit(&acc_full[acc]);    // accumulator complete
-        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        if (++acc == (uint32_t)NACC) { acc = 0; acc_phase ^= 1u; }
       }
     }
   } else if (warp < 2 + TC_EPI_WARPS) {
@@ -443,8 +445,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       int it = 0;   // tiles of this CTA so far: tile `it` uses accumulator it % 2, for the (it / 2)-th time
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
         if (G == 2 && (it & 1) != group) continue;
-        acc = (uint32_t)it & 1u;
-        acc_phase = ((uint32_t)it >> 1) & 1u;
+        acc = (uint32_t)(it % NACC);
+        acc_phase = (uint32_t)(it / NACC) & 1u;
         const int m0 = (tile / p.n_splits) * TC_BM;
         const int64_t m = (int64_t)m0 + row_in_tile;
         ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, p.spin_limit, IT_TC_EPI_BACKOFF);
@@ -734,7 +736,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
         }
       }
       if (!released) release();   // a warp that owns no columns of this CTA still has to sign off
-      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+      if (++acc == (uint32_t)NACC) { acc = 0; acc_phase ^= 1u; }
     }
   } else if (ADD) {
     // ------------------------------------------------------------------ gather the rows that the epilogue adds
@@ -1230,9 +1232,14 @@ constexpr size_t kWeightBudget = kSmemBudget - kSmemAux - 1024 /*per-column cons
 // input again: they are streamed through the stages instead, and every row tile reads them again out of the L2 (a CTA then loads
 // 48 KB for 128 x 256 x 64 multiply-adds, as before for 128 x 96 x 64, but in four stages of 48 KB instead of five of 16: resident
 // weights kept 80 KB in flight).  Resident against streamed, 1M rows: bf16 K = 768, 512 columns 1404 against 724 us; 512, 256 360 / 286;
-// 384, 256 309 / 244; 448, 192 322 / 254; 1024, 128 675 / 400; fp32 (500k rows) 600, 256 3970 / 1323; 512, 256 1686 / 1125; 1M rows
-// 320, 64 544 / 381; 384, 128 1000 / 879.  20k rows bf16 768, 512 73 / 51; 512, 256 16.0 / 15.0; but 10k rows fp32 384, 128 18.5 / 22.1:
+// 384, 256 309 / 244; 448, 192 322 / 254; 1024, 128 675 / 400; fp32, 64 columns per CTA (500k rows) 600, 256 3970 / 1323; 512, 256 1686 / 1125;
+// 1M rows 320, 64 544 / 381; 384, 128 1000 / 879.  20k rows bf16 768, 512 73 / 51; 512, 256 16.0 / 15.0; but 10k rows fp32 384, 128 18.5 / 22.1:
 // there the splits fill the SMs, so fp32 products of few tiles are streamed only from twice as many splits on.
+//
+// fp32 mode: an instruction of 2 c columns takes nearly as long for c = 64 as for 128, so a CTA takes up to 128 columns where their
+// weights stay resident or would need more than two times as many splits, with one accumulator instead of two (of 256 TMEM columns each):
+// 2M rows, K = 128, 128 columns 487 against 431 us; 1M rows 192, 96 366 / 259; 384, 128 877 / 618; 500k rows 600, 256 1325 / 826; 30k
+// rows 128, 128 16.0 / 13.3.  Not with fewer tiles than SMs, nor streamed in place of two resident splits (100k rows, 256, 128 65 / 72).
 bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_cols *out) {
   const bool tf32 = a.x_dtype == IT_F32;
   const int bk = TC_KBLOCK_BYTES / (tf32 ? 4 : 2), KB = (a.K1 + bk - 1) / bk + ((a.X2 ? a.K2 : 0) + bk - 1) / bk;
@@ -1241,8 +1248,9 @@ bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_
   out->stream = 0;
   const int n = out->n0p + out->n1p, step = want_scores ? head_dim : 16;
   if (n <= 0 || step % 16 != 0) return false;
-  // fp32 mode issues MMAs of 2 c columns and keeps 4 c TMEM columns of accumulators next to the split A stages
-  const int most = tf32 ? 64 : 256;
+  // fp32 mode issues MMAs of 2 c columns and keeps one or two accumulators of as many TMEM columns next to the split A stages
+  int most = tf32 ? 128 : 256;
+  if (tf32 && (a.M + TC_BM - 1) / TC_BM * ((n + most - 1) / most) < IT_NUM_SMS_FALLBACK) most = 64;   // few tiles: more CTAs
   for (int s = 1; s <= 16; ++s) {
     const int c = ((n + s - 1) / s + step - 1) / step * step;
     if (c > most) continue;
@@ -1255,7 +1263,7 @@ bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_
       if (wide * few <= c * s) break;
     }
     const bool few_tiles = tf32 && (a.M + TC_BM - 1) / TC_BM * few < 512;
-    if (few < s && !want_scores && (!few_tiles || s >= 2 * few)) {
+    if (few < s && !want_scores && (!few_tiles || s >= 2 * few) && (!tf32 || wide <= 64 || s > 2 * few)) {
       out->stream = 1;
       out->n_splits = few; out->nbc = wide; out->NB = wide * few;
     }
@@ -1329,7 +1337,7 @@ bool tc_shape(const it_gemm_args &a, const it_tc_cols &cols, int KB, bool want_s
     if (panels > out_panels) out_panels = panels;
   }
   // two groups of epilogue warps (alternate tiles, a staging tile each) when the second staging tile still fits
-  int epi_groups = IT_TC_EPI_GROUPS;
+  int epi_groups = tf32 && nbc > 64 ? 1 : IT_TC_EPI_GROUPS;   // (one accumulator: one tile at a time)
   if (staged && epi_groups == 2 && (kSmemBudget - kSmemAux - const_bytes - b_bytes - 2 * out_panels * panel_bytes) / stage_bytes < 3) {
     epi_groups = 1;
     if (!tf32) staged = false;   // measured: one group beats the direct stores in fp32 mode only (its tiles take long enough)
@@ -1376,7 +1384,8 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   const bool staged = sh.staged;
   const int smem = b_bytes + stages * sh.stage_bytes + epi_groups * out_panels * panel_bytes + kSmemAux + const_bytes;
   // fp32 mode: TMEM holds two accumulators of 2 nbc columns; what is left of its 512 columns stages the split A
-  int tstages = tf32 ? (512 - 4 * nbc) / TC_TSTAGE_COLS : 0;
+  const int n_acc = nbc > 64 ? 1 : 2;
+  int tstages = tf32 ? (512 - n_acc * 2 * nbc) / TC_TSTAGE_COLS : 0;
   if (tstages > TC_TSTAGES_MAX) tstages = TC_TSTAGES_MAX;
   IT_REQUIRE(!tf32 || tstages >= 2, IT_ERR_UNSUPPORTED, "tensor-core apply: no room in TMEM for two split A stages");
 
@@ -1391,7 +1400,7 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
 
   TcParams p;
   p.M = a.M; p.n_tiles_m = (int)((a.M + TC_BM - 1) / TC_BM); p.n_splits = n_splits; p.nbc = nbc;
-  p.kb1 = kb1; p.kb2 = kb2; p.NB = NB; p.stages = stages; p.tstages = tstages;
+  p.kb1 = kb1; p.kb2 = kb2; p.NB = NB; p.stages = stages; p.tstages = tstages; p.n_acc = n_acc;
   p.n0 = n0p; p.n0_real = a.n0; p.out0 = a.out0; p.out0_bf16 = a.dt0 == IT_BF16; p.bias0 = a.bias0; p.act0 = a.act0;
   p.n1 = n1p; p.n1_real = a.n1; p.out1 = a.out1; p.out1_bf16 = a.dt1 == IT_BF16;
   p.add_rows = (const char *)a.add_rows; p.add_idx = a.add_idx; p.add_pitch = a.n0 * s0; p.add_stage_bytes = (p.add_pitch + 127) / 128 * panel_bytes;

@@ -121,10 +121,12 @@ def test_dense_layer_parity(dtype, dims, act):
 
 
 @pytest.mark.parametrize("dtype,fi,fo,n", [("bf16", 768, 128, 129), ("bf16", 384, 264, 1), ("bf16", 776, 72, 300), ("bf16", 1536, 640, 128),
-                                           ("bf16", 320, 256, 40_000), ("f32", 512, 128, 127), ("f32", 600, 144, 257), ("f32", 384, 128, 40_000)])
+                                           ("bf16", 320, 256, 40_000), ("f32", 512, 128, 127), ("f32", 600, 144, 257), ("f32", 384, 128, 40_000),
+                                           ("f32", 128, 128, 20_000), ("f32", 192, 80, 40_001), ("f32", 512, 256, 10_000)])
 def test_weights_streamed_beside_the_operand(dtype, fi, fo, n):
     """Weights that leave a CTA few columns when they stay resident: row tiles and column splits with a remainder, more tiles than
-    CTAs (oracle and tolerance of the other dense layers: the products are the same)."""
+    CTAs; fp32 products of up to 128 columns per CTA, resident and streamed (oracle and tolerance of the other dense layers: the
+    products are the same)."""
     layer = make_plain_layer(3, "dense", "relu", fi, fo, dtype)
     w = small_workload(4, n, 1, dtype, [layer])
     got, _ = run_device(w)
