@@ -1,6 +1,7 @@
 // Graph ingest, validation, hub split into shadow rows, degree buckets.
 // Integer-only work.  The arrays that the interface reports are a pure function of (indptr, threshold) and reproducible bit for
 // bit; in the lists that the gather walks the order of the pieces inside a bin is that of atomics, which no result depends on.
+#include <mutex>
 #include <new>
 #include <type_traits>
 #include <stdarg.h>
@@ -441,6 +442,51 @@ __global__ void __launch_bounds__(PIECE_BINS) long_pieces_kernel(SplitParams p) 
 }
 
 // ----------------------------------------------------------------------------- host side
+// Status words of graphs: the validation's flags, later set by a kernel that gives up a wait.  They come from a fixed array, since an
+// allocation of four bytes costs as much as any (0.33 ms, and 0.26 to give it back: a quarter of the set-up of 5M vertices / 100M edges); beyond
+// that many graphs on a device at a time, and on devices beyond the first 64, a word is allocated.  A word is given back when nothing on the
+// device uses it any more: after the graph's arrays, whose release waits for the device.
+constexpr int STATUS_WORDS = 1024;
+static __device__ int g_status_words[STATUS_WORDS];
+namespace {
+constexpr int kMaxDevices = 64;
+std::mutex g_status_mu;
+int *g_status_base[kMaxDevices] = {nullptr};
+uint64_t g_status_taken[kMaxDevices][STATUS_WORDS / 64] = {};
+}  // namespace
+
+static it_status status_take(int device, int **out) {
+  if (device >= 0 && device < kMaxDevices) {
+    std::lock_guard<std::mutex> lk(g_status_mu);
+    if (!g_status_base[device]) {
+      void *p = nullptr;
+      IT_CUDA_TRY(cudaGetSymbolAddress(&p, g_status_words));
+      g_status_base[device] = static_cast<int *>(p);
+    }
+    for (int i = 0; i < STATUS_WORDS / 64; ++i) {
+      uint64_t &taken = g_status_taken[device][i];
+      if (taken == ~(uint64_t)0) continue;
+      const int bit = __builtin_ctzll(~taken);
+      taken |= (uint64_t)1 << bit;
+      *out = g_status_base[device] + i * 64 + bit;
+      return IT_OK;
+    }
+  }
+  IT_CUDA_TRY(cudaMalloc(out, sizeof(int)));
+  return IT_OK;
+}
+static void status_give_back(int device, int *word) {
+  if (device >= 0 && device < kMaxDevices) {
+    std::lock_guard<std::mutex> lk(g_status_mu);
+    const int64_t at = g_status_base[device] ? word - g_status_base[device] : -1;
+    if (at >= 0 && at < STATUS_WORDS) {
+      g_status_taken[device][at / 64] &= ~((uint64_t)1 << (at % 64));
+      return;
+    }
+  }
+  cudaFree(word);
+}
+
 // Nothing on the device may still use the graph's arrays: cudaFree waits for it.  (It may also be called while another thread
 // captures a stream, which a synchronisation of the device may not.)
 static void slab_free(it_graph *g) {
@@ -482,23 +528,26 @@ static size_t carve_split(SplitParams &p, char *slab, int64_t R, int64_t L, int6
   return off;
 }
 
-static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
-  // The arrays of the previous split are written over.  Where nothing but that split itself, which waited for its stream, has
-  // used them this needs no wait; else what still reads them, on any stream, comes first.
-  if (g->used.exchange(false)) slab_free(g);
-  forget_split(g);
-  g->threshold = T > 0 ? T : 0;
-  const int64_t n = g->n;
+// What a split of the graph at threshold T looks like: its parameters and how much room its arrays need at most.
+struct SplitPlan {
   SplitParams p{};
+  unsigned blocks;
+  int64_t R, L, P;      // shadow rows, long vertices, pieces
+  bool count_first;     // counted before the arrays are laid out
+};
+constexpr int64_t kFixedBounds[N_FIXED] = {0, 8, 32, 256, 1024};   // (list_of)
+
+static void plan_split(const it_graph *g, int64_t T, SplitPlan &s) {
+  SplitParams &p = s.p;
+  const int64_t n = g->n;
   p.ip = IndptrView{g->indptr, g->indptr_type == IT_I64};
   p.n = n; p.e = g->e; p.T = T;
   p.n_tiles = (n + SPLIT_TILE - 1) / SPLIT_TILE;
-  const unsigned split_blocks = (unsigned)((p.n_tiles + SPLIT_THREADS / 32 - 1) / (SPLIT_THREADS / 32));
+  s.blocks = (unsigned)((p.n_tiles + SPLIT_THREADS / 32 - 1) / (SPLIT_THREADS / 32));
   // degree buckets: {0, 8, 32, 256, 1024, everything longer}
-  const int64_t fixed[N_FIXED] = {0, 8, 32, 256, 1024};   // (list_of)
   p.B.nb = 0;
   for (int i = 0; i < N_FIXED; ++i)
-    if (T <= 0 || fixed[i] < T) p.B.b[p.B.nb++] = fixed[i];
+    if (T <= 0 || kFixedBounds[i] < T) p.B.b[p.B.nb++] = kFixedBounds[i];
   p.B.b[p.B.nb++] = T > 0 ? T : INT64_MAX;
 
   // A piece spans 128 / d of the source table, which has to stay small against the cache: the larger the table, the longer
@@ -515,22 +564,39 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   // at most one row per vertex and one more per T edges, a long vertex per long_above edges, a piece per piece_min of them
   // and one more each; only where that is far above the number of vertices are they counted before the arrays are laid out
   const int64_t e = g->e;
-  int64_t R = n + (T > 0 ? e / T : 0), L = n < e / p.long_above ? n : e / p.long_above, P = e / p.piece_min + L;
-  const bool count_first = R + P > n + n / 2 + (1 << 22) || R > (int64_t)INT32_MAX - 1;
+  s.R = n + (T > 0 ? e / T : 0); s.L = n < e / p.long_above ? n : e / p.long_above; s.P = e / p.piece_min + s.L;
+  s.count_first = s.R + s.P > n + n / 2 + (1 << 22) || s.R > (int64_t)INT32_MAX - 1;
+}
+
+// Grow the graph's allocation; what it holds is not kept.
+static it_status reserve(it_graph *g, size_t bytes) {
+  if (bytes <= g->slab_bytes) return IT_OK;
+  slab_free(g);
+  size_t room = bytes + bytes / 8;   // for the few more rows of another threshold, where the device has it
+  if (cudaMalloc(&g->slab, room) != cudaSuccess) {
+    cudaGetLastError();
+    g->slab = nullptr;
+    room = bytes;
+    IT_CUDA_TRY(cudaMalloc(&g->slab, room));
+  }
+  g->slab_bytes = room;
+  return IT_OK;
+}
+
+static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
+  // The arrays of the previous split are written over.  Where nothing but that split itself, which waited for its stream, has
+  // used them this needs no wait; else what still reads them, on any stream, comes first.
+  if (g->used.exchange(false)) slab_free(g);
+  forget_split(g);
+  g->threshold = T > 0 ? T : 0;
+  const int64_t n = g->n;
+  SplitPlan plan;
+  plan_split(g, T, plan);
+  SplitParams &p = plan.p;
+  const unsigned split_blocks = plan.blocks;
+  int64_t R = plan.R, L = plan.L, P = plan.P;
+  const bool count_first = plan.count_first;
   int64_t h[SPLIT_COLS + IT_MAX_BUCKETS] = {0};
-  auto reserve = [&](size_t bytes) -> it_status {   // grow the graph's allocation; what it holds is not kept
-    if (bytes <= g->slab_bytes) return IT_OK;
-    slab_free(g);
-    size_t room = bytes + bytes / 8;   // for the few more rows of another threshold, where the device has it
-    if (cudaMalloc(&g->slab, room) != cudaSuccess) {
-      cudaGetLastError();
-      g->slab = nullptr;
-      room = bytes;
-      IT_CUDA_TRY(cudaMalloc(&g->slab, room));
-    }
-    g->slab_bytes = room;
-    return IT_OK;
-  };
   auto count = [&]() -> it_status {
     IT_CUDA_TRY(cudaMemsetAsync(p.totals, 0, (size_t)((char *)p.tiles - (char *)p.totals), st));
     if (n > 0) {
@@ -546,7 +612,7 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
     return IT_OK;
   };
   if (count_first) {
-    IT_TRY(reserve(carve_split(p, nullptr, 0, 0, 0)));
+    IT_TRY(reserve(g, carve_split(p, nullptr, 0, 0, 0)));
     carve_split(p, g->slab, 0, 0, 0);
     IT_TRY(count());
     IT_TRY(read_totals());
@@ -556,7 +622,7 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
       return IT_ERR_UNSUPPORTED;
     }
   }
-  IT_TRY(reserve(carve_split(p, nullptr, R, L, P)));
+  IT_TRY(reserve(g, carve_split(p, nullptr, R, L, P)));
   carve_split(p, g->slab, R, L, P);
   IT_TRY(count());
   if (n > 0) {
@@ -590,7 +656,7 @@ static it_status split_impl(it_graph *g, int64_t T, cudaStream_t st) {
   for (int k = 0; k < N_LISTS; ++k) {
     g->h_list_offsets[k + 1] = g->h_list_offsets[k] + h[nb + 4 + k];
     g->h_list_edges[k] = h[SPLIT_COLS + k];
-    g->list_bounds[k] = k < N_FIXED && fixed[k] < p.long_above ? fixed[k] : p.long_above;   // whole vertices have no more edges
+    g->list_bounds[k] = k < N_FIXED && kFixedBounds[k] < p.long_above ? kFixedBounds[k] : p.long_above;   // whole vertices have no more edges
   }
   g->h_list_offsets[N_LISTS + 1] = n + (g->n_partial_rows - g->n_long);
   g->h_list_edges[N_LISTS] = h[SPLIT_COLS + IT_MAX_BUCKETS - 1];
@@ -629,8 +695,9 @@ static it_status create_impl(int64_t n, int64_t n_src, int64_t e, const void *in
   cudaStream_t st = (cudaStream_t)stream;
 
   // one word: the validation's flags, and later the status of the graph's kernels
-  int *d_status = nullptr;
-  IT_CUDA_TRY(cudaMalloc(&d_status, sizeof(int)));
+  int *d_status = nullptr, device = -1;
+  IT_CUDA_TRY(cudaGetDevice(&device));
+  IT_TRY(status_take(device, &d_status));
   IndptrView ip{indptr, indptr_type == IT_I64};
   cudaError_t ce = cudaMemsetAsync(d_status, 0, sizeof(int), st);
   int h_flags = 0;
@@ -644,9 +711,27 @@ static it_status create_impl(int64_t n, int64_t n_src, int64_t e, const void *in
     }
     ce = cudaGetLastError();
   }
+  // While the device looks the graph over: the handle, and the room for its first split (0.34 ms of the host's time; what fails here is
+  // reported below, after what the graph itself may be refused for)
+  it_graph *g = ce == cudaSuccess ? new (std::nothrow) it_graph() : nullptr;
+  it_status room = IT_OK;
+  if (g != nullptr) {
+    g->n = n; g->n_src = n_src; g->e = e; g->indptr = indptr; g->indptr_type = indptr_type;
+    g->indices = indices; g->edge_weights = edge_weights;
+    g->device = device;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device) == cudaSuccess && sms > 0) g->num_sms = sms;
+    SplitPlan plan;
+    plan_split(g, 0, plan);
+    if (!plan.count_first) room = reserve(g, carve_split(plan.p, nullptr, plan.R, plan.L, plan.P));
+  }
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_flags, d_status, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-  if (ce != cudaSuccess || h_flags != 0) cudaFree(d_status);
+  if (ce != cudaSuccess || h_flags != 0 || g == nullptr || room != IT_OK) {
+    if (g != nullptr) slab_free(g);
+    delete g;
+    status_give_back(device, d_status);
+  }
   if (ce != cudaSuccess) {
     it_set_error("graph validation failed to run: %s", cudaGetErrorString(ce));
     return IT_ERR_CUDA;
@@ -656,16 +741,9 @@ static it_status create_impl(int64_t n, int64_t n_src, int64_t e, const void *in
                  (h_flags & 4) ? " indptr[n] != n_edges;" : "", (h_flags & 8) ? " a source id is outside [0, n_sources);" : "");
     return IT_ERR_BAD_GRAPH;
   }
-
-  it_graph *g = new (std::nothrow) it_graph();
-  if (g == nullptr) cudaFree(d_status);
+  if (room != IT_OK) return room;   // (its text is set)
   IT_REQUIRE(g != nullptr, IT_ERR_OOM, "host allocation failed");
-  g->n = n; g->n_src = n_src; g->e = e; g->indptr = indptr; g->indptr_type = indptr_type;
-  g->indices = indices; g->edge_weights = edge_weights;
   g->d_status = d_status;   // zero: the flags were
-  cudaGetDevice(&g->device);
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device) == cudaSuccess && sms > 0) g->num_sms = sms;
   it_status rc = split_impl(g, 0, st);
   if (rc != IT_OK) { it_graph_destroy(g); return rc; }
   *out = g;
@@ -727,7 +805,7 @@ extern "C" it_status it_graph_check(it_graph *g, void *stream) {
 extern "C" it_status it_graph_destroy(it_graph *g) {
   if (!g) return IT_OK;
   slab_free(g);
-  cudaFree(g->d_status);
+  status_give_back(g->device, g->d_status);
   delete g;
   return IT_OK;
 }
