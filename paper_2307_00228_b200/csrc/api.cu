@@ -116,6 +116,13 @@ WeightBytes weight_bytes(const it_graph *g, const it_layer_desc *L) {
   return w;
 }
 
+// Whether the per-edge product of learned messages can add the source part, finish the message and reduce it itself.
+bool message_in_product(const it_graph *g, const it_layer_desc *L) {
+  it_gemm_args ga{};
+  ga.M = g->e; ga.x_dtype = L->feat_dtype; ga.X1 = g; ga.K1 = L->edge_dim; ga.n0 = L->msg_dim; ga.dt0 = ga.dt1 = L->feat_dtype;
+  return it_tc_adds_rows(ga);
+}
+
 // The scratch of a layer.  lean: without partial rows (long vertices are then reduced whole, one block each).
 LayerWs plan_layer(const it_graph *g, const it_layer_desc *L, bool lean = false) {
   LayerWs w;
@@ -163,12 +170,17 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L, bool lean = false)
       w.off_a = take(n * (fi + fe) * s);  // A = [aggregate of w_e h_u | aggregate of e_vu]
       w.off_b = off;
       break;
-    case PLAN_MSG:
-      w.off_partials = take(pieces * fm * 4);
+    case PLAN_MSG: {
+      const bool reduced = fe > 0 && message_in_product(g, L);
+      const size_t tiles = ((size_t)g->e + IT_MSG_TILE - 1) / IT_MSG_TILE;
+      w.off_partials = take(reduced ? 0 : pieces * fm * 4);
       w.off_a = take(n * fm * s);                            // A: aggregate of the messages
       w.off_b = take(n * fm * s);                            // P: source part of the message, one row per vertex
-      w.off_q = take(fe > 0 ? (size_t)g->e * fm * s : 0);    // Q, then the messages in place: one row per edge
+      // Q, then the messages in place: one row per edge; or, where their product reduces them, two partial rows per tile of edges
+      // with the tile's first vertex, and where vertices end
+      w.off_q = take(reduced ? it_align_up(tiles * 2 * fm * 4) + it_align_up(tiles * 4) + tiles * IT_MSG_TILE * 4 : (fe > 0 ? (size_t)g->e * fm * s : 0));
       break;
+    }
   }
   w.bytes = off;
   return w;
@@ -249,7 +261,7 @@ it_status run_apply(const StageCtx &c, const it_layer_desc *L, it_prep_kind kind
 
 // out [M, n_out] = act(X [M, K] * W [K, n_out] + bias): one plain dense product with W taken as it is.
 it_status run_dense(const StageCtx &c, int64_t M, const void *X, int K, const void *W, int n_out, const float *bias, it_act act, void *out,
-                    const void *add_rows = nullptr, const int32_t *add_idx = nullptr) {
+                    const void *add_rows = nullptr, const int32_t *add_idx = nullptr, const it_tc_reduce *reduce = nullptr) {
   const it_layer_desc *L = c.L;
   it_layer_desc d = *L;   // a view of the layer that names this product's weights
   d.op = IT_GATHER_NONE; d.in_dim = K; d.out_dim = n_out; d.W = W; d.heads = 1; d.edge_dim = 0; d.msg_dim = 0;
@@ -259,14 +271,8 @@ it_status run_dense(const StageCtx &c, int64_t M, const void *X, int K, const vo
   ga.n0 = n_out; ga.out0 = out; ga.dt0 = L->feat_dtype; ga.bias0 = bias; ga.act0 = act;
   ga.n1 = 0; ga.out1 = nullptr; ga.dt1 = L->feat_dtype; ga.out2 = nullptr;
   ga.add_rows = add_rows; ga.add_idx = add_idx;
+  if (reduce) ga.reduce = *reduce;
   return run_apply(c, &d, IT_PREP_DENSE, ga, nullptr);
-}
-
-// Whether the per-edge product of learned messages can add the source part and finish the message itself.
-bool message_in_product(const it_graph *g, const it_layer_desc *L) {
-  it_gemm_args ga{};
-  ga.M = g->e; ga.x_dtype = L->feat_dtype; ga.X1 = g; ga.K1 = L->edge_dim; ga.n0 = L->msg_dim; ga.dt0 = ga.dt1 = L->feat_dtype;
-  return it_tc_adds_rows(ga);
 }
 
 // The edge-feature half of the message [w_e h_u | e_vu]: the same reduce over the rows of the edge-feature
@@ -373,16 +379,26 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
         gg.src = table;
         return it_launch_gather(gg, c.st);
       } else {
-        // the edge part Q = e W_edge[in:] + b_edge, once per edge; m_j = act_edge(P[u_j] + Q[j]) in the product's epilogue, or
-        // (shapes that it does not take) in place; then the reduce over the message rows, which lie in edge order
+        // the edge part Q = e W_edge[in:] + b_edge, once per edge; the product's epilogue makes m_j = act_edge(P[u_j] + Q[j]) of it
+        // and reduces the messages; shapes that it does not take: in place, then the reduce over the rows, which lie in edge order
         void *Q = c.ws + c.w.off_q;
         const size_t es = (size_t)it_dtype_size(dt);
         const char *W_edge_part = (const char *)L->W_edge + (size_t)L->in_dim * L->msg_dim * es;
-        const bool whole = message_in_product(g, L);
-        IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, whole ? L->act_edge : IT_ACT_NONE, Q,
-                         whole ? table : nullptr, whole ? g->indices : nullptr));
+        if (message_in_product(g, L)) {
+          const size_t tiles = ((size_t)g->e + IT_MSG_TILE - 1) / IT_MSG_TILE;
+          int32_t *first = reinterpret_cast<int32_t *>((char *)Q + it_align_up(tiles * 2 * (size_t)L->msg_dim * 4));
+          int32_t *ends = reinterpret_cast<int32_t *>((char *)first + it_align_up(tiles * 4));
+          it_tc_reduce q;
+          q.indptr = g->indptr; q.indptr64 = g->indptr_type == IT_I64; q.n = g->n; q.tile_first = first; q.ends = ends; q.partial = reinterpret_cast<float *>(Q);
+          q.weights = L->use_edge_weights ? g->edge_weights : nullptr; q.dst = out; q.dst_ld = q.dim = L->msg_dim;
+          q.mode = gg.op == IT_GATHER_MAX ? 2 : (gg.op == IT_GATHER_MIN ? 3 : (q.weights ? 1 : 0)); q.is_mean = gg.op == IT_GATHER_MEAN;
+          if (!c.recording()) IT_TRY(it_launch_message_tiles(g, first, ends, c.st));
+          IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, L->act_edge, nullptr, table, g->indices, &q));
+          return c.recording() ? IT_OK : it_launch_message_combine(g, q, c.st);
+        }
+        IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, IT_ACT_NONE, Q));
         if (c.recording()) return IT_OK;
-        if (!whole) IT_TRY(it_launch_edge_messages(g, dt, L->msg_dim, table, Q, L->act_edge, c.st));
+        IT_TRY(it_launch_edge_messages(g, dt, L->msg_dim, table, Q, L->act_edge, c.st));
         gg.src = Q; gg.src_ld = 0; gg.per_edge_rows = 1;
         return it_launch_gather(gg, c.st);
       }

@@ -110,22 +110,24 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Named barriers of the epilogue warps (immediate operands): barrier 1 over all sixteen warps, or barriers 1 and 2
-// over the eight warps of a group.  The reducing form also tells every thread whether any of them failed.
+// over the eight warps of a group, or 1 to 4 over the four.  The reducing form also tells every thread whether any of them failed.
 __device__ __forceinline__ void epi_bar_sync(int groups, int group) {
   if (groups == 1) asm volatile("bar.sync 1, %0;" ::"n"(32 * TC_EPI_WARPS) : "memory");
+  else if (groups == 4) asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(8 * TC_EPI_WARPS) : "memory");
   else if (group == 0) asm volatile("bar.sync 1, %0;" ::"n"(16 * TC_EPI_WARPS) : "memory");
   else asm volatile("bar.sync 2, %0;" ::"n"(16 * TC_EPI_WARPS) : "memory");
 }
 #define IT_EPI_BAR_RED(ID, N)                                                        \
   asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"                 \
-               "bar.red.or.pred q, " #ID ", %2, p;\n\t"                              \
+               "bar.red.or.pred q, %3, %2, p;\n\t"                                   \
                "selp.u32 %0, 1, 0, q;\n\t}"                                          \
                : "=r"(r)                                                             \
-               : "r"((uint32_t)flag), "n"(N)                                         \
+               : "r"((uint32_t)flag), "n"(N), "r"((uint32_t)(ID))                    \
                : "memory")
 __device__ __forceinline__ bool epi_bar_any(int groups, int group, bool flag) {
   uint32_t r;
   if (groups == 1) IT_EPI_BAR_RED(1, 32 * TC_EPI_WARPS);
+  else if (groups == 4) IT_EPI_BAR_RED(1 + group, 8 * TC_EPI_WARPS);
   else if (group == 0) IT_EPI_BAR_RED(1, 16 * TC_EPI_WARPS);
   else IT_EPI_BAR_RED(2, 16 * TC_EPI_WARPS);
   return r != 0;
@@ -209,7 +211,8 @@ struct TcParams {
   // epilogue routing (columns are global column ids)
   int n0, n0_real; void *out0; int out0_bf16; const float *bias0; int act0;   // n0, n1: with their padding; *_real: what is stored
   int n1, n1_real; void *out1; int out1_bf16;
-  const char *add_rows; const int32_t *add_idx; int add_pitch, add_stage_bytes;   // ADD: the rows, bytes from one to the next, bytes of a ring stage
+  const char *add_rows; const int32_t *add_idx; int add_pitch, add_stage_bytes, add_stages;   // ADD: the rows, bytes from one to the next, bytes of a ring stage, stages
+  it_tc_reduce red;               // ADD: what becomes of the finished rows
   float *scores; const float *att_src; const float *att_dst; int heads, head_dim;  // GAT: scores [M, 2*heads]
   int *status;                    // set to 1 if a bounded wait gave up
   int tma_store;                  // 1: the epilogue stages each output tile in shared memory and writes it with TMA stores
@@ -219,14 +222,111 @@ struct TcParams {
   int no_loads;                   // test hook: the producer issues no copies, so every wait runs out
 };
 
-// ADD (bf16): four more warps gather a row per row of the tile into a ring in shared memory, copied asynchronously and ahead of
-// the product, and the epilogue adds it (learned messages: the source part of every edge's message).  The copies of up to four
-// tiles are in flight; with the epilogue's own loads in their place the kernel waited for them: 16M edges, 64 columns, whole layer 2.16 -> 1.95 ms.
-constexpr int TC_ADD_STAGES = 4;
+// ADD (bf16, learned messages: a row of the product is an edge): four more warps gather a row per row of the tile into a ring in
+// shared memory, copied asynchronously and ahead of the product, and the epilogue adds it (the source part of the edge's message).
+// With the epilogue's own loads in their place the kernel waited for them: 16M edges, 64 columns, whole layer 2.16 -> 1.95 ms.
+// The message takes the place of the row that was added, and the finished rows are reduced by destination where they lie: a tile is
+// 128 consecutive edges, so a run of consecutive vertices of which the first and the last may be cut.  A warp folds the vertices that
+// end in its rows, a column pair per lane; a vertex that crosses tiles leaves one fp32 row per tile for it_launch_message_combine.
+// ADD: warps of an epilogue group, four (four tiles at a time) for up to 64 columns, else eight.
+// Bound by issue slots and the latency of an epilogue warp's tile (16 of these warps, 5100 warp instructions per tile of 128 x 64, 2.2
+// per clock and SM; without the reduce the kernel takes 0.75 ms instead of 1.05).  Written out and reduced by the gather instead, the
+// message rows cost 4 GB of traffic: 1M vertices, 16M edges, 32 features, 64 columns, whole layer 1.60 against 1.26 ms.  Eight warps of
+// their own for the reduce, which leave 64 registers a thread: 1.57.
+constexpr int TC_ADD_STAGES_MAX = 8;
 constexpr int TC_THREADS_ADD = TC_THREADS_BF16 + 128;
+static_assert(IT_MSG_TILE == TC_BM, "a tile of edges is a tile of rows");
+constexpr int TC_SEG_WORDS = 2 * TC_BM + 4;   // ADD: per ring stage, the vertex that ends at a row (or -1), weight of a row, the vertex that ends before the tile
+constexpr int TC_IDS_AHEAD = 4;               // ADD: tiles that source ids are fetched ahead of the rows
+__host__ __device__ constexpr int tc_add_warps(int nbc) { return nbc <= 64 ? 4 : 8; }   // warps that fold a tile
+__device__ __forceinline__ uint32_t lds_b32(uint32_t at) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
+  return v;
+}
+// What the reduce of a tile's rows does with two neighbouring columns.
+enum { TC_FOLD_SUM = 0, TC_FOLD_WSUM = 1, TC_FOLD_MAX = 2, TC_FOLD_MIN = 3 };
+template <int MODE>
+__device__ __forceinline__ float2 tc_fold_id() {
+  const float x = MODE == TC_FOLD_MAX ? -INFINITY : (MODE == TC_FOLD_MIN ? INFINITY : 0.f);
+  return make_float2(x, x);
+}
+template <int MODE>
+__device__ __forceinline__ void tc_fold_row(float2 &a, uint32_t raw, float w) {   // a result and a row's two bf16 entries
+  if (MODE == TC_FOLD_SUM) {
+    asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(a.x), "+f"(a.y) : "r"(raw));
+  } else {
+    const float lo = __uint_as_float(raw << 16), hi = __uint_as_float(raw & 0xffff0000u);
+    if (MODE == TC_FOLD_WSUM) { a.x = fmaf(w, lo, a.x); a.y = fmaf(w, hi, a.y); }
+    else if (MODE == TC_FOLD_MAX) { a.x = fmaxf(a.x, w * lo); a.y = fmaxf(a.y, w * hi); }
+    else { a.x = fminf(a.x, w * lo); a.y = fminf(a.y, w * hi); }
+  }
+}
+
+// The reduce of one tile by the warps of its group.  tile_s: the tile (128-byte swizzled panels); seg: the vertex that ends at every row
+// (or -1), then the rows' weights; cut_before: the tile's first edge is not the first of its vertex; has_next: another tile follows.
+template <int MODE, int WARPS>
+__device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *seg, bool cut_before, bool has_next, int64_t tile, int gw, int lane,
+                                               const it_tc_reduce &q, int nbc) {
+  constexpr int RW = TC_BM / WARPS;   // a warp folds the vertices that end in its RW rows (the last one also the vertex that does not end)
+  const uint32_t chunk = (uint32_t)(lane >> 2) << 4;
+  // the tile's ends, 32 rows to a word, and the first row after the last end before mine
+  unsigned mine = 0;
+  int start = 0;
+#pragma unroll
+  for (int w = 0; w < TC_BM / 32; ++w) {
+    const unsigned ends = __ballot_sync(0xffffffffu, seg[w * 32 + lane] >= 0), before = ends & (gw * RW >= (w + 1) * 32 ? 0xffffffffu : (gw * RW <= w * 32 ? 0u : 0xffffu));
+    if (before) start = w * 32 + 32 - __clz(before);
+    if (gw * RW / 32 == w) mine = RW == 32 ? ends : (ends >> (gw * RW % 32)) & 0xffffu;
+  }
+  // rows [start, end] belong to one vertex; dest < 0: it goes on in the next tile
+  auto fold = [&](int end, int dest) {
+    const bool part = dest < 0 || (start == 0 && cut_before);
+    for (int c0 = 0; c0 < nbc; c0 += 64) {
+      float2 a = tc_fold_id<MODE>();
+      uint32_t row = tile_s + (uint32_t)(c0 >> 6) * (uint32_t)(TC_BM * TC_KBLOCK_BYTES) + (uint32_t)(start & ~7) * 128u + (uint32_t)(lane & 3) * 4u;
+      for (int r0 = start & ~7; r0 <= end; r0 += 8, row += 1024u) {   // eight rows at a time, whose places are known but for r0
+        uint32_t v[8], w[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          v[r] = lds_b32(row + (chunk ^ (uint32_t)(r << 4)) + (uint32_t)r * 128u);
+          w[r] = MODE == TC_FOLD_SUM || !q.weights ? 0x3f800000u : (uint32_t)seg[TC_BM + r0 + r];
+        }
+        if (r0 < start || end - r0 < 7) {   // rows of other vertices: a value that changes nothing, and weight 1
+          const int lo = start > r0 ? start - r0 : 0, hi = end - r0 < 7 ? end - r0 : 7;
+          const unsigned rows = (0xffu << lo) & (0xffu >> (7 - hi));
+          constexpr uint32_t id = MODE == TC_FOLD_MAX ? 0xff80ff80u : (MODE == TC_FOLD_MIN ? 0x7f807f80u : 0u);
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const uint32_t in = (uint32_t)((int)(rows << (31 - r)) >> 31);
+            v[r] = (v[r] & in) | (id & ~in);
+            if (MODE != TC_FOLD_SUM) w[r] = (w[r] & in) | (0x3f800000u & ~in);
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r) tc_fold_row<MODE>(a, v[r], __uint_as_float(w[r]));
+      }
+      const int c = c0 + 2 * lane;
+      if (c >= q.dim) continue;
+      if (part) {
+        *reinterpret_cast<float2 *>(q.partial + (tile * 2 + (start == 0 && cut_before ? 0 : 1)) * q.dim + c) = a;
+      } else {
+        if (q.is_mean) { const float inv = 1.f / (float)(end + 1 - start); a.x *= inv; a.y *= inv; }
+        *reinterpret_cast<__nv_bfloat162 *>(reinterpret_cast<__nv_bfloat16 *>(q.dst) + (int64_t)dest * q.dst_ld + c) = __floats2bfloat162_rn(a.x, a.y);
+      }
+    }
+  };
+  for (; mine; mine &= mine - 1) {
+    const int end = gw * RW + __ffs(mine) - 1;
+    fold(end, seg[end]);
+    start = end + 1;
+  }
+  if (gw == WARPS - 1 && has_next && start < TC_BM) fold(TC_BM - 1, -1);
+}
+
 // STREAM: the weights do not stay in shared memory; the k-block of them that belongs to an operand tile comes with it, in the same
 // stage.  (For weights so large that a CTA could keep few columns of them only: it_tc_columns.)
-template <bool TF32, bool ADD, bool STREAM>
+template <bool TF32, int ADD, bool STREAM>
 __global__ void __launch_bounds__(TF32 ? TC_THREADS_TF32 : (ADD ? TC_THREADS_ADD : TC_THREADS_BF16), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_x2,
                const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_o0,
@@ -247,18 +347,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
   unsigned char *smem_a = base + b_bytes;   // b_bytes is a multiple of 1024 (nbc is a multiple of 16)
   unsigned char *smem_out = smem_a + (size_t)p.stages * stage_bytes;   // output staging panels (TMA-store epilogue), 1024-byte aligned
   unsigned char *smem_add = smem_out + (size_t)p.out_panels * p.epi_groups * a_tile_bytes;   // ADD: ring of gathered rows, panels like the output's
-  uint64_t *bars = reinterpret_cast<uint64_t *>(smem_add + (ADD ? (size_t)TC_ADD_STAGES * p.add_stage_bytes : 0));
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem_add + (ADD ? (size_t)p.add_stages * p.add_stage_bytes : 0));
   uint64_t *full = bars;                    // [stages]  TMA landed
   uint64_t *empty = bars + p.stages;        // [stages]  the stage's readers are done (bf16: its MMAs; fp32: the split warps)
   uint64_t *ready = bars + 2 * p.stages;    // [TC_TSTAGES_MAX]  (fp32 mode) hi / lo parts written to TMEM
   uint64_t *a_free = ready + TC_TSTAGES_MAX;   // [TC_TSTAGES_MAX]  (fp32 mode) MMAs that read a TMEM stage are done
   uint64_t *b_full = a_free + TC_TSTAGES_MAX;  // [1]
-  const int NACC = TF32 ? p.n_acc : 2;      // accumulators: tiles in flight
+  const int NACC = TF32 ? p.n_acc : (ADD == 4 ? 4 : 2);   // accumulators: tiles in flight
   uint64_t *acc_full = b_full + 1;          // [NACC]
   uint64_t *acc_empty = acc_full + NACC;    // [NACC]
-  uint64_t *add_full = acc_empty + NACC;       // [TC_ADD_STAGES]  (ADD) the tile's rows have landed
-  uint64_t *add_empty = add_full + (ADD ? TC_ADD_STAGES : 0);   // [TC_ADD_STAGES]  (ADD) the epilogue has read them
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(add_empty + (ADD ? TC_ADD_STAGES : 0));
+  const int add_stages = ADD ? p.add_stages : 0;
+  uint64_t *add_full = acc_empty + NACC;        // [add_stages]  (ADD) the tile's rows and the ends of its vertices have landed
+  uint64_t *add_empty = add_full + add_stages;  // [add_stages]  (ADD) the tile is reduced
+  int32_t *seg_s = reinterpret_cast<int32_t *>(add_empty + add_stages);   // [add_stages][TC_SEG_WORDS]  (ADD)
+  int32_t *ids_s = seg_s + add_stages * TC_SEG_WORDS;   // [TC_IDS_AHEAD][TC_BM]  (ADD) source ids
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ids_s + (ADD ? TC_IDS_AHEAD * TC_BM : 0));
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   // per-column constants of this CTA's columns, 16-byte aligned: bias (0 where none applies), GAT attention vectors
   float *bias_s = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(tmem_slot + 2) + 15) & ~(uintptr_t)15);   // [nbc]
@@ -281,9 +384,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
     }
     mbar_init(b_full, 1);
     if (ADD)
-      for (int a = 0; a < TC_ADD_STAGES; ++a) {
+      for (int a = 0; a < add_stages; ++a) {
         mbar_init(&add_full[a], 128);
-        mbar_init(&add_empty[a], TC_EPI_WARPS / p.epi_groups);
+        mbar_init(&add_empty[a], ADD);
       }
     for (int a = 0; a < NACC; ++a) {
       mbar_init(&acc_full[a], 1);
@@ -442,19 +545,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       int last_u = -1;   // the last unit this warp owns (ownership: (unit0 + u) % n_sub == gsub)
       for (int u = n_units - 1; u >= 0; --u)
         if ((unit0 + u) % n_sub == gsub) { last_u = u; break; }
-      int it = 0;   // tiles of this CTA so far: tile `it` uses accumulator it % 2, for the (it / 2)-th time
+      int it = 0;   // tiles of this CTA so far: tile `it` uses accumulator it % NACC, for the (it / NACC)-th time
+      int slot = -1;   // ADD: of the ring of rows, and how often it came round
+      uint32_t slot_phase = 1;
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
-        if (G == 2 && (it & 1) != group) continue;
-        acc = (uint32_t)(it % NACC);
-        acc_phase = (uint32_t)(it / NACC) & 1u;
+        if (ADD && (++slot == add_stages || it == 0)) { slot = 0; slot_phase ^= 1u; }
+        if (G > 1 && (it & (G - 1)) != group) continue;   // (G and NACC are 1, 2 or 4)
+        acc = (uint32_t)it & (uint32_t)(NACC - 1);
+        acc_phase = (NACC == 4 ? (uint32_t)it >> 2 : (NACC == 2 ? (uint32_t)it >> 1 : (uint32_t)it)) & 1u;
         const int m0 = (tile / p.n_splits) * TC_BM;
         const int64_t m = (int64_t)m0 + row_in_tile;
         ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, p.spin_limit, IT_TC_EPI_BACKOFF);
-        if (ADD && ok) ok = mbar_wait(&add_full[it % TC_ADD_STAGES], (uint32_t)(it / TC_ADD_STAGES) & 1u, abort_flag, p.spin_limit);
-        if (issuer) tma_store_wait_read();   // the stores of this group's previous tile have read the staging tile
+        if (ADD && ok) ok = mbar_wait(&add_full[slot], slot_phase, abort_flag, p.spin_limit);
+        if (!ADD && issuer) tma_store_wait_read();   // the stores of this group's previous tile have read the staging tile
         // one decision for all warps of the group (they meet at named barriers below, so none may leave alone)
         __syncwarp();
-        if (epi_bar_any(G, group, !ok)) { ok = false; break; }
+        if (ADD) ok = __all_sync(0xffffffffu, ok);   // (the group decides together before the reduce)
+        else if (epi_bar_any(G, group, !ok)) { ok = false; break; }
+        if (ADD && !ok) { epi_bar_any(G, group, true); break; }
         tc_fence_after();
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * acc_cols;
         bool released = false;
@@ -462,7 +570,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           // One bf16 output in one column split: a warp's 16 columns at a time, activation on packed pairs.  This kernel is bound by
           // its issue slots: with the general loop below it spent 7300 warp instructions on a tile of 128 x 64, now 4700 (16M
           // edges, 32 edge features, 64 columns: 1.42 -> 1.0 ms; the whole layer 1.93 -> 1.53).
-          const uint32_t add_row = smem_u32(smem_add) + (uint32_t)(it % TC_ADD_STAGES) * (uint32_t)p.add_stage_bytes + (uint32_t)row_in_tile * 128u;
+          const uint32_t add_row = smem_u32(smem_add) + (uint32_t)slot * (uint32_t)p.add_stage_bytes + (uint32_t)row_in_tile * 128u;
           for (int c = gsub * 16; c < p.nbc; c += 16 * n_sub) {
             uint32_t r[16], w[8];
             tmem_ld16(taddr + (uint32_t)c, r);
@@ -481,21 +589,31 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
               if (lane == 0) mbar_arrive(&acc_empty[acc]);
               released = true;
             }
+            // the product rounded as if it had been stored, plus the gathered row, rounded once
+            __nv_bfloat162 h[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               const float4 b = b4[i >> 1];
-              // the product rounded as if it had been stored, plus the gathered row
-              const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[2 * i]) + ((i & 1) ? b.z : b.x), __uint_as_float(r[2 * i + 1]) + ((i & 1) ? b.w : b.y));
-              float v0 = __low2float(h), v1 = __high2float(h);
-              asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}"
-                  : "+f"(v0), "+f"(v1) : "r"(w[i]));
-              if (p.act0 == IT_ACT_ELU) { v0 = it_elu(v0); v1 = it_elu(v1); }
-              __nv_bfloat162 m = __floats2bfloat162_rn(v0, v1);
-              if (p.act0 == IT_ACT_RELU) m = __hmax2(m, __nv_bfloat162(__nv_bfloat16_raw{0}, __nv_bfloat16_raw{0}));
-              w[i] = *reinterpret_cast<uint32_t *>(&m);
+              h[i] = __floats2bfloat162_rn(__uint_as_float(r[2 * i]) + ((i & 1) ? b.z : b.x), __uint_as_float(r[2 * i + 1]) + ((i & 1) ? b.w : b.y));
             }
-            st_shared_v4(out_base + at0, w[0], w[1], w[2], w[3]);
-            st_shared_v4(out_base + at1, w[4], w[5], w[6], w[7]);
+            if (p.act0 == IT_ACT_ELU) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const float2 f = __bfloat1622float2(h[i]), g = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w[i]));
+                h[i] = __floats2bfloat162_rn(it_elu(f.x + g.x), it_elu(f.y + g.y));
+              }
+            } else {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) h[i] = __hadd2_rn(h[i], *reinterpret_cast<const __nv_bfloat162 *>(&w[i]));
+              if (p.act0 == IT_ACT_RELU) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) h[i] = __hmax2(h[i], __nv_bfloat162(__nv_bfloat16_raw{0}, __nv_bfloat16_raw{0}));
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) w[i] = *reinterpret_cast<uint32_t *>(&h[i]);
+            st_shared_v4(add_row + at0, w[0], w[1], w[2], w[3]);   // the message where the row lay
+            st_shared_v4(add_row + at1, w[4], w[5], w[6], w[7]);
           }
         }
         for (int u = 0; !ADD && u < n_units; ++u) {
@@ -586,9 +704,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           __syncwarp();
           if (lane == 0) mbar_arrive(&acc_empty[acc]);
         }
-        if (ADD) {   // the gathered rows have been read
+        if constexpr (ADD) {
+          const int32_t *seg = seg_s + slot * TC_SEG_WORDS;
+          const uint32_t tile_s = smem_u32(smem_add) + (uint32_t)slot * (uint32_t)p.add_stage_bytes;
+          const bool cut = tile > 0 && seg[2 * TC_BM] < 0, next = (int64_t)(tile + 1) * TC_BM < p.M;
+          const int gw = (warp - 2) % ADD;
+          if (epi_bar_any(G, group, false)) { ok = false; break; }   // the tile is complete
+          if (p.red.mode == TC_FOLD_SUM) tc_reduce_tile<TC_FOLD_SUM, ADD>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
+          else if (p.red.mode == TC_FOLD_WSUM) tc_reduce_tile<TC_FOLD_WSUM, ADD>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
+          else if (p.red.mode == TC_FOLD_MAX) tc_reduce_tile<TC_FOLD_MAX, ADD>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
+          else tc_reduce_tile<TC_FOLD_MIN, ADD>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
           __syncwarp();
-          if (lane == 0) mbar_arrive(&add_empty[it % TC_ADD_STAGES]);
+          if (lane == 0) mbar_arrive(&add_empty[slot]);
+          continue;
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the TMA store's reads
         epi_bar_sync(G, group);
@@ -600,7 +728,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           tma_store_commit();
         }
       }
-      if (issuer) tma_store_wait_all();   // the staging tile must outlive the last stores
+      if (!ADD && issuer) tma_store_wait_all();   // the staging tile must outlive the last stores
     } else
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
       const int64_t m = (int64_t)(tile / p.n_splits) * TC_BM + row_in_tile;
@@ -746,18 +874,30 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
     const int pieces = p.add_pitch >> 4;   // of a row; 1 .. 16
     const bool even = 32 % pieces == 0;
     const int r_first = lane / pieces, r_step = 32 / pieces, ch_mine = lane % pieces;
-    int32_t src = 0;
-    auto source = [&](int tile) -> int32_t {
-      const int64_t m = (int64_t)(tile / p.n_splits) * TC_BM + gw * 32 + lane;
-      return tile < n_tiles && m < p.M ? __ldcs(p.add_idx + m) : 0;   // (rows past the end: row 0, not stored)
+    // Everything comes by asynchronous copies, so that no register waits for a load: the ids of a tile TC_IDS_AHEAD tiles before its
+    // rows, each thread that of its row; with the rows, where the vertices of the tile end, and the edges' weights.
+    const int g_tid = gw * 32 + lane;
+    const it_tc_reduce &q = p.red;
+    auto copy4 = [&](const void *to, const void *from, bool in) {   // 4 bytes, or zeros
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(to)), "l"(from), "r"(in ? 4 : 0) : "memory");
     };
-    src = source(blockIdx.x);
+    auto fetch_ids = [&](int64_t tile, int at) {   // (rows past the end: row 0, not stored)
+      const int64_t m = tile * TC_BM + g_tid;
+      const bool in = tile < n_tiles && m < p.M;
+      copy4(ids_s + at * TC_BM + g_tid, p.add_idx + (in ? m : 0), in);
+    };
+    for (int d = 0; d < TC_IDS_AHEAD; ++d) {
+      fetch_ids((int64_t)blockIdx.x + (int64_t)d * gridDim.x, d);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
     bool ok = true;
-    int it = 0;
+    int it = 0, s = -1;
+    uint32_t s_phase = 1;
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
-      const int s = it % TC_ADD_STAGES;
-      const int32_t next = source(tile + gridDim.x);
-      ok = mbar_wait(&add_empty[s], ((uint32_t)(it / TC_ADD_STAGES) & 1u) ^ 1u, abort_flag, p.spin_limit, IT_TC_TMA_BACKOFF);
+      if (++s == add_stages || it == 0) { s = 0; s_phase ^= 1u; }
+      asm volatile("cp.async.wait_group %0;" ::"n"(TC_IDS_AHEAD - 1) : "memory");   // this thread's ids of this tile have landed
+      const int32_t src = ids_s[(it % TC_IDS_AHEAD) * TC_BM + g_tid];
+      ok = mbar_wait(&add_empty[s], s_phase ^ 1u, abort_flag, p.spin_limit, IT_TC_TMA_BACKOFF);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       const uint32_t stage = smem_u32(smem_add) + (uint32_t)s * (uint32_t)p.add_stage_bytes;
@@ -773,8 +913,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       } else {
         for (int q = lane; q < 32 * pieces; q += 32) copy(q / pieces, q % pieces);
       }
+      int32_t *seg = seg_s + s * TC_SEG_WORDS;
+      const int64_t e0 = (int64_t)tile * TC_BM;
+      copy4(seg + g_tid, q.ends + e0 + g_tid, true);   // (as long as whole tiles)
+      if (q.weights) copy4(seg + TC_BM + g_tid, q.weights + (e0 + g_tid < p.M ? e0 + g_tid : 0), true);
+      if (g_tid == 0 && tile > 0) copy4(seg + 2 * TC_BM, q.ends + e0 - 1, true);
+      __syncwarp();   // (this tile's ids have been read)
+      fetch_ids((int64_t)tile + (int64_t)TC_IDS_AHEAD * gridDim.x, it % TC_IDS_AHEAD);
+      asm volatile("cp.async.commit_group;" ::: "memory");
       asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&add_full[s])) : "memory");
-      src = next;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");   // no copy of this CTA may be in flight when it exits
   } else {
@@ -1219,7 +1366,7 @@ it_status make_map(CUtensorMap *map, const void *ptr, int elem, int64_t rows, in
 }
 
 constexpr int kSmemBudget = 227 * 1024;
-constexpr int kSmemAux = 1024 /*alignment slack*/ + 288 /*barriers, TMEM slot, abort flag, alignment*/;
+constexpr int kSmemAux = 1024 /*alignment slack*/ + 320 /*barriers, TMEM slot, abort flag, alignment*/;
 
 }  // namespace
 
@@ -1308,7 +1455,7 @@ it_status it_launch_prep_weights_tc(const it_prep_tc *list, int count, int *zero
 }
 
 namespace {
-struct TcShape { int b_bytes, const_bytes, out_panels, epi_groups, stages, stage_bytes; bool staged; };
+struct TcShape { int b_bytes, const_bytes, out_panels, epi_groups, stages, stage_bytes, ring; bool staged; };
 
 // How a product's shared memory is used.
 bool tc_shape(const it_gemm_args &a, const it_tc_cols &cols, int KB, bool want_scores, bool add, TcShape *out) {
@@ -1318,8 +1465,18 @@ bool tc_shape(const it_gemm_args &a, const it_tc_cols &cols, int KB, bool want_s
   const int panel_bytes = TC_BM * TC_KBLOCK_BYTES;
   // one operand tile (fp32 mode: the raw tile), and the weights that are streamed with it
   const int stage_bytes = panel_bytes + (cols.stream ? (tf32 ? 2 : 1) * nbc * TC_KBLOCK_BYTES : 0);
-  const int add_bytes = add ? TC_ADD_STAGES * ((a.n0 * 2 + 127) / 128) * panel_bytes + 2 * TC_ADD_STAGES * 8 : 0;   // ring of rows to add, its barriers
-  const int const_bytes = nbc * 4 * (want_scores ? 3 : 1) + add_bytes;          // bias (+ attention vectors) of this CTA's columns
+  const int const_bytes = nbc * 4 * (want_scores ? 3 : 1);          // bias (+ attention vectors) of this CTA's columns
+  if (add) {   // the ring of rows takes what three operand stages leave; every epilogue group holds one of its stages
+    const int slot = (a.n0 * 2 + 127) / 128 * panel_bytes + TC_SEG_WORDS * 4 + 2 * 8, groups = TC_EPI_WARPS / tc_add_warps(nbc);
+    const int fixed = TC_IDS_AHEAD * TC_BM * 4, left = kSmemBudget - kSmemAux - const_bytes - b_bytes - fixed;
+    int ring = (left - 3 * stage_bytes) / slot;
+    if (ring > TC_ADD_STAGES_MAX) ring = TC_ADD_STAGES_MAX;
+    if (n_splits != 1 || cols.stream || nbc > 128 || ring < groups + 1) return false;
+    int stages = (left - ring * slot) / stage_bytes;
+    if (stages > IT_TC_MAX_STAGES) stages = IT_TC_MAX_STAGES;
+    *out = TcShape{b_bytes, const_bytes + fixed + ring * slot, 0, groups, stages, stage_bytes, ring, true};
+    return true;
+  }
   // Staged epilogue (TMA stores): possible when, for every column split, the out0 columns and the out1 columns of
   // the CTA are whole 128-byte panels or reach the end of their output (the copy clips what lies past it), and three operand
   // stages still fit beside the staging tile (three stages already give the time of eight).
@@ -1348,7 +1505,7 @@ bool tc_shape(const it_gemm_args &a, const it_tc_cols &cols, int KB, bool want_s
   if (stages > IT_TC_MAX_STAGES) stages = IT_TC_MAX_STAGES;
   if (stages < 2) return false;
   out->b_bytes = b_bytes; out->const_bytes = const_bytes; out->out_panels = out_panels; out->epi_groups = epi_groups;
-  out->stages = stages; out->staged = staged; out->stage_bytes = stage_bytes;
+  out->stages = stages; out->staged = staged; out->stage_bytes = stage_bytes; out->ring = 0;
   return true;
 }
 }  // namespace
@@ -1358,7 +1515,7 @@ bool it_tc_adds_rows(const it_gemm_args &a) {
   TcShape sh;
   const int bk = TC_KBLOCK_BYTES / (a.x_dtype == IT_F32 ? 4 : 2), KB = (a.K1 + bk - 1) / bk + ((a.X2 ? a.K2 : 0) + bk - 1) / bk;
   return a.x_dtype == IT_BF16 && a.n1 == 0 && a.n0 <= 128 && it_tc_supported(a, 1, a.n0, false) && it_tc_columns(a, a.n0, false, &cols) &&
-         cols.n_splits == 1 && !cols.stream && tc_shape(a, cols, KB, false, true, &sh) && sh.staged;
+         tc_shape(a, cols, KB, false, true, &sh);
 }
 
 // B: weights prepared by it_launch_prep_weights_tc.  a.B / a.NB / a.out2 of the generic args are ignored:
@@ -1395,7 +1552,7 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   else m2 = m1;
   IT_TRY(make_map(&mb, B, elem, (int64_t)(tf32 ? 2 : 1) * NB, (int64_t)KB * bk, nbc));
   CUtensorMap mo0 = m1, mo1 = m1;   // placeholders unless the epilogue is staged
-  if (staged && a.n0 > 0) IT_TRY(make_map(&mo0, a.out0, s0, a.M, a.n0, TC_BM));
+  if (staged && a.n0 > 0 && a.out0) IT_TRY(make_map(&mo0, a.out0, s0, a.M, a.n0, TC_BM));
   if (staged && a.n1 > 0) IT_TRY(make_map(&mo1, a.out1, s1, a.M, a.n1, TC_BM));
 
   TcParams p;
@@ -1403,7 +1560,8 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   p.kb1 = kb1; p.kb2 = kb2; p.NB = NB; p.stages = stages; p.tstages = tstages; p.n_acc = n_acc;
   p.n0 = n0p; p.n0_real = a.n0; p.out0 = a.out0; p.out0_bf16 = a.dt0 == IT_BF16; p.bias0 = a.bias0; p.act0 = a.act0;
   p.n1 = n1p; p.n1_real = a.n1; p.out1 = a.out1; p.out1_bf16 = a.dt1 == IT_BF16;
-  p.add_rows = (const char *)a.add_rows; p.add_idx = a.add_idx; p.add_pitch = a.n0 * s0; p.add_stage_bytes = (p.add_pitch + 127) / 128 * panel_bytes;
+  p.add_rows = (const char *)a.add_rows; p.add_idx = a.add_idx; p.add_pitch = a.n0 * s0; p.add_stage_bytes = (p.add_pitch + 127) / 128 * panel_bytes; p.add_stages = sh.ring;
+  p.red = a.reduce;
   p.scores = scores; p.att_src = att_src; p.att_dst = att_dst; p.heads = heads; p.head_dim = head_dim > 0 ? head_dim : 1;
   p.status = status;
   p.tma_store = staged ? 1 : 0; p.out_panels = out_panels; p.epi_groups = epi_groups;
@@ -1421,9 +1579,9 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
     IT_LAUNCH(IT_K_GEMM_TC, bytes + more, flops, st, IT_CUDA_TRY(it_launch_pdl(kernel, dim3((unsigned)grid), dim3(threads), smem, st, m1, m2, mb, mo0, mo1, p)));
     return IT_OK;
   };
-  if (tf32) IT_TRY(cols.stream ? go(gemm_tc_kernel<true, false, true>, TC_THREADS_TF32, 0.0) : go(gemm_tc_kernel<true, false, false>, TC_THREADS_TF32, 0.0));
-  else if (a.add_rows) IT_TRY(go(gemm_tc_kernel<false, true, false>, TC_THREADS_ADD, (double)a.M * (4.0 + a.n0 * 2.0)));
-  else IT_TRY(cols.stream ? go(gemm_tc_kernel<false, false, true>, TC_THREADS_BF16, 0.0) : go(gemm_tc_kernel<false, false, false>, TC_THREADS_BF16, 0.0));
+  if (tf32) IT_TRY(cols.stream ? go(gemm_tc_kernel<true, 0, true>, TC_THREADS_TF32, 0.0) : go(gemm_tc_kernel<true, 0, false>, TC_THREADS_TF32, 0.0));
+  else if (a.add_rows) IT_TRY(tc_add_warps(nbc) == 4 ? go(gemm_tc_kernel<false, 4, false>, TC_THREADS_ADD, (double)a.M * 4.0) : go(gemm_tc_kernel<false, 8, false>, TC_THREADS_ADD, (double)a.M * 4.0));
+  else IT_TRY(cols.stream ? go(gemm_tc_kernel<false, 0, true>, TC_THREADS_BF16, 0.0) : go(gemm_tc_kernel<false, 0, false>, TC_THREADS_BF16, 0.0));
   IT_CUDA_TRY(cudaGetLastError());
   return IT_OK;
 }

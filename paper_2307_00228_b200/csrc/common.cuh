@@ -271,6 +271,20 @@ size_t it_gat_partial_bytes(const it_graph *g, int dim, int heads);
 //   [0, n0)        -> out0 (dtype dt0) = act0(C + bias0)
 //   [n0, n0+n1)    -> out1 (dtype dt1), raw
 //   [n0+n1, NB)    -> out2 (fp32), raw, row stride n2 = NB - n0 - n1
+// The rows of such a product as messages of the edges of a graph (bf16 tensor-core path): reduced by destination in its epilogue.
+#define IT_MSG_TILE 128          // edges per tile
+struct it_tc_reduce {
+  const void *indptr;            // of the graph
+  int indptr64;
+  int64_t n;                     // vertices
+  const int32_t *tile_first;     // [tiles] the vertex that edge IT_MSG_TILE * t belongs to
+  const int32_t *ends;           // [tiles * IT_MSG_TILE] the vertex whose last edge this is, or -1
+  float *partial;                // [tiles][2][dim]: what a vertex that crosses tiles has in a tile where it does not begin / does begin
+  const float *weights;          // of the edges, or NULL
+  void *dst;                     // bf16 rows: the reduce of every vertex
+  int dst_ld, dim;
+  int mode, is_mean;             // 0 sum, 1 weighted sum, 2 max, 3 min
+};
 struct it_gemm_args {
   int64_t M;
   it_dtype x_dtype;
@@ -280,9 +294,9 @@ struct it_gemm_args {
   int n0; void *out0; it_dtype dt0; const float *bias0; it_act act0;
   int n1; void *out1; it_dtype dt1;
   void *out2;
-  // tensor-core path, the shapes of it_tc_adds_rows: out0[m, :] = act0(round(C + bias0) + add_rows[add_idx[m], :]), rows of
-  // n0 elements of dt0; `round` to dt0, as if the product had been stored and read back
-  const void *add_rows; const int32_t *add_idx;
+  // tensor-core path, the shapes of it_tc_adds_rows: row m = act0(round(C + bias0) + add_rows[add_idx[m], :]), rows of n0 elements
+  // of dt0; `round` to dt0, as if the product had been stored and read back.  Row m is edge m: reduced, not stored (out0 unused)
+  const void *add_rows; const int32_t *add_idx; it_tc_reduce reduce;
   uint32_t spin_limit;   // tensor-core path: polls after which a barrier wait gives up (0 = the default)
   int no_loads;          // tensor-core path, test hook: issue no operand copies
 };
@@ -337,6 +351,10 @@ bool it_tc2_supported(const it_gemm2_args &a);
 it_status it_launch_gemm2_tc(const it_gemm2_args &a, const void *B1, const void *B2, int num_sms, int *status, cudaStream_t stream);
 
 // ----------------------------------------------------------------------------- message.cu
+// Learned messages that their product reduces: which vertex every tile of edges starts in, and where vertices end ...
+it_status it_launch_message_tiles(const it_graph *g, int32_t *tile_first, int32_t *ends, cudaStream_t stream);
+// ... and, after the product, the vertices that cross tiles and those without edges.
+it_status it_launch_message_combine(const it_graph *g, const it_tc_reduce &q, cudaStream_t stream);
 // Learned messages, edge by edge: M[j, :] = act(P[indices[j], :] + M[j, :]) in place (M arrives holding the per-edge
 // part Q), rows of `dim` elements of `dtype` (a multiple of 16 bytes).
 it_status it_launch_edge_messages(const it_graph *g, it_dtype dtype, int dim, const void *P, void *M, it_act act, cudaStream_t stream);

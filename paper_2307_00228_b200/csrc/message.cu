@@ -1,7 +1,8 @@
 // Elementwise kernels around the gather:
 //   * the learned message of every edge, m_j = act(P[u_j] + Q[j]) (the source part P was computed once per vertex, the
 //     edge part Q once per edge, both by the dense transform), written over Q so that the per-edge-row gather can
-//     reduce it;
+//     reduce it; or, where the product that makes Q finishes and reduces the messages itself (bf16), the two small kernels
+//     around it: the first vertex of every tile of edges, and the vertices that cross tiles;
 //   * for GAT layers whose logits read the edge features: the message row of every edge (a copy of its source's row)
 //     and its logit term per head (source score + the edge's share), so that the reduce can walk rows in edge order;
 //   * the receiver's finish of a partial-gather over source partitions (scale, zero the vertices without in-edges,
@@ -182,7 +183,153 @@ __global__ void __launch_bounds__(MSG_THREADS) aggregate_finish_kernel(const flo
   }
 }
 
+// ----------------------------------------------------------------------------- messages reduced by their product
+__device__ __forceinline__ int64_t bound_of(const void *indptr, int is64, int64_t v) {
+  return is64 ? (int64_t)__ldg(reinterpret_cast<const long long *>(indptr) + v) : (int64_t)__ldg(reinterpret_cast<const int32_t *>(indptr) + v);
+}
+
+// tile_first[t]: the vertex that edge IT_MSG_TILE * t belongs to; ends[j]: the vertex whose last edge j is (the others: cleared
+// before).  A thread per vertex; vertices of several tiles by the whole warp.  Bound by clearing the ends and reading indptr once.
+__global__ void __launch_bounds__(MSG_THREADS) message_tiles_kernel(const void *indptr, int is64, int64_t n, int32_t *__restrict__ tile_first,
+                                                                 int32_t *__restrict__ ends) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t v0 = ((int64_t)blockIdx.x * MSG_THREADS + threadIdx.x) - lane; v0 < n; v0 += (int64_t)gridDim.x * MSG_THREADS) {
+    const int64_t v = v0 + lane;
+    int64_t t0 = 0, count = 0;
+    if (v < n) {
+      const int64_t a = bound_of(indptr, is64, v), b = bound_of(indptr, is64, v + 1);
+      t0 = (a + IT_MSG_TILE - 1) / IT_MSG_TILE;
+      if (b > a) { count = (b - 1) / IT_MSG_TILE - t0 + 1; ends[b - 1] = (int32_t)v; }
+    }
+    if (count == 1) tile_first[t0] = (int32_t)v;
+    for (unsigned many = __ballot_sync(0xffffffffu, count > 1); many; many &= many - 1) {
+      const int l = __ffs(many) - 1;
+      const int64_t at = __shfl_sync(0xffffffffu, t0, l), c = __shfl_sync(0xffffffffu, count, l);
+      for (int64_t k = lane; k < c; k += 32) tile_first[at + k] = (int32_t)(v0 + l);
+    }
+  }
+}
+
+// The vertices that cross tiles, found at the tile after the one where they begin.  A warp looks at 32 tiles at once and folds the
+// parts of their vertices, two vertices of two tiles at a time; the whole block folds a vertex of many.  Parts are folded in edge
+// order.  Bound by the trips first vertex -> its bounds -> its parts, made once for 32 tiles (one tile per warp: 114 us for 125k).
+constexpr int MSG_JOIN_THREADS = 1024, MSG_JOIN_WARPS = MSG_JOIN_THREADS / 32, MSG_JOIN_BLOCK = 48 /* parts from which on a block takes a vertex */;
+__global__ void __launch_bounds__(MSG_JOIN_THREADS, 1) message_combine_kernel(it_tc_reduce q, int64_t n_tiles) {
+  __shared__ float4 part[MSG_JOIN_WARPS][32];
+  __shared__ int64_t todo[MSG_JOIN_THREADS];
+  __shared__ int n_todo;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = lane * 4;
+  const float id = q.mode == 2 ? -INFINITY : (q.mode == 3 ? INFINITY : 0.f);
+  auto fold = [&](float4 &a, const float4 &y) {
+    if (q.mode == 2) { a.x = fmaxf(a.x, y.x); a.y = fmaxf(a.y, y.y); a.z = fmaxf(a.z, y.z); a.w = fmaxf(a.w, y.w); }
+    else if (q.mode == 3) { a.x = fminf(a.x, y.x); a.y = fminf(a.y, y.y); a.z = fminf(a.z, y.z); a.w = fminf(a.w, y.w); }
+    else { a.x += y.x; a.y += y.y; a.z += y.z; a.w += y.w; }
+  };
+  // the parts of the vertex that begins in tile b - 1: part 0 lies there, part k in tile b - 1 + k
+  auto load = [&](int64_t b, int64_t k) { return __ldcs(reinterpret_cast<const float4 *>(q.partial + ((b - 1 + k) * 2 + (k == 0 ? 1 : 0)) * q.dim + c)); };
+  auto walk = [&](int64_t b, int64_t k0, int64_t k1) {
+    float4 a = make_float4(id, id, id, id);
+    if (c >= q.dim) return a;
+    int64_t k = k0;
+    for (; k + 8 <= k1; k += 8) {
+      float4 y[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) y[u] = load(b, k + u);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) fold(a, y[u]);
+    }
+    for (; k < k1; ++k) fold(a, load(b, k));
+    return a;
+  };
+  auto finish = [&](int64_t v, int64_t deg, float4 a) {
+    if (c >= q.dim) return;
+    if (q.is_mean) { const float inv = 1.f / (float)deg; a.x *= inv; a.y *= inv; a.z *= inv; a.w *= inv; }
+    const __nv_bfloat162 h0 = __floats2bfloat162_rn(a.x, a.y), h1 = __floats2bfloat162_rn(a.z, a.w);
+    *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(q.dst) + v * q.dst_ld + c) =
+        make_uint2(*reinterpret_cast<const uint32_t *>(&h0), *reinterpret_cast<const uint32_t *>(&h1));
+  };
+  for (int64_t b0 = 1 + (int64_t)blockIdx.x * MSG_JOIN_THREADS; b0 < n_tiles; b0 += (int64_t)gridDim.x * MSG_JOIN_THREADS) {
+    if (threadIdx.x == 0) n_todo = 0;
+    __syncthreads();
+    const int64_t b = b0 + threadIdx.x;
+    int64_t v = 0, deg = 0, parts = 0;   // 0 parts: no vertex begins in tile b - 1 and goes on in tile b
+    if (b < n_tiles) {
+      v = __ldg(q.tile_first + b);
+      const int64_t s = bound_of(q.indptr, q.indptr64, v), e = bound_of(q.indptr, q.indptr64, v + 1);
+      if (s < b * IT_MSG_TILE && s >= (b - 1) * IT_MSG_TILE) { parts = (e - 1) / IT_MSG_TILE - b + 2; deg = e - s; }
+    }
+    if (parts >= MSG_JOIN_BLOCK) todo[atomicAdd(&n_todo, 1)] = b;
+    const int64_t wb = b - lane;
+    for (unsigned two = __ballot_sync(0xffffffffu, parts == 2); two;) {
+      float4 x[2], y[2];
+      int l[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        l[u] = two ? __ffs(two) - 1 : -1;
+        two &= two - 1;   // (0 stays 0)
+        if (l[u] >= 0 && c < q.dim) { x[u] = load(wb + l[u], 0); y[u] = load(wb + l[u], 1); }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int64_t vv = __shfl_sync(0xffffffffu, v, l[u] & 31), dd = __shfl_sync(0xffffffffu, deg, l[u] & 31);
+        if (l[u] < 0) continue;
+        fold(x[u], y[u]);
+        finish(vv, dd, x[u]);
+      }
+    }
+    for (unsigned some = __ballot_sync(0xffffffffu, parts > 2 && parts < MSG_JOIN_BLOCK); some; some &= some - 1) {
+      const int l = __ffs(some) - 1;
+      const int64_t vv = __shfl_sync(0xffffffffu, v, l), dd = __shfl_sync(0xffffffffu, deg, l), pp = __shfl_sync(0xffffffffu, parts, l);
+      finish(vv, dd, walk(wb + l, 0, pp));
+    }
+    __syncthreads();
+    const int n = n_todo;
+    for (int i = 0; i < n; ++i) {
+      const int64_t tb = todo[i], tv = __ldg(q.tile_first + tb), s = bound_of(q.indptr, q.indptr64, tv), e = bound_of(q.indptr, q.indptr64, tv + 1);
+      const int64_t all = (e - 1) / IT_MSG_TILE - tb + 2, per = (all + MSG_JOIN_WARPS - 1) / MSG_JOIN_WARPS;
+      const int64_t k0 = warp * per < all ? warp * per : all, k1 = k0 + per < all ? k0 + per : all;
+      part[warp][lane] = walk(tb, k0, k1);
+      __syncthreads();
+      if (warp == 0) {
+        float4 a = part[0][lane];
+        for (int w = 1; w < MSG_JOIN_WARPS; ++w) fold(a, part[w][lane]);
+        finish(tv, e - s, a);
+      }
+      __syncthreads();
+    }
+  }
+}
+
 }  // namespace
+
+it_status it_launch_message_tiles(const it_graph *g, int32_t *tile_first, int32_t *ends, cudaStream_t st) {
+  if (g->e == 0) return IT_OK;
+  IT_CUDA_TRY(cudaMemsetAsync(ends, 0xff, (size_t)((g->e + IT_MSG_TILE - 1) / IT_MSG_TILE) * IT_MSG_TILE * sizeof(int32_t), st));
+  const int64_t want = (g->n + MSG_THREADS - 1) / MSG_THREADS, cap = (int64_t)g->num_sms * 8;
+  IT_LAUNCH(IT_K_EDGE_MSG, (double)g->n * (g->indptr_type == IT_I64 ? 8.0 : 4.0) + (double)g->e / IT_MSG_TILE * 4.0, 0, st,
+            message_tiles_kernel<<<(unsigned)(want < cap ? want : cap), MSG_THREADS, 0, st>>>(g->indptr, g->indptr_type == IT_I64, g->n, tile_first, ends));
+  IT_CUDA_TRY(cudaGetLastError());
+  return IT_OK;
+}
+
+it_status it_launch_message_combine(const it_graph *g, const it_tc_reduce &q, cudaStream_t st) {
+  const int64_t tiles = (g->e + IT_MSG_TILE - 1) / IT_MSG_TILE;
+  if (tiles > 1) {
+    const int64_t want = (tiles - 1 + MSG_JOIN_THREADS - 1) / MSG_JOIN_THREADS, cap = (int64_t)g->num_sms;
+    IT_LAUNCH(IT_K_COMBINE, (double)tiles * (2.0 * q.dim * 4.0 + q.dim * 2.0), 0, st,
+              message_combine_kernel<<<(unsigned)(want < cap ? want : cap), MSG_JOIN_THREADS, 0, st>>>(q, tiles));
+    IT_CUDA_TRY(cudaGetLastError());
+  }
+  if (g->h_list_offsets[1] > g->h_list_offsets[0]) {   // the vertices without edges
+    it_empty_rows_args er{};
+    er.g = g; er.row_lo = g->h_list_offsets[0]; er.row_hi = g->h_list_offsets[1];
+    er.kind = IT_EMPTY_VALUE; er.dst = q.dst; er.dim = q.dim; er.dtype = IT_BF16; er.pitch = (int64_t)q.dst_ld * 2; er.value = 0.f;
+    er.act = IT_ACT_NONE;
+    IT_TRY(it_launch_empty_rows(er, IT_K_GATHER_EMPTY, (double)(er.row_hi - er.row_lo) * (16.0 + q.dim * 2.0), st));
+  }
+  return IT_OK;
+}
 
 it_status it_launch_edge_messages(const it_graph *g, it_dtype dtype, int dim, const void *P, void *M, it_act act, cudaStream_t st) {
   const int es = it_dtype_size(dtype);

@@ -8,6 +8,8 @@ import torch
 from gpu_util import check_against_oracle, make_gat_layer, make_msg_layer, make_sage_layer, run_device, small_workload
 from paper_2307_00228_b200 import binding as B
 from paper_2307_00228_b200 import host
+from workloads import Workload
+from workloads import rng as wrng
 
 pytestmark = pytest.mark.gpu
 
@@ -47,6 +49,38 @@ def test_messages_finished_in_the_product(fm, act):
     w = small_workload(10, 701, 13, "bf16", [layer], hubs=(300, 41), threshold=128, edge_dim=16)
     got, _ = run_device(w)
     check_against_oracle(w, got, label=(fm, act))
+
+
+# in-degrees whose sums put the ends of vertices at, before and after the 128-edge tiles of the per-edge product, vertices of several
+# tiles and of so many that a block folds their parts, runs of vertices without edges longer than a tile, a last tile of few edges
+TILE_DEGREES = {
+    "one edge": [0, 1, 0],
+    "one tile": [0, 100, 28],
+    "a tile and an edge": [64, 64, 1],
+    "aligned": [128, 256, 0, 128, 16, 112],
+    "crossing": [127, 2, 127, 1, 300, 83] + [0] * 300 + [15, 17, 16, 0, 1, 31] * 9,
+    "long": [5, 6500, 3, 0, 129, 40] + [3] * 50,
+}
+
+
+@pytest.mark.parametrize("op,weights", [("sum", False), ("sum", True), ("mean", False), ("mean", True), ("max", False), ("min", True), ("gcn", True)])
+@pytest.mark.parametrize("degrees", TILE_DEGREES)
+@pytest.mark.parametrize("fm", [40, 128])
+def test_messages_reduced_by_their_product(op, weights, degrees, fm):
+    """bf16 messages are reduced tile by tile where they are made (oracle and tolerance of the other message tests: a sum in another
+    order differs in fp32 only)."""
+    layer = make_msg_layer(13, op, "none", 16, fm, 24, "bf16", act_edge="relu", weights=weights, edge_dim=8)
+    deg = np.asarray(TILE_DEGREES[degrees])
+    base = small_workload(14, len(deg), 1, "bf16", [layer], weights=True, edge_dim=8)
+    rng = np.random.default_rng(15)
+    e = int(deg.sum())
+    ef = wrng.f32_to_bf16_bits(rng.standard_normal((e, 8)).astype(np.float32))
+    w = Workload("tiles", len(deg), e, np.concatenate(([0], np.cumsum(deg))), rng.integers(0, len(deg), e).astype(np.int32),
+                 rng.random(e, dtype=np.float32), "bf16", base.x, [layer], 0, ef)
+    got, d = run_device(w)
+    check_against_oracle(w, got, label=(op, weights, degrees, fm))
+    again, _ = run_device(w, int32_indptr=True)
+    assert np.array_equal(got, again)
 
 
 def test_message_layers_stack_with_plain_layers():
