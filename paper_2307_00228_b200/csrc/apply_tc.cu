@@ -233,43 +233,67 @@ struct TcParams {
 // per clock and SM; without the reduce the kernel takes 0.75 ms instead of 1.05).  Written out and reduced by the gather instead, the
 // message rows cost 4 GB of traffic: 1M vertices, 16M edges, 32 features, 64 columns, whole layer 1.60 against 1.26 ms.  Eight warps of
 // their own for the reduce, which leave 64 registers a thread: 1.57.
+#ifndef IT_TC_NARROW
+#define IT_TC_NARROW 1
+#endif
 constexpr int TC_ADD_STAGES_MAX = 8;
 constexpr int TC_THREADS_ADD = TC_THREADS_BF16 + 128;
 static_assert(IT_MSG_TILE == TC_BM, "a tile of edges is a tile of rows");
 constexpr int TC_SEG_WORDS = 2 * TC_BM + 4;   // ADD: per ring stage, the vertex that ends at a row (or -1), weight of a row, the vertex that ends before the tile
 constexpr int TC_IDS_AHEAD = 4;               // ADD: tiles that source ids are fetched ahead of the rows
 __host__ __device__ constexpr int tc_add_warps(int nbc) { return nbc <= 64 ? 4 : 8; }   // warps that fold a tile
+// What the reduce of a tile's rows does with two neighbouring columns (it_tc_reduce).
+enum { TC_FOLD_SUM = 0, TC_FOLD_WSUM = 1, TC_FOLD_MAX = 2, TC_FOLD_MIN = 3, TC_FOLD_PMAX = 4, TC_FOLD_PMIN = 5, TC_FOLD_STORE = 6 };
+// The result so far of a column pair: two floats, or (unweighted maximum and minimum: nothing is rounded) the packed pair.
+template <int MODE>
+struct TcPair {
+  static constexpr bool PACKED = MODE == TC_FOLD_PMAX || MODE == TC_FOLD_PMIN;
+  static constexpr uint32_t ID = MODE == TC_FOLD_MAX || MODE == TC_FOLD_PMAX ? 0xff80ff80u : (MODE == TC_FOLD_MIN || MODE == TC_FOLD_PMIN ? 0x7f807f80u : 0u);   // bf16 pair that changes nothing
+  float2 a;
+  uint32_t q;
+  __device__ __forceinline__ void clear() {
+    q = ID;
+    a = make_float2(__uint_as_float(ID << 16), __uint_as_float(ID << 16));
+  }
+  __device__ __forceinline__ void row(uint32_t raw, float w) {
+    if constexpr (MODE == TC_FOLD_PMAX) asm("max.bf16x2 %0, %0, %1;" : "+r"(q) : "r"(raw));
+    else if constexpr (MODE == TC_FOLD_PMIN) asm("min.bf16x2 %0, %0, %1;" : "+r"(q) : "r"(raw));
+    else if constexpr (MODE == TC_FOLD_SUM) asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(a.x), "+f"(a.y) : "r"(raw));
+    else {
+      const float lo = __uint_as_float(raw << 16), hi = __uint_as_float(raw & 0xffff0000u);
+      if (MODE == TC_FOLD_WSUM) { a.x = fmaf(w, lo, a.x); a.y = fmaf(w, hi, a.y); }
+      else if (MODE == TC_FOLD_MAX) { a.x = fmaxf(a.x, w * lo); a.y = fmaxf(a.y, w * hi); }
+      else { a.x = fminf(a.x, w * lo); a.y = fminf(a.y, w * hi); }
+    }
+  }
+  __device__ __forceinline__ void join(int o) {   // with the lane o away
+    if constexpr (PACKED) { row(__shfl_xor_sync(0xffffffffu, q, o), 1.f); return; }
+    const float2 b = make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+    if (MODE == TC_FOLD_MAX) { a.x = fmaxf(a.x, b.x); a.y = fmaxf(a.y, b.y); }
+    else if (MODE == TC_FOLD_MIN) { a.x = fminf(a.x, b.x); a.y = fminf(a.y, b.y); }
+    else { a.x += b.x; a.y += b.y; }
+  }
+  __device__ __forceinline__ float2 value() const {
+    if constexpr (PACKED) return make_float2(__uint_as_float(q << 16), __uint_as_float(q & 0xffff0000u));
+    return a;
+  }
+};
 __device__ __forceinline__ uint32_t lds_b32(uint32_t at) {
   uint32_t v;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(at) : "memory");
   return v;
 }
-// What the reduce of a tile's rows does with two neighbouring columns.
-enum { TC_FOLD_SUM = 0, TC_FOLD_WSUM = 1, TC_FOLD_MAX = 2, TC_FOLD_MIN = 3 };
-template <int MODE>
-__device__ __forceinline__ float2 tc_fold_id() {
-  const float x = MODE == TC_FOLD_MAX ? -INFINITY : (MODE == TC_FOLD_MIN ? INFINITY : 0.f);
-  return make_float2(x, x);
-}
-template <int MODE>
-__device__ __forceinline__ void tc_fold_row(float2 &a, uint32_t raw, float w) {   // a result and a row's two bf16 entries
-  if (MODE == TC_FOLD_SUM) {
-    asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(a.x), "+f"(a.y) : "r"(raw));
-  } else {
-    const float lo = __uint_as_float(raw << 16), hi = __uint_as_float(raw & 0xffff0000u);
-    if (MODE == TC_FOLD_WSUM) { a.x = fmaf(w, lo, a.x); a.y = fmaf(w, hi, a.y); }
-    else if (MODE == TC_FOLD_MAX) { a.x = fmaxf(a.x, w * lo); a.y = fmaxf(a.y, w * hi); }
-    else { a.x = fminf(a.x, w * lo); a.y = fminf(a.y, w * hi); }
-  }
-}
 
 // The reduce of one tile by the warps of its group.  tile_s: the tile (128-byte swizzled panels); seg: the vertex that ends at every row
 // (or -1), then the rows' weights; cut_before: the tile's first edge is not the first of its vertex; has_next: another tile follows.
-template <int MODE, int WARPS>
+// Eight rows at a time, whose places are known but for the first one's; rows of up to 32 columns (NARROW) by half a warp each.
+template <int MODE, int WARPS, bool NARROW>
 __device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *seg, bool cut_before, bool has_next, int64_t tile, int gw, int lane,
                                                const it_tc_reduce &q, int nbc) {
   constexpr int RW = TC_BM / WARPS;   // a warp folds the vertices that end in its RW rows (the last one also the vertex that does not end)
-  const uint32_t chunk = (uint32_t)(lane >> 2) << 4;
+  constexpr int LDS = NARROW ? 4 : 8, STEP = NARROW ? 2 : 1;
+  const int half = NARROW ? lane >> 4 : 0, pair = NARROW ? lane & 15 : lane;
+  const uint32_t chunk = (uint32_t)(pair >> 2) << 4;
   // the tile's ends, 32 rows to a word, and the first row after the last end before mine
   unsigned mine = 0;
   int start = 0;
@@ -283,31 +307,35 @@ __device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *s
   auto fold = [&](int end, int dest) {
     const bool part = dest < 0 || (start == 0 && cut_before);
     for (int c0 = 0; c0 < nbc; c0 += 64) {
-      float2 a = tc_fold_id<MODE>();
+      TcPair<MODE> acc;
+      acc.clear();
       uint32_t row = tile_s + (uint32_t)(c0 >> 6) * (uint32_t)(TC_BM * TC_KBLOCK_BYTES) + (uint32_t)(start & ~7) * 128u + (uint32_t)(lane & 3) * 4u;
-      for (int r0 = start & ~7; r0 <= end; r0 += 8, row += 1024u) {   // eight rows at a time, whose places are known but for r0
-        uint32_t v[8], w[8];
+      for (int r0 = start & ~7; r0 <= end; r0 += 8, row += 1024u) {
+        uint32_t v[LDS], w[LDS];
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          v[r] = lds_b32(row + (chunk ^ (uint32_t)(r << 4)) + (uint32_t)r * 128u);
-          w[r] = MODE == TC_FOLD_SUM || !q.weights ? 0x3f800000u : (uint32_t)seg[TC_BM + r0 + r];
+        for (int i = 0; i < LDS; ++i) {
+          const uint32_t r = (uint32_t)(i * STEP + half);
+          v[i] = lds_b32(row + (chunk ^ (r << 4)) + r * 128u);
+          w[i] = 0x3f800000u;
+          if (MODE == TC_FOLD_WSUM || MODE == TC_FOLD_MAX || MODE == TC_FOLD_MIN) w[i] = (uint32_t)seg[TC_BM + r0 + (int)r];
         }
         if (r0 < start || end - r0 < 7) {   // rows of other vertices: a value that changes nothing, and weight 1
           const int lo = start > r0 ? start - r0 : 0, hi = end - r0 < 7 ? end - r0 : 7;
           const unsigned rows = (0xffu << lo) & (0xffu >> (7 - hi));
-          constexpr uint32_t id = MODE == TC_FOLD_MAX ? 0xff80ff80u : (MODE == TC_FOLD_MIN ? 0x7f807f80u : 0u);
 #pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            const uint32_t in = (uint32_t)((int)(rows << (31 - r)) >> 31);
-            v[r] = (v[r] & in) | (id & ~in);
-            if (MODE != TC_FOLD_SUM) w[r] = (w[r] & in) | (0x3f800000u & ~in);
+          for (int i = 0; i < LDS; ++i) {
+            const uint32_t in = (uint32_t)((int)(rows << (31 - (i * STEP + half))) >> 31);
+            v[i] = (v[i] & in) | (TcPair<MODE>::ID & ~in);
+            if (MODE == TC_FOLD_WSUM || MODE == TC_FOLD_MAX || MODE == TC_FOLD_MIN) w[i] = (w[i] & in) | (0x3f800000u & ~in);
           }
         }
 #pragma unroll
-        for (int r = 0; r < 8; ++r) tc_fold_row<MODE>(a, v[r], __uint_as_float(w[r]));
+        for (int i = 0; i < LDS; ++i) acc.row(v[i], __uint_as_float(w[i]));
       }
-      const int c = c0 + 2 * lane;
-      if (c >= q.dim) continue;
+      if (NARROW) acc.join(16);
+      const int c = c0 + 2 * pair;
+      if (half != 0 || c >= q.dim) continue;
+      float2 a = acc.value();
       if (part) {
         *reinterpret_cast<float2 *>(q.partial + (tile * 2 + (start == 0 && cut_before ? 0 : 1)) * q.dim + c) = a;
       } else {
@@ -324,9 +352,27 @@ __device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *s
   if (gw == WARPS - 1 && has_next && start < TC_BM) fold(TC_BM - 1, -1);
 }
 
+// TC_FOLD_STORE: the tile's rows as they are, row m of q.dst for edge m (`edges` of them).
+template <int WARPS>
+__device__ __forceinline__ void tc_store_tile(uint32_t tile_s, int64_t tile, int64_t edges, int gw, int lane, const it_tc_reduce &q) {
+  constexpr int RW = TC_BM / WARPS;
+  const int pieces = q.dim / 8;   // of 16 bytes
+  for (int i = lane; i < RW * pieces; i += 32) {
+    const int r = gw * RW + i / pieces, ch = i % pieces;
+    const int64_t m = tile * TC_BM + r;
+    if (m >= edges) break;
+    const uint32_t at = tile_s + (uint32_t)(ch >> 3) * (uint32_t)(TC_BM * TC_KBLOCK_BYTES) + (uint32_t)r * 128u + (uint32_t)(((ch & 7) ^ (r & 7)) << 4);
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
+    __stcs(reinterpret_cast<uint4 *>(q.dst) + m * pieces + ch, v);
+  }
+}
+
 // STREAM: the weights do not stay in shared memory; the k-block of them that belongs to an operand tile comes with it, in the same
 // stage.  (For weights so large that a CTA could keep few columns of them only: it_tc_columns.)
-template <bool TF32, int ADD, bool STREAM>
+// FOLD (with ADD): what becomes of the rows, TC_FOLD_*, a kernel each: one reduce in the code of all warps fits the instruction
+// caches, where six side by side cost 8 % of the layer.
+template <bool TF32, int ADD, bool STREAM, int FOLD, bool NARROW>
 __global__ void __launch_bounds__(TF32 ? TC_THREADS_TF32 : (ADD ? TC_THREADS_ADD : TC_THREADS_BF16), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_x2,
                const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_o0,
@@ -710,10 +756,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           const bool cut = tile > 0 && seg[2 * TC_BM] < 0, next = (int64_t)(tile + 1) * TC_BM < p.M;
           const int gw = (warp - 2) % ADD;
           if (epi_bar_any(G, group, false)) { ok = false; break; }   // the tile is complete
-          if (p.red.mode == TC_FOLD_SUM) tc_reduce_tile<TC_FOLD_SUM, ADD>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
-          else if (p.red.mode == TC_FOLD_WSUM) tc_reduce_tile<TC_FOLD_WSUM, ADD>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
-          else if (p.red.mode == TC_FOLD_MAX) tc_reduce_tile<TC_FOLD_MAX, ADD>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
-          else tc_reduce_tile<TC_FOLD_MIN, ADD>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
+          if constexpr (FOLD == TC_FOLD_STORE) tc_store_tile<ADD>(tile_s, tile, p.M, gw, lane, p.red);
+          else tc_reduce_tile<FOLD, ADD, NARROW>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
           __syncwarp();
           if (lane == 0) mbar_arrive(&add_empty[slot]);
           continue;
@@ -915,9 +959,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       }
       int32_t *seg = seg_s + s * TC_SEG_WORDS;
       const int64_t e0 = (int64_t)tile * TC_BM;
-      copy4(seg + g_tid, q.ends + e0 + g_tid, true);   // (as long as whole tiles)
+      if (q.ends) copy4(seg + g_tid, q.ends + e0 + g_tid, true);   // (as long as whole tiles)
       if (q.weights) copy4(seg + TC_BM + g_tid, q.weights + (e0 + g_tid < p.M ? e0 + g_tid : 0), true);
-      if (g_tid == 0 && tile > 0) copy4(seg + 2 * TC_BM, q.ends + e0 - 1, true);
+      if (q.ends && g_tid == 0 && tile > 0) copy4(seg + 2 * TC_BM, q.ends + e0 - 1, true);
       __syncwarp();   // (this tile's ids have been read)
       fetch_ids((int64_t)tile + (int64_t)TC_IDS_AHEAD * gridDim.x, it % TC_IDS_AHEAD);
       asm volatile("cp.async.commit_group;" ::: "memory");
@@ -1579,9 +1623,25 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
     IT_LAUNCH(IT_K_GEMM_TC, bytes + more, flops, st, IT_CUDA_TRY(it_launch_pdl(kernel, dim3((unsigned)grid), dim3(threads), smem, st, m1, m2, mb, mo0, mo1, p)));
     return IT_OK;
   };
-  if (tf32) IT_TRY(cols.stream ? go(gemm_tc_kernel<true, 0, true>, TC_THREADS_TF32, 0.0) : go(gemm_tc_kernel<true, 0, false>, TC_THREADS_TF32, 0.0));
-  else if (a.add_rows) IT_TRY(tc_add_warps(nbc) == 4 ? go(gemm_tc_kernel<false, 4, false>, TC_THREADS_ADD, (double)a.M * 4.0) : go(gemm_tc_kernel<false, 8, false>, TC_THREADS_ADD, (double)a.M * 4.0));
-  else IT_TRY(cols.stream ? go(gemm_tc_kernel<false, 0, true>, TC_THREADS_BF16, 0.0) : go(gemm_tc_kernel<false, 0, false>, TC_THREADS_BF16, 0.0));
+  if (tf32) IT_TRY(cols.stream ? go(gemm_tc_kernel<true, 0, true, 0, false>, TC_THREADS_TF32, 0.0) : go(gemm_tc_kernel<true, 0, false, 0, false>, TC_THREADS_TF32, 0.0));
+  else if (a.add_rows) {
+    auto fold = [&]<int MODE>() -> it_status {
+      const double more = (double)a.M * 4.0;
+      if (tc_add_warps(nbc) == 8) return go(gemm_tc_kernel<false, 8, false, MODE, false>, TC_THREADS_ADD, more);
+      if (IT_TC_NARROW && nbc <= 32 && MODE != TC_FOLD_STORE) return go(gemm_tc_kernel<false, 4, false, MODE, true>, TC_THREADS_ADD, more);
+      return go(gemm_tc_kernel<false, 4, false, MODE, false>, TC_THREADS_ADD, more);
+    };
+    switch (a.reduce.mode) {
+      case TC_FOLD_SUM: IT_TRY(fold.template operator()<TC_FOLD_SUM>()); break;
+      case TC_FOLD_WSUM: IT_TRY(fold.template operator()<TC_FOLD_WSUM>()); break;
+      case TC_FOLD_MAX: IT_TRY(fold.template operator()<TC_FOLD_MAX>()); break;
+      case TC_FOLD_MIN: IT_TRY(fold.template operator()<TC_FOLD_MIN>()); break;
+      case TC_FOLD_PMAX: IT_TRY(fold.template operator()<TC_FOLD_PMAX>()); break;
+      case TC_FOLD_PMIN: IT_TRY(fold.template operator()<TC_FOLD_PMIN>()); break;
+      default: IT_TRY(fold.template operator()<TC_FOLD_STORE>()); break;
+    }
+  }
+  else IT_TRY(cols.stream ? go(gemm_tc_kernel<false, 0, true, 0, false>, TC_THREADS_BF16, 0.0) : go(gemm_tc_kernel<false, 0, false, 0, false>, TC_THREADS_BF16, 0.0));
   IT_CUDA_TRY(cudaGetLastError());
   return IT_OK;
 }

@@ -278,12 +278,12 @@ struct it_tc_reduce {
   int indptr64;
   int64_t n;                     // vertices
   const int32_t *tile_first;     // [tiles] the vertex that edge IT_MSG_TILE * t belongs to
-  const int32_t *ends;           // [tiles * IT_MSG_TILE] the vertex whose last edge this is, or -1
+  const int32_t *ends;           // [tiles * IT_MSG_TILE] the vertex whose last edge this is, or -1 (mode 6: NULL)
   float *partial;                // [tiles][2][dim]: what a vertex that crosses tiles has in a tile where it does not begin / does begin
   const float *weights;          // of the edges, or NULL
   void *dst;                     // bf16 rows: the reduce of every vertex
   int dst_ld, dim;
-  int mode, is_mean;             // 0 sum, 1 weighted sum, 2 max, 3 min
+  int mode, is_mean;             // 0 sum, 1 weighted sum, 2 max, 3 min, 4 / 5 the same unweighted; 6: not reduced, row m of dst is edge m's
 };
 struct it_gemm_args {
   int64_t M;

@@ -220,10 +220,11 @@ __global__ void __launch_bounds__(MSG_JOIN_THREADS, 1) message_combine_kernel(it
   __shared__ int n_todo;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = lane * 4;
-  const float id = q.mode == 2 ? -INFINITY : (q.mode == 3 ? INFINITY : 0.f);
+  const bool is_max = q.mode == 2 || q.mode == 4, is_min = q.mode == 3 || q.mode == 5;
+  const float id = is_max ? -INFINITY : (is_min ? INFINITY : 0.f);
   auto fold = [&](float4 &a, const float4 &y) {
-    if (q.mode == 2) { a.x = fmaxf(a.x, y.x); a.y = fmaxf(a.y, y.y); a.z = fmaxf(a.z, y.z); a.w = fmaxf(a.w, y.w); }
-    else if (q.mode == 3) { a.x = fminf(a.x, y.x); a.y = fminf(a.y, y.y); a.z = fminf(a.z, y.z); a.w = fminf(a.w, y.w); }
+    if (is_max) { a.x = fmaxf(a.x, y.x); a.y = fmaxf(a.y, y.y); a.z = fmaxf(a.z, y.z); a.w = fmaxf(a.w, y.w); }
+    else if (is_min) { a.x = fminf(a.x, y.x); a.y = fminf(a.y, y.y); a.z = fminf(a.z, y.z); a.w = fminf(a.w, y.w); }
     else { a.x += y.x; a.y += y.y; a.z += y.z; a.w += y.w; }
   };
   // the parts of the vertex that begins in tile b - 1: part 0 lies there, part k in tile b - 1 + k

@@ -52,7 +52,7 @@ def test_messages_finished_in_the_product(fm, act):
 
 
 # in-degrees whose sums put the ends of vertices at, before and after the 128-edge tiles of the per-edge product, vertices of several
-# tiles and of so many that a block folds their parts, runs of vertices without edges longer than a tile, a last tile of few edges
+# tiles and of so many that a block folds their parts, runs of vertices without edges longer than a tile
 TILE_DEGREES = {
     "one edge": [0, 1, 0],
     "one tile": [0, 100, 28],
@@ -63,22 +63,39 @@ TILE_DEGREES = {
 }
 
 
-@pytest.mark.parametrize("op,weights", [("sum", False), ("sum", True), ("mean", False), ("mean", True), ("max", False), ("min", True), ("gcn", True)])
-@pytest.mark.parametrize("degrees", TILE_DEGREES)
-@pytest.mark.parametrize("fm", [40, 128])
-def test_messages_reduced_by_their_product(op, weights, degrees, fm):
-    """bf16 messages are reduced tile by tile where they are made (oracle and tolerance of the other message tests: a sum in another
-    order differs in fp32 only)."""
-    layer = make_msg_layer(13, op, "none", 16, fm, 24, "bf16", act_edge="relu", weights=weights, edge_dim=8)
-    deg = np.asarray(TILE_DEGREES[degrees])
-    base = small_workload(14, len(deg), 1, "bf16", [layer], weights=True, edge_dim=8)
-    rng = np.random.default_rng(15)
+def tile_workload(deg, layer, seed):
+    deg = np.asarray(deg)
+    base = small_workload(seed, len(deg), 0, "bf16", [layer])
+    rng = np.random.default_rng(seed)
     e = int(deg.sum())
-    ef = wrng.f32_to_bf16_bits(rng.standard_normal((e, 8)).astype(np.float32))
-    w = Workload("tiles", len(deg), e, np.concatenate(([0], np.cumsum(deg))), rng.integers(0, len(deg), e).astype(np.int32),
-                 rng.random(e, dtype=np.float32), "bf16", base.x, [layer], 0, ef)
-    got, d = run_device(w)
-    check_against_oracle(w, got, label=(op, weights, degrees, fm))
+    ef = wrng.f32_to_bf16_bits(rng.standard_normal((e, layer.edge_dim)).astype(np.float32))
+    return Workload("tiles", len(deg), e, np.concatenate(([0], np.cumsum(deg))), rng.integers(0, len(deg), e).astype(np.int32),
+                    rng.random(e, dtype=np.float32), "bf16", base.x, [layer], 0, ef)
+
+
+@pytest.mark.parametrize("degrees", TILE_DEGREES)
+@pytest.mark.parametrize("fm,weights", [(40, False), (128, True)])
+def test_messages_written_by_their_product(degrees, fm, weights):
+    """Few edges: tiles of finished messages are written, the last one in part (oracle and tolerance of the other message tests)."""
+    layer = make_msg_layer(13, "sum", "none", 16, fm, 24, "bf16", act_edge="relu", weights=weights, edge_dim=8)
+    w = tile_workload(TILE_DEGREES[degrees], layer, 14)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(degrees, fm))
+
+
+@pytest.mark.parametrize("op,weights,fm,tail", [("sum", False, 64, 0), ("sum", True, 24, 1), ("mean", False, 24, 127), ("mean", True, 120, 64), ("max", False, 64, 1),
+                                                ("min", True, 64, 0), ("max", False, 120, 5), ("gcn", True, 120, 127), ("min", False, 24, 0), ("max", True, 24, 3)])
+def test_messages_reduced_by_their_product(op, weights, fm, tail):
+    """Many edges: messages are reduced tile by tile where they are made; every pattern of ends of vertices, a last tile of `tail` edges
+    (0: a whole one).  Oracle and tolerance of the other message tests: a sum in another order differs in fp32 only."""
+    layer = make_msg_layer(15, op, "none", 16, fm, 24, "bf16", act_edge="elu" if op == "sum" else "relu", weights=weights, edge_dim=8)
+    bulk = np.random.default_rng(16).integers(0, 48, 58_000)
+    deg = [d for p in TILE_DEGREES.values() for d in p] + bulk.tolist()
+    deg.append((tail - sum(deg)) % 128)
+    assert sum(deg) % 128 == tail and sum(deg) > 5 << 18
+    w = tile_workload(deg, layer, 17)
+    got, _ = run_device(w)
+    check_against_oracle(w, got, label=(op, weights, fm, tail))
     again, _ = run_device(w, int32_indptr=True)
     assert np.array_equal(got, again)
 
