@@ -499,7 +499,7 @@ it_status launch_gat_small(const it_gat_args &a, StreamParams p, const GatPolicy
   if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(it_done_words(a.counters), 0, (size_t)g->n_long * sizeof(int), st));
   const double row_bytes = (double)pol.dim * sizeof(T);
   const double bytes = (double)g->e * (4.0 + 4.0 * H + row_bytes) + (double)g->n * (20.0 + 4.0 * H + row_bytes);
-  const SmallShare sh = small_share(g, LPR);
+  const SmallShare sh = small_share(g, LPR, true, a.per_edge_scores ? 5 : 8);   // (logit terms in edge order come cheaper: 20k vertices / 300k edges 43 us, with 8 47)
   const int smem = sh.short_blocks ? 2 * IT_SHORT_EDGES * THREADS * 16 : 0;
   static std::atomic<uint64_t> configured{0};
   IT_TRY(allow_dynamic_smem(gat_small_kernel<T, LPR, H>, 2 * IT_SHORT_EDGES * THREADS * 16, configured));

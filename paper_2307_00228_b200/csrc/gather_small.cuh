@@ -51,16 +51,17 @@ struct SmallShare {
   unsigned blocks;
   int short_blocks, short_lo, short_hi, total;
 };
-inline SmallShare small_share(const it_graph *g, int lpr) {
+// groups: lane groups take rows with edges too (else only those without); row: what a lane group's row costs, in edges.
+inline SmallShare small_share(const it_graph *g, int lpr, bool groups, int row) {
   SmallShare s;
   s.total = (int)g->h_list_offsets[g->n_lists];
   int64_t short_cost = 0, cost = 0;
   s.short_lo = s.short_hi = 0;
   for (int b = 0; b < g->n_lists; ++b) {
     const int64_t rows = g->h_list_offsets[b + 1] - g->h_list_offsets[b], edges = g->h_list_edges[b];
-    if (g->list_bounds[b] <= IT_SHORT_BELOW && b != g->n_lists - 1) {
+    if (b == 0 || (groups && g->list_bounds[b] <= IT_SHORT_BELOW && b != g->n_lists - 1)) {
       s.short_hi = (int)g->h_list_offsets[b + 1];
-      short_cost += (b == 0 ? rows * 4 : rows * 8 + edges) * lpr / 16;
+      short_cost += (b == 0 ? rows * row / 2 : rows * row + edges) * lpr / 16;
     } else {
       cost += rows * 16 + edges * 2 * lpr / 16;
     }
