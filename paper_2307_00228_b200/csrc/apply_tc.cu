@@ -230,12 +230,9 @@ struct TcParams {
 // end in its rows, a column pair per lane; a vertex that crosses tiles leaves one fp32 row per tile for it_launch_message_combine.
 // ADD: warps of an epilogue group, four (four tiles at a time) for up to 64 columns, else eight.
 // Bound by issue slots and the latency of an epilogue warp's tile (16 of these warps, 5100 warp instructions per tile of 128 x 64, 2.2
-// per clock and SM; without the reduce the kernel takes 0.75 ms instead of 1.05).  Written out and reduced by the gather instead, the
-// message rows cost 4 GB of traffic: 1M vertices, 16M edges, 32 features, 64 columns, whole layer 1.60 against 1.26 ms.  Eight warps of
+// per clock and SM; without the reduce the kernel takes 0.75 ms instead of 1.1).  Written out and reduced by the gather instead, the
+// message rows cost 4 GB of traffic: 1M vertices, 16M edges, 32 features, 64 columns, whole layer 1.58 against 1.33 ms.  Eight warps of
 // their own for the reduce, which leave 64 registers a thread: 1.57.
-#ifndef IT_TC_NARROW
-#define IT_TC_NARROW 1
-#endif
 constexpr int TC_ADD_STAGES_MAX = 8;
 constexpr int TC_THREADS_ADD = TC_THREADS_BF16 + 128;
 static_assert(IT_MSG_TILE == TC_BM, "a tile of edges is a tile of rows");
@@ -286,7 +283,8 @@ __device__ __forceinline__ uint32_t lds_b32(uint32_t at) {
 
 // The reduce of one tile by the warps of its group.  tile_s: the tile (128-byte swizzled panels); seg: the vertex that ends at every row
 // (or -1), then the rows' weights; cut_before: the tile's first edge is not the first of its vertex; has_next: another tile follows.
-// Eight rows at a time, whose places are known but for the first one's; rows of up to 32 columns (NARROW) by half a warp each.
+// Eight rows at a time, whose places are known but for the first one's; rows of up to 32 columns (NARROW) by half a warp each
+// (300k vertices / 5M edges, 32 columns: 381 us, by whole warps 408).
 template <int MODE, int WARPS, bool NARROW>
 __device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *seg, bool cut_before, bool has_next, int64_t tile, int gw, int lane,
                                                const it_tc_reduce &q, int nbc) {
@@ -1628,7 +1626,7 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
     auto fold = [&]<int MODE>() -> it_status {
       const double more = (double)a.M * 4.0;
       if (tc_add_warps(nbc) == 8) return go(gemm_tc_kernel<false, 8, false, MODE, false>, TC_THREADS_ADD, more);
-      if (IT_TC_NARROW && nbc <= 32 && MODE != TC_FOLD_STORE) return go(gemm_tc_kernel<false, 4, false, MODE, true>, TC_THREADS_ADD, more);
+      if (nbc <= 32 && MODE != TC_FOLD_STORE) return go(gemm_tc_kernel<false, 4, false, MODE, true>, TC_THREADS_ADD, more);
       return go(gemm_tc_kernel<false, 4, false, MODE, false>, TC_THREADS_ADD, more);
     };
     switch (a.reduce.mode) {
