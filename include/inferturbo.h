@@ -355,6 +355,9 @@ it_status it_debug_expire_wait(it_graph *g, it_dtype dtype, const void *x, void 
 /* The same hook for the kernel that it_infer uses where the update of one layer and the transform of the next run as one
  * (two products back to back, bf16): x and out are device [128, 64] bf16. */
 it_status it_debug_expire_wait_fused(it_graph *g, const void *x, void *out, void *workspace, size_t workspace_bytes, void *stream);
+/* And for the other forms of the product: 0, 1 messages reduced by four and by eight warps a tile, 2 messages written, 3 bf16 and
+ * 4 fp32 weights streamed beside the operand, 5 fp32 with one accumulator.  buffer: device, 256-byte aligned, at least 32 MB of zeros. */
+it_status it_debug_expire_wait_form(it_graph *g, int form, void *buffer, size_t bytes, void *stream);
 
 /* Frees the library-owned arrays of the graph.  NULL is accepted. */
 it_status it_graph_destroy(it_graph *g);

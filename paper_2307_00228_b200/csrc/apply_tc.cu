@@ -93,6 +93,43 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
   *abort_flag = 1;
   return false;
 }
+// Before a CTA may leave, what it set off has to be over, also where a role gave up a wait: copies would still write its shared memory,
+// and MMAs read it and write its TMEM, when both belong to another CTA.  A barrier's wait for one parity is always true (that of the
+// phase before the present one), so it has to be the parity of the phase that was armed last.  Bounded, and apart from the abort flag.
+__device__ __forceinline__ void mbar_drain(uint64_t *bar, uint32_t parity) {
+  for (uint32_t it = 0; it < TC_SPIN_LIMIT; ++it)
+    if (mbar_try_wait(bar, parity)) return;
+}
+// A ring whose position (`next`, `phase`: the stage and parity that the next copy would have) has come round from (0, 0): whether stage
+// s was armed at all, and the parity of its last time.
+struct RingStage { bool armed; uint32_t parity; };
+__host__ __device__ constexpr RingStage ring_last(uint32_t s, uint32_t next, uint32_t phase, bool came_round) {
+  return s < next ? RingStage{true, phase} : RingStage{came_round, phase ^ 1u};
+}
+constexpr bool ring_last_holds() {   // against every copy made in turn
+  for (uint32_t stages = 1; stages <= IT_TC_MAX_STAGES; ++stages)
+    for (uint32_t copies = 0; copies <= 3 * stages + 1; ++copies) {
+      uint32_t next = 0, phase = 0, parity[IT_TC_MAX_STAGES] = {};
+      bool armed[IT_TC_MAX_STAGES] = {}, came_round = false;
+      for (uint32_t i = 0; i < copies; ++i) {
+        armed[next] = true;
+        parity[next] = phase;
+        if (++next == stages) { next = 0; phase ^= 1u; came_round = true; }
+      }
+      for (uint32_t s = 0; s < stages; ++s) {
+        const RingStage r = ring_last(s, next, phase, came_round);
+        if (r.armed != armed[s] || (r.armed && r.parity != parity[s])) return false;
+      }
+    }
+  return true;
+}
+static_assert(ring_last_holds(), "the last copy into every stage of a ring");
+__device__ __forceinline__ void ring_drain(uint64_t *full, uint32_t stages, uint32_t next, uint32_t phase, bool came_round) {
+  for (uint32_t s = 0; s < stages; ++s) {
+    const RingStage r = ring_last(s, next, phase, came_round);
+    if (r.armed) mbar_drain(&full[s], r.parity);
+  }
+}
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int c0, int c1, uint64_t *bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
@@ -403,7 +440,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
   const int add_stages = ADD ? p.add_stages : 0;
   uint64_t *add_full = acc_empty + NACC;        // [add_stages]  (ADD) the tile's rows and the ends of its vertices have landed
   uint64_t *add_empty = add_full + add_stages;  // [add_stages]  (ADD) the tile is reduced
-  int32_t *seg_s = reinterpret_cast<int32_t *>(add_empty + add_stages);   // [add_stages][TC_SEG_WORDS]  (ADD)
+  uint64_t *mma_done = add_empty + add_stages;  // [1]  every MMA of the CTA is over
+  int32_t *seg_s = reinterpret_cast<int32_t *>(mma_done + 1);   // [add_stages][TC_SEG_WORDS]  (ADD)
   int32_t *ids_s = seg_s + add_stages * TC_SEG_WORDS;   // [TC_IDS_AHEAD][TC_BM]  (ADD) source ids
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(ids_s + (ADD ? TC_IDS_AHEAD * TC_BM : 0));
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
@@ -427,6 +465,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       mbar_init(&a_free[s], 1);
     }
     mbar_init(b_full, 1);
+    mbar_init(mma_done, 1);
     if (ADD)
       for (int a = 0; a < add_stages; ++a) {
         mbar_init(&add_full[a], 128);
@@ -475,7 +514,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
             tma_load_2d(smem_b + (size_t)(kb * parts + part) * b_tile_bytes, &map_b, kb * bk_elems, part * p.NB + col_base, b_full);
       }
       uint32_t stage = 0, phase = 0;
-      bool ok = true;
+      bool ok = true, came_round = false;
       for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
         const int m0 = (tile / p.n_splits) * TC_BM;
         for (int kb = 0; kb < KB; ++kb) {
@@ -488,15 +527,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           if (STREAM)
             for (int part = 0; part < parts; ++part)
               tma_load_2d(to + a_tile_bytes + part * b_tile_bytes, &map_b, kb * bk_elems, part * p.NB + col_base, &full[stage]);
-          if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
+          if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; came_round = true; }
         }
       }
-      if (!ok) {
-        // aborting: give the copies that were issued time to land before the CTA may exit (bounded)
-        for (int s = 0; s < p.stages; ++s)
-          for (uint32_t it = 0; it < TC_SPIN_LIMIT; ++it)
-            if (mbar_try_wait(&full[s], 0) || mbar_try_wait(&full[s], 1)) break;
-      }
+      if (!STREAM) mbar_drain(b_full, 0);
+      ring_drain(full, (uint32_t)p.stages, stage, phase, came_round);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -549,6 +584,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
         tc_commit(&acc_full[acc]);    // accumulator complete
         if (++acc == (uint32_t)NACC) { acc = 0; acc_phase ^= 1u; }
       }
+      tc_commit(mma_done);
+      mbar_drain(mma_done, 0);
     }
   } else if (warp < 2 + TC_EPI_WARPS) {
     // ------------------------------------------------------------------ epilogue
@@ -1159,7 +1196,8 @@ gemm2_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constan
   uint64_t *h_full = acc1_empty + 2;        // [2]  H tile of the group written to shared memory
   uint64_t *acc2_full = h_full + 2;         // [2]  second product complete (and H read)
   uint64_t *acc2_empty = acc2_full + 2;     // [2]
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc2_empty + 2);
+  uint64_t *mma_done = acc2_empty + 2;      // [1]  every MMA of the CTA is over
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mma_done + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   float *cst1 = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(tmem_slot + 2) + 15) & ~(uintptr_t)15);   // [N1] bias of H
   float *cst2 = cst1 + p.N1;                                                                                     // [N2] bias0 | 0
@@ -1173,6 +1211,7 @@ gemm2_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constan
       mbar_init(&empty[s], 1);
     }
     mbar_init(b_full, 1);
+    mbar_init(mma_done, 1);
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc1_full[a], 1);
       mbar_init(&acc1_empty[a], TC2_GROUP_WARPS);
@@ -1204,7 +1243,7 @@ gemm2_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constan
       for (int kb = 0; kb < KB1; ++kb) tma_load_2d(smem_b1 + (size_t)kb * b1_tile_bytes, &map_b1, kb * 64, 0, b_full);
       for (int kb = 0; kb < KB2; ++kb) tma_load_2d(smem_b2 + (size_t)kb * b2_tile_bytes, &map_b2, kb * 64, 0, b_full);
       uint32_t stage = 0, phase = 0;
-      bool ok = true;
+      bool ok = true, came_round = false;
       for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
         const int m0 = tile * TC_BM;
         for (int kb = 0; kb < KB1; ++kb) {
@@ -1213,15 +1252,11 @@ gemm2_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constan
           mbar_arrive_expect_tx(&full[stage], (uint32_t)a_tile_bytes);
           if (kb < p.kb1) tma_load_2d(smem_a + (size_t)stage * a_tile_bytes, &map_x1, kb * 64, m0, &full[stage]);
           else tma_load_2d(smem_a + (size_t)stage * a_tile_bytes, &map_x2, (kb - p.kb1) * 64, m0, &full[stage]);
-          if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
+          if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; came_round = true; }
         }
       }
-      if (!ok) {
-        // aborting: give the copies that were issued time to land before the CTA may exit (bounded)
-        for (int s = 0; s < p.stages; ++s)
-          for (uint32_t it = 0; it < TC_SPIN_LIMIT; ++it)
-            if (mbar_try_wait(&full[s], 0) || mbar_try_wait(&full[s], 1)) break;
-      }
+      mbar_drain(b_full, 0);
+      ring_drain(full, (uint32_t)p.stages, stage, phase, came_round);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -1272,6 +1307,8 @@ gemm2_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constan
         if (it > 0) ok = second(it - 1);
       }
       if (ok && it > 0) second(it - 1);
+      tc_commit(mma_done);
+      mbar_drain(mma_done, 0);
     }
   } else {
     // ------------------------------------------------------------------ epilogue: group g takes the tiles it % 2 == g
@@ -1736,4 +1773,31 @@ extern "C" it_status it_debug_expire_wait_fused(it_graph *g, const void *x, void
   a.n0 = 0; a.out0 = nullptr; a.bias0 = nullptr; a.n1 = 64; a.out1 = out;
   a.spin_limit = 4096; a.no_loads = 1;
   return it_launch_gemm2_tc(a, workspace, (const char *)workspace + 32 * 1024, g->num_sms, g->d_status, (cudaStream_t)stream);
+}
+
+// The same hook for the other forms of the product, which give up in other places: every pointer is the one zeroed buffer, of which nothing
+// is written (no accumulator is ever complete).
+extern "C" it_status it_debug_expire_wait_form(it_graph *g, int form, void *buffer, size_t bytes, void *stream) {
+  IT_REQUIRE(g != nullptr && buffer != nullptr && form >= 0 && form < 6, IT_ERR_INVALID_ARG, "NULL argument or unknown form");
+  IT_REQUIRE(bytes >= ((size_t)32 << 20) && ((uintptr_t)buffer % 256) == 0, IT_ERR_WORKSPACE, "needs 32 MB of aligned memory");
+  it_gemm_args a{};
+  a.x_dtype = form == 4 || form == 5 ? IT_F32 : IT_BF16;
+  a.dt0 = a.dt1 = a.x_dtype;
+  a.X1 = buffer; a.out0 = buffer; a.act0 = IT_ACT_NONE;
+  a.spin_limit = 4096; a.no_loads = 1;
+  if (form < 3) {   // 0, 1: rows added and reduced by four and by eight warps a tile; 2: written.  More tiles per CTA than the ring has stages
+    a.M = (int64_t)g->num_sms * (TC_ADD_STAGES_MAX + 2) * TC_BM; a.K1 = 16; a.n0 = form == 1 ? 128 : 64;
+    a.out0 = nullptr; a.add_rows = buffer; a.add_idx = (const int32_t *)buffer;
+    a.reduce.mode = form == 2 ? TC_FOLD_STORE : TC_FOLD_SUM;
+    a.reduce.n = 1; a.reduce.partial = (float *)buffer; a.reduce.dst = buffer; a.reduce.dst_ld = a.reduce.dim = a.n0;
+    if (form < 2) a.reduce.ends = a.reduce.tile_first = (const int32_t *)buffer;
+  } else if (form < 5) {   // 3, 4: streamed weights, more tiles than stages
+    a.M = 128; a.K1 = 1024; a.n0 = form == 4 ? 256 : 512;
+  } else {   // 5: fp32 with one accumulator
+    a.M = (int64_t)IT_NUM_SMS_FALLBACK * 2 * TC_BM; a.K1 = 64; a.n0 = 128;
+  }
+  it_tc_cols cols;
+  IT_REQUIRE(it_tc_columns(a, a.n0, false, &cols) && (form < 3 ? cols.n_splits == 1 && !cols.stream : (form < 5 ? cols.stream != 0 : cols.nbc > 64)),
+             IT_ERR_UNSUPPORTED, "the product no longer takes this form");
+  return it_launch_gemm_tc(a, buffer, nullptr, nullptr, 1, a.n0, nullptr, g->num_sms, g->d_status, (cudaStream_t)stream);
 }

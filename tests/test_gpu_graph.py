@@ -215,3 +215,23 @@ def test_a_wait_that_runs_out_is_reported_and_the_library_goes_on(tdtype):
     B.it_graph_check(d.graph)
     from gpu_util import to_numpy
     check_against_oracle(w, to_numpy(d.out))
+
+
+@pytest.mark.parametrize("form", range(6))
+def test_every_form_of_the_product_gives_up_by_itself(form):
+    """Messages reduced by four and by eight warps a tile and written, streamed weights of both types, one fp32 accumulator: each has roles
+    and barriers of its own, and each must return and be reported."""
+    from gpu_util import check_against_oracle, make_msg_layer, run_device, small_workload, to_numpy
+    layer = make_msg_layer(3, "sum", "none", 16, 64, 24, "bf16", act_edge="relu", edge_dim=16)
+    w = small_workload(4, 600, 12, "bf16", [layer], edge_dim=16)
+    _, d = run_device(w)
+    buf = torch.zeros(32 << 20, dtype=torch.uint8, device="cuda")
+    B.it_debug_expire_wait_form(d.graph, form, buf)
+    with pytest.raises(B.ItError) as e:
+        B.it_graph_check(d.graph)
+    assert e.value.status_name == "IT_ERR_TIMEOUT"
+    assert int(torch.count_nonzero(buf)) == 0
+    B.it_graph_check(d.graph)          # reported once
+    d.infer()
+    B.it_graph_check(d.graph)
+    check_against_oracle(w, to_numpy(d.out))
