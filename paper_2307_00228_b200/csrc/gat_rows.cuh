@@ -265,8 +265,7 @@ __global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_k
 #define IT_GAT_SHORT_BLOCKS 3   // resident CTAs per SM: 64 KB of staging each
 #endif
 // block / blocks: which share of the rows p.row_lo .. p.row_hi this block walks; short_buf: [2][E][THREADS] in shared memory.
-// EMPTY: rows without edges are among them.
-template <typename T, int LPR, int H, bool EMPTY = false>
+template <typename T, int LPR, int H>
 __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatParams &q, const GatPolicy<T, 16> &pol, int block, int blocks, uint4 *short_buf) {
   using Acc = GatAcc<T>;
   constexpr int E = LPR < IT_SHORT_EDGES ? LPR : IT_SHORT_EDGES;
@@ -281,11 +280,10 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
   constexpr uint32_t SLOT = THREADS * 16, BUF = E * SLOT;
   uint32_t buf = (uint32_t)__cvta_generic_to_shared(short_buf + threadIdx.x), other = buf + BUF;
   const int64_t sweep = (int64_t)blocks * (THREADS / LPR);
-  constexpr int NONE = EMPTY ? -1 : 0;   // length of a missing row
 
-  struct Row { int64_t j0; int len, most, dest, owner; float sd; };   // most: longest row of the warp's groups (NONE: no rows left)
+  struct Row { int64_t j0; int len, most, dest, owner; float sd; };   // most: longest row of the warp's groups (0: no rows left)
   auto load_row = [&](int64_t i0, Row &r) {
-    r.j0 = 0; r.len = NONE; r.dest = 0; r.owner = 0;
+    r.j0 = 0; r.len = 0; r.dest = 0; r.owner = 0;
     const int64_t i = i0 + lane / LPR;
     if (i < p.row_hi) {
       const it_row_meta m = load_meta(p.meta + i);
@@ -295,7 +293,6 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
   };
   auto finish_row = [&](Row &r) {   // the record has landed: what hangs on it
     r.most = __reduce_max_sync(0xffffffffu, r.len);
-    if (EMPTY && r.most == 0) r.most = 1;   // only rows without edges: a round in any case, which fetches what follows
     r.sd = __ldg(q.scores_dst + (int64_t)r.owner * (2 * H) + H + hl);   // owner 0 for a missing row: read, not used
   };
   auto load_ids = [&](const Row &r, int k) -> int32_t {
@@ -324,7 +321,7 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
   Row r0, r1, r2;
   load_row(i0, r0); load_row(i0 + sweep, r1); load_row(i0 + 2 * sweep, r2);
   finish_row(r0);
-  if (r0.most == NONE) return;   // warp-uniform
+  if (r0.most == 0) return;   // warp-uniform
   finish_row(r1);
   float x_a[PP], x_b[PP];
   int32_t idx_b = load_ids(r0, 0);
@@ -332,7 +329,7 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
   idx_b = r0.most > E ? load_ids(r0, E) : load_ids(r1, 0);
   Acc acc;
   float st[Acc::NS];
-  for (; r0.most > NONE; i0 += sweep) {
+  for (; r0.most > 0; i0 += sweep) {
     Row r3;
     load_row(i0 + 3 * sweep, r3);
     finish_row(r2);
@@ -356,9 +353,8 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
       for (int o = H; o < LPR; o <<= 1) mr = fmaxf(mr, __shfl_xor_sync(0xffffffffu, mr, o));
       const float m_new = fmaxf(m, mr);
       if (k0 > 0) {   // rows whose edges are used up: m_new = m, a factor of 1
-        float s = it_exp(m - m_new);
-        if (EMPTY && m_new == -INFINITY) s = 1.f;   // (a row without edges: nothing to rescale)
-        acc.scale(st, __shfl_sync(0xffffffffu, s, gbase + hc));
+        const float s = __shfl_sync(0xffffffffu, it_exp(m - m_new), gbase + hc);
+        acc.scale(st, s);
       }
       m = m_new;
 #pragma unroll
@@ -376,7 +372,7 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
       const uint32_t sw = buf; buf = other; other = sw;
     }
     const float mh = __shfl_sync(0xffffffffu, m, gbase + hc);
-    if (r0.len > NONE) {
+    if (r0.len > 0) {
       float full[GatPolicy<T, 16>::NS];
 #pragma unroll
       for (int k = 0; k < Acc::VEC; ++k) full[k] = st[k];
@@ -411,7 +407,19 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(Stream
   stage_bias(pol, bias_buf);
   if ((int)blockIdx.x < sh.short_blocks) {
     p.row_lo = sh.short_lo; p.row_hi = sh.short_hi;
-    gat_short_rows<T, LPR, H, true>(p, q, pol, blockIdx.x, sh.short_blocks, short_buf);
+    gat_short_rows<T, LPR, H>(p, q, pol, blockIdx.x, sh.short_blocks, short_buf);
+    return;
+  }
+  if ((int)blockIdx.x < sh.short_blocks + sh.empty_blocks) {
+    float none[NS];
+    pol.init(none);
+    small_empties(sh, [&](int b, int n) {
+      const int dest = lane < n ? __ldcs(&p.meta[b + lane].dest) : 0;
+      for (int k = 0; k < n; k += SL) {
+        const int d = __shfl_sync(0xffffffffu, dest, (k + slot) & 31);
+        if (k + slot < n) pol.end_row(none, d, 0, 0);
+      }
+    });
     return;
   }
   GatSmallWarp<T, LPR, H> gw(p, q, lane, (uint32_t)__cvta_generic_to_shared(&weights[threadIdx.x >> 5][0]));

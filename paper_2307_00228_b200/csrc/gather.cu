@@ -136,86 +136,14 @@ __global__ void __launch_bounds__(GATHER_THREADS) combine_kernel(CombineParams p
 }
 
 // ----------------------------------------------------------------------------- rows without edges
-// A warp takes 32 rows (their destinations with one coalesced load) and writes them 16 bytes per lane, four pieces in
-// flight; a value that is the same for every row is built once per block in shared memory.  Bound by the writes (and the
-// self terms): per-row kernels waited for each row's record, then its self term, before the row's store (5.3M raw 256-byte
-// rows: 340 -> 255 us; 615k GAT rows of 256 bytes: 82 -> 22; two layers of 8M rows of 128 bytes, one with self terms: 851 -> 638).
-struct EmptyRowsParams {
-  const it_row_meta *__restrict__ meta;
-  int64_t lo, hi;
-  char *dst;
-  const char *self;
-  int64_t pitch, self_pitch;
-  int kind, slices, dim, bf16, act;   // slices: 16-byte pieces of a row
-  float value;
-  const float *__restrict__ bias;
-};
-
-__device__ __forceinline__ uint4 pack_piece(const float (&v)[8], int bf16) {
-  if (!bf16) return make_uint4(__float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
-  uint32_t w[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
-    w[k] = *reinterpret_cast<uint32_t *>(&h);
-  }
-  return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 __global__ void __launch_bounds__(GATHER_THREADS) empty_rows_kernel(EmptyRowsParams p) {
   __shared__ uint4 row[128];   // rows of up to 512 entries
   if (p.kind != IT_EMPTY_SELF) {
-    for (int s = threadIdx.x; s < p.slices; s += GATHER_THREADS) {
-      const int per = p.bf16 ? 8 : 4;
-      float v[8];
-      for (int k = 0; k < 8; ++k) v[k] = p.kind == IT_EMPTY_BIAS ? act_apply(p.bias && k < per ? p.bias[s * per + k] : 0.f, p.act) : p.value;
-      row[s] = pack_piece(v, p.bf16);
-    }
+    for (int s = threadIdx.x; s < p.slices; s += GATHER_THREADS) row[s] = empty_piece(p, s);
     __syncthreads();
   }
-  const int lane = threadIdx.x & 31;
-  const int step_r = 32 / p.slices, step_s = 32 % p.slices;
-  for (int64_t b = p.lo + ((int64_t)blockIdx.x * (GATHER_THREADS / 32) + (threadIdx.x >> 5)) * 32; b < p.hi;
-       b += (int64_t)gridDim.x * GATHER_THREADS) {
-    const int n = (int)(p.hi - b < 32 ? p.hi - b : 32);
-    int dest = 0;
-    if (lane < n) dest = __ldcs(&p.meta[b + lane].dest);
-    int r = lane / p.slices, s = lane % p.slices;
-    for (int k = 0; k < p.slices; k += 4) {   // 32 rows x slices pieces, 32 at a time, four of those in flight
-      uint4 x[4];
-      int64_t at[4];
-      int sl[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int d = __shfl_sync(0xffffffffu, dest, r & 31);
-        sl[u] = s;
-        at[u] = r < n && k + u < p.slices ? (int64_t)d : -1;
-        if (at[u] >= 0) x[u] = p.kind == IT_EMPTY_SELF ? __ldcs(reinterpret_cast<const uint4 *>(p.self + at[u] * p.self_pitch) + s) : row[s];
-        r += step_r; s += step_s;
-        if (s >= p.slices) { s -= p.slices; ++r; }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (at[u] < 0) continue;
-        if (p.kind == IT_EMPTY_SELF && p.act != IT_ACT_NONE) {
-          float v[8];
-          const uint32_t w[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (p.bf16) {
-              v[2 * q] = act_apply(__uint_as_float(w[q] << 16), p.act);
-              v[2 * q + 1] = act_apply(__uint_as_float(w[q] & 0xffff0000u), p.act);
-            } else {
-              v[q] = act_apply(__uint_as_float(w[q]), p.act);
-              v[4 + q] = 0.f;
-            }
-          }
-          x[u] = pack_piece(v, p.bf16);
-        }
-        __stcs(reinterpret_cast<uint4 *>(p.dst + at[u] * p.pitch) + sl[u], x[u]);
-      }
-    }
-  }
+  for (int64_t b = p.lo + ((int64_t)blockIdx.x * (GATHER_THREADS / 32) + (threadIdx.x >> 5)) * 32; b < p.hi; b += (int64_t)gridDim.x * GATHER_THREADS)
+    empty_rows_warp(p, b, (int)(p.hi - b < 32 ? p.hi - b : 32), threadIdx.x & 31, [&](int s) { return row[s]; });
 }
 
 }  // namespace
@@ -223,7 +151,7 @@ __global__ void __launch_bounds__(GATHER_THREADS) empty_rows_kernel(EmptyRowsPar
 it_status it_launch_empty_rows(const it_empty_rows_args &a, int kid, double bytes, cudaStream_t st) {
   const it_graph *g = a.g;
   EmptyRowsParams p;
-  p.meta = g->list_meta; p.lo = a.row_lo; p.hi = a.row_hi; p.dst = (char *)a.dst; p.pitch = a.pitch; p.dim = a.dim;
+  p.meta = g->list_meta; p.lo = a.row_lo; p.hi = a.row_hi; p.dst = (char *)a.dst; p.pitch = a.pitch;
   p.self = (const char *)a.self; p.self_pitch = a.self_pitch; p.kind = (int)a.kind;
   p.slices = a.dim * it_dtype_size(a.dtype) / 16; p.bf16 = a.dtype == IT_BF16; p.act = (int)a.act;
   p.value = a.value; p.bias = a.bias;

@@ -28,7 +28,7 @@ struct SagePolicy {
   int col;
   float self[VEC];
 
-  void empty_rows(it_empty_rows_args &a) const {
+  __host__ __device__ void empty_rows(it_empty_rows_args &a) const {
     const bool raw = epi == IT_EPI_RAW_F32;
     a.kind = epi == IT_EPI_ADD_ACT ? IT_EMPTY_SELF : (epi == IT_EPI_BIAS_ACT ? IT_EMPTY_BIAS : IT_EMPTY_VALUE);
     a.dst = dst; a.dim = dim; a.dtype = raw || sizeof(T) == 4 ? IT_F32 : IT_BF16; a.pitch = (int64_t)dst_ld * (raw ? 4 : (int)sizeof(T));
@@ -166,7 +166,15 @@ __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gather_small_kernel(Str
   it_wait_prior();
   if ((int)blockIdx.x < sh.short_blocks) {
     p.row_lo = sh.short_lo; p.row_hi = sh.short_hi;
-    short_rows_pipe<T, LPRS, Policy, true, true>(p, pol, blockIdx.x, sh.short_blocks, small_stage);
+    if constexpr (LPR <= 16) short_rows_pipe<T, LPRS, Policy, true>(p, pol, blockIdx.x, sh.short_blocks, small_stage);
+    return;
+  }
+  if ((int)blockIdx.x < sh.short_blocks + sh.empty_blocks) {
+    it_empty_rows_args a;
+    pol.empty_rows(a);
+    const EmptyRowsParams er{p.meta, 0, sh.short_lo, (char *)a.dst, (const char *)a.self, a.pitch, a.self_pitch, (int)a.kind,
+                             a.dim * (a.dtype == IT_F32 ? 4 : 2) / 16, a.dtype == IT_BF16, (int)a.act, a.value, a.bias};
+    small_empties(sh, [&](int b, int n) { empty_rows_warp(er, b, n, lane, [&](int s) { return empty_piece(er, s); }); });
     return;
   }
   small_walk<true, false>(p, sh, lane, [&](const SmallRow &m, int32_t idx, float w) {

@@ -1,6 +1,6 @@
-// One kernel per layer for small graphs.  Some blocks walk the rows of at most 32 edges and those of none, a lane group per row, as
-// the kernel for short rows does; the others take the remaining rows, a warp per row (pieces of long
-// vertices, whole vertices), source rows straight into registers, and fold the pieces of a long vertex
+// One kernel per layer for small graphs.  Some blocks walk the rows of at most 32 edges, a lane group per row, as the kernel for short
+// rows does; some write the rows without edges, 32 of them per warp at a time; the others take the remaining rows, a warp per row
+// (pieces of long vertices, whole vertices), source rows straight into registers, and fold the pieces of a long vertex
 // in the warp that finishes the last of them.  The record of a warp's next-but-one row and the ids of its next row are in
 // flight while a row is reduced.
 // What bounds it: the dependent trips record -> ids -> source rows out of the L2 and the launch itself.  A layer of 10k
@@ -41,40 +41,58 @@ __device__ __forceinline__ bool last_piece(const PieceParams &q, int slot, int l
 
 constexpr int SMALL_BLOCKS = 3;   // resident CTAs per SM
 
-// How a launch is shared out: blocks [0, short_blocks) take entries [short_lo, short_hi) of the list, the others the rest, in
-// proportion to what they cost, since a launch is as long as its longer share.  A lane group's row costs about eight edges besides its
-// own, and a warp has 32 / lpr of them at a time; a warp's row about as much as sixteen, and the more steps the more lanes an edge
-// takes.  Rows without edges, which had a warp each, cost a lane group half a row.  Measured against twice / half of the lane groups'
-// share: attention, 30k vertices / 420k edges, 128-byte rows 63 us against 65 / 79; 30k / 400k, 512-byte rows 62 against 76 / 63; 100k /
-// 1.8M, 256-byte rows 127 against 143 / 147; GCN, 8k / 190k, 128- and 64-byte rows 33 against 34 / 38.
+// How a launch is shared out: the first blocks take entries [short_lo, short_hi) of the list, the next ones those before, the others
+// the rest, in proportion to what they cost, since a launch is as long as its longest share.  A lane group's row costs about eight
+// edges besides its own, and a warp has 32 / lpr of them at a time; a warp's row about as much as sixteen, and the more steps the more
+// lanes an edge takes.  Measured against twice / half of the lane groups' share: attention, 30k vertices / 420k edges, 128-byte rows
+// 63 us against 65 / 79; 30k / 400k, 512-byte rows 62 against 76 / 63; 100k / 1.8M, 256-byte rows 127 against 143 / 147; GCN, 8k / 190k,
+// 128- and 64-byte rows 33 against 34 / 38.
+// A row without edges costs about three (1, 2, 3, 4, 6, 9 of them: bf16 max over 768 columns, 100k vertices / 1.8M edges, power law, 2043,
+// 1051, 898, 881, 880, 895 us; fp32 max over 64, 76k / 0.94M 89, 68, 71, 71, 73, 73; attention, 30k / 420k, 84, 66, 66, 66, 66, 67).  By
+// lane groups or warps that take one at a time, each a trip to its record and one to its self term, the first of these took 1484 on
+// blocks of their own and 1070 among the rows of all warps.
 struct SmallShare {
   unsigned blocks;
-  int short_blocks, short_lo, short_hi, total;
+  int short_blocks, empty_blocks, short_lo, short_hi, total;   // (entries [0, short_lo): rows without edges)
 };
-// groups: lane groups take rows with edges too (else only those without); row: what a lane group's row costs, in edges.
+// groups: lane groups take the short rows; row: what a row of theirs costs, in edges.
 inline SmallShare small_share(const it_graph *g, int lpr, bool groups, int row) {
   SmallShare s;
   s.total = (int)g->h_list_offsets[g->n_lists];
+  s.short_lo = s.short_hi = (int)g->h_list_offsets[1];
   int64_t short_cost = 0, cost = 0;
-  s.short_lo = s.short_hi = 0;
-  for (int b = 0; b < g->n_lists; ++b) {
+  const int64_t empty_cost = (int64_t)s.short_lo * 3 * lpr / 16;
+  for (int b = 1; b < g->n_lists; ++b) {
     const int64_t rows = g->h_list_offsets[b + 1] - g->h_list_offsets[b], edges = g->h_list_edges[b];
-    if (b == 0 || (groups && g->list_bounds[b] <= IT_SHORT_BELOW && b != g->n_lists - 1)) {
+    if (groups && g->list_bounds[b] <= IT_SHORT_BELOW && b != g->n_lists - 1) {
       s.short_hi = (int)g->h_list_offsets[b + 1];
-      short_cost += (b == 0 ? rows * row / 2 : rows * row + edges) * lpr / 16;
+      short_cost += (rows * row + edges) * lpr / 16;
     } else {
       cost += rows * 16 + edges * 2 * lpr / 16;
     }
   }
-  const int rows = s.total - (s.short_hi - s.short_lo), most = g->num_sms * SMALL_BLOCKS;
-  const int want_short = (int)((s.short_hi - s.short_lo + THREADS / lpr - 1) / (THREADS / lpr)), want = (rows + THREADS / 32 - 1) / (THREADS / 32);
-  int share = short_cost > 0 ? (int)(most * short_cost / (short_cost + cost)) : 0;
-  if (share < 1 && want_short > 0) share = 1;
-  if (share > most - 1) share = most - 1;
-  s.short_blocks = share < want_short ? share : want_short;
-  const int left = most - s.short_blocks;
-  s.blocks = (unsigned)(s.short_blocks + (want < 1 ? 1 : (want < left ? want : left)));
+  const int most = g->num_sms * SMALL_BLOCKS;
+  const int64_t all = short_cost + cost + empty_cost;
+  auto part = [&](int64_t of, int want) {   // (at least a block where there is anything to do; two are left for the others)
+    int n = all > 0 ? (int)(most * of / all) : 0;
+    if (n < 1 && want > 0) n = 1;
+    if (n > most - 2) n = most - 2;
+    return n < want ? n : want;
+  };
+  s.short_blocks = part(short_cost, (s.short_hi - s.short_lo + THREADS / lpr - 1) / (THREADS / lpr));
+  s.empty_blocks = part(empty_cost, (s.short_lo + THREADS / 8 - 1) / (THREADS / 8));
+  const int used = s.short_blocks + s.empty_blocks, left = most - used > 1 ? most - used : 1, want = (s.total - s.short_hi + THREADS / 32 - 1) / (THREADS / 32);
+  s.blocks = (unsigned)(used + (want < 1 ? 1 : (want < left ? want : left)));
   return s;
+}
+
+// The rows without edges, a share of neighbours for every warp of their blocks.  rows(b, n): entries [b, b + n), n <= 32.
+template <class Rows>
+__device__ __forceinline__ void small_empties(const SmallShare &sh, Rows rows) {
+  const int warps = sh.empty_blocks * (THREADS / 32), each = (sh.short_lo + warps - 1) / warps;
+  int b = (((int)blockIdx.x - sh.short_blocks) * (THREADS / 32) + (int)(threadIdx.x >> 5)) * each;
+  const int end = b + each < sh.short_lo ? b + each : sh.short_lo;
+  for (; b < end; b += 32) rows(b, end - b < 32 ? end - b : 32);
 }
 
 // The rows of one warp, from the end of the list (pieces first) in turn, without the short rows.
@@ -82,13 +100,13 @@ inline SmallShare small_share(const it_graph *g, int lpr, bool groups, int row) 
 struct SmallRow { int j0, len, dest, owner; };   // (edges of a small graph are counted with 31 bits)
 template <bool WEIGHTED, bool OWNER, class Row>
 __device__ __forceinline__ void small_walk(const StreamParams &p, const SmallShare &sh, int lane, Row row) {
-  const int W = ((int)gridDim.x - sh.short_blocks) * (THREADS / 32), above = sh.total - sh.short_hi, n = above + sh.short_lo;
-  int i = ((int)blockIdx.x - sh.short_blocks) * (THREADS / 32) + (int)(threadIdx.x >> 5);
+  const int first = sh.short_blocks + sh.empty_blocks, W = ((int)gridDim.x - first) * (THREADS / 32), n = sh.total - sh.short_hi;
+  int i = ((int)blockIdx.x - first) * (THREADS / 32) + (int)(threadIdx.x >> 5);
   SmallRow m[3];
   auto fetch = [&](int at, SmallRow &x) {
     x = SmallRow{0, 0, 0, 0};
     if (at < n) {
-      const int entry = at < above ? sh.total - 1 - at : n - 1 - at;
+      const int entry = sh.total - 1 - at;
       const it_row_meta r = load_meta(p.meta + entry);
       x.j0 = (int)r.j0; x.len = r.len; x.dest = r.dest;
       if (OWNER) x.owner = __ldcs(p.owner + entry);

@@ -364,6 +364,83 @@ __global__ void __launch_bounds__(THREADS, IT_GATHER_MIN_BLOCKS) stream_rows_ker
   }
 }
 
+// ----------------------------------------------------------------------------- rows without edges
+// A warp takes up to 32 rows (their destinations with one coalesced load) and writes them 16 bytes per lane, four pieces in flight.
+// Bound by the writes (and the self terms): per-row kernels waited for each row's record, then its self term, before the row's store
+// (5.3M raw 256-byte rows: 340 -> 255 us; 615k GAT rows of 256 bytes: 82 -> 22; two layers of 8M rows of 128 bytes, one with self terms: 851 -> 638).
+struct EmptyRowsParams {
+  const it_row_meta *__restrict__ meta;
+  int64_t lo, hi;
+  char *dst;
+  const char *self;
+  int64_t pitch, self_pitch;
+  int kind, slices, bf16, act;   // slices: 16-byte pieces of a row
+  float value;
+  const float *__restrict__ bias;
+};
+__device__ __forceinline__ uint4 pack_piece(const float (&v)[8], int bf16) {
+  if (!bf16) return make_uint4(__float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3]));
+  uint32_t w[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+    w[k] = *reinterpret_cast<uint32_t *>(&h);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Piece s of a row that is the same for every vertex.
+__device__ __forceinline__ uint4 empty_piece(const EmptyRowsParams &p, int s) {
+  const int per = p.bf16 ? 8 : 4;
+  float v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = p.kind == IT_EMPTY_BIAS ? act_apply(p.bias && k < per ? __ldg(p.bias + s * per + k) : 0.f, p.act) : p.value;
+  return pack_piece(v, p.bf16);
+}
+
+// Rows [b, b + n) of the list, n <= 32, by a warp.  piece(s): piece s of a row that is the same for every vertex.
+template <class Piece>
+__device__ __forceinline__ void empty_rows_warp(const EmptyRowsParams &p, int64_t b, int n, int lane, Piece piece) {
+  int dest = 0;
+  if (lane < n) dest = __ldcs(&p.meta[b + lane].dest);
+  const int step_r = 32 / p.slices, step_s = 32 % p.slices, steps = (n * p.slices + 31) / 32;
+  int r = lane / p.slices, s = lane % p.slices;
+  for (int k = 0; k < steps; k += 4) {   // n rows x slices pieces, 32 at a time, four of those in flight
+    uint4 x[4];
+    int64_t at[4];
+    int sl[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int d = __shfl_sync(0xffffffffu, dest, r & 31);
+      sl[u] = s;
+      at[u] = r < n && k + u < steps ? (int64_t)d : -1;
+      if (at[u] >= 0) x[u] = p.kind == IT_EMPTY_SELF ? __ldcs(reinterpret_cast<const uint4 *>(p.self + at[u] * p.self_pitch) + s) : piece(s);
+      r += step_r; s += step_s;
+      if (s >= p.slices) { s -= p.slices; ++r; }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (at[u] < 0) continue;
+      if (p.kind == IT_EMPTY_SELF && p.act != IT_ACT_NONE) {
+        float v[8];
+        const uint32_t w[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (p.bf16) {
+            v[2 * q] = act_apply(__uint_as_float(w[q] << 16), p.act);
+            v[2 * q + 1] = act_apply(__uint_as_float(w[q] & 0xffff0000u), p.act);
+          } else {
+            v[q] = act_apply(__uint_as_float(w[q]), p.act);
+            v[4 + q] = 0.f;
+          }
+        }
+        x[u] = pack_piece(v, p.bf16);
+      }
+      __stcs(reinterpret_cast<uint4 *>(p.dst + at[u] * p.pitch) + sl[u], x[u]);
+    }
+  }
+}
+
 // ----------------------------------------------------------------------------- short rows: one lane group each, no edge stream
 // For rows of at most a few dozen edges the bookkeeping of a flat edge stream costs more than the edges.
 // Here a group of LPR lanes (16-byte slices, LPR >= 8) owns one row: lanes 0..7 of the group fetch eight
@@ -387,9 +464,8 @@ __global__ void __launch_bounds__(THREADS, IT_GATHER_MIN_BLOCKS) stream_rows_ker
 #define IT_SHORT_PIPE_WAVES 1    // grid = SMs x resident CTAs x this: every CTA is resident from the start and walks its rows
 #endif
 // block / blocks: which share of the rows p.row_lo .. p.row_hi this block walks; sbuf: SHORT_STAGE_BYTES of shared memory.
-// EMPTY: rows without edges are among them.
 constexpr int SHORT_STAGE_BYTES = IT_SHORT_EDGES * THREADS * 16;
-template <typename T, int LPR, class Policy, bool PAD, bool EMPTY = false>
+template <typename T, int LPR, class Policy, bool PAD>
 __device__ __forceinline__ void short_rows_pipe(const StreamParams &p, Policy &pol, int block, int blocks, uint4 *sbuf) {
   constexpr int NS = Policy::NS;
   constexpr int E = IT_SHORT_EDGES;   // edges per round
@@ -404,10 +480,9 @@ __device__ __forceinline__ void short_rows_pipe(const StreamParams &p, Policy &p
   const uint32_t my_buf = (uint32_t)__cvta_generic_to_shared(sbuf + threadIdx.x);
 
   struct Row { int64_t j0; int len, dest, owner; };
-  constexpr int NONE = EMPTY ? -1 : 0;   // length of a missing row
-  // the row this lane group takes in the sweep that starts at i0
+  // the row this lane group takes in the sweep that starts at i0 (len 0: none; rows of these buckets have edges)
   auto load_row = [&](int64_t i0) {
-    Row r{0, NONE, 0, 0};
+    Row r{0, 0, 0, 0};
     const int64_t i = i0 + lane / LPR;
     if (i < p.row_hi) {
       const it_row_meta m = load_meta(p.meta + i);
@@ -431,12 +506,11 @@ __device__ __forceinline__ void short_rows_pipe(const StreamParams &p, Policy &p
   load_idx(cur, 0, idx_c, w_c);
   for (; i0 < p.row_hi; i0 += sweep) {
     const Row nn = load_row(i0 + 2 * sweep);   // in flight for two rows
-    int maxlen = __reduce_max_sync(0xffffffffu, cur.len);
-    if (EMPTY && maxlen < 1) maxlen = 1;   // (a round in any case: it fetches the ids of the next rows)
+    const int maxlen = __reduce_max_sync(0xffffffffu, cur.len);
     float st[NS];
     pol.init(st);
-    const int len = active ? cur.len : NONE;
-    if (len > NONE) pol.begin_row(cur.dest, cur.owner);
+    const int len = active ? cur.len : 0;
+    if (len > 0) pol.begin_row(cur.dest, cur.owner);
     for (int k0 = 0; k0 < maxlen; k0 += E) {
       // the indices of the next round, in flight while this round's rows are
       int32_t idx_n; float w_n;
@@ -465,7 +539,7 @@ __device__ __forceinline__ void short_rows_pipe(const StreamParams &p, Policy &p
       }
       idx_c = idx_n; w_c = w_n;
     }
-    if (len > NONE) pol.end_row(st, cur.dest, cur.owner, len);
+    if (len > 0) pol.end_row(st, cur.dest, cur.owner, len);
     cur = nxt; nxt = nn;
   }
 }
