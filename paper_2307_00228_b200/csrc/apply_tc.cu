@@ -1466,6 +1466,10 @@ constexpr size_t kWeightBudget = kSmemBudget - kSmemAux - 1024 /*per-column cons
 // weights stay resident or would need more than two times as many splits, with one accumulator instead of two (of 256 TMEM columns each):
 // 2M rows, K = 128, 128 columns 487 against 431 us; 1M rows 192, 96 366 / 259; 384, 128 877 / 618; 500k rows 600, 256 1325 / 826; 30k
 // rows 128, 128 16.0 / 13.3.  Not with fewer tiles than SMs, nor streamed in place of two resident splits (100k rows, 256, 128 65 / 72).
+//
+// What a shape is refused for, and how many columns are prepared at most, is decided by the narrow form alone: a layer takes the same
+// arithmetic whatever its number of rows (a head of 128 columns, or more than 16 splits of 64, stays with the fp32 kernel), and scratch
+// does not grow.
 bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_cols *out) {
   const bool tf32 = a.x_dtype == IT_F32;
   const int bk = TC_KBLOCK_BYTES / (tf32 ? 4 : 2), KB = (a.K1 + bk - 1) / bk + ((a.X2 ? a.K2 : 0) + bk - 1) / bk;
@@ -1474,28 +1478,37 @@ bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_
   out->stream = 0;
   const int n = out->n0p + out->n1p, step = want_scores ? head_dim : 16;
   if (n <= 0 || step % 16 != 0) return false;
+  const int64_t tiles = (a.M + TC_BM - 1) / TC_BM;
+  // as few splits as fit with resident weights, of at most `most` columns and `NB` in all
+  auto resident = [&](int most, int NB) {
+    for (int s = 1; s <= 16; ++s) {
+      const int c = ((n + s - 1) / s + step - 1) / step * step;
+      if (c > most || c * s > NB) continue;
+      if ((size_t)(tf32 ? 2 : 1) * KB * c * TC_KBLOCK_BYTES > kWeightBudget) continue;
+      if (want_scores && c * s != n) continue;
+      out->n_splits = s; out->nbc = c; out->NB = c * s;
+      return true;
+    }
+    return false;
+  };
   // fp32 mode issues MMAs of 2 c columns and keeps one or two accumulators of as many TMEM columns next to the split A stages
+  if (!resident(tf32 ? 64 : 256, INT32_MAX)) return false;
+  const it_tc_cols narrow = *out;
   int most = tf32 ? 128 : 256;
-  if (tf32 && (a.M + TC_BM - 1) / TC_BM * ((n + most - 1) / most) < IT_NUM_SMS_FALLBACK) most = 64;   // few tiles: more CTAs
-  for (int s = 1; s <= 16; ++s) {
-    const int c = ((n + s - 1) / s + step - 1) / step * step;
-    if (c > most) continue;
-    if ((size_t)(tf32 ? 2 : 1) * KB * c * TC_KBLOCK_BYTES > kWeightBudget) continue;
-    if (want_scores && c * s != n) continue;
-    out->n_splits = s; out->nbc = c; out->NB = c * s;
-    int few = (n + most - 1) / most, wide = 0;
-    for (; few < s; ++few) {   // (no more prepared columns than the resident form has: scratch does not grow)
-      wide = ((n + few - 1) / few + 15) / 16 * 16;
-      if (wide * few <= c * s) break;
-    }
-    const bool few_tiles = tf32 && (a.M + TC_BM - 1) / TC_BM * few < 512;
-    if (few < s && !want_scores && (!few_tiles || s >= 2 * few) && (!tf32 || wide <= 64 || s > 2 * few)) {
-      out->stream = 1;
-      out->n_splits = few; out->nbc = wide; out->NB = wide * few;
-    }
-    return true;
+  if (tf32 && tiles * ((n + most - 1) / most) < IT_NUM_SMS_FALLBACK) most = 64;   // few tiles: more CTAs
+  if (tf32 && most > 64) resident(most, narrow.NB);
+  const int s = out->n_splits;
+  int few = (n + most - 1) / most, wide = 0;
+  for (; few < s; ++few) {   // (no more prepared columns than the resident form has)
+    wide = ((n + few - 1) / few + 15) / 16 * 16;
+    if (wide * few <= out->NB) break;
   }
-  return false;
+  const bool few_tiles = tf32 && tiles * few < 512;
+  if (few < s && !want_scores && (!few_tiles || s >= 2 * few) && (!tf32 || wide <= 64 || s > 2 * few)) {
+    out->stream = 1;
+    out->n_splits = few; out->nbc = wide; out->NB = wide * few;
+  }
+  return true;
 }
 
 bool it_tc_supported(const it_gemm_args &a, int heads, int head_dim, bool want_scores) {
@@ -1794,7 +1807,7 @@ extern "C" it_status it_debug_expire_wait_form(it_graph *g, int form, void *buff
   } else if (form < 5) {   // 3, 4: streamed weights, more tiles than stages
     a.M = 128; a.K1 = 1024; a.n0 = form == 4 ? 256 : 512;
   } else {   // 5: fp32 with one accumulator
-    a.M = (int64_t)IT_NUM_SMS_FALLBACK * 2 * TC_BM; a.K1 = 64; a.n0 = 128;
+    a.M = (int64_t)IT_NUM_SMS_FALLBACK * 2 * TC_BM; a.K1 = 128; a.n0 = 128;
   }
   it_tc_cols cols;
   IT_REQUIRE(it_tc_columns(a, a.n0, false, &cols) && (form < 3 ? cols.n_splits == 1 && !cols.stream : (form < 5 ? cols.stream != 0 : cols.nbc > 64)),
