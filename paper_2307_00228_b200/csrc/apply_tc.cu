@@ -1466,6 +1466,10 @@ constexpr size_t kWeightBudget = kSmemBudget - kSmemAux - 1024 /*per-column cons
 // weights stay resident or would need more than two times as many splits, with one accumulator instead of two (of 256 TMEM columns each):
 // 2M rows, K = 128, 128 columns 487 against 431 us; 1M rows 192, 96 366 / 259; 384, 128 877 / 618; 500k rows 600, 256 1325 / 826; 30k
 // rows 128, 128 16.0 / 13.3.  Not with fewer tiles than SMs, nor streamed in place of two resident splits (100k rows, 256, 128 65 / 72).
+// Then nothing hides a tile's epilogue, so it needs a K whose product takes longer: two splits of 64 against one, 1M rows, K = 32 / 64 /
+// 96 / 128: 128 columns 148 / 168 / 216 / 263 against 198 / 203 / 215 / 239 us, 96 columns 164 / 166 / 219 / 267 against 168 / 173 / 192 / 217,
+// 80 columns 176 / 168 / 230 / 276 against 153 / 158 / 180 / 208; 270k rows, K = 96: 70 / 71 / 73 (128, 96, 80 columns) against 74 / 65 / 62; few
+// tiles pay for the last wave: 20k rows, K = 64, 80 columns 9.7 / 10.9, K = 96, 96 columns 11.3 / 12.2; 70k rows, K = 32, 80 columns 15.3 / 15.9.
 //
 // What a shape is refused for, and how many columns are prepared at most, is decided by the narrow form alone: a layer takes the same
 // arithmetic whatever its number of rows (a head of 128 columns, or more than 16 splits of 64, stays with the fp32 kernel), and scratch
@@ -1496,7 +1500,10 @@ bool it_tc_columns(const it_gemm_args &a, int head_dim, bool want_scores, it_tc_
   const it_tc_cols narrow = *out;
   int most = tf32 ? 128 : 256;
   if (tf32 && tiles * ((n + most - 1) / most) < IT_NUM_SMS_FALLBACK) most = 64;   // few tiles: more CTAs
-  if (tf32 && most > 64) resident(most, narrow.NB);
+  if (tf32 && most > 64 && resident(most, narrow.NB)) {
+    const bool long_k = KB >= 4 || (tiles >= 2 * IT_NUM_SMS_FALLBACK && ((KB == 3 && out->nbc <= 96) || (out->nbc <= 80 && (KB >= 2 || tiles >= 1024))));
+    if (!long_k) *out = narrow;
+  }
   const int s = out->n_splits;
   int few = (n + most - 1) / most, wide = 0;
   for (; few < s; ++few) {   // (no more prepared columns than the resident form has)

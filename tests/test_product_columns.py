@@ -84,3 +84,11 @@ def test_fp32_products_are_taken_and_prepared_as_by_splits_of_64_columns(columns
             assert not (s[4] and stream)
             wide += nbc > 64
     assert wide > 100
+
+
+def test_short_fp32_products_keep_two_accumulators(columns):
+    """One accumulator of 65 to 128 columns leaves nothing to hide a tile's epilogue behind: not for K of up to 64 (128 columns: up to 96)."""
+    rows = [(1, m, k, 0, n, 0, 0) for k in (16, 32, 64, 96) for n in (96, 112, 128, 256) for m in MS if not (k == 96 and n == 96)]
+    assert all(ok and nbc <= 64 for ok, _, nbc, _, _ in columns(rows))
+    rows = [(1, m, k, 0, n, 0, 0) for k in (128, 192) for n in (96, 128) for m in MS[-3:] if not (k == 192 and n == 128)]
+    assert all(ok and nbc == r[4] for r, (ok, _, nbc, _, _) in zip(rows, columns(rows)))
