@@ -404,8 +404,8 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
           return c.recording() ? IT_OK : it_launch_message_combine(g, q, c.st);
         }
         it_tc_reduce rows{};
-        rows.mode = 6; rows.dst = Q; rows.dim = L->msg_dim;
-        IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, whole ? L->act_edge : IT_ACT_NONE, whole ? nullptr : Q,
+        rows.mode = 6;
+        IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, whole ? L->act_edge : IT_ACT_NONE, Q,
                          whole ? table : nullptr, whole ? g->indices : nullptr, whole ? &rows : nullptr));
         if (c.recording()) return IT_OK;
         if (!whole) IT_TRY(it_launch_edge_messages(g, dt, L->msg_dim, table, Q, L->act_edge, c.st));

@@ -145,6 +145,7 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, const void 
 }
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait_read_but_last() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Named barriers of the epilogue warps (immediate operands): barrier 1 over all sixteen warps, or barriers 1 and 2
 // over the eight warps of a group, or 1 to 4 over the four.  The reducing form also tells every thread whether any of them failed.
@@ -387,22 +388,6 @@ __device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *s
   if (gw == WARPS - 1 && has_next && start < TC_BM) fold(TC_BM - 1, -1);
 }
 
-// TC_FOLD_STORE: the tile's rows as they are, row m of q.dst for edge m (`edges` of them).
-template <int WARPS>
-__device__ __forceinline__ void tc_store_tile(uint32_t tile_s, int64_t tile, int64_t edges, int gw, int lane, const it_tc_reduce &q) {
-  constexpr int RW = TC_BM / WARPS;
-  const int pieces = q.dim / 8;   // of 16 bytes
-  for (int i = lane; i < RW * pieces; i += 32) {
-    const int r = gw * RW + i / pieces, ch = i % pieces;
-    const int64_t m = tile * TC_BM + r;
-    if (m >= edges) break;
-    const uint32_t at = tile_s + (uint32_t)(ch >> 3) * (uint32_t)(TC_BM * TC_KBLOCK_BYTES) + (uint32_t)r * 128u + (uint32_t)(((ch & 7) ^ (r & 7)) << 4);
-    uint4 v;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at) : "memory");
-    __stcs(reinterpret_cast<uint4 *>(q.dst) + m * pieces + ch, v);
-  }
-}
-
 // STREAM: the weights do not stay in shared memory; the k-block of them that belongs to an operand tile comes with it, in the same
 // stage.  (For weights so large that a CTA could keep few columns of them only: it_tc_columns.)
 // FOLD (with ADD): what becomes of the rows, TC_FOLD_*, a kernel each: one reduce in the code of all warps fits the instruction
@@ -469,7 +454,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
     if (ADD)
       for (int a = 0; a < add_stages; ++a) {
         mbar_init(&add_full[a], 128);
-        mbar_init(&add_empty[a], ADD);
+        mbar_init(&add_empty[a], FOLD == TC_FOLD_STORE ? 1 : ADD);
       }
     for (int a = 0; a < NACC; ++a) {
       mbar_init(&acc_full[a], 1);
@@ -629,6 +614,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
       int it = 0;   // tiles of this CTA so far: tile `it` uses accumulator it % NACC, for the (it / NACC)-th time
       int slot = -1;   // ADD: of the ring of rows, and how often it came round
       uint32_t slot_phase = 1;
+      // ADD, rows written: the stage of the group's previous tile, until its copy has read it.  (A ring of more stages than groups never
+      // waits for itself: a tile's stage needs an earlier tile of its group, or of the group that held the stage, to be over.)
+      int held = -1;
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
         if (ADD && (++slot == add_stages || it == 0)) { slot = 0; slot_phase ^= 1u; }
         if (G > 1 && (it & (G - 1)) != group) continue;   // (G and NACC are 1, 2 or 4)
@@ -786,15 +774,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           if (lane == 0) mbar_arrive(&acc_empty[acc]);
         }
         if constexpr (ADD) {
-          const int32_t *seg = seg_s + slot * TC_SEG_WORDS;
-          const uint32_t tile_s = smem_u32(smem_add) + (uint32_t)slot * (uint32_t)p.add_stage_bytes;
-          const bool cut = tile > 0 && seg[2 * TC_BM] < 0, next = (int64_t)(tile + 1) * TC_BM < p.M;
-          const int gw = (warp - 2) % ADD;
-          if (epi_bar_any(G, group, false)) { ok = false; break; }   // the tile is complete
-          if constexpr (FOLD == TC_FOLD_STORE) tc_store_tile<ADD>(tile_s, tile, p.M, gw, lane, p.red);
-          else tc_reduce_tile<FOLD, ADD, NARROW>(tile_s, seg, cut, next, tile, gw, lane, p.red, p.nbc);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&add_empty[slot]);
+          if constexpr (FOLD == TC_FOLD_STORE) {   // written from where it lies; its stage is free when the copy has read it
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if (epi_bar_any(G, group, false)) { ok = false; break; }   // the tile is complete
+            if (issuer) {
+              for (int k = 0; k < pan0; ++k) tma_store_2d(&map_o0, smem_add + (size_t)slot * p.add_stage_bytes + (size_t)k * a_tile_bytes, k * 64, m0);
+              tma_store_commit();
+              if (held >= 0) {
+                tma_store_wait_read_but_last();
+                mbar_arrive(&add_empty[held]);
+              }
+              held = slot;
+            }
+          } else {
+            const int32_t *seg = seg_s + slot * TC_SEG_WORDS;
+            const uint32_t tile_s = smem_u32(smem_add) + (uint32_t)slot * (uint32_t)p.add_stage_bytes;
+            const bool cut = tile > 0 && seg[2 * TC_BM] < 0, next = (int64_t)(tile + 1) * TC_BM < p.M;
+            if (epi_bar_any(G, group, false)) { ok = false; break; }   // the tile is complete
+            tc_reduce_tile<FOLD, ADD, NARROW>(tile_s, seg, cut, next, tile, (warp - 2) % ADD, lane, p.red, p.nbc);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&add_empty[slot]);
+          }
           continue;
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the TMA store's reads
@@ -807,7 +807,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           tma_store_commit();
         }
       }
-      if (!ADD && issuer) tma_store_wait_all();   // the staging tile must outlive the last stores
+      if ((!ADD || FOLD == TC_FOLD_STORE) && issuer) tma_store_wait_all();   // the staging tile must outlive the last stores
     } else
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
       const int64_t m = (int64_t)(tile / p.n_splits) * TC_BM + row_in_tile;

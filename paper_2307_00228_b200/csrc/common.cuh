@@ -283,7 +283,7 @@ struct it_tc_reduce {
   const float *weights;          // of the edges, or NULL
   void *dst;                     // bf16 rows: the reduce of every vertex
   int dst_ld, dim;
-  int mode, is_mean;             // 0 sum, 1 weighted sum, 2 max, 3 min, 4 / 5 the same unweighted; 6: not reduced, row m of dst is edge m's
+  int mode, is_mean;             // 0 sum, 1 weighted sum, 2 max, 3 min, 4 / 5 the same unweighted; 6: not reduced, row m of out0 is edge m's
 };
 struct it_gemm_args {
   int64_t M;
@@ -295,7 +295,7 @@ struct it_gemm_args {
   int n1; void *out1; it_dtype dt1;
   void *out2;
   // tensor-core path, the shapes of it_tc_adds_rows: row m = act0(round(C + bias0) + add_rows[add_idx[m], :]), rows of n0 elements
-  // of dt0; `round` to dt0, as if the product had been stored and read back.  Row m is edge m: reduced, not stored (out0 unused)
+  // of dt0; `round` to dt0, as if the product had been stored and read back.  Row m is edge m: reduced (out0 unused) or stored
   const void *add_rows; const int32_t *add_idx; it_tc_reduce reduce;
   uint32_t spin_limit;   // tensor-core path: polls after which a barrier wait gives up (0 = the default)
   int no_loads;          // tensor-core path, test hook: issue no operand copies

@@ -259,7 +259,7 @@ it_status launch_small(const it_gather_args &a, StreamParams sp, cudaStream_t st
   sp.weights = a.use_edge_weights ? sp.weights : nullptr;
   if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(it_done_words(a.counters), 0, (size_t)g->n_long * sizeof(int), st));
   auto go = [&]<int LPR>() -> it_status {
-    const SmallShare sh = small_share(g, LPR < 8 ? 8 : LPR, LPR <= 16, 8);   // (a row of 512 bytes takes the warp either way: 100k vertices / 1.6M edges 191 us, by groups 197)
+    const SmallShare sh = small_share(g, LPR < 8 ? 8 : LPR, LPR <= 16, a.per_edge_rows && LPR >= 8 ? 5 : 8);   // (a row of 512 bytes takes the warp either way: 100k vertices / 1.6M edges 191 us, by groups 197)
     IT_LAUNCH(IT_K_GATHER_SMALL, bytes, 0, st,
               IT_CUDA_TRY(it_launch_pdl(gather_small_kernel<T, LPR, Policy>, dim3(sh.blocks), dim3(THREADS), sh.short_blocks ? SHORT_STAGE_BYTES : 0, st, sp, pol,
                                         piece_params(g, it_done_words(a.counters)), sh, (const int64_t *)g->owner_indptr, (const int64_t *)g->shadow_indptr)));
