@@ -15,6 +15,7 @@ struct LayerWs {
   size_t off_counters;                              // it_gather_words() words
   size_t off_B, off_partials, off_a, off_b, off_q;  // a: aggregate A | self term S | scores ; b: Z | P ; q: per-edge part Q / messages
   size_t bytes;
+  bool reduced;   // PLAN_MSG: the messages are reduced in their product
 };
 
 bool is_pooling(it_gather_op op) { return op == IT_GATHER_SUM || op == IT_GATHER_MEAN || op == IT_GATHER_MAX || op == IT_GATHER_MIN; }
@@ -123,9 +124,17 @@ bool message_in_product(const it_graph *g, const it_layer_desc *L) {
   return it_tc_adds_rows(ga);
 }
 
-// ... and reduces it, where the few more launches around that are worth it (the messages written and reduced by the gather against
-// reduced in the product: 10k vertices / 100k edges 39 against 62 us, 30k / 400k 73 / 88, 100k / 1.5M 196 / 187, 300k / 5M 505 / 443).
-bool messages_reduced(const it_graph *g) { return g->e > 5 << 18; }
+// ... and reduces it, where that wins: what it saves is a write and a read of the message rows, what it costs is issue slots of the
+// product per edge and per end of a vertex, and three more launches.  Written by the product and reduced by the gather against reduced
+// in the product, bf16, 32 edge features, 16 edges per vertex: 64 columns, mean 1.4M / 2.5M / 5M / 12M edges 165 / 258 / 460 / 1060 against
+// 183 / 268 / 461 / 1023 us, max 165 / 258 / 459 / 1063 against 178 / 261 / 451 / 998; 128 columns, mean 288 / 460 / 847 / 1940 against 289 / 455 /
+// 835 / 1942, max 290 / 460 / 843 / 1939 against 281 / 441 / 807 / 1876; 16 edges, 32 columns, 12M 761 against 850; 10 and 4 edges per vertex, 8M,
+// 64 columns 749 / 928 against 791 / 1051.  With edge weights never: 64 and 128 columns, 12M 1086 / 1958 against 1146 / 2307.
+// Where the message rows do not fit (lean) they are reduced in any case: that takes 4 to 8 bytes of scratch per edge.
+bool messages_reduced(const it_graph *g, const it_layer_desc *L, bool lean) {
+  if (L->edge_dim == 0 || !message_in_product(g, L)) return false;
+  return lean || (!L->use_edge_weights && L->msg_dim >= 64 && g->e >= 14 * g->n && g->e * L->msg_dim >= (int64_t)320 << 20);
+}
 
 // The scratch of a layer.  lean: without partial rows (long vertices are then reduced whole, one block each).
 LayerWs plan_layer(const it_graph *g, const it_layer_desc *L, bool lean = false) {
@@ -137,6 +146,7 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L, bool lean = false)
   auto take = [&](size_t bytes) { size_t o = off; off += it_align_up(bytes); return o; };
   w.plan = plan_of(L);
   w.off_q = 0;
+  w.reduced = false;
   w.off_counters = take((lean ? IT_MAX_BUCKETS + 1 : it_gather_words(g)) * sizeof(int));
   w.off_B = take(weight_bytes(g, L).largest);
   switch (w.plan) {
@@ -175,7 +185,7 @@ LayerWs plan_layer(const it_graph *g, const it_layer_desc *L, bool lean = false)
       w.off_b = off;
       break;
     case PLAN_MSG: {
-      const bool reduced = fe > 0 && message_in_product(g, L) && messages_reduced(g);
+      const bool reduced = w.reduced = messages_reduced(g, L, lean);
       const size_t tiles = ((size_t)g->e + IT_MSG_TILE - 1) / IT_MSG_TILE;
       w.off_partials = take(reduced ? 0 : pieces * fm * 4);
       w.off_a = take(n * fm * s);                            // A: aggregate of the messages
@@ -390,7 +400,7 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
         const size_t es = (size_t)it_dtype_size(dt);
         const char *W_edge_part = (const char *)L->W_edge + (size_t)L->in_dim * L->msg_dim * es;
         const bool whole = message_in_product(g, L);
-        if (whole && messages_reduced(g)) {
+        if (c.w.reduced) {
           const size_t tiles = ((size_t)g->e + IT_MSG_TILE - 1) / IT_MSG_TILE;
           int32_t *first = reinterpret_cast<int32_t *>((char *)Q + it_align_up(tiles * 2 * (size_t)L->msg_dim * 4));
           int32_t *ends = reinterpret_cast<int32_t *>((char *)first + it_align_up(tiles * 4));

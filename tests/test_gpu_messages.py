@@ -86,18 +86,72 @@ def test_messages_written_by_their_product(degrees, fm, weights):
 @pytest.mark.parametrize("op,weights,fm,tail", [("sum", False, 64, 0), ("sum", True, 24, 1), ("mean", False, 24, 127), ("mean", True, 120, 64), ("max", False, 64, 1),
                                                 ("min", True, 64, 0), ("max", False, 120, 5), ("gcn", True, 120, 127), ("min", False, 24, 0), ("max", True, 24, 3)])
 def test_messages_reduced_by_their_product(op, weights, fm, tail):
-    """Many edges: messages are reduced tile by tile where they are made; every pattern of ends of vertices, a last tile of `tail` edges
-    (0: a whole one).  Oracle and tolerance of the other message tests: a sum in another order differs in fp32 only."""
+    """Many edges: written by the product with the caller's workspace, reduced tile by tile where they are made without one (their rows
+    then do not fit); every pattern of ends of vertices, a last tile of `tail` edges (0: a whole one).  Oracle and tolerance of the other
+    message tests: a sum in another order differs in fp32 only."""
     layer = make_msg_layer(15, op, "none", 16, fm, 24, "bf16", act_edge="elu" if op == "sum" else "relu", weights=weights, edge_dim=8)
-    bulk = np.random.default_rng(16).integers(0, 48, 58_000)
+    bulk = np.random.default_rng(16).integers(0, 48, 58_000) if fm < 120 else np.random.default_rng(16).integers(0, 96, 29_000)
     deg = [d for p in TILE_DEGREES.values() for d in p] + bulk.tolist()
     deg.append((tail - sum(deg)) % 128)
     assert sum(deg) % 128 == tail and sum(deg) > 5 << 18
     w = tile_workload(deg, layer, 17)
-    got, _ = run_device(w)
+    got, d = run_device(w)
     check_against_oracle(w, got, label=(op, weights, fm, tail))
     again, _ = run_device(w, int32_indptr=True)
     assert np.array_equal(got, again)
+    assert w.e * fm * 2 > 32 << 20   # the message rows alone exceed the built-in scratch
+    reduced = static_forward(d)
+    assert_same_reduce(op, d.out.float(), reduced.float())
+    assert torch.equal(reduced, static_forward(d))
+
+
+def static_forward(d):
+    out = torch.full_like(d.out, float("nan"))
+    B.it_layer_forward_static(d.graph, d.layers[0], d.x, out)
+    B.it_graph_check(d.graph)
+    return out
+
+
+def assert_same_reduce(op, a, b):
+    """Two orders of the same reduce: max and min the same bits; sums differ by a rounding (2^-8) of the bf16 aggregate and one of the output,
+    of products of the order of the largest."""
+    if op in ("max", "min"):
+        assert torch.equal(a.nan_to_num(nan=12345.0), b.nan_to_num(nan=12345.0))
+        return
+    ok = torch.isfinite(a)
+    assert torch.equal(ok, torch.isfinite(b))
+    assert (a[ok] - b[ok]).abs().max() <= 2.0 ** -7 * a[ok].abs().max()
+
+
+@pytest.mark.parametrize("op,fm,deg_max", [("max", 64, 90), ("mean", 128, 60), ("mean", 72, 80)])
+def test_messages_reduced_by_their_product_with_a_workspace(op, fm, deg_max):
+    """As many edges as make the reduce in the product the faster form: the scratch then holds no message rows (oracle and tolerance of
+    the other message tests)."""
+    e = (320 << 20) // fm + 1000
+    deg = np.random.default_rng(21).integers(0, deg_max, 2 * e // (deg_max - 1) + 1000)
+    layer = make_msg_layer(22, op, "none", 16, fm, 24, "bf16", act_edge="relu", edge_dim=8)
+    w = tile_workload(deg, layer, 23)
+    assert w.e >= e and w.e >= 14 * w.n
+    got, d = run_device(w)
+    assert B.it_workspace_bytes(d.graph, d.layers) < w.e * fm * 2
+    check_against_oracle(w, got, label=(op, fm))
+
+
+@pytest.mark.parametrize("op,fm", [("max", 64), ("min", 24), ("sum", 40), ("mean", 120), ("max", 8), ("sum", 16)])
+def test_infinite_and_undefined_messages_reduce_the_same_in_their_product(op, fm):
+    """Messages of +-inf and NaN, and the narrowest rows: the reduce in the product gives what the gather gives of the written rows (max and
+    min: the same bits; sums: to the rounding of bf16 outputs, infinities and NaN where they are)."""
+    layer = make_msg_layer(31, op, "none", 16, fm, 24, "bf16", act_edge="none", edge_dim=8)
+    deg = [d for p in TILE_DEGREES.values() for d in p] + np.random.default_rng(32).integers(0, 60, (32 << 20) // (2 * fm) // 25).tolist()
+    w = tile_workload(deg, layer, 33)
+    rng = np.random.default_rng(34)
+    bits = w.edge_feat.view(np.uint16)
+    bits[rng.random(w.e) < 0.01, 0] = 0x7f80    # inf times weights of both signs
+    bits[rng.random(w.e) < 0.002, 1] = 0x7fc0
+    got, d = run_device(w)
+    assert w.e * fm * 2 > 32 << 20
+    assert not torch.isfinite(d.out).all() and torch.isfinite(d.out).any()
+    assert_same_reduce(op, d.out.float(), static_forward(d).float())
 
 
 def test_message_layers_stack_with_plain_layers():
