@@ -1460,7 +1460,10 @@ constexpr size_t kWeightBudget = kSmemBudget - kSmemAux - 1024 /*per-column cons
 // weights kept 80 KB in flight).  Resident against streamed, 1M rows: bf16 K = 768, 512 columns 1404 against 724 us; 512, 256 360 / 286;
 // 384, 256 309 / 244; 448, 192 322 / 254; 1024, 128 675 / 400; fp32, 64 columns per CTA (500k rows) 600, 256 3970 / 1323; 512, 256 1686 / 1125;
 // 1M rows 320, 64 544 / 381; 384, 128 1000 / 879.  20k rows bf16 768, 512 73 / 51; 512, 256 16.0 / 15.0; but 10k rows fp32 384, 128 18.5 / 22.1:
-// there the splits fill the SMs, so fp32 products of few tiles are streamed only from twice as many splits on.
+// there the splits fill the SMs, so fp32 products of few tiles are streamed only from twice as many splits on.  bf16 ones always are: where
+// resident splits would fit one wave, whole calls (weights prepared, launches overlapped) at 2k / 5k / 9k rows take, resident against
+// streamed, K = 768, 256 columns 16.0 / 17.3 / 38.8 against 17.3 / 17.3 / 17.4 us; 512, 256 - / 14.9 / 15.0 against - / 14.5 / 14.5; 1024, 128
+// 15.1 / 15.1 / 26.3 against 14.9 / 15.2 / 15.3; 768, 512 21.5 / 63 / 69 against 22.5 / 22.2 / 43.3.
 //
 // fp32 mode: an instruction of 2 c columns takes nearly as long for c = 64 as for 128, so a CTA takes up to 128 columns where their
 // weights stay resident or would need more than two times as many splits, with one accumulator instead of two (of 256 TMEM columns each):
