@@ -445,7 +445,8 @@ __global__ void __launch_bounds__(PIECE_BINS) long_pieces_kernel(SplitParams p) 
 // Status words of graphs: the validation's flags, later set by a kernel that gives up a wait.  They come from a fixed array, since an
 // allocation of four bytes costs as much as any (0.33 ms, and 0.26 to give it back: a quarter of the set-up of 5M vertices / 100M edges); beyond
 // that many graphs on a device at a time, and on devices beyond the first 64, a word is allocated.  A word is given back when nothing on the
-// device uses it any more: after the graph's arrays, whose release waits for the device.
+// device uses it any more: after the graph's arrays, whose release waits for the device, or after a wait for the stream; where there was
+// neither (`quiet` false) it stays taken, since what is still queued may write it.
 constexpr int STATUS_WORDS = 1024;
 static __device__ int g_status_words[STATUS_WORDS];
 namespace {
@@ -475,12 +476,12 @@ static it_status status_take(int device, int **out) {
   IT_CUDA_TRY(cudaMalloc(out, sizeof(int)));
   return IT_OK;
 }
-static void status_give_back(int device, int *word) {
+static void status_give_back(int device, int *word, bool quiet) {
   if (device >= 0 && device < kMaxDevices) {
     std::lock_guard<std::mutex> lk(g_status_mu);
     const int64_t at = g_status_base[device] ? word - g_status_base[device] : -1;
     if (at >= 0 && at < STATUS_WORDS) {
-      g_status_taken[device][at / 64] &= ~((uint64_t)1 << (at % 64));
+      if (quiet) g_status_taken[device][at / 64] &= ~((uint64_t)1 << (at % 64));
       return;
     }
   }
@@ -728,11 +729,13 @@ static it_status create_impl(int64_t n, int64_t n_src, int64_t e, const void *in
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(&h_flags, d_status, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
   if (ce != cudaSuccess || h_flags != 0 || g == nullptr || room != IT_OK) {
+    const bool quiet = ce == cudaSuccess || cudaStreamSynchronize(st) == cudaSuccess;
     if (g != nullptr) slab_free(g);
     delete g;
-    status_give_back(device, d_status);
+    status_give_back(device, d_status, quiet);
   }
   if (ce != cudaSuccess) {
+    cudaGetLastError();   // (reported here, and by no later call)
     it_set_error("graph validation failed to run: %s", cudaGetErrorString(ce));
     return IT_ERR_CUDA;
   }
@@ -804,8 +807,9 @@ extern "C" it_status it_graph_check(it_graph *g, void *stream) {
 
 extern "C" it_status it_graph_destroy(it_graph *g) {
   if (!g) return IT_OK;
+  const bool quiet = g->slab != nullptr;   // (its release waits)
   slab_free(g);
-  status_give_back(g->device, g->d_status);
+  status_give_back(g->device, g->d_status, quiet);
   delete g;
   return IT_OK;
 }

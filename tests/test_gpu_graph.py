@@ -235,3 +235,33 @@ def test_every_form_of_the_product_gives_up_by_itself(form):
     d.infer()
     B.it_graph_check(d.graph)
     check_against_oracle(w, to_numpy(d.out))
+
+
+def test_more_graphs_than_status_words():
+    """A device has a fixed number of status words; the graphs beyond have one of their own, and words are given back and taken again: a
+    timeout is reported by the graph that it happened on, and by none that takes its word later."""
+    ip, ix = random_csr(5, 20, 3)
+    ip, ix = torch.from_numpy(ip).cuda(), torch.from_numpy(ix).cuda()
+    x, o = torch.zeros((128, 64), device="cuda"), torch.empty((128, 64), device="cuda")
+    ws = torch.empty(1 << 16, dtype=torch.uint8, device="cuda")
+    graphs = [B.it_graph_create(ip, ix) for _ in range(1040)]
+    for k in (0, 700, 1039):   # the last one has a word of its own
+        B.it_debug_expire_wait(graphs[k], x, o, ws)
+    torch.cuda.synchronize()
+    for k, g in enumerate(graphs):
+        if k == 700:
+            B.it_graph_destroy(g)      # with its timeout unreported
+        elif k in (0, 1039):
+            with pytest.raises(B.ItError) as e:
+                B.it_graph_check(g)
+            assert e.value.status_name == "IT_ERR_TIMEOUT"
+        else:
+            B.it_graph_check(g)
+    again = B.it_graph_create(ip, ix)  # takes the word of the destroyed one
+    B.it_graph_check(again)
+    for k, g in enumerate(graphs):
+        if k != 700:
+            B.it_graph_destroy(g)
+    for g in [B.it_graph_create(ip, ix) for _ in range(1040)]:
+        B.it_graph_check(g)
+        B.it_graph_destroy(g)

@@ -49,3 +49,24 @@ def test_a_refused_launch_is_reported_once(kind):
     gather()
     torch.cuda.synchronize()
     assert bool(torch.isfinite(out).all())
+
+
+def test_a_refused_creation_leaves_nothing_behind():
+    """The validation cannot be queued or waited for: the creation is refused, the next graphs are not, and start without a timeout."""
+    w = small_workload(3, 300, 9, "f32", [make_sage_layer(1, "mean", "none", 32, 32, "f32")])
+    ip, ix = torch.from_numpy(w.indptr).cuda(), torch.from_numpy(w.indices).cuda()
+    torch.cuda.synchronize()
+    with _InvalidCapture() as stream:
+        for _ in range(3):
+            with pytest.raises(B.ItError) as ei:
+                B.it_graph_create(ip, ix, stream=stream)
+            assert ei.value.status_name == "IT_ERR_CUDA"
+    bad = ix.clone()
+    bad[0] = w.n
+    for _ in range(3):
+        with pytest.raises(B.ItError) as ei:
+            B.it_graph_create(ip, bad)
+        assert ei.value.status_name == "IT_ERR_BAD_GRAPH"
+        g = B.it_graph_create(ip, ix)
+        B.it_graph_check(g)
+        B.it_graph_destroy(g)
