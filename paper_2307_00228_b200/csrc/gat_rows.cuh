@@ -230,12 +230,13 @@ template <int LPR, int H> constexpr int gat_bytes_per_warp() { return ring_bytes
 template <typename T, int LPR, int H>
 __global__ void __launch_bounds__(THREADS, IT_GAT_CHUNK_BLOCKS) gat_rows_chunk_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol) {
   extern __shared__ uint4 ring_raw[];
+  static_assert(gat_bytes_per_warp<LPR, H>() % 16 == 0, "a warp's weights are written 16 bytes at a time");
   const int lane = threadIdx.x & 31;
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(ring_raw) + (uint32_t)(threadIdx.x >> 5) * (uint32_t)gat_bytes_per_warp<LPR, H>();
   RingWarp<T, 16, LPR, GatAcc<T>, false, gat_stage_rows<LPR>()> rw;
   rw.setup(base, p.src, p.src_pitch, p.slices, lane);
   pol.setup(lane % LPR);
-  __shared__ float bias_buf[256];
+  __shared__ __align__(16) float bias_buf[256];   // (read 16 bytes at a time)
   stage_bias(pol, bias_buf);
   GatWarp<T, LPR, H> gw(p, q, lane, base + ring_bytes_per_warp<16, false, gat_stage_rows<LPR>()>());
   ChunkCursor<false, true> cur(p, lane);
@@ -387,7 +388,7 @@ __device__ __forceinline__ void gat_short_rows(const StreamParams &p, const GatP
 template <typename T, int LPR, int H>
 __global__ void __launch_bounds__(THREADS, IT_GAT_SHORT_BLOCKS) gat_short_rows_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol) {
   extern __shared__ uint4 short_buf[];
-  __shared__ float bias_buf[256];
+  __shared__ __align__(16) float bias_buf[256];   // (read 16 bytes at a time)
   pol.setup(threadIdx.x % LPR);
   stage_bias(pol, bias_buf);
   gat_short_rows<T, LPR, H>(p, q, pol, blockIdx.x, gridDim.x, short_buf);
@@ -398,8 +399,8 @@ template <typename T, int LPR, int H>
 __global__ void __launch_bounds__(THREADS, SMALL_BLOCKS) gat_small_kernel(StreamParams p, GatParams q, GatPolicy<T, 16> pol, PieceParams pq, SmallShare sh) {
   constexpr int SL = 32 / LPR, U = 4, VEC = GatAcc<T>::VEC, NS = GatPolicy<T, 16>::NS;   // U rows in flight per lane
   extern __shared__ uint4 short_buf[];
-  __shared__ float weights[THREADS / 32][32 * H];
-  __shared__ float bias_buf[256];
+  __shared__ __align__(16) float weights[THREADS / 32][32 * H];
+  __shared__ __align__(16) float bias_buf[256];   // (read 16 bytes at a time)
   it_allow_next();
   const int lane = threadIdx.x & 31, slot = lane / LPR, t = lane % LPR;
   pol.setup(t);
