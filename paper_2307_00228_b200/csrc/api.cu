@@ -405,16 +405,16 @@ it_status stage_gather(const StageCtx &c, const void *table, const float *scores
           int32_t *first = reinterpret_cast<int32_t *>((char *)Q + it_align_up(tiles * 2 * (size_t)L->msg_dim * 4));
           int32_t *ends = reinterpret_cast<int32_t *>((char *)first + it_align_up(tiles * 4));
           it_tc_reduce q;
-          q.indptr = g->indptr; q.indptr64 = g->indptr_type == IT_I64; q.n = g->n; q.tile_first = first; q.ends = ends; q.partial = reinterpret_cast<float *>(Q);
+          q.indptr = g->indptr; q.indptr64 = g->indptr_type == IT_I64; q.tile_first = first; q.ends = ends; q.partial = reinterpret_cast<float *>(Q);
           q.weights = L->use_edge_weights ? g->edge_weights : nullptr; q.dst = out; q.dst_ld = q.dim = L->msg_dim;
-          const int plain = q.weights ? 0 : 2;   // (the unweighted forms of max and min)
-          q.mode = gg.op == IT_GATHER_MAX ? 2 + plain : (gg.op == IT_GATHER_MIN ? 3 + plain : (q.weights ? 1 : 0)); q.is_mean = gg.op == IT_GATHER_MEAN;
+          q.mode = gg.op == IT_GATHER_MAX ? (q.weights ? IT_MSG_WMAX : IT_MSG_MAX) : (gg.op == IT_GATHER_MIN ? (q.weights ? IT_MSG_WMIN : IT_MSG_MIN) : (q.weights ? IT_MSG_WSUM : IT_MSG_SUM));
+          q.is_mean = gg.op == IT_GATHER_MEAN;
           if (!c.recording()) IT_TRY(it_launch_message_tiles(g, first, ends, c.st));
           IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, L->act_edge, nullptr, table, g->indices, &q));
           return c.recording() ? IT_OK : it_launch_message_combine(g, q, c.st);
         }
         it_tc_reduce rows{};
-        rows.mode = 6;
+        rows.mode = IT_MSG_STORE;
         IT_TRY(run_dense(c, g->e, g->edge_feat, L->edge_dim, W_edge_part, L->msg_dim, L->bias_edge, whole ? L->act_edge : IT_ACT_NONE, Q,
                          whole ? table : nullptr, whole ? g->indices : nullptr, whole ? &rows : nullptr));
         if (c.recording()) return IT_OK;

@@ -2,8 +2,10 @@
 //   C[M, NB] = X1[M, K1] * B[0:K1, :] + X2[M, K2] * B[K1:, :]
 // with tcgen05.mma (accumulators in TMEM), operands staged in shared memory by TMA
 // (128-byte swizzle), the small weight matrix resident in shared memory for the life of the
-// CTA, two TMEM accumulator buffers so that the epilogue of one 128-row tile overlaps the
-// main loop of the next, and bias / activation / dtype routing / GAT scores in the epilogue.
+// CTA (or, too large for that, streamed beside the operand), two TMEM accumulator buffers so that
+// the epilogue of one 128-row tile overlaps the main loop of the next (four where learned messages
+// are made, one where fp32 takes more than 64 columns), and bias / activation / dtype routing / GAT
+// scores in the epilogue.
 //
 // Two operand modes:
 //   bf16 : kind::f16 with bf16 inputs, fp32 accumulation.
@@ -147,11 +149,10 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_read_but_last() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-// Named barriers of the epilogue warps (immediate operands): barrier 1 over all sixteen warps, or barriers 1 and 2
-// over the eight warps of a group, or 1 to 4 over the four.  The reducing form also tells every thread whether any of them failed.
+// Named barriers of the epilogue warps: barrier 1 over all sixteen, or barriers 1 and 2 over the eight of a group, or 1 to 4 over the
+// four.  The reducing form also tells every thread whether any of them failed.
 __device__ __forceinline__ void epi_bar_sync(int groups, int group) {
   if (groups == 1) asm volatile("bar.sync 1, %0;" ::"n"(32 * TC_EPI_WARPS) : "memory");
-  else if (groups == 4) asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(8 * TC_EPI_WARPS) : "memory");
   else if (group == 0) asm volatile("bar.sync 1, %0;" ::"n"(16 * TC_EPI_WARPS) : "memory");
   else asm volatile("bar.sync 2, %0;" ::"n"(16 * TC_EPI_WARPS) : "memory");
 }
@@ -255,7 +256,7 @@ struct TcParams {
   int *status;                    // set to 1 if a bounded wait gave up
   int tma_store;                  // 1: the epilogue stages each output tile in shared memory and writes it with TMA stores
   int out_panels;                 // 16 KB panels of one staging tile (128 rows x 128 bytes each)
-  int epi_groups;                 // staged epilogue: 1, or 2 groups of eight warps that take alternate tiles (one staging tile each)
+  int epi_groups;                 // staged epilogue: 1, or 2 groups of eight warps (ADD: or 4 of four) that take tiles in turn (one staging tile each)
   uint32_t spin_limit;            // polls after which a wait on a barrier gives up
   int no_loads;                   // test hook: the producer issues no copies, so every wait runs out
 };
@@ -267,23 +268,20 @@ struct TcParams {
 // 128 consecutive edges, so a run of consecutive vertices of which the first and the last may be cut.  A warp folds the vertices that
 // end in its rows, a column pair per lane; a vertex that crosses tiles leaves one fp32 row per tile for it_launch_message_combine.
 // ADD: warps of an epilogue group, four (four tiles at a time) for up to 64 columns, else eight.
-// Bound by issue slots and the latency of an epilogue warp's tile (16 of these warps, 5100 warp instructions per tile of 128 x 64, 2.2
-// per clock and SM; without the reduce the kernel takes 0.75 ms instead of 1.1).  Written out and reduced by the gather instead, the
-// message rows cost 4 GB of traffic: 1M vertices, 16M edges, 32 features, 64 columns, whole layer 1.58 against 1.33 ms.  Eight warps of
-// their own for the reduce, which leave 64 registers a thread: 1.57.
+// Bound by issue slots and the latency of an epilogue warp's tile.  Written from the ring and reduced by the gather instead, the message
+// rows cost 4 GB of traffic (which of the two: messages_reduced).  Eight warps of their own for the reduce, which leave 64 registers a
+// thread: whole layer of 1M vertices, 16M edges, 32 features, 64 columns 1.57 ms instead of 1.33.
 constexpr int TC_ADD_STAGES_MAX = 8;
 constexpr int TC_THREADS_ADD = TC_THREADS_BF16 + 128;
 static_assert(IT_MSG_TILE == TC_BM, "a tile of edges is a tile of rows");
 constexpr int TC_SEG_WORDS = 2 * TC_BM + 4;   // ADD: per ring stage, the vertex that ends at a row (or -1), weight of a row, the vertex that ends before the tile
 constexpr int TC_IDS_AHEAD = 4;               // ADD: tiles that source ids are fetched ahead of the rows
 __host__ __device__ constexpr int tc_add_warps(int nbc) { return nbc <= 64 ? 4 : 8; }   // warps that fold a tile
-// What the reduce of a tile's rows does with two neighbouring columns (it_tc_reduce).
-enum { TC_FOLD_SUM = 0, TC_FOLD_WSUM = 1, TC_FOLD_MAX = 2, TC_FOLD_MIN = 3, TC_FOLD_PMAX = 4, TC_FOLD_PMIN = 5, TC_FOLD_STORE = 6 };
 // The result so far of a column pair: two floats, or (unweighted maximum and minimum: nothing is rounded) the packed pair.
-template <int MODE>
+template <it_msg_mode MODE>
 struct TcPair {
-  static constexpr bool PACKED = MODE == TC_FOLD_PMAX || MODE == TC_FOLD_PMIN;
-  static constexpr uint32_t ID = MODE == TC_FOLD_MAX || MODE == TC_FOLD_PMAX ? 0xff80ff80u : (MODE == TC_FOLD_MIN || MODE == TC_FOLD_PMIN ? 0x7f807f80u : 0u);   // bf16 pair that changes nothing
+  static constexpr bool PACKED = MODE == IT_MSG_MAX || MODE == IT_MSG_MIN;
+  static constexpr uint32_t ID = MODE == IT_MSG_WMAX || MODE == IT_MSG_MAX ? 0xff80ff80u : (MODE == IT_MSG_WMIN || MODE == IT_MSG_MIN ? 0x7f807f80u : 0u);   // bf16 pair that changes nothing
   float2 a;
   uint32_t q;
   __device__ __forceinline__ void clear() {
@@ -291,21 +289,21 @@ struct TcPair {
     a = make_float2(__uint_as_float(ID << 16), __uint_as_float(ID << 16));
   }
   __device__ __forceinline__ void row(uint32_t raw, float w) {
-    if constexpr (MODE == TC_FOLD_PMAX) asm("max.bf16x2 %0, %0, %1;" : "+r"(q) : "r"(raw));
-    else if constexpr (MODE == TC_FOLD_PMIN) asm("min.bf16x2 %0, %0, %1;" : "+r"(q) : "r"(raw));
-    else if constexpr (MODE == TC_FOLD_SUM) asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(a.x), "+f"(a.y) : "r"(raw));
+    if constexpr (MODE == IT_MSG_MAX) asm("max.bf16x2 %0, %0, %1;" : "+r"(q) : "r"(raw));
+    else if constexpr (MODE == IT_MSG_MIN) asm("min.bf16x2 %0, %0, %1;" : "+r"(q) : "r"(raw));
+    else if constexpr (MODE == IT_MSG_SUM) asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}" : "+f"(a.x), "+f"(a.y) : "r"(raw));
     else {
       const float lo = __uint_as_float(raw << 16), hi = __uint_as_float(raw & 0xffff0000u);
-      if (MODE == TC_FOLD_WSUM) { a.x = fmaf(w, lo, a.x); a.y = fmaf(w, hi, a.y); }
-      else if (MODE == TC_FOLD_MAX) { a.x = fmaxf(a.x, w * lo); a.y = fmaxf(a.y, w * hi); }
+      if (MODE == IT_MSG_WSUM) { a.x = fmaf(w, lo, a.x); a.y = fmaf(w, hi, a.y); }
+      else if (MODE == IT_MSG_WMAX) { a.x = fmaxf(a.x, w * lo); a.y = fmaxf(a.y, w * hi); }
       else { a.x = fminf(a.x, w * lo); a.y = fminf(a.y, w * hi); }
     }
   }
   __device__ __forceinline__ void join(int o) {   // with the lane o away
     if constexpr (PACKED) { row(__shfl_xor_sync(0xffffffffu, q, o), 1.f); return; }
     const float2 b = make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
-    if (MODE == TC_FOLD_MAX) { a.x = fmaxf(a.x, b.x); a.y = fmaxf(a.y, b.y); }
-    else if (MODE == TC_FOLD_MIN) { a.x = fminf(a.x, b.x); a.y = fminf(a.y, b.y); }
+    if (MODE == IT_MSG_WMAX) { a.x = fmaxf(a.x, b.x); a.y = fmaxf(a.y, b.y); }
+    else if (MODE == IT_MSG_WMIN) { a.x = fminf(a.x, b.x); a.y = fminf(a.y, b.y); }
     else { a.x += b.x; a.y += b.y; }
   }
   __device__ __forceinline__ float2 value() const {
@@ -323,7 +321,7 @@ __device__ __forceinline__ uint32_t lds_b32(uint32_t at) {
 // (or -1), then the rows' weights; cut_before: the tile's first edge is not the first of its vertex; has_next: another tile follows.
 // Eight rows at a time, whose places are known but for the first one's; rows of up to 32 columns (NARROW) by half a warp each
 // (300k vertices / 5M edges, 32 columns: 381 us, by whole warps 408).
-template <int MODE, int WARPS, bool NARROW>
+template <it_msg_mode MODE, int WARPS, bool NARROW>
 __device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *seg, bool cut_before, bool has_next, int64_t tile, int gw, int lane,
                                                const it_tc_reduce &q, int nbc) {
   constexpr int RW = TC_BM / WARPS;   // a warp folds the vertices that end in its RW rows (the last one also the vertex that does not end)
@@ -353,7 +351,7 @@ __device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *s
           const uint32_t r = (uint32_t)(i * STEP + half);
           v[i] = lds_b32(row + (chunk ^ (r << 4)) + r * 128u);
           w[i] = 0x3f800000u;
-          if (MODE == TC_FOLD_WSUM || MODE == TC_FOLD_MAX || MODE == TC_FOLD_MIN) w[i] = (uint32_t)seg[TC_BM + r0 + (int)r];
+          if (MODE == IT_MSG_WSUM || MODE == IT_MSG_WMAX || MODE == IT_MSG_WMIN) w[i] = (uint32_t)seg[TC_BM + r0 + (int)r];
         }
         if (r0 < start || end - r0 < 7) {   // rows of other vertices: a value that changes nothing, and weight 1
           const int lo = start > r0 ? start - r0 : 0, hi = end - r0 < 7 ? end - r0 : 7;
@@ -362,7 +360,7 @@ __device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *s
           for (int i = 0; i < LDS; ++i) {
             const uint32_t in = (uint32_t)((int)(rows << (31 - (i * STEP + half))) >> 31);
             v[i] = (v[i] & in) | (TcPair<MODE>::ID & ~in);
-            if (MODE == TC_FOLD_WSUM || MODE == TC_FOLD_MAX || MODE == TC_FOLD_MIN) w[i] = (w[i] & in) | (0x3f800000u & ~in);
+            if (MODE == IT_MSG_WSUM || MODE == IT_MSG_WMAX || MODE == IT_MSG_WMIN) w[i] = (w[i] & in) | (0x3f800000u & ~in);
           }
         }
 #pragma unroll
@@ -390,9 +388,9 @@ __device__ __forceinline__ void tc_reduce_tile(uint32_t tile_s, const int32_t *s
 
 // STREAM: the weights do not stay in shared memory; the k-block of them that belongs to an operand tile comes with it, in the same
 // stage.  (For weights so large that a CTA could keep few columns of them only: it_tc_columns.)
-// FOLD (with ADD): what becomes of the rows, TC_FOLD_*, a kernel each: one reduce in the code of all warps fits the instruction
+// FOLD (with ADD; else IT_MSG_STORE): what becomes of the rows, IT_MSG_*, a kernel each: one reduce in the code of all warps fits the instruction
 // caches, where six side by side cost 8 % of the layer.
-template <bool TF32, int ADD, bool STREAM, int FOLD, bool NARROW>
+template <bool TF32, int ADD, bool STREAM, it_msg_mode FOLD, bool NARROW>
 __global__ void __launch_bounds__(TF32 ? TC_THREADS_TF32 : (ADD ? TC_THREADS_ADD : TC_THREADS_BF16), 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_x2,
                const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_o0,
@@ -436,7 +434,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
 
   // fp32 mode: columns [nbc, 2 nbc) of an accumulator hold A_hi * B_lo, added to the first half by the epilogue
   const uint32_t acc_cols = (uint32_t)p.nbc * (TF32 ? 2u : 1u);
-  const uint32_t a_col0 = NACC * acc_cols;   // fp32 mode: the split A stages follow the two accumulators
+  const uint32_t a_col0 = NACC * acc_cols;   // fp32 mode: the split A stages follow the accumulators
   uint32_t tmem_cols = 32;
   while (tmem_cols < NACC * acc_cols + (TF32 ? (uint32_t)p.tstages * TC_TSTAGE_COLS : 0u)) tmem_cols <<= 1;
 
@@ -454,7 +452,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
     if (ADD)
       for (int a = 0; a < add_stages; ++a) {
         mbar_init(&add_full[a], 128);
-        mbar_init(&add_empty[a], FOLD == TC_FOLD_STORE ? 1 : ADD);
+        mbar_init(&add_empty[a], FOLD == IT_MSG_STORE ? 1 : ADD);
       }
     for (int a = 0; a < NACC; ++a) {
       mbar_init(&acc_full[a], 1);
@@ -637,8 +635,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
         bool released = false;
         if constexpr (ADD) {
           // One bf16 output in one column split: a warp's 16 columns at a time, activation on packed pairs.  This kernel is bound by
-          // its issue slots: with the general loop below it spent 7300 warp instructions on a tile of 128 x 64, now 4700 (16M
-          // edges, 32 edge features, 64 columns: 1.42 -> 1.0 ms; the whole layer 1.93 -> 1.53).
+          // its issue slots: the general loop below in its place took 1.42 ms instead of 1.0 (16M edges, 32 edge features, 64 columns).
           const uint32_t add_row = smem_u32(smem_add) + (uint32_t)slot * (uint32_t)p.add_stage_bytes + (uint32_t)row_in_tile * 128u;
           for (int c = gsub * 16; c < p.nbc; c += 16 * n_sub) {
             uint32_t r[16], w[8];
@@ -774,7 +771,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           if (lane == 0) mbar_arrive(&acc_empty[acc]);
         }
         if constexpr (ADD) {
-          if constexpr (FOLD == TC_FOLD_STORE) {   // written from where it lies; its stage is free when the copy has read it
+          if constexpr (FOLD == IT_MSG_STORE) {   // written from where it lies; its stage is free when the copy has read it
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             if (epi_bar_any(G, group, false)) { ok = false; break; }   // the tile is complete
             if (issuer) {
@@ -807,7 +804,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_x1, const __grid_constant
           tma_store_commit();
         }
       }
-      if ((!ADD || FOLD == TC_FOLD_STORE) && issuer) tma_store_wait_all();   // the staging tile must outlive the last stores
+      if (FOLD == IT_MSG_STORE && issuer) tma_store_wait_all();   // the staging tile must outlive the last stores
     } else
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
       const int64_t m = (int64_t)(tile / p.n_splits) * TC_BM + row_in_tile;
@@ -1642,7 +1639,7 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
   const int epi_groups = sh.epi_groups, stages = sh.stages, s0 = a.dt0 == IT_BF16 ? 2 : 4, s1 = a.dt1 == IT_BF16 ? 2 : 4;
   const bool staged = sh.staged;
   const int smem = b_bytes + stages * sh.stage_bytes + epi_groups * out_panels * panel_bytes + kSmemAux + const_bytes;
-  // fp32 mode: TMEM holds two accumulators of 2 nbc columns; what is left of its 512 columns stages the split A
+  // fp32 mode: TMEM holds two accumulators of 2 nbc columns (one beyond 64 columns); what is left of its 512 columns stages the split A
   const int n_acc = nbc > 64 ? 1 : 2;
   int tstages = tf32 ? (512 - n_acc * 2 * nbc) / TC_TSTAGE_COLS : 0;
   if (tstages > TC_TSTAGES_MAX) tstages = TC_TSTAGES_MAX;
@@ -1681,25 +1678,26 @@ it_status it_launch_gemm_tc(const it_gemm_args &a, const void *B, const float *a
     IT_LAUNCH(IT_K_GEMM_TC, bytes + more, flops, st, IT_CUDA_TRY(it_launch_pdl(kernel, dim3((unsigned)grid), dim3(threads), smem, st, m1, m2, mb, mo0, mo1, p)));
     return IT_OK;
   };
-  if (tf32) IT_TRY(cols.stream ? go(gemm_tc_kernel<true, 0, true, 0, false>, TC_THREADS_TF32, 0.0) : go(gemm_tc_kernel<true, 0, false, 0, false>, TC_THREADS_TF32, 0.0));
+  if (tf32) IT_TRY(cols.stream ? go(gemm_tc_kernel<true, 0, true, IT_MSG_STORE, false>, TC_THREADS_TF32, 0.0) : go(gemm_tc_kernel<true, 0, false, IT_MSG_STORE, false>, TC_THREADS_TF32, 0.0));
   else if (a.add_rows) {
-    auto fold = [&]<int MODE>() -> it_status {
+    auto fold = [&]<it_msg_mode MODE>() -> it_status {
       const double more = (double)a.M * 4.0;
       if (tc_add_warps(nbc) == 8) return go(gemm_tc_kernel<false, 8, false, MODE, false>, TC_THREADS_ADD, more);
-      if (nbc <= 32 && MODE != TC_FOLD_STORE) return go(gemm_tc_kernel<false, 4, false, MODE, true>, TC_THREADS_ADD, more);
+      if (nbc <= 32 && MODE != IT_MSG_STORE) return go(gemm_tc_kernel<false, 4, false, MODE, true>, TC_THREADS_ADD, more);
       return go(gemm_tc_kernel<false, 4, false, MODE, false>, TC_THREADS_ADD, more);
     };
     switch (a.reduce.mode) {
-      case TC_FOLD_SUM: IT_TRY(fold.template operator()<TC_FOLD_SUM>()); break;
-      case TC_FOLD_WSUM: IT_TRY(fold.template operator()<TC_FOLD_WSUM>()); break;
-      case TC_FOLD_MAX: IT_TRY(fold.template operator()<TC_FOLD_MAX>()); break;
-      case TC_FOLD_MIN: IT_TRY(fold.template operator()<TC_FOLD_MIN>()); break;
-      case TC_FOLD_PMAX: IT_TRY(fold.template operator()<TC_FOLD_PMAX>()); break;
-      case TC_FOLD_PMIN: IT_TRY(fold.template operator()<TC_FOLD_PMIN>()); break;
-      default: IT_TRY(fold.template operator()<TC_FOLD_STORE>()); break;
+      case IT_MSG_SUM: IT_TRY(fold.template operator()<IT_MSG_SUM>()); break;
+      case IT_MSG_WSUM: IT_TRY(fold.template operator()<IT_MSG_WSUM>()); break;
+      case IT_MSG_WMAX: IT_TRY(fold.template operator()<IT_MSG_WMAX>()); break;
+      case IT_MSG_WMIN: IT_TRY(fold.template operator()<IT_MSG_WMIN>()); break;
+      case IT_MSG_MAX: IT_TRY(fold.template operator()<IT_MSG_MAX>()); break;
+      case IT_MSG_MIN: IT_TRY(fold.template operator()<IT_MSG_MIN>()); break;
+      case IT_MSG_STORE: IT_TRY(fold.template operator()<IT_MSG_STORE>()); break;
+      default: IT_REQUIRE(false, IT_ERR_INVALID_ARG, "tensor-core apply: no such reduce (%d)", (int)a.reduce.mode);
     }
   }
-  else IT_TRY(cols.stream ? go(gemm_tc_kernel<false, 0, true, 0, false>, TC_THREADS_BF16, 0.0) : go(gemm_tc_kernel<false, 0, false, 0, false>, TC_THREADS_BF16, 0.0));
+  else IT_TRY(cols.stream ? go(gemm_tc_kernel<false, 0, true, IT_MSG_STORE, false>, TC_THREADS_BF16, 0.0) : go(gemm_tc_kernel<false, 0, false, IT_MSG_STORE, false>, TC_THREADS_BF16, 0.0));
   IT_CUDA_TRY(cudaGetLastError());
   return IT_OK;
 }
@@ -1811,8 +1809,8 @@ extern "C" it_status it_debug_expire_wait_form(it_graph *g, int form, void *buff
   if (form < 3) {   // 0, 1: rows added and reduced by four and by eight warps a tile; 2: written.  More tiles per CTA than the ring has stages
     a.M = (int64_t)g->num_sms * (TC_ADD_STAGES_MAX + 2) * TC_BM; a.K1 = 16; a.n0 = form == 1 ? 128 : 64;
     a.out0 = nullptr; a.add_rows = buffer; a.add_idx = (const int32_t *)buffer;
-    a.reduce.mode = form == 2 ? TC_FOLD_STORE : TC_FOLD_SUM;
-    a.reduce.n = 1; a.reduce.partial = (float *)buffer; a.reduce.dst = buffer; a.reduce.dst_ld = a.reduce.dim = a.n0;
+    a.reduce.mode = form == 2 ? IT_MSG_STORE : IT_MSG_SUM;
+    a.reduce.partial = (float *)buffer; a.reduce.dst = buffer; a.reduce.dst_ld = a.reduce.dim = a.n0;
     if (form < 2) a.reduce.ends = a.reduce.tile_first = (const int32_t *)buffer;
   } else if (form < 5) {   // 3, 4: streamed weights, more tiles than stages
     a.M = 128; a.K1 = 1024; a.n0 = form == 4 ? 256 : 512;

@@ -271,19 +271,21 @@ size_t it_gat_partial_bytes(const it_graph *g, int dim, int heads);
 //   [0, n0)        -> out0 (dtype dt0) = act0(C + bias0)
 //   [n0, n0+n1)    -> out1 (dtype dt1), raw
 //   [n0+n1, NB)    -> out2 (fp32), raw, row stride n2 = NB - n0 - n1
-// The rows of such a product as messages of the edges of a graph (bf16 tensor-core path): reduced by destination in its epilogue.
+// The rows of such a product as messages of the edges of a graph (bf16 tensor-core path): reduced by destination in its epilogue, or stored.
 #define IT_MSG_TILE 128          // edges per tile
+enum it_msg_mode { IT_MSG_SUM = 0, IT_MSG_WSUM = 1 /* w: times the edge's weight */, IT_MSG_WMAX = 2, IT_MSG_WMIN = 3, IT_MSG_MAX = 4, IT_MSG_MIN = 5,
+                   IT_MSG_STORE = 6 /* not reduced: row m of out0 is edge m's, the fields below are unused */ };
 struct it_tc_reduce {
   const void *indptr;            // of the graph
   int indptr64;
-  int64_t n;                     // vertices
   const int32_t *tile_first;     // [tiles] the vertex that edge IT_MSG_TILE * t belongs to
-  const int32_t *ends;           // [tiles * IT_MSG_TILE] the vertex whose last edge this is, or -1 (mode 6: NULL)
+  const int32_t *ends;           // [tiles * IT_MSG_TILE] the vertex whose last edge this is, or -1
   float *partial;                // [tiles][2][dim]: what a vertex that crosses tiles has in a tile where it does not begin / does begin
   const float *weights;          // of the edges, or NULL
   void *dst;                     // bf16 rows: the reduce of every vertex
   int dst_ld, dim;
-  int mode, is_mean;             // 0 sum, 1 weighted sum, 2 max, 3 min, 4 / 5 the same unweighted; 6: not reduced, row m of out0 is edge m's
+  it_msg_mode mode;
+  int is_mean;
 };
 struct it_gemm_args {
   int64_t M;

@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(MSG_JOIN_THREADS, 1) message_combine_kernel(it
   __shared__ int n_todo;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = lane * 4;
-  const bool is_max = q.mode == 2 || q.mode == 4, is_min = q.mode == 3 || q.mode == 5;
+  const bool is_max = q.mode == IT_MSG_WMAX || q.mode == IT_MSG_MAX, is_min = q.mode == IT_MSG_WMIN || q.mode == IT_MSG_MIN;
   const float id = is_max ? -INFINITY : (is_min ? INFINITY : 0.f);
   auto fold = [&](float4 &a, const float4 &y) {
     if (is_max) { a.x = fmaxf(a.x, y.x); a.y = fmaxf(a.y, y.y); a.z = fmaxf(a.z, y.z); a.w = fmaxf(a.w, y.w); }
