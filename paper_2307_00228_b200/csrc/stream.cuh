@@ -662,6 +662,19 @@ it_status allow_dynamic_smem(Kernel kernel, int smem, std::atomic<uint64_t> &don
   return IT_OK;
 }
 
+// How much of an SM's L1 a kernel would have as shared memory (per cent), set once per device like the above.
+template <class Kernel>
+it_status split_l1(Kernel kernel, int percent, std::atomic<uint64_t> &done) {
+  int dev = -1;
+  IT_CUDA_TRY(cudaGetDevice(&dev));
+  const uint64_t bit = (dev >= 0 && dev < 64) ? (uint64_t)1 << dev : 0;
+  if (bit == 0 || !(done.load(std::memory_order_acquire) & bit)) {
+    IT_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent));
+    done.fetch_or(bit, std::memory_order_release);
+  }
+  return IT_OK;
+}
+
 // ----------------------------------------------------------------------------- bucket dispatch
 // Longest rows first so that the tail of the launch sequence is made of short rows.
 // bytes_of(bucket, rows) gives the algorithmic bytes of a launch; kid_* the instrumentation ids.
