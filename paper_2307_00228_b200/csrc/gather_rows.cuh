@@ -259,7 +259,7 @@ it_status launch_small(const it_gather_args &a, StreamParams sp, cudaStream_t st
   sp.weights = a.use_edge_weights ? sp.weights : nullptr;
   if (!a.zeroed && g->n_long > 0) IT_CUDA_TRY(cudaMemsetAsync(it_done_words(a.counters), 0, (size_t)g->n_long * sizeof(int), st));
   auto go = [&]<int LPR>() -> it_status {
-    const SmallShare sh = small_share(g, LPR < 8 ? 8 : LPR, LPR <= 16, a.per_edge_rows && LPR >= 8 ? 5 : 8);   // (a row of 512 bytes takes the warp either way: 100k vertices / 1.6M edges 191 us, by groups 197)
+    const SmallShare sh = small_share(g, LPR, LPR <= 16, a.per_edge_rows && LPR >= 8 ? 5 : 8);   // (a row of 512 bytes takes the warp either way: 100k vertices / 1.6M edges 191 us, by groups 197)
     // The kernel starts early, on SMs split for the product's shared memory, and without a preference it ran with the little L1 that
     // leaves, or not, by the sizes around it: fp32 max 128-32-48-32, 31k vertices / 246k edges 109 or 120 us, now 111; bf16 mean 768-256-64,
     // 30k / 600k with hubs 177 -> 157, fp32 max 64-128-96-64, 43k / 404k 212 -> 189.  Half is what three blocks' staging takes (none: 10k / 100k

@@ -55,20 +55,35 @@ struct SmallShare {
   unsigned blocks;
   int short_blocks, empty_blocks, short_lo, short_hi, total;   // (entries [0, short_lo): rows without edges)
 };
+// That is the split of work that never waits for a whole row; where there are few rows for every warp, what counts is the longest warp.
+// Rows that take a warp are dealt in turn, so a share of theirs that begins another round for a few rows is that much longer: then the
+// lane groups get fewer blocks, or more, such that neither share is more than 12 % longer than it could be (in trips to memory: a lane
+// group's row one and one per eight edges, a warp's row one and one per step).  bf16 GCN 96-64-64, 55k / 616k with hubs 66 -> 58 us (two rounds
+// of pieces to one), fp32 GCN 64-128-48, 38k / 561k 94 -> 84, attention, 23k / 281k, 256-byte rows 79 -> 70, bf16 sum 128-32-64, 125k / 1.8M 146 -> 121.
 // groups: lane groups take the short rows; row: what a row of theirs costs, in edges.
-inline SmallShare small_share(const it_graph *g, int lpr, bool groups, int row) {
+inline SmallShare small_share(const it_graph *g, int lpr_row, bool groups, int row) {
   SmallShare s;
+  const int lpr = lpr_row < 8 ? 8 : lpr_row;
   s.total = (int)g->h_list_offsets[g->n_lists];
   s.short_lo = s.short_hi = (int)g->h_list_offsets[1];
   int64_t short_cost = 0, cost = 0;
+  struct { int rows, trips; } walk[IT_MAX_BUCKETS + 1];   // lists whose rows take a warp, longest first
+  int n_walk = 0;
+  double short_trips = 0;   // of all lane groups
+  const int step = 128 / (lpr_row < 4 ? 4 : lpr_row);   // edges in flight of a warp's row
   const int64_t empty_cost = (int64_t)s.short_lo * 3 * lpr / 16;
-  for (int b = 1; b < g->n_lists; ++b) {
+  for (int b = g->n_lists; b-- > 1;) {
     const int64_t rows = g->h_list_offsets[b + 1] - g->h_list_offsets[b], edges = g->h_list_edges[b];
+    if (rows == 0) continue;
     if (groups && g->list_bounds[b] <= IT_SHORT_BELOW && b != g->n_lists - 1) {
-      s.short_hi = (int)g->h_list_offsets[b + 1];
+      if (s.short_hi < (int)g->h_list_offsets[b + 1]) s.short_hi = (int)g->h_list_offsets[b + 1];
       short_cost += (rows * row + edges) * lpr / 16;
+      // (the groups of a warp wait for the longest of their rows)
+      short_trips += (double)rows * row / 8 + (g->list_bounds[b] <= IT_SHORT_EDGES ? (double)rows : (double)edges / 8 + 0.7 * (double)rows);
     } else {
       cost += rows * 16 + edges * 2 * lpr / 16;
+      walk[n_walk].rows = (int)rows;
+      walk[n_walk++].trips = 1 + ((int)edges / (int)rows + step - 1) / step;
     }
   }
   const int most = g->num_sms * SMALL_BLOCKS;
@@ -79,8 +94,42 @@ inline SmallShare small_share(const it_graph *g, int lpr, bool groups, int row) 
     if (n > most - 2) n = most - 2;
     return n < want ? n : want;
   };
-  s.short_blocks = part(short_cost, (s.short_hi - s.short_lo + THREADS / lpr - 1) / (THREADS / lpr));
+  const int per_block = THREADS / lpr, want_short = (s.short_hi - s.short_lo + per_block - 1) / per_block;
   s.empty_blocks = part(empty_cost, (s.short_lo + THREADS / 8 - 1) / (THREADS / 8));
+  s.short_blocks = part(short_cost, want_short);
+  const int rest = most - s.empty_blocks;
+  if (n_walk > 0 && want_short > 0) {
+    const double per_group = short_trips / per_block;
+    auto longest = [&](int short_blocks) {   // trips of the longest warp
+      const int warps = (rest - short_blocks) * (THREADS / 32);
+      int at = 0, round = 0, trips = 0;
+      for (int i = 0; i < n_walk; ++i) {
+        at += walk[i].rows;
+        const int to = (at + warps - 1) / warps;
+        trips += (to - round) * walk[i].trips;
+        round = to;
+      }
+      return trips;
+    };
+    auto first = [&](auto holds) {   // the first number of short blocks in [1, rest) from which on a condition holds
+      int lo = 1, hi = rest;
+      while (lo < hi) {
+        const int mid = (lo + hi) / 2;
+        if (holds(mid)) hi = mid;
+        else lo = mid + 1;
+      }
+      return lo;
+    };
+    const int cross = first([&](int x) { return per_group <= (double)x * longest(x); });   // the lane groups' is the shorter share
+    double best = cross < rest ? longest(cross) : per_group / (rest - 1);
+    if (cross > 1 && per_group / (cross - 1) < best) best = per_group / (cross - 1);
+    best *= 1.12;
+    const int most_short = first([&](int x) { return longest(x) > best; }) - 1, least_short = (int)(per_group / best) + 1;
+    int n = s.short_blocks < most_short ? s.short_blocks : most_short;
+    if (n < least_short) n = least_short;
+    if (n > rest - 1) n = rest - 1;
+    s.short_blocks = n < want_short ? n : want_short;
+  }
   const int used = s.short_blocks + s.empty_blocks, left = most - used > 1 ? most - used : 1, want = (s.total - s.short_hi + THREADS / 32 - 1) / (THREADS / 32);
   s.blocks = (unsigned)(used + (want < 1 ? 1 : (want < left ? want : left)));
   return s;
